@@ -3,6 +3,7 @@
 // spmspv.cu.
 #include <cstdio>
 #include <cstring>
+#include <mutex>
 #include <new>
 
 #include "spdp_internal.h"
@@ -19,8 +20,31 @@ void note_cuda_error(cudaError_t e, const char* what) {
 
 namespace {
 
+// Scratch memory of calls that need some (spdp_spmm's partial sums): one pool per device, apart from the device's
+// default pool.  The default pool gives its memory back to the driver at every synchronisation, so a call after one
+// allocated again (0.45 ms on the prefill of 1024 tokens, against the 0.43 ms of its kernels).  This pool keeps at
+// most kScratchKeep bytes over a synchronisation and gives everything back when the device's last handle goes.
+// Stream-ordered: calls on several streams or threads get memory of their own.
+constexpr int kMaxDevices = 64;
+constexpr uint64_t kScratchKeep = uint64_t(96) << 20;
+struct ScratchPool {
+    cudaMemPool_t pool;
+    int64_t handles;
+};
+std::mutex g_scratch_mu;
+ScratchPool g_scratch[kMaxDevices];
+
+void count_handle(int device, int by) {
+    if (device < 0 || device >= kMaxDevices) return;
+    std::lock_guard<std::mutex> lock(g_scratch_mu);
+    ScratchPool& sp = g_scratch[device];
+    sp.handles += by;
+    if (sp.handles == 0 && sp.pool != nullptr) cudaMemPoolTrimTo(sp.pool, 0);
+}
+
 void release(spdp_matrix* h) {
     if (h == nullptr) return;
+    count_handle(h->device, -1);
     cudaFree(h->tileoffset);
     cudaFree(h->colinfo);
     cudaFree(h->bitmap);
@@ -58,6 +82,7 @@ spdp_status new_handle(int64_t M, int64_t K, int pad_elems, spdp_matrix** out) {
     cudaError_t e = cudaGetDevice(&h->device);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&h->sm_count, cudaDevAttrMultiProcessorCount, h->device);
     if (e != cudaSuccess) { note_cuda_error(e, "device query"); delete h; return SPDP_ERR_CUDA; }
+    count_handle(h->device, 1);
     *out = h;
     return SPDP_OK;
 }
@@ -121,6 +146,29 @@ spdp_status launch_decode(const spdp_matrix* h, const __half* x, int rule, float
 bool rule_ok(int rule) { return rule == SPDP_DP_NONE || rule == SPDP_DP_ABS_GT || rule == SPDP_DP_MASK; }
 
 }  // namespace
+
+spdp_status scratch_alloc(int device, size_t bytes, cudaStream_t s, void** out) {
+    if (device < 0 || device >= kMaxDevices) return SPDP_ERR_UNSUPPORTED_SHAPE;
+    cudaMemPool_t pool = nullptr;
+    {
+        std::lock_guard<std::mutex> lock(g_scratch_mu);
+        ScratchPool& sp = g_scratch[device];
+        if (sp.pool == nullptr) {
+            cudaMemPoolProps props = {};
+            props.allocType = cudaMemAllocationTypePinned;
+            props.handleTypes = cudaMemHandleTypeNone;
+            props.location.type = cudaMemLocationTypeDevice;
+            props.location.id = device;
+            SPDP_CUDA_TRY(cudaMemPoolCreate(&sp.pool, &props));
+            uint64_t keep = kScratchKeep;
+            SPDP_CUDA_TRY(cudaMemPoolSetAttribute(sp.pool, cudaMemPoolAttrReleaseThreshold, &keep));
+        }
+        pool = sp.pool;
+    }
+    SPDP_CUDA_TRY(cudaMallocFromPoolAsync(out, bytes, pool, s));
+    return SPDP_OK;
+}
+
 }  // namespace spdp
 
 namespace spdp {

@@ -90,6 +90,9 @@ void note_cuda_error(cudaError_t e, const char* what);
 
 inline bool valid(const spdp_matrix* h) { return h != nullptr && h->magic == kMagic; }
 
+// api.cu: stream-ordered scratch memory for one call (given back with cudaFreeAsync on the same stream).
+spdp_status scratch_alloc(int device, size_t bytes, cudaStream_t s, void** out);
+
 // pack.cu
 spdp_status pack_device(spdp_matrix* h, const __half* W, int64_t ldw, cudaStream_t s);
 spdp_status unpack_device(const spdp_matrix* h, __half* W, int64_t ldw, cudaStream_t s);

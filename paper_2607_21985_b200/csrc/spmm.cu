@@ -5,30 +5,34 @@
 // there.  On Blackwell the tensor cores read both operands straight from shared memory
 // (tcgen05.mma) and accumulate in tensor memory, so the layout-alignment stage becomes the decode
 // itself: W is given to the tensor cores M-major (rows contiguous), which is how a column tile
-// lies in Tiled-CBC, so a lane that owns 8 consecutive rows of a column (one bitmap byte: its
-// values are one contiguous run, rank = set bits before the byte, Sec. 4.2.1) writes exactly one
-// 16-byte piece of the operand tile per column.  No registers hold accumulators, no ldmatrix pass.
+// lies in Tiled-CBC.
 //
-// K is walked in blocks of kKB columns = 4 GTiles.  Warp roles (both kernels below):
-//   * copy warp, one thread: everything that moves data.  The 4 GTiles of a K-block are consecutive in
-//     storage order, so their Values are ONE contiguous span (TileOffset[g] .. TileOffset[g+4]), their
-//     Bitmap words another, their ColInfo words a third: three bulk copies (cp.async.bulk) per K-block
-//     bring the block as stored.  An X tile (kKB columns x tokens, 128-byte swizzle, zero beyond K
-//     and N) is one tiled bulk-tensor copy.  All copies complete on shared-memory barriers.
-//   * tensor-core warp, one thread: when a block's decoded tile and X tile are there it issues the
-//     block's tcgen05.mma (K = 16 each) and commits them to the stage's barrier.
-//   * 16 decode warps: warp w decodes columns w, w+16, w+32, w+48 of the block into the operand tile
-//     and arrives on the stage's barriers.  They issue no copies and meet no CTA-wide barrier in the loop.
-// Every wait is bounded; every copy writes only the shared memory of the CTA that issued it.
+// K is walked in K-blocks of 64 columns = 4 GTiles.  Warp roles (both kernels below):
+//   * copy warp: consecutive GTiles of a row tile are consecutive in storage order, so their Values are ONE
+//     contiguous span (TileOffset[g] .. TileOffset[g + n]), their Bitmap words another, their ColInfo words a
+//     third: three bulk copies (cp.async.bulk) bring a K-block as stored.
+//   * X tiles (64 columns x tokens, 128-byte swizzle, zero beyond K and N) are tiled bulk-tensor copies.
+//   * tensor-core warp, one thread: when decoded columns and their X tile are there it issues the
+//     tcgen05.mma (K = 16 each) and commits them to the barriers of what they read.
+//   * 24 decode warps, the first 16 of which also store the accumulators at the end.
+// All copies complete on shared-memory barriers; every wait is bounded; every copy writes only the shared
+// memory of the CTA that issued it.
 //
-// Two kernels share this structure:
-//   one::spmm_kernel   one CTA = one row tile (256 rows = two M = 128 accumulators) x 256 tokens.
-//   pair::spmm_kernel  two CTAs on neighbouring SMs (a cluster of 2) = one row tile x 512 tokens:
-//                      tcgen05.mma.cta_group::2 multiplies M = 256 (128 rows from each CTA's shared memory)
-//                      by N = 256 (128 tokens from each CTA's shared memory) and leaves 128 rows x 256 fp32
-//                      columns in each CTA's tensor memory; two such accumulators fill the 512 columns.  Each
-//                      CTA decodes only ITS 128 rows of every column tile: half the decode per token.
-// The launch picks the one with fewer rounds of CTAs x cost per K-block (small N: the first).
+// Decode (Sec. 4.2.1).  A lane expands 4 consecutive rows (one nibble of a bitmap word) of a column at a
+// time, so that a warp's loads for 128 rows fall into at most 256 contiguous bytes: rank = set bits before the
+// nibble, three aligned 32-bit loads cover its at most 4 values wherever they start, two funnel shifts align
+// them, and two byte permutes with selectors computed from the nibble put them into their rows, one 8-byte store
+// per lane.  (A walk over the 8 rows of a bitmap byte with predicated 16-bit loads, as before, took twice the
+// instructions, and 43-49 % of the shared-memory wavefronts were bank conflicts.)
+//
+//   one::   one CTA = one row tile (256 rows = two M = 128 accumulators) x up to 32, 128 or 256 tokens.  The CTAs stay for
+//           the whole call: whole rounds of tiles first, one tile per CTA; the K-blocks of the tiles that are left are cut
+//           into equal contiguous ranges, one per CTA.  A tile fed by several CTAs leaves fp32 partial sums in scratch
+//           memory, which a second kernel adds in CTA order (the result does not depend on timing).
+//   pair::  two CTAs on neighbouring SMs (a cluster of 2) = one row tile x 512 tokens: tcgen05.mma.cta_group::2
+//           multiplies M = 256 (128 rows from each CTA's shared memory) by N = 256 (128 tokens from each CTA's shared
+//           memory) and leaves 128 rows x 256 fp32 columns in each CTA's tensor memory; two such accumulators fill the
+//           512 columns.  Each CTA decodes only ITS 128 rows of every column tile: half the decode per token.
 #include <cuda.h>
 
 #include <algorithm>
@@ -43,30 +47,35 @@ namespace {
 
 using namespace dev;
 
-constexpr int kWarps = 16;             // decode warps
-constexpr int kKB = 64;                // columns per K-block: 4 GTiles, 4 tensor-core steps of K = 16 per accumulator
+// Decode warps: kGroups groups of 8; a group decodes every kGroups-th sub-block of 32 columns, 4 columns a warp, so that
+// one group's waits and scan overlap the others' decode (two groups: 79 us against 73 on 148 row tiles x 4096 x 128 tokens).
+constexpr int kGroups = 3;
+constexpr int kGroupWarps = 8;
+constexpr int kWarps = kGroups * kGroupWarps;
+constexpr int kStoreWarps = 16;        // the first 16 store the accumulators
+constexpr int kThreads = (kWarps + 3) * 32;   // and three warps for copies and the tensor cores
+constexpr int kKB = 64;                // columns per K-block: one 128-byte swizzle row of X per token
+constexpr int kSub = 32;               // columns per sub-block
+constexpr int kSubs = kKB / kSub;
 constexpr int kGTB = kKB / kTileK;     // GTiles per K-block
-constexpr int kNI = 256;               // the N of the tensor-core instruction
-constexpr int kTmemCols = 512;         // both kernels use all of tensor memory: two accumulators of 128 rows x kNI columns
+constexpr int kBlockWarps = kSubs * kGroupWarps;      // warps that decode a K-block
+static_assert(kSub == 4 * kGroupWarps, "a scan takes 4 columns");
+static_assert(kWarps >= kStoreWarps, "16 warps store");
 // A (decoded W), M-major without swizzle: 16-byte piece = 8 consecutive rows of one column; the 8
 // columns of a k-group are 16 bytes apart (a core matrix of 128 bytes), the 16 row chunks of a
-// 128-row tile 144 bytes apart (128 + 16: the 16-byte pieces that the lanes of a quarter warp store for
-// one column then fall into different banks), the k-groups 16 * 144 bytes apart.
+// 128-row tile 144 bytes apart (128 + 16: the pieces that a warp stores for one column then fall into
+// different banks), the k-groups 16 * 144 bytes apart.
 constexpr int kAChunkStride = 144;                 // stride byte offset: next 8 rows
 constexpr int kAKGroupStride = 16 * kAChunkStride; // leading byte offset: next 8 columns
-constexpr int kATileBytes = (kKB / 8) * kAKGroupStride;    // 128 rows x kKB columns
-// B (X tile), K-major with the 128-byte swizzle: a token's kKB columns are one 128-byte row, written by
-// one tiled bulk-tensor copy per K-block; 8 tokens form a 1024-byte swizzle atom (the stride byte offset),
-// and a tensor-core step of K = 16 starts 32 bytes further into the row.
+// B (X tile), K-major with the 128-byte swizzle: a token's kKB columns are one 128-byte row; 8 tokens form a
+// 1024-byte swizzle atom (the stride byte offset), and a tensor-core step of K = 16 starts 32 bytes further.
 constexpr int kBRowBytes = 2 * kKB;
 constexpr int kBAtomBytes = 8 * kBRowBytes;
 #ifndef SPDP_SPMM_WAIT_TRIES
 #define SPDP_SPMM_WAIT_TRIES (1 << 22)
 #endif
 constexpr int kWaitTries = SPDP_SPMM_WAIT_TRIES;
-constexpr int kCompValues = kKB * kTileM;          // the most values a K-block stores
 static_assert(kBRowBytes == 128, "one X row of a K-block is one 128-byte swizzle row");
-static_assert(kKB % 16 == 0 && kKB == 4 * kWarps, "a warp decodes 4 columns of a K-block, one per quarter of its scan");
 
 struct Params {
     const uint32_t* tileoffset;
@@ -78,23 +87,20 @@ struct Params {
     int64_t ldy;
     int ydt;
     int M, K, C;
-    int nblocks;            // token blocks: CTA (or CTA pair) = row tile * nblocks + token block
-    // CTA-pair kernel only: pair i works on tile tile0 + i / kslices, on slice i % kslices of the tile's K-blocks; with
-    // kslices > 1 it leaves fp32 partial sums in partial[i][token in tile][row in tile] instead of writing Y.
+    int nblocks;            // token blocks: tile = row tile * nblocks + token block
+    int nkb;                // K-blocks of a tile
+    // one::  CTA w takes tiles w, w + workers, ... for `rounds` rounds; rest_units = K-blocks of the tiles after those, cut
+    // into `sharers` equal ranges for CTAs 0 .. sharers - 1
+    int workers, rounds, sharers;
+    unsigned rest_units;
+    // pair:: pair i works on tile tile0 + i / kslices, on slice i % kslices of the tile's K-blocks
     int tile0, kslices;
-    float* partial;
+    float* partial;         // partial sums [slot][token in tile < ptok][256 rows]; slot = pair i, or 2 * CTA + (0: its first
+                            // piece, 1: its last); pair:: null = whole tiles
+    int ptok;
     int* status;
     int64_t values_len;
 };
-
-struct CompStage {                              // one K-block as stored
-    alignas(128) unsigned short vals[kCompValues + 16];   // the values of its 4 GTiles, contiguous
-    alignas(16) uint32_t bm[kKB][8];            // bitmaps
-    alignas(16) uint32_t ci[kKB];               // ColInfo words
-    uint32_t to[kGTB + 1];                      // TileOffset words of the block's GTiles (+ the next one)
-};
-static_assert(offsetof(CompStage, bm) % 16 == 0 && offsetof(CompStage, ci) % 16 == 0 && sizeof(CompStage) % 16 == 0,
-              "bulk copies need 16-byte aligned destinations");
 
 // Shared-memory operand descriptor of tcgen05.mma: start address, leading byte offset, stride byte
 // offset (all in 16-byte units), descriptor version of this architecture, layout (bits 61-63: 0 = no
@@ -107,19 +113,36 @@ __device__ __forceinline__ uint64_t operand_desc(uint32_t smem_addr, uint32_t lb
     d |= static_cast<uint64_t>(layout) << 61;
     return d;
 }
-// Instruction descriptor: fp16 x fp16 -> fp32, A M-major (bit 15), B K-major, M rows, N = kNI.
-template <int kM>
-constexpr uint32_t kInstrDesc = (1u << 4) | (1u << 15) | (static_cast<uint32_t>(kNI >> 3) << 17) | (static_cast<uint32_t>(kM >> 4) << 24);
+// Instruction descriptor: fp16 x fp16 -> fp32, A M-major (bit 15), B K-major, kM rows, kN tokens.
+template <int kM, int kN>
+constexpr uint32_t kInstrDesc = (1u << 4) | (1u << 15) | (static_cast<uint32_t>(kN >> 3) << 17) | (static_cast<uint32_t>(kM >> 4) << 24);
 // D[tmem] (+)= A * B, one CTA (M = 128) or a CTA pair (M = 256).
+template <int kN>
 __device__ __forceinline__ void mma_f16_one(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc, bool accumulate) {
     asm volatile("{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
                  " tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}"
-                 ::"r"(d_tmem), "l"(a_desc), "l"(b_desc), "r"(kInstrDesc<128>), "r"(accumulate ? 1u : 0u) : "memory");
+                 ::"r"(d_tmem), "l"(a_desc), "l"(b_desc), "r"(kInstrDesc<128, kN>), "r"(accumulate ? 1u : 0u) : "memory");
 }
+template <int kN>
 __device__ __forceinline__ void mma_f16_pair(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc, bool accumulate) {
     asm volatile("{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
                  " tcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %3, p;\n}"
-                 ::"r"(d_tmem), "l"(a_desc), "l"(b_desc), "r"(kInstrDesc<256>), "r"(accumulate ? 1u : 0u) : "memory");
+                 ::"r"(d_tmem), "l"(a_desc), "l"(b_desc), "r"(kInstrDesc<256, kN>), "r"(accumulate ? 1u : 0u) : "memory");
+}
+// Lets `bar` complete when the products this thread has issued so far are done.
+__device__ __forceinline__ void commit_one(unsigned long long* bar) {
+    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(smem_u32(bar)) : "memory");
+}
+__device__ __forceinline__ void commit_pair(unsigned long long* bar) {
+    asm volatile("tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(smem_u32(bar)) : "memory");
+}
+// True in one lane of the (converged) warp.  The copies and the tensor-core instructions take their operands from
+// uniform registers: behind this test the compiler knows that one lane is active and fills them directly, behind
+// `lane == 0` it loops over the lanes (95 us against 79 on 148 row tiles x 4096 x 128 tokens).
+__device__ __forceinline__ bool elect_one() {
+    unsigned e;
+    asm volatile("{\n .reg .pred p;\n elect.sync _|p, 0xFFFFFFFF;\n selp.u32 %0, 1, 0, p;\n}" : "=r"(e));
+    return e != 0u;
 }
 __device__ __forceinline__ void barrier_init(unsigned long long* bar, uint32_t arrivals) {
     asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(bar)), "r"(arrivals) : "memory");
@@ -156,15 +179,509 @@ __device__ __forceinline__ void pair_sync() {
     asm volatile("barrier.cluster.arrive.release.aligned;\n barrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
 // Bulk copy global -> shared (16-byte aligned, a multiple of 16 bytes), completing on a shared-memory barrier.
-__device__ __forceinline__ void bulk_copy(void* dst, const void* src, uint32_t bytes, unsigned long long* bar) {
+__device__ __forceinline__ void bulk_copy(uint32_t dst, const void* src, uint32_t bytes, unsigned long long* bar) {
     asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
-                 ::"r"(smem_u32(dst)), "l"(src), "r"(bytes), "r"(smem_u32(bar)) : "memory");
+                 ::"r"(dst), "l"(src), "r"(bytes), "r"(smem_u32(bar)) : "memory");
 }
 // Tiled bulk-tensor copy of the box at (column k, token n) of the X tensor map.
 __device__ __forceinline__ void tensor_copy(void* dst, const CUtensorMap* map, int k, int n, unsigned long long* bar) {
     asm volatile("cp.async.bulk.tensor.2d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];"
                  ::"r"(smem_u32(dst)), "l"(reinterpret_cast<uint64_t>(map)), "r"(k), "r"(n), "r"(smem_u32(bar)) : "memory");
 }
+
+
+template <int kOff>
+__device__ __forceinline__ unsigned lds_at(uint32_t addr) {
+    unsigned v;
+    asm volatile("ld.shared.u32 %0, [%1+%2];" : "=r"(v) : "r"(addr), "n"(kOff));
+    return v;
+}
+__device__ __forceinline__ void sts_v2(uint32_t addr, unsigned a, unsigned b) {
+    asm volatile("st.shared.v2.u32 [%0], {%1, %2};" ::"r"(addr), "r"(a), "r"(b) : "memory");
+}
+__device__ __forceinline__ unsigned permute(unsigned a, unsigned b, unsigned sel) {
+    unsigned r;
+    asm("prmt.b32 %0, %1, %2, %3;" : "=r"(r) : "r"(a), "r"(b), "r"(sel));
+    return r;
+}
+
+// Scan of 4 columns: lane (q, w) = (lane / 8, lane % 8) counts bitmap word w of column j0 + q; an 8-lane prefix sum
+// gives the shared-memory address of the word's first value, stored beside the word in the warp's table.  start[g] =
+// address of the first value of the g-th GTile, ngt = GTiles that exist, limit = values that are there.
+__device__ __forceinline__ void scan4(const Params& p, const uint32_t (*bm)[8], const uint32_t* ci, const uint32_t* start, int ngt,
+                                      uint32_t limit, int j0, int lane, uint2* tab) {
+    const int q = lane >> 3, w = lane & 7, j = j0 + q;
+    unsigned word = 0u, first = start[0];
+    if ((j >> 4) < ngt) {
+        const uint32_t ciw = ci[j];
+        word = bm[j][w];
+        first = start[j >> 4] + 2u * (ciw >> 16);
+        if (!SPDP_CHECK(p.status, (first - start[0]) / 2u, ciw & 0xFFFFu, limit, kSiteValuesSpan)) {   // checked build only
+            word = 0u;
+            first = start[0];
+        }
+    }
+    const unsigned cnt = __popc(word);
+    unsigned inc = cnt;
+    scan8_level<1>(inc);
+    scan8_level<2>(inc);
+    scan8_level<4>(inc);
+    tab[lane] = make_uint2(word, first + 2u * (inc - cnt));
+}
+
+// Expands kSteps x 128 rows into the operand tile: step q is row half q % kHalves of column q / kHalves.  A lane takes
+// nibble lane % 8 (bits sh .. sh + 3, `below` = the bits under them) of word lane / 8 of the half; tab_l points at that
+// word's table entry of column 0 (half 0), a_dst at the lane's place in the operand tile, half_bytes further is the next
+// half's tile, 16 bytes further the next column (at most 8: one k-group).  The loads of 4 steps are issued together; they
+// may reach 12 bytes past the stored values.  What bounds it is shared memory: 2 wavefronts for the table, one or two for
+// each value load, 2 for the store.  (Selectors from a 16-entry table in shared memory instead of the two multiplications
+// cost 2 more wavefronts per step and 3 % on the whole kernel.)
+template <int kSteps, int kHalves>
+__device__ __forceinline__ void expand4(uint32_t tab_l, uint32_t a_dst, uint32_t half_bytes, unsigned below, unsigned sh) {
+    static_assert(kSteps % 4 == 0 && kSteps / kHalves <= 8, "4 steps at a time, one k-group");
+#pragma unroll
+    for (int q0 = 0; q0 < kSteps; q0 += 4) {
+        unsigned a[4], s0[4], s1[4], s2[4], bits[4];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            const uint2 v = lds_v2(tab_l + 64u * ((q0 + q) / kHalves) + 32u * ((q0 + q) % kHalves));
+            a[q] = v.y + 2u * __popc(v.x & below);              // address of my nibble's first value (a multiple of 2)
+            bits[q] = (((v.x >> sh) & 15u) * 0x00204081u) & 0x01010101u;        // bit i of the nibble -> byte i
+        }
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            const uint32_t al = a[q] & ~3u;
+            s0[q] = lds_at<0>(al);
+            s1[q] = lds_at<4>(al);
+            s2[q] = lds_at<8>(al);
+        }
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            const unsigned mis = a[q] << 3;                     // 16 if the first value is an upper half (mod 32)
+            const unsigned t0 = __funnelshift_r(s0[q], s1[q], mis), t1 = __funnelshift_r(s1[q], s2[q], mis);
+            // byte i: 0x22 * (set bits before row i) + 0x10 = the two byte selectors of row i's value
+            const unsigned sel = bits[q] * 0x22222200u + 0x10101010u;
+            const unsigned m = bits[q] * 0xFFu;
+            sts_v2(a_dst + ((q0 + q) % kHalves) * half_bytes + ((q0 + q) / kHalves) * 16u, permute(t0, t1, sel) & permute(m, m, 0x1100u),
+                   permute(t0, t1, sel >> 16) & permute(m, m, 0x3322u));
+        }
+    }
+}
+
+// Accumulators of one tile: tensor-memory lanes [lane_base, +32) x columns [c_begin, c_end) of the tile's tokens (first
+// token n0).  A thread holds one row, 16 tokens at a time, so a warp's stores of one token are 32 consecutive rows.  With
+// slot >= 0 they go, as fp32, into that slot of the scratch memory instead of Y.  The whole warp calls this together.
+__device__ __forceinline__ void store_accumulators(const Params& p, uint32_t tmem, int lane_base, int c_begin, int c_end,
+                                                   int r, int row_in, int64_t n0, int slot) {
+    const int64_t row = static_cast<int64_t>(r) * kTileM + row_in;
+    const int valid = static_cast<int>(min(p.N - n0, static_cast<int64_t>(c_end)));
+    float* part = p.partial + (static_cast<size_t>(slot < 0 ? 0 : slot) * p.ptok) * kTileM + row_in;
+    for (int c0 = c_begin; c0 < valid; c0 += 16) {
+        uint32_t v[16];
+        asm volatile("tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%16];"
+                     : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7]),
+                       "=r"(v[8]), "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]), "=r"(v[14]), "=r"(v[15])
+                     : "r"(tmem + (static_cast<uint32_t>(lane_base) << 16) + c0) : "memory");
+        asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+        if (slot >= 0) {
+#pragma unroll
+            for (int i = 0; i < 16; ++i)
+                if (c0 + i < valid) part[static_cast<size_t>(c0 + i) * kTileM] = __uint_as_float(v[i]);
+        } else if (row < p.M) {
+#pragma unroll
+            for (int i = 0; i < 16; ++i)
+                if (c0 + i < valid) store_y(p.Y, p.ydt, (n0 + c0 + i) * p.ldy + row, __uint_as_float(v[i]));
+        }
+        __syncwarp();
+    }
+}
+
+// ===================================================================================================
+namespace one {     // one CTA = one row tile x kNI tokens
+
+template <int kNIT>
+struct Form {
+    static constexpr int kNI = kNIT;                                  // the N of the tensor-core instruction = tokens per tile
+    static constexpr int kTmemCols = 2 * kNI;                         // two accumulators: the row halves
+    static constexpr int kBBytes = kNI * kBRowBytes;
+    static constexpr int kATileBytes = (kSub / 8) * kAKGroupStride;   // 128 rows x kSub columns
+    static constexpr int kABytes = 2 * kATileBytes;
+    static constexpr int kAStages = 4;                                // decoded sub-blocks
+    static constexpr int kBStages = kNI <= 128 ? 3 : 2;
+    static constexpr int kMeta = 8;                                   // stored K-blocks in flight, at most
+    static_assert(kBBytes % 1024 == 0, "every X tile on a swizzle-atom boundary");
+};
+
+// CTA w's share of the tiles that are cut along K: K-blocks [rest_begin(w), rest_begin(w + 1)).
+__device__ __forceinline__ unsigned rest_begin(const Params& p, unsigned w) {
+    return static_cast<unsigned>(static_cast<unsigned long long>(p.rest_units) * w / static_cast<unsigned>(p.sharers));
+}
+// The CTA whose share holds K-block u of them.
+__device__ __forceinline__ unsigned rest_owner(const Params& p, unsigned u) {
+    const unsigned long long num = static_cast<unsigned long long>(u + 1u) * static_cast<unsigned>(p.sharers) + p.rest_units - 1u;
+    return static_cast<unsigned>(num / p.rest_units) - 1u;
+}
+// The k-th piece of CTA w's work: K-blocks [kb0, kb0 + n) of a tile; slot = where its partial sums go, -1: the
+// piece is the whole tile.  (A CTA's range of the shared part is no longer than a tile, so it is one or two pieces.)
+struct Piece { int tile, kb0, n, slot; };
+__device__ __forceinline__ bool piece(const Params& p, int w, int k, Piece& s) {
+    if (k < p.rounds) {
+        s.tile = k * p.workers + w;
+        s.kb0 = 0;
+        s.n = p.nkb;
+        s.slot = -1;
+        return true;
+    }
+    if (w >= p.sharers || p.rest_units == 0u) return false;
+    const unsigned u0 = rest_begin(p, w), u1 = rest_begin(p, w + 1);
+    const unsigned nkb = static_cast<unsigned>(p.nkb);
+    const unsigned t0 = u0 / nkb, t = t0 + static_cast<unsigned>(k - p.rounds);
+    const unsigned lo = max(u0, t * nkb), hi = min(u1, (t + 1u) * nkb);
+    if (lo >= hi) return false;
+    s.tile = p.rounds * p.workers + static_cast<int>(t);
+    s.kb0 = static_cast<int>(lo - t * nkb);
+    s.n = static_cast<int>(hi - lo);
+    s.slot = (s.n == p.nkb) ? -1 : 2 * w + (t != t0 ? 1 : 0);
+    return true;
+}
+
+struct alignas(16) Meta {                       // a K-block as stored, without its values
+    alignas(16) uint32_t bm[kKB][8];            // bitmaps
+    alignas(16) uint32_t ci[kKB];               // ColInfo words
+    uint32_t start[kGTB];                       // shared-memory address of each GTile's first value
+    uint32_t limit;                             // (checked build) values of the K-block
+    uint32_t vstart;                            // copy warp: virtual ring offset of its values
+    int ngt;                                    // GTiles it really has
+};
+
+template <class F>
+struct __align__(1024) Smem {
+    unsigned char B[F::kBStages][F::kBBytes];       // X tiles (each on a 1024-byte boundary: swizzle atoms)
+    unsigned char A[F::kAStages][F::kABytes];       // decoded W
+    Meta meta[F::kMeta];
+    alignas(16) uint2 tab[kWarps][32];              // per warp: bitmap word and the address of its first value
+    alignas(8) unsigned long long comp_full[F::kMeta];  // the stored K-block has arrived
+    alignas(8) unsigned long long comp_free[F::kMeta];  // the decode warps are done with it
+    alignas(8) unsigned long long a_ready[F::kAStages]; // A stage is written
+    alignas(8) unsigned long long a_free[F::kAStages];  // the tensor cores are done with it
+    alignas(8) unsigned long long x_full[F::kBStages];  // the X tile has arrived
+    alignas(8) unsigned long long x_free[F::kBStages];  // the tensor cores are done with it
+    alignas(8) unsigned long long acc_full;         // the piece's products are complete
+    alignas(8) unsigned long long acc_free;         // its accumulators have been stored
+    alignas(8) unsigned long long drained;          // every product that was issued is complete
+    uint32_t tmem_base;
+    int abort;
+    alignas(128) unsigned char ring[1];             // values of the K-blocks in flight (fills the rest): the sparser the
+                                                    // matrix, the more K-blocks are on their way
+};
+constexpr uint32_t kSmemBytes = 227u * 1024u;       // the dynamic shared memory is aligned by hand
+template <class F>
+constexpr uint32_t kRingBytes = (kSmemBytes - 1024u - static_cast<uint32_t>(offsetof(Smem<F>, ring)) - 64u) / 128u * 128u;
+
+template <class F>
+__global__ void __launch_bounds__(kThreads, 1)
+spmm_kernel(const __grid_constant__ Params p, const __grid_constant__ CUtensorMap xmap) {
+    static_assert(kRingBytes<F> >= 2 * kKB * kTileM * 2, "the ring holds at least two full K-blocks");
+    extern __shared__ unsigned char smem_raw[];
+    Smem<F>& sm = *reinterpret_cast<Smem<F>*>(smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u));
+    const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
+    const int me = static_cast<int>(blockIdx.x);
+
+    // ---- set-up: the barriers and tensor memory ----
+    if (t == 0) {
+#pragma unroll
+        for (int s = 0; s < F::kMeta; ++s) {
+            barrier_init(&sm.comp_full[s], 1);
+            barrier_init(&sm.comp_free[s], kBlockWarps);
+        }
+#pragma unroll
+        for (int s = 0; s < F::kAStages; ++s) {
+            barrier_init(&sm.a_ready[s], kGroupWarps);
+            barrier_init(&sm.a_free[s], 1);
+        }
+#pragma unroll
+        for (int s = 0; s < F::kBStages; ++s) {
+            barrier_init(&sm.x_full[s], 1);
+            barrier_init(&sm.x_free[s], 1);
+        }
+        barrier_init(&sm.acc_full, 1);
+        barrier_init(&sm.acc_free, kStoreWarps);
+        barrier_init(&sm.drained, 1);
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+        sm.abort = 0;
+    }
+    __syncwarp();
+    if (warp == 1) {
+        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;"
+                     ::"r"(smem_u32(&sm.tmem_base)), "n"(F::kTmemCols) : "memory");
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+    }
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+    __syncthreads();
+    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+    const uint32_t tmem = sm.tmem_base;
+    // A wait that runs out (it never should) clears `ok`: the thread's role ends, the others' waits run out in turn, the
+    // status word gets SPDP_ERR_TIMEOUT and the outputs stay unwritten.  No bounded wait covers the time of the kernel
+    // before this one in the stream: whatever depends on X first waits for that kernel (griddepcontrol.wait).
+    bool ok = true;
+    Piece s;
+
+    if (warp == kWarps) {
+        // ================= tensor-core warp: one thread issues the products =================
+        if (elect_one()) {
+            unsigned i = 0, u = 0;                                      // sub-blocks and K-blocks so far
+            bool issued = false;
+            asm volatile("griddepcontrol.wait;" ::: "memory");
+            for (int k = 0; ok && piece(p, me, k, s); ++k) {
+                if (k > 0) {
+                    ok = wait_parity(&sm.acc_free, (k - 1) & 1);
+                    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+                }
+                for (int kb = 0; ok && kb < s.n; ++kb, ++u) {
+                    const unsigned sb = u % F::kBStages;
+                    ok = wait_parity(&sm.x_full[sb], (u / F::kBStages) & 1);                    // the X tile is in place
+                    for (int h = 0; ok && h < kSubs; ++h, ++i) {
+                        const unsigned sa = i % F::kAStages;
+                        ok = wait_parity(&sm.a_ready[sa], (i / F::kAStages) & 1);               // the decoded W is in place
+                        if (!ok) break;
+                        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+                        const uint64_t ad0 = operand_desc(smem_u32(&sm.A[sa][0]), kAKGroupStride, kAChunkStride, 0u);
+                        const uint64_t bd0 = operand_desc(smem_u32(&sm.B[sb][0]), 16, kBAtomBytes, 2u) + ((h * 2 * kSub) >> 4);
+#pragma unroll
+                        for (int a = 0; a < 2; ++a) {                   // the two row halves
+#pragma unroll
+                            for (int kk = 0; kk < kSub / 16; ++kk)      // the start address is the low field, in 16-byte units
+                                mma_f16_one<F::kNI>(tmem + a * F::kNI, ad0 + ((a * F::kATileBytes + kk * 2 * kAKGroupStride) >> 4),
+                                                    bd0 + ((kk * 32) >> 4), kb > 0 || h > 0 || kk > 0);
+                        }
+                        commit_one(&sm.a_free[sa]);
+                        issued = true;
+                    }
+                    if (ok) commit_one(&sm.x_free[sb]);
+                }
+                if (ok) commit_one(&sm.acc_full);
+            }
+            if (issued) {                                               // tensor memory is not freed under running products
+                commit_one(&sm.drained);
+                ok = wait_parity(&sm.drained, 0u) && ok;
+            }
+        }
+        __syncwarp();           // the other lanes wait here, not on a barrier in shared memory
+    } else if (warp == kWarps + 1) {
+        // ================= copy warp: moves the stored K-blocks =================
+        // The lanes hold the TileOffset words of 32 K-blocks (and of the next 32) and walk them together; one lane issues.
+        unsigned i = 0, done = 0;                                       // K-blocks started / known to be decoded
+        uint32_t vhead = 0, vtail = 0, pos = 0;                         // virtual ring offsets, and vhead's position in the ring
+        const uint32_t ring = smem_u32(&sm.ring[0]);
+        for (int k = 0; piece(p, me, k, s); ++k) {
+            const int64_t g_row = static_cast<int64_t>(s.tile / p.nblocks) * p.C;
+            uint32_t cur[kGTB + 1], nxt[kGTB + 1];
+            auto fetch = [&](int b, uint32_t (&o)[kGTB + 1]) {          // words of K-block kb0 + b + lane: its GTiles and the one after
+                const int g0 = (s.kb0 + b + lane) * kGTB;
+#pragma unroll
+                for (int q = 0; q <= kGTB; ++q) o[q] = (b + lane < s.n) ? __ldg(p.tileoffset + g_row + min(g0 + q, p.C)) : 0u;
+            };
+            fetch(0, cur);
+            for (int b = 0; b < s.n; b += 32) {
+                fetch(b + 32, nxt);
+                const int lim = min(32, s.n - b);
+                for (int q = 0; q < lim; ++q, ++i) {
+                    uint32_t to[kGTB + 1];
+#pragma unroll
+                    for (int e = 0; e <= kGTB; ++e) to[e] = __shfl_sync(0xFFFFFFFFu, cur[e], q);
+                    const int g0 = (s.kb0 + b + q) * kGTB;
+                    const int ngt = min(kGTB, p.C - g0);
+                    const uint32_t nvals = to[kGTB] - to[0];
+                    if (to[kGTB] < to[0] || nvals > static_cast<uint32_t>(kKB * kTileM) ||
+                        static_cast<int64_t>(to[kGTB]) > p.values_len) {                // not what the format says
+                        atomicCAS(p.status, 0, SPDP_ERR_OVERFLOW);
+                        *static_cast<volatile int*>(&sm.abort) = 1;                     // the outputs stay unwritten
+                        ok = false;
+                    }
+                    const uint32_t bytes = ok ? 2u * nvals : 0u;
+                    if (pos + bytes > kRingBytes<F>) {                  // the values of a K-block stay in one piece
+                        vhead += kRingBytes<F> - pos;
+                        pos = 0;
+                    }
+                    while (i - done >= F::kMeta || vhead + bytes - vtail > kRingBytes<F>) {
+                        if (done == i) { vtail = vhead; continue; }
+                        if (done == 0u) asm volatile("griddepcontrol.wait;" ::: "memory");      // the decode waits for products, these for X
+                        if (ok) ok = wait_parity(&sm.comp_free[done % F::kMeta], (done / F::kMeta) & 1);
+                        ++done;
+                        vtail = done < i ? sm.meta[done % F::kMeta].vstart : vhead;
+                    }
+                    ok = __all_sync(0xFFFFFFFFu, ok);
+                    const unsigned m = i % F::kMeta;
+                    Meta& mt = sm.meta[m];
+                    if (elect_one()) {
+                        mt.vstart = vhead;
+                        mt.ngt = ok ? ngt : 0;                          // after a failure nothing is copied any more
+                        mt.limit = nvals;
+#pragma unroll
+                        for (int e = 0; e < kGTB; ++e) mt.start[e] = ring + pos + (ok ? 2u * (to[e] - to[0]) : 0u);
+                        if (ok) {
+                            expect_bytes(&sm.comp_full[m], bytes + static_cast<uint32_t>(ngt) * (kTileK * 32u + kTileK * 4u));
+                            bulk_copy(smem_u32(&mt.bm[0][0]), p.bitmap + (g_row + g0) * kTileK * 4, static_cast<uint32_t>(ngt) * kTileK * 32u, &sm.comp_full[m]);
+                            bulk_copy(smem_u32(&mt.ci[0]), p.colinfo + (g_row + g0) * kTileK, static_cast<uint32_t>(ngt) * kTileK * 4u, &sm.comp_full[m]);
+                            if (bytes) bulk_copy(ring + pos, p.values + to[0], bytes, &sm.comp_full[m]);
+                        } else {
+                            arrive(&sm.comp_full[m]);
+                        }
+                    }
+                    __syncwarp();
+                    vhead += ok ? bytes : 0u;
+                    pos += ok ? bytes : 0u;
+                }
+#pragma unroll
+                for (int q = 0; q <= kGTB; ++q) cur[q] = nxt[q];
+            }
+        }
+        // before the CTA may leave, every copy that was started has arrived
+        for (unsigned q = (i > F::kMeta ? i - F::kMeta : 0u); q < i; ++q) ok = wait_parity(&sm.comp_full[q % F::kMeta], (q / F::kMeta) & 1) && ok;
+        __syncwarp();
+    } else if (warp == kWarps + 2) {
+        // ================= X warp: one thread moves the X tiles =================
+        if (elect_one()) {
+            asm volatile("griddepcontrol.wait;" ::: "memory");          // X may come from the kernel before this one
+            unsigned u = 0;
+            for (int k = 0; piece(p, me, k, s); ++k) {
+                const int n0 = (s.tile % p.nblocks) * F::kNI;
+                for (int kb = 0; kb < s.n; ++kb, ++u) {
+                    const unsigned sb = u % F::kBStages;
+                    if (u >= F::kBStages && ok) ok = wait_parity(&sm.x_free[sb], (u / F::kBStages - 1u) & 1);
+                    if (!ok) { arrive(&sm.x_full[sb]); continue; }
+                    expect_bytes(&sm.x_full[sb], F::kBBytes);
+                    tensor_copy(&sm.B[sb][0], &xmap, (s.kb0 + kb) * kKB, n0, &sm.x_full[sb]);
+                }
+            }
+            for (unsigned q = (u > F::kBStages ? u - F::kBStages : 0u); q < u; ++q) ok = wait_parity(&sm.x_full[q % F::kBStages], (q / F::kBStages) & 1) && ok;
+        }
+        __syncwarp();
+    } else {
+        // ================= decode warps =================
+        const unsigned group = static_cast<unsigned>(warp) / kGroupWarps, wm = static_cast<unsigned>(warp) % kGroupWarps;
+        const unsigned sh = pinned(4u * (lane & 7)), below = pinned((1u << sh) - 1u);
+        const uint32_t tab_l = pinned(smem_u32(&sm.tab[warp][0]) + 8u * (lane >> 3));
+        const uint32_t a_lane = pinned(smem_u32(&sm.A[0][0]) + (lane >> 1) * kAChunkStride + (lane & 1) * 8 +
+                                       (wm >> 1) * kAKGroupStride + (wm & 1u) * 64u);
+        unsigned i0 = 0;                                                // sub-blocks before this piece
+        for (int k = 0; ok && piece(p, me, k, s); ++k) {
+            const unsigned i1 = i0 + static_cast<unsigned>(s.n) * kSubs;
+            for (unsigned i = i0 + (group + kGroups - i0 % kGroups) % kGroups; i < i1; i += kGroups) {
+                const unsigned u = i / kSubs, m = u % F::kMeta, sa = i % F::kAStages;
+                ok = wait_parity(&sm.comp_full[m], (u / F::kMeta) & 1);                          // the stored K-block has arrived
+                __syncwarp();
+                const Meta& mt = sm.meta[m];
+                scan4(p, mt.bm, mt.ci, mt.start, mt.ngt, mt.limit, static_cast<int>((i % kSubs) * kSub + 4u * wm), lane, &sm.tab[warp][0]);
+                __syncwarp();
+                if (i >= F::kAStages) {
+                    if (i < 2 * F::kAStages) asm volatile("griddepcontrol.wait;" ::: "memory");  // the products wait for X
+                    ok = wait_parity(&sm.a_free[sa], (i / F::kAStages - 1u) & 1) && ok;          // the tensor cores are done with this A stage
+                }
+                ok = __all_sync(0xFFFFFFFFu, ok);
+                if (!ok) break;
+                expand4<8, 2>(tab_l, a_lane + sa * F::kABytes, F::kATileBytes, below, sh);
+                // the operand tile was written through the generic proxy; the tensor cores read through the async proxy
+                asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+                __syncwarp();
+                if (lane == 0) {
+                    arrive(&sm.a_ready[sa]);
+                    arrive(&sm.comp_free[m]);
+                }
+            }
+            i0 = i1;
+            if (warp >= kStoreWarps) continue;
+            // ---- the piece's products are complete: store the accumulators ----
+            asm volatile("griddepcontrol.wait;" ::: "memory");          // Y and the scratch may belong to the kernel before this one
+            if (ok) ok = wait_parity(&sm.acc_full, k & 1);
+            asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+            ok = __all_sync(0xFFFFFFFFu, ok);
+            if (ok && !__any_sync(0xFFFFFFFFu, *static_cast<volatile int*>(&sm.abort) != 0)) {
+                // warp w: row half (w / 4) % 2, tensor-memory lanes 32 * (w % 4).., token columns [(w / 8) * kNI / 2, + kNI / 2)
+                const int half = (warp >> 2) & 1, cbase = (warp >> 3) * (F::kNI / 2), lane_base = 32 * (warp & 3);
+                store_accumulators(p, tmem + half * F::kNI, lane_base, cbase, cbase + F::kNI / 2, s.tile / p.nblocks,
+                                   half * 128 + lane_base + lane, static_cast<int64_t>(s.tile % p.nblocks) * F::kNI, s.slot);
+            }
+            asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+            __syncwarp();
+            if (lane == 0) arrive(&sm.acc_free);
+            __syncwarp();
+        }
+    }
+    if (!ok) {
+        *static_cast<volatile int*>(&sm.abort) = 1;
+        atomicCAS(p.status, 0, SPDP_ERR_TIMEOUT);
+    }
+    __syncwarp();
+    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+    __syncthreads();
+    if (warp == 1)
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "n"(F::kTmemCols) : "memory");
+}
+
+// Adds, in CTA order, the partial sums of the tiles that several CTAs fed, and writes their part of Y.  A thread takes 4
+// consecutive rows of one token.
+__global__ void __launch_bounds__(256)
+reduce_pieces_kernel(const Params p, int tile0, int tiles, int tile_tokens) {
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    const int64_t total = static_cast<int64_t>(tiles) * p.ptok * (kTileM / 4);
+    const unsigned nkb = static_cast<unsigned>(p.nkb);
+    for (int64_t i = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x; i < total;
+         i += static_cast<int64_t>(gridDim.x) * blockDim.x) {
+        const int row_in = 4 * static_cast<int>(i % (kTileM / 4));
+        const int64_t q = i / (kTileM / 4);
+        const int tok = static_cast<int>(q % p.ptok);
+        const unsigned t = static_cast<unsigned>(q / p.ptok);            // tile tile0 + t
+        const unsigned first = rest_owner(p, t * nkb), last = rest_owner(p, (t + 1u) * nkb - 1u);
+        if (first == last) continue;                                     // one CTA had the whole tile: it stored Y itself
+        const int tile = tile0 + static_cast<int>(t);
+        const int64_t n = static_cast<int64_t>(tile % p.nblocks) * tile_tokens + tok;
+        const int64_t row = static_cast<int64_t>(tile / p.nblocks) * kTileM + row_in;
+        if (n >= p.N || row >= p.M) continue;
+        float4 sum = make_float4(0.f, 0.f, 0.f, 0.f);
+        for (unsigned w = first; w <= last; ++w) {
+            const unsigned slot = 2u * w + (rest_begin(p, w) / nkb != t ? 1u : 0u);
+            const float4 v = *reinterpret_cast<const float4*>(p.partial + (static_cast<size_t>(slot) * p.ptok + tok) * kTileM + row_in);
+            sum.x += v.x;
+            sum.y += v.y;
+            sum.z += v.z;
+            sum.w += v.w;
+        }
+        const float v[4] = {sum.x, sum.y, sum.z, sum.w};
+#pragma unroll
+        for (int e = 0; e < 4; ++e)
+            if (row + e < p.M) store_y(p.Y, p.ydt, n * p.ldy + row + e, v[e]);
+    }
+}
+
+}  // namespace one
+
+// ===================================================================================================
+namespace pair {    // two CTAs (a cluster of 2) = one row tile x 512 tokens
+
+constexpr int kNI = 256;                      // the N of the tensor-core instruction
+constexpr int kTmemCols = 512;
+constexpr int kATileBytes = (kKB / 8) * kAKGroupStride;    // 128 rows x kKB columns
+constexpr int kCompValues = kKB * kTileM;     // the most values a K-block stores
+constexpr int kNTiles = 2;                    // accumulators per CTA
+constexpr int kNT = kNTiles * kNI;            // tokens per CTA pair
+constexpr int kStages = 3;                    // operand tiles (decoded W, X) in flight
+constexpr int kCStages = 2;                   // stored K-blocks in flight
+constexpr int kBTileBytes = (kNI / 2) * kBRowBytes;    // this CTA's 128 tokens of one X tile
+constexpr int kBBytes = kNTiles * kBTileBytes;
+static_assert(kNTiles * kNI == kTmemCols, "the accumulators fill tensor memory");
+
+struct CompStage {                              // one K-block as stored
+    alignas(128) unsigned short vals[kCompValues + 16];   // the values of its 4 GTiles, contiguous
+    alignas(16) uint32_t bm[kKB][8];            // bitmaps
+    alignas(16) uint32_t ci[kKB];               // ColInfo words
+    uint32_t start[kGTB];                       // shared-memory address of each GTile's first value
+    uint32_t limit;                             // (checked build) values of the block
+};
+static_assert(offsetof(CompStage, bm) % 16 == 0 && offsetof(CompStage, ci) % 16 == 0 && sizeof(CompStage) % 16 == 0,
+              "bulk copies need 16-byte aligned destinations");
 
 // TileOffset words of K-block kb of row tile r: its GTiles and the one after (Sec. 4.1); a short last block
 // repeats its end.
@@ -195,278 +712,14 @@ __device__ __forceinline__ bool load_comp(const Params& p, int r, int kb, const 
         nvals = 0u;
     }
 #pragma unroll
-    for (int i = 0; i <= kGTB; ++i) cs.to[i] = nvals ? o.to[i] : 0u;
+    for (int i = 0; i < kGTB; ++i) cs.start[i] = smem_u32(&cs.vals[0]) + (nvals ? 2u * (o.to[i] - o.to[0]) : 0u);
+    cs.limit = nvals;
     expect_bytes(bar, 2u * nvals + static_cast<uint32_t>(ngt) * (kTileK * 32u + kTileK * 4u));
-    if (nvals) bulk_copy(&cs.vals[0], p.values + o.to[0], 2u * nvals, bar);
-    bulk_copy(&cs.bm[0][0], p.bitmap + g0 * kTileK * 4, static_cast<uint32_t>(ngt) * kTileK * 32u, bar);
-    bulk_copy(&cs.ci[0], p.colinfo + g0 * kTileK, static_cast<uint32_t>(ngt) * kTileK * 4u, bar);
+    if (nvals) bulk_copy(smem_u32(&cs.vals[0]), p.values + o.to[0], 2u * nvals, bar);
+    bulk_copy(smem_u32(&cs.bm[0][0]), p.bitmap + g0 * kTileK * 4, static_cast<uint32_t>(ngt) * kTileK * 32u, bar);
+    bulk_copy(smem_u32(&cs.ci[0]), p.colinfo + g0 * kTileK, static_cast<uint32_t>(ngt) * kTileK * 4u, bar);
     return good;
 }
-
-// The walk over one bitmap byte (Sec. 4.2.1): `first` = shared-memory address of the byte's first value; a set
-// bit takes the next value, a clear bit leaves a zero.  Returns the 8 rows as 8 fp16.
-#define SPDP_WALK_ROW(R, BIT) \
-    " lop3.or.b32 t|p, %4, " #BIT ", 0, 0xC0, 0;\n @p ld.shared.u16 v" #R ", [a];\n @p add.u32 a, a, 2;\n"
-__device__ __forceinline__ uint4 walk_byte(unsigned bits, uint32_t first) {
-    uint4 o;
-    asm("{\n .reg .pred p;\n .reg .b16 v<8>;\n .reg .b32 t, a;\n mov.u32 a, %5;\n"
-        " mov.b16 v0, 0;\n mov.b16 v1, 0;\n mov.b16 v2, 0;\n mov.b16 v3, 0;\n"
-        " mov.b16 v4, 0;\n mov.b16 v5, 0;\n mov.b16 v6, 0;\n mov.b16 v7, 0;\n"
-        SPDP_WALK_ROW(0, 1) SPDP_WALK_ROW(1, 2) SPDP_WALK_ROW(2, 4) SPDP_WALK_ROW(3, 8)
-        SPDP_WALK_ROW(4, 16) SPDP_WALK_ROW(5, 32) SPDP_WALK_ROW(6, 64)
-        " lop3.or.b32 t|p, %4, 128, 0, 0xC0, 0;\n @p ld.shared.u16 v7, [a];\n"
-        " mov.b32 %0, {v0, v1};\n mov.b32 %1, {v2, v3};\n mov.b32 %2, {v4, v5};\n mov.b32 %3, {v6, v7};\n}"
-        : "=r"(o.x), "=r"(o.y), "=r"(o.z), "=r"(o.w) : "r"(bits), "r"(first));
-    return o;
-}
-#undef SPDP_WALK_ROW
-
-// One scan for the warp's 4 columns (warp, warp + 16, +32, +48) of the K-block in `cs`: lane (q, w) = (lane / 8,
-// lane % 8) counts bitmap word w of column q, and an 8-lane prefix sum gives the index, inside the stage, of the
-// word's first value (the column's start = its GTile's TileOffset relative to the block's first + its ColInfo
-// offset, Sec. 4.1).  `ngt` = GTiles the block really has; the columns of the others are empty.
-__device__ __forceinline__ void scan_columns(const Params& p, const CompStage& cs, int ngt, int warp, int lane,
-                                             unsigned& w8, unsigned& base_w) {
-    const int q = lane >> 3, w = lane & 7;
-    const int jq = warp + kWarps * q;
-    unsigned start = 0u;
-    w8 = 0u;
-    if ((jq >> 4) < ngt) {
-        const uint32_t ciw = cs.ci[jq];
-        start = cs.to[jq >> 4] - cs.to[0] + (ciw >> 16);
-        w8 = cs.bm[jq][w];
-        if (!SPDP_CHECK(p.status, start, ciw & 0xFFFFu, cs.to[ngt] - cs.to[0], kSiteValuesSpan)) w8 = 0u;   // checked build only
-    }
-    const unsigned cnt = __popc(w8);
-    unsigned inc = cnt;
-    scan8_level<1>(inc);
-    scan8_level<2>(inc);
-    scan8_level<4>(inc);
-    base_w = start + inc - cnt;
-}
-
-// Epilogue of both kernels: tensor-memory lanes [lane_base, +32) x columns [c_begin, c_end) -> Y rows `row`,
-// tokens n0 + column.  A thread holds one row, 16 tokens at a time, so a warp's stores of one token are 32
-// consecutive rows.
-__device__ __forceinline__ void store_accumulators(const Params& p, uint32_t tmem, int lane_base, int c_begin, int c_end,
-                                                   int64_t row, int64_t n0) {
-    for (int c0 = c_begin; c0 < c_end; c0 += 16) {
-        if (n0 + c0 >= p.N) break;                                          // warp-uniform
-        uint32_t v[16];
-        asm volatile("tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%16];"
-                     : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7]),
-                       "=r"(v[8]), "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]), "=r"(v[14]), "=r"(v[15])
-                     : "r"(tmem + (static_cast<uint32_t>(lane_base) << 16) + c0) : "memory");
-        asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-        if (row < p.M) {
-#pragma unroll
-            for (int i = 0; i < 16; ++i) {
-                const int64_t n = n0 + c0 + i;
-                if (n < p.N) store_y(p.Y, p.ydt, n * p.ldy + row, __uint_as_float(v[i]));
-            }
-        }
-    }
-}
-
-// The same for a slice of K: the accumulators go, as fp32, to dst[column * 256 + row] (row = my row inside the row tile).
-__device__ __forceinline__ void store_partial(float* dst, uint32_t tmem, int lane_base, int c_begin, int c_end, int row,
-                                              int valid_columns) {
-    for (int c0 = c_begin; c0 < c_end; c0 += 16) {
-        if (c0 >= valid_columns) break;                                     // warp-uniform
-        uint32_t v[16];
-        asm volatile("tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%16];"
-                     : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7]),
-                       "=r"(v[8]), "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]), "=r"(v[14]), "=r"(v[15])
-                     : "r"(tmem + (static_cast<uint32_t>(lane_base) << 16) + c0) : "memory");
-        asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-#pragma unroll
-        for (int i = 0; i < 16; ++i)
-            if (c0 + i < valid_columns) dst[static_cast<size_t>(c0 + i) * kTileM + row] = __uint_as_float(v[i]);
-    }
-}
-
-// ===================================================================================================
-namespace one {     // one CTA = one row tile x 256 tokens
-
-constexpr int kThreads = (kWarps + 2) * 32;   // decode warps + the tensor-core warp + the copy warp
-constexpr int kNT = kNI;                      // tokens per CTA
-constexpr int kStages = 2;
-constexpr int kBBytes = kNT * kBRowBytes;
-
-struct __align__(1024) Smem {
-    unsigned char B[kStages][kBBytes];              // X tiles (each stage starts on a 1024-byte boundary: swizzle atoms)
-    unsigned char A[kStages][2][kATileBytes];       // decoded W, two 128-row tiles per stage
-    CompStage comp[kStages];
-    alignas(8) unsigned long long mma_done[kStages];    // the tensor cores are done with A stage s and B stage s
-    alignas(8) unsigned long long a_ready[kStages];     // the decode warps have written A stage s (and read comp stage s)
-    alignas(8) unsigned long long x_full[kStages];      // the X tile of B stage s has arrived
-    alignas(8) unsigned long long comp_full[kStages];   // the stored K-block of comp stage s has arrived
-    uint32_t tmem_base;
-    int abort;
-};
-constexpr size_t kSmemBytes = sizeof(Smem) + 1024;      // the dynamic shared memory is aligned by hand
-static_assert(kSmemBytes <= 227 * 1024, "shared memory of one CTA");
-static_assert(kBBytes % 1024 == 0, "every B stage on a swizzle-atom boundary");
-
-// Decodes the warp's 4 columns into the operand tiles at `a_stage`: per column, a lane owns the 8 rows of bitmap
-// byte `lane`, fetches its word and the index of the word's first value from the scan lane, adds the set bits
-// below its byte (its rank, Sec. 4.2.1) and walks the byte.
-__device__ __forceinline__ void decode_block(const Params& p, const CompStage& cs, int ngt, int warp, int lane,
-                                             unsigned char* a_stage) {
-    unsigned w8, base_w;
-    scan_columns(p, cs, ngt, warp, lane, w8, base_w);
-    const int sh = 8 * (lane & 3);
-    const unsigned below = (1u << sh) - 1u;
-    const uint32_t vals = smem_u32(&cs.vals[0]);
-    uint4 piece[4];
-#pragma unroll
-    for (int qq = 0; qq < 4; ++qq) {
-        const unsigned word = __shfl_sync(0xFFFFFFFFu, w8, 8 * qq + (lane >> 2));
-        const unsigned base = __shfl_sync(0xFFFFFFFFu, base_w, 8 * qq + (lane >> 2));
-        const unsigned bits = (word >> sh) & 0xFFu;
-        piece[qq] = walk_byte(bits, vals + 2u * (base + __popc(word & below)));
-    }
-    // the stores come after all four walks, so that the walks' loads are free to overlap
-    unsigned char* mine = a_stage + (lane >> 4) * kATileBytes + (lane & 15) * kAChunkStride;
-#pragma unroll
-    for (int qq = 0; qq < 4; ++qq) {
-        const int j = warp + kWarps * qq;
-        *reinterpret_cast<uint4*>(mine + (j >> 3) * kAKGroupStride + (j & 7) * 16) = piece[qq];
-    }
-}
-
-__global__ void __launch_bounds__(kThreads, 1)
-spmm_kernel(const __grid_constant__ Params p, const __grid_constant__ CUtensorMap xmap) {
-    extern __shared__ unsigned char smem_raw[];
-    Smem& sm = *reinterpret_cast<Smem*>(smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u));
-    const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
-    const int r = static_cast<int>(blockIdx.x / static_cast<unsigned>(p.nblocks));
-    const int nb = static_cast<int>(blockIdx.x - static_cast<unsigned>(r) * static_cast<unsigned>(p.nblocks));
-    const int64_t n0 = static_cast<int64_t>(nb) * kNT;
-
-    // ---- set-up: the barriers, and tensor memory ----
-    if (t == 0) {
-#pragma unroll
-        for (int s = 0; s < kStages; ++s) {
-            barrier_init(&sm.mma_done[s], 1);
-            barrier_init(&sm.a_ready[s], kWarps);
-            barrier_init(&sm.x_full[s], 1);
-            barrier_init(&sm.comp_full[s], 1);
-        }
-        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-        sm.abort = 0;
-    }
-    if (warp == 0) {
-        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;"
-                     ::"r"(smem_u32(&sm.tmem_base)), "n"(kTmemCols) : "memory");
-        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
-    }
-    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-    __syncthreads();
-    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-    const uint32_t tmem = sm.tmem_base;
-    const int nkb = (p.C + kGTB - 1) / kGTB;
-    // A wait that runs out (it never should) clears `ok`: the thread then stops waiting but keeps walking the
-    // same barriers as the others, the status word gets SPDP_ERR_TIMEOUT and the outputs stay unwritten.
-    bool ok = true;
-
-    if (warp == kWarps) {
-        // ================= tensor-core warp: one thread issues the K-blocks' products =================
-        if (lane == 0) {
-            for (int kb = 0; kb < nkb; ++kb) {
-                const int s = kb % kStages;
-                const unsigned phase = (kb / kStages) & 1;
-                if (ok) ok = wait_parity(&sm.a_ready[s], phase);         // the decoded W tile is in place
-                if (ok) ok = wait_parity(&sm.x_full[s], phase);          // and so is the X tile
-                asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-                const uint64_t ad0 = operand_desc(smem_u32(&sm.A[s][0][0]), kAKGroupStride, kAChunkStride, 0u);
-                const uint64_t bd0 = operand_desc(smem_u32(&sm.B[s][0]), 16, kBAtomBytes, 2u);
-#pragma unroll
-                for (int h = 0; h < 2; ++h) {
-#pragma unroll
-                    for (int kk = 0; kk < kKB / 16; ++kk)    // the start address is the descriptor's low field, in 16-byte units
-                        mma_f16_one(tmem + h * kNI, ad0 + ((h * kATileBytes + kk * 2 * kAKGroupStride) >> 4), bd0 + ((kk * 32) >> 4),
-                                    kb > 0 || kk > 0);
-                }
-                asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];"
-                             ::"r"(smem_u32(&sm.mma_done[s])) : "memory");
-            }
-        }
-        __syncwarp();           // the other lanes wait here, not on a barrier in shared memory
-    } else if (warp == kWarps + 1) {
-        // ================= copy warp: one thread moves the stored K-blocks and the X tiles =================
-        if (lane == 0) {
-            auto load_x = [&](int kb) {
-                expect_bytes(&sm.x_full[kb % kStages], kBBytes);
-                tensor_copy(&sm.B[kb % kStages][0], &xmap, kb * kKB, static_cast<int>(n0), &sm.x_full[kb % kStages]);
-            };
-            for (int kb = 0; kb < kStages && kb < nkb; ++kb) {
-                ok = load_comp(p, r, kb, fetch_offsets(p, r, nkb, kb), sm.comp[kb % kStages], &sm.comp_full[kb % kStages]) && ok;
-                load_x(kb);
-            }
-            Offsets next = fetch_offsets(p, r, nkb, kStages);
-            for (int kb = 0; kb + kStages < nkb; ++kb) {
-                const int s = kb % kStages;
-                const unsigned phase = (kb / kStages) & 1;
-                // the stored block kb + kStages goes where block kb was decoded from, once every decode warp is done with it
-                if (ok) ok = wait_parity(&sm.a_ready[s], phase);
-                ok = load_comp(p, r, kb + kStages, next, sm.comp[s], &sm.comp_full[s]) && ok;
-                next = fetch_offsets(p, r, nkb, kb + kStages + 1);
-                // the X tile of block kb + kStages goes where block kb multiplies from, once that work is complete
-                if (ok) ok = wait_parity(&sm.mma_done[s], phase);
-                load_x(kb + kStages);
-            }
-        }
-        __syncwarp();
-    } else {
-        // ================= decode warps =================
-        for (int kb = 0; kb < nkb; ++kb) {
-            const int s = kb % kStages;
-            const unsigned phase = (kb / kStages) & 1;
-            if (ok) ok = wait_parity(&sm.comp_full[s], phase);                           // the stored block has arrived
-            if (kb >= kStages && ok) ok = wait_parity(&sm.mma_done[s], phase ^ 1u);     // the tensor cores are done with this A stage
-            decode_block(p, sm.comp[s], min(kGTB, p.C - kGTB * kb), warp, lane, &sm.A[s][0][0]);
-            // the operand tile was written through the generic proxy; the tensor cores read through the async proxy
-            asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-            __syncwarp();
-            if (lane == 0) arrive(&sm.a_ready[s]);
-        }
-    }
-    // the last blocks' tensor-core work
-    for (int kb = (nkb > kStages ? nkb - kStages : 0); ok && kb < nkb; ++kb)
-        ok = wait_parity(&sm.mma_done[kb % kStages], (kb / kStages) & 1);
-    if (!ok) {
-        sm.abort = 1;
-        if (lane == 0) atomicCAS(p.status, 0, SPDP_ERR_TIMEOUT);
-    }
-    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-    __syncthreads();
-
-    // ---- epilogue.  Warp w reads lanes 32*(w%4).. of accumulator (w/4)%2, token columns [(w/8)*128, +128) ----
-    if (!sm.abort && warp < kWarps) {
-        const int half = (warp >> 2) & 1, lane_base = 32 * (warp & 3), cbase = (warp >> 3) * (kNT / 2);
-        store_accumulators(p, tmem + half * kNI, lane_base, cbase, cbase + kNT / 2,
-                           static_cast<int64_t>(r) * kTileM + half * 128 + lane_base + lane, n0);
-    }
-    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-    __syncthreads();
-    if (warp == 0)
-        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "n"(kTmemCols) : "memory");
-}
-
-}  // namespace one
-
-// ===================================================================================================
-namespace pair {    // two CTAs (a cluster of 2) = one row tile x 512 tokens
-
-constexpr int kThreads = (kWarps + 3) * 32;   // decode warps + the tensor-core warp, the copy warp and the relay warp
-constexpr int kNTiles = 2;                    // accumulators per CTA
-constexpr int kNT = kNTiles * kNI;            // tokens per CTA pair
-constexpr int kStages = 3;                    // operand tiles (decoded W, X) in flight
-constexpr int kCStages = 2;                   // stored K-blocks in flight
-constexpr int kBTileBytes = (kNI / 2) * kBRowBytes;    // this CTA's 128 tokens of one X tile
-constexpr int kBBytes = kNTiles * kBTileBytes;
-static_assert(kNTiles * kNI == kTmemCols, "the accumulators fill tensor memory");
 
 struct __align__(1024) Smem {
     unsigned char B[kStages][kBBytes];              // my halves of the X tiles (each on a 1024-byte boundary: swizzle atoms)
@@ -477,41 +730,13 @@ struct __align__(1024) Smem {
     alignas(8) unsigned long long ready[kStages];       // A stage s is written and my X tiles of B stage s have arrived
                                                         // (first CTA: and the second CTA says the same of its own)
     alignas(8) unsigned long long comp_full[kCStages];  // the stored K-block of comp stage s has arrived
+    alignas(16) uint2 tab[kWarps][32];              // per warp: bitmap word and the address of its first value
     uint32_t tmem_base;
     int abort;
 };
 constexpr size_t kSmemBytes = sizeof(Smem) + 1024;      // the dynamic shared memory is aligned by hand
 static_assert(kSmemBytes <= 227 * 1024, "shared memory of one CTA");
 static_assert(kBTileBytes % 1024 == 0, "every X tile on a swizzle-atom boundary");
-
-// Decodes my 128 rows (half `c` of the row tile) of the warp's 4 columns into the operand tile `a_tile`, in two
-// passes: in a pass the lower half warp takes one column, the upper the next; a lane owns the 8 rows of bitmap
-// byte 16 c + lane % 16, fetches its word and the index of the word's first value from the scan lane, adds the
-// set bits below its byte (its rank, Sec. 4.2.1) and walks the byte.
-__device__ __forceinline__ void decode_block(const Params& p, const CompStage& cs, int ngt, int c, int warp, int lane,
-                                             unsigned char* a_tile) {
-    unsigned w8, base_w;
-    scan_columns(p, cs, ngt, warp, lane, w8, base_w);
-    const int sh = 8 * (lane & 3);
-    const unsigned below = (1u << sh) - 1u;
-    const uint32_t vals = smem_u32(&cs.vals[0]);
-    const int hw = lane >> 4, l16 = lane & 15;
-    uint4 piece[2];
-#pragma unroll
-    for (int ps = 0; ps < 2; ++ps) {
-        const int src = 8 * (2 * ps + hw) + 4 * c + (l16 >> 2);       // the scan lane of (my column, my word)
-        const unsigned word = __shfl_sync(0xFFFFFFFFu, w8, src);
-        const unsigned base = __shfl_sync(0xFFFFFFFFu, base_w, src);
-        const unsigned bits = (word >> sh) & 0xFFu;
-        piece[ps] = walk_byte(bits, vals + 2u * (base + __popc(word & below)));
-    }
-    // the stores come after both walks, so that the walks' loads are free to overlap
-#pragma unroll
-    for (int ps = 0; ps < 2; ++ps) {
-        const int j = warp + kWarps * (2 * ps + hw);
-        *reinterpret_cast<uint4*>(a_tile + l16 * kAChunkStride + (j >> 3) * kAKGroupStride + (j & 7) * 16) = piece[ps];
-    }
-}
 
 __global__ void __launch_bounds__(kThreads, 1)
 spmm_kernel(const __grid_constant__ Params p, const __grid_constant__ CUtensorMap xmap) {
@@ -532,15 +757,16 @@ spmm_kernel(const __grid_constant__ Params p, const __grid_constant__ CUtensorMa
 #pragma unroll
         for (int s = 0; s < kStages; ++s) {
             barrier_init(&sm.mma_done[s], 1);
-            barrier_init(&sm.a_ready[s], kWarps);
+            barrier_init(&sm.a_ready[s], kBlockWarps);
             // arrivals on ready[]: my decode warps, my copy thread (with the X tiles' bytes), in the first CTA the second CTA
-            barrier_init(&sm.ready[s], kWarps + 1 + (c == 0 ? 1 : 0));
+            barrier_init(&sm.ready[s], kBlockWarps + 1 + (c == 0 ? 1 : 0));
         }
 #pragma unroll
         for (int s = 0; s < kCStages; ++s) barrier_init(&sm.comp_full[s], 1);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         sm.abort = 0;
     }
+    __syncwarp();
     if (warp == 0) {
         asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;"
                      ::"r"(smem_u32(&sm.tmem_base)), "n"(kTmemCols) : "memory");
@@ -552,7 +778,7 @@ spmm_kernel(const __grid_constant__ Params p, const __grid_constant__ CUtensorMa
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     const uint32_t tmem = sm.tmem_base;
     // my K-blocks: slice `slice` of the tile's nkb_all; kb below counts from the slice's first block kb0
-    const int nkb_all = (p.C + kGTB - 1) / kGTB;
+    const int nkb_all = p.nkb;
     const int kb0 = static_cast<int>(static_cast<int64_t>(nkb_all) * slice / p.kslices);
     const int nkb = static_cast<int>(static_cast<int64_t>(nkb_all) * (slice + 1) / p.kslices) - kb0;
     // A wait that runs out (it never should) clears `ok`: the thread then stops waiting but keeps walking the
@@ -560,7 +786,8 @@ spmm_kernel(const __grid_constant__ Params p, const __grid_constant__ CUtensorMa
     bool ok = true;
 
     if (warp == kWarps) {
-        if (lane == 0 && c == 0) {
+        const bool one = elect_one();
+        if (one && c == 0) {
             // ================= tensor-core thread (first CTA): issues the K-blocks' products for the pair =================
             for (int kb = 0; kb < nkb; ++kb) {
                 const int s = kb % kStages;
@@ -571,13 +798,12 @@ spmm_kernel(const __grid_constant__ Params p, const __grid_constant__ CUtensorMa
                 for (int i = 0; i < ntiles; ++i) {
 #pragma unroll
                     for (int kk = 0; kk < kKB / 16; ++kk)    // the start address is the descriptor's low field, in 16-byte units
-                        mma_f16_pair(tmem + i * kNI, ad0 + ((kk * 2 * kAKGroupStride) >> 4), bd0 + ((i * kBTileBytes + kk * 32) >> 4),
+                        mma_f16_pair<kNI>(tmem + i * kNI, ad0 + ((kk * 2 * kAKGroupStride) >> 4), bd0 + ((i * kBTileBytes + kk * 32) >> 4),
                                      kb > 0 || kk > 0);
                 }
-                asm volatile("tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.b64 [%0];"
-                             ::"r"(smem_u32(&sm.mma_done[s])) : "memory");
+                commit_pair(&sm.mma_done[s]);
             }
-        } else if (lane == 0) {
+        } else if (one) {
             // ================= second CTA: tell the first when my tiles of a block are ready =================
             for (int kb = 0; kb < nkb; ++kb) {
                 const int s = kb % kStages;
@@ -588,7 +814,7 @@ spmm_kernel(const __grid_constant__ Params p, const __grid_constant__ CUtensorMa
         __syncwarp();           // the other lanes wait here, not on a barrier in shared memory
     } else if (warp == kWarps + 1) {
         // ================= copy warp: one thread moves the stored K-blocks and my halves of the X tiles =================
-        if (lane == 0) {
+        if (elect_one()) {
             // my 128 tokens of the X tiles of K-block kb: one tiled bulk-tensor copy per tile
             auto load_x = [&](int kb) {
                 unsigned long long* bar = &sm.ready[kb % kStages];
@@ -628,13 +854,20 @@ spmm_kernel(const __grid_constant__ Params p, const __grid_constant__ CUtensorMa
         }
         __syncwarp();
     } else {
-        // ================= decode warps =================
-        for (int kb = 0; kb < nkb; ++kb) {
-            const int s = kb % kStages;
-            const unsigned phase = (kb / kStages) & 1;
+        // ================= decode warps: my 128 rows of 4 columns of every sub-block of the group =================
+        const unsigned group = static_cast<unsigned>(warp) / kGroupWarps, wm = static_cast<unsigned>(warp) % kGroupWarps;
+        const unsigned sh = pinned(4u * (lane & 7)), below = pinned((1u << sh) - 1u);
+        const uint32_t tab_l = pinned(smem_u32(&sm.tab[warp][0]) + 32u * c + 8u * (lane >> 3));
+        const uint32_t a_lane = pinned(smem_u32(&sm.A[0][0]) + (lane >> 1) * kAChunkStride + (lane & 1) * 8);
+        for (unsigned i = group; i < static_cast<unsigned>(nkb) * kSubs; i += kGroups) {
+            const unsigned kb = i / kSubs, s = kb % kStages, j0 = (i % kSubs) * kSub + 4u * wm;      // my first column of the K-block
             if (ok) ok = wait_parity(&sm.comp_full[kb % kCStages], (kb / kCStages) & 1);    // the stored block has arrived
-            if (kb >= kStages && ok) ok = wait_parity(&sm.mma_done[s], phase ^ 1u);         // the tensor cores are done with this A stage
-            decode_block(p, sm.comp[kb % kCStages], min(kGTB, p.C - kGTB * (kb0 + kb)), c, warp, lane, &sm.A[s][0]);
+            const CompStage& cs = sm.comp[kb % kCStages];
+            __syncwarp();
+            scan4(p, cs.bm, cs.ci, cs.start, min(kGTB, p.C - kGTB * (kb0 + static_cast<int>(kb))), cs.limit, static_cast<int>(j0), lane, &sm.tab[warp][0]);
+            __syncwarp();
+            if (kb >= kStages && ok) ok = wait_parity(&sm.mma_done[s], ((kb / kStages) & 1u) ^ 1u);  // the tensor cores are done with this A stage
+            expand4<4, 1>(tab_l, a_lane + s * kATileBytes + (j0 >> 3) * kAKGroupStride + (j0 & 7u) * 16u, 0u, below, sh);
             // the operand tile was written through the generic proxy; the tensor cores read through the async proxy
             asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
             __syncwarp();
@@ -655,14 +888,10 @@ spmm_kernel(const __grid_constant__ Params p, const __grid_constant__ CUtensorMa
     __syncthreads();
 
     // ---- epilogue.  Warp w reads lanes 32*(w%4).. (my rows 32*(w%4)..), token columns [(w/4)*128, +128) of the 512 ----
-    if (!sm.abort && warp < kWarps) {
+    if (!sm.abort && warp < kStoreWarps) {
         const int lane_base = 32 * (warp & 3), cbase = (warp >> 2) * (kNT / 4);
-        if (p.partial == nullptr)
-            store_accumulators(p, tmem, lane_base, cbase, cbase + kNT / 4,
-                               static_cast<int64_t>(r) * kTileM + c * 128 + lane_base + lane, n0);
-        else
-            store_partial(p.partial + static_cast<size_t>(pr) * kNT * kTileM, tmem, lane_base, cbase, cbase + kNT / 4,
-                          c * 128 + lane_base + lane, static_cast<int>(min(static_cast<int64_t>(kNT), p.N - n0)));
+        store_accumulators(p, tmem, lane_base, cbase, cbase + kNT / 4, r, c * 128 + lane_base + lane, n0,
+                           p.partial == nullptr ? -1 : static_cast<int>(pr));
     }
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
@@ -671,27 +900,40 @@ spmm_kernel(const __grid_constant__ Params p, const __grid_constant__ CUtensorMa
         asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(tmem), "n"(kTmemCols) : "memory");
 }
 
-// Adds the K-slices of the tiles that were cut along K, in slice order, and writes their part of Y.
-__global__ void reduce_slices_kernel(const Params p, int tiles) {
-    const int64_t total = static_cast<int64_t>(tiles) * kNT * kTileM;
+// Adds the K-slices of the tiles that were cut along K, in slice order, and writes their part of Y.  A thread takes 4
+// consecutive rows of one token.
+__global__ void __launch_bounds__(256)
+reduce_slices_kernel(const Params p, int tiles) {
+    const int64_t total = static_cast<int64_t>(tiles) * p.ptok * (kTileM / 4);
     for (int64_t i = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x; i < total;
          i += static_cast<int64_t>(gridDim.x) * blockDim.x) {
-        const int row_in = static_cast<int>(i % kTileM);
-        const int col = static_cast<int>((i / kTileM) % kNT);
-        const int tt = static_cast<int>(i / (static_cast<int64_t>(kTileM) * kNT));
-        const unsigned tile = static_cast<unsigned>(p.tile0 + tt);
-        const int r = static_cast<int>(tile / static_cast<unsigned>(p.nblocks));
-        const int nb = static_cast<int>(tile - static_cast<unsigned>(r) * static_cast<unsigned>(p.nblocks));
-        const int64_t n = static_cast<int64_t>(nb) * kNT + col, row = static_cast<int64_t>(r) * kTileM + row_in;
+        const int row_in = 4 * static_cast<int>(i % (kTileM / 4));
+        const int64_t q = i / (kTileM / 4);
+        const int tok = static_cast<int>(q % p.ptok), tt = static_cast<int>(q / p.ptok);
+        const int tile = p.tile0 + tt;
+        const int64_t n = static_cast<int64_t>(tile % p.nblocks) * kNT + tok, row = static_cast<int64_t>(tile / p.nblocks) * kTileM + row_in;
         if (n >= p.N || row >= p.M) continue;
-        const float* src = p.partial + (static_cast<size_t>(tt) * p.kslices * kNT + col) * kTileM + row_in;
-        float sum = 0.f;
-        for (int sl = 0; sl < p.kslices; ++sl) sum += src[static_cast<size_t>(sl) * kNT * kTileM];
-        store_y(p.Y, p.ydt, n * p.ldy + row, sum);
+        const float* src = p.partial + (static_cast<size_t>(tt) * p.kslices * p.ptok + tok) * kTileM + row_in;
+        float4 sum = make_float4(0.f, 0.f, 0.f, 0.f);
+        for (int sl = 0; sl < p.kslices; ++sl) {
+            const float4 v = *reinterpret_cast<const float4*>(src + static_cast<size_t>(sl) * p.ptok * kTileM);
+            sum.x += v.x;
+            sum.y += v.y;
+            sum.z += v.z;
+            sum.w += v.w;
+        }
+        const float v[4] = {sum.x, sum.y, sum.z, sum.w};
+#pragma unroll
+        for (int e = 0; e < 4; ++e)
+            if (row + e < p.M) store_y(p.Y, p.ydt, n * p.ldy + row + e, v[e]);
     }
 }
 
 }  // namespace pair
+
+using One32 = one::Form<32>;
+using One128 = one::Form<128>;
+using One256 = one::Form<256>;
 
 }  // namespace
 
@@ -703,8 +945,9 @@ spdp_status configure_spmm_kernel() {
     if (dev < 0 || dev >= 64) return SPDP_ERR_UNSUPPORTED_SHAPE;
     std::lock_guard<std::mutex> lock(mu);
     if (!configured[dev]) {
-        SPDP_CUDA_TRY(cudaFuncSetAttribute(one::spmm_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                           static_cast<int>(one::kSmemBytes)));
+        SPDP_CUDA_TRY(cudaFuncSetAttribute(one::spmm_kernel<One32>, cudaFuncAttributeMaxDynamicSharedMemorySize, one::kSmemBytes));
+        SPDP_CUDA_TRY(cudaFuncSetAttribute(one::spmm_kernel<One128>, cudaFuncAttributeMaxDynamicSharedMemorySize, one::kSmemBytes));
+        SPDP_CUDA_TRY(cudaFuncSetAttribute(one::spmm_kernel<One256>, cudaFuncAttributeMaxDynamicSharedMemorySize, one::kSmemBytes));
         SPDP_CUDA_TRY(cudaFuncSetAttribute(pair::spmm_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                            static_cast<int>(pair::kSmemBytes)));
         configured[dev] = true;
@@ -742,11 +985,101 @@ spdp_status encode_x(CUtensorMap* map, const __half* X, int64_t N, int64_t K, in
         return SPDP_ERR_INVALID_ARG;
     return SPDP_OK;
 }
+
+// How a call is cut.  kernel 0, 1, 2: 32, 128 or 256 tokens per CTA, `workers` CTAs, `rounds` whole rounds of tiles, the
+// K-blocks of the `rest` tiles after them cut into `sharers` ranges.  kernel 3: CTA pairs, 512 tokens, all tiles but the last
+// `rest` whole, those cut into `slices` slices each (sharers = rest * slices).
+struct Plan {
+    double us;
+    int kernel;
+    int workers, rounds, sharers, slices;
+    int64_t tiles, rest;
+};
+constexpr double kBlockUs[4] = {1.02, 1.02, 1.15, 0.98};  // a K-block (64 columns x 256 rows x the kernel's tokens), us
+constexpr double kTileUs = 3.0;                           // a tile's start and end
+constexpr double kReduceUs = 2.5, kReducePerMB = 0.45;    // the second kernel; writing and reading a MB of partial sums
+constexpr int kTokens[4] = {One32::kNI, One128::kNI, One256::kNI, pair::kNT};
+
+// The estimate of a call's time is (K-blocks of the busiest CTA) x (time of a K-block) + what the partial sums cost on
+// their way through memory.
+Plan make_plan(int64_t R, int64_t nkb, int64_t N, int sms) {
+    Plan best = {};
+    best.us = -1.0;
+    for (int f = 0; f < 4; ++f) {
+#ifdef SPDP_SPMM_FORCE
+        if (f != SPDP_SPMM_FORCE) continue;
+#endif
+        Plan q = {};
+        q.kernel = f;
+        q.tiles = R * ((N + kTokens[f] - 1) / kTokens[f]);
+        const int64_t slots = f == 3 ? sms / 2 : sms;                            // CTAs or pairs resident at once
+        const int64_t rounds = q.tiles / slots, left = q.tiles - rounds * slots;
+        const double mb = static_cast<double>(std::min<int64_t>(N, kTokens[f])) * kTileM * 4.0e-6;   // MB of a tile's sums
+        const double whole = (kBlockUs[f] * static_cast<double>(nkb) + kTileUs) * static_cast<double>(rounds);
+        q.rounds = static_cast<int>(rounds);
+        q.slices = 1;
+        q.sharers = left > 0 ? static_cast<int>(left) : 1;
+        q.workers = static_cast<int>(rounds > 0 ? slots : left);
+        q.rest = f == 3 ? 0 : left;
+        q.us = whole + (left > 0 ? kBlockUs[f] * static_cast<double>(nkb) + kTileUs : 0.0);
+        if (best.us < 0.0 || q.us < best.us) best = q;
+        if (left == 0) continue;
+        for (int64_t share = 2 * left; share < 2 * slots; share *= 2) {          // more CTAs (pairs) than tiles
+            int64_t w = std::min(share, slots);
+            if (f == 3) {
+                q.slices = static_cast<int>(std::min<int64_t>(w / left, nkb));
+                w = q.slices * left;
+                q.rest = left;
+            }
+            if (w <= left || w > left * nkb) break;
+            q.sharers = static_cast<int>(w);
+            q.workers = static_cast<int>(rounds > 0 ? slots : w);
+            q.us = whole + kBlockUs[f] * static_cast<double>((left * nkb + w - 1) / w) + kTileUs + kReduceUs +
+                   (f == 3 && rounds > 0 ? kTileUs : 0.0) + kReducePerMB * mb * static_cast<double>(w + left);
+            if (q.us < best.us) best = q;
+        }
+    }
+    return best;
+}
+
+template <class F>
+spdp_status launch_one(const Params& p, const CUtensorMap& xmap, cudaStream_t s) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(static_cast<unsigned>(p.workers));
+    cfg.blockDim = dim3(kThreads);
+    cfg.dynamicSmemBytes = one::kSmemBytes;
+    cfg.stream = s;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    SPDP_CUDA_TRY(cudaLaunchKernelEx(&cfg, one::spmm_kernel<F>, p, xmap));
+    return SPDP_OK;
+}
+
+spdp_status launch_pairs(const Params& p, const CUtensorMap& xmap, int64_t pairs, cudaStream_t s) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(static_cast<unsigned>(2 * pairs));
+    cfg.blockDim = dim3(kThreads);
+    cfg.dynamicSmemBytes = pair::kSmemBytes;
+    cfg.stream = s;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = 2;
+    attr[0].val.clusterDim.y = 1;
+    attr[0].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    SPDP_CUDA_TRY(cudaLaunchKernelEx(&cfg, pair::spmm_kernel, p, xmap));
+    return SPDP_OK;
+}
+
 }  // namespace
 
 spdp_status launch_spmm(const spdp_matrix* h, const __half* X, int64_t N, int64_t ldx, void* Y, int64_t ldy, int ydt,
                         cudaStream_t s) {
-    Params p;
+    Params p = {};
     p.tileoffset = h->tileoffset;
     p.colinfo = h->colinfo;
     p.bitmap = h->bitmap;
@@ -760,70 +1093,62 @@ spdp_status launch_spmm(const spdp_matrix* h, const __half* X, int64_t N, int64_
     p.C = static_cast<int>(h->C);
     p.status = h->status_word;
     p.values_len = h->values_len;
-    p.tile0 = 0;
+    p.nkb = static_cast<int>((h->K + kKB - 1) / kKB);
+    const Plan plan = make_plan(h->R, p.nkb, N, h->sm_count > 1 ? h->sm_count : 2);
+    if (plan.tiles * p.nkb >= (int64_t(1) << 31)) return SPDP_ERR_UNSUPPORTED_SHAPE;
+    const int nt = kTokens[plan.kernel];
+    p.nblocks = static_cast<int>((N + nt - 1) / nt);
+    p.ptok = static_cast<int>(std::min<int64_t>(N, nt));
     p.kslices = 1;
-    p.partial = nullptr;
-    // Which kernel: rounds of CTAs over the SMs x the measured cost of a K-block (a pair's CTA decodes half as much:
-    // 3 : 4).  A last round of the pair kernel that would hold at most half the pairs is cut along K instead: its
-    // tiles are spread over all pairs as K-slices that leave fp32 partial sums in scratch memory, and a small
-    // kernel adds the slices in order (so the result does not depend on timing).
-    const int64_t sms = h->sm_count > 0 ? h->sm_count : 1;
-    const int64_t slots = sms / 2 > 0 ? sms / 2 : 1;                         // pairs resident at once
-    const int64_t ctas_one = h->R * ((N + one::kNT - 1) / one::kNT);
-    const int64_t tiles = h->R * ((N + pair::kNT - 1) / pair::kNT);         // pair tiles
-    const int64_t nkb = (h->C + kGTB - 1) / kGTB;
-    const int64_t full = (tiles / slots) * slots, rest = tiles - full;
-    int64_t slices = 1;
-    if (full > 0 && rest > 0 && 2 * rest <= slots) slices = std::min<int64_t>(std::min<int64_t>(slots / rest, nkb), 64);
-    const double cost_pair = 3.0 * (static_cast<double>(full / slots) + (rest > 0 ? 1.0 / static_cast<double>(slices) : 0.0) +
-                                    (slices > 1 ? 0.1 : 0.0));
-    const double cost_one = 4.0 * static_cast<double>((ctas_one + sms - 1) / sms);
-    const bool use_pair = cost_pair < cost_one;
-    if (std::max(ctas_one, 2 * tiles * slices) >= (int64_t(1) << 31)) return SPDP_ERR_UNSUPPORTED_SHAPE;
     CUtensorMap xmap;
-    spdp_status st = encode_x(&xmap, X, N, h->K, ldx, use_pair ? kNI / 2 : one::kNT);
+    spdp_status st = encode_x(&xmap, X, N, h->K, ldx, plan.kernel == 3 ? pair::kNI / 2 : nt);
     if (st != SPDP_OK) return st;
-    if (!use_pair) {
-        p.nblocks = static_cast<int>((N + one::kNT - 1) / one::kNT);
-        one::spmm_kernel<<<static_cast<unsigned>(ctas_one), one::kThreads, one::kSmemBytes, s>>>(p, xmap);
-        SPDP_CUDA_TRY(cudaGetLastError());
-        return SPDP_OK;
+    const bool cut = plan.rest > 0 && plan.sharers > plan.rest;              // partial sums and a second kernel
+    if (cut) {
+        const size_t slots = static_cast<size_t>(plan.kernel == 3 ? plan.sharers : 2 * plan.sharers);
+        st = scratch_alloc(h->device, slots * p.ptok * kTileM * sizeof(float), s, reinterpret_cast<void**>(&p.partial));
+        if (st != SPDP_OK) return st;
     }
-    p.nblocks = static_cast<int>((N + pair::kNT - 1) / pair::kNT);
-    auto launch_pairs = [&](int64_t pairs) -> spdp_status {
-        cudaLaunchConfig_t cfg = {};
-        cfg.gridDim = dim3(static_cast<unsigned>(2 * pairs));
-        cfg.blockDim = dim3(pair::kThreads);
-        cfg.dynamicSmemBytes = pair::kSmemBytes;
-        cfg.stream = s;
-        cudaLaunchAttribute attr[1];
-        attr[0].id = cudaLaunchAttributeClusterDimension;
-        attr[0].val.clusterDim.x = 2;
-        attr[0].val.clusterDim.y = 1;
-        attr[0].val.clusterDim.z = 1;
-        cfg.attrs = attr;
-        cfg.numAttrs = 1;
-        SPDP_CUDA_TRY(cudaLaunchKernelEx(&cfg, pair::spmm_kernel, p, xmap));
-        return SPDP_OK;
-    };
-    if (slices == 1) return launch_pairs(tiles);
-    // whole tiles first, then the last tiles cut along K, then the sum of their slices
-    st = launch_pairs(full);
-    if (st != SPDP_OK) return st;
-    float* scratch = nullptr;
-    const size_t scratch_bytes = static_cast<size_t>(rest * slices) * pair::kNT * kTileM * sizeof(float);
-    SPDP_CUDA_TRY(cudaMallocAsync(reinterpret_cast<void**>(&scratch), scratch_bytes, s));     // stream-ordered, from the device's pool
-    p.tile0 = static_cast<int>(full);
-    p.kslices = static_cast<int>(slices);
-    p.partial = scratch;
-    st = launch_pairs(rest * slices);
-    if (st == SPDP_OK) {
-        const int64_t elems = rest * pair::kNT * kTileM;
-        pair::reduce_slices_kernel<<<static_cast<unsigned>(std::min<int64_t>((elems + 255) / 256, 4096)), 256, 0, s>>>(
-            p, static_cast<int>(rest));
-        if (cudaGetLastError() != cudaSuccess) st = SPDP_ERR_CUDA;
+    if (plan.kernel == 3) {
+        Params whole = p;                                                    // whole tiles first, then the last tiles cut along K
+        whole.partial = nullptr;
+        if (plan.tiles > plan.rest) st = launch_pairs(whole, xmap, plan.tiles - plan.rest, s);
+        if (st == SPDP_OK && cut) {
+            p.tile0 = static_cast<int>(plan.tiles - plan.rest);
+            p.kslices = plan.slices;
+            st = launch_pairs(p, xmap, plan.rest * plan.slices, s);
+            if (st == SPDP_OK) {
+                const int64_t threads = plan.rest * p.ptok * (kTileM / 4);
+                pair::reduce_slices_kernel<<<static_cast<unsigned>(std::min<int64_t>((threads + 255) / 256, int64_t(8) * h->sm_count)), 256, 0, s>>>(
+                    p, static_cast<int>(plan.rest));
+                if (cudaGetLastError() != cudaSuccess) st = SPDP_ERR_CUDA;
+            }
+        }
+    } else {
+        p.workers = plan.workers;
+        p.rounds = plan.rounds;
+        p.sharers = plan.sharers;
+        p.rest_units = static_cast<unsigned>(plan.rest * p.nkb);
+        st = plan.kernel == 0 ? launch_one<One32>(p, xmap, s) : plan.kernel == 1 ? launch_one<One128>(p, xmap, s) : launch_one<One256>(p, xmap, s);
+        if (st == SPDP_OK && cut) {
+            const int64_t threads = plan.rest * p.ptok * (kTileM / 4);
+            cudaLaunchConfig_t cfg = {};
+            cfg.gridDim = dim3(static_cast<unsigned>(std::min<int64_t>((threads + 255) / 256, int64_t(8) * h->sm_count)));
+            cfg.blockDim = dim3(256);
+            cfg.stream = s;
+            cudaLaunchAttribute attr[1];
+            attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+            attr[0].val.programmaticStreamSerializationAllowed = 1;
+            cfg.attrs = attr;
+            cfg.numAttrs = 1;
+            const cudaError_t e = cudaLaunchKernelEx(&cfg, one::reduce_pieces_kernel, p, plan.rounds * plan.workers, static_cast<int>(plan.rest), nt);
+            if (e != cudaSuccess) {
+                note_cuda_error(e, "reduce_pieces_kernel");
+                st = SPDP_ERR_CUDA;
+            }
+        }
     }
-    cudaFreeAsync(scratch, s);
+    if (cut) cudaFreeAsync(p.partial, s);
     return st;
 }
 

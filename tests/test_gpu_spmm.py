@@ -117,3 +117,29 @@ def test_spmm_rejects_bad_arguments(S):
             S.spdp_spmm(h, Xo[:, :32], Y)                                  # row stride not a multiple of 8 elements
     finally:
         S.spdp_free(h)
+
+
+@pytest.mark.parametrize("R,K,N", [(150, 520, 20), (149, 1000, 30), (5, 5000, 40), (3, 640, 33), (1, 12800, 128), (1, 130, 256),
+                                   (7, 3000, 129), (2, 20000, 1), (37, 64, 513), (2, 65, 31)])
+@pytest.mark.parametrize("sp", [0.0, 0.5, 0.95])
+def test_spmm_work_cuts(S, R, K, N, sp):
+    """How the work is cut over CTAs: whole rounds plus a shared rest (150 and 149 row tiles), CTA ranges that start in one
+    row tile and end in the next (5, 7), many CTAs on one row tile (1, 2), K-blocks of one column, full columns
+    (the ring of stored values at its fullest) and nearly empty ones.  Integers: every partial sum is exact."""
+    rng = np.random.Generator(np.random.PCG64(R * 1000 + K))
+    M = 256 * R - 3
+    W = rng.integers(-4, 5, (M, K)).astype(np.float16)
+    W[rng.random((M, K)) < sp] = 0
+    X = rng.integers(-2, 3, (N, K)).astype(np.float16)
+    Y_ref = X.astype(np.float32) @ W.astype(np.float32).T              # exact: |sums| <= 20000 * 8 < 2^24
+    h = S.spdp_pack_tiled_cbc(dev(W))
+    try:
+        Xd = torch.zeros((N, (K + 7) // 8 * 8), dtype=torch.float16, device="cuda")     # a token starts on a 16-byte boundary
+        Xd[:, :K] = dev(X)
+        Y = torch.full((N, M), float("nan"), dtype=torch.float32, device="cuda")
+        S.spdp_spmm(h, Xd[:, :K], Y)
+        torch.cuda.synchronize()
+        assert S.spdp_last_device_status(h) == 0
+        assert np.array_equal(Y.cpu().numpy(), Y_ref)
+    finally:
+        S.spdp_free(h)
