@@ -473,8 +473,6 @@ spdp_status configure_spmspv_batch_kernel() {
 spdp_status launch_spmspv_batch(const spdp_matrix* h, const __half* x, int64_t ldx, int batch, int rule, float thr,
                                 const uint32_t* mask, int64_t mask_stride, void* y, int64_t ldy, int ydt,
                                 cudaStream_t s) {
-    spdp_status st = configure_spmspv_batch_kernel();
-    if (st != SPDP_OK) return st;
     Params p;
     p.tileoffset = h->tileoffset;
     p.colinfo = h->colinfo;

@@ -543,8 +543,6 @@ spdp_status launch_spmspv_q4(const spdp_matrix* h, const __half* x, int rule, fl
     p.workspace = h->workspace;
     p.status = h->status_word;
     p.values_len = h->values_len;
-    spdp_status st = configure_spmspv_q4_kernel();
-    if (st != SPDP_OK) return st;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(static_cast<unsigned>(h->num_ctas));
     cfg.blockDim = dim3(kThreads);
