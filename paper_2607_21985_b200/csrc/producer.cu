@@ -12,6 +12,10 @@ namespace {
 
 __global__ void swiglu_dp_kernel(const __half* __restrict__ gate, const __half* __restrict__ up, int64_t K, float thr,
                                  __half* __restrict__ x_out, uint32_t* __restrict__ mask_out, int* __restrict__ count) {
+    // The kernel after this one (the decode call) may start its matrix-only prologue now; what the kernel before this one
+    // wrote or still reads (gate, up, x_out, mask_out) is touched only after the wait.
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    asm volatile("griddepcontrol.wait;" ::: "memory");
     const int64_t j = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
     bool active = false;
     if (j < K) {
@@ -34,8 +38,16 @@ spdp_status launch_swiglu_dp(const __half* gate, const __half* up, int64_t K, fl
     if (count != nullptr) SPDP_CUDA_TRY(cudaMemsetAsync(count, 0, sizeof(int), s));
     const int threads = 256;
     const int64_t blocks = (((K + 31) / 32) * 32 + threads - 1) / threads;
-    swiglu_dp_kernel<<<static_cast<unsigned>(blocks), threads, 0, s>>>(gate, up, K, thr, x_out, mask_out, count);
-    SPDP_CUDA_TRY(cudaGetLastError());
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(static_cast<unsigned>(blocks));
+    cfg.blockDim = dim3(threads);
+    cfg.stream = s;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    SPDP_CUDA_TRY(cudaLaunchKernelEx(&cfg, swiglu_dp_kernel, gate, up, K, thr, x_out, mask_out, count));
     return SPDP_OK;
 }
 
