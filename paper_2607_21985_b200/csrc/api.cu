@@ -6,6 +6,7 @@
 #include <mutex>
 #include <new>
 
+#include "spdp_hostdev.h"
 #include "spdp_internal.h"
 
 namespace spdp {
@@ -91,7 +92,7 @@ spdp_status new_handle(int64_t M, int64_t K, int pad_elems, spdp_matrix** out) {
 // ranges) and (re)allocates what depends on it: the split-K workspace (all zero = every tree node empty).
 spdp_status build_partition(spdp_matrix* h, int num_ctas) {
     const int64_t NGT = h->NGT;
-    int P = num_ctas > 0 ? num_ctas : h->sm_count * default_ctas_per_sm();
+    int P = num_ctas > 0 ? num_ctas : hostdev::default_ctas(h->R, h->C, h->sm_count * default_ctas_per_sm());
     if (P > 1024) P = 1024;          // the kernel's range arithmetic is 32-bit: NGT < 2^22 times P must fit
     if (P > NGT) P = static_cast<int>(NGT);
     if (P < 1) P = 1;

@@ -26,6 +26,26 @@ SPDP_HD int range_owner(unsigned ngt, unsigned num_ctas, unsigned g) {
     return static_cast<int>(num / ngt) - 1;
 }
 
+// Default number of CTAs of a decode call on R row tiles of C GTiles each, at most `most` (one per SM).  Three things
+// pull: a GTile costs its CTA about 0.1 us; every level of the split-K tree costs an exchange through L2; and a CTA
+// whose range crosses into the next row tile reduces twice.  So small layers take fewer CTAs, whole numbers of them per
+// row tile, and large ones all.  Measured in us at 50 % density, half the columns skipped (all SMs -> this rule):
+// 1024x1024 6.3 -> 5.6 (64 CTAs), 2048x2048 6.3 -> 6.0 (128), 8192x1024 6.7 -> 6.1 (128), 512x4096 6.7 -> 6.2 (64);
+// 11008x4096 keeps all 148 (12.3 against 12.9 with 129).
+inline int default_ctas(int64_t R, int64_t C, int most) {
+    const int64_t ngt = R * C;
+    int best = most < ngt ? most : static_cast<int>(ngt);
+    auto cost = [&](int64_t p) {
+        const int64_t segments = (p % R == 0) ? p / R : p / R + 2;        // CTAs that feed a row tile, at most
+        int levels = 0;
+        while ((int64_t(1) << levels) < segments) ++levels;
+        return 0.1 * static_cast<double>((ngt + p - 1) / p) + 0.4 * levels + (p % R == 0 ? 0.0 : 0.2);
+    };
+    for (int64_t p = R; p <= most && p <= ngt; p += R)
+        if (cost(p) < cost(best)) best = static_cast<int>(p);
+    return best < 1 ? 1 : best;
+}
+
 // Checked build: is [first, first + count) inside [0, limit)?  A violation is encoded as
 // kCheckBase - site (site = a small number naming the access in the source) for the status word;
 // the caller then skips the access.  Nothing traps and nothing asserts.

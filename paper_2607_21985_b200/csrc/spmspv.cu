@@ -533,8 +533,6 @@ spmspv_kernel(const Params p) {
 // only then wait for the previous kernel (griddepcontrol.wait) before they touch x, y or the
 // workspace.  Back-to-back calls overlap one call's tail with the next call's prologue.
 spdp_status launch_kernel(const Params& p, int num_ctas, cudaStream_t s) {
-    spdp_status st = configure_spmspv_kernel();        // a flag test after the first call on a device
-    if (st != SPDP_OK) return st;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(static_cast<unsigned>(num_ctas));
     cfg.blockDim = dim3(kThreads);
@@ -587,7 +585,7 @@ __global__ void noalloc_setup_kernel(NoAllocScratch* sc, int words) {
 int default_ctas_per_sm() { return kCtasPerSm; }
 
 // Opts the kernel in to its large dynamic shared memory, once per device (handle creation calls
-// this, so spdp_spmspv itself only launches).
+// this, so spdp_spmspv itself only launches; the call without a handle does it itself).
 spdp_status configure_spmspv_kernel() {
     static std::mutex mu;
     static bool configured[64] = {};
@@ -655,8 +653,9 @@ spdp_status launch_spmspv_noalloc(const uint32_t* tileoffset, const uint32_t* co
         sc = scratch_of[dev];
         sms = sm_count_of[dev];
     }
-    int P = sms * kCtasPerSm < kNoAllocMaxCtas ? sms * kCtasPerSm : kNoAllocMaxCtas;
-    if (P > NGT) P = static_cast<int>(NGT);
+    const spdp_status conf = configure_spmspv_kernel();         // a flag test after the first call on a device
+    if (conf != SPDP_OK) return conf;
+    const int P = hostdev::default_ctas(R, C, sms * kCtasPerSm < kNoAllocMaxCtas ? sms * kCtasPerSm : kNoAllocMaxCtas);
     noalloc_setup_kernel<<<(P * kTileM + 1023) / 1024, 256, 0, s>>>(sc, P * kTileM);
     SPDP_CUDA_TRY(cudaGetLastError());
     Params p;

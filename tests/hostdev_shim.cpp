@@ -10,3 +10,4 @@ int shim_span_ok(unsigned long long first, unsigned long long count, unsigned lo
 }
 int shim_check_code(int site) { return spdp::hostdev::check_code(site); }
 }
+extern "C" int shim_default_ctas(long long r, long long c, int most) { return spdp::hostdev::default_ctas(r, c, most); }

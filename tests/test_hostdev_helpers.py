@@ -49,3 +49,13 @@ def test_span_check_fires_only_outside_the_range(H):
     assert not ok(16, 1, 16) and not ok(0, 17, 16) and not ok(17, 0, 16)
     assert not ok((1 << 64) - 1, 2, 1 << 40)                          # first + count would wrap
     assert H.shim_check_code(3) == -1003 and H.shim_check_code(0) == -1000
+
+
+@pytest.mark.parametrize("R,C,most", [(1, 1, 148), (1, 64, 148), (2, 1024, 148), (4, 64, 148), (16, 256, 148), (43, 256, 148), (112, 512, 148),
+                                      (148, 7, 148), (149, 7, 148), (300, 1, 148), (16, 256, 1), (1, 1, 1), (4096, 1023, 148)])
+def test_default_ctas_in_range(H, R, C, most):
+    H.shim_default_ctas.argtypes = [ctypes.c_longlong, ctypes.c_longlong, ctypes.c_int]
+    p = H.shim_default_ctas(R, C, most)
+    assert 1 <= p <= min(most, R * C)
+    if R * C >= 300 * most:
+        assert p > 0.9 * most                          # a large layer uses (nearly) every SM
