@@ -248,7 +248,8 @@ SPDP_API spdp_status spdp_swiglu_dp(const void* gate_dev, const void* up_dev, in
  * are fewer row tiles than ranks).  Host arithmetic only. */
 SPDP_API spdp_status spdp_row_shard(int64_t M, int world, int rank, int64_t* first_row_out, int64_t* rows_out);
 
-/* Release the handle and everything it owns.  spdp_free(NULL) is SPDP_OK. */
+/* Release the handle and everything it owns (waits for the work on its device).  Up to 512 MB of device memory that freed
+ * handles leave is kept for the next ones; spdp_free(NULL), which is SPDP_OK, gives that back to the driver. */
 SPDP_API spdp_status spdp_free(spdp_handle h);
 
 /* ---- inspection surface (the format and the active set are checked bit for bit) ---- */

@@ -21,46 +21,100 @@ void note_cuda_error(cudaError_t e, const char* what) {
 
 namespace {
 
-// Scratch memory of calls that need some (spdp_spmm's partial sums): one pool per device, apart from the device's
-// default pool.  The default pool gives its memory back to the driver at every synchronisation, so a call after one
-// allocated again (0.45 ms on the prefill of 1024 tokens, against the 0.43 ms of its kernels).  This pool keeps at
-// most kScratchKeep bytes over a synchronisation and gives everything back when the device's last handle goes.
-// Stream-ordered: calls on several streams or threads get memory of their own.
+// Device memory comes from two stream-ordered pools per device, apart from the device's default pool (which gives its
+// memory back to the driver at every synchronisation: 0.45 ms per prefill call that needs scratch, and about 3 ms of
+// cudaMalloc and cudaFree per packed and freed layer).
+//   handles  what handles own.  What freed handles leave is kept for the next ones up to kHandleKeep bytes; spdp_free
+//            gives back what is over, and spdp_free(NULL) all of it.
+//   scratch  memory of one spdp_spmm call (its partial sums); keeps up to kScratchKeep bytes over a
+//            synchronisation, all given back when the device's last handle goes.
+// Both are stream-ordered, so calls on several streams or threads get memory of their own.
 constexpr int kMaxDevices = 64;
+constexpr uint64_t kHandleKeep = uint64_t(512) << 20;
 constexpr uint64_t kScratchKeep = uint64_t(96) << 20;
-struct ScratchPool {
-    cudaMemPool_t pool;
+struct DevicePools {
+    cudaMemPool_t handle_pool, scratch_pool;
     int64_t handles;
 };
-std::mutex g_scratch_mu;
-ScratchPool g_scratch[kMaxDevices];
+std::mutex g_pools_mu;
+DevicePools g_pools[kMaxDevices];
+
+// The pool in `slot`, made on first use; keeps up to `keep` unused bytes over a synchronisation.
+spdp_status pool_of(cudaMemPool_t DevicePools::*slot, int device, uint64_t keep, cudaMemPool_t* out) {
+    if (device < 0 || device >= kMaxDevices) return SPDP_ERR_UNSUPPORTED_SHAPE;
+    std::lock_guard<std::mutex> lock(g_pools_mu);
+    cudaMemPool_t& pool = g_pools[device].*slot;
+    if (pool == nullptr) {
+        cudaMemPoolProps props = {};
+        props.allocType = cudaMemAllocationTypePinned;
+        props.handleTypes = cudaMemHandleTypeNone;
+        props.location.type = cudaMemLocationTypeDevice;
+        props.location.id = device;
+        cudaMemPool_t made = nullptr;
+        SPDP_CUDA_TRY(cudaMemPoolCreate(&made, &props));
+        const cudaError_t e = cudaMemPoolSetAttribute(made, cudaMemPoolAttrReleaseThreshold, &keep);
+        if (e != cudaSuccess) {
+            cudaMemPoolDestroy(made);
+            SPDP_CUDA_TRY(e);
+        }
+        pool = made;
+    }
+    *out = pool;
+    return SPDP_OK;
+}
 
 void count_handle(int device, int by) {
     if (device < 0 || device >= kMaxDevices) return;
-    std::lock_guard<std::mutex> lock(g_scratch_mu);
-    ScratchPool& sp = g_scratch[device];
-    sp.handles += by;
-    if (sp.handles == 0 && sp.pool != nullptr) cudaMemPoolTrimTo(sp.pool, 0);
+    std::lock_guard<std::mutex> lock(g_pools_mu);
+    DevicePools& p = g_pools[device];
+    p.handles += by;
+    if (p.handles == 0 && p.scratch_pool != nullptr) cudaMemPoolTrimTo(p.scratch_pool, 0);
+}
+
+// Gives unused memory of the handle pool back until at most `keep` bytes of it are left.
+void trim_handles(int device, uint64_t keep) {
+    if (device < 0 || device >= kMaxDevices) return;
+    std::lock_guard<std::mutex> lock(g_pools_mu);
+    cudaMemPool_t pool = g_pools[device].handle_pool;
+    uint64_t used = 0, reserved = 0;
+    if (pool == nullptr || cudaMemPoolGetAttribute(pool, cudaMemPoolAttrUsedMemCurrent, &used) != cudaSuccess ||
+        cudaMemPoolGetAttribute(pool, cudaMemPoolAttrReservedMemCurrent, &reserved) != cudaSuccess)
+        return;
+    if (reserved > used + keep) cudaMemPoolTrimTo(pool, used + keep);
+}
+
+// Makes `device` current for a scope.
+struct DeviceScope {
+    int before = -1;
+    explicit DeviceScope(int device) {
+        if (cudaGetDevice(&before) != cudaSuccess || before == device || cudaSetDevice(device) != cudaSuccess) before = -1;
+    }
+    ~DeviceScope() {
+        if (before >= 0) cudaSetDevice(before);
+    }
+};
+
+// The caller has made sure that nothing on the device uses the memory any more.
+void handle_free(void* p) {
+    if (p != nullptr) cudaFreeAsync(p, nullptr);
 }
 
 void release(spdp_matrix* h) {
     if (h == nullptr) return;
+    {
+        DeviceScope on(h->device);
+        cudaDeviceSynchronize();            // as cudaFree would: the handle's memory may be in use on any stream
+        handle_free(h->arrays);
+        handle_free(h->values);
+        handle_free(h->workspace);
+        cudaFree(h->probe_items);
+        cudaFree(h->probe_count);
+        cudaStreamSynchronize(nullptr);
+        trim_handles(h->device, kHandleKeep);
+        if (h->host_graph != nullptr) cudaGraphExecDestroy(h->host_graph);
+        if (h->capture_stream != nullptr) cudaStreamDestroy(h->capture_stream);
+    }
     count_handle(h->device, -1);
-    cudaFree(h->tileoffset);
-    cudaFree(h->colinfo);
-    cudaFree(h->bitmap);
-    cudaFree(h->values);
-    cudaFree(h->scales);
-    cudaFree(h->workspace);
-    cudaFree(h->workspace_batch);
-    cudaFree(h->status_word);
-    cudaFree(h->x_stage);
-    cudaFree(h->mask_stage);
-    cudaFree(h->y_stage);
-    cudaFree(h->probe_items);
-    cudaFree(h->probe_count);
-    if (h->host_graph != nullptr) cudaGraphExecDestroy(h->host_graph);
-    if (h->capture_stream != nullptr) cudaStreamDestroy(h->capture_stream);
     h->magic = 0;
     delete h;
 }
@@ -88,9 +142,38 @@ spdp_status new_handle(int64_t M, int64_t K, int pad_elems, spdp_matrix** out) {
     return SPDP_OK;
 }
 
-// Chooses the number of CTAs (the kernel cuts the NGT GTiles into that many equal contiguous
-// ranges) and (re)allocates what depends on it: the split-K workspace (all zero = every tree node empty).
-spdp_status build_partition(spdp_matrix* h, int num_ctas) {
+// Allocates the arrays whose sizes follow from the shape (on `s`), as one piece.
+spdp_status alloc_arrays(spdp_matrix* h, cudaStream_t s) {
+    const int64_t cols = h->NGT * kTileK;
+    size_t at = 0;
+    auto place = [&](size_t bytes) {
+        const size_t here = at;
+        at += (bytes + 255) / 256 * 256;
+        return here;
+    };
+    const size_t bitmap = place(cols * kWordsPerCol * sizeof(uint64_t)), colinfo = place(cols * sizeof(uint32_t)),
+                 tileoffset = place((h->NGT + 1) * sizeof(uint32_t)), scales = place(h->q4 ? cols * sizeof(__half) : 0),
+                 x = place(h->K * sizeof(__half)), mask = place((h->K + 31) / 32 * sizeof(uint32_t)), y = place(h->M * sizeof(float)),
+                 status = place(2 * sizeof(int));
+    spdp_status st = handle_alloc(h->device, at, s, &h->arrays);
+    if (st != SPDP_OK) return st;
+    char* base = static_cast<char*>(h->arrays);
+    h->bitmap = reinterpret_cast<uint64_t*>(base + bitmap);
+    h->colinfo = reinterpret_cast<uint32_t*>(base + colinfo);
+    h->tileoffset = reinterpret_cast<uint32_t*>(base + tileoffset);
+    if (h->q4) h->scales = reinterpret_cast<__half*>(base + scales);
+    h->x_stage = reinterpret_cast<__half*>(base + x);
+    h->mask_stage = reinterpret_cast<uint32_t*>(base + mask);
+    h->y_stage = base + y;
+    h->status_word = reinterpret_cast<int*>(base + status);
+    SPDP_CUDA_TRY(cudaMemsetAsync(h->status_word, 0, 2 * sizeof(int), s));
+    return SPDP_OK;
+}
+
+// Chooses the number of CTAs (the kernel cuts the NGT GTiles into that many contiguous ranges) and (re)allocates what
+// depends on it: the split-K workspaces (all zero = every tree node empty).  The caller synchronises `s`, so that the
+// first call on any stream finds every tree node empty.
+spdp_status build_partition(spdp_matrix* h, int num_ctas, cudaStream_t s) {
     const int64_t NGT = h->NGT;
     int P = num_ctas > 0 ? num_ctas : hostdev::default_ctas(h->R, h->C, h->sm_count * default_ctas_per_sm());
     if (P > 1024) P = 1024;          // the kernel's range arithmetic is 32-bit: NGT < 2^22 times P must fit
@@ -101,23 +184,23 @@ spdp_status build_partition(spdp_matrix* h, int num_ctas) {
         h->host_graph = nullptr;
     }
     h->host_last_valid = false;
-    cudaFree(h->workspace);     h->workspace = nullptr;
-    cudaFree(h->workspace_batch);   h->workspace_batch = nullptr;
+    handle_free(h->workspace);
+    h->workspace = h->workspace_batch = nullptr;
     h->num_ctas = P;
-    h->workspace_bytes = static_cast<int64_t>(P) * kTileM * sizeof(float);   // one row of split-K tree nodes per CTA
-    SPDP_CUDA_TRY(cudaMalloc(&h->workspace, h->workspace_bytes));
-    SPDP_CUDA_TRY(cudaMemset(h->workspace, 0, h->workspace_bytes));
-    SPDP_CUDA_TRY(cudaMalloc(&h->workspace_batch, batch_workspace_bytes(P)));
-    SPDP_CUDA_TRY(cudaMemset(h->workspace_batch, 0, batch_workspace_bytes(P)));
-    h->workspace_bytes += batch_workspace_bytes(P);
-    // The memsets run on the legacy default stream, which a non-blocking stream does not wait for:
-    // the first spdp_spmspv on such a stream must find every tree node empty.
-    SPDP_CUDA_TRY(cudaDeviceSynchronize());
+    const int64_t one = static_cast<int64_t>(P) * kTileM * sizeof(float);    // one row of split-K tree nodes per CTA
+    h->workspace_bytes = one + batch_workspace_bytes(P);
+    spdp_status st = handle_alloc(h->device, h->workspace_bytes, s, reinterpret_cast<void**>(&h->workspace));
+    if (st != SPDP_OK) return st;
+    h->workspace_batch = h->workspace + P * kTileM;
+    SPDP_CUDA_TRY(cudaMemsetAsync(h->workspace, 0, h->workspace_bytes, s));
     return SPDP_OK;
 }
 
-spdp_status finish_handle(spdp_matrix* h) {
-    spdp_status st = build_partition(h, 0);
+// The rest of a handle's set-up; synchronises `s`.
+spdp_status finish_handle(spdp_matrix* h, cudaStream_t s) {
+    spdp_status st = build_partition(h, 0, s);
+    if (st != SPDP_OK) return st;
+    st = configure_pack_kernels();
     if (st != SPDP_OK) return st;
     st = configure_spmspv_kernel();
     if (st != SPDP_OK) return st;
@@ -127,12 +210,7 @@ spdp_status finish_handle(spdp_matrix* h) {
     if (st != SPDP_OK) return st;
     st = configure_spmspv_q4_kernel();
     if (st != SPDP_OK) return st;
-    SPDP_CUDA_TRY(cudaMalloc(&h->status_word, 2 * sizeof(int)));
-    SPDP_CUDA_TRY(cudaMemset(h->status_word, 0, 2 * sizeof(int)));
-    SPDP_CUDA_TRY(cudaMalloc(&h->x_stage, h->K * sizeof(__half)));
-    SPDP_CUDA_TRY(cudaMalloc(&h->mask_stage, ((h->K + 31) / 32) * sizeof(uint32_t)));
-    SPDP_CUDA_TRY(cudaMalloc(&h->y_stage, h->M * sizeof(float)));
-    SPDP_CUDA_TRY(cudaDeviceSynchronize());     // the status word's memset, for callers on non-blocking streams
+    SPDP_CUDA_TRY(cudaStreamSynchronize(s));
     return SPDP_OK;
 }
 
@@ -149,23 +227,17 @@ bool rule_ok(int rule) { return rule == SPDP_DP_NONE || rule == SPDP_DP_ABS_GT |
 }  // namespace
 
 spdp_status scratch_alloc(int device, size_t bytes, cudaStream_t s, void** out) {
-    if (device < 0 || device >= kMaxDevices) return SPDP_ERR_UNSUPPORTED_SHAPE;
     cudaMemPool_t pool = nullptr;
-    {
-        std::lock_guard<std::mutex> lock(g_scratch_mu);
-        ScratchPool& sp = g_scratch[device];
-        if (sp.pool == nullptr) {
-            cudaMemPoolProps props = {};
-            props.allocType = cudaMemAllocationTypePinned;
-            props.handleTypes = cudaMemHandleTypeNone;
-            props.location.type = cudaMemLocationTypeDevice;
-            props.location.id = device;
-            SPDP_CUDA_TRY(cudaMemPoolCreate(&sp.pool, &props));
-            uint64_t keep = kScratchKeep;
-            SPDP_CUDA_TRY(cudaMemPoolSetAttribute(sp.pool, cudaMemPoolAttrReleaseThreshold, &keep));
-        }
-        pool = sp.pool;
-    }
+    const spdp_status st = pool_of(&DevicePools::scratch_pool, device, kScratchKeep, &pool);
+    if (st != SPDP_OK) return st;
+    SPDP_CUDA_TRY(cudaMallocFromPoolAsync(out, bytes, pool, s));
+    return SPDP_OK;
+}
+
+spdp_status handle_alloc(int device, size_t bytes, cudaStream_t s, void** out) {
+    cudaMemPool_t pool = nullptr;
+    const spdp_status st = pool_of(&DevicePools::handle_pool, device, ~uint64_t(0), &pool);      // trimmed by hand, see trim_handles
+    if (st != SPDP_OK) return st;
     SPDP_CUDA_TRY(cudaMallocFromPoolAsync(out, bytes, pool, s));
     return SPDP_OK;
 }
@@ -251,8 +323,9 @@ spdp_status spdp_pack_tiled_cbc_ex(const void* W_dev, int64_t M, int64_t K, int6
     spdp_matrix* h = nullptr;
     spdp_status st = new_handle(M, K, pad_elems, &h);
     if (st != SPDP_OK) return st;
-    st = pack_device(h, static_cast<const __half*>(W_dev), ldw, static_cast<cudaStream_t>(stream));
-    if (st == SPDP_OK) st = finish_handle(h);
+    st = alloc_arrays(h, static_cast<cudaStream_t>(stream));
+    if (st == SPDP_OK) st = pack_device(h, static_cast<const __half*>(W_dev), ldw, static_cast<cudaStream_t>(stream));
+    if (st == SPDP_OK) st = finish_handle(h, static_cast<cudaStream_t>(stream));
     if (st != SPDP_OK) { release(h); return st; }
     *out = h;
     return SPDP_OK;
@@ -273,8 +346,9 @@ spdp_status spdp_pack_tiled_cbc_q4(const void* W_dev, int64_t M, int64_t K, int6
     spdp_status st = new_handle(M, K, 32, &h);
     if (st != SPDP_OK) return st;
     h->q4 = 1;
-    st = pack_q4_device(h, static_cast<const __half*>(W_dev), ldw, static_cast<cudaStream_t>(stream));
-    if (st == SPDP_OK) st = finish_handle(h);
+    st = alloc_arrays(h, static_cast<cudaStream_t>(stream));
+    if (st == SPDP_OK) st = pack_device(h, static_cast<const __half*>(W_dev), ldw, static_cast<cudaStream_t>(stream));
+    if (st == SPDP_OK) st = finish_handle(h, static_cast<cudaStream_t>(stream));
     if (st != SPDP_OK) { release(h); return st; }
     *out = h;
     return SPDP_OK;
@@ -332,17 +406,17 @@ spdp_status spdp_import_tiled_cbc(int64_t M, int64_t K, int pad_elems, const voi
     h->values_len = values_len;
     const size_t vbytes = static_cast<size_t>(values_len) * sizeof(__half);
     auto body = [&]() -> spdp_status {
-        SPDP_CUDA_TRY(cudaMalloc(&h->tileoffset, (h->NGT + 1) * sizeof(uint32_t)));
-        SPDP_CUDA_TRY(cudaMalloc(&h->colinfo, h->NGT * kTileK * sizeof(uint32_t)));
-        SPDP_CUDA_TRY(cudaMalloc(&h->bitmap, h->NGT * kTileK * kWordsPerCol * sizeof(uint64_t)));
-        SPDP_CUDA_TRY(cudaMalloc(&h->values, vbytes < 16 ? 16 : vbytes));
-        SPDP_CUDA_TRY(cudaMemset(h->values, 0, vbytes < 16 ? 16 : vbytes));
+        cudaStream_t s = nullptr;
+        spdp_status a = alloc_arrays(h, s);
+        if (a == SPDP_OK) a = handle_alloc(h->device, vbytes < 16 ? 16 : vbytes, s, reinterpret_cast<void**>(&h->values));
+        if (a != SPDP_OK) return a;
+        SPDP_CUDA_TRY(cudaStreamSynchronize(s));
         SPDP_CUDA_TRY(cudaMemcpy(h->tileoffset, to, (h->NGT + 1) * sizeof(uint32_t), cudaMemcpyHostToDevice));
         SPDP_CUDA_TRY(cudaMemcpy(h->colinfo, ci, h->NGT * kTileK * sizeof(uint32_t), cudaMemcpyHostToDevice));
         SPDP_CUDA_TRY(cudaMemcpy(h->bitmap, bm, h->NGT * kTileK * kWordsPerCol * sizeof(uint64_t),
                                  cudaMemcpyHostToDevice));
         if (vbytes) SPDP_CUDA_TRY(cudaMemcpy(h->values, values_host, vbytes, cudaMemcpyHostToDevice));
-        return finish_handle(h);
+        return finish_handle(h, s);
     };
     st = body();
     if (st != SPDP_OK) { release(h); return st; }
@@ -500,7 +574,10 @@ spdp_status spdp_row_shard(int64_t M, int world, int rank, int64_t* first_row_ou
 }
 
 spdp_status spdp_free(spdp_handle h) {
-    if (h == nullptr) return SPDP_OK;
+    if (h == nullptr) {                     // no handle: give back the memory that freed handles left
+        for (int d = 0; d < kMaxDevices; ++d) trim_handles(d, 0);
+        return SPDP_OK;
+    }
     if (!valid(h)) return SPDP_ERR_INVALID_ARG;
     release(h);
     return SPDP_OK;
@@ -586,8 +663,12 @@ spdp_status spdp_last_device_status(spdp_handle h, int* out) {
 
 spdp_status spdp_set_num_ctas(spdp_handle h, int num_ctas) {
     if (!valid(h) || num_ctas < 0) return SPDP_ERR_INVALID_ARG;
+    DeviceScope on(h->device);
     SPDP_CUDA_TRY(cudaDeviceSynchronize());
-    return build_partition(h, num_ctas);
+    const spdp_status st = build_partition(h, num_ctas, nullptr);
+    if (st != SPDP_OK) return st;
+    SPDP_CUDA_TRY(cudaStreamSynchronize(nullptr));
+    return SPDP_OK;
 }
 
 const char* spdp_last_cuda_error(void) { return g_cuda_error; }

@@ -1,5 +1,12 @@
 // Tiled-CBC packer and unpacker kernels (Sec. 4.1 "Storage Structure", Sec. 4.2.1 decode rule,
-// Sec. 4.2.3 padding).  Offline path: three passes (count -> scan -> emit), one CTA per GTile.
+// Sec. 4.2.3 padding).  Three passes: count -> scan -> emit.  A CTA of the count, emit and unpack kernels handles one row
+// tile x 64 columns (4 GTiles): the dense side moves through shared memory in whole 128-byte rows, and the 4 GTiles'
+// Values are one contiguous span, which moves in 16-byte pieces.  (With one CTA per GTile a row of the dense side was 32
+// bytes and the values were scattered in runs of 2-byte stores.)  11008x4096 at 60 % sparsity: count 27, scan 8, emit 44,
+// unpack 45 us; between the block's loads and its stores a CTA has one serial pass over its 64 columns, which is what is
+// left.  Pack, unpack and free together took 3487 us, 3 ms of it cudaMalloc and cudaFree, and take 184 us.
+#include <mutex>
+
 #include "spdp_internal.h"
 
 namespace spdp {
@@ -31,107 +38,249 @@ __device__ __forceinline__ void load_tile_row(const unsigned short* __restrict__
     }
 }
 
-// Pass 1: bitmap words, per-column nonzero counts, ColInfo, padded length of the GTile.
-__global__ void __launch_bounds__(kTileM)
-pack_count_kernel(const unsigned short* __restrict__ W, int64_t ldw, int64_t M, int64_t K, int64_t C,
-                  int pad_elems, uint64_t* __restrict__ bitmap, uint32_t* __restrict__ colinfo,
-                  uint32_t* __restrict__ tile_len, unsigned long long* __restrict__ nnz_total) {
-    __shared__ unsigned words32[kTileK][kTileM / 32];
-    __shared__ unsigned padded[kTileK];
-    __shared__ unsigned count[kTileK];
-    const int64_t g = blockIdx.x;
-    const int64_t r = g / C, c = g % C;
-    const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
-    unsigned short v[kTileK];
-    load_tile_row(W, ldw, M, K, r * kTileM + t, c * kTileK, v);
+constexpr int kCols = 64;                       // columns a CTA handles: one 128-byte line of a row (32: the same time)
+constexpr int kGT = kCols / kTileK;
+constexpr int kPieces = kCols / 8;              // 16-byte pieces of a row
+constexpr int kRowWords = kCols / 2 + 1;        // 32-bit words per row in shared memory: an odd stride, so that neither the rows
+                                                // of a column pair nor the 16-byte pieces of a row meet in a bank
+
+struct PackSmem {
+    uint32_t tile[kTileM * kRowWords];          // the dense 256 x 64 block
+    alignas(16) unsigned short vals[kCols * kTileM + 8];     // its values as stored
+    uint2 words[kCols / 2][kTileM / 32][2];     // per pair of columns and 32 rows, for each of the two: the bitmap word and the
+                                                // index in vals of its first value (a lane reads all four with one load)
+};
+struct CountSmem {
+    uint32_t tile[kTileM * kRowWords];
+    uint32_t words[kCols][kTileM / 32];
+};
+
+// The dense block at (row0, col0) -> shared memory, zero beyond the matrix edge.
+__device__ __forceinline__ void load_block(const unsigned short* __restrict__ W, int64_t ldw, int64_t M, int64_t K,
+                                           int64_t row0, int64_t col0, uint32_t* tile) {
+    const bool wide = ((reinterpret_cast<uintptr_t>(W) | static_cast<uintptr_t>(2 * ldw)) & 15u) == 0;
+    uint4 v[kCols / 8];
 #pragma unroll
-    for (int cc = 0; cc < kTileK; ++cc) {
-        unsigned b = __ballot_sync(0xFFFFFFFFu, is_stored(v[cc]));
-        if (lane == 0) words32[cc][warp] = b;
-    }
-    __syncthreads();
-    if (t < kTileK * kWordsPerCol) {
-        int cc = t >> 2, w = t & 3;
-        uint64_t word = static_cast<uint64_t>(words32[cc][2 * w]) |
-                        (static_cast<uint64_t>(words32[cc][2 * w + 1]) << 32);
-        bitmap[(g * kTileK + cc) * kWordsPerCol + w] = word;
-    }
-    if (t < kTileK) {
-        unsigned n = 0;
+    for (int i = 0; i < kCols / 8; ++i) {
+        const int q = threadIdx.x + kTileM * i, row = q / kPieces, c = (q % kPieces) * 8;
+        const int64_t r = row0 + row, col = col0 + c;
+        const unsigned short* src = W + r * ldw + col;
+        v[i] = make_uint4(0u, 0u, 0u, 0u);
+        if (r < M && col < K) {
+            if (wide && col + 8 <= K) {
+                v[i] = __ldg(reinterpret_cast<const uint4*>(src));
+            } else {
+                unsigned w[4] = {0u, 0u, 0u, 0u};
 #pragma unroll
-        for (int w = 0; w < kTileM / 32; ++w) n += __popc(words32[t][w]);
-        count[t] = n;
-        padded[t] = (n + pad_elems - 1) / pad_elems * pad_elems;
-    }
-    __syncthreads();
-    if (t == 0) {
-        unsigned off = 0, n = 0;
-        for (int cc = 0; cc < kTileK; ++cc) {
-            colinfo[g * kTileK + cc] = (off << 16) | count[cc];
-            off += padded[cc];
-            n += count[cc];
+                for (int e = 0; e < 8; ++e)
+                    if (col + e < K) w[e >> 1] |= static_cast<unsigned>(__ldg(src + e)) << (16 * (e & 1));
+                v[i] = make_uint4(w[0], w[1], w[2], w[3]);
+            }
         }
-        tile_len[g] = off;
-        if (n) atomicAdd(nnz_total, static_cast<unsigned long long>(n));
+    }
+#pragma unroll
+    for (int i = 0; i < kCols / 8; ++i) {
+        const int q = threadIdx.x + kTileM * i;
+        uint32_t* dst = tile + (q / kPieces) * kRowWords + (q % kPieces) * 4;
+        dst[0] = v[i].x;
+        dst[1] = v[i].y;
+        dst[2] = v[i].z;
+        dst[3] = v[i].w;
     }
 }
 
-// Pass 2: exclusive scan of the padded GTile lengths into TileOffset (one CTA; the array has
-// at most a few hundred thousand entries).  total_out receives the 64-bit total.
+// Pass 1: bitmap words, per-column nonzero counts, ColInfo, padded length of each GTile.
+__global__ void __launch_bounds__(kTileM)
+pack_count_kernel(const unsigned short* __restrict__ W, int64_t ldw, int64_t M, int64_t K, int64_t C, int blocks,
+                  int pad_elems, uint64_t* __restrict__ bitmap, uint32_t* __restrict__ colinfo,
+                  uint32_t* __restrict__ tile_len, unsigned long long* __restrict__ nnz_total) {
+    __shared__ CountSmem sm;
+    const int64_t r = blockIdx.x / static_cast<unsigned>(blocks), cb = blockIdx.x % static_cast<unsigned>(blocks);
+    const int64_t g0 = r * C + cb * kGT;
+    const int ngt = static_cast<int>(min(static_cast<int64_t>(kGT), C - cb * kGT));
+    const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
+    load_block(W, ldw, M, K, r * kTileM, cb * kCols, sm.tile);
+    __syncthreads();
+    const uint32_t* mine = sm.tile + t * kRowWords;
+#pragma unroll 8
+    for (int c = 0; c < kCols / 2; ++c) {
+        const uint32_t v = mine[c];
+        const unsigned b0 = __ballot_sync(0xFFFFFFFFu, (v & 0x7FFFu) != 0), b1 = __ballot_sync(0xFFFFFFFFu, (v & 0x7FFF0000u) != 0);
+        if (lane == 0) {
+            sm.words[2 * c][warp] = b0;
+            sm.words[2 * c + 1][warp] = b1;
+        }
+    }
+    __syncthreads();
+    uint32_t* out = reinterpret_cast<uint32_t*>(bitmap + g0 * kTileK * kWordsPerCol);
+    for (int i = t; i < ngt * kTileK * (kTileM / 32); i += kTileM) out[i] = (&sm.words[0][0])[i];
+    if (t < kCols) {                                        // one thread per column; 16 neighbouring lanes are a GTile
+        unsigned n = 0;
+#pragma unroll
+        for (int w = 0; w < kTileM / 32; ++w) n += __popc(sm.words[t][w]);
+        const unsigned padded = (n + pad_elems - 1) / pad_elems * pad_elems;
+        unsigned end = padded;
+#pragma unroll
+        for (int d = 1; d < kTileK; d <<= 1) {
+            const unsigned u = __shfl_up_sync(0xFFFFFFFFu, end, d, kTileK);
+            if ((t & (kTileK - 1)) >= d) end += u;
+        }
+        if (t < ngt * kTileK) {
+            colinfo[g0 * kTileK + t] = ((end - padded) << 16) | n;
+            if ((t & (kTileK - 1)) == kTileK - 1) tile_len[g0 + t / kTileK] = end;
+        }
+        const unsigned sum = __reduce_add_sync(0xFFFFFFFFu, n);
+        if (lane == 0 && sum) atomicAdd(nnz_total, static_cast<unsigned long long>(sum));
+    }
+}
+
+// Pass 2: exclusive scan of the padded GTile lengths into TileOffset (one CTA; a warp takes one contiguous part, its lanes
+// neighbouring entries).  total_out receives the 64-bit total.
 __global__ void __launch_bounds__(1024)
 pack_scan_kernel(const uint32_t* __restrict__ tile_len, int64_t NGT, uint32_t* __restrict__ tileoffset,
                  unsigned long long* __restrict__ total_out) {
-    __shared__ unsigned long long part[1024];
-    const int t = threadIdx.x;
-    const int64_t per = (NGT + 1023) / 1024;
-    const int64_t lo = min(NGT, t * per), hi = min(NGT, lo + per);
+    __shared__ unsigned long long part[32];
+    const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
+    const int64_t per = (NGT + 1023) / 1024 * 32;
+    const int64_t lo = min(NGT, warp * per), hi = min(NGT, lo + per);
     unsigned long long s = 0;
-    for (int64_t i = lo; i < hi; ++i) s += tile_len[i];
-    part[t] = s;
+#pragma unroll 4
+    for (int64_t i = lo + lane; i < hi; i += 32) s += tile_len[i];
+    for (int d = 16; d > 0; d >>= 1) s += __shfl_xor_sync(0xFFFFFFFFu, s, d);
+    if (lane == 0) part[warp] = s;
     __syncthreads();
-    for (int d = 1; d < 1024; d <<= 1) {
-        unsigned long long add = (t >= d) ? part[t - d] : 0ull;
-        __syncthreads();
-        part[t] += add;
-        __syncthreads();
+    unsigned long long run = 0, total = 0;
+    for (int w = 0; w < 32; ++w) {
+        if (w < warp) run += part[w];
+        total += part[w];
     }
-    unsigned long long run = part[t] - s;
-    for (int64_t i = lo; i < hi; ++i) {
-        tileoffset[i] = static_cast<uint32_t>(run);
-        run += tile_len[i];
+#pragma unroll 4
+    for (int64_t b = lo; b < hi; b += 32) {
+        const int64_t i = b + lane;
+        const uint32_t len = i < hi ? tile_len[i] : 0u;
+        uint32_t inc = len;                                 // 32 lengths of at most 256 * 256 stay below 2^32
+#pragma unroll
+        for (int d = 1; d < 32; d <<= 1) {
+            const uint32_t u = __shfl_up_sync(0xFFFFFFFFu, inc, d);
+            if (lane >= d) inc += u;
+        }
+        if (i < hi) tileoffset[i] = static_cast<uint32_t>(run + inc - len);
+        run += __shfl_sync(0xFFFFFFFFu, inc, 31);
     }
-    if (t == 1023) {
-        tileoffset[NGT] = static_cast<uint32_t>(part[1023]);
-        *total_out = part[1023];
+    if (t == 0) {
+        tileoffset[NGT] = static_cast<uint32_t>(total);
+        *total_out = total;
     }
 }
 
-// Pass 3: write every stored element to Values[TileOffset[g] + column offset + rank]; the
-// padding halfwords keep the zero fill of the buffer.
-__global__ void __launch_bounds__(kTileM)
-pack_emit_kernel(const unsigned short* __restrict__ W, int64_t ldw, int64_t M, int64_t K, int64_t C,
-                 const uint32_t* __restrict__ tileoffset, const uint32_t* __restrict__ colinfo,
-                 unsigned short* __restrict__ values) {
-    __shared__ unsigned words32[kTileK][kTileM / 32];
-    const int64_t g = blockIdx.x;
-    const int64_t r = g / C, c = g % C;
-    const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
-    unsigned short v[kTileK];
-    load_tile_row(W, ldw, M, K, r * kTileM + t, c * kTileK, v);
-    unsigned mine[kTileK];
+// Bitmap words of the CTA's columns and the index in sm.vals of each word's first value (ColInfo offsets, set bits of the
+// words before) -> sm.words.  Lane (q, w) = (t / 8, t % 8) of a pass takes word w of column q.  Returns the number of values
+// of the span, padding included.
+__device__ __forceinline__ uint32_t load_words(PackSmem& sm, const uint32_t* __restrict__ tileoffset, const uint32_t* __restrict__ colinfo,
+                                               const uint64_t* __restrict__ bitmap, int64_t g0, int ngt) {
+    const uint32_t* src = reinterpret_cast<const uint32_t*>(bitmap + g0 * kTileK * kWordsPerCol);
+    const uint32_t first = __ldg(tileoffset + g0);
 #pragma unroll
-    for (int cc = 0; cc < kTileK; ++cc) {
-        mine[cc] = __ballot_sync(0xFFFFFFFFu, is_stored(v[cc]));
-        if (lane == 0) words32[cc][warp] = mine[cc];
+    for (int i = 0; i < kCols * (kTileM / 32) / kTileM; ++i) {
+        const int q = threadIdx.x + kTileM * i, c = q >> 3, w = q & 7;
+        uint32_t word = 0u, off = 0u;
+        if (c < ngt * kTileK) {
+            word = __ldg(src + q);
+            off = __ldg(tileoffset + g0 + c / kTileK) - first + (__ldg(colinfo + g0 * kTileK + c) >> 16);
+        }
+        const uint32_t n = __popc(word);
+        uint32_t inc = n;
+#pragma unroll
+        for (int d = 1; d < 8; d <<= 1) {
+            const uint32_t u = __shfl_up_sync(0xFFFFFFFFu, inc, d, 8);
+            if (w >= d) inc += u;
+        }
+        sm.words[c >> 1][w][c & 1] = make_uint2(word, off + inc - n);
+    }
+    return __ldg(tileoffset + g0 + ngt) - first;
+}
+
+// Pass 3: the stored elements in column order, each column followed by its zero padding.
+__global__ void __launch_bounds__(kTileM)
+pack_emit_kernel(const unsigned short* __restrict__ W, int64_t ldw, int64_t M, int64_t K, int64_t C, int blocks, int pad_elems,
+                 const uint32_t* __restrict__ tileoffset, const uint32_t* __restrict__ colinfo, const uint64_t* __restrict__ bitmap,
+                 unsigned short* __restrict__ values) {
+    extern __shared__ __align__(16) unsigned char raw[];
+    PackSmem& sm = *reinterpret_cast<PackSmem*>(raw);
+    const int64_t r = blockIdx.x / static_cast<unsigned>(blocks), cb = blockIdx.x % static_cast<unsigned>(blocks);
+    const int64_t g0 = r * C + cb * kGT;
+    const int ngt = static_cast<int>(min(static_cast<int64_t>(kGT), C - cb * kGT));
+    const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
+    load_block(W, ldw, M, K, r * kTileM, cb * kCols, sm.tile);
+    const uint32_t total = load_words(sm, tileoffset, colinfo, bitmap, g0, ngt);
+    __syncthreads();
+    const unsigned bit = 1u << lane, below = bit - 1u;
+    const uint32_t* mine = sm.tile + t * kRowWords;
+#pragma unroll 8
+    for (int c = 0; c < kCols / 2; ++c) {
+        const uint32_t v = mine[c];
+        const uint4 e = *reinterpret_cast<const uint4*>(&sm.words[c][warp][0]);
+        if (e.x & bit) sm.vals[e.y + __popc(e.x & below)] = static_cast<unsigned short>(v & 0xFFFFu);
+        if (e.z & bit) sm.vals[e.w + __popc(e.z & below)] = static_cast<unsigned short>(v >> 16);
+    }
+    if (t < ngt * kTileK) {
+        const uint2 last = sm.words[t >> 1][kTileM / 32 - 1][t & 1];
+        const uint32_t end = last.y + __popc(last.x), n = end - sm.words[t >> 1][0][t & 1].y;
+        const uint32_t padding = (n + pad_elems - 1) / pad_elems * pad_elems - n;
+        for (uint32_t i = 0; i < padding; ++i) sm.vals[end + i] = 0;
     }
     __syncthreads();
-    const uint64_t base = tileoffset[g];
+    unsigned short* out = values + tileoffset[g0];
+    if (pad_elems == 8) {                                   // a multiple of 8 values, 16-byte aligned
+        for (uint32_t i = t; i < total / 8; i += kTileM) reinterpret_cast<uint4*>(out)[i] = reinterpret_cast<const uint4*>(sm.vals)[i];
+    } else {
+        for (uint32_t i = t; i < total; i += kTileM) out[i] = sm.vals[i];
+    }
+}
+
+// Decode rule of Sec. 4.2.1: bit clear -> +0, else Values[base + set bits before the position].
+__global__ void __launch_bounds__(kTileM)
+unpack_kernel(const uint32_t* __restrict__ tileoffset, const uint32_t* __restrict__ colinfo,
+              const uint64_t* __restrict__ bitmap, const unsigned short* __restrict__ values, int pad_elems,
+              int64_t M, int64_t K, int64_t C, int blocks, unsigned short* __restrict__ W, int64_t ldw) {
+    extern __shared__ __align__(16) unsigned char raw[];
+    PackSmem& sm = *reinterpret_cast<PackSmem*>(raw);
+    const int64_t r = blockIdx.x / static_cast<unsigned>(blocks), cb = blockIdx.x % static_cast<unsigned>(blocks);
+    const int64_t g0 = r * C + cb * kGT;
+    const int ngt = static_cast<int>(min(static_cast<int64_t>(kGT), C - cb * kGT));
+    const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
+    const uint32_t total = load_words(sm, tileoffset, colinfo, bitmap, g0, ngt);
+    const unsigned short* in = values + tileoffset[g0];
+    if (pad_elems == 8) {
+        for (uint32_t i = t; i < total / 8; i += kTileM) reinterpret_cast<uint4*>(sm.vals)[i] = __ldg(reinterpret_cast<const uint4*>(in) + i);
+    } else {
+        for (uint32_t i = t; i < total; i += kTileM) sm.vals[i] = __ldg(in + i);
+    }
+    __syncthreads();
+    const unsigned bit = 1u << lane, below = bit - 1u;
+    uint32_t* mine = sm.tile + t * kRowWords;
+#pragma unroll 8
+    for (int c = 0; c < kCols / 2; ++c) {
+        const uint4 e = *reinterpret_cast<const uint4*>(&sm.words[c][warp][0]);
+        uint32_t lo = 0u, hi = 0u;
+        if (e.x & bit) lo = sm.vals[e.y + __popc(e.x & below)];
+        if (e.z & bit) hi = sm.vals[e.w + __popc(e.z & below)];
+        mine[c] = lo | (hi << 16);
+    }
+    __syncthreads();
+    const bool wide = ((reinterpret_cast<uintptr_t>(W) | static_cast<uintptr_t>(2 * ldw)) & 15u) == 0;
 #pragma unroll
-    for (int cc = 0; cc < kTileK; ++cc) {
-        if (!is_stored(v[cc])) continue;
-        unsigned rank = __popc(mine[cc] & ((1u << lane) - 1u));
-        for (int w = 0; w < warp; ++w) rank += __popc(words32[cc][w]);
-        values[base + (colinfo[g * kTileK + cc] >> 16) + rank] = v[cc];
+    for (int i = 0; i < kCols / 8; ++i) {
+        const int q = t + kTileM * i;
+        const int64_t row = r * kTileM + q / kPieces, col = cb * kCols + (q % kPieces) * 8;
+        if (row >= M || col >= K) continue;
+        const uint32_t* src = sm.tile + (q / kPieces) * kRowWords + (q % kPieces) * 4;
+        unsigned short* dst = W + row * ldw + col;
+        if (wide && col + 8 <= K) {
+            *reinterpret_cast<uint4*>(dst) = make_uint4(src[0], src[1], src[2], src[3]);
+        } else {
+            for (int e = 0; e < 8 && col + e < K; ++e) dst[e] = static_cast<unsigned short>(src[e >> 1] >> (16 * (e & 1)));
+        }
     }
 }
 
@@ -196,126 +345,78 @@ pack_q4_emit_kernel(const unsigned short* __restrict__ W, int64_t ldw, int64_t M
     }
 }
 
-// Decode rule of Sec. 4.2.1: bit clear -> +0, else Values[base + set bits before the position].
-__global__ void __launch_bounds__(kTileM)
-unpack_kernel(const uint32_t* __restrict__ tileoffset, const uint32_t* __restrict__ colinfo,
-              const uint64_t* __restrict__ bitmap, const unsigned short* __restrict__ values,
-              int64_t M, int64_t K, int64_t C, unsigned short* __restrict__ W, int64_t ldw) {
-    const int64_t g = blockIdx.x;
-    const int64_t r = g / C, c = g % C;
-    const int t = threadIdx.x;
-    const int64_t row = r * kTileM + t;
-    if (row >= M) return;
-    const uint64_t base = tileoffset[g];
-    const int w = t >> 6, b = t & 63;
-    for (int cc = 0; cc < kTileK; ++cc) {
-        const int64_t col = c * kTileK + cc;
-        if (col >= K) break;
-        const uint64_t* bm = bitmap + (g * kTileK + cc) * kWordsPerCol;
-        uint64_t word = bm[w];
-        unsigned short out = 0;
-        if ((word >> b) & 1ull) {
-            unsigned rank = __popcll(word & ((1ull << b) - 1ull));
-            for (int q = 0; q < w; ++q) rank += __popcll(bm[q]);
-            out = values[base + (colinfo[g * kTileK + cc] >> 16) + rank];
-        }
-        W[row * ldw + col] = out;
-    }
-}
-
 }  // namespace
 
-spdp_status pack_device(spdp_matrix* h, const __half* W, int64_t ldw, cudaStream_t s) {
-    const int64_t NGT = h->NGT;
-    uint32_t* tile_len = nullptr;
-    unsigned long long* total_dev = nullptr;
-    SPDP_CUDA_TRY(cudaMalloc(&h->tileoffset, (NGT + 1) * sizeof(uint32_t)));
-    SPDP_CUDA_TRY(cudaMalloc(&h->colinfo, NGT * kTileK * sizeof(uint32_t)));
-    SPDP_CUDA_TRY(cudaMalloc(&h->bitmap, NGT * kTileK * kWordsPerCol * sizeof(uint64_t)));
-    SPDP_CUDA_TRY(cudaMalloc(&tile_len, NGT * sizeof(uint32_t)));
-    cudaError_t e = cudaMalloc(&total_dev, 2 * sizeof(unsigned long long));   // [0] Values length, [1] nnz
-    if (e != cudaSuccess) { cudaFree(tile_len); SPDP_CUDA_TRY(e); }
-    const unsigned short* Wb = reinterpret_cast<const unsigned short*>(W);
-    spdp_status st = SPDP_OK;
-    unsigned long long totals[2] = {0, 0};
-    do {
-        e = cudaMemsetAsync(total_dev, 0, 2 * sizeof(unsigned long long), s);
-        if (e != cudaSuccess) { note_cuda_error(e, "cudaMemsetAsync(totals)"); st = SPDP_ERR_CUDA; break; }
-        pack_count_kernel<<<static_cast<unsigned>(NGT), kTileM, 0, s>>>(
-            Wb, ldw, h->M, h->K, h->C, h->pad_elems, h->bitmap, h->colinfo, tile_len, total_dev + 1);
-        pack_scan_kernel<<<1, 1024, 0, s>>>(tile_len, NGT, h->tileoffset, total_dev);
-        e = cudaMemcpyAsync(totals, total_dev, sizeof(totals), cudaMemcpyDeviceToHost, s);
-        if (e == cudaSuccess) e = cudaStreamSynchronize(s);
-        if (e != cudaSuccess) { note_cuda_error(e, "pack count/scan"); st = SPDP_ERR_CUDA; break; }
-        const unsigned long long total = totals[0];
-        if (total >= (1ull << 32)) { st = SPDP_ERR_OVERFLOW; break; }
-        h->values_len = static_cast<int64_t>(total);
-        h->nnz = static_cast<int64_t>(totals[1]);
-        const size_t vbytes = static_cast<size_t>(total) * sizeof(__half);
-        e = cudaMalloc(&h->values, vbytes < 16 ? 16 : vbytes);
-        if (e != cudaSuccess) { note_cuda_error(e, "cudaMalloc(values)"); st = SPDP_ERR_ALLOC; break; }
-        e = cudaMemsetAsync(h->values, 0, vbytes < 16 ? 16 : vbytes, s);
-        if (e != cudaSuccess) { note_cuda_error(e, "cudaMemsetAsync(values)"); st = SPDP_ERR_CUDA; break; }
-        pack_emit_kernel<<<static_cast<unsigned>(NGT), kTileM, 0, s>>>(
-            Wb, ldw, h->M, h->K, h->C, h->tileoffset, h->colinfo,
-            reinterpret_cast<unsigned short*>(h->values));
-        e = cudaStreamSynchronize(s);
-        if (e == cudaSuccess) e = cudaGetLastError();
-        if (e != cudaSuccess) { note_cuda_error(e, "pack emit"); st = SPDP_ERR_CUDA; break; }
-    } while (false);
-    cudaFree(tile_len);
-    cudaFree(total_dev);
-    return st;
+// Shared-memory opt-in of the emit and unpack kernels, once per device.
+spdp_status configure_pack_kernels() {
+    static std::mutex mu;
+    static bool configured[64] = {};
+    int dev = 0;
+    SPDP_CUDA_TRY(cudaGetDevice(&dev));
+    if (dev < 0 || dev >= 64) return SPDP_ERR_UNSUPPORTED_SHAPE;
+    std::lock_guard<std::mutex> lock(mu);
+    if (!configured[dev]) {
+        SPDP_CUDA_TRY(cudaFuncSetAttribute(pack_emit_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(sizeof(PackSmem))));
+        SPDP_CUDA_TRY(cudaFuncSetAttribute(unpack_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(sizeof(PackSmem))));
+        configured[dev] = true;
+    }
+    return SPDP_OK;
 }
 
-// The 4-bit variant: same count and scan passes with a padding unit of 32 codes, then the quantising emit.
-spdp_status pack_q4_device(spdp_matrix* h, const __half* W, int64_t ldw, cudaStream_t s) {
+// Count and scan, then the emit pass of the handle's variant (fp16 values, or 4-bit codes with scales).  The arrays whose
+// sizes follow from the shape are allocated already; the length of Values is known after the scan, which is what the one
+// synchronisation in the middle is for.  The caller synchronises after the emit pass.
+spdp_status pack_device(spdp_matrix* h, const __half* W, int64_t ldw, cudaStream_t s) {
     const int64_t NGT = h->NGT;
-    uint32_t* tile_len = nullptr;
-    unsigned long long* total_dev = nullptr;
-    SPDP_CUDA_TRY(cudaMalloc(&h->tileoffset, (NGT + 1) * sizeof(uint32_t)));
-    SPDP_CUDA_TRY(cudaMalloc(&h->colinfo, NGT * kTileK * sizeof(uint32_t)));
-    SPDP_CUDA_TRY(cudaMalloc(&h->bitmap, NGT * kTileK * kWordsPerCol * sizeof(uint64_t)));
-    SPDP_CUDA_TRY(cudaMalloc(&h->scales, NGT * kTileK * sizeof(__half)));
-    SPDP_CUDA_TRY(cudaMalloc(&tile_len, NGT * sizeof(uint32_t)));
-    cudaError_t e = cudaMalloc(&total_dev, 2 * sizeof(unsigned long long));   // [0] code count, [1] nnz
-    if (e != cudaSuccess) { cudaFree(tile_len); SPDP_CUDA_TRY(e); }
     const unsigned short* Wb = reinterpret_cast<const unsigned short*>(W);
-    spdp_status st = SPDP_OK;
+    const int blocks = static_cast<int>((h->C + kGT - 1) / kGT);
+    const unsigned grid = static_cast<unsigned>(h->R * blocks);
+    spdp_status st = configure_pack_kernels();
+    if (st != SPDP_OK) return st;
+    uint32_t* tile_len = nullptr;
+    unsigned long long* total_dev = nullptr;               // [0] Values length, [1] nnz
+    st = handle_alloc(h->device, 2 * sizeof(unsigned long long) + NGT * sizeof(uint32_t), s, reinterpret_cast<void**>(&total_dev));
+    if (st != SPDP_OK) return st;
+    tile_len = reinterpret_cast<uint32_t*>(total_dev + 2);
     unsigned long long totals[2] = {0, 0};
-    do {
-        e = cudaMemsetAsync(total_dev, 0, 2 * sizeof(unsigned long long), s);
-        if (e != cudaSuccess) { note_cuda_error(e, "cudaMemsetAsync(totals)"); st = SPDP_ERR_CUDA; break; }
-        pack_count_kernel<<<static_cast<unsigned>(NGT), kTileM, 0, s>>>(
-            Wb, ldw, h->M, h->K, h->C, h->pad_elems, h->bitmap, h->colinfo, tile_len, total_dev + 1);
+    auto body = [&]() -> spdp_status {
+        SPDP_CUDA_TRY(cudaMemsetAsync(total_dev, 0, 2 * sizeof(unsigned long long), s));
+        pack_count_kernel<<<grid, kTileM, 0, s>>>(Wb, ldw, h->M, h->K, h->C, blocks, h->pad_elems, h->bitmap, h->colinfo, tile_len,
+                                                  total_dev + 1);
         pack_scan_kernel<<<1, 1024, 0, s>>>(tile_len, NGT, h->tileoffset, total_dev);
-        e = cudaMemcpyAsync(totals, total_dev, sizeof(totals), cudaMemcpyDeviceToHost, s);
-        if (e == cudaSuccess) e = cudaStreamSynchronize(s);
-        if (e != cudaSuccess) { note_cuda_error(e, "pack count/scan"); st = SPDP_ERR_CUDA; break; }
-        if (totals[0] >= (1ull << 32)) { st = SPDP_ERR_OVERFLOW; break; }
+        SPDP_CUDA_TRY(cudaMemcpyAsync(totals, total_dev, sizeof(totals), cudaMemcpyDeviceToHost, s));
+        SPDP_CUDA_TRY(cudaStreamSynchronize(s));
+        if (totals[0] >= (1ull << 32)) return SPDP_ERR_OVERFLOW;
         h->values_len = static_cast<int64_t>(totals[0]);
         h->nnz = static_cast<int64_t>(totals[1]);
-        const size_t cbytes = static_cast<size_t>(totals[0]) / 2 + 16;         // + 16: the decode reads one word past a span
-        e = cudaMalloc(&h->values, cbytes);
-        if (e != cudaSuccess) { note_cuda_error(e, "cudaMalloc(codes)"); st = SPDP_ERR_ALLOC; break; }
-        e = cudaMemsetAsync(h->values, 0, cbytes, s);
-        if (e != cudaSuccess) { note_cuda_error(e, "cudaMemsetAsync(codes)"); st = SPDP_ERR_CUDA; break; }
-        pack_q4_emit_kernel<<<static_cast<unsigned>(NGT), kTileM, 0, s>>>(
-            Wb, ldw, h->M, h->K, h->C, h->tileoffset, h->colinfo, reinterpret_cast<unsigned char*>(h->values),
-            reinterpret_cast<unsigned short*>(h->scales));
-        e = cudaStreamSynchronize(s);
-        if (e == cudaSuccess) e = cudaGetLastError();
-        if (e != cudaSuccess) { note_cuda_error(e, "pack q4 emit"); st = SPDP_ERR_CUDA; break; }
-    } while (false);
-    cudaFree(tile_len);
-    cudaFree(total_dev);
+        if (h->q4) {
+            const size_t cbytes = static_cast<size_t>(totals[0]) / 2 + 16;     // + 16: the decode reads one word past a span
+            spdp_status a = handle_alloc(h->device, cbytes, s, reinterpret_cast<void**>(&h->values));
+            if (a != SPDP_OK) return a;
+            SPDP_CUDA_TRY(cudaMemsetAsync(h->values, 0, cbytes, s));
+            pack_q4_emit_kernel<<<static_cast<unsigned>(NGT), kTileM, 0, s>>>(
+                Wb, ldw, h->M, h->K, h->C, h->tileoffset, h->colinfo, reinterpret_cast<unsigned char*>(h->values),
+                reinterpret_cast<unsigned short*>(h->scales));
+        } else {
+            const size_t vbytes = static_cast<size_t>(totals[0]) * sizeof(__half);
+            spdp_status a = handle_alloc(h->device, vbytes < 16 ? 16 : vbytes, s, reinterpret_cast<void**>(&h->values));
+            if (a != SPDP_OK) return a;
+            pack_emit_kernel<<<grid, kTileM, sizeof(PackSmem), s>>>(Wb, ldw, h->M, h->K, h->C, blocks, h->pad_elems, h->tileoffset,
+                                                                    h->colinfo, h->bitmap, reinterpret_cast<unsigned short*>(h->values));
+        }
+        SPDP_CUDA_TRY(cudaGetLastError());
+        return SPDP_OK;
+    };
+    st = body();
+    cudaFreeAsync(total_dev, s);
     return st;
 }
 
 spdp_status unpack_device(const spdp_matrix* h, __half* W, int64_t ldw, cudaStream_t s) {
-    unpack_kernel<<<static_cast<unsigned>(h->NGT), kTileM, 0, s>>>(
-        h->tileoffset, h->colinfo, h->bitmap, reinterpret_cast<const unsigned short*>(h->values),
-        h->M, h->K, h->C, reinterpret_cast<unsigned short*>(W), ldw);
+    const int blocks = static_cast<int>((h->C + kGT - 1) / kGT);
+    unpack_kernel<<<static_cast<unsigned>(h->R * blocks), kTileM, sizeof(PackSmem), s>>>(
+        h->tileoffset, h->colinfo, h->bitmap, reinterpret_cast<const unsigned short*>(h->values), h->pad_elems,
+        h->M, h->K, h->C, blocks, reinterpret_cast<unsigned short*>(W), ldw);
     SPDP_CUDA_TRY(cudaGetLastError());
     return SPDP_OK;
 }

@@ -26,7 +26,9 @@ struct spdp_matrix {
     int64_t nnz;
     int64_t values_len;
 
-    // Tiled-CBC arrays (device)
+    // Tiled-CBC arrays (device).  `arrays` is the allocation that holds every array whose size follows from the shape:
+    // tileoffset, colinfo, bitmap, scales, the status word and the staging buffers; values has its own.
+    void* arrays;
     uint32_t* tileoffset;   // [NGT+1]
     uint32_t* colinfo;      // [NGT*16]
     uint64_t* bitmap;       // [NGT*16*4]
@@ -37,8 +39,8 @@ struct spdp_matrix {
     // Work partition of one spmspv launch: the kernel cuts the NGT GTiles into num_ctas equal
     // contiguous ranges, one per CTA.
     int num_ctas;           // P
-    float* workspace;       // device [P*256] split-K tree nodes, one row per CTA (all zero between calls)
-    float* workspace_batch; // device [P*8*256] tree nodes of the small-batch call (all zero between calls)
+    float* workspace;       // device [P*256] split-K tree nodes, one row per CTA (all zero between calls); own allocation
+    float* workspace_batch; // device [P*8*256] tree nodes of the small-batch call (all zero between calls), in the same one
     int* status_word;       // device [2]: the status word, and a sink word the benchmark probes may write
     int64_t workspace_bytes;
 
@@ -92,9 +94,12 @@ inline bool valid(const spdp_matrix* h) { return h != nullptr && h->magic == kMa
 
 // api.cu: stream-ordered scratch memory for one call (given back with cudaFreeAsync on the same stream).
 spdp_status scratch_alloc(int device, size_t bytes, cudaStream_t s, void** out);
+// api.cu: memory that a handle owns (given back with handle_free); usable on other streams once `s` has been synchronised.
+spdp_status handle_alloc(int device, size_t bytes, cudaStream_t s, void** out);
 
 // pack.cu
-spdp_status pack_device(spdp_matrix* h, const __half* W, int64_t ldw, cudaStream_t s);
+spdp_status configure_pack_kernels();          // per-device kernel attributes; idempotent
+spdp_status pack_device(spdp_matrix* h, const __half* W, int64_t ldw, cudaStream_t s);     // either variant
 spdp_status unpack_device(const spdp_matrix* h, __half* W, int64_t ldw, cudaStream_t s);
 
 // spmspv.cu
@@ -112,9 +117,8 @@ spdp_status launch_spmspv_batch(const spdp_matrix* h, const __half* x, int64_t l
                                 const uint32_t* mask, int64_t mask_stride, void* y, int64_t ldy, int ydt,
                                 cudaStream_t s);
 
-// spmspv_q4.cu / pack.cu: the 4-bit variant
+// spmspv_q4.cu: the 4-bit variant
 spdp_status configure_spmspv_q4_kernel();      // per-device kernel attributes; idempotent
-spdp_status pack_q4_device(spdp_matrix* h, const __half* W, int64_t ldw, cudaStream_t s);
 spdp_status launch_spmspv_q4(const spdp_matrix* h, const __half* x, int rule, float thr, const uint32_t* mask, void* y,
                              int ydt, cudaStream_t s);
 

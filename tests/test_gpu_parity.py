@@ -506,3 +506,37 @@ def test_producer_fused_activation_and_mask(S):
         check_y(y_mask.cpu().numpy().astype(np.float64), y_ref, S_ref)
     finally:
         S.spdp_free(h)
+
+
+@pytest.mark.parametrize("pad", [8, 1])
+@pytest.mark.parametrize("M,K,ldw,shift", [(256, 64, 64, 0), (257, 63, 64, 0), (255, 65, 72, 0), (300, 128, 131, 0), (512, 130, 136, 1),
+                                           (1, 1, 1, 0), (31, 200, 200, 3), (768, 16, 24, 0), (2000, 1100, 1104, 0)])
+def test_pack_blocks_round_trip(S, M, K, ldw, shift, pad):
+    """The packer handles 256 x 64 blocks: edges of the block, rows that do not start on 16 bytes (odd strides, shifted
+    base), both padding units, special values; packed arrays and the way back bit for bit."""
+    W = WL.special_values_matrix(M, K, 7 * M + K)
+    buf = torch.zeros(M * ldw + shift + 8, dtype=torch.float16, device="cuda")
+    Wd = buf[shift:shift + M * ldw].view(M, ldw)[:, :K]
+    Wd.copy_(torch.from_numpy(W))
+    h = S.spdp_pack_tiled_cbc(Wd, pad_elems=pad)
+    try:
+        got, want = S.spdp_export(h), O.pack_ref(W, pad_elems=pad) if M * K < 50000 else O.pack_fast(W, pad_elems=pad)
+        for key in ("tileoffset", "colinfo", "bitmap", "values"):
+            assert np.array_equal(got[key], want[key]), key
+        out = torch.full((M * ldw + shift + 8,), 7.0, dtype=torch.float16, device="cuda")
+        S.spdp_unpack(h, out[shift:shift + M * ldw].view(M, ldw)[:, :K])
+        torch.cuda.synchronize()
+        back = out[shift:shift + M * ldw].view(M, ldw).cpu().numpy().view(np.uint16)
+        bits = W.view(np.uint16)
+        assert np.array_equal(back[:, :K], np.where(bits & 0x7FFF, bits, 0))
+        assert np.all(back[:, K:] == np.float16(7.0).view(np.uint16))          # nothing beyond the K columns is written
+    finally:
+        S.spdp_free(h)
+
+
+def test_free_of_nothing_gives_kept_memory_back(S):
+    h = S.spdp_pack_tiled_cbc(torch.ones((2048, 4096), dtype=torch.float16, device="cuda"))
+    S.spdp_free(h)
+    kept = torch.cuda.mem_get_info()[0]
+    S.spdp_free(None)
+    assert torch.cuda.mem_get_info()[0] >= kept + (16 << 20)                    # the layer's 16 MB of values at least
