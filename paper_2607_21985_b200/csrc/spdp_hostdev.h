@@ -20,8 +20,10 @@ namespace hostdev {
 SPDP_HD unsigned range_begin(unsigned ngt, unsigned num_ctas, unsigned c) { return (ngt * c) / num_ctas; }
 
 // The CTA whose range holds GTile g: ceil((g + 1) * num_ctas / NGT) - 1.  The numerator can reach
-// 2^32 + 2^22 at the limits, so this one is 64-bit (it runs twice per row tile, not per GTile).
+// 2^32 + 2^22 at the limits; where it cannot, 32-bit arithmetic does (a 64-bit division takes several hundred clocks, and
+// this stands between the last column tile of a row tile and its store).
 SPDP_HD int range_owner(unsigned ngt, unsigned num_ctas, unsigned g) {
+    if (ngt <= 0xFFFFFFFFu / (num_ctas + 1u)) return static_cast<int>(((g + 1u) * num_ctas + ngt - 1u) / ngt) - 1;
     const unsigned long long num = static_cast<unsigned long long>(g + 1u) * num_ctas + ngt - 1u;
     return static_cast<int>(num / ngt) - 1;
 }

@@ -46,7 +46,6 @@ constexpr int kThreads = kWarps * 32;
 constexpr int kChunkCols = SPDP_CHUNK_COLS; // columns handled between two pipeline drains
 constexpr int kCtasPerSm = SPDP_CTAS_PER_SM;
 constexpr uint32_t kNullRec = 0xFFFFFFFFu;
-constexpr int kListPasses = (kChunkCols / 8 + kThreads - 1) / kThreads;     // 8-position units a thread lists per batch
 constexpr int kChunkGT = kChunkCols / kTileK;
 constexpr int kRecPad = kGroup * (kDepth * kWarps + 1);   // null records behind the last real one
 
@@ -93,8 +92,9 @@ struct __align__(128) Smem {
                                                         //      follows the last record for kRecPad entries, so a warp
                                                         //      can fetch kDepth groups ahead without a range test
     alignas(16) unsigned short xact[kChunkCols + kGroup];   // its activation x_j (fp16 bits)
+    Segments segments[2][2];                            // of the batch's two row tiles, for alternating batches
     float red_first[kWarps][kTileM];                    // row reduction of a batch's first piece (flushed mid-stream)
-    uint32_t warp_total[kListPasses][kWarps][2];        // list phase: records listed by each warp per pass (all, piece A)
+    uint32_t warp_total[kWarps];                        // list phase: records listed by each warp
 };
 static_assert(offsetof(Smem, rec) % 16 == 0 && offsetof(Smem, xact) % 16 == 0 && offsetof(Smem, tab) % 16 == 0, "16-byte shared loads need aligned tables");
 static_assert(sizeof(float) * kWarps * kTileM <= size_t(kWarps) * kDepth * kStageBytes, "red must fit in the ring");
@@ -166,21 +166,17 @@ __device__ __forceinline__ int range_owner(const Params& p, unsigned g) {
 // row inside the tile; the rows are independent, nothing here synchronises threads).  A row tile
 // fed by one segment is stored directly; otherwise the segments' sums meet along the fixed tree of
 // tree_combine and the thread that completes the root stores y.
-__device__ __forceinline__ void finish_row_tile(const Params& p, int r, const float (*red)[kTileM], int tt) {
+__device__ __forceinline__ void finish_row_tile(const Params& p, int r, Segments seg, const float (*red)[kTileM], int tt) {
     float part = 0.f;
-#pragma unroll
+#pragma unroll 8
     for (int w = 0; w < kWarps; ++w) part += red[w][tt];
     const int64_t row = static_cast<int64_t>(r) * kTileM + tt;
     if (row >= p.M) return;
-    const int q0 = range_owner(p, static_cast<unsigned>(r) * p.C);                 // first and last CTA feeding row tile r
-    const int nseg = range_owner(p, static_cast<unsigned>(r + 1) * p.C - 1u) - q0 + 1;
-    if (!SPDP_CHECK(p.status, q0, nseg, p.num_ctas, kSiteTreeNodes) ||
-        !SPDP_CHECK(p.status, static_cast<int>(blockIdx.x) - q0, 1, nseg, kSiteTreeNodes) ||
+    const int my_seg = static_cast<int>(blockIdx.x) - seg.q0;
+    if (!SPDP_CHECK(p.status, seg.q0, seg.nseg, p.num_ctas, kSiteTreeNodes) || !SPDP_CHECK(p.status, my_seg, 1, seg.nseg, kSiteTreeNodes) ||
         !SPDP_CHECK(p.status, row, 1, p.M, kSiteOutputRow))
         return;
-    if (tree_combine(part, reinterpret_cast<unsigned*>(p.workspace) + tt, kTileM, q0, nseg,
-                     static_cast<int>(blockIdx.x) - q0))
-        store_y(p.y, p.ydt, row, part);
+    if (tree_combine(part, reinterpret_cast<unsigned*>(p.workspace) + tt, kTileM, seg.q0, seg.nseg, my_seg)) store_y(p.y, p.ydt, row, part);
 }
 
 // One persistent CTA per GTile range; every warp runs its own fetch -> decode pipeline.
@@ -189,7 +185,7 @@ __device__ __forceinline__ void finish_row_tile(const Params& p, int r, const fl
 // that the usual CTA range (the tail of one row tile and the head of the next) is one batch.
 // Per batch:
 //   (1) all warps: the pieces' ColInfo / TileOffset words and the active-column list from x
-//       (a thread tests 8 columns, warp scans + prefix sums place them), one record per active
+//       (ballots + prefix sums place them), one record per active
 //       column tile -- Sec. 4.2 steps (1)-(3);
 //   (2) each warp takes groups of kGroup active column tiles round-robin.  It keeps kDepth
 //       groups in flight: the padded values of a column tile arrive with 16-byte asynchronous
@@ -239,7 +235,9 @@ spmspv_kernel(const Params p) {
 #pragma unroll
     for (int k = 0; k < 8; ++k) acc[k] = 0.f;
 
+    int parity = 1;
     for (unsigned g0 = g_begin; g0 < g_end;) {
+        parity ^= 1;
         // ---- the batch: piece A = [gA, gA + ngtA) of row tile rA, optionally piece B of row tile rA + 1 ----
         const int rA = static_cast<int>(g0 / static_cast<unsigned>(p.C));
         const int cA = static_cast<int>(g0 - static_cast<unsigned>(rA) * static_cast<unsigned>(p.C));
@@ -251,7 +249,7 @@ spmspv_kernel(const Params p) {
         const bool doneA = (cA + ngtA == p.C) || (g0 == g_end);     // piece A ends its row tile's share of this CTA
         const int jA0 = cA * kTileK;
         const int nA = min((cA + ngtA) * kTileK, p.K) - jA0;         // columns of piece A
-        const int vB0 = (ngtA * kTileK + 31) & ~31;                  // piece B starts at this list position
+        const int vB0 = (ngtA * kTileK + 63) & ~63;                  // piece B starts at this list position
         int ngtB = 0, nB = 0;
         bool doneB = false;
         if (doneA && g0 < g_end && cA + ngtA == p.C) {
@@ -264,6 +262,13 @@ spmspv_kernel(const Params p) {
         const unsigned gB = g0;
         g0 += ngtB;
         const int rB = rA + 1;
+        if (t < 2) {        // read behind several barriers, and not written again before the threads that read it have passed one
+            const unsigned r = static_cast<unsigned>(t == 0 ? rA : rB);
+            Segments seg;
+            seg.q0 = range_owner(p, min(r * p.C, static_cast<unsigned>(p.NGT) - 1u));
+            seg.nseg = range_owner(p, min((r + 1u) * p.C, static_cast<unsigned>(p.NGT)) - 1u) - seg.q0 + 1;
+            sm.segments[parity][t] = seg;
+        }
         const int nlist = (ngtB > 0) ? vB0 + nB : nA;               // list positions (A, padding, B)
 
         // ---- (1) active-column list of the batch (ballots + prefix sums) and its records ----
@@ -299,108 +304,45 @@ spmspv_kernel(const Params p) {
         }
         cp_async_wait<0>();
         __syncthreads();
-        // A thread lists 8 consecutive positions per pass (unit (pass * kThreads + t)): the DP test on its
-        // 8 activations gives an 8-bit mask, a warp scan of the counts its place among the warp's
-        // records; the warps' totals meet in shared memory, every thread derives its first record index
-        // from them, and the records are written in list order.  Piece B starts on a whole group of
-        // kGroup records: the padding is inserted in front of its first record.
-        unsigned m8[kListPasses], below[kListPasses];
-#pragma unroll
-        for (int k = 0; k < kListPasses; ++k) {
-            const int v0 = (k * kThreads + t) * 8;                       // first list position of my unit
-            unsigned m = 0;
-            if (v0 < nlist) {
-                const int lim = ((v0 < vB0) ? nA : nlist) - v0;          // positions of the unit that hold a column
-                if (p.rule == SPDP_DP_ABS_GT) {
-                    const uint4 xv = *reinterpret_cast<const uint4*>(&sm.stage.x[v0]);
-                    const unsigned xw[4] = {xv.x, xv.y, xv.z, xv.w};
-#pragma unroll
-                    for (int i = 0; i < 4; ++i) {
-                        const float lo = __half2float(__ushort_as_half(static_cast<unsigned short>(xw[i] & 0xFFFFu)));
-                        const float hi = __half2float(__ushort_as_half(static_cast<unsigned short>(xw[i] >> 16)));
-                        m |= (!(fabsf(lo) <= p.thr) ? 1u : 0u) << (2 * i);
-                        m |= (!(fabsf(hi) <= p.thr) ? 1u : 0u) << (2 * i + 1);
-                    }
-                } else if (p.rule == SPDP_DP_MASK) {
-                    // units of the padding between the two pieces hold no column: they must not touch
-                    // the mask (their word can lie one past its end)
-                    if (lim > 0) {
-                        const int j0 = (v0 < vB0) ? jA0 + v0 : v0 - vB0; // a multiple of 8
-                        m = (__ldg(p.mask + (j0 >> 5)) >> (j0 & 31)) & 0xFFu;
-                    }
-                } else {
-                    m = 0xFFu;
+        const bool two = (ngtB > 0);
+        const unsigned thr2 = threshold_pair(p.thr);
+        const unsigned slotA = gA * kTileK, slotB = gB * kTileK - vB0;                       // column slot of list position 0
+        const ListTotals list = build_list<kWarps, kChunkCols, kGroup>(
+            sm.warp_total, sm.tab[warp].bm[0], nA, vB0, nlist, two,
+            [&](int v) -> unsigned {                                                         // the DP test on the columns of positions v, v + 1
+                if (p.rule == SPDP_DP_ABS_GT) return abs_gt_keep(*reinterpret_cast<const unsigned*>(&sm.stage.x[v]), thr2);
+                if (p.rule == SPDP_DP_MASK) {
+                    const int j = min((two && v >= vB0) ? v - vB0 : jA0 + v, (p.K - 1) & ~1); // even: both bits lie in one word
+                    const unsigned w = __ldg(p.mask + (j >> 5)) >> (j & 31);
+                    return (w & 1u) | ((w & 2u) << 30);
                 }
-                m &= (lim >= 8) ? 0xFFu : (lim > 0 ? (1u << lim) - 1u : 0u);
-            }
-            m8[k] = m;
-            const unsigned c = __popc(m);
-            unsigned inc = c;
+                return 0xFFFFFFFFu;
+            },
+            [&](int item, int v, bool k0, bool k1, bool in_b) {
+                const uint2 cp = *reinterpret_cast<const uint2*>(&sm.stage.colinfo[v]);       // ColInfo: offset << 16 | nnz
+                const unsigned ci[2] = {cp.x, cp.y}, x2 = *reinterpret_cast<const unsigned*>(&sm.stage.x[v]);
+                const unsigned slot = (in_b ? slotB : slotA) + v, to = sm.stage.tileoff[v >> 4];
 #pragma unroll
-            for (int d = 1; d < 32; d <<= 1) {
-                const unsigned u = __shfl_up_sync(0xFFFFFFFFu, inc, d);
-                if (lane >= d) inc += u;
-            }
-            below[k] = inc - c;
-            const unsigned totA = __reduce_add_sync(0xFFFFFFFFu, (v0 < vB0) ? c : 0u);
-            if (lane == 31) {
-                sm.warp_total[k][warp][0] = inc;
-                sm.warp_total[k][warp][1] = totA;
-            }
-        }
-        __syncthreads();
-        int nact, nactA_pad;
-        {
-            unsigned base[kListPasses], total = 0, realA = 0;
-#pragma unroll
-            for (int k = 0; k < kListPasses; ++k) {
-                const unsigned tl = (lane < kWarps) ? sm.warp_total[k][lane][0] : 0u;
-                const unsigned tla = (lane < kWarps) ? sm.warp_total[k][lane][1] : 0u;
-                base[k] = total + __reduce_add_sync(0xFFFFFFFFu, lane < warp ? tl : 0u);   // before my warp's unit run
-                total += __reduce_add_sync(0xFFFFFFFFu, tl);
-                realA += __reduce_add_sync(0xFFFFFFFFu, tla);                             // records of piece A
-            }
-            const unsigned pad = (ngtB > 0) ? (kGroup - realA % kGroup) % kGroup : 0u;
-            total += pad;
-            nact = static_cast<int>(total);
-            nactA_pad = (ngtB > 0) ? static_cast<int>(realA + pad) : ((nact + kGroup - 1) / kGroup) * kGroup;
-            const unsigned slotA0 = gA * kTileK - jA0, slotB0 = gB * kTileK;                 // column slot of column 0
-#pragma unroll
-            for (int k = 0; k < kListPasses; ++k) {
-                const unsigned m = m8[k];
-                if (m != 0u) {
-                    const int v0 = (k * kThreads + t) * 8;
-                    const bool inB = v0 >= vB0;
-                    const unsigned slot0 = inB ? slotB0 + (v0 - vB0) : slotA0 + jA0 + v0;   // column slot of position v0
-                    int item = static_cast<int>(base[k] + (inB ? pad : 0u) + below[k]);
-                    const unsigned to = sm.stage.tileoff[v0 >> 4];
-                    const uint4 xv = *reinterpret_cast<const uint4*>(&sm.stage.x[v0]);
-                    const uint4 c0 = *reinterpret_cast<const uint4*>(&sm.stage.colinfo[v0]);
-                    const uint4 c1 = *reinterpret_cast<const uint4*>(&sm.stage.colinfo[v0 + 4]);
-                    const unsigned xw[4] = {xv.x, xv.y, xv.z, xv.w};
-                    const unsigned ci[8] = {c0.x, c0.y, c0.z, c0.w, c1.x, c1.y, c1.z, c1.w};   // ColInfo: offset << 16 | nnz
-#pragma unroll
-                    for (int b = 0; b < 8; ++b) {
-                        if ((m >> b) & 1u) {
-                            const unsigned start = to + (ci[b] >> 16), pieces = ((ci[b] & 0xFFFFu) + 7u) >> 3;
-                            const bool ok = SPDP_CHECK(p.status, item, 1, kChunkCols, kSiteRecordIndex);
-                            if (ok && SPDP_CHECK(p.status, start, 8u * pieces, p.values_len, kSiteValuesSpan) &&
-                                SPDP_CHECK(p.status, 0, pieces, 32, kSitePieces) &&
-                                SPDP_CHECK(p.status, slot0 + b, 1, p.NGT * kTileK, kSiteBitmapSlot)) {
-                                sm.rec[item] = make_uint2(start, ((slot0 + b) << 6) | pieces);
-                                sm.xact[item] = static_cast<unsigned short>((b & 1) ? (xw[b >> 1] >> 16) : (xw[b >> 1] & 0xFFFFu));
-                            } else if (ok) {
-                                sm.rec[item] = make_uint2(0u, kNullRec);       // checked build only: the tile is left out
-                            }
-                            ++item;
-                        }
+                for (int k = 0; k < 2; ++k) {
+                    if (!(k ? k1 : k0)) continue;
+                    const unsigned start = to + (ci[k] >> 16), pieces = ((ci[k] & 0xFFFFu) + 7u) >> 3;
+                    const bool ok = SPDP_CHECK(p.status, item, 1, kChunkCols, kSiteRecordIndex);
+                    if (ok && SPDP_CHECK(p.status, start, 8u * pieces, p.values_len, kSiteValuesSpan) &&
+                        SPDP_CHECK(p.status, 0, pieces, 32, kSitePieces) &&
+                        SPDP_CHECK(p.status, slot + k, 1, p.NGT * kTileK, kSiteBitmapSlot)) {
+                        sm.rec[item] = make_uint2(start, ((slot + k) << 6) | pieces);
+                        sm.xact[item] = static_cast<unsigned short>(x2 >> (16 * k));
+                    } else if (ok) {
+                        sm.rec[item] = make_uint2(0u, kNullRec);                              // checked build only: the tile is left out
                     }
+                    ++item;
                 }
-            }
-            // null records: the padding in front of piece B and behind the last record
-            if (warp == 0 && lane < static_cast<int>(pad)) sm.rec[realA + lane] = make_uint2(0u, kNullRec);
-            if (t < kRecPad) sm.rec[nact + t] = make_uint2(0u, kNullRec);
-        }
+            });
+        const int nact = list.nact;
+        const int nactA_pad = two ? list.real_a + list.pad : ((nact + kGroup - 1) / kGroup) * kGroup;
+        // null records: the padding in front of piece B and behind the last record
+        if (warp == 0 && lane < list.pad) sm.rec[list.real_a + lane] = make_uint2(0u, kNullRec);
+        if (t < kRecPad) sm.rec[nact + t] = make_uint2(0u, kNullRec);
         __syncthreads();       // the records are complete; the staging area becomes the ring again
         const int ngroups = (nact + kGroup - 1) / kGroup;
 
@@ -505,7 +447,6 @@ spmspv_kernel(const Params p) {
         __syncthreads();       // all pipelines drained: the ring is idle
 
         // ---- (3) finish the row tiles this batch completed ----
-        const bool two = (ngtB > 0);
         const bool done_last = two ? doneB : doneA;             // does the batch's last piece end its row tile here?
         if (done_last) {
 #pragma unroll
@@ -520,9 +461,9 @@ spmspv_kernel(const Params p) {
         // batch; the other warps go straight on to the next batch's list phase.  Neither red[] nor
         // red_first[] is written again before these threads have passed the next __syncthreads.
         if (t < kTileM) {
-            if (done_last) finish_row_tile(p, two ? rB : rA, sm.red, t);
+            if (done_last) finish_row_tile(p, two ? rB : rA, sm.segments[parity][two ? 1 : 0], sm.red, t);
         } else if (t < 2 * kTileM) {
-            if (two) finish_row_tile(p, rA, sm.red_first, t - kTileM);
+            if (two) finish_row_tile(p, rA, sm.segments[parity][0], sm.red_first, t - kTileM);
         }
     }
 }

@@ -135,20 +135,6 @@ __device__ __forceinline__ void rebuild_word(unsigned (&a)[4], unsigned WA, unsi
         : "r"(WA), "r"(FA), "r"(WB), "r"(FB), "r"(below[0]), "r"(below[1]), "r"(below[2]), "r"(below[3]),
           "r"(bit[0]), "r"(bit[1]), "r"(bit[2]), "r"(bit[3]));
 }
-// The DP test of Sec. 4.2 step (3) on a pair of fp16 activations: 0xFFFF in each half whose column is
-// kept, i.e. NOT(|x| <= thr).  thr2 holds, twice, the largest fp16 value that does not exceed thr:
-// for an fp16 x that is the same test as the fp32 comparison, and "greater than or unordered" keeps
-// NaN activations and makes a NaN threshold keep everything, as the fp32 form does.
-__device__ __forceinline__ unsigned abs_gt_keep(unsigned x2, unsigned thr2) {
-    unsigned r;
-    asm("{\n .reg .b32 a;\n and.b32 a, %1, 0x7FFF7FFF;\n set.gtu.u32.f16x2 %0, a, %2;\n}" : "=r"(r) : "r"(x2), "r"(thr2));
-    return r;
-}
-__device__ __forceinline__ unsigned threshold_pair(float thr) {
-    unsigned short h;
-    asm("cvt.rm.f16.f32 %0, %1;" : "=h"(h) : "f"(thr));
-    return static_cast<unsigned>(h) * 0x00010001u;
-}
 // D += A (16 rows x 8 column tiles, fp16) * B (8 column tiles x 8 tokens, fp16), fp32 accumulate.
 __device__ __forceinline__ void mma_16x8x8(float (&c)[4], unsigned a01, unsigned a23, unsigned b01) {
     asm volatile("mma.sync.aligned.m16n8k8.row.col.f32.f16.f16.f32 {%0,%1,%2,%3}, {%4,%5}, {%6}, {%0,%1,%2,%3};"

@@ -109,6 +109,71 @@ constexpr int kSiteBitmapSlot = 4;      // column slot inside Bitmap / ColInfo
 constexpr int kSiteTreeNodes = 5;       // split-K segments of a row tile inside the workspace
 constexpr int kSiteOutputRow = 6;       // output row inside y
 
+// The DP test of Sec. 4.2 step (3) on a pair of fp16 activations: 0xFFFF in each half whose column is
+// kept, i.e. NOT(|x| <= thr).  thr2 holds, twice, the largest fp16 value that does not exceed thr:
+// for an fp16 x that is the same test as the fp32 comparison, and "greater than or unordered" keeps
+// NaN activations and makes a NaN threshold keep everything, as the fp32 form does.
+__device__ __forceinline__ unsigned abs_gt_keep(unsigned x2, unsigned thr2) {
+    unsigned r;
+    asm("{\n .reg .b32 a;\n and.b32 a, %1, 0x7FFF7FFF;\n set.gtu.u32.f16x2 %0, a, %2;\n}" : "=r"(r) : "r"(x2), "r"(thr2));
+    return r;
+}
+__device__ __forceinline__ unsigned threshold_pair(float thr) {
+    unsigned short h;
+    asm("cvt.rm.f16.f32 %0, %1;" : "=h"(h) : "f"(thr));
+    return static_cast<unsigned>(h) * 0x00010001u;
+}
+
+// Active-column list of a batch (Sec. 4.2 steps (1)-(3)).  List positions [0, nlist) hold the columns of piece A
+// ([0, nA)), then, if `two`, from vB0 (a multiple of 64) those of piece B.  keep(v) tests the two columns at positions v
+// and v + 1 (v even, also beyond the list's end) and answers in bits 0 and 31; write(item, v, k0, k1, inB) stores the records
+// of those that are kept, from record `item` on.  Records are written in list order; piece B starts on a whole group of kGroup records (`pad` null records
+// in front of it, which the caller writes).  A warp takes a contiguous run of 64-position chunks and keeps their ballots in
+// `kept` (its own shared memory, two words per chunk); the warps' totals meet in shared memory.
+// The work follows the length of the list, and the code is short: in a call of a few microseconds every line of it is
+// fetched for the first time, and what an unrolled phase skips costs as much as what it runs.  Clocks for a list of 256 /
+// 512 / 6200 columns: 8 columns per thread in two fixed passes 2300 / 2300 / 4550, one column per lane in 11 fixed steps
+// 2600 / 2600 / 4600, one column per lane in a loop 1260 / 1440 / 7200, this 1450 / 1500 / 4500 (unrolled by 4; rolled 4820).
+struct ListTotals { int nact, real_a, pad; };         // records (padding included), records of piece A, null records behind them
+template <int kWarps, int kMaxCols, int kGroup, class Keep, class Write>
+__device__ __forceinline__ ListTotals build_list(uint32_t* warp_total, uint32_t* kept, int nA, int vB0, int nlist, bool two, Keep keep,
+                                                 Write write) {
+    static_assert(kMaxCols < 65536 && kWarps <= 32, "two counts share a word; one lane per warp total");
+    static_assert((kMaxCols / 64 + kWarps - 1) / kWarps <= 16, "a warp's ballots fit 32 words");
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int chunks = (nlist + 63) >> 6, per = (chunks + kWarps - 1) / kWarps, c0 = warp * per, c1 = min(c0 + per, chunks);
+    unsigned mine = 0u;                                               // records of my chunks; upper half: those of piece A
+#pragma unroll 4
+    for (int c = c0; c < c1; ++c) {
+        const int v = c * 64 + 2 * lane;
+        const bool in_a = !two || c * 64 < vB0;
+        const int lim = in_a ? nA : nlist;
+        const unsigned k = keep(v);                                   // no branches: the lanes stay together
+        const unsigned m0 = __ballot_sync(0xFFFFFFFFu, (k & 1u) != 0u && v < lim), m1 = __ballot_sync(0xFFFFFFFFu, (k >> 31) != 0u && v + 1 < lim);
+        if (lane == 0) *reinterpret_cast<uint2*>(kept + 2 * (c - c0)) = make_uint2(m0, m1);
+        mine += (__popc(m0) + __popc(m1)) * (in_a ? 0x10001u : 1u);
+    }
+    if (lane == 0) warp_total[warp] = mine;
+    __syncthreads();
+    const unsigned w = (lane < kWarps) ? warp_total[lane] : 0u;
+    const unsigned all = __reduce_add_sync(0xFFFFFFFFu, w);
+    unsigned item0 = __reduce_add_sync(0xFFFFFFFFu, lane < warp ? w : 0u) & 0xFFFFu;
+    ListTotals r;
+    r.real_a = static_cast<int>(all >> 16);
+    r.pad = two ? (kGroup - r.real_a % kGroup) % kGroup : 0;
+    r.nact = static_cast<int>(all & 0xFFFFu) + r.pad;
+    const unsigned below = (1u << lane) - 1u;
+#pragma unroll 4
+    for (int c = c0; c < c1; ++c) {
+        const uint2 m = *reinterpret_cast<const uint2*>(kept + 2 * (c - c0));
+        const bool in_b = two && c * 64 >= vB0;
+        write(static_cast<int>(item0) + (in_b ? r.pad : 0) + __popc(m.x & below) + __popc(m.y & below), c * 64 + 2 * lane,
+              ((m.x >> lane) & 1u) != 0u, ((m.y >> lane) & 1u) != 0u, in_b);
+        item0 += __popc(m.x) + __popc(m.y);
+    }
+    return r;
+}
+
 // A partial sum is kept in the workspace XOR this key, so that the all-zero word means "empty".
 // NaN sums are made canonical first, which keeps a stored word from ever being zero.
 constexpr unsigned kNodeKey = 0xFFC0DEADu;
@@ -139,6 +204,10 @@ __device__ __forceinline__ bool tree_combine(float& part, unsigned* nodes, int64
     }
     return true;
 }
+
+// First and last CTA that feed a row tile, worked out at the start of a batch (before the wait for the previous kernel)
+// and kept in shared memory: behind the last column tile the divisions took 530 clocks.
+struct Segments { int q0, nseg; };
 
 }  // namespace dev
 }  // namespace spdp

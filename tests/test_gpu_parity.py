@@ -540,3 +540,36 @@ def test_free_of_nothing_gives_kept_memory_back(S):
     kept = torch.cuda.mem_get_info()[0]
     S.spdp_free(None)
     assert torch.cuda.mem_get_info()[0] >= kept + (16 << 20)                    # the layer's 16 MB of values at least
+
+
+@pytest.mark.parametrize("K", [1, 2, 31, 63, 64, 65, 127, 129, 1023, 3100, 8191, 8193])
+@pytest.mark.parametrize("ctas", [0, 1, 2, 5])
+def test_active_list_edges(S, K, ctas):
+    """The list phase walks pairs of columns in chunks of 64: lists that end anywhere in a chunk, ranges that hold the tail of
+    one row tile and the head of the next (CTA counts that do not divide the row tiles), every rule.  Integers: exact."""
+    rng = np.random.Generator(np.random.PCG64(K))
+    M = 700
+    W = rng.integers(-4, 5, (M, K)).astype(np.float16)
+    W[rng.random((M, K)) < 0.5] = 0
+    x = rng.integers(-3, 4, K).astype(np.float16)
+    h, h4 = S.spdp_pack_tiled_cbc(dev(W)), S.spdp_pack_tiled_cbc_q4(dev(np.clip(W, -1, 1)))   # scale 1/7: codes -7, 0, 7
+    s7 = np.float32(np.float16(1 / 7)) * np.float32(7)
+    keep = rng.random(K) < 0.4
+    try:
+        for hh, Wq, f in ((h, W, 1.0), (h4, np.clip(W, -1, 1), float(s7))):
+            S.spdp_set_num_ctas(hh, ctas)
+            for rule, thr, act in ((O.DP_NONE, 0.0, np.ones(K, bool)), (O.DP_ABS_GT, 1.0, np.abs(x) > 1), (O.DP_MASK, 0.0, keep)):
+                y = torch.full((M,), float("nan"), dtype=torch.float32, device="cuda")
+                S.spdp_spmspv(hh, dev(x), rule, thr, y, mask=dev(O.active_to_words(keep).view(np.int32)) if rule == O.DP_MASK else None)
+                torch.cuda.synchronize()
+                want = Wq.astype(np.float64) @ np.where(act, x, 0).astype(np.float64) * f
+                got = y.cpu().numpy().astype(np.float64)
+                if f == 1.0:
+                    assert np.array_equal(got, want), (rule, ctas)
+                else:                                                  # products of code 7 and scale * x: a rounding per sum
+                    scale = np.abs(Wq).astype(np.float64) @ np.abs(np.where(act, x, 0)).astype(np.float64) + 1
+                    assert np.all(np.abs(got - want) <= 2.0 ** -24 * (K + 32) * scale), (rule, ctas)
+            assert S.spdp_last_device_status(hh) == 0
+    finally:
+        S.spdp_free(h)
+        S.spdp_free(h4)
