@@ -99,6 +99,13 @@ void handle_free(void* p) {
     if (p != nullptr) cudaFreeAsync(p, nullptr);
 }
 
+void drop_host_graph(spdp_matrix* h) {
+    if (h->host_exec != nullptr) cudaGraphExecDestroy(h->host_exec);
+    if (h->host_graph != nullptr) cudaGraphDestroy(h->host_graph);
+    h->host_exec = nullptr;
+    h->host_graph = nullptr;
+}
+
 void release(spdp_matrix* h) {
     if (h == nullptr) return;
     {
@@ -111,7 +118,7 @@ void release(spdp_matrix* h) {
         cudaFree(h->probe_count);
         cudaStreamSynchronize(nullptr);
         trim_handles(h->device, kHandleKeep);
-        if (h->host_graph != nullptr) cudaGraphExecDestroy(h->host_graph);
+        drop_host_graph(h);
         if (h->capture_stream != nullptr) cudaStreamDestroy(h->capture_stream);
     }
     count_handle(h->device, -1);
@@ -179,13 +186,11 @@ spdp_status build_partition(spdp_matrix* h, int num_ctas, cudaStream_t s) {
     if (P > 1024) P = 1024;          // the kernel's range arithmetic is 32-bit: NGT < 2^22 times P must fit
     if (P > NGT) P = static_cast<int>(NGT);
     if (P < 1) P = 1;
-    if (h->host_graph != nullptr) {         // it holds the old workspace and CTA count
-        cudaGraphExecDestroy(h->host_graph);
-        h->host_graph = nullptr;
-    }
-    h->host_last_valid = false;
     handle_free(h->workspace);
     h->workspace = h->workspace_batch = nullptr;
+    // a recorded host-vector call holds the old workspace and CTA count: it is recorded anew
+    drop_host_graph(h);
+    h->host_calls = 0;
     h->num_ctas = P;
     const int64_t one = static_cast<int64_t>(P) * kTileM * sizeof(float);    // one row of split-K tree nodes per CTA
     h->workspace_bytes = one + batch_workspace_bytes(P);
@@ -247,9 +252,7 @@ spdp_status handle_alloc(int device, size_t bytes, cudaStream_t s, void** out) {
 namespace spdp {
 namespace {
 
-// copy in -> kernel -> copy out, enqueued on s.  (Letting the kernel store y straight into pinned host
-// memory and reading x through a small kernel instead of the copy engine was slower: 101 against 75 us
-// per call on the 28672 x 8192 layer.)
+// copy in -> kernel -> copy out, enqueued on s.
 spdp_status enqueue_host_call(spdp_matrix* h, const void* x_host, int rule, float thr, const void* mask_host,
                               void* y_host, int ydt, cudaStream_t s) {
     SPDP_CUDA_TRY(cudaMemcpyAsync(h->x_stage, x_host, h->K * sizeof(__half), cudaMemcpyHostToDevice, s));
@@ -264,45 +267,67 @@ spdp_status enqueue_host_call(spdp_matrix* h, const void* x_host, int rule, floa
     return SPDP_OK;
 }
 
-bool is_pinned(const void* p) {
+// The device address of pinned host memory, or null.
+void* pinned_address(const void* p) {
     cudaPointerAttributes a;
     if (cudaPointerGetAttributes(&a, p) != cudaSuccess) {
         cudaGetLastError();
-        return false;
+        return nullptr;
     }
-    return a.type == cudaMemoryTypeHost;
+    return a.type == cudaMemoryTypeHost ? a.devicePointer : nullptr;
 }
 
-bool same_key(const spdp_matrix::HostCallKey& a, const spdp_matrix::HostCallKey& b) {
-    return a.x == b.x && a.mask == b.mask && a.y == b.y && a.rule == b.rule && a.ydt == b.ydt &&
-           a.num_ctas == b.num_ctas && std::memcmp(&a.thr, &b.thr, sizeof(float)) == 0;
+// The host-vector call with pinned buffers, whose device addresses the kernels use: a small kernel fetches x (and the mask) once, the
+// decode kernel stores y over the bus.  No copy engine between the steps, and programmatic launch between the two kernels.
+// us per call, copy engine -> this: 1024x1024 31 -> 20, 11008x4096 31 -> 27, 28672x8192 68 -> 62.  (Letting every CTA of the
+// decode kernel read its part of x over the bus: 48 and 140 us on the last two, because every row tile reads x again.)
+int mask_words(const spdp_matrix* h, int rule) { return rule == SPDP_DP_MASK ? static_cast<int>((h->K + 31) / 32) : 0; }
+spdp_status enqueue_pinned_call(spdp_matrix* h, const spdp_matrix::HostCall& c, cudaStream_t s) {
+    const int words = mask_words(h, c.rule);
+    spdp_status st = launch_fetch(c.x, h->K, h->x_stage, c.mask, words, h->mask_stage, s);
+    if (st != SPDP_OK) return st;
+    return launch_decode(h, h->x_stage, c.rule, c.thr, words ? h->mask_stage : nullptr, c.y, c.ydt, s);
 }
 
-// Records the host-vector call once (on a private stream) and keeps the instantiated graph.
-spdp_status record_host_graph(spdp_matrix* h, const spdp_matrix::HostCallKey& key) {
-    if (h->host_graph != nullptr) {
-        cudaGraphExecDestroy(h->host_graph);
-        h->host_graph = nullptr;
-    }
+// Records the two kernels once (on a private stream) and keeps the instantiated graph: one launch instead of two saves
+// 4 to 6 us of a call.
+spdp_status record_host_graph(spdp_matrix* h, const spdp_matrix::HostCall& c) {
     if (h->capture_stream == nullptr)
         SPDP_CUDA_TRY(cudaStreamCreateWithFlags(&h->capture_stream, cudaStreamNonBlocking));
     SPDP_CUDA_TRY(cudaStreamBeginCapture(h->capture_stream, cudaStreamCaptureModeThreadLocal));
-    spdp_status st = enqueue_host_call(h, key.x, key.rule, key.thr, key.mask, key.y, key.ydt, h->capture_stream);
-    cudaGraph_t g = nullptr;
-    cudaError_t e = cudaStreamEndCapture(h->capture_stream, &g);
-    if (st != SPDP_OK || e != cudaSuccess || g == nullptr) {
-        if (g != nullptr) cudaGraphDestroy(g);
-        cudaGetLastError();
+    spdp_status st = enqueue_pinned_call(h, c, h->capture_stream);
+    cudaError_t e = cudaStreamEndCapture(h->capture_stream, &h->host_graph);
+    size_t roots = 1, nodes = 2;
+    cudaGraphNode_t all[2] = {};
+    if (st == SPDP_OK && e == cudaSuccess) e = cudaGraphGetRootNodes(h->host_graph, &h->host_nodes[0], &roots);
+    if (st == SPDP_OK && e == cudaSuccess) e = cudaGraphGetNodes(h->host_graph, all, &nodes);
+    if (st == SPDP_OK && e == cudaSuccess) e = (roots == 1 && nodes == 2) ? cudaGraphInstantiate(&h->host_exec, h->host_graph, 0) : cudaErrorUnknown;
+    if (st != SPDP_OK || e != cudaSuccess) {
+        if (e != cudaSuccess) note_cuda_error(e, "recording the host-vector call");
+        h->host_exec = nullptr;
+        drop_host_graph(h);
         return st != SPDP_OK ? st : SPDP_ERR_CUDA;
     }
-    e = cudaGraphInstantiate(&h->host_graph, g, 0);
-    cudaGraphDestroy(g);
-    if (e != cudaSuccess) {
-        h->host_graph = nullptr;
-        note_cuda_error(e, "cudaGraphInstantiate");
-        return SPDP_ERR_CUDA;
+    h->host_nodes[1] = all[0] == h->host_nodes[0] ? all[1] : all[0];
+    h->host_args = c;
+    return SPDP_OK;
+}
+
+// Launches the recorded graph with the arguments of this call.
+spdp_status replay_pinned_call(spdp_matrix* h, const spdp_matrix::HostCall& c, cudaStream_t s) {
+    const int words = mask_words(h, c.rule);
+    const spdp_matrix::HostCall& had = h->host_args;
+    if (c.x != had.x || c.mask != had.mask || c.rule != had.rule) {
+        const spdp_status st = set_fetch_node(h->host_exec, h->host_nodes[0], c.x, h->K, h->x_stage, c.mask, words, h->mask_stage);
+        if (st != SPDP_OK) { drop_host_graph(h); return st; }
     }
-    h->host_graph_key = key;
+    if (c.y != had.y || c.rule != had.rule || c.ydt != had.ydt || std::memcmp(&c.thr, &had.thr, sizeof(float)) != 0) {
+        const auto set = h->q4 ? set_spmspv_q4_node : set_spmspv_node;
+        const spdp_status st = set(h, h->host_exec, h->host_nodes[1], h->x_stage, c.rule, c.thr, words ? h->mask_stage : nullptr, c.y, c.ydt);
+        if (st != SPDP_OK) { drop_host_graph(h); return st; }
+    }
+    h->host_args = c;
+    SPDP_CUDA_TRY(cudaGraphLaunch(h->host_exec, s));
     return SPDP_OK;
 }
 
@@ -516,31 +541,26 @@ spdp_status spdp_spmspv_host(spdp_handle h, const void* x_host, spdp_dp_rule rul
     int dev = -1;
     if (cudaGetDevice(&dev) != cudaSuccess || dev != h->device) return SPDP_ERR_INVALID_ARG;   // wrong current device
     cudaStream_t s = static_cast<cudaStream_t>(stream);
-    // A decode loop calls this with the same pinned buffers every step.  The second call in a row with
-    // the same arguments records copy-in, kernel and copy-out as one graph; from then on the call is a
-    // single graph launch.  Anything else (pageable memory, changing buffers, a capturing stream) takes
-    // the three plain operations.
-    const spdp_matrix::HostCallKey key = {x_host, rule == SPDP_DP_MASK ? mask_host : nullptr, y_host,
-                                          static_cast<int>(rule), static_cast<int>(ydt), h->num_ctas, thr};
-    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-    const bool capturing = cudaStreamIsCapturing(s, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone;
-    bool replay = false;
-    if (!capturing) {
-        if (h->host_graph != nullptr && same_key(key, h->host_graph_key)) {
-            replay = true;
-        } else if (h->host_last_valid && same_key(key, h->host_last) && is_pinned(x_host) && is_pinned(y_host) &&
-                   (key.mask == nullptr || is_pinned(key.mask))) {
-            replay = record_host_graph(h, key) == SPDP_OK;
-        }
-    }
-    h->host_last = key;
-    h->host_last_valid = true;
-    if (replay) {
-        SPDP_CUDA_TRY(cudaGraphLaunch(h->host_graph, s));
+    // What is pinned is looked up on every call, and every call's arguments go into the recorded graph: nothing is assumed
+    // about a buffer because an earlier one had its address.
+    spdp_matrix::HostCall c = {};
+    c.rule = rule;
+    c.thr = thr;
+    c.ydt = ydt;
+    c.x = static_cast<const __half*>(pinned_address(x_host));
+    c.y = c.x != nullptr ? pinned_address(y_host) : nullptr;
+    if (rule == SPDP_DP_MASK && c.y != nullptr) c.mask = static_cast<const uint32_t*>(pinned_address(mask_host));
+    spdp_status st;
+    if (c.y == nullptr || (rule == SPDP_DP_MASK && c.mask == nullptr)) {
+        st = enqueue_host_call(h, x_host, rule, thr, mask_host, y_host, ydt, s);
     } else {
-        spdp_status st = enqueue_host_call(h, x_host, rule, thr, mask_host, y_host, ydt, s);
-        if (st != SPDP_OK) return st;
+        cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+        const bool capturing = cudaStreamIsCapturing(s, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone;
+        // a handle that is called again gets its graph (recording takes longer than one call saves)
+        if (!capturing && h->host_exec == nullptr && ++h->host_calls == 2 && record_host_graph(h, c) != SPDP_OK) cudaGetLastError();
+        st = (!capturing && h->host_exec != nullptr) ? replay_pinned_call(h, c, s) : enqueue_pinned_call(h, c, s);
     }
+    if (st != SPDP_OK) return st;
     SPDP_CUDA_TRY(cudaStreamSynchronize(s));
     return SPDP_OK;
 }

@@ -31,7 +31,49 @@ __global__ void swiglu_dp_kernel(const __half* __restrict__ gate, const __half* 
     }
 }
 
+// Fetches the vectors of a host-vector call over the bus: one 16-byte load per thread where the address allows it.
+__global__ void fetch_kernel(const __half* __restrict__ x, int K, __half* __restrict__ x_out, const uint32_t* __restrict__ mask, int mask_words,
+                             uint32_t* __restrict__ mask_out) {
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    asm volatile("griddepcontrol.wait;" ::: "memory");                  // the buffers may still be read by the call before
+    const int t = blockIdx.x * blockDim.x + threadIdx.x, n = gridDim.x * blockDim.x;
+    const bool wide = (reinterpret_cast<uintptr_t>(x) & 15u) == 0;
+    const int pieces = wide ? K / 8 : 0;
+    for (int i = t; i < pieces; i += n) reinterpret_cast<uint4*>(x_out)[i] = reinterpret_cast<const uint4*>(x)[i];
+    for (int i = 8 * pieces + t; i < K; i += n) x_out[i] = x[i];
+    for (int i = t; i < mask_words; i += n) mask_out[i] = mask[i];
+}
+
 }  // namespace
+
+constexpr int kFetchThreads = 128;
+
+spdp_status set_fetch_node(cudaGraphExec_t exec, cudaGraphNode_t node, const __half* x, int64_t K, __half* x_out, const uint32_t* mask,
+                           int mask_words, uint32_t* mask_out) {
+    int k32 = static_cast<int>(K);
+    void* args[6] = {&x, &k32, &x_out, &mask, &mask_words, &mask_out};
+    cudaKernelNodeParams k = {};
+    k.func = reinterpret_cast<void*>(fetch_kernel);
+    k.gridDim = dim3(static_cast<unsigned>((K + 8 * kFetchThreads - 1) / (8 * kFetchThreads)));
+    k.blockDim = dim3(kFetchThreads);
+    k.kernelParams = args;
+    SPDP_CUDA_TRY(cudaGraphExecKernelNodeSetParams(exec, node, &k));
+    return SPDP_OK;
+}
+
+spdp_status launch_fetch(const __half* x, int64_t K, __half* x_out, const uint32_t* mask, int mask_words, uint32_t* mask_out, cudaStream_t s) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(static_cast<unsigned>((K + 8 * kFetchThreads - 1) / (8 * kFetchThreads)));
+    cfg.blockDim = dim3(kFetchThreads);
+    cfg.stream = s;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    SPDP_CUDA_TRY(cudaLaunchKernelEx(&cfg, fetch_kernel, x, static_cast<int>(K), x_out, mask, mask_words, mask_out));
+    return SPDP_OK;
+}
 
 spdp_status launch_swiglu_dp(const __half* gate, const __half* up, int64_t K, float thr, __half* x_out, uint32_t* mask_out,
                              int* count, cudaStream_t s) {

@@ -49,19 +49,19 @@ struct spdp_matrix {
     uint32_t* mask_stage;   // device [ceil(K/32)]
     void* y_stage;          // device [M] fp32-sized
 
-    // spdp_spmspv_host with the same pinned buffers and arguments as the call before: the three
-    // operations (copy in, kernel, copy out) are kept as one instantiated graph and replayed.
-    struct HostCallKey {
-        const void* x;
-        const void* mask;
+    // spdp_spmspv_host with pinned buffers: its two kernels, recorded once as a graph whose nodes get each call's arguments.
+    struct HostCall {
+        const __half* x;                // device addresses of the pinned buffers
+        const uint32_t* mask;
         void* y;
-        int rule, ydt, num_ctas;
+        int rule, ydt;
         float thr;
     };
-    HostCallKey host_last;          // arguments of the previous host-vector call
-    bool host_last_valid;
-    HostCallKey host_graph_key;     // arguments the graph below was recorded with
-    cudaGraphExec_t host_graph;     // null: none
+    int64_t host_calls;             // pinned calls so far
+    cudaGraph_t host_graph;         // null: not recorded yet
+    cudaGraphExec_t host_exec;
+    cudaGraphNode_t host_nodes[2];  // fetch, decode
+    HostCall host_args;             // the arguments that host_exec holds
     cudaStream_t capture_stream;    // private stream used only to record that graph
 
     // Benchmark probe (spdp_probe_gather): the list of active column tiles it reads, built on first use.
@@ -122,7 +122,17 @@ spdp_status configure_spmspv_q4_kernel();      // per-device kernel attributes; 
 spdp_status launch_spmspv_q4(const spdp_matrix* h, const __half* x, int rule, float thr, const uint32_t* mask, void* y,
                              int ydt, cudaStream_t s);
 
+// The kernel of a node of an instantiated graph gets the arguments of another call on the same handle.
+spdp_status set_spmspv_node(const spdp_matrix* h, cudaGraphExec_t exec, cudaGraphNode_t node, const __half* x, int rule, float thr,
+                            const uint32_t* mask, void* y, int ydt);
+spdp_status set_spmspv_q4_node(const spdp_matrix* h, cudaGraphExec_t exec, cudaGraphNode_t node, const __half* x, int rule, float thr,
+                               const uint32_t* mask, void* y, int ydt);
+spdp_status set_fetch_node(cudaGraphExec_t exec, cudaGraphNode_t node, const __half* x, int64_t K, __half* x_out, const uint32_t* mask,
+                           int mask_words, uint32_t* mask_out);
+
 // producer.cu
+// x (and mask_words words of mask) from pinned host memory, by their device addresses, into device buffers.
+spdp_status launch_fetch(const __half* x, int64_t K, __half* x_out, const uint32_t* mask, int mask_words, uint32_t* mask_out, cudaStream_t s);
 spdp_status launch_swiglu_dp(const __half* gate, const __half* up, int64_t K, float thr, __half* x_out, uint32_t* mask_out,
                              int* count, cudaStream_t s);
 

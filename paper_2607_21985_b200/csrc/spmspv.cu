@@ -542,8 +542,7 @@ spdp_status configure_spmspv_kernel() {
     return SPDP_OK;
 }
 
-spdp_status launch_spmspv(const spdp_matrix* h, const __half* x, int rule, float thr,
-                          const uint32_t* mask, void* y, int ydt, cudaStream_t s) {
+static Params make_params(const spdp_matrix* h, const __half* x, int rule, float thr, const uint32_t* mask, void* y, int ydt) {
     Params p;
     p.tileoffset = h->tileoffset;
     p.colinfo = h->colinfo;
@@ -564,7 +563,26 @@ spdp_status launch_spmspv(const spdp_matrix* h, const __half* x, int rule, float
     p.workspace = h->workspace;
     p.status = h->status_word;
     p.values_len = h->values_len;
-    return launch_kernel(p, h->num_ctas, s);
+    return p;
+}
+
+spdp_status launch_spmspv(const spdp_matrix* h, const __half* x, int rule, float thr,
+                          const uint32_t* mask, void* y, int ydt, cudaStream_t s) {
+    return launch_kernel(make_params(h, x, rule, thr, mask, y, ydt), h->num_ctas, s);
+}
+
+spdp_status set_spmspv_node(const spdp_matrix* h, cudaGraphExec_t exec, cudaGraphNode_t node, const __half* x, int rule, float thr,
+                        const uint32_t* mask, void* y, int ydt) {
+    Params p = make_params(h, x, rule, thr, mask, y, ydt);
+    void* args[1] = {&p};
+    cudaKernelNodeParams k = {};
+    k.func = reinterpret_cast<void*>(spmspv_kernel);
+    k.gridDim = dim3(static_cast<unsigned>(h->num_ctas));
+    k.blockDim = dim3(kThreads);
+    k.sharedMemBytes = sizeof(Smem);
+    k.kernelParams = args;
+    SPDP_CUDA_TRY(cudaGraphExecKernelNodeSetParams(exec, node, &k));
+    return SPDP_OK;
 }
 
 spdp_status launch_spmspv_noalloc(const uint32_t* tileoffset, const uint32_t* colinfo, const uint64_t* bitmap,

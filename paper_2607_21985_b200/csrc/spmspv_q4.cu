@@ -459,8 +459,7 @@ spdp_status configure_spmspv_q4_kernel() {
 // The launch carries the programmatic-stream-serialization attribute, as the fp16 kernel's does: the CTAs may
 // start while the previous kernel in the stream drains, stage the matrix metadata of their range, and wait
 // for the previous kernel (griddepcontrol.wait) before they touch x, y or the workspace.
-spdp_status launch_spmspv_q4(const spdp_matrix* h, const __half* x, int rule, float thr, const uint32_t* mask, void* y,
-                             int ydt, cudaStream_t s) {
+static Params make_params(const spdp_matrix* h, const __half* x, int rule, float thr, const uint32_t* mask, void* y, int ydt) {
     Params p;
     p.tileoffset = h->tileoffset;
     p.colinfo = h->colinfo;
@@ -482,6 +481,12 @@ spdp_status launch_spmspv_q4(const spdp_matrix* h, const __half* x, int rule, fl
     p.workspace = h->workspace;
     p.status = h->status_word;
     p.values_len = h->values_len;
+    return p;
+}
+
+spdp_status launch_spmspv_q4(const spdp_matrix* h, const __half* x, int rule, float thr, const uint32_t* mask, void* y,
+                             int ydt, cudaStream_t s) {
+    const Params p = make_params(h, x, rule, thr, mask, y, ydt);
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(static_cast<unsigned>(h->num_ctas));
     cfg.blockDim = dim3(kThreads);
@@ -493,6 +498,20 @@ spdp_status launch_spmspv_q4(const spdp_matrix* h, const __half* x, int rule, fl
     cfg.attrs = attr;
     cfg.numAttrs = 1;
     SPDP_CUDA_TRY(cudaLaunchKernelEx(&cfg, spmspv_q4_kernel, p));
+    return SPDP_OK;
+}
+
+spdp_status set_spmspv_q4_node(const spdp_matrix* h, cudaGraphExec_t exec, cudaGraphNode_t node, const __half* x, int rule, float thr,
+                        const uint32_t* mask, void* y, int ydt) {
+    Params p = make_params(h, x, rule, thr, mask, y, ydt);
+    void* args[1] = {&p};
+    cudaKernelNodeParams k = {};
+    k.func = reinterpret_cast<void*>(spmspv_q4_kernel);
+    k.gridDim = dim3(static_cast<unsigned>(h->num_ctas));
+    k.blockDim = dim3(kThreads);
+    k.sharedMemBytes = sizeof(Smem);
+    k.kernelParams = args;
+    SPDP_CUDA_TRY(cudaGraphExecKernelNodeSetParams(exec, node, &k));
     return SPDP_OK;
 }
 

@@ -573,3 +573,37 @@ def test_active_list_edges(S, K, ctas):
     finally:
         S.spdp_free(h)
         S.spdp_free(h4)
+
+
+@pytest.mark.parametrize("K", [8, 1000, 4099])
+@pytest.mark.parametrize("pin_x,pin_y,shift", [(True, True, 0), (True, True, 1), (True, False, 0), (False, True, 0), (False, False, 3)])
+def test_host_vectors_buffers(S, K, pin_x, pin_y, shift):
+    """Pinned and pageable buffers in every mix, pinned x that does not start on 16 bytes, mask rule and threshold, both output
+    types; first call, recorded call and replays agree with the device-vector call bit for bit."""
+    rng = np.random.Generator(np.random.PCG64(K + shift))
+    M = 900
+    W = rng.standard_normal((M, K)).astype(np.float16)
+    W[rng.random((M, K)) < 0.5] = 0
+    x = rng.standard_normal(K).astype(np.float16)
+    words = O.active_to_words(rng.random(K) < 0.5).view(np.int32)
+    buf = torch.zeros(K + shift, dtype=torch.float16)
+    buf = buf.pin_memory() if pin_x else buf
+    xh = buf[shift:]
+    xh.copy_(torch.from_numpy(x))
+    mh = torch.from_numpy(words.copy())
+    mh = mh.pin_memory() if pin_x else mh
+    h = S.spdp_pack_tiled_cbc(dev(W))
+    try:
+        for rule, mask in ((O.DP_ABS_GT, None), (O.DP_MASK, mh)):
+            for dt in (torch.float16, torch.float32):
+                want = torch.empty(M, dtype=dt, device="cuda")
+                S.spdp_spmspv(h, dev(x), rule, 0.5, want, mask=None if mask is None else mask.cuda())
+                for k in range(4):
+                    yh = torch.full((M,), float("nan"), dtype=dt)
+                    yh = yh.pin_memory() if pin_y else yh
+                    for call in range(3):
+                        yh.fill_(float("nan"))
+                        S.spdp_spmspv_host(h, xh, rule, 0.5, yh, mask_host=mask)
+                        assert torch.equal(yh, want.cpu()), (rule, dt, k, call)
+    finally:
+        S.spdp_free(h)
