@@ -231,3 +231,26 @@ def test_batch_non_finite_values_follow_the_documented_reading(S):
     assert np.isnan(Y[1, 5]) and np.isfinite(Y_ref[1, 5])             # (a): 0 * Inf where the definition omits
     check(Y[1:2, rows], Y_ref[1:2, rows], S_ref[1:2, rows])           # ... and nowhere else
     assert np.isnan(Y[2]).all()                                       # (b): every row of the token
+
+
+@pytest.mark.parametrize("B", [3, 5, 8])
+@pytest.mark.parametrize("M,K,sp", [(256, 8, 0.0), (256, 8, 0.97), (511, 2049, 0.3), (257, 4100, 0.9), (1024, 7, 0.5), (31, 2047, 0.0)])
+def test_batch_expansion_edges(S, M, K, sp, B):
+    """Columns from empty to full (every nibble pattern and both alignments of its first value), lists that end anywhere in a
+    K-block, one to three batches per CTA.  Integers: every partial sum is exact."""
+    rng = np.random.Generator(np.random.PCG64(M + K))
+    W = rng.integers(-4, 5, (M, K)).astype(np.float16)
+    W[rng.random((M, K)) < sp] = 0
+    W[:, ::5] = np.where(rng.random((M, len(range(0, K, 5)))) < 0.95, rng.integers(1, 5, (M, len(range(0, K, 5)))), 0)   # nearly full columns
+    X = rng.integers(-3, 4, (B, K)).astype(np.float16)
+    want = np.where(np.abs(X) > 1, X, 0).astype(np.float32) @ W.astype(np.float32).T
+    h = S.spdp_pack_tiled_cbc(torch.from_numpy(W).cuda())
+    try:
+        for ctas in (0, 2):
+            S.spdp_set_num_ctas(h, ctas)
+            Y = torch.full((B, M), float("nan"), dtype=torch.float32, device="cuda")
+            S.spdp_spmspv_batch(h, torch.from_numpy(X).cuda(), O.DP_ABS_GT, 1.0, Y)
+            torch.cuda.synchronize()
+            assert np.array_equal(Y.cpu().numpy(), want)
+    finally:
+        S.spdp_free(h)
