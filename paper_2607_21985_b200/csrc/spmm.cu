@@ -296,6 +296,97 @@ __device__ __forceinline__ void store_accumulators(const Params& p, uint32_t tme
     }
 }
 
+struct alignas(16) Meta {                       // a K-block as stored, without its values
+    alignas(16) uint32_t bm[kKB][8];            // bitmaps
+    alignas(16) uint32_t ci[kKB];               // ColInfo words
+    uint32_t start[kGTB];                       // shared-memory address of each GTile's first value
+    uint32_t limit;                             // (checked build) values of the K-block
+    uint32_t vstart;                            // copy warp: virtual ring offset of its values
+    int ngt;                                    // GTiles it really has
+};
+
+// ---- the copy warp's work: stored K-blocks into a ring ----
+struct CopyState {
+    unsigned i = 0, done = 0;                               // K-blocks started / known to be decoded
+    uint32_t vhead = 0, vtail = 0, pos = 0;                 // virtual ring offsets, and vhead's position in the ring
+};
+// Starts the copies of K-blocks kb0 .. kb0 + n - 1 of the row tile whose first GTile is g_row.  The values of the blocks in
+// flight lie in a ring of bytes, so that the sparser the matrix, the more blocks are on their way; bitmaps and ColInfo in
+// kMeta slots.  The lanes hold the TileOffset words of 32 K-blocks (and of the next 32) and walk them together; one lane
+// issues.  After a failure nothing is copied any more, but every block's barrier still completes.
+template <int kMeta>
+__device__ __forceinline__ bool copy_blocks(const Params& p, CopyState& c, uint32_t ring, uint32_t ring_bytes, Meta* meta, unsigned long long* full,
+                                            unsigned long long* freed, int* abort, int64_t g_row, int kb0, int n, int lane, bool ok) {
+    uint32_t cur[kGTB + 1], nxt[kGTB + 1];
+    auto fetch = [&](int b, uint32_t (&o)[kGTB + 1]) {      // words of K-block kb0 + b + lane: its GTiles and the one after
+        const int g0 = (kb0 + b + lane) * kGTB;
+#pragma unroll
+        for (int q = 0; q <= kGTB; ++q) o[q] = (b + lane < n) ? __ldg(p.tileoffset + g_row + min(g0 + q, p.C)) : 0u;
+    };
+    fetch(0, cur);
+    for (int b = 0; b < n; b += 32) {
+        fetch(b + 32, nxt);
+        const int lim = min(32, n - b);
+        for (int q = 0; q < lim; ++q, ++c.i) {
+            uint32_t to[kGTB + 1];
+#pragma unroll
+            for (int e = 0; e <= kGTB; ++e) to[e] = __shfl_sync(0xFFFFFFFFu, cur[e], q);
+            const int g0 = (kb0 + b + q) * kGTB;
+            const int ngt = min(kGTB, p.C - g0);
+            const uint32_t nvals = to[kGTB] - to[0];
+            if (to[kGTB] < to[0] || nvals > static_cast<uint32_t>(kKB * kTileM) ||
+                static_cast<int64_t>(to[kGTB]) > p.values_len) {                        // not what the format says
+                atomicCAS(p.status, 0, SPDP_ERR_OVERFLOW);
+                *static_cast<volatile int*>(abort) = 1;                                 // the outputs stay unwritten
+                ok = false;
+            }
+            const uint32_t bytes = ok ? 2u * nvals : 0u;
+            if (c.pos + bytes > ring_bytes) {               // the values of a K-block stay in one piece
+                c.vhead += ring_bytes - c.pos;
+                c.pos = 0;
+            }
+            while (c.i - c.done >= kMeta || c.vhead + bytes - c.vtail > ring_bytes) {
+                if (c.done == c.i) { c.vtail = c.vhead; continue; }
+                if (c.done == 0u) asm volatile("griddepcontrol.wait;" ::: "memory");    // the decode waits for products, these for X
+                if (ok) ok = wait_parity(&freed[c.done % kMeta], (c.done / kMeta) & 1);
+                ++c.done;
+                c.vtail = c.done < c.i ? meta[c.done % kMeta].vstart : c.vhead;
+            }
+            ok = __all_sync(0xFFFFFFFFu, ok);
+            const unsigned m = c.i % kMeta;
+            Meta& mt = meta[m];
+            if (elect_one()) {
+                mt.vstart = c.vhead;
+                mt.ngt = ok ? ngt : 0;
+                mt.limit = nvals;
+#pragma unroll
+                for (int e = 0; e < kGTB; ++e) mt.start[e] = ring + c.pos + (ok ? 2u * (to[e] - to[0]) : 0u);
+                if (ok) {
+                    expect_bytes(&full[m], bytes + static_cast<uint32_t>(ngt) * (kTileK * 32u + kTileK * 4u));
+                    bulk_copy(smem_u32(&mt.bm[0][0]), p.bitmap + (g_row + g0) * kTileK * 4, static_cast<uint32_t>(ngt) * kTileK * 32u, &full[m]);
+                    bulk_copy(smem_u32(&mt.ci[0]), p.colinfo + (g_row + g0) * kTileK, static_cast<uint32_t>(ngt) * kTileK * 4u, &full[m]);
+                    if (bytes) bulk_copy(ring + c.pos, p.values + to[0], bytes, &full[m]);
+                } else {
+                    arrive(&full[m]);
+                }
+            }
+            __syncwarp();
+            c.vhead += ok ? bytes : 0u;
+            c.pos += ok ? bytes : 0u;
+        }
+#pragma unroll
+        for (int q = 0; q <= kGTB; ++q) cur[q] = nxt[q];
+    }
+    return ok;
+}
+// Before the CTA may leave, every copy that was started has arrived.
+template <int kMeta>
+__device__ __forceinline__ bool await_copies(const CopyState& c, unsigned long long* full) {
+    bool ok = true;
+    for (unsigned q = (c.i > kMeta ? c.i - kMeta : 0u); q < c.i; ++q) ok = wait_parity(&full[q % kMeta], (q / kMeta) & 1) && ok;
+    return ok;
+}
+
 // ===================================================================================================
 namespace one {     // one CTA = one row tile x kNI tokens
 
@@ -314,11 +405,15 @@ struct Form {
 
 // CTA w's share of the tiles that are cut along K: K-blocks [rest_begin(w), rest_begin(w + 1)).
 __device__ __forceinline__ unsigned rest_begin(const Params& p, unsigned w) {
-    return static_cast<unsigned>(static_cast<unsigned long long>(p.rest_units) * w / static_cast<unsigned>(p.sharers));
+    const unsigned sharers = static_cast<unsigned>(p.sharers);
+    if (p.rest_units <= 0xFFFFFFFFu / (sharers + 1u)) return p.rest_units * w / sharers;    // a 64-bit division takes hundreds of clocks
+    return static_cast<unsigned>(static_cast<unsigned long long>(p.rest_units) * w / sharers);
 }
 // The CTA whose share holds K-block u of them.
 __device__ __forceinline__ unsigned rest_owner(const Params& p, unsigned u) {
-    const unsigned long long num = static_cast<unsigned long long>(u + 1u) * static_cast<unsigned>(p.sharers) + p.rest_units - 1u;
+    const unsigned sharers = static_cast<unsigned>(p.sharers);
+    if (p.rest_units <= 0xFFFFFFFFu / (sharers + 1u)) return ((u + 1u) * sharers + p.rest_units - 1u) / p.rest_units - 1u;
+    const unsigned long long num = static_cast<unsigned long long>(u + 1u) * sharers + p.rest_units - 1u;
     return static_cast<unsigned>(num / p.rest_units) - 1u;
 }
 // The k-th piece of CTA w's work: K-blocks [kb0, kb0 + n) of a tile; slot = where its partial sums go, -1: the
@@ -344,15 +439,6 @@ __device__ __forceinline__ bool piece(const Params& p, int w, int k, Piece& s) {
     s.slot = (s.n == p.nkb) ? -1 : 2 * w + (t != t0 ? 1 : 0);
     return true;
 }
-
-struct alignas(16) Meta {                       // a K-block as stored, without its values
-    alignas(16) uint32_t bm[kKB][8];            // bitmaps
-    alignas(16) uint32_t ci[kKB];               // ColInfo words
-    uint32_t start[kGTB];                       // shared-memory address of each GTile's first value
-    uint32_t limit;                             // (checked build) values of the K-block
-    uint32_t vstart;                            // copy warp: virtual ring offset of its values
-    int ngt;                                    // GTiles it really has
-};
 
 template <class F>
 struct __align__(1024) Smem {
@@ -470,75 +556,11 @@ spmm_kernel(const __grid_constant__ Params p, const __grid_constant__ CUtensorMa
         __syncwarp();           // the other lanes wait here, not on a barrier in shared memory
     } else if (warp == kWarps + 1) {
         // ================= copy warp: moves the stored K-blocks =================
-        // The lanes hold the TileOffset words of 32 K-blocks (and of the next 32) and walk them together; one lane issues.
-        unsigned i = 0, done = 0;                                       // K-blocks started / known to be decoded
-        uint32_t vhead = 0, vtail = 0, pos = 0;                         // virtual ring offsets, and vhead's position in the ring
-        const uint32_t ring = smem_u32(&sm.ring[0]);
-        for (int k = 0; piece(p, me, k, s); ++k) {
-            const int64_t g_row = static_cast<int64_t>(s.tile / p.nblocks) * p.C;
-            uint32_t cur[kGTB + 1], nxt[kGTB + 1];
-            auto fetch = [&](int b, uint32_t (&o)[kGTB + 1]) {          // words of K-block kb0 + b + lane: its GTiles and the one after
-                const int g0 = (s.kb0 + b + lane) * kGTB;
-#pragma unroll
-                for (int q = 0; q <= kGTB; ++q) o[q] = (b + lane < s.n) ? __ldg(p.tileoffset + g_row + min(g0 + q, p.C)) : 0u;
-            };
-            fetch(0, cur);
-            for (int b = 0; b < s.n; b += 32) {
-                fetch(b + 32, nxt);
-                const int lim = min(32, s.n - b);
-                for (int q = 0; q < lim; ++q, ++i) {
-                    uint32_t to[kGTB + 1];
-#pragma unroll
-                    for (int e = 0; e <= kGTB; ++e) to[e] = __shfl_sync(0xFFFFFFFFu, cur[e], q);
-                    const int g0 = (s.kb0 + b + q) * kGTB;
-                    const int ngt = min(kGTB, p.C - g0);
-                    const uint32_t nvals = to[kGTB] - to[0];
-                    if (to[kGTB] < to[0] || nvals > static_cast<uint32_t>(kKB * kTileM) ||
-                        static_cast<int64_t>(to[kGTB]) > p.values_len) {                // not what the format says
-                        atomicCAS(p.status, 0, SPDP_ERR_OVERFLOW);
-                        *static_cast<volatile int*>(&sm.abort) = 1;                     // the outputs stay unwritten
-                        ok = false;
-                    }
-                    const uint32_t bytes = ok ? 2u * nvals : 0u;
-                    if (pos + bytes > kRingBytes<F>) {                  // the values of a K-block stay in one piece
-                        vhead += kRingBytes<F> - pos;
-                        pos = 0;
-                    }
-                    while (i - done >= F::kMeta || vhead + bytes - vtail > kRingBytes<F>) {
-                        if (done == i) { vtail = vhead; continue; }
-                        if (done == 0u) asm volatile("griddepcontrol.wait;" ::: "memory");      // the decode waits for products, these for X
-                        if (ok) ok = wait_parity(&sm.comp_free[done % F::kMeta], (done / F::kMeta) & 1);
-                        ++done;
-                        vtail = done < i ? sm.meta[done % F::kMeta].vstart : vhead;
-                    }
-                    ok = __all_sync(0xFFFFFFFFu, ok);
-                    const unsigned m = i % F::kMeta;
-                    Meta& mt = sm.meta[m];
-                    if (elect_one()) {
-                        mt.vstart = vhead;
-                        mt.ngt = ok ? ngt : 0;                          // after a failure nothing is copied any more
-                        mt.limit = nvals;
-#pragma unroll
-                        for (int e = 0; e < kGTB; ++e) mt.start[e] = ring + pos + (ok ? 2u * (to[e] - to[0]) : 0u);
-                        if (ok) {
-                            expect_bytes(&sm.comp_full[m], bytes + static_cast<uint32_t>(ngt) * (kTileK * 32u + kTileK * 4u));
-                            bulk_copy(smem_u32(&mt.bm[0][0]), p.bitmap + (g_row + g0) * kTileK * 4, static_cast<uint32_t>(ngt) * kTileK * 32u, &sm.comp_full[m]);
-                            bulk_copy(smem_u32(&mt.ci[0]), p.colinfo + (g_row + g0) * kTileK, static_cast<uint32_t>(ngt) * kTileK * 4u, &sm.comp_full[m]);
-                            if (bytes) bulk_copy(ring + pos, p.values + to[0], bytes, &sm.comp_full[m]);
-                        } else {
-                            arrive(&sm.comp_full[m]);
-                        }
-                    }
-                    __syncwarp();
-                    vhead += ok ? bytes : 0u;
-                    pos += ok ? bytes : 0u;
-                }
-#pragma unroll
-                for (int q = 0; q <= kGTB; ++q) cur[q] = nxt[q];
-            }
-        }
-        // before the CTA may leave, every copy that was started has arrived
-        for (unsigned q = (i > F::kMeta ? i - F::kMeta : 0u); q < i; ++q) ok = wait_parity(&sm.comp_full[q % F::kMeta], (q / F::kMeta) & 1) && ok;
+        CopyState cs;
+        for (int k = 0; piece(p, me, k, s); ++k)
+            ok = copy_blocks<F::kMeta>(p, cs, smem_u32(&sm.ring[0]), kRingBytes<F>, sm.meta, sm.comp_full, sm.comp_free, &sm.abort,
+                                       static_cast<int64_t>(s.tile / p.nblocks) * p.C, s.kb0, s.n, lane, ok);
+        ok = await_copies<F::kMeta>(cs, sm.comp_full) && ok;
         __syncwarp();
     } else if (warp == kWarps + 2) {
         // ================= X warp: one thread moves the X tiles =================
@@ -641,8 +663,10 @@ reduce_pieces_kernel(const Params p, int tile0, int tiles, int tile_tokens) {
         const int64_t row = static_cast<int64_t>(tile / p.nblocks) * kTileM + row_in;
         if (n >= p.N || row >= p.M) continue;
         float4 sum = make_float4(0.f, 0.f, 0.f, 0.f);
+        const unsigned first_slot = 2u * first + (rest_begin(p, first) < t * nkb ? 1u : 0u);     // the only one that may start in the tile before
+#pragma unroll 4
         for (unsigned w = first; w <= last; ++w) {
-            const unsigned slot = 2u * w + (rest_begin(p, w) / nkb != t ? 1u : 0u);
+            const unsigned slot = w == first ? first_slot : 2u * w;
             const float4 v = *reinterpret_cast<const float4*>(p.partial + (static_cast<size_t>(slot) * p.ptok + tok) * kTileM + row_in);
             sum.x += v.x;
             sum.y += v.y;
@@ -664,78 +688,38 @@ namespace pair {    // two CTAs (a cluster of 2) = one row tile x 512 tokens
 constexpr int kNI = 256;                      // the N of the tensor-core instruction
 constexpr int kTmemCols = 512;
 constexpr int kATileBytes = (kKB / 8) * kAKGroupStride;    // 128 rows x kKB columns
-constexpr int kCompValues = kKB * kTileM;     // the most values a K-block stores
+constexpr int kThreads = (kWarps + 4) * 32;   // decode, tensor-core, copy, relay and X warps
 constexpr int kNTiles = 2;                    // accumulators per CTA
 constexpr int kNT = kNTiles * kNI;            // tokens per CTA pair
-constexpr int kStages = 3;                    // operand tiles (decoded W, X) in flight
-constexpr int kCStages = 2;                   // stored K-blocks in flight
+constexpr int kStages = 3;                    // decoded W in flight
+constexpr int kXStages = 2;                   // X tiles in flight
+constexpr int kMeta = 6;                      // stored K-blocks in flight, at most
 constexpr int kBTileBytes = (kNI / 2) * kBRowBytes;    // this CTA's 128 tokens of one X tile
 constexpr int kBBytes = kNTiles * kBTileBytes;
 static_assert(kNTiles * kNI == kTmemCols, "the accumulators fill tensor memory");
 
-struct CompStage {                              // one K-block as stored
-    alignas(128) unsigned short vals[kCompValues + 16];   // the values of its 4 GTiles, contiguous
-    alignas(16) uint32_t bm[kKB][8];            // bitmaps
-    alignas(16) uint32_t ci[kKB];               // ColInfo words
-    uint32_t start[kGTB];                       // shared-memory address of each GTile's first value
-    uint32_t limit;                             // (checked build) values of the block
-};
-static_assert(offsetof(CompStage, bm) % 16 == 0 && offsetof(CompStage, ci) % 16 == 0 && sizeof(CompStage) % 16 == 0,
-              "bulk copies need 16-byte aligned destinations");
-
-// TileOffset words of K-block kb of row tile r: its GTiles and the one after (Sec. 4.1); a short last block
-// repeats its end.
-struct Offsets { uint32_t to[kGTB + 1]; };
-__device__ __forceinline__ Offsets fetch_offsets(const Params& p, int r, int nkb, int kb) {
-    Offsets o;
-#pragma unroll
-    for (int i = 0; i <= kGTB; ++i) o.to[i] = 0u;
-    if (kb < nkb) {
-        const int ngt = min(kGTB, p.C - kGTB * kb);
-        const uint32_t* src = p.tileoffset + static_cast<int64_t>(r) * p.C + kGTB * kb;
-#pragma unroll
-        for (int i = 0; i <= kGTB; ++i) o.to[i] = __ldg(src + min(i, ngt));
-    }
-    return o;
-}
-// Starts the copies of the stored K-block kb of row tile r: Values, Bitmap and ColInfo of its GTiles, three
-// contiguous spans (Sec. 4.1).  Returns false (and copies no values) if TileOffset is not what the format says.
-__device__ __forceinline__ bool load_comp(const Params& p, int r, int kb, const Offsets& o, CompStage& cs,
-                                          unsigned long long* bar) {
-    const int ngt = min(kGTB, p.C - kGTB * kb);
-    const int64_t g0 = static_cast<int64_t>(r) * p.C + kGTB * kb;
-    uint32_t nvals = o.to[kGTB] - o.to[0];
-    bool good = true;
-    if (o.to[kGTB] < o.to[0] || nvals > static_cast<uint32_t>(kCompValues) || static_cast<int64_t>(o.to[kGTB]) > p.values_len) {
-        atomicCAS(p.status, 0, SPDP_ERR_OVERFLOW);
-        good = false;
-        nvals = 0u;
-    }
-#pragma unroll
-    for (int i = 0; i < kGTB; ++i) cs.start[i] = smem_u32(&cs.vals[0]) + (nvals ? 2u * (o.to[i] - o.to[0]) : 0u);
-    cs.limit = nvals;
-    expect_bytes(bar, 2u * nvals + static_cast<uint32_t>(ngt) * (kTileK * 32u + kTileK * 4u));
-    if (nvals) bulk_copy(smem_u32(&cs.vals[0]), p.values + o.to[0], 2u * nvals, bar);
-    bulk_copy(smem_u32(&cs.bm[0][0]), p.bitmap + g0 * kTileK * 4, static_cast<uint32_t>(ngt) * kTileK * 32u, bar);
-    bulk_copy(smem_u32(&cs.ci[0]), p.colinfo + g0 * kTileK, static_cast<uint32_t>(ngt) * kTileK * 4u, bar);
-    return good;
-}
-
 struct __align__(1024) Smem {
-    unsigned char B[kStages][kBBytes];              // my halves of the X tiles (each on a 1024-byte boundary: swizzle atoms)
+    unsigned char B[kXStages][kBBytes];             // my halves of the X tiles (each on a 1024-byte boundary: swizzle atoms)
     unsigned char A[kStages][kATileBytes];          // decoded W: my 128 rows
-    CompStage comp[kCStages];
+    Meta meta[kMeta];
     alignas(8) unsigned long long mma_done[kStages];    // the tensor cores are done with A stage s and B stage s (both CTAs)
-    alignas(8) unsigned long long a_ready[kStages];     // my decode warps have written A stage s (and read the stored block)
+    alignas(8) unsigned long long comp_free[kMeta];     // my decode warps are done with the stored K-block
     alignas(8) unsigned long long ready[kStages];       // A stage s is written and my X tiles of B stage s have arrived
                                                         // (first CTA: and the second CTA says the same of its own)
-    alignas(8) unsigned long long comp_full[kCStages];  // the stored K-block of comp stage s has arrived
+    alignas(8) unsigned long long comp_full[kMeta];     // the stored K-block has arrived
     alignas(16) uint2 tab[kWarps][32];              // per warp: bitmap word and the address of its first value
     uint32_t tmem_base;
     int abort;
+    alignas(128) unsigned char ring[1];                 // values of the K-blocks in flight (fills the rest).  With two fixed
+                                                        // stages of a full K-block's size the decode waited for copies, and with
+                                                        // three X stages the ring is short of space where the matrix is dense.
+                                                        // us, fixed stages / ring, 3 X / ring, 2 X: 28672x8192 x 1024 at 50 %
+                                                        // 410 / 394 / 397, 4001x4096 x 300 at 30 % 31 / 38 / 30, 4096x4096 x 1024
+                                                        // 53 / 57 / 50
 };
-constexpr size_t kSmemBytes = sizeof(Smem) + 1024;      // the dynamic shared memory is aligned by hand
-static_assert(kSmemBytes <= 227 * 1024, "shared memory of one CTA");
+constexpr size_t kSmemBytes = 227 * 1024;               // the dynamic shared memory is aligned by hand
+constexpr uint32_t kRingBytes = (static_cast<uint32_t>(kSmemBytes) - 1024u - static_cast<uint32_t>(offsetof(Smem, ring)) - 64u) / 128u * 128u;
+static_assert(kRingBytes >= 2 * kKB * kTileM, "the ring holds at least one full K-block");
 static_assert(kBTileBytes % 1024 == 0, "every X tile on a swizzle-atom boundary");
 
 __global__ void __launch_bounds__(kThreads, 1)
@@ -757,12 +741,14 @@ spmm_kernel(const __grid_constant__ Params p, const __grid_constant__ CUtensorMa
 #pragma unroll
         for (int s = 0; s < kStages; ++s) {
             barrier_init(&sm.mma_done[s], 1);
-            barrier_init(&sm.a_ready[s], kBlockWarps);
             // arrivals on ready[]: my decode warps, my copy thread (with the X tiles' bytes), in the first CTA the second CTA
             barrier_init(&sm.ready[s], kBlockWarps + 1 + (c == 0 ? 1 : 0));
         }
 #pragma unroll
-        for (int s = 0; s < kCStages; ++s) barrier_init(&sm.comp_full[s], 1);
+        for (int s = 0; s < kMeta; ++s) {
+            barrier_init(&sm.comp_full[s], 1);
+            barrier_init(&sm.comp_free[s], kBlockWarps);
+        }
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         sm.abort = 0;
     }
@@ -794,7 +780,7 @@ spmm_kernel(const __grid_constant__ Params p, const __grid_constant__ CUtensorMa
                 if (ok) ok = wait_parity(&sm.ready[s], (kb / kStages) & 1);      // both CTAs' decoded W tiles and X tiles are in place
                 asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
                 const uint64_t ad0 = operand_desc(smem_u32(&sm.A[s][0]), kAKGroupStride, kAChunkStride, 0u);
-                const uint64_t bd0 = operand_desc(smem_u32(&sm.B[s][0]), 16, kBAtomBytes, 2u);
+                const uint64_t bd0 = operand_desc(smem_u32(&sm.B[kb % kXStages][0]), 16, kBAtomBytes, 2u);
                 for (int i = 0; i < ntiles; ++i) {
 #pragma unroll
                     for (int kk = 0; kk < kKB / 16; ++kk)    // the start address is the descriptor's low field, in 16-byte units
@@ -813,32 +799,22 @@ spmm_kernel(const __grid_constant__ Params p, const __grid_constant__ CUtensorMa
         }
         __syncwarp();           // the other lanes wait here, not on a barrier in shared memory
     } else if (warp == kWarps + 1) {
-        // ================= copy warp: one thread moves the stored K-blocks and my halves of the X tiles =================
+        // ================= copy warp: moves the stored K-blocks =================
+        CopyState cs;
+        ok = copy_blocks<kMeta>(p, cs, smem_u32(&sm.ring[0]), kRingBytes, sm.meta, sm.comp_full, sm.comp_free, &sm.abort,
+                                static_cast<int64_t>(r) * p.C, kb0, nkb, lane, ok);
+        ok = await_copies<kMeta>(cs, sm.comp_full) && ok;
+        __syncwarp();
+    } else if (warp == kWarps + 3) {
+        // ================= X warp: one thread moves my halves of the X tiles =================
         if (elect_one()) {
-            // my 128 tokens of the X tiles of K-block kb: one tiled bulk-tensor copy per tile
-            auto load_x = [&](int kb) {
-                unsigned long long* bar = &sm.ready[kb % kStages];
-                expect_bytes(bar, static_cast<uint32_t>(ntiles) * kBTileBytes);
-                for (int i = 0; i < ntiles; ++i)
-                    tensor_copy(&sm.B[kb % kStages][i * kBTileBytes], &xmap, (kb0 + kb) * kKB, static_cast<int>(n0) + i * kNI + c * (kNI / 2), bar);
-            };
-            for (int kb = 0; kb < kCStages && kb < nkb; ++kb)
-                ok = load_comp(p, r, kb0 + kb, fetch_offsets(p, r, nkb_all, kb0 + kb), sm.comp[kb % kCStages], &sm.comp_full[kb % kCStages]) && ok;
-            for (int kb = 0; kb < kStages && kb < nkb; ++kb) load_x(kb);
-            Offsets next = fetch_offsets(p, r, nkb_all, kb0 + kCStages);
             for (int kb = 0; kb < nkb; ++kb) {
-                // the stored block kb + kCStages goes where block kb was decoded from, once my decode warps are done with it
-                if (kb + kCStages < nkb) {
-                    if (ok) ok = wait_parity(&sm.a_ready[kb % kStages], (kb / kStages) & 1);
-                    ok = load_comp(p, r, kb0 + kb + kCStages, next, sm.comp[kb % kCStages], &sm.comp_full[kb % kCStages]) && ok;
-                    next = fetch_offsets(p, r, nkb_all, kb0 + kb + kCStages + 1);
-                }
-                // my X tiles of block kb + 1 go where block kb + 1 - kStages multiplied from, once that work is complete
-                const int kx = kb + 1;
-                if (kx >= kStages && kx < nkb) {
-                    if (ok) ok = wait_parity(&sm.mma_done[kx % kStages], ((kx / kStages) - 1) & 1);
-                    load_x(kx);
-                }
+                // my X tiles of block kb go where block kb - kXStages multiplied from, once that work is complete
+                const int s = kb % kStages, before = kb - kXStages;
+                if (before >= 0 && ok) ok = wait_parity(&sm.mma_done[before % kStages], (before / kStages) & 1);
+                expect_bytes(&sm.ready[s], static_cast<uint32_t>(ntiles) * kBTileBytes);
+                for (int i = 0; i < ntiles; ++i)            // my 128 tokens of each tile: one tiled bulk-tensor copy
+                    tensor_copy(&sm.B[kb % kXStages][i * kBTileBytes], &xmap, (kb0 + kb) * kKB, static_cast<int>(n0) + i * kNI + c * (kNI / 2), &sm.ready[s]);
             }
         }
         __syncwarp();
@@ -861,10 +837,11 @@ spmm_kernel(const __grid_constant__ Params p, const __grid_constant__ CUtensorMa
         const uint32_t a_lane = pinned(smem_u32(&sm.A[0][0]) + (lane >> 1) * kAChunkStride + (lane & 1) * 8);
         for (unsigned i = group; i < static_cast<unsigned>(nkb) * kSubs; i += kGroups) {
             const unsigned kb = i / kSubs, s = kb % kStages, j0 = (i % kSubs) * kSub + 4u * wm;      // my first column of the K-block
-            if (ok) ok = wait_parity(&sm.comp_full[kb % kCStages], (kb / kCStages) & 1);    // the stored block has arrived
-            const CompStage& cs = sm.comp[kb % kCStages];
+            const unsigned m = kb % kMeta;
+            if (ok) ok = wait_parity(&sm.comp_full[m], (kb / kMeta) & 1);                   // the stored block has arrived
+            const Meta& mt = sm.meta[m];
             __syncwarp();
-            scan4(p, cs.bm, cs.ci, cs.start, min(kGTB, p.C - kGTB * (kb0 + static_cast<int>(kb))), cs.limit, static_cast<int>(j0), lane, &sm.tab[warp][0]);
+            scan4(p, mt.bm, mt.ci, mt.start, mt.ngt, mt.limit, static_cast<int>(j0), lane, &sm.tab[warp][0]);
             __syncwarp();
             if (kb >= kStages && ok) ok = wait_parity(&sm.mma_done[s], ((kb / kStages) & 1u) ^ 1u);  // the tensor cores are done with this A stage
             expand4<4, 1>(tab_l, a_lane + s * kATileBytes + (j0 >> 3) * kAKGroupStride + (j0 & 7u) * 16u, 0u, below, sh);
@@ -872,7 +849,7 @@ spmm_kernel(const __grid_constant__ Params p, const __grid_constant__ CUtensorMa
             asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
             __syncwarp();
             if (lane == 0) {
-                arrive(&sm.a_ready[s]);
+                arrive(&sm.comp_free[m]);
                 arrive(&sm.ready[s]);
             }
         }
@@ -888,7 +865,7 @@ spmm_kernel(const __grid_constant__ Params p, const __grid_constant__ CUtensorMa
     __syncthreads();
 
     // ---- epilogue.  Warp w reads lanes 32*(w%4).. (my rows 32*(w%4)..), token columns [(w/4)*128, +128) of the 512 ----
-    if (!sm.abort && warp < kStoreWarps) {
+    if (!*static_cast<volatile int*>(&sm.abort) && warp < kStoreWarps) {
         const int lane_base = 32 * (warp & 3), cbase = (warp >> 2) * (kNT / 4);
         store_accumulators(p, tmem, lane_base, cbase, cbase + kNT / 4, r, c * 128 + lane_base + lane, n0,
                            p.partial == nullptr ? -1 : static_cast<int>(pr));
@@ -995,13 +972,16 @@ struct Plan {
     int workers, rounds, sharers, slices;
     int64_t tiles, rest;
 };
-constexpr double kBlockUs[4] = {1.02, 1.02, 1.15, 0.98};  // a K-block (64 columns x 256 rows x the kernel's tokens), us
-constexpr double kTileUs = 3.0;                           // a tile's start and end
-constexpr double kReduceUs = 2.5, kReducePerMB = 0.45;    // the second kernel; writing and reading a MB of partial sums
+// The estimate of a call's time: (K-blocks of the busiest CTA) x (time of a K-block) + a tile's start and end + what the
+// partial sums cost.  Fitted to the four kernels' times on 7 layers from 512x512 to 28672x2048 with 16 to 1000 tokens each
+// (50 % density; within 7 % on average): the choice costs 0.8 % on average against the best of the four, 12 % at worst.
+constexpr double kCallUs = 3.1;                                         // a call's fixed part
+constexpr double kBlockUs[4] = {0.96, 0.97, 1.19, 0.75};                // a K-block (64 columns x 256 rows), us
+constexpr double kBlockTokenUs[4] = {5.7e-4, 2.6e-4, 0.0, 3.9e-4};      // and per token of the tile
+constexpr double kTileUs = 2.8, kTileTokenUs = 5.7e-3;                  // a tile's start and end, and per token
+constexpr double kReduceUs = 2.5, kReducePerMB = 0.285;                 // the second kernel; writing and reading a MB of partial sums
 constexpr int kTokens[4] = {One32::kNI, One128::kNI, One256::kNI, pair::kNT};
 
-// The estimate of a call's time is (K-blocks of the busiest CTA) x (time of a K-block) + what the partial sums cost on
-// their way through memory.
 Plan make_plan(int64_t R, int64_t nkb, int64_t N, int sms) {
     Plan best = {};
     best.us = -1.0;
@@ -1014,14 +994,15 @@ Plan make_plan(int64_t R, int64_t nkb, int64_t N, int sms) {
         q.tiles = R * ((N + kTokens[f] - 1) / kTokens[f]);
         const int64_t slots = f == 3 ? sms / 2 : sms;                            // CTAs or pairs resident at once
         const int64_t rounds = q.tiles / slots, left = q.tiles - rounds * slots;
-        const double mb = static_cast<double>(std::min<int64_t>(N, kTokens[f])) * kTileM * 4.0e-6;   // MB of a tile's sums
-        const double whole = (kBlockUs[f] * static_cast<double>(nkb) + kTileUs) * static_cast<double>(rounds);
+        const double tok = static_cast<double>(std::min<int64_t>(N, kTokens[f])), mb = tok * kTileM * 4.0e-6;   // MB of a tile's sums
+        const double block = kBlockUs[f] + kBlockTokenUs[f] * tok, tile = kTileUs + kTileTokenUs * tok;
+        const double whole = kCallUs + (block * static_cast<double>(nkb) + tile) * static_cast<double>(rounds);
         q.rounds = static_cast<int>(rounds);
         q.slices = 1;
         q.sharers = left > 0 ? static_cast<int>(left) : 1;
         q.workers = static_cast<int>(rounds > 0 ? slots : left);
         q.rest = f == 3 ? 0 : left;
-        q.us = whole + (left > 0 ? kBlockUs[f] * static_cast<double>(nkb) + kTileUs : 0.0);
+        q.us = whole + (left > 0 ? block * static_cast<double>(nkb) + tile : 0.0);
         if (best.us < 0.0 || q.us < best.us) best = q;
         if (left == 0) continue;
         for (int64_t share = 2 * left; share < 2 * slots; share *= 2) {          // more CTAs (pairs) than tiles
@@ -1034,8 +1015,7 @@ Plan make_plan(int64_t R, int64_t nkb, int64_t N, int sms) {
             if (w <= left || w > left * nkb) break;
             q.sharers = static_cast<int>(w);
             q.workers = static_cast<int>(rounds > 0 ? slots : w);
-            q.us = whole + kBlockUs[f] * static_cast<double>((left * nkb + w - 1) / w) + kTileUs + kReduceUs +
-                   (f == 3 && rounds > 0 ? kTileUs : 0.0) + kReducePerMB * mb * static_cast<double>(w + left);
+            q.us = whole + block * static_cast<double>((left * nkb + w - 1) / w) + tile + kReduceUs + kReducePerMB * mb * static_cast<double>(w + left);
             if (q.us < best.us) best = q;
         }
     }
@@ -1061,7 +1041,7 @@ spdp_status launch_one(const Params& p, const CUtensorMap& xmap, cudaStream_t s)
 spdp_status launch_pairs(const Params& p, const CUtensorMap& xmap, int64_t pairs, cudaStream_t s) {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(static_cast<unsigned>(2 * pairs));
-    cfg.blockDim = dim3(kThreads);
+    cfg.blockDim = dim3(pair::kThreads);
     cfg.dynamicSmemBytes = pair::kSmemBytes;
     cfg.stream = s;
     cudaLaunchAttribute attr[1];
