@@ -692,12 +692,13 @@ constexpr int kThreads = (kWarps + 4) * 32;   // decode, tensor-core, copy, rela
 constexpr int kNTiles = 2;                    // accumulators per CTA
 constexpr int kNT = kNTiles * kNI;            // tokens per CTA pair
 constexpr int kStages = 3;                    // decoded W in flight
-constexpr int kXStages = 2;                   // X tiles in flight
 constexpr int kMeta = 6;                      // stored K-blocks in flight, at most
 constexpr int kBTileBytes = (kNI / 2) * kBRowBytes;    // this CTA's 128 tokens of one X tile
 constexpr int kBBytes = kNTiles * kBTileBytes;
 static_assert(kNTiles * kNI == kTmemCols, "the accumulators fill tensor memory");
 
+// kXStages = X tiles in flight
+template <int kXStages>
 struct __align__(1024) Smem {
     unsigned char B[kXStages][kBBytes];             // my halves of the X tiles (each on a 1024-byte boundary: swizzle atoms)
     unsigned char A[kStages][kATileBytes];          // decoded W: my 128 rows
@@ -711,21 +712,24 @@ struct __align__(1024) Smem {
     uint32_t tmem_base;
     int abort;
     alignas(128) unsigned char ring[1];                 // values of the K-blocks in flight (fills the rest).  With two fixed
-                                                        // stages of a full K-block's size the decode waited for copies, and with
-                                                        // three X stages the ring is short of space where the matrix is dense.
-                                                        // us, fixed stages / ring, 3 X / ring, 2 X: 28672x8192 x 1024 at 50 %
-                                                        // 410 / 394 / 397, 4001x4096 x 300 at 30 % 31 / 38 / 30, 4096x4096 x 1024
-                                                        // 53 / 57 / 50
+                                                        // stages of a full K-block's size the decode waited for copies:
+                                                        // 28672x8192 x 1024 at 50 % 410 us, this 397
 };
 constexpr size_t kSmemBytes = 227 * 1024;               // the dynamic shared memory is aligned by hand
-constexpr uint32_t kRingBytes = (static_cast<uint32_t>(kSmemBytes) - 1024u - static_cast<uint32_t>(offsetof(Smem, ring)) - 64u) / 128u * 128u;
-static_assert(kRingBytes >= 2 * kKB * kTileM, "the ring holds at least one full K-block");
+template <int kXStages>
+constexpr uint32_t kRingBytes = (static_cast<uint32_t>(kSmemBytes) - 1024u - static_cast<uint32_t>(offsetof(Smem<kXStages>, ring)) - 64u) / 128u * 128u;
+// A third X tile in flight pays where the ring still holds four K-blocks beside it; where it does not, the decode waits for
+// copies instead.  us with 2 / 3 X tiles, 18944x3872 x 416 tokens at 67 %: 66 / 60; 18944x4096 x 512 at 90, 50, 30 %: 70 / 62,
+// 71 / 70, 74 / 85; 4096x4096 x 1024 at 50 %: 50 / 57.
+constexpr int64_t kThirdXBytes = 13 * 1024;             // bytes of values per K-block up to which there are three
 static_assert(kBTileBytes % 1024 == 0, "every X tile on a swizzle-atom boundary");
 
+template <int kXStages>
 __global__ void __launch_bounds__(kThreads, 1)
 spmm_kernel(const __grid_constant__ Params p, const __grid_constant__ CUtensorMap xmap) {
+    static_assert(kRingBytes<kXStages> >= 2 * kKB * kTileM, "the ring holds at least one full K-block");
     extern __shared__ unsigned char smem_raw[];
-    Smem& sm = *reinterpret_cast<Smem*>(smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u));
+    Smem<kXStages>& sm = *reinterpret_cast<Smem<kXStages>*>(smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u));
     const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
     const int c = static_cast<int>(blockIdx.x & 1u);                  // my rank in the pair = my half of the row tile
     const unsigned pr = blockIdx.x >> 1;
@@ -801,7 +805,7 @@ spmm_kernel(const __grid_constant__ Params p, const __grid_constant__ CUtensorMa
     } else if (warp == kWarps + 1) {
         // ================= copy warp: moves the stored K-blocks =================
         CopyState cs;
-        ok = copy_blocks<kMeta>(p, cs, smem_u32(&sm.ring[0]), kRingBytes, sm.meta, sm.comp_full, sm.comp_free, &sm.abort,
+        ok = copy_blocks<kMeta>(p, cs, smem_u32(&sm.ring[0]), kRingBytes<kXStages>, sm.meta, sm.comp_full, sm.comp_free, &sm.abort,
                                 static_cast<int64_t>(r) * p.C, kb0, nkb, lane, ok);
         ok = await_copies<kMeta>(cs, sm.comp_full) && ok;
         __syncwarp();
@@ -925,8 +929,8 @@ spdp_status configure_spmm_kernel() {
         SPDP_CUDA_TRY(cudaFuncSetAttribute(one::spmm_kernel<One32>, cudaFuncAttributeMaxDynamicSharedMemorySize, one::kSmemBytes));
         SPDP_CUDA_TRY(cudaFuncSetAttribute(one::spmm_kernel<One128>, cudaFuncAttributeMaxDynamicSharedMemorySize, one::kSmemBytes));
         SPDP_CUDA_TRY(cudaFuncSetAttribute(one::spmm_kernel<One256>, cudaFuncAttributeMaxDynamicSharedMemorySize, one::kSmemBytes));
-        SPDP_CUDA_TRY(cudaFuncSetAttribute(pair::spmm_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                           static_cast<int>(pair::kSmemBytes)));
+        SPDP_CUDA_TRY(cudaFuncSetAttribute(pair::spmm_kernel<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(pair::kSmemBytes)));
+        SPDP_CUDA_TRY(cudaFuncSetAttribute(pair::spmm_kernel<3>, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(pair::kSmemBytes)));
         configured[dev] = true;
     }
     return SPDP_OK;
@@ -1038,7 +1042,7 @@ spdp_status launch_one(const Params& p, const CUtensorMap& xmap, cudaStream_t s)
     return SPDP_OK;
 }
 
-spdp_status launch_pairs(const Params& p, const CUtensorMap& xmap, int64_t pairs, cudaStream_t s) {
+spdp_status launch_pairs(const Params& p, const CUtensorMap& xmap, int64_t pairs, int64_t block_bytes, cudaStream_t s) {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(static_cast<unsigned>(2 * pairs));
     cfg.blockDim = dim3(pair::kThreads);
@@ -1051,7 +1055,7 @@ spdp_status launch_pairs(const Params& p, const CUtensorMap& xmap, int64_t pairs
     attr[0].val.clusterDim.z = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    SPDP_CUDA_TRY(cudaLaunchKernelEx(&cfg, pair::spmm_kernel, p, xmap));
+    SPDP_CUDA_TRY(cudaLaunchKernelEx(&cfg, block_bytes <= pair::kThirdXBytes ? pair::spmm_kernel<3> : pair::spmm_kernel<2>, p, xmap));
     return SPDP_OK;
 }
 
@@ -1090,13 +1094,14 @@ spdp_status launch_spmm(const spdp_matrix* h, const __half* X, int64_t N, int64_
         if (st != SPDP_OK) return st;
     }
     if (plan.kernel == 3) {
+        const int64_t block_bytes = 2 * h->values_len / (h->R * p.nkb);      // values of an average K-block
         Params whole = p;                                                    // whole tiles first, then the last tiles cut along K
         whole.partial = nullptr;
-        if (plan.tiles > plan.rest) st = launch_pairs(whole, xmap, plan.tiles - plan.rest, s);
+        if (plan.tiles > plan.rest) st = launch_pairs(whole, xmap, plan.tiles - plan.rest, block_bytes, s);
         if (st == SPDP_OK && cut) {
             p.tile0 = static_cast<int>(plan.tiles - plan.rest);
             p.kslices = plan.slices;
-            st = launch_pairs(p, xmap, plan.rest * plan.slices, s);
+            st = launch_pairs(p, xmap, plan.rest * plan.slices, block_bytes, s);
             if (st == SPDP_OK) {
                 const int64_t threads = plan.rest * p.ptok * (kTileM / 4);
                 pair::reduce_slices_kernel<<<static_cast<unsigned>(std::min<int64_t>((threads + 255) / 256, int64_t(8) * h->sm_count)), 256, 0, s>>>(
