@@ -1,15 +1,19 @@
-"""Builds libspdp.so (the C-ABI CUDA library) in-tree for sm_100a with nvcc."""
+"""Builds libspdp.so (the C-ABI CUDA library) in-tree for sm_100a with nvcc, and the small C module through which
+Python makes the per-token calls."""
 from __future__ import annotations
 
 import glob
 import os
 import subprocess
 import sys
+import sysconfig
 
 HERE = os.path.dirname(os.path.abspath(__file__))
 ROOT = os.path.dirname(HERE)
 LIB = os.path.join(HERE, "libspdp.so")
 LIB_CHECKED = os.path.join(HERE, "libspdp_checked.so")      # same sources with -DSPDP_CHECKED
+PYCALL = os.path.join(HERE, "_pycall.so")
+PYCALL_SOURCE = os.path.join(HERE, "csrc", "pycall.c")
 SOURCES = sorted(glob.glob(os.path.join(HERE, "csrc", "*.cu")))
 HEADERS = sorted(glob.glob(os.path.join(HERE, "csrc", "*.h")) + glob.glob(os.path.join(HERE, "csrc", "*.cuh"))
                  + glob.glob(os.path.join(ROOT, "include", "*.h")))
@@ -44,7 +48,18 @@ def _compile(lib: str, extra, verbose: bool) -> str:
     return lib
 
 
+def build_pycall(force: bool = False) -> str:
+    """The C module behind the per-token calls of spdp.py (csrc/pycall.c)."""
+    if not force and os.path.exists(PYCALL) and os.path.getmtime(PYCALL) >= os.path.getmtime(PYCALL_SOURCE):
+        return PYCALL
+    tmp = PYCALL + f".tmp{os.getpid()}"
+    subprocess.run(["gcc", "-O2", "-Wall", "-shared", "-fPIC", "-I", sysconfig.get_paths()["include"], "-o", tmp, PYCALL_SOURCE], check=True)
+    os.replace(tmp, PYCALL)
+    return PYCALL
+
+
 def build(force: bool = False, verbose: bool = False) -> str:
+    build_pycall(force)
     if not force and up_to_date():
         return LIB
     return _compile(LIB, [], verbose)

@@ -7,6 +7,7 @@ first call raises.
 from __future__ import annotations
 
 import ctypes
+import functools
 import os
 
 import numpy as np
@@ -87,6 +88,14 @@ def lib():
         L.spdp_last_cuda_error.argtypes = []
         L.spdp_status_string.restype = ctypes.c_char_p
         L.spdp_status_string.argtypes = [ci]
+        try:
+            from . import _pycall
+        except ImportError as e:
+            raise RuntimeError("the _pycall module is missing: build it with `python -m paper_2607_21985_b200.build`") from e
+        # the per-token calls: same entry points, arguments converted in C (csrc/pycall.c)
+        for name in ("spmspv", "spmspv_batch", "spmm", "swiglu_dp"):
+            address = ctypes.cast(getattr(L, "spdp_" + name), ctypes.c_void_p).value
+            setattr(L, "call_" + name, functools.partial(getattr(_pycall, name), address))
         _lib = L
     return _lib
 
@@ -203,7 +212,7 @@ def spdp_spmspv(h: int, x, rule: int, thr: float, y, mask=None, stream=None) -> 
     ydt = SPDP_Y_F32 if y.dtype == torch.float32 else SPDP_Y_F16
     if y.dtype not in (torch.float16, torch.float32) or x.dtype != torch.float16:
         raise ValueError("x must be fp16 and y fp16 or fp32")
-    st = lib().spdp_spmspv(h, _dev_ptr(x, "x"), rule, float(thr), _dev_ptr(mask, "mask", True), _dev_ptr(y, "y"),
+    st = lib().call_spmspv(h, _dev_ptr(x, "x"), rule, float(thr), _dev_ptr(mask, "mask", True), _dev_ptr(y, "y"),
                            ydt, _stream(stream))
     _check(st, "spdp_spmspv")
 
@@ -250,7 +259,7 @@ def spdp_spmspv_batch(h: int, X, rule: int, thr: float, Y, mask=None, stream=Non
     mstride = 0 if mask is None else (int(mask.stride(0)) if B > 1 else int(mask.shape[1]))
     if not X.is_cuda or not Y.is_cuda or (mask is not None and not mask.is_cuda):
         raise ValueError("X, Y and mask must be CUDA tensors")
-    st = lib().spdp_spmspv_batch(h, X.data_ptr(), ldx, B, rule, float(thr),
+    st = lib().call_spmspv_batch(h, X.data_ptr(), ldx, B, rule, float(thr),
                                  None if mask is None else mask.data_ptr(), mstride, Y.data_ptr(), ldy, ydt,
                                  _stream(stream))
     _check(st, "spdp_spmspv_batch")
@@ -269,13 +278,13 @@ def spdp_spmm(h: int, X, Y, stream=None) -> None:
     ldx = int(X.stride(0)) if N > 1 else max(int(X.shape[1]), int(X.stride(0)))
     ldy = int(Y.stride(0)) if N > 1 else max(int(Y.shape[1]), int(Y.stride(0)))
     ydt = SPDP_Y_F32 if Y.dtype == torch.float32 else SPDP_Y_F16
-    _check(lib().spdp_spmm(h, X.data_ptr(), N, ldx, Y.data_ptr(), ldy, ydt, _stream(stream)), "spdp_spmm")
+    _check(lib().call_spmm(h, X.data_ptr(), N, ldx, Y.data_ptr(), ldy, ydt, _stream(stream)), "spdp_spmm")
 
 
 def spdp_swiglu_dp(gate, up, thr: float, x_out, mask_out, count_out=None, stream=None) -> None:
     """x_out = silu(gate) * up (fp16 CUDA [K]) and the K-bit keep-mask of its columns in one pass."""
     K = int(gate.shape[0])
-    st = lib().spdp_swiglu_dp(_dev_ptr(gate, "gate"), _dev_ptr(up, "up"), K, float(thr), _dev_ptr(x_out, "x_out"),
+    st = lib().call_swiglu_dp(_dev_ptr(gate, "gate"), _dev_ptr(up, "up"), K, float(thr), _dev_ptr(x_out, "x_out"),
                               _dev_ptr(mask_out, "mask_out"), _dev_ptr(count_out, "count_out", True), _stream(stream))
     _check(st, "spdp_swiglu_dp")
 
