@@ -329,11 +329,12 @@ spmspv_batch_kernel(const Params p) {
                     const int rem = static_cast<int>(rc.y & 63u) - lane7;
                     const unsigned char* src = offset_wide<2>(val_src, rc.x);
                     const uint32_t dst = ring_w + stage * kStageBytes + tile * kSlotBytes + 16 * lane7;
+                    // the bitmap first: the scan waits for it alone (28672x8192 x 8 tokens 108 -> 106.6 us)
+                    cp_async4(bdst, offset_wide<32>(bm_src, rc.y >> 6));
                     cp_async16<0>(dst, src, rem);
                     cp_async16<128>(dst, src, rem);
                     cp_async16<256>(dst, src, rem);
                     cp_async16<384>(dst, src, rem);
-                    cp_async4(bdst, offset_wide<32>(bm_src, rc.y >> 6));
                 } else {
                     sts_u32(bdst, 0u);
                 }
