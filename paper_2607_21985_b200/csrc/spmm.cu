@@ -230,14 +230,14 @@ __device__ __forceinline__ void scan4(const Params& p, const uint32_t (*bm)[8], 
 }
 
 // Expands kSteps x 128 rows into the operand tile: step q is row half q % kHalves of column q / kHalves.  A lane takes
-// nibble lane % 8 (bits sh .. sh + 3, `below` = the bits under them) of word lane / 8 of the half; tab_l points at that
+// nibble lane % 8 (see nibble_top, nibble_below) of word lane / 8 of the half; tab_l points at that
 // word's table entry of column 0 (half 0), a_dst at the lane's place in the operand tile, half_bytes further is the next
 // half's tile, 16 bytes further the next column (at most 8: one k-group).  The loads of 4 steps are issued together; they
 // may reach 12 bytes past the stored values.  What bounds it is shared memory: 2 wavefronts for the table, one or two for
 // each value load, 2 for the store.  (Selectors from a 16-entry table in shared memory instead of the two multiplications
 // cost 2 more wavefronts per step and 3 % on the whole kernel.)
 template <int kSteps, int kHalves>
-__device__ __forceinline__ void expand4(uint32_t tab_l, uint32_t a_dst, uint32_t half_bytes, unsigned below, unsigned sh) {
+__device__ __forceinline__ void expand4(uint32_t tab_l, uint32_t a_dst, uint32_t half_bytes, unsigned below, unsigned top) {
     static_assert(kSteps % 4 == 0 && kSteps / kHalves <= 8, "4 steps at a time, one k-group");
 #pragma unroll
     for (int q0 = 0; q0 < kSteps; q0 += 4) {
@@ -245,8 +245,8 @@ __device__ __forceinline__ void expand4(uint32_t tab_l, uint32_t a_dst, uint32_t
 #pragma unroll
         for (int q = 0; q < 4; ++q) {
             const uint2 v = lds_v2(tab_l + 64u * ((q0 + q) / kHalves) + 32u * ((q0 + q) % kHalves));
-            a[q] = v.y + 2u * __popc(v.x & below);              // address of my nibble's first value (a multiple of 2)
-            bits[q] = (((v.x >> sh) & 15u) * 0x00204081u) & 0x01010101u;        // bit i of the nibble -> byte i
+            a[q] = v.y + 2u * __popc(v.x * below);              // address of my nibble's first value (a multiple of 2)
+            bits[q] = (((v.x * top) >> 28) * 0x00204081u) & 0x01010101u;        // bit i of the nibble -> byte i
         }
 #pragma unroll
         for (int q = 0; q < 4; ++q) {
@@ -262,7 +262,7 @@ __device__ __forceinline__ void expand4(uint32_t tab_l, uint32_t a_dst, uint32_t
             // byte i: 0x22 * (set bits before row i) + 0x10 = the two byte selectors of row i's value
             const unsigned sel = bits[q] * 0x22222200u + 0x10101010u;
             const unsigned m = bits[q] * 0xFFu;
-            sts_v2(a_dst + ((q0 + q) % kHalves) * half_bytes + ((q0 + q) / kHalves) * 16u, permute(t0, t1, sel) & permute(m, m, 0x1100u),
+            sts_v2(a_dst + ((q0 + q) % kHalves) * half_bytes + ((q0 + q) / kHalves) * 16u, permute(t0, 0u, bits[q] * 0x21CCu + 0x4444u),
                    permute(t0, t1, sel >> 16) & permute(m, m, 0x3322u));
         }
     }
@@ -583,7 +583,7 @@ spmm_kernel(const __grid_constant__ Params p, const __grid_constant__ CUtensorMa
     } else {
         // ================= decode warps =================
         const unsigned group = static_cast<unsigned>(warp) / kGroupWarps, wm = static_cast<unsigned>(warp) % kGroupWarps;
-        const unsigned sh = pinned(4u * (lane & 7)), below = pinned((1u << sh) - 1u);
+        const unsigned top = pinned(nibble_top(lane & 7)), below = pinned(nibble_below(lane & 7));
         const uint32_t tab_l = pinned(smem_u32(&sm.tab[warp][0]) + 8u * (lane >> 3));
         const uint32_t a_lane = pinned(smem_u32(&sm.A[0][0]) + (lane >> 1) * kAChunkStride + (lane & 1) * 8 +
                                        (wm >> 1) * kAKGroupStride + (wm & 1u) * 64u);
@@ -603,7 +603,7 @@ spmm_kernel(const __grid_constant__ Params p, const __grid_constant__ CUtensorMa
                 }
                 ok = __all_sync(0xFFFFFFFFu, ok);
                 if (!ok) break;
-                expand4<8, 2>(tab_l, a_lane + sa * F::kABytes, F::kATileBytes, below, sh);
+                expand4<8, 2>(tab_l, a_lane + sa * F::kABytes, F::kATileBytes, below, top);
                 // the operand tile was written through the generic proxy; the tensor cores read through the async proxy
                 asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
                 __syncwarp();
@@ -836,7 +836,7 @@ spmm_kernel(const __grid_constant__ Params p, const __grid_constant__ CUtensorMa
     } else {
         // ================= decode warps: my 128 rows of 4 columns of every sub-block of the group =================
         const unsigned group = static_cast<unsigned>(warp) / kGroupWarps, wm = static_cast<unsigned>(warp) % kGroupWarps;
-        const unsigned sh = pinned(4u * (lane & 7)), below = pinned((1u << sh) - 1u);
+        const unsigned top = pinned(nibble_top(lane & 7)), below = pinned(nibble_below(lane & 7));
         const uint32_t tab_l = pinned(smem_u32(&sm.tab[warp][0]) + 32u * c + 8u * (lane >> 3));
         const uint32_t a_lane = pinned(smem_u32(&sm.A[0][0]) + (lane >> 1) * kAChunkStride + (lane & 1) * 8);
         for (unsigned i = group; i < static_cast<unsigned>(nkb) * kSubs; i += kGroups) {
@@ -848,7 +848,7 @@ spmm_kernel(const __grid_constant__ Params p, const __grid_constant__ CUtensorMa
             scan4(p, mt.bm, mt.ci, mt.start, mt.ngt, mt.limit, static_cast<int>(j0), lane, &sm.tab[warp][0]);
             __syncwarp();
             if (kb >= kStages && ok) ok = wait_parity(&sm.mma_done[s], ((kb / kStages) & 1u) ^ 1u);  // the tensor cores are done with this A stage
-            expand4<4, 1>(tab_l, a_lane + s * kATileBytes + (j0 >> 3) * kAKGroupStride + (j0 & 7u) * 16u, 0u, below, sh);
+            expand4<4, 1>(tab_l, a_lane + s * kATileBytes + (j0 >> 3) * kAKGroupStride + (j0 & 7u) * 16u, 0u, below, top);
             // the operand tile was written through the generic proxy; the tensor cores read through the async proxy
             asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
             __syncwarp();

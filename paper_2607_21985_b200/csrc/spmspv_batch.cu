@@ -113,8 +113,8 @@ __device__ __forceinline__ unsigned lds_at(uint32_t addr) {
     asm volatile("ld.shared.u32 %0, [%1+%2];" : "=r"(v) : "r"(addr), "n"(kOff));
     return v;
 }
-// Expands 4 consecutive rows of a column tile (Sec. 4.2.1), the nibble at bit sh of the 32-bit bitmap word W: `first` is the
-// shared-memory address of the word's first value, `below` the bits under the nibble.  rank = set bits before the nibble;
+// Expands 4 consecutive rows of a column tile (Sec. 4.2.1), one nibble (nibble_top, nibble_below) of the 32-bit bitmap word W:
+// `first` is the shared-memory address of the word's first value.  rank = set bits before the nibble;
 // three aligned 32-bit loads cover its at most 4 values wherever they start, two funnel shifts align them, and byte
 // permutes put them into their rows, zero where the bit is clear.  In two parts, so that the loads of several nibbles
 // are under way together.  (One value at a time -- a popcount, a predicated 16-bit load and a select per row -- takes as
@@ -122,14 +122,14 @@ __device__ __forceinline__ unsigned lds_at(uint32_t addr) {
 // memory and the integer pipe together, about two thirds of each: two warps per K-block with 32 accumulators each, 24 warps
 // per SM, gained nothing.)
 struct Nibble { unsigned a, s0, s1, s2, bits; };
-__device__ __forceinline__ Nibble fetch_nibble(unsigned W, uint32_t first, unsigned below, unsigned sh) {
+__device__ __forceinline__ Nibble fetch_nibble(unsigned W, uint32_t first, unsigned below, unsigned top) {
     Nibble n;
-    n.a = first + 2u * __popc(W & below);
+    n.a = first + 2u * __popc(W * below);
     const uint32_t al = n.a & ~3u;
     n.s0 = lds_at<0>(al);
     n.s1 = lds_at<4>(al);
     n.s2 = lds_at<8>(al);
-    n.bits = (((W >> sh) & 15u) * 0x00204081u) & 0x01010101u;           // bit i of the nibble -> byte i
+    n.bits = (((W * top) >> 28) * 0x00204081u) & 0x01010101u;           // bit i of the nibble -> byte i
     return n;
 }
 __device__ __forceinline__ void place_nibble(const Nibble& n, unsigned& r01, unsigned& r23) {
@@ -137,7 +137,7 @@ __device__ __forceinline__ void place_nibble(const Nibble& n, unsigned& r01, uns
     const unsigned t0 = __funnelshift_r(n.s0, n.s1, mis), t1 = __funnelshift_r(n.s1, n.s2, mis);
     const unsigned sel = n.bits * 0x22222200u + 0x10101010u;            // byte i: the two byte selectors of row i's value
     const unsigned m = n.bits * 0xFFu;
-    r01 = permute(t0, t1, sel) & permute(m, m, 0x1100u);
+    r01 = permute(t0, 0u, n.bits * 0x21CCu + 0x4444u);                  // rows 0, 1 need t0 alone: a clear row selects zero bytes
     r23 = permute(t0, t1, sel >> 16) & permute(m, m, 0x3322u);
 }
 // D += A (16 rows x 8 column tiles, fp16) * B (8 column tiles x 8 tokens, fp16), fp32 accumulate.
@@ -160,7 +160,7 @@ spmspv_batch_kernel(const Params p) {
     // decode role: lane (gid, tig) expands rows 4*gid .. 4*gid + 3 of every bitmap word for tiles 2*tig, 2*tig + 1; in the
     // instruction's fragments they are rows gid and gid + 8 of two 16-row blocks
     const int gid = lane >> 2, tig = lane & 3;
-    const unsigned sh = pinned(4u * gid), below = pinned((1u << sh) - 1u);
+    const unsigned top = pinned(nibble_top(gid)), below = pinned(nibble_below(gid));
     const uint32_t ring_w = smem_u32(&sm.ring[warp][0][0]);
     const uint32_t bm_w = smem_u32(&sm.tab[warp].bm[0][0]);
     constexpr uint32_t kVoFromBm = kDepth * kTabWords * 4;
@@ -376,8 +376,8 @@ spmspv_batch_kernel(const Params p) {
                     Nibble a[2], b[2];
 #pragma unroll
                     for (int e = 0; e < 2; ++e) {
-                        a[e] = fetch_nibble(WA[w + e], FA[w + e], below, sh);
-                        b[e] = fetch_nibble(WB[w + e], FB[w + e], below, sh);
+                        a[e] = fetch_nibble(WA[w + e], FA[w + e], below, top);
+                        b[e] = fetch_nibble(WB[w + e], FB[w + e], below, top);
                     }
 #pragma unroll
                     for (int e = 0; e < 2; ++e) {
