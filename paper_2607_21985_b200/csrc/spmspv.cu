@@ -115,7 +115,8 @@ __device__ __forceinline__ bool column_active(int rule, float thr, const uint32_
 // One decode step (Sec. 4.2.1): the 2 consecutive rows this lane owns inside the 32-bit bitmap
 // word W.  `first` is the shared-memory address of the word's first value, `below` masks the bits
 // of lower rows, m0 and m1 are the lane's two bits.  rank = set bits before the position; a set
-// bit takes the next value and adds value * x to its row's fp32 accumulator.  fma.rn.f32.f16
+// bit takes the next value and adds value * x to its row's fp32 accumulator.  (A multiplication in place of the mask, as in
+// the batch and 4-bit kernels, costs 1 %: here the FMA pipe has the products to do.)  fma.rn.f32.f16
 // multiplies two fp16 exactly and accumulates in fp32.  x32 holds two activations; kUpper picks one.
 #if SPDP_FMA_MODE == 0
 #define SPDP_FMA2(X)                                  \
