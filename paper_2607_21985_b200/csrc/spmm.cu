@@ -979,13 +979,16 @@ struct Plan {
     int64_t tiles, rest;
 };
 // The estimate of a call's time: (K-blocks of the busiest CTA) x (time of a K-block) + a tile's start and end + what the
-// partial sums cost.  Fitted to the four kernels' times on 7 layers from 512x512 to 28672x2048 with 16 to 1000 tokens each
-// (50 % density; within 7 % on average): the choice costs 0.8 % on average against the best of the four, 12 % at worst.
-constexpr double kCallUs = 3.1;                                         // a call's fixed part
-constexpr double kBlockUs[4] = {0.96, 0.97, 1.19, 0.75};                // a K-block (64 columns x 256 rows), us
-constexpr double kBlockTokenUs[4] = {5.7e-4, 2.6e-4, 0.0, 3.9e-4};      // and per token of the tile
-constexpr double kTileUs = 2.8, kTileTokenUs = 5.7e-3;                  // a tile's start and end, and per token
-constexpr double kReduceUs = 2.5, kReducePerMB = 0.285;                 // the second kernel; writing and reading a MB of partial sums
+// partial sums cost.  Fitted to the four kernels' times, calls in a row on a stream, on 10 layers from 512x512 to 28672x8192
+// (30 to 80 % sparse) with 16 to 1024 tokens each: the choice costs 1 % on average against the best that was measured, 17 % at
+// worst.  (Fitted to graph replays, where the CTA pairs' plain launch costs nothing, it took pairs for small layers, and cuts that
+// cross tiles as readily as those that do not: 1024x1024 x 32 tokens 14.4 -> 8.3 us, 2048x2048 x 64 16.5 -> 12.8, 4096x4096 x
+// 128 22.9 -> 19.6, x 16 17.7 -> 14.8, 4096x11008 x 128 34.0 -> 31.4, 4001x4098 x 200 30.8 -> 26.3.)
+constexpr double kCallUs[4] = {3.0, 3.7, 3.2, 6.5};                     // a call's fixed part; the pairs' launch waits for the kernel before
+constexpr double kBlockUs[4] = {0.88, 0.97, 1.22, 0.69};                // a K-block (64 columns x 256 rows), us
+constexpr double kBlockTokenUs[4] = {8.3e-4, 1.8e-4, 0.0, 4.8e-4};      // and per token of the tile
+constexpr double kTileUs = 2.1, kTileTokenUs = 2.3e-3;                  // a tile's start and end, and per token
+constexpr double kReduceUs = 1.9, kReducePerMB = 0.223;                 // the second kernel; writing and reading a MB of partial sums
 constexpr int kTokens[4] = {One32::kNI, One128::kNI, One256::kNI, pair::kNT};
 
 Plan make_plan(int64_t R, int64_t nkb, int64_t N, int sms) {
@@ -1002,7 +1005,7 @@ Plan make_plan(int64_t R, int64_t nkb, int64_t N, int sms) {
         const int64_t rounds = q.tiles / slots, left = q.tiles - rounds * slots;
         const double tok = static_cast<double>(std::min<int64_t>(N, kTokens[f])), mb = tok * kTileM * 4.0e-6;   // MB of a tile's sums
         const double block = kBlockUs[f] + kBlockTokenUs[f] * tok, tile = kTileUs + kTileTokenUs * tok;
-        const double whole = kCallUs + (block * static_cast<double>(nkb) + tile) * static_cast<double>(rounds);
+        const double whole = kCallUs[f] + (block * static_cast<double>(nkb) + tile) * static_cast<double>(rounds);
         q.rounds = static_cast<int>(rounds);
         q.slices = 1;
         q.sharers = left > 0 ? static_cast<int>(left) : 1;
@@ -1011,19 +1014,23 @@ Plan make_plan(int64_t R, int64_t nkb, int64_t N, int sms) {
         q.us = whole + (left > 0 ? block * static_cast<double>(nkb) + tile : 0.0);
         if (best.us < 0.0 || q.us < best.us) best = q;
         if (left == 0) continue;
-        for (int64_t share = 2 * left; share < 2 * slots; share *= 2) {          // more CTAs (pairs) than tiles
-            int64_t w = std::min(share, slots);
+        const auto consider = [&](int64_t w) {                                   // w CTAs (pairs) share the tiles that are left
             if (f == 3) {
                 q.slices = static_cast<int>(std::min<int64_t>(w / left, nkb));
                 w = q.slices * left;
                 q.rest = left;
             }
-            if (w <= left || w > left * nkb) break;
+            if (w <= left || w > left * nkb) return;
             q.sharers = static_cast<int>(w);
             q.workers = static_cast<int>(rounds > 0 ? slots : w);
-            q.us = whole + block * static_cast<double>((left * nkb + w - 1) / w) + tile + kReduceUs + kReducePerMB * mb * static_cast<double>(w + left);
+            // a CTA whose range crosses into the next tile starts and ends two
+            q.us = whole + block * static_cast<double>((left * nkb + w - 1) / w) + tile * (w % left ? 2.0 : 1.0) + kReduceUs +
+                   kReducePerMB * mb * static_cast<double>(w + left);
             if (q.us < best.us) best = q;
-        }
+        };
+        for (int64_t share = 2 * left; share < slots; share *= 2) consider(share);
+        consider(slots / left * left);                                           // the most that do not cross tiles
+        if (f != 3) consider(slots);
     }
     return best;
 }
