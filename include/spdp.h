@@ -192,8 +192,9 @@ SPDP_API spdp_status spdp_spmm(spdp_handle h, const void* X_dev, int64_t N, int6
 
 /* Same product with HOST vectors (Sec. 4.2): brings x_host (fp16 [K], ideally pinned) to a
  * staging buffer of the handle, runs spdp_spmspv, leaves y in y_host ([M] of ydt) and
- * synchronises `stream`.  mask_host is uint32[ceil(K/32)] or NULL.  Pinned buffers are read and written by
- * the kernels themselves; pageable ones are copied before and after the kernel. */
+ * synchronises `stream`.  mask_host is uint32[ceil(K/32)] or NULL.  The buffers may start at any byte.  Where
+ * all of them lie in page-locked memory (each in one allocation or registration) and on a multiple of their element's size,
+ * the kernels read and write them directly; else they are copied before and after the kernel. */
 SPDP_API spdp_status spdp_spmspv_host(spdp_handle h, const void* x_host, spdp_dp_rule rule, float thr,
                              const void* mask_host, void* y_host, spdp_ydtype ydt, void* stream);
 

@@ -1,6 +1,8 @@
 // C ABI of libspdp (declared in spdp.h): argument checks, handle life cycle, host-side layout
 // of the split-K work partition.  Every numerical step runs in the kernels of pack.cu and
 // spmspv.cu.
+#include <cuda.h>
+
 #include <cstdio>
 #include <cstring>
 #include <mutex>
@@ -267,14 +269,34 @@ spdp_status enqueue_host_call(spdp_matrix* h, const void* x_host, int rule, floa
     return SPDP_OK;
 }
 
-// The device address of pinned host memory, or null.
-void* pinned_address(const void* p) {
-    cudaPointerAttributes a;
-    if (cudaPointerGetAttributes(&a, p) != cudaSuccess) {
-        cudaGetLastError();
-        return nullptr;
-    }
-    return a.type == cudaMemoryTypeHost ? a.devicePointer : nullptr;
+// The page-locked range that holds a host address, asked of the driver in one call (looked up through the runtime: the library
+// does not link libcuda).
+using PointerAttributesFn = CUresult (*)(unsigned, CUpointer_attribute*, void**, CUdeviceptr);
+PointerAttributesFn pointer_attributes_fn() {
+    static PointerAttributesFn fn = [] {
+        void* f = nullptr;
+        cudaDriverEntryPointQueryResult q;
+        if (cudaGetDriverEntryPoint("cuPointerGetAttributes", &f, cudaEnableDefault, &q) != cudaSuccess || q != cudaDriverEntryPointSuccess) f = nullptr;
+        return reinterpret_cast<PointerAttributesFn>(f);
+    }();
+    return fn;
+}
+hostdev::PinnedRange pinned_range(const void* p) {
+    const PointerAttributesFn get = pointer_attributes_fn();
+    unsigned type = 0, managed = 0;
+    CUdeviceptr device = 0, start = 0;
+    size_t size = 0;
+    CUpointer_attribute what[] = {CU_POINTER_ATTRIBUTE_MEMORY_TYPE, CU_POINTER_ATTRIBUTE_IS_MANAGED, CU_POINTER_ATTRIBUTE_DEVICE_POINTER,
+                                  CU_POINTER_ATTRIBUTE_RANGE_START_ADDR, CU_POINTER_ATTRIBUTE_RANGE_SIZE};
+    void* out[] = {&type, &managed, &device, &start, &size};
+    // pageable memory is no error here: every attribute comes back zero
+    if (get == nullptr || get(5, what, out, reinterpret_cast<CUdeviceptr>(p)) != CUDA_SUCCESS || type != CU_MEMORYTYPE_HOST || managed != 0 || device == 0)
+        return {0, 0, 0};
+    return {static_cast<uint64_t>(start), static_cast<uint64_t>(size), static_cast<uint64_t>(device)};
+}
+// The address through which the kernels may use a host buffer, or null (see hostdev::direct_address).
+void* direct_address(const void* p, size_t bytes, size_t align) {
+    return reinterpret_cast<void*>(static_cast<uintptr_t>(hostdev::direct_address(reinterpret_cast<uintptr_t>(p), bytes, align, pinned_range(p))));
 }
 
 // The host-vector call with pinned buffers, whose device addresses the kernels use: a small kernel fetches x (and the mask) once, the
@@ -542,14 +564,16 @@ spdp_status spdp_spmspv_host(spdp_handle h, const void* x_host, spdp_dp_rule rul
     if (cudaGetDevice(&dev) != cudaSuccess || dev != h->device) return SPDP_ERR_INVALID_ARG;   // wrong current device
     cudaStream_t s = static_cast<cudaStream_t>(stream);
     // What is pinned is looked up on every call, and every call's arguments go into the recorded graph: nothing is assumed
-    // about a buffer because an earlier one had its address.
+    // about a buffer because an earlier one had its address.  A buffer that a kernel may not touch takes the copies.
     spdp_matrix::HostCall c = {};
     c.rule = rule;
     c.thr = thr;
     c.ydt = ydt;
-    c.x = static_cast<const __half*>(pinned_address(x_host));
-    c.y = c.x != nullptr ? pinned_address(y_host) : nullptr;
-    if (rule == SPDP_DP_MASK && c.y != nullptr) c.mask = static_cast<const uint32_t*>(pinned_address(mask_host));
+    const size_t ysize = ydt == SPDP_Y_F32 ? sizeof(float) : sizeof(__half);
+    c.x = static_cast<const __half*>(direct_address(x_host, h->K * sizeof(__half), sizeof(__half)));
+    c.y = c.x != nullptr ? direct_address(y_host, h->M * ysize, ysize) : nullptr;
+    if (rule == SPDP_DP_MASK && c.y != nullptr)
+        c.mask = static_cast<const uint32_t*>(direct_address(mask_host, mask_words(h, rule) * sizeof(uint32_t), sizeof(uint32_t)));
     spdp_status st;
     if (c.y == nullptr || (rule == SPDP_DP_MASK && c.mask == nullptr)) {
         st = enqueue_host_call(h, x_host, rule, thr, mask_host, y_host, ydt, s);

@@ -48,6 +48,18 @@ inline int default_ctas(int64_t R, int64_t C, int most) {
     return best < 1 ? 1 : best;
 }
 
+// Host memory as the driver describes it: the page-locked range that holds an address (size 0: none, the memory is pageable
+// or the device's) and the device address of that address.
+struct PinnedRange { uint64_t start, size, device; };
+
+// The address through which a kernel may read or write the `bytes` bytes at host address p, whose elements are `align` bytes:
+// the device address if one page-locked range holds all of them and it is a multiple of `align`; else 0, and the bytes have to
+// be copied.  (A copy takes any address.  A kernel's access to a misaligned element or beyond the range is a device fault.)
+inline uint64_t direct_address(uint64_t p, uint64_t bytes, uint64_t align, const PinnedRange& r) {
+    if (r.size == 0 || p < r.start || p - r.start > r.size || bytes > r.size - (p - r.start)) return 0;
+    return r.device % align == 0 ? r.device : 0;
+}
+
 // Checked build: is [first, first + count) inside [0, limit)?  A violation is encoded as
 // kCheckBase - site (site = a small number naming the access in the source) for the status word;
 // the caller then skips the access.  Nothing traps and nothing asserts.

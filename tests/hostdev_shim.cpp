@@ -11,3 +11,7 @@ int shim_span_ok(unsigned long long first, unsigned long long count, unsigned lo
 int shim_check_code(int site) { return spdp::hostdev::check_code(site); }
 }
 extern "C" int shim_default_ctas(long long r, long long c, int most) { return spdp::hostdev::default_ctas(r, c, most); }
+extern "C" unsigned long long shim_direct_address(unsigned long long p, unsigned long long bytes, unsigned long long align,
+                                                  unsigned long long start, unsigned long long size, unsigned long long device) {
+    return spdp::hostdev::direct_address(p, bytes, align, {start, size, device});
+}

@@ -607,3 +607,35 @@ def test_host_vectors_buffers(S, K, pin_x, pin_y, shift):
                         assert torch.equal(yh, want.cpu()), (rule, dt, k, call)
     finally:
         S.spdp_free(h)
+
+
+@pytest.mark.parametrize("x_at,gap_y,gap_mask", [(0, 0, 0), (1, 0, 0), (0, 1, 0), (0, 2, 0), (0, 0, 1), (0, 0, 2)])
+@pytest.mark.parametrize("dtype", [np.float16, np.float32])
+def test_host_vectors_at_any_byte_of_a_pinned_arena(S, x_at, gap_y, gap_mask, dtype):
+    """x, y and the mask words one behind the other in one pinned arena, at bytes that are no multiple of their elements'
+    size: such buffers are copied (the kernels must not touch them) and give what the device-vector call gives."""
+    M, K = 600, 1001
+    rng = np.random.Generator(np.random.PCG64(17))
+    W = rng.standard_normal((M, K)).astype(np.float16)
+    W[rng.random((M, K)) < 0.5] = 0
+    x = rng.standard_normal(K).astype(np.float16)
+    words = O.active_to_words(rng.random(K) < 0.5)
+    arena = torch.zeros(16384, dtype=torch.uint8).pin_memory().numpy()
+    y_at = x_at + 2 * K + gap_y
+    mask_at = y_at + M * dtype().itemsize + gap_mask
+    xh = np.frombuffer(arena, np.float16, K, x_at)
+    yh = np.frombuffer(arena, dtype, M, y_at)
+    mh = np.frombuffer(arena, np.uint32, words.size, mask_at)
+    xh[:], mh[:] = x, words
+    h = S.spdp_pack_tiled_cbc(dev(W))
+    try:
+        for rule, mask in ((O.DP_ABS_GT, None), (O.DP_MASK, mh)):
+            want = torch.empty(M, dtype=torch.float16 if dtype == np.float16 else torch.float32, device="cuda")
+            S.spdp_spmspv(h, dev(x), rule, 0.5, want, mask=None if mask is None else dev(words))
+            for call in range(3):
+                yh[:] = np.nan
+                S.spdp_spmspv_host(h, xh, rule, 0.5, yh, mask_host=mask)
+                assert np.array_equal(yh, want.cpu().numpy()), (rule, call)
+                assert np.array_equal(xh, x) and np.array_equal(mh, words)
+    finally:
+        S.spdp_free(h)

@@ -59,3 +59,17 @@ def test_default_ctas_in_range(H, R, C, most):
     assert 1 <= p <= min(most, R * C)
     if R * C >= 300 * most:
         assert p > 0.9 * most                          # a large layer uses (nearly) every SM
+
+
+def test_kernels_touch_only_whole_aligned_pinned_buffers(H):
+    """Which host buffers the kernels use directly: all bytes inside one page-locked range, elements on their size."""
+    f = H.shim_direct_address
+    f.argtypes, f.restype = [ctypes.c_ulonglong] * 6, ctypes.c_ulonglong
+    start, size, dev = 0x7F0000000000, 4096, 0x700000000000
+    at = lambda off, n, align: f(start + off, n, align, start, size, dev + off)
+    assert at(0, 4096, 4) == dev and at(8, 100, 4) == dev + 8 and at(2, 10, 2) == dev + 2 and at(4096, 0, 2) == dev + 4096
+    assert at(0, 4097, 2) == 0 and at(4000, 98, 2) == 0 and at(4095, 2, 1) == 0          # runs past the range
+    assert at(1, 10, 2) == 0 and at(10002, 4, 4) == 0 and at(10, 40, 4) == 0 and at(2, 4, 4) == 0     # off the element's size
+    assert f(start - 8, 4, 4, start, size, dev) == 0                                     # before it
+    assert f(start, 4, 4, 0, 0, 0) == 0                                                  # pageable
+    assert f(start + 8, (1 << 64) - 4, 4, start, size, dev + 8) == 0                     # a length that would wrap
