@@ -10,7 +10,9 @@
 namespace spdp {
 namespace {
 
-__global__ void swiglu_dp_kernel(const __half* __restrict__ gate, const __half* __restrict__ up, int64_t K, float thr,
+// gate and up are not __restrict__: the kernels that write them may still run when this one starts, and the read-only path that
+// const __restrict__ allows is for data that nothing writes in the kernel's lifetime.
+__global__ void swiglu_dp_kernel(const __half* gate, const __half* up, int64_t K, float thr,
                                  __half* __restrict__ x_out, uint32_t* __restrict__ mask_out, int* __restrict__ count) {
     // The kernel after this one (the decode call) may start its matrix-only prologue now; what the kernel before this one
     // wrote or still reads (gate, up, x_out, mask_out) is touched only after the wait.
@@ -32,7 +34,7 @@ __global__ void swiglu_dp_kernel(const __half* __restrict__ gate, const __half* 
 }
 
 // Fetches the vectors of a host-vector call over the bus: one 16-byte load per thread where the address allows it.
-__global__ void fetch_kernel(const __half* __restrict__ x, int K, __half* __restrict__ x_out, const uint32_t* __restrict__ mask, int mask_words,
+__global__ void fetch_kernel(const __half* x, int K, __half* __restrict__ x_out, const uint32_t* mask, int mask_words,
                              uint32_t* __restrict__ mask_out) {
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     asm volatile("griddepcontrol.wait;" ::: "memory");                  // the buffers may still be read by the call before

@@ -53,7 +53,8 @@ struct Params {
     const __half* values;
     const __half* x;            // [batch][ldx]
     int64_t ldx;
-    const uint32_t* mask;       // [batch][mask_stride] words, or null
+    const uint32_t* mask;       // [batch][mask_stride] words, or null.  x and mask: written by kernels that may still run when this
+                                // one starts, so read after griddepcontrol.wait and never through the read-only path (__ldg)
     int64_t mask_stride;
     void* y;                    // [batch][ldy]
     int64_t ldy;
@@ -252,7 +253,7 @@ spmspv_batch_kernel(const Params p) {
                         k1 = abs_gt_keep(xv.y, thr2);
                     } else if (p.rule == SPDP_DP_MASK) {
                         const int j = j0 + v0;                              // a multiple of 4
-                        const unsigned bits = __ldg(p.mask + b * p.mask_stride + (j >> 5)) >> (j & 31);
+                        const unsigned bits = p.mask[b * p.mask_stride + (j >> 5)] >> (j & 31);    // no __ldg, see Params
                         k0 = ((bits & 1u) ? 0x0000FFFFu : 0u) | ((bits & 2u) ? 0xFFFF0000u : 0u);
                         k1 = ((bits & 4u) ? 0x0000FFFFu : 0u) | ((bits & 8u) ? 0xFFFF0000u : 0u);
                     }

@@ -58,7 +58,8 @@ struct Params {
     const unsigned char* codes;
     const __half* scales;
     const __half* x;
-    const uint32_t* mask;
+    const uint32_t* mask;   // x and mask: written by kernels that may still run when this one starts, so read after
+                            // griddepcontrol.wait and never through the read-only path (__ldg)
     void* y;
     float thr;
     int rule;
@@ -295,7 +296,7 @@ spmspv_q4_kernel(const Params p) {
                 if (p.rule == SPDP_DP_ABS_GT) return abs_gt_keep(*reinterpret_cast<const unsigned*>(&sm.stage.x[v]), thr2);
                 if (p.rule == SPDP_DP_MASK) {
                     const int j = min((two && v >= vB0) ? v - vB0 : jA0 + v, (p.K - 1) & ~1); // even: both bits lie in one word
-                    const unsigned w = __ldg(p.mask + (j >> 5)) >> (j & 31);
+                    const unsigned w = p.mask[j >> 5] >> (j & 31);                    // an ordinary load, see Params
                     return (w & 1u) | ((w & 2u) << 30);
                 }
                 return 0xFFFFFFFFu;

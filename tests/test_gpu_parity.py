@@ -639,3 +639,46 @@ def test_host_vectors_at_any_byte_of_a_pinned_arena(S, x_at, gap_y, gap_mask, dt
                 assert np.array_equal(xh, x) and np.array_equal(mh, words)
     finally:
         S.spdp_free(h)
+
+
+@pytest.mark.parametrize("down", ["fp16", "q4", "batch"])
+def test_projections_and_producer_overlap_on_one_stream(S, down):
+    """A gated MLP as a decode loop runs it: gate and up projection, the producer, the down projection with its mask, token
+    after token in the same buffers without a synchronisation, so that every kernel starts beside the one whose results it
+    reads.  Bit for bit what the same calls give when each waits for the one before."""
+    rng = np.random.Generator(np.random.PCG64(29))
+    D, F, steps, tokens = 1000, 2808, 60, 3 if down == "batch" else 1
+    sparse = lambda m, k: (rng.standard_normal((m, k)) * (rng.random((m, k)) < 0.5) * 0.1).astype(np.float16)
+    hg, hu = S.spdp_pack_tiled_cbc(dev(sparse(F, D))), S.spdp_pack_tiled_cbc(dev(sparse(F, D)))
+    Wd = dev(sparse(D, F))
+    hd = S.spdp_pack_tiled_cbc_q4(Wd) if down == "q4" else S.spdp_pack_tiled_cbc(Wd)
+    X = dev(rng.standard_normal((steps, tokens, D)).astype(np.float16))
+    gate, up = (torch.empty(F, dtype=torch.float16, device="cuda") for _ in range(2))
+    h = torch.empty((tokens, F), dtype=torch.float16, device="cuda")
+    mask = torch.empty((tokens, (F + 31) // 32), dtype=torch.int32, device="cuda")
+
+    def run(wait):
+        Y = torch.full((steps, tokens, D), float("nan"), dtype=torch.float32, device="cuda")
+        for s in range(steps):
+            for b in range(tokens):
+                S.spdp_spmspv(hg, X[s, b], O.DP_ABS_GT, 0.7, gate)
+                wait()
+                S.spdp_spmspv(hu, X[s, b], O.DP_ABS_GT, 0.7, up)
+                wait()
+                S.spdp_swiglu_dp(gate, up, 0.4, h[b], mask[b])
+                wait()
+            if down == "batch":
+                S.spdp_spmspv_batch(hd, h, O.DP_MASK, 0.0, Y[s], mask=mask)
+            else:
+                S.spdp_spmspv(hd, h[0], O.DP_MASK, 0.0, Y[s, 0], mask=mask[0])
+            wait()
+        torch.cuda.synchronize()
+        return Y.cpu().numpy()
+    try:
+        want = run(torch.cuda.synchronize)
+        assert np.isfinite(want).all() and len(np.unique(want[:, 0, 0])) == steps
+        for _ in range(5):
+            assert np.array_equal(run(lambda: None), want)
+    finally:
+        for x in (hg, hu, hd):
+            S.spdp_free(x)
