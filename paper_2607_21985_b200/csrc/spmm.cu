@@ -296,6 +296,16 @@ __device__ __forceinline__ void store_accumulators(const Params& p, uint32_t tme
     }
 }
 
+// A CTA that gave up fills its slots of the scratch memory with this word, so that the second kernel leaves the rows it feeds
+// unwritten instead of adding what an earlier call left there.  No sum can be this word: a NaN that arithmetic makes is 0x7FFFFFFF.
+// (Only the fourth rows are tested, one comparison per 16 bytes.  A word per CTA beside the slots, written by every CTA and
+// read by the second kernel, cost each cut call 0.2 to 0.6 us.)
+constexpr unsigned kNoSum = 0x7FFFDEADu;
+__device__ __forceinline__ void void_rows(const Params& p, int slot, int row0, int rows, int t, int nthreads) {
+    unsigned* part = reinterpret_cast<unsigned*>(p.partial) + static_cast<size_t>(slot) * p.ptok * kTileM;
+    for (int i = t; i < p.ptok * rows; i += nthreads) part[static_cast<size_t>(i / rows) * kTileM + row0 + i % rows] = kNoSum;
+}
+
 struct alignas(16) Meta {                       // a K-block as stored, without its values
     alignas(16) uint32_t bm[kKB][8];            // bitmaps
     alignas(16) uint32_t ci[kKB];               // ColInfo words
@@ -638,6 +648,11 @@ spmm_kernel(const __grid_constant__ Params p, const __grid_constant__ CUtensorMa
     __syncwarp();
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
+    if (*static_cast<volatile int*>(&sm.abort) != 0 && p.partial != nullptr && me < p.sharers) {
+        void_rows(p, 2 * me, 0, kTileM, t, kThreads);
+        void_rows(p, 2 * me + 1, 0, kTileM, t, kThreads);
+        __syncwarp();
+    }
     if (warp == 1)
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "n"(F::kTmemCols) : "memory");
 }
@@ -663,11 +678,13 @@ reduce_pieces_kernel(const Params p, int tile0, int tiles, int tile_tokens) {
         const int64_t row = static_cast<int64_t>(tile / p.nblocks) * kTileM + row_in;
         if (n >= p.N || row >= p.M) continue;
         float4 sum = make_float4(0.f, 0.f, 0.f, 0.f);
+        bool there = true;                                               // no CTA of the tile gave up
         const unsigned first_slot = 2u * first + (rest_begin(p, first) < t * nkb ? 1u : 0u);     // the only one that may start in the tile before
 #pragma unroll 4
         for (unsigned w = first; w <= last; ++w) {
             const unsigned slot = w == first ? first_slot : 2u * w;
             const float4 v = *reinterpret_cast<const float4*>(p.partial + (static_cast<size_t>(slot) * p.ptok + tok) * kTileM + row_in);
+            there = there && __float_as_uint(v.w) != kNoSum;
             sum.x += v.x;
             sum.y += v.y;
             sum.z += v.z;
@@ -676,7 +693,7 @@ reduce_pieces_kernel(const Params p, int tile0, int tiles, int tile_tokens) {
         const float v[4] = {sum.x, sum.y, sum.z, sum.w};
 #pragma unroll
         for (int e = 0; e < 4; ++e)
-            if (row + e < p.M) store_y(p.Y, p.ydt, n * p.ldy + row + e, v[e]);
+            if (there && row + e < p.M) store_y(p.Y, p.ydt, n * p.ldy + row + e, v[e]);
     }
 }
 
@@ -873,6 +890,8 @@ spmm_kernel(const __grid_constant__ Params p, const __grid_constant__ CUtensorMa
         const int lane_base = 32 * (warp & 3), cbase = (warp >> 2) * (kNT / 4);
         store_accumulators(p, tmem, lane_base, cbase, cbase + kNT / 4, r, c * 128 + lane_base + lane, n0,
                            p.partial == nullptr ? -1 : static_cast<int>(pr));
+    } else if (*static_cast<volatile int*>(&sm.abort) && p.partial != nullptr) {
+        void_rows(p, static_cast<int>(pr), c * 128, 128, t, kThreads);
     }
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
@@ -898,8 +917,10 @@ reduce_slices_kernel(const Params p, int tiles) {
         if (n >= p.N || row >= p.M) continue;
         const float* src = p.partial + (static_cast<size_t>(tt) * p.kslices * p.ptok + tok) * kTileM + row_in;
         float4 sum = make_float4(0.f, 0.f, 0.f, 0.f);
+        bool there = true;                                               // no CTA of the tile gave up
         for (int sl = 0; sl < p.kslices; ++sl) {
             const float4 v = *reinterpret_cast<const float4*>(src + static_cast<size_t>(sl) * p.ptok * kTileM);
+            there = there && __float_as_uint(v.w) != kNoSum;
             sum.x += v.x;
             sum.y += v.y;
             sum.z += v.z;
@@ -908,7 +929,7 @@ reduce_slices_kernel(const Params p, int tiles) {
         const float v[4] = {sum.x, sum.y, sum.z, sum.w};
 #pragma unroll
         for (int e = 0; e < 4; ++e)
-            if (row + e < p.M) store_y(p.Y, p.ydt, n * p.ldy + row + e, v[e]);
+            if (there && row + e < p.M) store_y(p.Y, p.ydt, n * p.ldy + row + e, v[e]);
     }
 }
 

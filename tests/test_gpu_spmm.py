@@ -143,3 +143,49 @@ def test_spmm_work_cuts(S, R, K, N, sp):
         assert np.array_equal(Y.cpu().numpy(), Y_ref)
     finally:
         S.spdp_free(h)
+
+
+class _DeviceWords:
+    """int32 view of device memory at an address."""
+    def __init__(self, address, n):
+        self.__cuda_array_interface__ = dict(shape=(n,), typestr="<i4", data=(address, False), version=3)
+
+
+@pytest.mark.parametrize("R,K,N", [(6, 4096, 32), (6, 8192, 40), (5, 4096, 512), (6, 8192, 512), (16, 4098, 300)])
+def test_spmm_leaves_a_refused_tile_unwritten(S, R, K, N):
+    """A TileOffset word that cannot be (the kernel's own check refuses the K-blocks at it and copies nothing): the status says
+    so, and the tile's outputs stay unwritten although other CTAs have left their partial sums of it and the scratch memory
+    still holds an earlier call's.  The shapes are cut along K, with 32, 128 and 256 tokens per CTA and with CTA pairs."""
+    rng = np.random.Generator(np.random.PCG64(R))
+    M, C = 256 * R, (K + 15) // 16
+    W = rng.integers(-4, 5, (M, K)).astype(np.float16)
+    W[rng.random((M, K)) < 0.5] = 0
+    X = torch.zeros((N, (K + 7) // 8 * 8), dtype=torch.float16, device="cuda")
+    X[:, :K] = dev(rng.integers(-2, 3, (N, K)).astype(np.float16))
+    Y_ref = X[:, :K].float().cpu().numpy() @ W.astype(np.float32).T
+    h = S.spdp_pack_tiled_cbc(dev(W))
+    try:
+        def call():
+            Y = torch.full((N, M), float("nan"), dtype=torch.float32, device="cuda")
+            S.spdp_spmm(h, X[:, :K], Y)
+            torch.cuda.synchronize()
+            return Y.cpu().numpy(), S.spdp_last_device_status(h)
+        Y, status = call()
+        assert status == 0 and np.array_equal(Y, Y_ref)
+        info = S.spdp_get_info(h)
+        words = torch.as_tensor(_DeviceWords(info.tileoffset_dev, info.NGT + 1), device="cuda")
+        at = 3 * C + 4 * (C // 8)                              # between two K-blocks in the middle of row tile 3
+        good = int(words[at])
+        words[at] = -1                                         # 2^32 - 1 values: beyond the array
+        torch.cuda.synchronize()                               # the kernels may read the matrix ahead of the stream
+        Y, status = call()
+        words[at] = good
+        torch.cuda.synchronize()
+        assert status == S.SPDP_ERR_OVERFLOW
+        assert np.isnan(Y[:, 768:1024]).all()
+        far = np.r_[0:512, 5 * 256:M]
+        assert np.array_equal(Y[:, far], Y_ref[:, far])        # a CTA may share the neighbouring tiles, not these
+        Y, status = call()
+        assert status == 0 and np.array_equal(Y, Y_ref)
+    finally:
+        S.spdp_free(h)
