@@ -150,14 +150,15 @@ __device__ __forceinline__ void barrier_init(unsigned long long* bar, uint32_t a
 __device__ __forceinline__ void arrive(unsigned long long* bar) {
     asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(bar)) : "memory");
 }
+__device__ __forceinline__ bool phase_done(unsigned long long* bar, unsigned parity) {
+    unsigned done;
+    asm volatile("{\n .reg .pred p;\n mbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n selp.u32 %0, 1, 0, p;\n}"
+                 : "=r"(done) : "r"(smem_u32(bar)), "r"(parity) : "memory");
+    return done != 0u;
+}
 __device__ __forceinline__ bool wait_parity(unsigned long long* bar, unsigned parity) {
     const uint32_t a = smem_u32(bar);
-    {   // the phase is usually complete already: a test costs less than a wait that may suspend
-        unsigned done;
-        asm volatile("{\n .reg .pred p;\n mbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n selp.u32 %0, 1, 0, p;\n}"
-                     : "=r"(done) : "r"(a), "r"(parity) : "memory");
-        if (done) return true;
-    }
+    if (phase_done(bar, parity)) return true;       // usually: a test costs less than a wait that may suspend
     for (int tries = 0; tries < kWaitTries; ++tries) {
         unsigned done;
         asm volatile("{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n selp.u32 %0, 1, 0, p;\n}"
@@ -411,6 +412,7 @@ struct Form {
     static constexpr int kBStages = kNI <= 128 ? 3 : 2;
     static constexpr int kMeta = 8;                                   // stored K-blocks in flight, at most
     static_assert(kBBytes % 1024 == 0, "every X tile on a swizzle-atom boundary");
+    static_assert(kAStages == 2 * kSubs && kAStages >= kGroups, "the first A stages are the first two K-blocks, and every decode warp has a sub-block among the next kAStages");
 };
 
 // CTA w's share of the tiles that are cut along K: K-blocks [rest_begin(w), rest_begin(w + 1)).
@@ -600,27 +602,36 @@ spmm_kernel(const __grid_constant__ Params p, const __grid_constant__ CUtensorMa
         unsigned i0 = 0;                                                // sub-blocks before this piece
         for (int k = 0; ok && piece(p, me, k, s); ++k) {
             const unsigned i1 = i0 + static_cast<unsigned>(s.n) * kSubs;
-            for (unsigned i = i0 + (group + kGroups - i0 % kGroups) % kGroups; i < i1; i += kGroups) {
-                const unsigned u = i / kSubs, m = u % F::kMeta, sa = i % F::kAStages;
-                ok = wait_parity(&sm.comp_full[m], (u / F::kMeta) & 1);                          // the stored K-block has arrived
-                __syncwarp();
-                const Meta& mt = sm.meta[m];
-                scan4(p, mt.bm, mt.ci, mt.start, mt.ngt, mt.limit, static_cast<int>((i % kSubs) * kSub + 4u * wm), lane, &sm.tab[warp][0]);
-                __syncwarp();
-                if (i >= F::kAStages) {
-                    if (i < 2 * F::kAStages) asm volatile("griddepcontrol.wait;" ::: "memory");  // the products wait for X
-                    ok = wait_parity(&sm.a_free[sa], (i / F::kAStages - 1u) & 1) && ok;          // the tensor cores are done with this A stage
+            unsigned i = i0 + (group + kGroups - i0 % kGroups) % kGroups;
+            for (unsigned upto = min(i1, static_cast<unsigned>(F::kAStages));; upto = i1) {
+                for (; i < upto; i += kGroups) {
+                    const unsigned u = i / kSubs, m = u % F::kMeta, sa = i % F::kAStages;
+                    ok = wait_parity(&sm.comp_full[m], (u / F::kMeta) & 1);                          // the stored K-block has arrived
+                    __syncwarp();
+                    const Meta& mt = sm.meta[m];
+                    scan4(p, mt.bm, mt.ci, mt.start, mt.ngt, mt.limit, static_cast<int>((i % kSubs) * kSub + 4u * wm), lane, &sm.tab[warp][0]);
+                    __syncwarp();
+                    if (i >= F::kAStages) {
+                        if (i < 2 * F::kAStages) asm volatile("griddepcontrol.wait;" ::: "memory");  // the products wait for X
+                        ok = wait_parity(&sm.a_free[sa], (i / F::kAStages - 1u) & 1) && ok;          // the tensor cores are done with this A stage
+                    }
+                    ok = __all_sync(0xFFFFFFFFu, ok);
+                    if (!ok) break;
+                    expand4<8, 2>(tab_l, a_lane + sa * F::kABytes, F::kATileBytes, below, top);
+                    // the operand tile was written through the generic proxy; the tensor cores read through the async proxy
+                    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+                    __syncwarp();
+                    if (lane == 0) {
+                        arrive(&sm.a_ready[sa]);
+                        arrive(&sm.comp_free[m]);
+                    }
                 }
-                ok = __all_sync(0xFFFFFFFFu, ok);
-                if (!ok) break;
-                expand4<8, 2>(tab_l, a_lane + sa * F::kABytes, F::kATileBytes, below, top);
-                // the operand tile was written through the generic proxy; the tensor cores read through the async proxy
-                asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-                __syncwarp();
-                if (lane == 0) {
-                    arrive(&sm.a_ready[sa]);
-                    arrive(&sm.comp_free[m]);
-                }
+                if (!ok || upto == i1) break;
+                // Behind the first A stages (the first two K-blocks, which find room in any case) a K-block may still be outside
+                // because the ring is full: then its copy waits for decodes, these for products, and they for X.  (Once, between
+                // two loops: a test in the loop costs 0.4 %, the wait without a test 1 % of a small call.)
+                if (i < i1 && !phase_done(&sm.comp_full[i / kSubs % F::kMeta], (i / kSubs / F::kMeta) & 1))
+                    asm volatile("griddepcontrol.wait;" ::: "memory");
             }
             i0 = i1;
             if (warp >= kStoreWarps) continue;

@@ -189,3 +189,33 @@ def test_spmm_leaves_a_refused_tile_unwritten(S, R, K, N):
         assert status == 0 and np.array_equal(Y, Y_ref)
     finally:
         S.spdp_free(h)
+
+
+@pytest.mark.parametrize("R,K,N", [(20, 4096, 200), (20, 4096, 30), (37, 1024, 128), (6, 8192, 512)])
+@pytest.mark.parametrize("sp", [0.0, 0.9])
+def test_spmm_calls_in_a_row(S, R, K, N, sp):
+    """Calls in a row start beside one another; in the second and third pass a copy just before the call makes its input.
+    Full columns: the ring of stored values holds two K-blocks, so the copies stop before the call ahead has ended."""
+    rng = np.random.Generator(np.random.PCG64(R))
+    M = 256 * R
+    W = rng.integers(1, 5, (M, K)).astype(np.float16)
+    W[rng.random((M, K)) < sp] = 0
+    h = S.spdp_pack_tiled_cbc(dev(W))
+    try:
+        X = [dev(rng.integers(-2, 3, (N, K)).astype(np.float16)) for _ in range(4)]
+        buf = torch.empty((N, K), dtype=torch.float16, device="cuda")
+        Wd = dev(W).double()
+        want = [x.double() @ Wd.T for x in X]
+        Y = torch.empty((4, N, M), dtype=torch.float32, device="cuda")
+        for repeat in range(3):
+            Y.fill_(float("nan"))
+            for x, y in zip(X, Y):
+                if repeat:
+                    buf.copy_(x)
+                S.spdp_spmm(h, buf if repeat else x, y)
+            torch.cuda.synchronize()
+            for y, ref in zip(Y, want):
+                assert torch.equal(y.double(), ref)            # integers: every sum is exact
+        assert S.spdp_last_device_status(h) == 0
+    finally:
+        S.spdp_free(h)
