@@ -70,6 +70,8 @@ typedef struct {
     int64_t values_len;        /* = TileOffset[NGT], padding included                           */
     int64_t packed_bytes;      /* bytes of TileOffset + ColInfo + Bitmap + Values               */
     int64_t workspace_bytes;   /* split-K scratch owned by the handle                           */
+    /* The arrays lie in cudaMalloc allocations: one starts at values_dev, one at bitmap_dev, which holds the other two behind it.
+     * They may be read by a peer or exported to another process, until the handle is freed. */
     const void* tileoffset_dev;  /* uint32[NGT+1]  start of each GTile in Values (elements)      */
     const void* colinfo_dev;     /* uint32[NGT*16] (column start inside its GTile) << 16 | nnz   */
     const void* bitmap_dev;      /* uint64[NGT*16*4] bit b of word w = row 64*w+b of the column tile */
@@ -247,8 +249,10 @@ SPDP_API spdp_status spdp_swiglu_dp(const void* gate_dev, const void* up_dev, in
  * are fewer row tiles than ranks).  Host arithmetic only. */
 SPDP_API spdp_status spdp_row_shard(int64_t M, int world, int rank, int64_t* first_row_out, int64_t* rows_out);
 
-/* Release the handle and everything it owns (waits for the work on its device).  Up to 512 MB of device memory that freed
- * handles leave is kept for the next ones; spdp_free(NULL), which is SPDP_OK, gives that back to the driver. */
+/* Release the handle and everything it owns (waits for the work on its device).  Up to 512 MB per device of what freed handles
+ * leave is kept for the next ones.  spdp_free(NULL), which is SPDP_OK, gives that back to the driver, and the unused scratch
+ * memory of spdp_spmm (up to 96 MB, else kept until the device's last handle goes): call it when another allocator needs
+ * the memory. */
 SPDP_API spdp_status spdp_free(spdp_handle h);
 
 /* ---- inspection surface (the format and the active set are checked bit for bit) ---- */

@@ -3,6 +3,7 @@
 // spmspv.cu.
 #include <cuda.h>
 
+#include <algorithm>
 #include <cstdio>
 #include <cstring>
 #include <mutex>
@@ -23,29 +24,81 @@ void note_cuda_error(cudaError_t e, const char* what) {
 
 namespace {
 
-// Device memory comes from two stream-ordered pools per device, apart from the device's default pool (which gives its
-// memory back to the driver at every synchronisation: 0.45 ms per prefill call that needs scratch, and about 3 ms of
-// cudaMalloc and cudaFree per packed and freed layer).
-//   handles  what handles own.  What freed handles leave is kept for the next ones up to kHandleKeep bytes; spdp_free
-//            gives back what is over, and spdp_free(NULL) all of it.
-//   scratch  memory of one spdp_spmm call (its partial sums); keeps up to kScratchKeep bytes over a
-//            synchronisation, all given back when the device's last handle goes.
-// Both are stream-ordered, so calls on several streams or threads get memory of their own.
+// What a handle owns comes from cudaMalloc, so that the arrays behind spdp_get_info can be reached by a peer and exported to
+// another process like any other.  cudaMalloc and cudaFree are slow (about 3 ms per packed and freed layer), so blocks of freed
+// handles are kept for the next ones, at most kKeptBlocks of them and kHandleKeep bytes per device; spdp_free(NULL), and an
+// allocation that finds no memory, give them back to the driver.  A block is put here only when nothing on the device uses it
+// any more, so the next owner may be any thread and any stream.
+// The partial sums of one spdp_spmm call come from a stream-ordered pool (calls on several streams or threads get memory of their
+// own), apart from the device's default pool, which gives its memory back at every synchronisation: 0.45 ms per call.
+// It keeps up to kScratchKeep bytes over a synchronisation, all given back when the device's last handle goes and by
+// spdp_free(NULL).
 constexpr int kMaxDevices = 64;
 constexpr uint64_t kHandleKeep = uint64_t(512) << 20;
+constexpr int kKeptBlocks = 64;
 constexpr uint64_t kScratchKeep = uint64_t(96) << 20;
-struct DevicePools {
-    cudaMemPool_t handle_pool, scratch_pool;
+struct DeviceMemory {
+    DeviceBlock kept[kKeptBlocks];      // oldest first
+    int num_kept;
+    uint64_t bytes_kept;
+    cudaMemPool_t scratch_pool;
     int64_t handles;
 };
-std::mutex g_pools_mu;
-DevicePools g_pools[kMaxDevices];
+std::mutex g_memory_mu;
+DeviceMemory g_memory[kMaxDevices];
 
-// The pool in `slot`, made on first use; keeps up to `keep` unused bytes over a synchronisation.
-spdp_status pool_of(cudaMemPool_t DevicePools::*slot, int device, uint64_t keep, cudaMemPool_t* out) {
+// Takes block i out of the list (the lock is held).
+DeviceBlock take_kept(DeviceMemory& m, int i) {
+    const DeviceBlock b = m.kept[i];
+    for (int k = i + 1; k < m.num_kept; ++k) m.kept[k - 1] = m.kept[k];
+    --m.num_kept;
+    m.bytes_kept -= b.bytes;
+    return b;
+}
+
+// Gives every block that freed handles left on the device back to the driver.  Answers whether there was one.
+bool give_back_blocks(int device) {
+    bool any = false;
+    for (;;) {
+        DeviceBlock b = {};
+        {
+            std::lock_guard<std::mutex> lock(g_memory_mu);
+            DeviceMemory& m = g_memory[device];
+            if (m.num_kept > 0) b = take_kept(m, m.num_kept - 1);
+        }
+        if (b.p == nullptr) return any;
+        cudaFree(b.p);
+        any = true;
+    }
+}
+
+// A freed handle's block, for the next handle.  The caller has made sure that nothing on the device uses it any more.
+void keep_block(int device, DeviceBlock& block) {
+    const DeviceBlock b = block;
+    block = {};
+    if (b.p == nullptr) return;
+    if (b.bytes > kHandleKeep) { cudaFree(b.p); return; }
+    for (;;) {
+        DeviceBlock old = {};
+        {
+            std::lock_guard<std::mutex> lock(g_memory_mu);
+            DeviceMemory& m = g_memory[device];
+            if (m.num_kept < kKeptBlocks && m.bytes_kept + b.bytes <= kHandleKeep) {
+                m.kept[m.num_kept++] = b;
+                m.bytes_kept += b.bytes;
+                return;
+            }
+            old = take_kept(m, 0);
+        }
+        cudaFree(old.p);
+    }
+}
+
+// The stream-ordered pool of spdp_spmm's partial sums, made on first use.
+spdp_status scratch_pool_of(int device, cudaMemPool_t* out) {
     if (device < 0 || device >= kMaxDevices) return SPDP_ERR_UNSUPPORTED_SHAPE;
-    std::lock_guard<std::mutex> lock(g_pools_mu);
-    cudaMemPool_t& pool = g_pools[device].*slot;
+    std::lock_guard<std::mutex> lock(g_memory_mu);
+    cudaMemPool_t& pool = g_memory[device].scratch_pool;
     if (pool == nullptr) {
         cudaMemPoolProps props = {};
         props.allocType = cudaMemAllocationTypePinned;
@@ -54,6 +107,7 @@ spdp_status pool_of(cudaMemPool_t DevicePools::*slot, int device, uint64_t keep,
         props.location.id = device;
         cudaMemPool_t made = nullptr;
         SPDP_CUDA_TRY(cudaMemPoolCreate(&made, &props));
+        uint64_t keep = kScratchKeep;
         const cudaError_t e = cudaMemPoolSetAttribute(made, cudaMemPoolAttrReleaseThreshold, &keep);
         if (e != cudaSuccess) {
             cudaMemPoolDestroy(made);
@@ -65,24 +119,19 @@ spdp_status pool_of(cudaMemPool_t DevicePools::*slot, int device, uint64_t keep,
     return SPDP_OK;
 }
 
-void count_handle(int device, int by) {
-    if (device < 0 || device >= kMaxDevices) return;
-    std::lock_guard<std::mutex> lock(g_pools_mu);
-    DevicePools& p = g_pools[device];
-    p.handles += by;
-    if (p.handles == 0 && p.scratch_pool != nullptr) cudaMemPoolTrimTo(p.scratch_pool, 0);
+void trim_scratch(int device) {
+    std::lock_guard<std::mutex> lock(g_memory_mu);
+    if (g_memory[device].scratch_pool != nullptr) cudaMemPoolTrimTo(g_memory[device].scratch_pool, 0);
 }
 
-// Gives unused memory of the handle pool back until at most `keep` bytes of it are left.
-void trim_handles(int device, uint64_t keep) {
+void count_handle(int device, int by) {
     if (device < 0 || device >= kMaxDevices) return;
-    std::lock_guard<std::mutex> lock(g_pools_mu);
-    cudaMemPool_t pool = g_pools[device].handle_pool;
-    uint64_t used = 0, reserved = 0;
-    if (pool == nullptr || cudaMemPoolGetAttribute(pool, cudaMemPoolAttrUsedMemCurrent, &used) != cudaSuccess ||
-        cudaMemPoolGetAttribute(pool, cudaMemPoolAttrReservedMemCurrent, &reserved) != cudaSuccess)
-        return;
-    if (reserved > used + keep) cudaMemPoolTrimTo(pool, used + keep);
+    bool last;
+    {
+        std::lock_guard<std::mutex> lock(g_memory_mu);
+        last = (g_memory[device].handles += by) == 0;
+    }
+    if (last) trim_scratch(device);
 }
 
 // Makes `device` current for a scope.
@@ -96,11 +145,6 @@ struct DeviceScope {
     }
 };
 
-// The caller has made sure that nothing on the device uses the memory any more.
-void handle_free(void* p) {
-    if (p != nullptr) cudaFreeAsync(p, nullptr);
-}
-
 void drop_host_graph(spdp_matrix* h) {
     if (h->host_exec != nullptr) cudaGraphExecDestroy(h->host_exec);
     if (h->host_graph != nullptr) cudaGraphDestroy(h->host_graph);
@@ -112,14 +156,15 @@ void release(spdp_matrix* h) {
     if (h == nullptr) return;
     {
         DeviceScope on(h->device);
-        cudaDeviceSynchronize();            // as cudaFree would: the handle's memory may be in use on any stream
-        handle_free(h->arrays);
-        handle_free(h->values);
-        handle_free(h->workspace);
+        // the handle's memory may be in use on any stream (cudaFree would wait for them too)
+        const bool idle = cudaDeviceSynchronize() == cudaSuccess;
+        for (DeviceBlock* b : {&h->arrays, &h->values_block, &h->workspace_block, &h->packing}) {
+            if (idle) keep_block(h->device, *b);
+            else cudaFree(b->p);
+        }
+        if (!idle) cudaGetLastError();
         cudaFree(h->probe_items);
         cudaFree(h->probe_count);
-        cudaStreamSynchronize(nullptr);
-        trim_handles(h->device, kHandleKeep);
         drop_host_graph(h);
         if (h->capture_stream != nullptr) cudaStreamDestroy(h->capture_stream);
     }
@@ -164,9 +209,9 @@ spdp_status alloc_arrays(spdp_matrix* h, cudaStream_t s) {
                  tileoffset = place((h->NGT + 1) * sizeof(uint32_t)), scales = place(h->q4 ? cols * sizeof(__half) : 0),
                  x = place(h->K * sizeof(__half)), mask = place((h->K + 31) / 32 * sizeof(uint32_t)), y = place(h->M * sizeof(float)),
                  status = place(2 * sizeof(int));
-    spdp_status st = handle_alloc(h->device, at, s, &h->arrays);
+    spdp_status st = handle_alloc(h->device, at, &h->arrays);
     if (st != SPDP_OK) return st;
-    char* base = static_cast<char*>(h->arrays);
+    char* base = static_cast<char*>(h->arrays.p);
     h->bitmap = reinterpret_cast<uint64_t*>(base + bitmap);
     h->colinfo = reinterpret_cast<uint32_t*>(base + colinfo);
     h->tileoffset = reinterpret_cast<uint32_t*>(base + tileoffset);
@@ -188,7 +233,7 @@ spdp_status build_partition(spdp_matrix* h, int num_ctas, cudaStream_t s) {
     if (P > 1024) P = 1024;          // the kernel's range arithmetic is 32-bit: NGT < 2^22 times P must fit
     if (P > NGT) P = static_cast<int>(NGT);
     if (P < 1) P = 1;
-    handle_free(h->workspace);
+    keep_block(h->device, h->workspace_block);      // idle: a new handle has none, spdp_set_num_ctas has waited for the device
     h->workspace = h->workspace_batch = nullptr;
     // a recorded host-vector call holds the old workspace and CTA count: it is recorded anew
     drop_host_graph(h);
@@ -196,8 +241,9 @@ spdp_status build_partition(spdp_matrix* h, int num_ctas, cudaStream_t s) {
     h->num_ctas = P;
     const int64_t one = static_cast<int64_t>(P) * kTileM * sizeof(float);    // one row of split-K tree nodes per CTA
     h->workspace_bytes = one + batch_workspace_bytes(P);
-    spdp_status st = handle_alloc(h->device, h->workspace_bytes, s, reinterpret_cast<void**>(&h->workspace));
+    spdp_status st = handle_alloc(h->device, h->workspace_bytes, &h->workspace_block);
     if (st != SPDP_OK) return st;
+    h->workspace = static_cast<float*>(h->workspace_block.p);
     h->workspace_batch = h->workspace + P * kTileM;
     SPDP_CUDA_TRY(cudaMemsetAsync(h->workspace, 0, h->workspace_bytes, s));
     return SPDP_OK;
@@ -218,6 +264,7 @@ spdp_status finish_handle(spdp_matrix* h, cudaStream_t s) {
     st = configure_spmspv_q4_kernel();
     if (st != SPDP_OK) return st;
     SPDP_CUDA_TRY(cudaStreamSynchronize(s));
+    keep_block(h->device, h->packing);
     return SPDP_OK;
 }
 
@@ -235,17 +282,39 @@ bool rule_ok(int rule) { return rule == SPDP_DP_NONE || rule == SPDP_DP_ABS_GT |
 
 spdp_status scratch_alloc(int device, size_t bytes, cudaStream_t s, void** out) {
     cudaMemPool_t pool = nullptr;
-    const spdp_status st = pool_of(&DevicePools::scratch_pool, device, kScratchKeep, &pool);
+    const spdp_status st = scratch_pool_of(device, &pool);
     if (st != SPDP_OK) return st;
     SPDP_CUDA_TRY(cudaMallocFromPoolAsync(out, bytes, pool, s));
     return SPDP_OK;
 }
 
-spdp_status handle_alloc(int device, size_t bytes, cudaStream_t s, void** out) {
-    cudaMemPool_t pool = nullptr;
-    const spdp_status st = pool_of(&DevicePools::handle_pool, device, ~uint64_t(0), &pool);      // trimmed by hand, see trim_handles
-    if (st != SPDP_OK) return st;
-    SPDP_CUDA_TRY(cudaMallocFromPoolAsync(out, bytes, pool, s));
+// A block of 2 MB or more is a whole number of the driver's 2 MB pages anyway; a kept one serves where less than an eighth of it
+// (or 64 KB) would lie idle.
+spdp_status handle_alloc(int device, size_t bytes, DeviceBlock* out) {
+    if (device < 0 || device >= kMaxDevices) return SPDP_ERR_UNSUPPORTED_SHAPE;
+    const size_t unit = bytes >= (size_t(2) << 20) ? size_t(2) << 20 : 512;
+    bytes = (bytes + unit - 1) / unit * unit;
+    {
+        std::lock_guard<std::mutex> lock(g_memory_mu);
+        DeviceMemory& m = g_memory[device];
+        int best = -1;
+        for (int i = 0; i < m.num_kept; ++i)
+            if (m.kept[i].bytes >= bytes && m.kept[i].bytes - bytes <= std::max(bytes / 8, size_t(64) << 10) &&
+                (best < 0 || m.kept[i].bytes < m.kept[best].bytes))
+                best = i;
+        if (best >= 0) {
+            *out = take_kept(m, best);
+            return SPDP_OK;
+        }
+    }
+    void* p = nullptr;
+    cudaError_t e = cudaMalloc(&p, bytes);
+    if (e == cudaErrorMemoryAllocation && give_back_blocks(device)) {
+        cudaGetLastError();
+        e = cudaMalloc(&p, bytes);
+    }
+    SPDP_CUDA_TRY(e);
+    *out = {p, bytes};
     return SPDP_OK;
 }
 
@@ -455,8 +524,9 @@ spdp_status spdp_import_tiled_cbc(int64_t M, int64_t K, int pad_elems, const voi
     auto body = [&]() -> spdp_status {
         cudaStream_t s = nullptr;
         spdp_status a = alloc_arrays(h, s);
-        if (a == SPDP_OK) a = handle_alloc(h->device, vbytes < 16 ? 16 : vbytes, s, reinterpret_cast<void**>(&h->values));
+        if (a == SPDP_OK) a = handle_alloc(h->device, vbytes < 16 ? 16 : vbytes, &h->values_block);
         if (a != SPDP_OK) return a;
+        h->values = static_cast<__half*>(h->values_block.p);
         SPDP_CUDA_TRY(cudaStreamSynchronize(s));
         SPDP_CUDA_TRY(cudaMemcpy(h->tileoffset, to, (h->NGT + 1) * sizeof(uint32_t), cudaMemcpyHostToDevice));
         SPDP_CUDA_TRY(cudaMemcpy(h->colinfo, ci, h->NGT * kTileK * sizeof(uint32_t), cudaMemcpyHostToDevice));
@@ -619,7 +689,10 @@ spdp_status spdp_row_shard(int64_t M, int world, int rank, int64_t* first_row_ou
 
 spdp_status spdp_free(spdp_handle h) {
     if (h == nullptr) {                     // no handle: give back the memory that freed handles left
-        for (int d = 0; d < kMaxDevices; ++d) trim_handles(d, 0);
+        for (int d = 0; d < kMaxDevices; ++d) {
+            give_back_blocks(d);
+            trim_scratch(d);
+        }
         return SPDP_OK;
     }
     if (!valid(h)) return SPDP_ERR_INVALID_ARG;

@@ -4,7 +4,8 @@
 // Values are one contiguous span, which moves in 16-byte pieces.  (With one CTA per GTile a row of the dense side was 32
 // bytes and the values were scattered in runs of 2-byte stores.)  11008x4096 at 60 % sparsity: count 27, scan 8, emit 44,
 // unpack 45 us; between the block's loads and its stores a CTA has one serial pass over its 64 columns, which is what is
-// left.  Pack, unpack and free together took 3487 us, 3 ms of it cudaMalloc and cudaFree, and take 184 us.
+// left.  Pack, unpack and free together took 3487 us, 3 ms of it cudaMalloc and cudaFree, and take 175 us (memory of freed handles is
+// kept, see api.cu).
 #include <mutex>
 
 #include "spdp_internal.h"
@@ -375,41 +376,39 @@ spdp_status pack_device(spdp_matrix* h, const __half* W, int64_t ldw, cudaStream
     if (st != SPDP_OK) return st;
     uint32_t* tile_len = nullptr;
     unsigned long long* total_dev = nullptr;               // [0] Values length, [1] nnz
-    st = handle_alloc(h->device, 2 * sizeof(unsigned long long) + NGT * sizeof(uint32_t), s, reinterpret_cast<void**>(&total_dev));
+    st = handle_alloc(h->device, 2 * sizeof(unsigned long long) + NGT * sizeof(uint32_t), &h->packing);
     if (st != SPDP_OK) return st;
+    total_dev = static_cast<unsigned long long*>(h->packing.p);
     tile_len = reinterpret_cast<uint32_t*>(total_dev + 2);
     unsigned long long totals[2] = {0, 0};
-    auto body = [&]() -> spdp_status {
-        SPDP_CUDA_TRY(cudaMemsetAsync(total_dev, 0, 2 * sizeof(unsigned long long), s));
-        pack_count_kernel<<<grid, kTileM, 0, s>>>(Wb, ldw, h->M, h->K, h->C, blocks, h->pad_elems, h->bitmap, h->colinfo, tile_len,
-                                                  total_dev + 1);
-        pack_scan_kernel<<<1, 1024, 0, s>>>(tile_len, NGT, h->tileoffset, total_dev);
-        SPDP_CUDA_TRY(cudaMemcpyAsync(totals, total_dev, sizeof(totals), cudaMemcpyDeviceToHost, s));
-        SPDP_CUDA_TRY(cudaStreamSynchronize(s));
-        if (totals[0] >= (1ull << 32)) return SPDP_ERR_OVERFLOW;
-        h->values_len = static_cast<int64_t>(totals[0]);
-        h->nnz = static_cast<int64_t>(totals[1]);
-        if (h->q4) {
-            const size_t cbytes = static_cast<size_t>(totals[0]) / 2 + 16;     // + 16: the decode reads one word past a span
-            spdp_status a = handle_alloc(h->device, cbytes, s, reinterpret_cast<void**>(&h->values));
-            if (a != SPDP_OK) return a;
-            SPDP_CUDA_TRY(cudaMemsetAsync(h->values, 0, cbytes, s));
-            pack_q4_emit_kernel<<<static_cast<unsigned>(NGT), kTileM, 0, s>>>(
-                Wb, ldw, h->M, h->K, h->C, h->tileoffset, h->colinfo, reinterpret_cast<unsigned char*>(h->values),
-                reinterpret_cast<unsigned short*>(h->scales));
-        } else {
-            const size_t vbytes = static_cast<size_t>(totals[0]) * sizeof(__half);
-            spdp_status a = handle_alloc(h->device, vbytes < 16 ? 16 : vbytes, s, reinterpret_cast<void**>(&h->values));
-            if (a != SPDP_OK) return a;
-            pack_emit_kernel<<<grid, kTileM, sizeof(PackSmem), s>>>(Wb, ldw, h->M, h->K, h->C, blocks, h->pad_elems, h->tileoffset,
-                                                                    h->colinfo, h->bitmap, reinterpret_cast<unsigned short*>(h->values));
-        }
-        SPDP_CUDA_TRY(cudaGetLastError());
-        return SPDP_OK;
-    };
-    st = body();
-    cudaFreeAsync(total_dev, s);
-    return st;
+    SPDP_CUDA_TRY(cudaMemsetAsync(total_dev, 0, 2 * sizeof(unsigned long long), s));
+    pack_count_kernel<<<grid, kTileM, 0, s>>>(Wb, ldw, h->M, h->K, h->C, blocks, h->pad_elems, h->bitmap, h->colinfo, tile_len,
+                                              total_dev + 1);
+    pack_scan_kernel<<<1, 1024, 0, s>>>(tile_len, NGT, h->tileoffset, total_dev);
+    SPDP_CUDA_TRY(cudaMemcpyAsync(totals, total_dev, sizeof(totals), cudaMemcpyDeviceToHost, s));
+    SPDP_CUDA_TRY(cudaStreamSynchronize(s));
+    if (totals[0] >= (1ull << 32)) return SPDP_ERR_OVERFLOW;
+    h->values_len = static_cast<int64_t>(totals[0]);
+    h->nnz = static_cast<int64_t>(totals[1]);
+    if (h->q4) {
+        const size_t cbytes = static_cast<size_t>(totals[0]) / 2 + 16;     // + 16: the decode reads one word past a span
+        spdp_status a = handle_alloc(h->device, cbytes, &h->values_block);
+        if (a != SPDP_OK) return a;
+        h->values = static_cast<__half*>(h->values_block.p);
+        SPDP_CUDA_TRY(cudaMemsetAsync(h->values, 0, cbytes, s));
+        pack_q4_emit_kernel<<<static_cast<unsigned>(NGT), kTileM, 0, s>>>(
+            Wb, ldw, h->M, h->K, h->C, h->tileoffset, h->colinfo, reinterpret_cast<unsigned char*>(h->values),
+            reinterpret_cast<unsigned short*>(h->scales));
+    } else {
+        const size_t vbytes = static_cast<size_t>(totals[0]) * sizeof(__half);
+        spdp_status a = handle_alloc(h->device, vbytes < 16 ? 16 : vbytes, &h->values_block);
+        if (a != SPDP_OK) return a;
+        h->values = static_cast<__half*>(h->values_block.p);
+        pack_emit_kernel<<<grid, kTileM, sizeof(PackSmem), s>>>(Wb, ldw, h->M, h->K, h->C, blocks, h->pad_elems, h->tileoffset,
+                                                                h->colinfo, h->bitmap, reinterpret_cast<unsigned short*>(h->values));
+    }
+    SPDP_CUDA_TRY(cudaGetLastError());
+    return SPDP_OK;
 }
 
 spdp_status unpack_device(const spdp_matrix* h, __half* W, int64_t ldw, cudaStream_t s) {

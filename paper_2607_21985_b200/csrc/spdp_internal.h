@@ -14,6 +14,12 @@ constexpr int kTileK = 16;         // column tiles per GTile (Sec. 4.2.3)
 constexpr int kWordsPerCol = 4;    // 64-bit bitmap words per column tile (Sec. 4.1)
 constexpr uint64_t kMagic = 0x5350445042323030ull;   // "SPDPB200"
 
+// A piece of device memory from cudaMalloc that a handle owns (see handle_alloc).
+struct DeviceBlock {
+    void* p;
+    size_t bytes;
+};
+
 }  // namespace spdp
 
 // Host-side state behind an spdp_handle.
@@ -28,7 +34,7 @@ struct spdp_matrix {
 
     // Tiled-CBC arrays (device).  `arrays` is the allocation that holds every array whose size follows from the shape:
     // tileoffset, colinfo, bitmap, scales, the status word and the staging buffers; values has its own.
-    void* arrays;
+    spdp::DeviceBlock arrays, values_block;
     uint32_t* tileoffset;   // [NGT+1]
     uint32_t* colinfo;      // [NGT*16]
     uint64_t* bitmap;       // [NGT*16*4]
@@ -39,8 +45,10 @@ struct spdp_matrix {
     // Work partition of one spmspv launch: the kernel cuts the NGT GTiles into num_ctas equal
     // contiguous ranges, one per CTA.
     int num_ctas;           // P
-    float* workspace;       // device [P*256] split-K tree nodes, one row per CTA (all zero between calls); own allocation
-    float* workspace_batch; // device [P*8*256] tree nodes of the small-batch call (all zero between calls), in the same one
+    float* workspace;       // device [P*256] split-K tree nodes, one row per CTA (all zero between calls)
+    float* workspace_batch; // device [P*8*256] tree nodes of the small-batch call (all zero between calls)
+    spdp::DeviceBlock workspace_block;  // both
+    spdp::DeviceBlock packing;          // lengths and totals while packing
     int* status_word;       // device [2]: the status word, and a sink word the benchmark probes may write
     int64_t workspace_bytes;
 
@@ -94,8 +102,8 @@ inline bool valid(const spdp_matrix* h) { return h != nullptr && h->magic == kMa
 
 // api.cu: stream-ordered scratch memory for one call (given back with cudaFreeAsync on the same stream).
 spdp_status scratch_alloc(int device, size_t bytes, cudaStream_t s, void** out);
-// api.cu: memory that a handle owns (given back with handle_free); usable on other streams once `s` has been synchronised.
-spdp_status handle_alloc(int device, size_t bytes, cudaStream_t s, void** out);
+// api.cu: memory that a handle owns, usable on any stream; release() keeps it for the next handle.
+spdp_status handle_alloc(int device, size_t bytes, DeviceBlock* out);
 
 // pack.cu
 spdp_status configure_pack_kernels();          // per-device kernel attributes; idempotent

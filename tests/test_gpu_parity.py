@@ -542,6 +542,53 @@ def test_free_of_nothing_gives_kept_memory_back(S):
     assert torch.cuda.mem_get_info()[0] >= kept + (16 << 20)                    # the layer's 16 MB of values at least
 
 
+def test_packed_arrays_can_be_exported_to_another_process(S):
+    """What spdp_get_info names are ordinary device allocations: the runtime gives an interprocess handle for them, for a new
+    handle and for one that got the memory of a freed one."""
+    import ctypes
+    rt = ctypes.CDLL("libcudart.so.12")
+    W = torch.ones((1024, 2048), dtype=torch.float16, device="cuda")
+    for _ in range(2):
+        h = S.spdp_pack_tiled_cbc(W)
+        try:
+            info = S.spdp_get_info(h)
+            for p in (info.values_dev, info.bitmap_dev, info.colinfo_dev, info.tileoffset_dev):
+                assert rt.cudaIpcGetMemHandle(ctypes.create_string_buffer(64), ctypes.c_void_p(p)) == 0
+        finally:
+            S.spdp_free(h)
+
+
+def test_threads_pack_and_free_side_by_side(S):
+    """Memory of freed handles goes to the next ones, on other threads and streams too: every layer keeps its own arrays."""
+    import concurrent.futures as cf
+
+    def work(seed):
+        torch.cuda.set_device(0)
+        rng = np.random.Generator(np.random.PCG64(seed))
+        side = torch.cuda.Stream()
+        with torch.cuda.stream(side):
+            for step in range(12):
+                M, K = 256 * int(rng.integers(1, 6)), 16 * int(rng.integers(1, 40))
+                W = rng.integers(-4, 5, (M, K)).astype(np.float16)
+                W[rng.random((M, K)) < 0.5] = 0
+                x = rng.integers(-3, 4, K).astype(np.float16)
+                Wd, xd, y = dev(W), dev(x), torch.full((M,), float("nan"), dtype=torch.float32, device="cuda")
+                back = torch.empty_like(Wd)
+                h = S.spdp_pack_tiled_cbc(Wd, stream=side)
+                try:
+                    for _ in range(3):
+                        S.spdp_spmspv(h, xd, O.DP_NONE, 0.0, y, stream=side)
+                    S.spdp_unpack(h, back, stream=side)
+                    side.synchronize()
+                finally:
+                    S.spdp_free(h)
+                assert np.array_equal(y.cpu().numpy(), W.astype(np.float32) @ x.astype(np.float32))
+                assert np.array_equal(back.cpu().numpy(), np.where(W == 0, np.float16(0), W))
+        return seed
+    with cf.ThreadPoolExecutor(6) as pool:
+        assert list(pool.map(work, range(6))) == list(range(6))
+
+
 @pytest.mark.parametrize("K", [1, 2, 31, 63, 64, 65, 127, 129, 1023, 3100, 8191, 8193])
 @pytest.mark.parametrize("ctas", [0, 1, 2, 5])
 def test_active_list_edges(S, K, ctas):
