@@ -1023,7 +1023,7 @@ constexpr double kTileUs = 2.1, kTileTokenUs = 2.3e-3;                  // a til
 constexpr double kReduceUs = 1.9, kReducePerMB = 0.223;                 // the second kernel; writing and reading a MB of partial sums
 constexpr int kTokens[4] = {One32::kNI, One128::kNI, One256::kNI, pair::kNT};
 
-Plan make_plan(int64_t R, int64_t nkb, int64_t N, int sms) {
+Plan make_plan(int64_t R, int64_t nkb, int64_t N, int sms, bool may_cut) {
     Plan best = {};
     best.us = -1.0;
     for (int f = 0; f < 4; ++f) {
@@ -1045,7 +1045,7 @@ Plan make_plan(int64_t R, int64_t nkb, int64_t N, int sms) {
         q.rest = f == 3 ? 0 : left;
         q.us = whole + (left > 0 ? block * static_cast<double>(nkb) + tile : 0.0);
         if (best.us < 0.0 || q.us < best.us) best = q;
-        if (left == 0) continue;
+        if (left == 0 || !may_cut) continue;
         const auto consider = [&](int64_t w) {                                   // w CTAs (pairs) share the tiles that are left
             if (f == 3) {
                 q.slices = static_cast<int>(std::min<int64_t>(w / left, nkb));
@@ -1118,33 +1118,14 @@ spdp_status launch_reduce(Kernel kernel, const spdp_matrix* h, int64_t tiles, cu
     return SPDP_OK;
 }
 
-}  // namespace
-
-spdp_status launch_spmm(const spdp_matrix* h, const __half* X, int64_t N, int64_t ldx, void* Y, int64_t ldy, int ydt,
-                        cudaStream_t s) {
-    Params p = {};
-    p.tileoffset = h->tileoffset;
-    p.colinfo = h->colinfo;
-    p.bitmap = h->bitmap;
-    p.values = h->values;
-    p.N = N;
-    p.Y = Y;
-    p.ldy = ldy;
-    p.ydt = ydt;
-    p.M = static_cast<int>(h->M);
-    p.K = static_cast<int>(h->K);
-    p.C = static_cast<int>(h->C);
-    p.status = h->status_word;
-    p.values_len = h->values_len;
-    p.nkb = static_cast<int>((h->K + kKB - 1) / kKB);
-    const Plan plan = make_plan(h->R, p.nkb, N, h->sm_count > 1 ? h->sm_count : 2);
+spdp_status run_plan(const spdp_matrix* h, Params p, const Plan& plan, const __half* X, int64_t ldx, cudaStream_t s) {
     if (plan.tiles * p.nkb >= (int64_t(1) << 31)) return SPDP_ERR_UNSUPPORTED_SHAPE;
     const int nt = kTokens[plan.kernel];
-    p.nblocks = static_cast<int>((N + nt - 1) / nt);
-    p.ptok = static_cast<int>(std::min<int64_t>(N, nt));
+    p.nblocks = static_cast<int>((p.N + nt - 1) / nt);
+    p.ptok = static_cast<int>(std::min<int64_t>(p.N, nt));
     p.kslices = 1;
     CUtensorMap xmap;
-    spdp_status st = encode_x(&xmap, X, N, h->K, ldx, plan.kernel == 3 ? pair::kNI / 2 : nt);
+    spdp_status st = encode_x(&xmap, X, p.N, h->K, ldx, plan.kernel == 3 ? pair::kNI / 2 : nt);
     if (st != SPDP_OK) return st;
     const bool cut = plan.rest > 0 && plan.sharers > plan.rest;              // partial sums and a second kernel
     if (cut) {
@@ -1173,6 +1154,32 @@ spdp_status launch_spmm(const spdp_matrix* h, const __half* X, int64_t N, int64_
             st = launch_reduce(one::reduce_pieces_kernel, h, plan.rest, s, p, plan.rounds * plan.workers, static_cast<int>(plan.rest), nt);
     }
     if (cut) cudaFreeAsync(p.partial, s);
+    return st;
+}
+
+}  // namespace
+
+spdp_status launch_spmm(const spdp_matrix* h, const __half* X, int64_t N, int64_t ldx, void* Y, int64_t ldy, int ydt,
+                        cudaStream_t s) {
+    Params p = {};
+    p.tileoffset = h->tileoffset;
+    p.colinfo = h->colinfo;
+    p.bitmap = h->bitmap;
+    p.values = h->values;
+    p.N = N;
+    p.Y = Y;
+    p.ldy = ldy;
+    p.ydt = ydt;
+    p.M = static_cast<int>(h->M);
+    p.K = static_cast<int>(h->K);
+    p.C = static_cast<int>(h->C);
+    p.status = h->status_word;
+    p.values_len = h->values_len;
+    p.nkb = static_cast<int>((h->K + kKB - 1) / kKB);
+    const int sms = h->sm_count > 1 ? h->sm_count : 2;
+    spdp_status st = run_plan(h, p, make_plan(h->R, p.nkb, N, sms, true), X, ldx, s);
+    // No memory for partial sums: whole tiles only, which need none.  Slower, and another order of the sums.
+    if (st == SPDP_ERR_ALLOC) st = run_plan(h, p, make_plan(h->R, p.nkb, N, sms, false), X, ldx, s);
     return st;
 }
 

@@ -219,3 +219,37 @@ def test_spmm_calls_in_a_row(S, R, K, N, sp):
         assert S.spdp_last_device_status(h) == 0
     finally:
         S.spdp_free(h)
+
+
+@pytest.mark.parametrize("R,K,N", [(6, 8192, 512), (43, 4096, 200), (8, 4096, 1024)])
+def test_spmm_without_memory_for_partial_sums(S, R, K, N):
+    """Shapes whose tiles are cut along K (75, 61 and 34 MB of partial sums), called while the device has less memory than that
+    left: whole tiles then, same results."""
+    rng = np.random.Generator(np.random.PCG64(R))
+    M = 256 * R
+    W = rng.integers(-4, 5, (M, K)).astype(np.float16)
+    W[rng.random((M, K)) < 0.5] = 0
+    X = dev(rng.integers(-2, 3, (N, K)).astype(np.float16))
+    want = torch.from_numpy(X.float().cpu().numpy() @ W.astype(np.float32).T)
+    h = S.spdp_pack_tiled_cbc(dev(W))
+    Y = torch.full((2, N, M), float("nan"), dtype=torch.float32, device="cuda")
+    hold = []
+    try:
+        S.spdp_free(None)                                      # the scratch memory that the library keeps
+        torch.cuda.empty_cache()
+        for piece in (1 << 30, 64 << 20, 8 << 20):
+            while torch.cuda.mem_get_info()[0] > piece + (16 << 20):
+                hold.append(torch.empty(min(torch.cuda.mem_get_info()[0] - (16 << 20), 16 << 30) // piece * piece, dtype=torch.uint8, device="cuda"))
+        assert torch.cuda.mem_get_info()[0] < 30 << 20
+        S.spdp_spmm(h, X, Y[0])
+        torch.cuda.synchronize()
+        hold.clear()
+        torch.cuda.empty_cache()
+        S.spdp_spmm(h, X, Y[1])
+        torch.cuda.synchronize()
+        assert S.spdp_last_device_status(h) == 0
+    finally:
+        hold.clear()
+        torch.cuda.empty_cache()
+        S.spdp_free(h)
+    assert torch.equal(Y[0].cpu(), want) and torch.equal(Y[1].cpu(), want)
