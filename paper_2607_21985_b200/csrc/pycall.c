@@ -6,19 +6,57 @@
 #include <Python.h>
 #include <stdint.h>
 
+/* What ctypes takes for a number or an address besides an int: one of its own simple values (a handle or stream kept as a
+ * c_void_p, say) and anything with _as_parameter_.  A new reference, or NULL with the error set. */
+static PyObject* plain(PyObject* o) {
+    static PyObject* simple = NULL;
+    PyObject* v = PyObject_GetAttrString(o, "_as_parameter_");
+    if (v != NULL) return v;
+    PyErr_Clear();
+    if (simple == NULL) {
+        PyObject* m = PyImport_ImportModule("ctypes");
+        simple = m != NULL ? PyObject_GetAttrString(m, "_SimpleCData") : NULL;
+        Py_XDECREF(m);
+        if (simple == NULL) return NULL;
+    }
+    switch (PyObject_IsInstance(o, simple)) {
+        case 1: return PyObject_GetAttrString(o, "value");
+        case 0: PyErr_Format(PyExc_TypeError, "an int or None, not %.80s", Py_TYPE(o)->tp_name);
+    }
+    return NULL;
+}
+
+/* kind 'p': an address, or None for a null pointer; 'i': an integer.  Kept out of the converters, which are inlined. */
+static __attribute__((noinline)) int from_other(PyObject* o, char kind, void** ptr, int64_t* i64) {
+    PyObject* v = plain(o);
+    int ok = v != NULL;
+    if (ok && kind == 'p' && v == Py_None) *ptr = NULL;
+    else if (ok && PyLong_Check(v)) {
+        if (kind == 'p') *ptr = PyLong_AsVoidPtr(v);
+        else *i64 = PyLong_AsLongLong(v);
+        ok = !PyErr_Occurred();
+    } else if (ok) {
+        PyErr_Format(PyExc_TypeError, "an int or None, not %.80s", Py_TYPE(o)->tp_name);
+        ok = 0;
+    }
+    Py_XDECREF(v);
+    return ok;
+}
 static int as_ptr(PyObject* o, void** out) {
     if (o == Py_None) { *out = NULL; return 1; }
+    if (!PyLong_Check(o)) return from_other(o, 'p', out, NULL);
     *out = PyLong_AsVoidPtr(o);
     return !(*out == NULL && PyErr_Occurred());
 }
 static int as_i64(PyObject* o, int64_t* out) {
+    if (!PyLong_Check(o)) return from_other(o, 'i', NULL, out);
     *out = PyLong_AsLongLong(o);
     return !(*out == -1 && PyErr_Occurred());
 }
 static int as_int(PyObject* o, int* out) {
-    const long v = PyLong_AsLong(o);
-    if (v == -1 && PyErr_Occurred()) return 0;
-    if (v != (long)(int)v) { PyErr_SetString(PyExc_OverflowError, "argument does not fit a C int"); return 0; }
+    int64_t v;
+    if (!as_i64(o, &v)) return 0;
+    if (v != (int64_t)(int)v) { PyErr_SetString(PyExc_OverflowError, "argument does not fit a C int"); return 0; }
     *out = (int)v;
     return 1;
 }

@@ -44,3 +44,22 @@ def test_arguments_arrive(L):
     assert seen == [(5, (1 << 64) - 16, 2, -0.25, None, 7, 1, None)]
     with pytest.raises(OverflowError):
         _pycall.spmspv(ctypes.cast(cb, ctypes.c_void_p).value, 5, 6, 1 << 40, 0.0, None, 7, 1, 0)
+
+
+def test_ctypes_values_are_taken_as_ctypes_takes_them(L):
+    """A handle or stream kept as a ctypes value (or an object that names its own) goes through as it does through ctypes itself."""
+    from paper_2607_21985_b200 import _pycall
+    seen = []
+    vp, ci = ctypes.c_void_p, ctypes.c_int
+    sig = ctypes.CFUNCTYPE(ci, vp, vp, ci, ctypes.c_float, vp, vp, ci, vp)
+    cb = sig(lambda *a: seen.append(a) or 0)
+
+    class Stream:
+        _as_parameter_ = 99
+    args = (vp(5), 6, ci(2), 0.5, vp(None), vp(7), 1, Stream())
+    assert cb(*args) == 0 and _pycall.spmspv(ctypes.cast(cb, vp).value, *args) == 0
+    assert seen == [(5, 6, 2, 0.5, None, 7, 1, 99)] * 2
+    for bad in ("x", b"x", 5.0, vp, object(), ctypes.c_float(1.0)):
+        with pytest.raises(TypeError):
+            _pycall.spmspv(ctypes.cast(cb, vp).value, bad, *args[1:])
+    assert len(seen) == 2
