@@ -12,7 +12,7 @@ HERE = os.path.dirname(os.path.abspath(__file__))
 ROOT = os.path.dirname(HERE)
 LIB = os.path.join(HERE, "libspdp.so")
 LIB_CHECKED = os.path.join(HERE, "libspdp_checked.so")      # same sources with -DSPDP_CHECKED
-PYCALL = os.path.join(HERE, "_pycall.so")
+PYCALL = os.path.join(HERE, "_pycall" + sysconfig.get_config_var("EXT_SUFFIX"))    # one per interpreter: each imports its own
 PYCALL_SOURCE = os.path.join(HERE, "csrc", "pycall.c")
 SOURCES = sorted(glob.glob(os.path.join(HERE, "csrc", "*.cu")))
 HEADERS = sorted(glob.glob(os.path.join(HERE, "csrc", "*.h")) + glob.glob(os.path.join(HERE, "csrc", "*.cuh"))
@@ -50,7 +50,7 @@ def _compile(lib: str, extra, verbose: bool) -> str:
 
 def build_pycall(force: bool = False) -> str:
     """The C module behind the per-token calls of spdp.py (csrc/pycall.c)."""
-    if not force and os.path.exists(PYCALL) and os.path.getmtime(PYCALL) >= os.path.getmtime(PYCALL_SOURCE):
+    if not force and os.path.exists(PYCALL) and all(os.path.getmtime(f) <= os.path.getmtime(PYCALL) for f in (PYCALL_SOURCE, os.path.abspath(__file__))):
         return PYCALL
     tmp = PYCALL + f".tmp{os.getpid()}"
     subprocess.run(["gcc", "-O2", "-Wall", "-shared", "-fPIC", "-I", sysconfig.get_paths()["include"], "-o", tmp, PYCALL_SOURCE], check=True)

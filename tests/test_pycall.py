@@ -63,3 +63,13 @@ def test_ctypes_values_are_taken_as_ctypes_takes_them(L):
         with pytest.raises(TypeError):
             _pycall.spmspv(ctypes.cast(cb, vp).value, bad, *args[1:])
     assert len(seen) == 2
+
+
+def test_module_belongs_to_this_interpreter(L):
+    """A module built for another Python is neither imported nor taken for up to date."""
+    import importlib.machinery
+    import os
+    from paper_2607_21985_b200 import _pycall
+    suffix = importlib.machinery.EXTENSION_SUFFIXES[0]
+    assert "cpython" in suffix and os.path.basename(build.PYCALL) == "_pycall" + suffix
+    assert os.path.samefile(_pycall.__file__, build.PYCALL)
