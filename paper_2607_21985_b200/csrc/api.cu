@@ -233,19 +233,26 @@ spdp_status build_partition(spdp_matrix* h, int num_ctas, cudaStream_t s) {
     if (P > 1024) P = 1024;          // the kernel's range arithmetic is 32-bit: NGT < 2^22 times P must fit
     if (P > NGT) P = static_cast<int>(NGT);
     if (P < 1) P = 1;
+    const int64_t one = static_cast<int64_t>(P) * kTileM * sizeof(float);    // one row of split-K tree nodes per CTA
+    const int64_t bytes = one + batch_workspace_bytes(P);
+    // the new workspace first: where there is no memory for it the handle keeps the one it has
+    DeviceBlock fresh = {};
+    const spdp_status st = handle_alloc(h->device, bytes, &fresh);
+    if (st != SPDP_OK) return st;
+    const cudaError_t e = cudaMemsetAsync(fresh.p, 0, bytes, s);
+    if (e != cudaSuccess) {
+        keep_block(h->device, fresh);
+        SPDP_CUDA_TRY(e);
+    }
     keep_block(h->device, h->workspace_block);      // idle: a new handle has none, spdp_set_num_ctas has waited for the device
-    h->workspace = h->workspace_batch = nullptr;
+    h->workspace_block = fresh;
+    h->workspace = static_cast<float*>(fresh.p);
+    h->workspace_batch = h->workspace + P * kTileM;
+    h->workspace_bytes = bytes;
+    h->num_ctas = P;
     // a recorded host-vector call holds the old workspace and CTA count: it is recorded anew
     drop_host_graph(h);
     h->host_calls = 0;
-    h->num_ctas = P;
-    const int64_t one = static_cast<int64_t>(P) * kTileM * sizeof(float);    // one row of split-K tree nodes per CTA
-    h->workspace_bytes = one + batch_workspace_bytes(P);
-    spdp_status st = handle_alloc(h->device, h->workspace_bytes, &h->workspace_block);
-    if (st != SPDP_OK) return st;
-    h->workspace = static_cast<float*>(h->workspace_block.p);
-    h->workspace_batch = h->workspace + P * kTileM;
-    SPDP_CUDA_TRY(cudaMemsetAsync(h->workspace, 0, h->workspace_bytes, s));
     return SPDP_OK;
 }
 

@@ -542,6 +542,45 @@ def test_free_of_nothing_gives_kept_memory_back(S):
     assert torch.cuda.mem_get_info()[0] >= kept + (16 << 20)                    # the layer's 16 MB of values at least
 
 
+def test_handle_keeps_its_workspace_where_there_is_no_memory_for_a_new_one(S):
+    """1024 CTAs need a workspace of 9.4 MB; with less than that free the call is refused and the handle works on as it was."""
+    import ctypes
+    rt = ctypes.CDLL("libcudart.so.12")
+    rng = np.random.Generator(np.random.PCG64(5))
+    W = rng.integers(-4, 5, (4096, 1024)).astype(np.float16)                    # 1024 GTiles
+    x = rng.integers(-3, 4, 1024).astype(np.float16)
+    want = W.astype(np.float32) @ x.astype(np.float32)
+    h, xd, y = S.spdp_pack_tiled_cbc(dev(W)), dev(x), torch.empty(4096, dtype=torch.float32, device="cuda")
+    hold = []
+    try:
+        ctas = S.spdp_get_info(h).num_ctas
+        S.spdp_free(None)
+        torch.cuda.empty_cache()
+        free = lambda: torch.cuda.mem_get_info()[0]
+        while free() > 8 << 20:
+            p = ctypes.c_void_p()
+            assert rt.cudaMalloc(ctypes.byref(p), ctypes.c_size_t(max((free() - (6 << 20)) >> 21 << 20, 2 << 20))) == 0
+            hold.append(p)
+        with pytest.raises(S.SpdpError, match="ERR_ALLOC"):
+            S.spdp_set_num_ctas(h, 1024)
+        assert S.spdp_get_info(h).num_ctas == ctas
+        for _ in range(2):
+            y.fill_(float("nan"))
+            S.spdp_spmspv(h, xd, O.DP_NONE, 0.0, y)
+            assert np.array_equal(y.cpu().numpy(), want)
+        for p in hold:
+            assert rt.cudaFree(p) == 0
+        hold = []
+        S.spdp_set_num_ctas(h, 1024)
+        assert S.spdp_get_info(h).num_ctas == 1024
+        S.spdp_spmspv(h, xd, O.DP_NONE, 0.0, y)
+        assert np.array_equal(y.cpu().numpy(), want)
+    finally:
+        for p in hold:
+            rt.cudaFree(p)
+        S.spdp_free(h)
+
+
 def test_packed_arrays_can_be_exported_to_another_process(S):
     """What spdp_get_info names are ordinary device allocations: the runtime gives an interprocess handle for them, for a new
     handle and for one that got the memory of a freed one."""
