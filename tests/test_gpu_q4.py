@@ -122,3 +122,28 @@ def test_q4_exact_when_weights_lie_on_the_grid_and_other_calls_are_refused(S):
             S.spdp_unpack(h, torch.zeros((M, K), dtype=torch.float16, device="cuda"))
     finally:
         S.spdp_free(h)
+
+
+@pytest.mark.parametrize("K", [8, 1000, 4099])
+def test_q4_host_vectors_in_pinned_buffers(S, K):
+    """The host-vector call on a 4-bit handle with pinned buffers: first call, recorded call and replays with other buffers,
+    rule, threshold and output type agree with the device-vector call bit for bit."""
+    rng = np.random.Generator(np.random.PCG64(K))
+    M = 900
+    W = rng.standard_normal((M, K)).astype(np.float16)
+    W[rng.random((M, K)) < 0.5] = 0
+    words = O.active_to_words(rng.random(K) < 0.5)
+    mask = torch.from_numpy(words.view(np.int32)).pin_memory()
+    h = S.spdp_pack_tiled_cbc_q4(dev(W))
+    try:
+        for call in range(12):
+            x = rng.standard_normal(K).astype(np.float16)
+            xh = torch.from_numpy(x).pin_memory()
+            dt = torch.float32 if call % 4 == 3 else torch.float16
+            rule, thr = (O.DP_MASK, 0.0) if call % 3 == 2 else (O.DP_ABS_GT, 0.25 * (call // 3))
+            want, yh = torch.empty(M, dtype=dt, device="cuda"), torch.full((M,), float("nan"), dtype=dt).pin_memory()
+            S.spdp_spmspv(h, dev(x), rule, thr, want, mask=dev(words) if rule == O.DP_MASK else None)
+            S.spdp_spmspv_host(h, xh, rule, thr, yh, mask_host=mask if rule == O.DP_MASK else None)
+            assert torch.equal(yh, want.cpu()), call
+    finally:
+        S.spdp_free(h)

@@ -253,3 +253,65 @@ def test_spmm_without_memory_for_partial_sums(S, R, K, N):
         torch.cuda.empty_cache()
         S.spdp_free(h)
     assert torch.equal(Y[0].cpu(), want) and torch.equal(Y[1].cpu(), want)
+
+
+CUT = [(6, 4096, 32), (6, 8192, 40), (43, 4096, 128), (6, 8192, 512), (16, 4104, 300)]      # 32, 128, 128, 256 tokens per CTA, CTA pairs
+
+
+def _cut_layer(S, R, K, N, count):
+    """A layer, `count` inputs and their exact products; on integers every partial sum is exact."""
+    rng = np.random.Generator(np.random.PCG64(R + N))
+    W = rng.integers(-4, 5, (256 * R, K)).astype(np.float16)
+    W[rng.random(W.shape) < 0.5] = 0
+    X = [dev(rng.integers(-2, 3, (N, K)).astype(np.float16)) for _ in range(count)]
+    Wd = dev(W).double()
+    return S.spdp_pack_tiled_cbc(dev(W)), X, [(x.double() @ Wd.T).float() for x in X]
+
+
+@pytest.mark.parametrize("R,K,N", CUT)
+def test_spmm_cut_tiles_in_a_graph(S, R, K, N):
+    """A captured call whose partial sums are memory of the graph: replays on new inputs, with direct calls in between."""
+    h, X, want = _cut_layer(S, R, K, N, 3)
+    try:
+        buf, Y = torch.zeros_like(X[0]), torch.empty_like(want[0])
+        direct = torch.empty_like(Y)
+        S.spdp_spmm(h, buf, Y)
+        torch.cuda.synchronize()
+        graph = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(graph):
+            S.spdp_spmm(h, buf, Y)
+            S.spdp_spmm(h, buf, Y)
+        for _ in range(2):
+            for x, w in zip(X, want):
+                buf.copy_(x)
+                Y.fill_(float("nan"))
+                graph.replay()
+                S.spdp_spmm(h, X[0], direct)
+                graph.replay()
+                torch.cuda.synchronize()
+                assert torch.equal(Y, w) and torch.equal(direct, want[0])
+        assert S.spdp_last_device_status(h) == 0
+        del graph
+    finally:
+        S.spdp_free(h)
+
+
+@pytest.mark.parametrize("a,b", [(0, 3), (1, 4), (2, 2), (4, 4)])
+def test_spmm_cut_tiles_on_two_streams(S, a, b):
+    """Calls on two streams that may run side by side, on two handles or on the same one: each has partial sums of its own."""
+    layers = [_cut_layer(S, *CUT[a], 2), None]
+    layers[1] = layers[0] if a == b else _cut_layer(S, *CUT[b], 2)
+    streams = [torch.cuda.Stream(), torch.cuda.Stream()]
+    try:
+        Y = [[torch.full_like(w, float("nan")) for w in want for _ in range(4)] for _, _, want in layers]
+        torch.cuda.synchronize()
+        for k in range(len(Y[0])):
+            for (h, X, _), s, y in zip(layers, streams, Y):
+                S.spdp_spmm(h, X[k // 4], y[k], stream=s)
+        torch.cuda.synchronize()
+        for (h, _, want), y in zip(layers, Y):
+            assert all(torch.equal(y[k], want[k // 4]) for k in range(len(y)))
+            assert S.spdp_last_device_status(h) == 0
+    finally:
+        for h in {layers[0][0], layers[1][0]}:
+            S.spdp_free(h)
