@@ -70,8 +70,8 @@ typedef struct {
     int64_t values_len;        /* = TileOffset[NGT], padding included                           */
     int64_t packed_bytes;      /* bytes of TileOffset + ColInfo + Bitmap + Values               */
     int64_t workspace_bytes;   /* split-K scratch owned by the handle                           */
-    /* The arrays lie in cudaMalloc allocations: one starts at values_dev, one at bitmap_dev, which holds the other two behind it.
-     * They may be read by a peer or exported to another process, until the handle is freed. */
+    /* The arrays lie inside cudaMalloc allocations, several in one: they may be read by a peer or exported to another process
+     * (an exported handle stands for the whole allocation, whose start cuMemGetAddressRange tells), until the handle is freed. */
     const void* tileoffset_dev;  /* uint32[NGT+1]  start of each GTile in Values (elements)      */
     const void* colinfo_dev;     /* uint32[NGT*16] (column start inside its GTile) << 16 | nnz   */
     const void* bitmap_dev;      /* uint64[NGT*16*4] bit b of word w = row 64*w+b of the column tile */

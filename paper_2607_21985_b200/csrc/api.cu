@@ -3,10 +3,8 @@
 // spmspv.cu.
 #include <cuda.h>
 
-#include <algorithm>
 #include <cstdio>
 #include <cstring>
-#include <mutex>
 #include <new>
 
 #include "spdp_hostdev.h"
@@ -23,116 +21,6 @@ void note_cuda_error(cudaError_t e, const char* what) {
 }
 
 namespace {
-
-// What a handle owns comes from cudaMalloc, so that the arrays behind spdp_get_info can be reached by a peer and exported to
-// another process like any other.  cudaMalloc and cudaFree are slow (about 3 ms per packed and freed layer), so blocks of freed
-// handles are kept for the next ones, at most kKeptBlocks of them and kHandleKeep bytes per device; spdp_free(NULL), and an
-// allocation that finds no memory, give them back to the driver.  A block is put here only when nothing on the device uses it
-// any more, so the next owner may be any thread and any stream.
-// The partial sums of one spdp_spmm call come from a stream-ordered pool (calls on several streams or threads get memory of their
-// own), apart from the device's default pool, which gives its memory back at every synchronisation: 0.45 ms per call.
-// It keeps up to kScratchKeep bytes over a synchronisation, all given back when the device's last handle goes and by
-// spdp_free(NULL).
-constexpr int kMaxDevices = 64;
-constexpr uint64_t kHandleKeep = uint64_t(512) << 20;
-constexpr int kKeptBlocks = 64;
-constexpr uint64_t kScratchKeep = uint64_t(96) << 20;
-struct DeviceMemory {
-    DeviceBlock kept[kKeptBlocks];      // oldest first
-    int num_kept;
-    uint64_t bytes_kept;
-    cudaMemPool_t scratch_pool;
-    int64_t handles;
-};
-std::mutex g_memory_mu;
-DeviceMemory g_memory[kMaxDevices];
-
-// Takes block i out of the list (the lock is held).
-DeviceBlock take_kept(DeviceMemory& m, int i) {
-    const DeviceBlock b = m.kept[i];
-    for (int k = i + 1; k < m.num_kept; ++k) m.kept[k - 1] = m.kept[k];
-    --m.num_kept;
-    m.bytes_kept -= b.bytes;
-    return b;
-}
-
-// Gives every block that freed handles left on the device back to the driver.  Answers whether there was one.
-bool give_back_blocks(int device) {
-    bool any = false;
-    for (;;) {
-        DeviceBlock b = {};
-        {
-            std::lock_guard<std::mutex> lock(g_memory_mu);
-            DeviceMemory& m = g_memory[device];
-            if (m.num_kept > 0) b = take_kept(m, m.num_kept - 1);
-        }
-        if (b.p == nullptr) return any;
-        cudaFree(b.p);
-        any = true;
-    }
-}
-
-// A freed handle's block, for the next handle.  The caller has made sure that nothing on the device uses it any more.
-void keep_block(int device, DeviceBlock& block) {
-    const DeviceBlock b = block;
-    block = {};
-    if (b.p == nullptr) return;
-    if (b.bytes > kHandleKeep) { cudaFree(b.p); return; }
-    for (;;) {
-        DeviceBlock old = {};
-        {
-            std::lock_guard<std::mutex> lock(g_memory_mu);
-            DeviceMemory& m = g_memory[device];
-            if (m.num_kept < kKeptBlocks && m.bytes_kept + b.bytes <= kHandleKeep) {
-                m.kept[m.num_kept++] = b;
-                m.bytes_kept += b.bytes;
-                return;
-            }
-            old = take_kept(m, 0);
-        }
-        cudaFree(old.p);
-    }
-}
-
-// The stream-ordered pool of spdp_spmm's partial sums, made on first use.
-spdp_status scratch_pool_of(int device, cudaMemPool_t* out) {
-    if (device < 0 || device >= kMaxDevices) return SPDP_ERR_UNSUPPORTED_SHAPE;
-    std::lock_guard<std::mutex> lock(g_memory_mu);
-    cudaMemPool_t& pool = g_memory[device].scratch_pool;
-    if (pool == nullptr) {
-        cudaMemPoolProps props = {};
-        props.allocType = cudaMemAllocationTypePinned;
-        props.handleTypes = cudaMemHandleTypeNone;
-        props.location.type = cudaMemLocationTypeDevice;
-        props.location.id = device;
-        cudaMemPool_t made = nullptr;
-        SPDP_CUDA_TRY(cudaMemPoolCreate(&made, &props));
-        uint64_t keep = kScratchKeep;
-        const cudaError_t e = cudaMemPoolSetAttribute(made, cudaMemPoolAttrReleaseThreshold, &keep);
-        if (e != cudaSuccess) {
-            cudaMemPoolDestroy(made);
-            SPDP_CUDA_TRY(e);
-        }
-        pool = made;
-    }
-    *out = pool;
-    return SPDP_OK;
-}
-
-void trim_scratch(int device) {
-    std::lock_guard<std::mutex> lock(g_memory_mu);
-    if (g_memory[device].scratch_pool != nullptr) cudaMemPoolTrimTo(g_memory[device].scratch_pool, 0);
-}
-
-void count_handle(int device, int by) {
-    if (device < 0 || device >= kMaxDevices) return;
-    bool last;
-    {
-        std::lock_guard<std::mutex> lock(g_memory_mu);
-        last = (g_memory[device].handles += by) == 0;
-    }
-    if (last) trim_scratch(device);
-}
 
 // Makes `device` current for a scope.
 struct DeviceScope {
@@ -158,10 +46,7 @@ void release(spdp_matrix* h) {
         DeviceScope on(h->device);
         // the handle's memory may be in use on any stream (cudaFree would wait for them too)
         const bool idle = cudaDeviceSynchronize() == cudaSuccess;
-        for (DeviceBlock* b : {&h->arrays, &h->values_block, &h->workspace_block, &h->packing}) {
-            if (idle) keep_block(h->device, *b);
-            else cudaFree(b->p);
-        }
+        for (DeviceBlock* b : {&h->arrays, &h->values_block, &h->workspace_block, &h->packing}) handle_give(h->device, *b, idle);
         if (!idle) cudaGetLastError();
         cudaFree(h->probe_items);
         cudaFree(h->probe_count);
@@ -241,10 +126,10 @@ spdp_status build_partition(spdp_matrix* h, int num_ctas, cudaStream_t s) {
     if (st != SPDP_OK) return st;
     const cudaError_t e = cudaMemsetAsync(fresh.p, 0, bytes, s);
     if (e != cudaSuccess) {
-        keep_block(h->device, fresh);
+        handle_give(h->device, fresh, true);
         SPDP_CUDA_TRY(e);
     }
-    keep_block(h->device, h->workspace_block);      // idle: a new handle has none, spdp_set_num_ctas has waited for the device
+    handle_give(h->device, h->workspace_block, true);      // idle: a new handle has none, spdp_set_num_ctas has waited for the device
     h->workspace_block = fresh;
     h->workspace = static_cast<float*>(fresh.p);
     h->workspace_batch = h->workspace + P * kTileM;
@@ -271,7 +156,7 @@ spdp_status finish_handle(spdp_matrix* h, cudaStream_t s) {
     st = configure_spmspv_q4_kernel();
     if (st != SPDP_OK) return st;
     SPDP_CUDA_TRY(cudaStreamSynchronize(s));
-    keep_block(h->device, h->packing);
+    handle_give(h->device, h->packing, true);
     return SPDP_OK;
 }
 
@@ -284,51 +169,6 @@ spdp_status launch_decode(const spdp_matrix* h, const __half* x, int rule, float
 }
 
 bool rule_ok(int rule) { return rule == SPDP_DP_NONE || rule == SPDP_DP_ABS_GT || rule == SPDP_DP_MASK; }
-
-}  // namespace
-
-spdp_status scratch_alloc(int device, size_t bytes, cudaStream_t s, void** out) {
-    cudaMemPool_t pool = nullptr;
-    const spdp_status st = scratch_pool_of(device, &pool);
-    if (st != SPDP_OK) return st;
-    SPDP_CUDA_TRY(cudaMallocFromPoolAsync(out, bytes, pool, s));
-    return SPDP_OK;
-}
-
-// A block of 2 MB or more is a whole number of the driver's 2 MB pages anyway; a kept one serves where less than an eighth of it
-// (or 64 KB) would lie idle.
-spdp_status handle_alloc(int device, size_t bytes, DeviceBlock* out) {
-    if (device < 0 || device >= kMaxDevices) return SPDP_ERR_UNSUPPORTED_SHAPE;
-    const size_t unit = bytes >= (size_t(2) << 20) ? size_t(2) << 20 : 512;
-    bytes = (bytes + unit - 1) / unit * unit;
-    {
-        std::lock_guard<std::mutex> lock(g_memory_mu);
-        DeviceMemory& m = g_memory[device];
-        int best = -1;
-        for (int i = 0; i < m.num_kept; ++i)
-            if (m.kept[i].bytes >= bytes && m.kept[i].bytes - bytes <= std::max(bytes / 8, size_t(64) << 10) &&
-                (best < 0 || m.kept[i].bytes < m.kept[best].bytes))
-                best = i;
-        if (best >= 0) {
-            *out = take_kept(m, best);
-            return SPDP_OK;
-        }
-    }
-    void* p = nullptr;
-    cudaError_t e = cudaMalloc(&p, bytes);
-    if (e == cudaErrorMemoryAllocation && give_back_blocks(device)) {
-        cudaGetLastError();
-        e = cudaMalloc(&p, bytes);
-    }
-    SPDP_CUDA_TRY(e);
-    *out = {p, bytes};
-    return SPDP_OK;
-}
-
-}  // namespace spdp
-
-namespace spdp {
-namespace {
 
 // copy in -> kernel -> copy out, enqueued on s.
 spdp_status enqueue_host_call(spdp_matrix* h, const void* x_host, int rule, float thr, const void* mask_host,
@@ -696,10 +536,7 @@ spdp_status spdp_row_shard(int64_t M, int world, int rank, int64_t* first_row_ou
 
 spdp_status spdp_free(spdp_handle h) {
     if (h == nullptr) {                     // no handle: give back the memory that freed handles left
-        for (int d = 0; d < kMaxDevices; ++d) {
-            give_back_blocks(d);
-            trim_scratch(d);
-        }
+        give_back_all();
         return SPDP_OK;
     }
     if (!valid(h)) return SPDP_ERR_INVALID_ARG;

@@ -4,8 +4,8 @@
 // Values are one contiguous span, which moves in 16-byte pieces.  (With one CTA per GTile a row of the dense side was 32
 // bytes and the values were scattered in runs of 2-byte stores.)  11008x4096 at 60 % sparsity: count 27, scan 8, emit 44,
 // unpack 45 us; between the block's loads and its stores a CTA has one serial pass over its 64 columns, which is what is
-// left.  Pack, unpack and free together took 3487 us, 3 ms of it cudaMalloc and cudaFree, and take 175 us (memory of freed handles is
-// kept, see api.cu).
+// left.  Pack, unpack and free together took 3487 us, 3 ms of it cudaMalloc and cudaFree, and take 176 us (memory of freed handles is
+// kept, see memory.cu).
 #include <mutex>
 
 #include "spdp_internal.h"

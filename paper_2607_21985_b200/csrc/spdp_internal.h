@@ -14,10 +14,12 @@ constexpr int kTileK = 16;         // column tiles per GTile (Sec. 4.2.3)
 constexpr int kWordsPerCol = 4;    // 64-bit bitmap words per column tile (Sec. 4.1)
 constexpr uint64_t kMagic = 0x5350445042323030ull;   // "SPDPB200"
 
-// A piece of device memory from cudaMalloc that a handle owns (see handle_alloc).
+// A piece of device memory that a handle owns (memory.cu).
+struct Slab;
 struct DeviceBlock {
     void* p;
     size_t bytes;
+    Slab* slab;     // the slab it is part of, or null: an allocation of its own
 };
 
 }  // namespace spdp
@@ -100,10 +102,17 @@ void note_cuda_error(cudaError_t e, const char* what);
 
 inline bool valid(const spdp_matrix* h) { return h != nullptr && h->magic == kMagic; }
 
-// api.cu: stream-ordered scratch memory for one call (given back with cudaFreeAsync on the same stream).
-spdp_status scratch_alloc(int device, size_t bytes, cudaStream_t s, void** out);
-// api.cu: memory that a handle owns, usable on any stream; release() keeps it for the next handle.
+// memory.cu
+// Memory that a handle owns, usable on any stream, on the current device (`device`).
 spdp_status handle_alloc(int device, size_t bytes, DeviceBlock* out);
+// Takes it back for the next handle and empties `block`.  `idle`: nothing on the device uses it any more; else it is not used again.
+void handle_give(int device, DeviceBlock& block, bool idle);
+// A handle came (+1) or went (-1).
+void count_handle(int device, int by);
+// Everything that is kept and not in use goes back to the driver, on every device.
+void give_back_all();
+// Stream-ordered scratch memory for one call (given back with cudaFreeAsync on the same stream).
+spdp_status scratch_alloc(int device, size_t bytes, cudaStream_t s, void** out);
 
 // pack.cu
 spdp_status configure_pack_kernels();          // per-device kernel attributes; idempotent
