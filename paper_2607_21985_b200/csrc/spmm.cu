@@ -1027,9 +1027,6 @@ Plan make_plan(int64_t R, int64_t nkb, int64_t N, int sms, bool may_cut) {
     Plan best = {};
     best.us = -1.0;
     for (int f = 0; f < 4; ++f) {
-#ifdef SPDP_SPMM_FORCE
-        if (f != SPDP_SPMM_FORCE) continue;
-#endif
         Plan q = {};
         q.kernel = f;
         q.tiles = R * ((N + kTokens[f] - 1) / kTokens[f]);

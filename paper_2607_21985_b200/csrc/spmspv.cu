@@ -21,9 +21,6 @@ namespace {
 
 using namespace dev;
 
-#ifndef SPDP_FMA_MODE
-#define SPDP_FMA_MODE 0      // 0: mixed-precision fma.rn.f32.f16, 1: cvt + fp32 fma
-#endif
 #ifndef SPDP_WARPS
 #define SPDP_WARPS 24
 #endif
@@ -33,11 +30,8 @@ using namespace dev;
 #ifndef SPDP_CHUNK_COLS
 #define SPDP_CHUNK_COLS 8192
 #endif
-#ifndef SPDP_DEPTH
-#define SPDP_DEPTH 2
-#endif
 constexpr int kWarps = SPDP_WARPS;         // warps per CTA; every warp fetches and decodes its own column tiles
-constexpr int kDepth = SPDP_DEPTH;         // groups a warp keeps in flight
+constexpr int kDepth = 2;         // groups a warp keeps in flight (the ring positions alternate)
 constexpr int kGroup = 4;                  // active column tiles per group (one fetch / decode unit of a warp)
 constexpr int kSlotBytes = 2 * kTileM + 32;  // a column tile's values (at most 256 fp16) + 32 bytes so that the
                                              // four tiles of a group start 8 banks apart
@@ -119,18 +113,9 @@ __device__ __forceinline__ bool column_active(int rule, float thr, const uint32_
 // bit takes the next value and adds value * x to its row's fp32 accumulator.  (A multiplication in place of the mask, as in
 // the batch and 4-bit kernels, costs 1 %: here the FMA pipe has the products to do.)  fma.rn.f32.f16
 // multiplies two fp16 exactly and accumulates in fp32.  x32 holds two activations; kUpper picks one.
-#if SPDP_FMA_MODE == 0
 #define SPDP_FMA2(X)                                  \
     " @p0 fma.rn.f32.f16 %0, v0, " X ", %0;\n"        \
     " @p1 fma.rn.f32.f16 %1, v1, " X ", %1;\n"
-#else
-#define SPDP_FMA2(X)                                  \
-    " .reg .f32 f0, f1, fx;\n"                        \
-    " cvt.f32.f16 fx, " X ";\n"                       \
-    " @p0 cvt.f32.f16 f0, v0;\n @p1 cvt.f32.f16 f1, v1;\n" \
-    " @p0 fma.rn.f32 %0, f0, fx, %0;\n"               \
-    " @p1 fma.rn.f32 %1, f1, fx, %1;\n"
-#endif
 #define SPDP_DECODE_BODY(X)                           \
     "{\n"                                             \
     " .reg .pred p0, p1;\n"                           \
@@ -421,13 +406,8 @@ spmspv_kernel(const Params p) {
             fetch_group(rec_nxt, dv, db);  // refill it with the group kDepth ahead (null records past the end)
             rec_nxt += 8u * kGroup * kWarps;
             lq += kWarps;
-            if (kDepth == 2) {
-                dv ^= kStageBytes;
-                db ^= 128u;
-            } else {
-                dv = (dv == (kDepth - 1) * kStageBytes) ? 0u : dv + kStageBytes;
-                db = (db == (kDepth - 1) * 128u) ? 0u : db + 128u;
-            }
+            dv ^= kStageBytes;             // the other of the two ring positions
+            db ^= 128u;
         };
         auto park_first = [&]() {      // my share of the first piece is complete: park it, restart from zero
 #pragma unroll

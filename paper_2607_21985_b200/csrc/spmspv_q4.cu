@@ -33,11 +33,8 @@ using namespace dev;
 #ifndef SPDP_Q4_CHUNK_COLS
 #define SPDP_Q4_CHUNK_COLS 8192
 #endif
-#ifndef SPDP_Q4_DEPTH
-#define SPDP_Q4_DEPTH 2
-#endif
 constexpr int kWarps = SPDP_Q4_WARPS;         // warps per CTA; every warp fetches and decodes its own column tiles
-constexpr int kDepth = SPDP_Q4_DEPTH;         // groups a warp keeps in flight
+constexpr int kDepth = 2;         // groups a warp keeps in flight (the ring positions alternate)
 constexpr int kGroup = 4;                  // active column tiles per group (one fetch / decode unit of a warp)
 constexpr int kSlotPad = 16;                 // bytes in front of a slot's codes: the decode reads the two 32-bit words that
                                              // END at a lane's last code, the first of which may lie before the codes
@@ -168,12 +165,12 @@ __device__ __forceinline__ void finish_row_tile(const Params& p, int r, Segments
 //       (ballots + prefix sums place them), one record per active
 //       column tile -- Sec. 4.2 steps (1)-(3);
 //   (2) each warp takes groups of kGroup active column tiles round-robin.  It keeps kDepth
-//       groups in flight: the padded values of a column tile arrive with 16-byte asynchronous
+//       groups in flight: the padded codes of a column tile arrive with 16-byte asynchronous
 //       copies (lane = one 16-byte piece of one of the group's tiles), its 8 bitmap words with
-//       4-byte ones; inactive columns are never touched.  Decode (Sec. 4.2.1): lane owns 2
-//       consecutive rows of every second bitmap word, rank = set bits before them, values read from
-//       shared memory, fp32 accumulation in registers.  Where the first piece's groups end the
-//       warp parks its sums in shared memory and starts the second piece from zero;
+//       4-byte ones; inactive columns are never touched.  Decode (Sec. 4.2.1): a lane owns 8
+//       consecutive rows, one byte of the bitmap; rank = set bits before them; its codes are one span of at most 8 nibbles in
+//       shared memory, walked from the last row to the first; fp32 accumulation in registers.  Where the
+//       first piece's groups end the warp parks its sums in shared memory and starts the second piece from zero;
 //   (3) batch end: cross-warp row reduction, split-K combine and store of every row tile that
 //       the batch completed (two groups of 256 threads work side by side).
 __global__ void __launch_bounds__(kThreads, kCtasPerSm)
@@ -390,13 +387,8 @@ spmspv_q4_kernel(const Params p) {
             fetch_group(rec_nxt, dv, db);  // refill it with the group kDepth ahead (null records past the end)
             rec_nxt += 8u * kGroup * kWarps;
             lq += kWarps;
-            if (kDepth == 2) {
-                dv ^= kStageBytes;
-                db ^= 128u;
-            } else {
-                dv = (dv == (kDepth - 1) * kStageBytes) ? 0u : dv + kStageBytes;
-                db = (db == (kDepth - 1) * 128u) ? 0u : db + 128u;
-            }
+            dv ^= kStageBytes;             // the other of the two ring positions
+            db ^= 128u;
         };
         auto park_first = [&]() {      // my share of the first piece is complete: park it, restart from zero
 #pragma unroll
