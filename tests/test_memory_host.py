@@ -17,9 +17,9 @@ class Block(ctypes.Structure):
 
 @pytest.fixture()
 def M(tmp_path):
-    out = tmp_path / "libmemory_shim.so"
+    out = tmp_path / "libmemory_shim.so"          # -Bsymbolic: its own cudaMalloc, also where torch has loaded the real one
     cuda = os.environ.get("CUDA_HOME", "/usr/local/cuda")
-    subprocess.run(["g++", "-std=c++17", "-O1", "-shared", "-fPIC", "-I", os.path.join(cuda, "include"), "-I", os.path.join(ROOT, "include"),
+    subprocess.run(["g++", "-std=c++17", "-O1", "-shared", "-fPIC", "-Wl,-Bsymbolic", "-I", os.path.join(cuda, "include"), "-I", os.path.join(ROOT, "include"),
                     "-I", os.path.join(ROOT, "paper_2607_21985_b200", "csrc"), "-o", str(out), os.path.join(ROOT, "tests", "memory_shim.cpp")], check=True)
     L = ctypes.CDLL(str(out))
     L.shim_limit.argtypes = [ctypes.c_ulonglong]
