@@ -91,7 +91,7 @@ typedef struct {
  *   ldw       leading dimension in elements, >= K.
  *   tile_m, tile_k  must be 256 and 16 (the format's constants), else SPDP_ERR_UNSUPPORTED_SHAPE.
  *   out       receives the handle.  The call allocates device memory, runs on `stream` and
- *             synchronises it once (packing is an offline step).  W_dev is not retained.
+ *             synchronises it twice (packing is an offline step).  W_dev is not retained.
  * GTile (r, c) has linear index r*C + c; its 16 ColInfo words and 64 bitmap words are
  * contiguous; Values holds, per GTile and per column, the column's nonzeros in row order
  * followed by 0x0000 padding up to a multiple of 8 elements. */
@@ -180,15 +180,21 @@ SPDP_API spdp_status spdp_spmspv_batch(spdp_handle h, const void* x_dev, int64_t
  *           encoded on the host at every call), else SPDP_ERR_INVALID_ARG.
  *   N       >= 1 tokens.
  *   Y_dev   [N][ldy] of ydt, device, ldy >= M elements between tokens; all N*M entries are written.
- * Asynchronous on `stream`.  Usually one kernel and no allocation.  When the last round of CTAs would
- * leave more than half of the SMs idle, the tiles of that round are cut along K instead: a second launch
- * leaves fp32 partial sums in scratch memory taken from the device's stream-ordered pool (cudaMallocAsync /
- * cudaFreeAsync on `stream`, 0.5 MB per slice) and a third adds the slices in a fixed order.  The handle's
- * workspace is never touched, so calls on one handle may overlap.  The waits inside the kernel (on
- * shared-memory barriers that the copies and the tensor cores complete) are bounded; one that runs
- * out records SPDP_ERR_TIMEOUT in the handle's status word and the CTA leaves its outputs unwritten;
- * TileOffset words that do not describe a K-block that fits shared memory record SPDP_ERR_OVERFLOW
- * the same way.  SPDP_ERR_CUDA if the driver's tensor-map encoder cannot be found. */
+ * Asynchronous on `stream`; one to three kernels.  A tile of the result (256 rows x 32 to 512 tokens) is one CTA's
+ * work, or a pair's.  Where whole tiles would leave SMs idle, which is the rule for short prompts and small
+ * layers, the tiles that do not fill a round (often all of them) are cut along K: several CTAs leave fp32 partial
+ * sums of a tile in scratch memory and a further kernel adds them in a fixed order.  Which tiles are
+ * cut follows from M, K, N and the number of SMs alone, so repeated calls give identical bits.
+ *   The scratch memory, up to 77 MB on 148 SMs, comes from a stream-ordered pool of the library's (cudaMallocFromPoolAsync /
+ * cudaFreeAsync on `stream`; in a stream capture it becomes memory of the graph).  The pool keeps up to 96 MB until the
+ * device's last handle is freed; spdp_free(NULL) gives back what is unused.  Where there is no memory for it the call
+ * cuts nothing: slower, and the sums in another order.
+ *   The handle's workspace is never touched, so calls on one handle may overlap.
+ *   The waits inside the kernels (on shared-memory barriers that the copies and the tensor cores complete) are
+ * bounded.  One that runs out records SPDP_ERR_TIMEOUT in the handle's status word, and the rows and tokens that the CTA
+ * would have written, or left partial sums of, stay unwritten; TileOffset words that do not describe a K-block that fits
+ * shared memory record SPDP_ERR_OVERFLOW the same way.  A status other than 0 therefore means that Y is incomplete.
+ * SPDP_ERR_CUDA if the driver's tensor-map encoder cannot be found. */
 SPDP_API spdp_status spdp_spmm(spdp_handle h, const void* X_dev, int64_t N, int64_t ldx, void* Y_dev, int64_t ldy,
                       spdp_ydtype ydt, void* stream);
 
@@ -293,9 +299,10 @@ SPDP_API spdp_status spdp_probe_gather(spdp_handle h, const void* x_dev, spdp_dp
  * Synchronises the device. */
 SPDP_API spdp_status spdp_last_device_status(spdp_handle h, int* out);
 
-/* Tuning knob: number of CTAs spdp_spmspv launches (0 = default, one per SM; at most 1024 and at
- * most one per GTile are used).  Takes effect on
- * the next call; re-derives the handle's split-K workspace layout (may reallocate it). */
+/* Tuning knob: number of CTAs spdp_spmspv launches (0 = default: one per SM, fewer on small
+ * layers; at most 1024 and at most one per GTile are used).  Takes effect on
+ * the next call; re-derives the handle's split-K workspace.  Waits for the device.  Where there is no memory for the new
+ * workspace (SPDP_ERR_ALLOC) the handle stays as it was. */
 SPDP_API spdp_status spdp_set_num_ctas(spdp_handle h, int num_ctas);
 
 /* Text of the last CUDA runtime error seen by the library on this thread ("" if none). */

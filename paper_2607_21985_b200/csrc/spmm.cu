@@ -1012,8 +1012,8 @@ struct Plan {
 };
 // The estimate of a call's time: (K-blocks of the busiest CTA) x (time of a K-block) + a tile's start and end + what the
 // partial sums cost.  Fitted to the four kernels' times, calls in a row on a stream, on 10 layers from 512x512 to 28672x8192
-// (30 to 80 % sparse) with 16 to 1024 tokens each: the choice costs 1 % on average against the best that was measured, 17 % at
-// worst.  (Fitted to graph replays, where the CTA pairs' plain launch costs nothing, it took pairs for small layers, and cuts that
+// (30 to 80 % sparse) with 16 to 1024 tokens each.  Measured again over those 80 calls, the form that is chosen is 0.6 % behind the best form on
+// average, 8 % at worst (512x512 x 16 tokens, 8.3 against 7.6 us).  (Fitted to graph replays, where the CTA pairs' plain launch costs nothing, it took pairs for small layers, and cuts that
 // cross tiles as readily as those that do not: 1024x1024 x 32 tokens 14.4 -> 8.3 us, 2048x2048 x 64 16.5 -> 12.8, 4096x4096 x
 // 128 22.9 -> 19.6, x 16 17.7 -> 14.8, 4096x11008 x 128 34.0 -> 31.4, 4001x4098 x 200 30.8 -> 26.3.)
 constexpr double kCallUs[4] = {3.0, 3.7, 3.2, 6.5};                     // a call's fixed part; the pairs' launch waits for the kernel before

@@ -348,7 +348,8 @@ spmspv_kernel(const Params p) {
                 const int rem = static_cast<int>(rc.y & 63u) - lane7;                  // my 16-byte pieces left
                 const unsigned char* src = offset_wide<2>(val_src, rc.x);
                 const uint32_t dst = val_dst + dv_f;
-                // the bitmap first: the scan waits for it alone (28672x8192 44.6 -> 44.0 us, 28672x4096 at 30 % 40.0 -> 39.0)
+                // the bitmap first: the scan waits for it alone (28672x8192 in a graph 45.2 -> 44.6 us, in a row 45.7 ->
+                // 45.1; 28672x4096 at 30 % 27.5 -> 27.1)
                 cp_async4(bdst, offset_wide<32>(bm_src, rc.y >> 6));
                 cp_async16<0>(dst, src, rem);
                 cp_async16<128>(dst, src, rem);

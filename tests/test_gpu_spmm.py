@@ -84,10 +84,10 @@ def test_spmm_exact_on_integers_and_strided_tensors(S):
 @pytest.mark.parametrize("R,K,N", [(80, 200, 1), (80, 200, 256), (80, 72, 300), (40, 136, 600), (30, 264, 700), (3, 520, 1100),
                                    (76, 264, 100), (150, 520, 300), (75, 2048, 700)])
 def test_spmm_both_kernels(S, R, K, N):
-    """The launch chooses between a CTA per row tile (256 tokens) and a CTA pair per row tile (512 tokens) by the
-    rounds of CTAs each needs: many row tiles with few tokens take the first, the rest the second.  These shapes
-    reach both, with one and with several token blocks, ragged in M, K and N.  The last three leave a last round of
-    two CTA pairs on a 148-SM GPU: those tiles are cut along K and their slices added by a second kernel."""
+    """The launch chooses among CTAs of 32, 128 and 256 tokens and CTA pairs of 512 by an estimate of each one's time.  On
+    148 SMs these shapes reach all four, with one and with several token blocks, ragged in M, K and N, without a cut in the
+    one-CTA forms.  The last two take pairs and leave a last round of two: those tiles are cut along K and their slices added by
+    a second kernel.  (Cut tiles of the one-CTA forms: test_spmm_work_cuts.)"""
     rw, rx = WL._rngs(100 + R)
     M = 256 * R - 37
     W = WL.prune_global_magnitude(WL.normal_weights(rw, M, K), 0.5).astype(np.float16)
@@ -120,12 +120,14 @@ def test_spmm_rejects_bad_arguments(S):
 
 
 @pytest.mark.parametrize("R,K,N", [(150, 520, 20), (149, 1000, 30), (5, 5000, 40), (3, 640, 33), (1, 12800, 128), (1, 130, 256),
-                                   (7, 3000, 129), (2, 20000, 1), (37, 64, 513), (2, 65, 31)])
+                                   (7, 3000, 129), (2, 20000, 1), (37, 64, 513), (2, 65, 31),
+                                   (50, 1280, 20), (50, 1280, 60), (50, 2000, 200), (250, 1280, 20)])
 @pytest.mark.parametrize("sp", [0.0, 0.5, 0.95])
 def test_spmm_work_cuts(S, R, K, N, sp):
-    """How the work is cut over CTAs: whole rounds plus a shared rest (150 and 149 row tiles), CTA ranges that start in one
-    row tile and end in the next (5, 7), many CTAs on one row tile (1, 2), K-blocks of one column, full columns
-    (the ring of stored values at its fullest) and nearly empty ones.  Integers: every partial sum is exact."""
+    """How the work is cut over CTAs: whole rounds plus a shared rest (150, 149 and 250 row tiles), CTA ranges that start in one
+    row tile and end in the next (50 and 250 row tiles on 148 SMs, with 32, 128 and 256 tokens per CTA), a whole number of CTAs per
+    row tile (5, 7), many on one (1, 2), K-blocks of one column, full columns (the ring of stored values at its fullest)
+    and nearly empty ones.  Integers: every partial sum is exact."""
     rng = np.random.Generator(np.random.PCG64(R * 1000 + K))
     M = 256 * R - 3
     W = rng.integers(-4, 5, (M, K)).astype(np.float16)
