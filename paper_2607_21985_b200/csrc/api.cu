@@ -145,8 +145,6 @@ spdp_status build_partition(spdp_matrix* h, int num_ctas, cudaStream_t s) {
 spdp_status finish_handle(spdp_matrix* h, cudaStream_t s) {
     spdp_status st = build_partition(h, 0, s);
     if (st != SPDP_OK) return st;
-    st = configure_pack_kernels();
-    if (st != SPDP_OK) return st;
     st = configure_spmspv_kernel();
     if (st != SPDP_OK) return st;
     st = configure_spmspv_batch_kernel();

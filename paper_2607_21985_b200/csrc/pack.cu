@@ -1,14 +1,15 @@
 // Tiled-CBC packer and unpacker kernels (Sec. 4.1 "Storage Structure", Sec. 4.2.1 decode rule,
 // Sec. 4.2.3 padding).  Three passes: count -> scan -> emit.  A CTA of the count, emit and unpack kernels handles one row
-// tile x 64 columns (4 GTiles): the dense side moves through shared memory in whole 128-byte rows, and the 4 GTiles'
-// Values are one contiguous span, which moves in 16-byte pieces.  (With one CTA per GTile a row of the dense side was 32
-// bytes and the values were scattered in runs of 2-byte stores.)  11008x4096 at 60 % sparsity: count 27, scan 8, emit 44,
-// unpack 45 us; between the block's loads and its stores a CTA has one serial pass over its 64 columns, which is what is
-// left.  Pack, unpack and free together took 3487 us, 3 ms of it cudaMalloc and cudaFree, and take 176 us (memory of freed handles is
-// kept, see memory.cu).
-#include <mutex>
-
+// tile x 64 columns (4 GTiles); a warp has 32 of its rows and a lane two neighbouring columns, so that the dense side moves in whole
+// 128-byte lines between memory and registers, and a lane walks down its columns with a running place in the values: no
+// rank, no popcount and no staging of the block.  The 4 GTiles' Values are one contiguous span, which passes through shared memory
+// and moves in 16-byte pieces.  (With the block in shared memory and a lane per row, a ballot or a popcount per row and column,
+// the three took 5300, 8000 and 8500 warp instructions per block, twice to three times what they take now.)
+// 11008x4096 at 60 % sparsity, each kernel alone with cold caches: count 28.9 -> 21.6 us, scan 9.3 -> 6.4, emit 45.4 -> 32.4, unpack
+// 46.2 -> 27.6; the bytes alone would take 14, 0, 20 and 20.  Pack, unpack and free together 173 -> 133 us (memory of freed
+// handles is kept, see memory.cu), the rest of it synchronisations.
 #include "spdp_internal.h"
+#include "spmspv_device.cuh"
 
 namespace spdp {
 namespace {
@@ -39,86 +40,63 @@ __device__ __forceinline__ void load_tile_row(const unsigned short* __restrict__
     }
 }
 
-constexpr int kCols = 64;                       // columns a CTA handles: one 128-byte line of a row (32: the same time)
+constexpr int kCols = 64;                       // columns a CTA handles: one 128-byte line of a row (a lane has two of them)
 constexpr int kGT = kCols / kTileK;
-constexpr int kPieces = kCols / 8;              // 16-byte pieces of a row
-constexpr int kRowWords = kCols / 2 + 1;        // 32-bit words per row in shared memory: an odd stride, so that neither the rows
-                                                // of a column pair nor the 16-byte pieces of a row meet in a bank
+constexpr int kWords = kTileM / 32;             // 32-bit bitmap words of a column tile; warp w has the rows of word w
+static_assert(kTileM == 32 * kWords && kCols == 64, "a warp per bitmap word, a lane per pair of columns");
 
-struct PackSmem {
-    uint32_t tile[kTileM * kRowWords];          // the dense 256 x 64 block
-    alignas(16) unsigned short vals[kCols * kTileM + 8];     // its values as stored
-    uint2 words[kCols / 2][kTileM / 32][2];     // per pair of columns and 32 rows, for each of the two: the bitmap word and the
-                                                // index in vals of its first value (a lane reads all four with one load)
-};
-struct CountSmem {
-    uint32_t tile[kTileM * kRowWords];
-    uint32_t words[kCols][kTileM / 32];
-};
-
-// The dense block at (row0, col0) -> shared memory, zero beyond the matrix edge.
-__device__ __forceinline__ void load_block(const unsigned short* __restrict__ W, int64_t ldw, int64_t M, int64_t K,
-                                           int64_t row0, int64_t col0, uint32_t* tile) {
-    const bool wide = ((reinterpret_cast<uintptr_t>(W) | static_cast<uintptr_t>(2 * ldw)) & 15u) == 0;
-    uint4 v[kCols / 8];
+// Elements (row + i, col) and (row + i, col + 1) of the dense matrix, i < kRows, as one word each; zero beyond the edge.  With
+// col = 64 * b + 2 * lane a warp reads whole 128-byte lines.
+template <int kRows>
+__device__ __forceinline__ void load_rows(const unsigned short* __restrict__ W, int64_t ldw, int64_t M, int64_t K, int64_t row, int64_t col,
+                                          uint32_t (&v)[kRows]) {
+    const unsigned short* src = W + row * ldw + col;
+    if (((reinterpret_cast<uintptr_t>(W) | static_cast<uintptr_t>(2 * ldw)) & 3u) == 0 && col + 1 < K) {
 #pragma unroll
-    for (int i = 0; i < kCols / 8; ++i) {
-        const int q = threadIdx.x + kTileM * i, row = q / kPieces, c = (q % kPieces) * 8;
-        const int64_t r = row0 + row, col = col0 + c;
-        const unsigned short* src = W + r * ldw + col;
-        v[i] = make_uint4(0u, 0u, 0u, 0u);
-        if (r < M && col < K) {
-            if (wide && col + 8 <= K) {
-                v[i] = __ldg(reinterpret_cast<const uint4*>(src));
-            } else {
-                unsigned w[4] = {0u, 0u, 0u, 0u};
+        for (int i = 0; i < kRows; ++i) v[i] = row + i < M ? __ldg(reinterpret_cast<const uint32_t*>(src + i * ldw)) : 0u;
+    } else {
 #pragma unroll
-                for (int e = 0; e < 8; ++e)
-                    if (col + e < K) w[e >> 1] |= static_cast<unsigned>(__ldg(src + e)) << (16 * (e & 1));
-                v[i] = make_uint4(w[0], w[1], w[2], w[3]);
-            }
+        for (int i = 0; i < kRows; ++i) {
+            v[i] = row + i < M && col < K ? __ldg(src + i * ldw) : 0u;
+            if (row + i < M && col + 1 < K) v[i] |= static_cast<uint32_t>(__ldg(src + i * ldw + 1)) << 16;
         }
     }
-#pragma unroll
-    for (int i = 0; i < kCols / 8; ++i) {
-        const int q = threadIdx.x + kTileM * i;
-        uint32_t* dst = tile + (q / kPieces) * kRowWords + (q % kPieces) * 4;
-        dst[0] = v[i].x;
-        dst[1] = v[i].y;
-        dst[2] = v[i].z;
-        dst[3] = v[i].w;
-    }
+}
+// 0xFFFF in each half that holds an element to be stored: anything but +-0 (NaN compares unordered, which counts).
+__device__ __forceinline__ uint32_t stored_halves(uint32_t v) {
+    uint32_t r;
+    asm("set.neu.u32.f16x2 %0, %1, %2;" : "=r"(r) : "r"(v), "r"(0u));
+    return r;
 }
 
-// Pass 1: bitmap words, per-column nonzero counts, ColInfo, padded length of each GTile.
+// Pass 1: bitmap words, per-column nonzero counts, ColInfo, padded length of each GTile.  A lane collects the bits of its two
+// columns over the 32 rows of its warp, one comparison and one logic operation for two elements; nothing is staged and
+// nothing is exchanged until the words are there.
 __global__ void __launch_bounds__(kTileM)
 pack_count_kernel(const unsigned short* __restrict__ W, int64_t ldw, int64_t M, int64_t K, int64_t C, int blocks,
                   int pad_elems, uint64_t* __restrict__ bitmap, uint32_t* __restrict__ colinfo,
                   uint32_t* __restrict__ tile_len, unsigned long long* __restrict__ nnz_total) {
-    __shared__ CountSmem sm;
+    __shared__ uint32_t words[kCols][kWords + 1];
     const int64_t r = blockIdx.x / static_cast<unsigned>(blocks), cb = blockIdx.x % static_cast<unsigned>(blocks);
     const int64_t g0 = r * C + cb * kGT;
     const int ngt = static_cast<int>(min(static_cast<int64_t>(kGT), C - cb * kGT));
     const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
-    load_block(W, ldw, M, K, r * kTileM, cb * kCols, sm.tile);
-    __syncthreads();
-    const uint32_t* mine = sm.tile + t * kRowWords;
-#pragma unroll 8
-    for (int c = 0; c < kCols / 2; ++c) {
-        const uint32_t v = mine[c];
-        const unsigned b0 = __ballot_sync(0xFFFFFFFFu, (v & 0x7FFFu) != 0), b1 = __ballot_sync(0xFFFFFFFFu, (v & 0x7FFF0000u) != 0);
-        if (lane == 0) {
-            sm.words[2 * c][warp] = b0;
-            sm.words[2 * c + 1][warp] = b1;
-        }
+    uint32_t v[32], low = 0u, high = 0u;                    // rows 0-15 and 16-31: first column's bits below, second's above
+    load_rows<32>(W, ldw, M, K, r * kTileM + 32 * warp, cb * kCols + 2 * lane, v);
+#pragma unroll
+    for (int i = 0; i < 16; ++i) {
+        low |= stored_halves(v[i]) & (0x00010001u << i);
+        high |= stored_halves(v[16 + i]) & (0x00010001u << i);
     }
+    words[2 * lane][warp] = __byte_perm(low, high, 0x5410);
+    words[2 * lane + 1][warp] = __byte_perm(low, high, 0x7632);
     __syncthreads();
     uint32_t* out = reinterpret_cast<uint32_t*>(bitmap + g0 * kTileK * kWordsPerCol);
-    for (int i = t; i < ngt * kTileK * (kTileM / 32); i += kTileM) out[i] = (&sm.words[0][0])[i];
+    for (int i = t; i < ngt * kTileK * kWords; i += kTileM) out[i] = words[i / kWords][i % kWords];
     if (t < kCols) {                                        // one thread per column; 16 neighbouring lanes are a GTile
         unsigned n = 0;
 #pragma unroll
-        for (int w = 0; w < kTileM / 32; ++w) n += __popc(sm.words[t][w]);
+        for (int w = 0; w < kWords; ++w) n += __popc(words[t][w]);
         const unsigned padded = (n + pad_elems - 1) / pad_elems * pad_elems;
         unsigned end = padded;
 #pragma unroll
@@ -136,36 +114,53 @@ pack_count_kernel(const unsigned short* __restrict__ W, int64_t ldw, int64_t M, 
 }
 
 // Pass 2: exclusive scan of the padded GTile lengths into TileOffset (one CTA; a warp takes one contiguous part, its lanes
-// neighbouring entries).  total_out receives the 64-bit total.
+// 4 neighbouring entries at a time).  total_out receives the 64-bit total.
 __global__ void __launch_bounds__(1024)
 pack_scan_kernel(const uint32_t* __restrict__ tile_len, int64_t NGT, uint32_t* __restrict__ tileoffset,
                  unsigned long long* __restrict__ total_out) {
     __shared__ unsigned long long part[32];
     const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
-    const int64_t per = (NGT + 1023) / 1024 * 32;
-    const int64_t lo = min(NGT, warp * per), hi = min(NGT, lo + per);
+    const int64_t per = (NGT + 4095) / 4096 * 128, lo = min(NGT, warp * per), hi = min(NGT, lo + per);
+    auto lengths = [&](int64_t i) {                         // entries i .. i + 3 (i a multiple of 4), zero from hi on
+        if (i + 4 <= hi) return *reinterpret_cast<const uint4*>(tile_len + i);
+        return make_uint4(i < hi ? tile_len[i] : 0u, i + 1 < hi ? tile_len[i + 1] : 0u, i + 2 < hi ? tile_len[i + 2] : 0u, 0u);
+    };
     unsigned long long s = 0;
 #pragma unroll 4
-    for (int64_t i = lo + lane; i < hi; i += 32) s += tile_len[i];
+    for (int64_t i = lo + 4 * lane; i < hi; i += 128) {
+        const uint4 v = lengths(i);
+        s += static_cast<unsigned long long>(v.x + v.y) + (v.z + v.w);
+    }
     for (int d = 16; d > 0; d >>= 1) s += __shfl_xor_sync(0xFFFFFFFFu, s, d);
     if (lane == 0) part[warp] = s;
     __syncthreads();
     unsigned long long run = 0, total = 0;
+#pragma unroll
     for (int w = 0; w < 32; ++w) {
-        if (w < warp) run += part[w];
-        total += part[w];
+        const unsigned long long v = part[w];
+        if (w < warp) run += v;
+        total += v;
     }
-#pragma unroll 4
-    for (int64_t b = lo; b < hi; b += 32) {
-        const int64_t i = b + lane;
-        const uint32_t len = i < hi ? tile_len[i] : 0u;
-        uint32_t inc = len;                                 // 32 lengths of at most 256 * 256 stay below 2^32
+#pragma unroll 2
+    for (int64_t b = lo; b < hi; b += 128) {
+        const int64_t i = b + 4 * lane;
+        const uint4 v = lengths(i);
+        const uint32_t sum = v.x + v.y + v.z + v.w;         // 128 lengths of at most 16 * 256 stay below 2^32
+        uint32_t inc = sum;
 #pragma unroll
         for (int d = 1; d < 32; d <<= 1) {
             const uint32_t u = __shfl_up_sync(0xFFFFFFFFu, inc, d);
             if (lane >= d) inc += u;
         }
-        if (i < hi) tileoffset[i] = static_cast<uint32_t>(run + inc - len);
+        const uint32_t at = static_cast<uint32_t>(run) + inc - sum;
+        const uint4 o = make_uint4(at, at + v.x, at + v.x + v.y, at + v.x + v.y + v.z);
+        if (i + 4 <= hi) {
+            *reinterpret_cast<uint4*>(tileoffset + i) = o;
+        } else {
+            if (i < hi) tileoffset[i] = o.x;
+            if (i + 1 < hi) tileoffset[i + 1] = o.y;
+            if (i + 2 < hi) tileoffset[i + 2] = o.z;
+        }
         run += __shfl_sync(0xFFFFFFFFu, inc, 31);
     }
     if (t == 0) {
@@ -174,16 +169,24 @@ pack_scan_kernel(const uint32_t* __restrict__ tile_len, int64_t NGT, uint32_t* _
     }
 }
 
+// What the emit and unpack kernels keep in shared memory: the block's values as stored, and per bitmap word and column the
+// word and the index in vals of its first value.
+struct BlockSmem {
+    alignas(16) unsigned short vals[kCols * kTileM + 8];
+    alignas(16) uint2 words[kWords][kCols + 2];             // (a lane reads its two columns with one load)
+};
+static_assert(sizeof(uint2) * (kCols + 2) % 16 == 0, "pairs of columns on 16-byte boundaries");
+
 // Bitmap words of the CTA's columns and the index in sm.vals of each word's first value (ColInfo offsets, set bits of the
 // words before) -> sm.words.  Lane (q, w) = (t / 8, t % 8) of a pass takes word w of column q.  Returns the number of values
 // of the span, padding included.
-__device__ __forceinline__ uint32_t load_words(PackSmem& sm, const uint32_t* __restrict__ tileoffset, const uint32_t* __restrict__ colinfo,
+__device__ __forceinline__ uint32_t load_words(BlockSmem& sm, const uint32_t* __restrict__ tileoffset, const uint32_t* __restrict__ colinfo,
                                                const uint64_t* __restrict__ bitmap, int64_t g0, int ngt) {
     const uint32_t* src = reinterpret_cast<const uint32_t*>(bitmap + g0 * kTileK * kWordsPerCol);
     const uint32_t first = __ldg(tileoffset + g0);
 #pragma unroll
-    for (int i = 0; i < kCols * (kTileM / 32) / kTileM; ++i) {
-        const int q = threadIdx.x + kTileM * i, c = q >> 3, w = q & 7;
+    for (int i = 0; i < kCols * kWords / kTileM; ++i) {
+        const int q = threadIdx.x + kTileM * i, c = q / kWords, w = q % kWords;
         uint32_t word = 0u, off = 0u;
         if (c < ngt * kTileK) {
             word = __ldg(src + q);
@@ -192,13 +195,35 @@ __device__ __forceinline__ uint32_t load_words(PackSmem& sm, const uint32_t* __r
         const uint32_t n = __popc(word);
         uint32_t inc = n;
 #pragma unroll
-        for (int d = 1; d < 8; d <<= 1) {
-            const uint32_t u = __shfl_up_sync(0xFFFFFFFFu, inc, d, 8);
+        for (int d = 1; d < kWords; d <<= 1) {
+            const uint32_t u = __shfl_up_sync(0xFFFFFFFFu, inc, d, kWords);
             if (w >= d) inc += u;
         }
-        sm.words[c >> 1][w][c & 1] = make_uint2(word, off + inc - n);
+        sm.words[w][c] = make_uint2(word, off + inc - n);
     }
     return __ldg(tileoffset + g0 + ngt) - first;
+}
+
+// One row of a lane's two columns: the value of a set bit goes to (comes from) the column's next place in sm.vals; `bit` is
+// the row's.  a0, a1: shared-memory addresses of the next places.
+__device__ __forceinline__ void emit_row(uint32_t v, uint32_t w0, uint32_t w1, uint32_t bit, uint32_t& a0, uint32_t& a1) {
+    asm volatile("{\n .reg .pred p, q;\n .reg .b32 t;\n .reg .b16 l, h;\n"
+                 " lop3.or.b32 t|p, %3, %5, 0, 0xC0, 0;\n lop3.or.b32 t|q, %4, %5, 0, 0xC0, 0;\n"
+                 " mov.b32 {l, h}, %2;\n"
+                 " @p st.shared.u16 [%0], l;\n @p add.u32 %0, %0, 2;\n"
+                 " @q st.shared.u16 [%1], h;\n @q add.u32 %1, %1, 2;\n}"
+                 : "+r"(a0), "+r"(a1) : "r"(v), "r"(w0), "r"(w1), "r"(bit) : "memory");
+}
+__device__ __forceinline__ uint32_t unpack_row(uint32_t w0, uint32_t w1, uint32_t bit, uint32_t& a0, uint32_t& a1) {
+    uint32_t v;
+    asm volatile("{\n .reg .pred p, q;\n .reg .b32 t;\n .reg .b16 l, h;\n"
+                 " lop3.or.b32 t|p, %3, %5, 0, 0xC0, 0;\n lop3.or.b32 t|q, %4, %5, 0, 0xC0, 0;\n"
+                 " mov.b16 l, 0;\n mov.b16 h, 0;\n"
+                 " @p ld.shared.u16 l, [%0];\n @p add.u32 %0, %0, 2;\n"
+                 " @q ld.shared.u16 h, [%1];\n @q add.u32 %1, %1, 2;\n"
+                 " mov.b32 %2, {l, h};\n}"
+                 : "+r"(a0), "+r"(a1), "=r"(v) : "r"(w0), "r"(w1), "r"(bit));
+    return v;
 }
 
 // Pass 3: the stored elements in column order, each column followed by its zero padding.
@@ -206,27 +231,23 @@ __global__ void __launch_bounds__(kTileM)
 pack_emit_kernel(const unsigned short* __restrict__ W, int64_t ldw, int64_t M, int64_t K, int64_t C, int blocks, int pad_elems,
                  const uint32_t* __restrict__ tileoffset, const uint32_t* __restrict__ colinfo, const uint64_t* __restrict__ bitmap,
                  unsigned short* __restrict__ values) {
-    extern __shared__ __align__(16) unsigned char raw[];
-    PackSmem& sm = *reinterpret_cast<PackSmem*>(raw);
+    __shared__ BlockSmem sm;
     const int64_t r = blockIdx.x / static_cast<unsigned>(blocks), cb = blockIdx.x % static_cast<unsigned>(blocks);
     const int64_t g0 = r * C + cb * kGT;
     const int ngt = static_cast<int>(min(static_cast<int64_t>(kGT), C - cb * kGT));
     const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
-    load_block(W, ldw, M, K, r * kTileM, cb * kCols, sm.tile);
+    uint32_t v[32];
+    load_rows<32>(W, ldw, M, K, r * kTileM + 32 * warp, cb * kCols + 2 * lane, v);
     const uint32_t total = load_words(sm, tileoffset, colinfo, bitmap, g0, ngt);
     __syncthreads();
-    const unsigned bit = 1u << lane, below = bit - 1u;
-    const uint32_t* mine = sm.tile + t * kRowWords;
-#pragma unroll 8
-    for (int c = 0; c < kCols / 2; ++c) {
-        const uint32_t v = mine[c];
-        const uint4 e = *reinterpret_cast<const uint4*>(&sm.words[c][warp][0]);
-        if (e.x & bit) sm.vals[e.y + __popc(e.x & below)] = static_cast<unsigned short>(v & 0xFFFFu);
-        if (e.z & bit) sm.vals[e.w + __popc(e.z & below)] = static_cast<unsigned short>(v >> 16);
-    }
+    const uint4 e = *reinterpret_cast<const uint4*>(&sm.words[warp][2 * lane]);
+    const uint32_t base = static_cast<uint32_t>(__cvta_generic_to_shared(&sm.vals[0]));
+    uint32_t a0 = base + 2u * e.y, a1 = base + 2u * e.w;
+#pragma unroll
+    for (int i = 0; i < 32; ++i) emit_row(v[i], e.x, e.z, 1u << i, a0, a1);
     if (t < ngt * kTileK) {
-        const uint2 last = sm.words[t >> 1][kTileM / 32 - 1][t & 1];
-        const uint32_t end = last.y + __popc(last.x), n = end - sm.words[t >> 1][0][t & 1].y;
+        const uint2 last = sm.words[kWords - 1][t];
+        const uint32_t end = last.y + __popc(last.x), n = end - sm.words[0][t].y;
         const uint32_t padding = (n + pad_elems - 1) / pad_elems * pad_elems - n;
         for (uint32_t i = 0; i < padding; ++i) sm.vals[end + i] = 0;
     }
@@ -244,43 +265,38 @@ __global__ void __launch_bounds__(kTileM)
 unpack_kernel(const uint32_t* __restrict__ tileoffset, const uint32_t* __restrict__ colinfo,
               const uint64_t* __restrict__ bitmap, const unsigned short* __restrict__ values, int pad_elems,
               int64_t M, int64_t K, int64_t C, int blocks, unsigned short* __restrict__ W, int64_t ldw) {
-    extern __shared__ __align__(16) unsigned char raw[];
-    PackSmem& sm = *reinterpret_cast<PackSmem*>(raw);
+    __shared__ BlockSmem sm;
     const int64_t r = blockIdx.x / static_cast<unsigned>(blocks), cb = blockIdx.x % static_cast<unsigned>(blocks);
     const int64_t g0 = r * C + cb * kGT;
     const int ngt = static_cast<int>(min(static_cast<int64_t>(kGT), C - cb * kGT));
     const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
-    const uint32_t total = load_words(sm, tileoffset, colinfo, bitmap, g0, ngt);
-    const unsigned short* in = values + tileoffset[g0];
-    if (pad_elems == 8) {
-        for (uint32_t i = t; i < total / 8; i += kTileM) reinterpret_cast<uint4*>(sm.vals)[i] = __ldg(reinterpret_cast<const uint4*>(in) + i);
+    const uint32_t v0 = __ldg(tileoffset + g0), n = __ldg(tileoffset + g0 + ngt) - v0;
+    const unsigned short* in = values + v0;
+    if (pad_elems == 8) {                                   // asynchronous, so that all pieces and the words are on their way together
+        for (uint32_t i = t; i < n / 8; i += kTileM)
+            dev::cp_async16<0>(static_cast<uint32_t>(__cvta_generic_to_shared(&sm.vals[8 * i])), in + 8 * i, 1);
+        dev::cp_async_commit();
     } else {
-        for (uint32_t i = t; i < total; i += kTileM) sm.vals[i] = __ldg(in + i);
+        for (uint32_t i = t; i < n; i += kTileM) sm.vals[i] = __ldg(in + i);
     }
+    load_words(sm, tileoffset, colinfo, bitmap, g0, ngt);
+    dev::cp_async_wait<0>();
     __syncthreads();
-    const unsigned bit = 1u << lane, below = bit - 1u;
-    uint32_t* mine = sm.tile + t * kRowWords;
-#pragma unroll 8
-    for (int c = 0; c < kCols / 2; ++c) {
-        const uint4 e = *reinterpret_cast<const uint4*>(&sm.words[c][warp][0]);
-        uint32_t lo = 0u, hi = 0u;
-        if (e.x & bit) lo = sm.vals[e.y + __popc(e.x & below)];
-        if (e.z & bit) hi = sm.vals[e.w + __popc(e.z & below)];
-        mine[c] = lo | (hi << 16);
-    }
-    __syncthreads();
-    const bool wide = ((reinterpret_cast<uintptr_t>(W) | static_cast<uintptr_t>(2 * ldw)) & 15u) == 0;
-#pragma unroll
-    for (int i = 0; i < kCols / 8; ++i) {
-        const int q = t + kTileM * i;
-        const int64_t row = r * kTileM + q / kPieces, col = cb * kCols + (q % kPieces) * 8;
-        if (row >= M || col >= K) continue;
-        const uint32_t* src = sm.tile + (q / kPieces) * kRowWords + (q % kPieces) * 4;
-        unsigned short* dst = W + row * ldw + col;
-        if (wide && col + 8 <= K) {
-            *reinterpret_cast<uint4*>(dst) = make_uint4(src[0], src[1], src[2], src[3]);
+    const uint4 e = *reinterpret_cast<const uint4*>(&sm.words[warp][2 * lane]);
+    const uint32_t base = static_cast<uint32_t>(__cvta_generic_to_shared(&sm.vals[0]));
+    uint32_t a0 = base + 2u * e.y, a1 = base + 2u * e.w;
+    const int64_t row = r * kTileM + 32 * warp, col = cb * kCols + 2 * lane;
+    unsigned short* dst = W + row * ldw + col;
+    const bool wide = ((reinterpret_cast<uintptr_t>(W) | static_cast<uintptr_t>(2 * ldw)) & 3u) == 0 && col + 1 < K;
+#pragma unroll 16
+    for (int i = 0; i < 32; ++i, dst += ldw) {
+        const uint32_t v = unpack_row(e.x, e.z, 1u << i, a0, a1);
+        if (row + i >= M || col >= K) continue;
+        if (wide) {
+            *reinterpret_cast<uint32_t*>(dst) = v;
         } else {
-            for (int e = 0; e < 8 && col + e < K; ++e) dst[e] = static_cast<unsigned short>(src[e >> 1] >> (16 * (e & 1)));
+            dst[0] = static_cast<unsigned short>(v & 0xFFFFu);
+            if (col + 1 < K) dst[1] = static_cast<unsigned short>(v >> 16);
         }
     }
 }
@@ -348,22 +364,6 @@ pack_q4_emit_kernel(const unsigned short* __restrict__ W, int64_t ldw, int64_t M
 
 }  // namespace
 
-// Shared-memory opt-in of the emit and unpack kernels, once per device.
-spdp_status configure_pack_kernels() {
-    static std::mutex mu;
-    static bool configured[64] = {};
-    int dev = 0;
-    SPDP_CUDA_TRY(cudaGetDevice(&dev));
-    if (dev < 0 || dev >= 64) return SPDP_ERR_UNSUPPORTED_SHAPE;
-    std::lock_guard<std::mutex> lock(mu);
-    if (!configured[dev]) {
-        SPDP_CUDA_TRY(cudaFuncSetAttribute(pack_emit_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(sizeof(PackSmem))));
-        SPDP_CUDA_TRY(cudaFuncSetAttribute(unpack_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(sizeof(PackSmem))));
-        configured[dev] = true;
-    }
-    return SPDP_OK;
-}
-
 // Count and scan, then the emit pass of the handle's variant (fp16 values, or 4-bit codes with scales).  The arrays whose
 // sizes follow from the shape are allocated already; the length of Values is known after the scan, which is what the one
 // synchronisation in the middle is for.  The caller synchronises after the emit pass.
@@ -372,11 +372,9 @@ spdp_status pack_device(spdp_matrix* h, const __half* W, int64_t ldw, cudaStream
     const unsigned short* Wb = reinterpret_cast<const unsigned short*>(W);
     const int blocks = static_cast<int>((h->C + kGT - 1) / kGT);
     const unsigned grid = static_cast<unsigned>(h->R * blocks);
-    spdp_status st = configure_pack_kernels();
-    if (st != SPDP_OK) return st;
     uint32_t* tile_len = nullptr;
     unsigned long long* total_dev = nullptr;               // [0] Values length, [1] nnz
-    st = handle_alloc(h->device, 2 * sizeof(unsigned long long) + NGT * sizeof(uint32_t), &h->packing);
+    spdp_status st = handle_alloc(h->device, 2 * sizeof(unsigned long long) + NGT * sizeof(uint32_t), &h->packing);
     if (st != SPDP_OK) return st;
     total_dev = static_cast<unsigned long long*>(h->packing.p);
     tile_len = reinterpret_cast<uint32_t*>(total_dev + 2);
@@ -404,7 +402,7 @@ spdp_status pack_device(spdp_matrix* h, const __half* W, int64_t ldw, cudaStream
         spdp_status a = handle_alloc(h->device, vbytes < 16 ? 16 : vbytes, &h->values_block);
         if (a != SPDP_OK) return a;
         h->values = static_cast<__half*>(h->values_block.p);
-        pack_emit_kernel<<<grid, kTileM, sizeof(PackSmem), s>>>(Wb, ldw, h->M, h->K, h->C, blocks, h->pad_elems, h->tileoffset,
+        pack_emit_kernel<<<grid, kTileM, 0, s>>>(Wb, ldw, h->M, h->K, h->C, blocks, h->pad_elems, h->tileoffset,
                                                                 h->colinfo, h->bitmap, reinterpret_cast<unsigned short*>(h->values));
     }
     SPDP_CUDA_TRY(cudaGetLastError());
@@ -413,7 +411,7 @@ spdp_status pack_device(spdp_matrix* h, const __half* W, int64_t ldw, cudaStream
 
 spdp_status unpack_device(const spdp_matrix* h, __half* W, int64_t ldw, cudaStream_t s) {
     const int blocks = static_cast<int>((h->C + kGT - 1) / kGT);
-    unpack_kernel<<<static_cast<unsigned>(h->R * blocks), kTileM, sizeof(PackSmem), s>>>(
+    unpack_kernel<<<static_cast<unsigned>(h->R * blocks), kTileM, 0, s>>>(
         h->tileoffset, h->colinfo, h->bitmap, reinterpret_cast<const unsigned short*>(h->values), h->pad_elems,
         h->M, h->K, h->C, blocks, reinterpret_cast<unsigned short*>(W), ldw);
     SPDP_CUDA_TRY(cudaGetLastError());

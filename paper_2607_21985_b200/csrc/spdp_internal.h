@@ -115,7 +115,6 @@ void give_back_all();
 spdp_status scratch_alloc(int device, size_t bytes, cudaStream_t s, void** out);
 
 // pack.cu
-spdp_status configure_pack_kernels();          // per-device kernel attributes; idempotent
 spdp_status pack_device(spdp_matrix* h, const __half* W, int64_t ldw, cudaStream_t s);     // either variant
 spdp_status unpack_device(const spdp_matrix* h, __half* W, int64_t ldw, cudaStream_t s);
 
