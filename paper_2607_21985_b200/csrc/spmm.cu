@@ -105,6 +105,9 @@ struct Params {
 // Shared-memory operand descriptor of tcgen05.mma: start address, leading byte offset, stride byte
 // offset (all in 16-byte units), descriptor version of this architecture, layout (bits 61-63: 0 = no
 // swizzle, 2 = 128-byte swizzle).
+template <uint32_t kSbo, uint32_t kLayout>
+constexpr uint32_t kDescHigh = (kSbo >> 4) | (1u << 14) | (kLayout << 29);
+__device__ __forceinline__ uint32_t desc_low(uint32_t smem_addr, uint32_t lbo) { return ((smem_addr & 0x3FFFFu) >> 4) | ((lbo >> 4) << 16); }
 __device__ __forceinline__ uint64_t operand_desc(uint32_t smem_addr, uint32_t lbo, uint32_t sbo, uint32_t layout) {
     uint64_t d = (smem_addr & 0x3FFFFu) >> 4;
     d |= static_cast<uint64_t>(lbo >> 4) << 16;
@@ -116,12 +119,13 @@ __device__ __forceinline__ uint64_t operand_desc(uint32_t smem_addr, uint32_t lb
 // Instruction descriptor: fp16 x fp16 -> fp32, A M-major (bit 15), B K-major, kM rows, kN tokens.
 template <int kM, int kN>
 constexpr uint32_t kInstrDesc = (1u << 4) | (1u << 15) | (static_cast<uint32_t>(kN >> 3) << 17) | (static_cast<uint32_t>(kM >> 4) << 24);
-// D[tmem] (+)= A * B, one CTA (M = 128) or a CTA pair (M = 256).
-template <int kN>
-__device__ __forceinline__ void mma_f16_one(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc, bool accumulate) {
-    asm volatile("{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
-                 " tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}"
-                 ::"r"(d_tmem), "l"(a_desc), "l"(b_desc), "r"(kInstrDesc<128, kN>), "r"(accumulate ? 1u : 0u) : "memory");
+// D[tmem] (+)= A * B, one CTA (M = 128) or a CTA pair (M = 256).  The one-CTA form takes the operand descriptors as halves: the upper
+// ones are constants, and the lower ones move by constants, without a carry.
+template <int kN, uint32_t kAHigh, uint32_t kBHigh>
+__device__ __forceinline__ void mma_f16_one(uint32_t d_tmem, uint32_t a_low, uint32_t b_low, uint32_t accumulate) {
+    asm volatile("{\n .reg .pred p;\n .reg .b64 a, b;\n setp.ne.b32 p, %4, 0;\n mov.b64 a, {%1, %5};\n mov.b64 b, {%2, %6};\n"
+                 " tcgen05.mma.cta_group::1.kind::f16 [%0], a, b, %3, p;\n}"
+                 ::"r"(d_tmem), "r"(a_low), "r"(b_low), "r"(kInstrDesc<128, kN>), "r"(accumulate), "n"(kAHigh), "n"(kBHigh) : "memory");
 }
 template <int kN>
 __device__ __forceinline__ void mma_f16_pair(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc, bool accumulate) {
@@ -307,6 +311,41 @@ __device__ __forceinline__ void void_rows(const Params& p, int slot, int row0, i
     for (int i = t; i < p.ptok * rows; i += nthreads) part[static_cast<size_t>(i / rows) * kTileM + row0 + i % rows] = kNoSum;
 }
 
+// The second kernel of a cut call: a block of 256 threads takes 4 tokens x 256 rows of a tile, a thread 4 consecutive rows of
+// one token.  What bounds it is the partial sums' way through L2, behind a launch and one chain of latencies: what a block has to know of
+// its tile is worked out once, with 32-bit divisions, and before the wait for the first kernel.  (With elements dealt out over a
+// fixed grid a thread took 320 instructions, most of them 64-bit divisions behind that wait.)  us per call, before -> now:
+// 1024x1024 x 64 tokens 10.4 -> 8.8, 2048x2048 x 128 15.2 -> 13.2, 4096x11008 x 128 31.2 -> 29.4, 11008x4096 x 128 35.4 -> 33.9.
+constexpr int kReduceTokens = 4;
+// Adds the partial sums of 4 rows at `first` and, count - 1 of them and `stride` floats apart, from `next` on, in this order, and
+// stores them at token n, rows row .. row + 3.
+__device__ __forceinline__ void add_partials(const Params& p, const float* first, const float* next, size_t stride, int count, int64_t n, int64_t row) {
+    float4 sum = __ldcg(reinterpret_cast<const float4*>(first));
+    bool there = __float_as_uint(sum.w) != kNoSum;                   // no CTA of the tile gave up
+#pragma unroll 4
+    for (int i = 1; i < count; ++i) {
+        const float4 v = __ldcg(reinterpret_cast<const float4*>(next));
+        next += stride;
+        there = there && __float_as_uint(v.w) != kNoSum;
+        sum.x += v.x;
+        sum.y += v.y;
+        sum.z += v.z;
+        sum.w += v.w;
+    }
+    if (!there) return;
+    const int64_t at = n * p.ldy + row;
+    if (p.ydt != SPDP_Y_F32 && row + 4 <= p.M && ((reinterpret_cast<uintptr_t>(p.Y) + 2u * static_cast<uintptr_t>(at)) & 7u) == 0) {
+        const __half2 lo = __floats2half2_rn(sum.x, sum.y), hi = __floats2half2_rn(sum.z, sum.w);
+        *reinterpret_cast<uint2*>(static_cast<__half*>(p.Y) + at) =
+            make_uint2(*reinterpret_cast<const unsigned*>(&lo), *reinterpret_cast<const unsigned*>(&hi));
+        return;
+    }
+    const float v[4] = {sum.x, sum.y, sum.z, sum.w};
+#pragma unroll
+    for (int e = 0; e < 4; ++e)
+        if (row + e < p.M) store_y(p.Y, p.ydt, at + e, v[e]);
+}
+
 struct alignas(16) Meta {                       // a K-block as stored, without its values
     alignas(16) uint32_t bm[kKB][8];            // bitmaps
     alignas(16) uint32_t ci[kKB];               // ColInfo words
@@ -408,11 +447,14 @@ struct Form {
     static constexpr int kBBytes = kNI * kBRowBytes;
     static constexpr int kATileBytes = (kSub / 8) * kAKGroupStride;   // 128 rows x kSub columns
     static constexpr int kABytes = 2 * kATileBytes;
-    static constexpr int kAStages = 4;                                // decoded sub-blocks
+    static constexpr int kAStages = kNI == 32 ? 6 : 4;                // decoded sub-blocks.  Three groups decode at once, so four
+        // leave one to spare and the groups wait a fifth of their time for the tensor cores to be done with a stage.  Six, where
+        // X tiles are small: 4096x4096 x 16 tokens 13.0 -> 11.7 us, 28672x8192 x 16 99.9 -> 95.6 (with 128 tokens five stages and two
+        // X tiles gained nothing).
     static constexpr int kBStages = kNI <= 128 ? 3 : 2;
     static constexpr int kMeta = 8;                                   // stored K-blocks in flight, at most
     static_assert(kBBytes % 1024 == 0, "every X tile on a swizzle-atom boundary");
-    static_assert(kAStages == 2 * kSubs && kAStages >= kGroups, "the first A stages are the first two K-blocks, and every decode warp has a sub-block among the next kAStages");
+    static_assert(kAStages >= 2 * kSubs && kAStages >= kGroups, "the first two K-blocks fit in the first A stages, and every decode warp has a sub-block among the next kAStages");
 };
 
 // CTA w's share of the tiles that are cut along K: K-blocks [rest_begin(w), rest_begin(w + 1)).
@@ -528,35 +570,37 @@ spmm_kernel(const __grid_constant__ Params p, const __grid_constant__ CUtensorMa
     if (warp == kWarps) {
         // ================= tensor-core warp: one thread issues the products =================
         if (elect_one()) {
-            unsigned i = 0, u = 0;                                      // sub-blocks and K-blocks so far
+            unsigned sa = 0, pa = 0, sb = 0, pb = 0;                    // stage and parity of the next sub-block and X tile
             bool issued = false;
+            const uint32_t a_base = desc_low(smem_u32(&sm.A[0][0]), kAKGroupStride), b_base = desc_low(smem_u32(&sm.B[0][0]), 16);
             asm volatile("griddepcontrol.wait;" ::: "memory");
             for (int k = 0; ok && piece(p, me, k, s); ++k) {
                 if (k > 0) {
                     ok = wait_parity(&sm.acc_free, (k - 1) & 1);
                     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
                 }
-                for (int kb = 0; ok && kb < s.n; ++kb, ++u) {
-                    const unsigned sb = u % F::kBStages;
-                    ok = wait_parity(&sm.x_full[sb], (u / F::kBStages) & 1);                    // the X tile is in place
-                    for (int h = 0; ok && h < kSubs; ++h, ++i) {
-                        const unsigned sa = i % F::kAStages;
-                        ok = wait_parity(&sm.a_ready[sa], (i / F::kAStages) & 1);               // the decoded W is in place
+                for (int kb = 0; ok && kb < s.n; ++kb) {
+                    ok = wait_parity(&sm.x_full[sb], pb);                                       // the X tile is in place
+                    for (int h = 0; ok && h < kSubs; ++h) {
+                        ok = wait_parity(&sm.a_ready[sa], pa);                                  // the decoded W is in place
                         if (!ok) break;
                         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-                        const uint64_t ad0 = operand_desc(smem_u32(&sm.A[sa][0]), kAKGroupStride, kAChunkStride, 0u);
-                        const uint64_t bd0 = operand_desc(smem_u32(&sm.B[sb][0]), 16, kBAtomBytes, 2u) + ((h * 2 * kSub) >> 4);
+                        const uint32_t al = a_base + sa * (F::kABytes >> 4), bl = b_base + sb * (F::kBBytes >> 4) + h * ((2 * kSub) >> 4);
+                        const uint32_t add = static_cast<uint32_t>(kb + h);      // the first product of a piece starts the sums
 #pragma unroll
                         for (int a = 0; a < 2; ++a) {                   // the two row halves
 #pragma unroll
                             for (int kk = 0; kk < kSub / 16; ++kk)      // the start address is the low field, in 16-byte units
-                                mma_f16_one<F::kNI>(tmem + a * F::kNI, ad0 + ((a * F::kATileBytes + kk * 2 * kAKGroupStride) >> 4),
-                                                    bd0 + ((kk * 32) >> 4), kb > 0 || h > 0 || kk > 0);
+                                mma_f16_one<F::kNI, kDescHigh<kAChunkStride, 0u>, kDescHigh<kBAtomBytes, 2u>>(
+                                    tmem + a * F::kNI, al + ((a * F::kATileBytes + kk * 2 * kAKGroupStride) >> 4), bl + ((kk * 32) >> 4),
+                                    kk > 0 ? 1u : add);
                         }
                         commit_one(&sm.a_free[sa]);
                         issued = true;
+                        if (++sa == F::kAStages) { sa = 0; pa ^= 1u; }
                     }
                     if (ok) commit_one(&sm.x_free[sb]);
+                    if (++sb == F::kBStages) { sb = 0; pb ^= 1u; }
                 }
                 if (ok) commit_one(&sm.acc_full);
             }
@@ -603,7 +647,7 @@ spmm_kernel(const __grid_constant__ Params p, const __grid_constant__ CUtensorMa
         for (int k = 0; ok && piece(p, me, k, s); ++k) {
             const unsigned i1 = i0 + static_cast<unsigned>(s.n) * kSubs;
             unsigned i = i0 + (group + kGroups - i0 % kGroups) % kGroups;
-            for (unsigned upto = min(i1, static_cast<unsigned>(F::kAStages));; upto = i1) {
+            for (unsigned upto = min(i1, 2u * kSubs);; upto = upto < F::kAStages ? min(i1, static_cast<unsigned>(F::kAStages)) : i1) {
                 for (; i < upto; i += kGroups) {
                     const unsigned u = i / kSubs, m = u % F::kMeta, sa = i % F::kAStages;
                     ok = wait_parity(&sm.comp_full[m], (u / F::kMeta) & 1);                          // the stored K-block has arrived
@@ -627,7 +671,7 @@ spmm_kernel(const __grid_constant__ Params p, const __grid_constant__ CUtensorMa
                     }
                 }
                 if (!ok || upto == i1) break;
-                // Behind the first A stages (the first two K-blocks, which find room in any case) a K-block may still be outside
+                // Behind the first two K-blocks, which find room in any case, and behind the first A stages a K-block may still be outside
                 // because the ring is full: then its copy waits for decodes, these for products, and they for X.  (Once, between
                 // two loops: a test in the loop costs 0.4 %, the wait without a test 1 % of a small call.)
                 if (i < i1 && !phase_done(&sm.comp_full[i / kSubs % F::kMeta], (i / kSubs / F::kMeta) & 1))
@@ -668,44 +712,22 @@ spmm_kernel(const __grid_constant__ Params p, const __grid_constant__ CUtensorMa
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "n"(F::kTmemCols) : "memory");
 }
 
-// Adds, in CTA order, the partial sums of the tiles that several CTAs fed, and writes their part of Y.  A thread takes 4
-// consecutive rows of one token.
+// Adds, in CTA order, the partial sums of the tiles that several CTAs fed, and writes their part of Y.
 __global__ void __launch_bounds__(256)
-reduce_pieces_kernel(const Params p, int tile0, int tiles, int tile_tokens) {
+reduce_pieces_kernel(const Params p, int tile0, int chunks, int tile_tokens) {
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-    asm volatile("griddepcontrol.wait;" ::: "memory");
-    const int64_t total = static_cast<int64_t>(tiles) * p.ptok * (kTileM / 4);
-    const unsigned nkb = static_cast<unsigned>(p.nkb);
-    for (int64_t i = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x; i < total;
-         i += static_cast<int64_t>(gridDim.x) * blockDim.x) {
-        const int row_in = 4 * static_cast<int>(i % (kTileM / 4));
-        const int64_t q = i / (kTileM / 4);
-        const int tok = static_cast<int>(q % p.ptok);
-        const unsigned t = static_cast<unsigned>(q / p.ptok);            // tile tile0 + t
-        const unsigned first = rest_owner(p, t * nkb), last = rest_owner(p, (t + 1u) * nkb - 1u);
-        if (first == last) continue;                                     // one CTA had the whole tile: it stored Y itself
-        const int tile = tile0 + static_cast<int>(t);
-        const int64_t n = static_cast<int64_t>(tile % p.nblocks) * tile_tokens + tok;
-        const int64_t row = static_cast<int64_t>(tile / p.nblocks) * kTileM + row_in;
-        if (n >= p.N || row >= p.M) continue;
-        float4 sum = make_float4(0.f, 0.f, 0.f, 0.f);
-        bool there = true;                                               // no CTA of the tile gave up
-        const unsigned first_slot = 2u * first + (rest_begin(p, first) < t * nkb ? 1u : 0u);     // the only one that may start in the tile before
-#pragma unroll 4
-        for (unsigned w = first; w <= last; ++w) {
-            const unsigned slot = w == first ? first_slot : 2u * w;
-            const float4 v = *reinterpret_cast<const float4*>(p.partial + (static_cast<size_t>(slot) * p.ptok + tok) * kTileM + row_in);
-            there = there && __float_as_uint(v.w) != kNoSum;
-            sum.x += v.x;
-            sum.y += v.y;
-            sum.z += v.z;
-            sum.w += v.w;
-        }
-        const float v[4] = {sum.x, sum.y, sum.z, sum.w};
-#pragma unroll
-        for (int e = 0; e < 4; ++e)
-            if (there && row + e < p.M) store_y(p.Y, p.ydt, n * p.ldy + row + e, v[e]);
-    }
+    const unsigned t = blockIdx.x / static_cast<unsigned>(chunks), nkb = static_cast<unsigned>(p.nkb);      // tile tile0 + t
+    const int tok = static_cast<int>(blockIdx.x - t * static_cast<unsigned>(chunks)) * kReduceTokens + static_cast<int>(threadIdx.x >> 6);
+    const unsigned first = rest_owner(p, t * nkb), last = rest_owner(p, (t + 1u) * nkb - 1u);
+    const unsigned tile = static_cast<unsigned>(tile0) + t, r = tile / static_cast<unsigned>(p.nblocks), nb = tile - r * static_cast<unsigned>(p.nblocks);
+    const int row_in = 4 * static_cast<int>(threadIdx.x & 63u);
+    const int64_t n = static_cast<int64_t>(nb) * tile_tokens + tok, row = static_cast<int64_t>(r) * kTileM + row_in;
+    const unsigned first_slot = 2u * first + (rest_begin(p, first) < t * nkb ? 1u : 0u);     // the only one that may start in the tile before
+    const size_t slot = static_cast<size_t>(p.ptok) * kTileM;
+    const float* sums = p.partial + static_cast<size_t>(tok) * kTileM + row_in;
+    asm volatile("griddepcontrol.wait;" ::: "memory");          // (every thread: the kernel after this one relies on it)
+    if (first == last || tok >= p.ptok || n >= p.N || row >= p.M) return;        // a tile that one CTA had is stored already
+    add_partials(p, sums + first_slot * slot, sums + 2u * (first + 1u) * slot, 2u * slot, static_cast<int>(last - first) + 1, n, row);
 }
 
 }  // namespace one
@@ -911,37 +933,20 @@ spmm_kernel(const __grid_constant__ Params p, const __grid_constant__ CUtensorMa
         asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(tmem), "n"(kTmemCols) : "memory");
 }
 
-// Adds the K-slices of the tiles that were cut along K, in slice order, and writes their part of Y.  A thread takes 4
-// consecutive rows of one token.
+// Adds the K-slices of the tiles that were cut along K, in slice order, and writes their part of Y.
 __global__ void __launch_bounds__(256)
-reduce_slices_kernel(const Params p, int tiles) {
+reduce_slices_kernel(const Params p, int chunks) {
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    const unsigned t = blockIdx.x / static_cast<unsigned>(chunks);
+    const int tok = static_cast<int>(blockIdx.x - t * static_cast<unsigned>(chunks)) * kReduceTokens + static_cast<int>(threadIdx.x >> 6);
+    const unsigned tile = static_cast<unsigned>(p.tile0) + t, r = tile / static_cast<unsigned>(p.nblocks), nb = tile - r * static_cast<unsigned>(p.nblocks);
+    const int row_in = 4 * static_cast<int>(threadIdx.x & 63u);
+    const int64_t n = static_cast<int64_t>(nb) * kNT + tok, row = static_cast<int64_t>(r) * kTileM + row_in;
+    const size_t slot = static_cast<size_t>(p.ptok) * kTileM;
+    const float* sums = p.partial + static_cast<size_t>(t) * p.kslices * slot + static_cast<size_t>(tok) * kTileM + row_in;
     asm volatile("griddepcontrol.wait;" ::: "memory");
-    const int64_t total = static_cast<int64_t>(tiles) * p.ptok * (kTileM / 4);
-    for (int64_t i = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x; i < total;
-         i += static_cast<int64_t>(gridDim.x) * blockDim.x) {
-        const int row_in = 4 * static_cast<int>(i % (kTileM / 4));
-        const int64_t q = i / (kTileM / 4);
-        const int tok = static_cast<int>(q % p.ptok), tt = static_cast<int>(q / p.ptok);
-        const int tile = p.tile0 + tt;
-        const int64_t n = static_cast<int64_t>(tile % p.nblocks) * kNT + tok, row = static_cast<int64_t>(tile / p.nblocks) * kTileM + row_in;
-        if (n >= p.N || row >= p.M) continue;
-        const float* src = p.partial + (static_cast<size_t>(tt) * p.kslices * p.ptok + tok) * kTileM + row_in;
-        float4 sum = make_float4(0.f, 0.f, 0.f, 0.f);
-        bool there = true;                                               // no CTA of the tile gave up
-        for (int sl = 0; sl < p.kslices; ++sl) {
-            const float4 v = *reinterpret_cast<const float4*>(src + static_cast<size_t>(sl) * p.ptok * kTileM);
-            there = there && __float_as_uint(v.w) != kNoSum;
-            sum.x += v.x;
-            sum.y += v.y;
-            sum.z += v.z;
-            sum.w += v.w;
-        }
-        const float v[4] = {sum.x, sum.y, sum.z, sum.w};
-#pragma unroll
-        for (int e = 0; e < 4; ++e)
-            if (there && row + e < p.M) store_y(p.Y, p.ydt, n * p.ldy + row + e, v[e]);
-    }
+    if (tok >= p.ptok || n >= p.N || row >= p.M) return;
+    add_partials(p, sums, sums + slot, slot, p.kslices, n, row);
 }
 
 }  // namespace pair
@@ -1097,13 +1102,12 @@ spdp_status launch_pairs(const Params& p, const CUtensorMap& xmap, int64_t pairs
     return SPDP_OK;
 }
 
-// The second kernel of a call whose last `tiles` tiles were cut: 4 rows of one token per thread, launched programmatically
+// The second kernel of a call whose last `tiles` tiles were cut, launched programmatically
 // (behind CTA pairs, which wait for a plain launch themselves: 2 us of every call that is cut, 4001x4098 x 300 33.0 -> 31.2).
 template <class Kernel, class... Args>
-spdp_status launch_reduce(Kernel kernel, const spdp_matrix* h, int64_t tiles, cudaStream_t s, const Params& p, Args... args) {
-    const int64_t threads = tiles * p.ptok * (kTileM / 4);
+spdp_status launch_reduce(Kernel kernel, int64_t tiles, int chunks, cudaStream_t s, const Params& p, Args... args) {
     cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(static_cast<unsigned>(std::min<int64_t>((threads + 255) / 256, int64_t(8) * h->sm_count)));
+    cfg.gridDim = dim3(static_cast<unsigned>(tiles * chunks));
     cfg.blockDim = dim3(256);
     cfg.stream = s;
     cudaLaunchAttribute attr[1];
@@ -1130,6 +1134,7 @@ spdp_status run_plan(const spdp_matrix* h, Params p, const Plan& plan, const __h
         st = scratch_alloc(h->device, slots * p.ptok * kTileM * sizeof(float), s, reinterpret_cast<void**>(&p.partial));
         if (st != SPDP_OK) return st;
     }
+    const int chunks = (p.ptok + kReduceTokens - 1) / kReduceTokens;
     if (plan.kernel == 3) {
         const int64_t block_bytes = 2 * h->values_len / (h->R * p.nkb);      // values of an average K-block
         Params whole = p;                                                    // whole tiles first, then the last tiles cut along K
@@ -1139,7 +1144,7 @@ spdp_status run_plan(const spdp_matrix* h, Params p, const Plan& plan, const __h
             p.tile0 = static_cast<int>(plan.tiles - plan.rest);
             p.kslices = plan.slices;
             st = launch_pairs(p, xmap, plan.rest * plan.slices, block_bytes, s);
-            if (st == SPDP_OK) st = launch_reduce(pair::reduce_slices_kernel, h, plan.rest, s, p, static_cast<int>(plan.rest));
+            if (st == SPDP_OK) st = launch_reduce(pair::reduce_slices_kernel, plan.rest, chunks, s, p, chunks);
         }
     } else {
         p.workers = plan.workers;
@@ -1148,7 +1153,7 @@ spdp_status run_plan(const spdp_matrix* h, Params p, const Plan& plan, const __h
         p.rest_units = static_cast<unsigned>(plan.rest * p.nkb);
         st = plan.kernel == 0 ? launch_one<One32>(p, xmap, s) : plan.kernel == 1 ? launch_one<One128>(p, xmap, s) : launch_one<One256>(p, xmap, s);
         if (st == SPDP_OK && cut)
-            st = launch_reduce(one::reduce_pieces_kernel, h, plan.rest, s, p, plan.rounds * plan.workers, static_cast<int>(plan.rest), nt);
+            st = launch_reduce(one::reduce_pieces_kernel, plan.rest, chunks, s, p, plan.rounds * plan.workers, chunks, nt);
     }
     if (cut) cudaFreeAsync(p.partial, s);
     return st;

@@ -317,3 +317,32 @@ def test_spmm_cut_tiles_on_two_streams(S, a, b):
     finally:
         for h in {layers[0][0], layers[1][0]}:
             S.spdp_free(h)
+
+
+@pytest.mark.parametrize("R,K,N", [(4, 2048, 30), (4, 2048, 1), (3, 1280, 129), (75, 2048, 700)])
+@pytest.mark.parametrize("dt", [torch.float16, torch.float32])
+def test_spmm_cut_tiles_into_any_y(S, R, K, N, dt):
+    """The second kernel of a cut call stores 4 rows at once where Y allows it: rows that end inside such a group, tokens that
+    are no multiple of the block's, and a Y whose base and row stride are off the 8-byte boundary give the same bits as an aligned
+    Y, and nothing outside Y is written.  (75 row tiles x 700 tokens: K-slices of CTA pairs, the others ranges of one-CTA forms.)"""
+    M = 256 * R - 6
+    g = torch.Generator(device="cuda").manual_seed(R * K + N)
+    W = torch.randn(M, K, generator=g, device="cuda").half() * (torch.rand(M, K, generator=g, device="cuda") < 0.5)
+    X = torch.randn(N, K, generator=g, device="cuda").half()
+    h = S.spdp_pack_tiled_cbc(W)
+    try:
+        want = torch.full((N, M + 2), float("nan"), dtype=dt, device="cuda")[:, :M]       # rows start on 8-byte boundaries
+        S.spdp_spmm(h, X, want)
+        torch.cuda.synchronize()
+        assert S.spdp_last_device_status(h) == 0 and not torch.isnan(want).any()
+        err = (want.double() - X.double() @ W.double().T).abs()
+        assert bool((err <= 1e-3 * (X.double().abs() @ W.double().abs().T) + 1e-5).all())
+        for pad, at in ((0, 0), (1, 1), (3, 2), (5, 3)):
+            buf = torch.full((N * (M + pad) + at + 8,), 7.0, dtype=dt, device="cuda")
+            Y = buf[at:at + N * (M + pad)].view(N, M + pad)
+            S.spdp_spmm(h, X, Y[:, :M])
+            torch.cuda.synchronize()
+            assert torch.equal(Y[:, :M], want)
+            assert bool((Y[:, M:] == 7.0).all()) and bool((buf[:at] == 7.0).all()) and bool((buf[at + N * (M + pad):] == 7.0).all())
+    finally:
+        S.spdp_free(h)
