@@ -812,6 +812,7 @@ spmm_kernel(const __grid_constant__ Params p, const __grid_constant__ CUtensorMa
                      ::"r"(smem_u32(&sm.tmem_base)), "n"(kTmemCols) : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
     }
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
     pair_sync();                       // both CTAs' barriers and tensor memory exist before either reaches into the other
@@ -822,11 +823,13 @@ spmm_kernel(const __grid_constant__ Params p, const __grid_constant__ CUtensorMa
     const int kb0 = static_cast<int>(static_cast<int64_t>(nkb_all) * slice / p.kslices);
     const int nkb = static_cast<int>(static_cast<int64_t>(nkb_all) * (slice + 1) / p.kslices) - kb0;
     // A wait that runs out (it never should) clears `ok`: the thread then stops waiting but keeps walking the
-    // same barriers as the others, the status word gets SPDP_ERR_TIMEOUT and the outputs stay unwritten.
+    // same barriers as the others, the status word gets SPDP_ERR_TIMEOUT and the outputs stay unwritten.  As in the one-CTA forms,
+    // whatever depends on X first waits for the kernel before this one (griddepcontrol.wait), which no bounded wait covers.
     bool ok = true;
 
     if (warp == kWarps) {
         const bool one = elect_one();
+        asm volatile("griddepcontrol.wait;" ::: "memory");
         if (one && c == 0) {
             // ================= tensor-core thread (first CTA): issues the K-blocks' products for the pair =================
             for (int kb = 0; kb < nkb; ++kb) {
@@ -862,6 +865,7 @@ spmm_kernel(const __grid_constant__ Params p, const __grid_constant__ CUtensorMa
     } else if (warp == kWarps + 3) {
         // ================= X warp: one thread moves my halves of the X tiles =================
         if (elect_one()) {
+            asm volatile("griddepcontrol.wait;" ::: "memory");          // X may come from the kernel before this one
             for (int kb = 0; kb < nkb; ++kb) {
                 // my X tiles of block kb go where block kb - kXStages multiplied from, once that work is complete
                 const int s = kb % kStages, before = kb - kXStages;
@@ -876,6 +880,7 @@ spmm_kernel(const __grid_constant__ Params p, const __grid_constant__ CUtensorMa
         // ================= relay warp (first CTA): the tensor cores' completion arrives on the first CTA's barrier;
         // one thread passes it on to the second CTA's =================
         if (lane == 0 && c == 0) {
+            asm volatile("griddepcontrol.wait;" ::: "memory");
             for (int kb = 0; kb < nkb; ++kb) {
                 const int s = kb % kStages;
                 if (ok) ok = wait_parity(&sm.mma_done[s], (kb / kStages) & 1);
@@ -892,6 +897,9 @@ spmm_kernel(const __grid_constant__ Params p, const __grid_constant__ CUtensorMa
         for (unsigned i = group; i < static_cast<unsigned>(nkb) * kSubs; i += kGroups) {
             const unsigned kb = i / kSubs, s = kb % kStages, j0 = (i % kSubs) * kSub + 4u * wm;      // my first column of the K-block
             const unsigned m = kb % kMeta;
+            // The first K-block finds room in the ring in any case and kStages of them are decoded before any product; one that
+            // is still outside then waits for room, and so, like everything behind the first products, for X.
+            if (kb > 0 && kb < 2 * kStages && (kb >= kStages || !phase_done(&sm.comp_full[m], 0u))) asm volatile("griddepcontrol.wait;" ::: "memory");
             if (ok) ok = wait_parity(&sm.comp_full[m], (kb / kMeta) & 1);                   // the stored block has arrived
             const Meta& mt = sm.meta[m];
             __syncwarp();
@@ -908,7 +916,8 @@ spmm_kernel(const __grid_constant__ Params p, const __grid_constant__ CUtensorMa
             }
         }
     }
-    // the last blocks' tensor-core work
+    // the last blocks' tensor-core work, for which X has to be there; Y and the scratch may belong to the kernel before this one, too
+    asm volatile("griddepcontrol.wait;" ::: "memory");
     for (int kb = (nkb > kStages ? nkb - kStages : 0); ok && kb < nkb; ++kb)
         ok = wait_parity(&sm.mma_done[kb % kStages], (kb / kStages) & 1);
     if (!ok) {
@@ -1021,7 +1030,7 @@ struct Plan {
 // average, 8 % at worst (512x512 x 16 tokens, 8.3 against 7.6 us).  (Fitted to graph replays, where the CTA pairs' plain launch costs nothing, it took pairs for small layers, and cuts that
 // cross tiles as readily as those that do not: 1024x1024 x 32 tokens 14.4 -> 8.3 us, 2048x2048 x 64 16.5 -> 12.8, 4096x4096 x
 // 128 22.9 -> 19.6, x 16 17.7 -> 14.8, 4096x11008 x 128 34.0 -> 31.4, 4001x4098 x 200 30.8 -> 26.3.)
-constexpr double kCallUs[4] = {3.0, 3.7, 3.2, 6.5};                     // a call's fixed part; the pairs' launch waits for the kernel before
+constexpr double kCallUs[4] = {3.0, 3.7, 3.2, 6.5};                     // a call's fixed part
 constexpr double kBlockUs[4] = {0.88, 0.97, 1.22, 0.69};                // a K-block (64 columns x 256 rows), us
 constexpr double kBlockTokenUs[4] = {8.3e-4, 1.8e-4, 0.0, 4.8e-4};      // and per token of the tile
 constexpr double kTileUs = 2.1, kTileTokenUs = 2.3e-3;                  // a tile's start and end, and per token
@@ -1085,25 +1094,29 @@ spdp_status launch_one(const Params& p, const CUtensorMap& xmap, cudaStream_t s)
     return SPDP_OK;
 }
 
+// Programmatic launch for the pairs too: a call's set-up, first copies and first three decoded K-blocks overlap the kernel before.
+// us per call, calls in a row: 4001x4098 x 300 tokens 32.8 -> 28.7, 4096x4096 x 300 28.7 -> 25.3, x 1024 48.1 -> 44.6, 11008x4096 x 300
+// 60.3 -> 56.6.
 spdp_status launch_pairs(const Params& p, const CUtensorMap& xmap, int64_t pairs, int64_t block_bytes, cudaStream_t s) {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(static_cast<unsigned>(2 * pairs));
     cfg.blockDim = dim3(pair::kThreads);
     cfg.dynamicSmemBytes = pair::kSmemBytes;
     cfg.stream = s;
-    cudaLaunchAttribute attr[1];
+    cudaLaunchAttribute attr[2];
     attr[0].id = cudaLaunchAttributeClusterDimension;
     attr[0].val.clusterDim.x = 2;
     attr[0].val.clusterDim.y = 1;
     attr[0].val.clusterDim.z = 1;
+    attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[1].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
-    cfg.numAttrs = 1;
+    cfg.numAttrs = 2;
     SPDP_CUDA_TRY(cudaLaunchKernelEx(&cfg, block_bytes <= pair::kThirdXBytes ? pair::spmm_kernel<3> : pair::spmm_kernel<2>, p, xmap));
     return SPDP_OK;
 }
 
-// The second kernel of a call whose last `tiles` tiles were cut, launched programmatically
-// (behind CTA pairs, which wait for a plain launch themselves: 2 us of every call that is cut, 4001x4098 x 300 33.0 -> 31.2).
+// The second kernel of a call whose last `tiles` tiles were cut, launched programmatically.
 template <class Kernel, class... Args>
 spdp_status launch_reduce(Kernel kernel, int64_t tiles, int chunks, cudaStream_t s, const Params& p, Args... args) {
     cudaLaunchConfig_t cfg = {};
