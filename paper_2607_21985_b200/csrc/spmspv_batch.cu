@@ -114,6 +114,9 @@ __device__ __forceinline__ unsigned lds_at(uint32_t addr) {
     asm volatile("ld.shared.u32 %0, [%1+%2];" : "=r"(v) : "r"(addr), "n"(kOff));
     return v;
 }
+__device__ __forceinline__ unsigned nibble_bits(unsigned W, unsigned top) {     // bit i of the nibble -> byte i
+    return (((W * top) >> 28) * 0x00204081u) & 0x01010101u;
+}
 // Expands 4 consecutive rows of a column tile (Sec. 4.2.1), one nibble (nibble_top, nibble_below) of the 32-bit bitmap word W:
 // `first` is the shared-memory address of the word's first value.  rank = set bits before the nibble;
 // three aligned 32-bit loads cover its at most 4 values wherever they start, two funnel shifts align them, and byte
@@ -122,18 +125,21 @@ __device__ __forceinline__ unsigned lds_at(uint32_t addr) {
 // many instructions and four times the popcounts: 116 us against 113 on the largest layer.  What bounds both is shared
 // memory (its wavefronts take 75 % of the clocks on the largest layer) with the integer pipe behind it (55 %): two warps per K-block with 32 accumulators each, 24 warps
 // per SM, gained nothing.)
+template <bool kSparse>
 struct Nibble { unsigned a, s0, s1, s2, bits; };
-__device__ __forceinline__ Nibble fetch_nibble(unsigned W, uint32_t first, unsigned below, unsigned top) {
-    Nibble n;
+template <bool kSparse>
+__device__ __forceinline__ Nibble<kSparse> fetch_nibble(unsigned W, uint32_t first, unsigned below, unsigned top) {
+    Nibble<kSparse> n;
     n.a = first + 2u * __popc(W * below);
     const uint32_t al = n.a & ~3u;
     n.s0 = lds_at<0>(al);
     n.s1 = lds_at<4>(al);
     n.s2 = lds_at<8>(al);
-    n.bits = (((W * top) >> 28) * 0x00204081u) & 0x01010101u;           // bit i of the nibble -> byte i
+    n.bits = nibble_bits(W, top);
     return n;
 }
-__device__ __forceinline__ void place_nibble(const Nibble& n, unsigned& r01, unsigned& r23) {
+template <bool kSparse>
+__device__ __forceinline__ void place_nibble(const Nibble<kSparse>& n, unsigned& r01, unsigned& r23) {
     const unsigned mis = n.a << 3;                                      // 16 if the first value is an upper half (mod 32)
     const unsigned t0 = __funnelshift_r(n.s0, n.s1, mis), t1 = __funnelshift_r(n.s1, n.s2, mis);
     const unsigned sel = n.bits * 0x22222200u + 0x10101010u;            // byte i: the two byte selectors of row i's value
@@ -141,12 +147,36 @@ __device__ __forceinline__ void place_nibble(const Nibble& n, unsigned& r01, uns
     r01 = permute(t0, 0u, n.bits * 0x21CCu + 0x4444u);                  // rows 0, 1 need t0 alone: a clear row selects zero bytes
     r23 = permute(t0, t1, sel >> 16) & permute(m, m, 0x3322u);
 }
+// The form for sparse layers: the two values that rows 0 and 1 may have and the two that rows 2 and 3 may have are loaded one by one,
+// whether they are there or not.  A 16-bit load leaves the upper half of its register zero, which is what a clear row selects, so that
+// nothing has to be aligned or masked: 18 instructions in place of 24 for 4 rows, 5 of them on the integer pipe in place of
+// 11, but one shared-memory access more, and those cost more the denser the layer is.
+template <>
+struct Nibble<true> { unsigned v0, v1, v2, v3, bits; };
+template <>
+__device__ __forceinline__ Nibble<true> fetch_nibble<true>(unsigned W, uint32_t first, unsigned below, unsigned top) {
+    Nibble<true> n;
+    n.bits = nibble_bits(W, top);
+    const uint32_t a01 = first + 2u * __popc(W * below), a23 = __dp4a(n.bits, 0x00000202u, a01);      // + 2 * (bits of rows 0, 1)
+    n.v0 = lds_u16(a01);
+    n.v1 = lds_u16(a01 + 2u);
+    n.v2 = lds_u16(a23);
+    n.v3 = lds_u16(a23 + 2u);
+    return n;
+}
+template <>
+__device__ __forceinline__ void place_nibble<true>(const Nibble<true>& n, unsigned& r01, unsigned& r23) {
+    // selectors, row 0 in the low byte: 0x10 with bit 0; 0x10 or (with bit 0) 0x54 with bit 1; zero bytes otherwise
+    r01 = permute(n.v0, n.v1, n.bits * 0x43DEu + 0x3232u);
+    r23 = permute(n.v2, n.v3, __dp2a_hi(0xDE0043DEu, n.bits, 0x3232u));      // the same of bits 2 and 3
+}
 // D += A (16 rows x 8 column tiles, fp16) * B (8 column tiles x 8 tokens, fp16), fp32 accumulate.
 __device__ __forceinline__ void mma_16x8x8(float (&c)[4], unsigned a01, unsigned a23, unsigned b01) {
     asm volatile("mma.sync.aligned.m16n8k8.row.col.f32.f16.f16.f32 {%0,%1,%2,%3}, {%4,%5}, {%6}, {%0,%1,%2,%3};"
                  : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3]) : "r"(a01), "r"(a23), "r"(b01));
 }
 
+template <bool kSparse>
 __global__ void __launch_bounds__(kThreads, 1)
 spmspv_batch_kernel(const Params p) {
     extern __shared__ __align__(128) unsigned char smem_raw[];
@@ -374,17 +404,17 @@ spmspv_batch_kernel(const Params p) {
                 const unsigned WB[4] = {wB.x, wB.y, wB.z, wB.w}, FB[4] = {fB.x, fB.y, fB.z, fB.w};
 #pragma unroll
                 for (int w = 0; w < 4; w += 2) {                                     // rows 32 * (4h + w) ..
-                    Nibble a[2], b[2];
+                    Nibble<kSparse> a[2], b[2];
 #pragma unroll
                     for (int e = 0; e < 2; ++e) {
-                        a[e] = fetch_nibble(WA[w + e], FA[w + e], below, top);
-                        b[e] = fetch_nibble(WB[w + e], FB[w + e], below, top);
+                        a[e] = fetch_nibble<kSparse>(WA[w + e], FA[w + e], below, top);
+                        b[e] = fetch_nibble<kSparse>(WB[w + e], FB[w + e], below, top);
                     }
 #pragma unroll
                     for (int e = 0; e < 2; ++e) {
                         unsigned A01, A23, B01, B23;
-                        place_nibble(a[e], A01, A23);
-                        place_nibble(b[e], B01, B23);
+                        place_nibble<kSparse>(a[e], A01, A23);
+                        place_nibble<kSparse>(b[e], B01, B23);
                         mma_16x8x8(acc[2 * (4 * h + w + e)], permute(A01, B01, 0x5410u), permute(A01, B01, 0x7632u), b01);
                         mma_16x8x8(acc[2 * (4 * h + w + e) + 1], permute(A23, B23, 0x5410u), permute(A23, B23, 0x7632u), b01);
                     }
@@ -465,13 +495,17 @@ spdp_status configure_spmspv_batch_kernel() {
     if (dev < 0 || dev >= 64) return SPDP_ERR_UNSUPPORTED_SHAPE;
     std::lock_guard<std::mutex> lock(mu);
     if (!configured[dev]) {
-        SPDP_CUDA_TRY(cudaFuncSetAttribute(spmspv_batch_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                           static_cast<int>(sizeof(Smem))));
+        SPDP_CUDA_TRY(cudaFuncSetAttribute(spmspv_batch_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(sizeof(Smem))));
+        SPDP_CUDA_TRY(cudaFuncSetAttribute(spmspv_batch_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(sizeof(Smem))));
         configured[dev] = true;
     }
     return SPDP_OK;
 }
 
+// Layers whose average column tile holds at most this many values take the form with 16-bit loads.  us, aligned words / 16-bit loads,
+// at 60, 70, 80 and 90 % sparsity (102, 77, 51, 26 values): 28672x8192 x 8 tokens 96.0 / 102.6, 93.3 / 93.4, 92.1 / 85.7, 91.8 / 83.7;
+// 4096x4096 x 8 13.9 / 14.1, 13.5 / 13.3, 13.1 / 12.4, 13.0 / 12.2; 11008x4096 x 3 25.3 / 26.0, 24.7 / 24.3, 23.9 / 22.5, 23.6 / 22.0.
+constexpr int64_t kSparseValues = 80;
 spdp_status launch_spmspv_batch(const spdp_matrix* h, const __half* x, int64_t ldx, int batch, int rule, float thr,
                                 const uint32_t* mask, int64_t mask_stride, void* y, int64_t ldy, int ydt,
                                 cudaStream_t s) {
@@ -509,7 +543,8 @@ spdp_status launch_spmspv_batch(const spdp_matrix* h, const __half* x, int64_t l
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    SPDP_CUDA_TRY(cudaLaunchKernelEx(&cfg, spmspv_batch_kernel, p));
+    const bool sparse = h->nnz <= kSparseValues * h->R * h->K;
+    SPDP_CUDA_TRY(cudaLaunchKernelEx(&cfg, sparse ? spmspv_batch_kernel<true> : spmspv_batch_kernel<false>, p));
     return SPDP_OK;
 }
 
