@@ -12,7 +12,7 @@
 //   * the list phase also reads the active columns' scales and keeps scale * x (exact in fp32) per record;
 //   * decode (Sec. 4.2.1): lane l owns rows 8l .. 8l+7 of a column tile (one bitmap byte); rank = set bits
 //     before that byte; its codes are one span of at most 8 nibbles, read as two 32-bit words,
-//     funnel-shifted into one register and walked bit by bit (five instructions per row).
+//     funnel-shifted into one register and walked bit by bit (four instructions per row).
 #include <cstddef>
 #include <mutex>
 
@@ -105,27 +105,35 @@ static_assert(kWarps >= 16, "two groups of 256 threads finish two row tiles side
 // The walk over a lane's 8 rows (Sec. 4.2.1 with 4-bit codes), from the last row to the first: `span` holds the
 // lane's codes with the LAST one in the top nibble; a set bit takes the top nibble and shifts the span left.
 // mad.hi(span, 16, 2^23-as-float bits) = (span >> 28) | 0x4B000000 = 2^23 + code as a float, so one subtraction
-// turns the code into code - 8 without a conversion; acc[row] += (code - 8) * (scale * x).  Five instructions per
-// row, the last two predicated.  `bits` has the lane's 8 rows in its top byte.  (The 16 of the multiply-high in a register,
-// so that it stays one, is slower: 42.0 us on 28672x8192 against 41.0.)
-#define SPDP_Q4_ROW(K)                                              \
-    " lop3.or.b32 t|p, %9, " #K ", 0, 0xC0, 0;\n"                  \
+// turns the code into code - 8 without a conversion; acc[row] += (code - 8) * (scale * x).  Four instructions per
+// row, the last two predicated.  `bits` has the lane's 8 rows in its top byte; all of them are tested ahead of the walk, as mask and
+// comparison, for which the compiler has shorter code than for a test in front of each row (what bounds this kernel is issue: 28672x8192 41.4 -> 39.3 us, 20480x5632 22.5 -> 21.5, 1024x1024 6.2 -> 6.0).  (The 16 of
+// the multiply-high in a register, so that it stays one, is slower: 42.0 us on 28672x8192 against 41.0.)
+#define SPDP_Q4_ROW                                                 \
     " mad.hi.u32 c, %8, 16, 0x4B000000;\n"                         \
     " add.f32 w, c, 0fCB000008;\n"
 __device__ __forceinline__ void walk_codes(unsigned bits, unsigned span, float sx, float (&acc)[8]) {
     asm volatile(
         "{\n"
-        " .reg .pred p;\n"
+        " .reg .pred p0, p1, p2, p3, p4, p5, p6, p7;\n"
         " .reg .b32 t, c;\n"
         " .reg .f32 w;\n"
-        SPDP_Q4_ROW(128 << 24) " @p fma.rn.f32 %7, w, %10, %7;\n @p mul.lo.u32 %8, %8, 16;\n"
-        SPDP_Q4_ROW(64 << 24)  " @p fma.rn.f32 %6, w, %10, %6;\n @p mul.lo.u32 %8, %8, 16;\n"
-        SPDP_Q4_ROW(32 << 24)  " @p fma.rn.f32 %5, w, %10, %5;\n @p mul.lo.u32 %8, %8, 16;\n"
-        SPDP_Q4_ROW(16 << 24)  " @p fma.rn.f32 %4, w, %10, %4;\n @p mul.lo.u32 %8, %8, 16;\n"
-        SPDP_Q4_ROW(8 << 24)   " @p fma.rn.f32 %3, w, %10, %3;\n @p mul.lo.u32 %8, %8, 16;\n"
-        SPDP_Q4_ROW(4 << 24)   " @p fma.rn.f32 %2, w, %10, %2;\n @p mul.lo.u32 %8, %8, 16;\n"
-        SPDP_Q4_ROW(2 << 24)   " @p fma.rn.f32 %1, w, %10, %1;\n @p mul.lo.u32 %8, %8, 16;\n"
-        SPDP_Q4_ROW(1 << 24)   " @p fma.rn.f32 %0, w, %10, %0;\n"
+        " and.b32 t, %9, 0x80000000; setp.ne.u32 p7, t, 0;\n"
+        " and.b32 t, %9, 0x40000000; setp.ne.u32 p6, t, 0;\n"
+        " and.b32 t, %9, 0x20000000; setp.ne.u32 p5, t, 0;\n"
+        " and.b32 t, %9, 0x10000000; setp.ne.u32 p4, t, 0;\n"
+        " and.b32 t, %9, 0x08000000; setp.ne.u32 p3, t, 0;\n"
+        " and.b32 t, %9, 0x04000000; setp.ne.u32 p2, t, 0;\n"
+        " and.b32 t, %9, 0x02000000; setp.ne.u32 p1, t, 0;\n"
+        " and.b32 t, %9, 0x01000000; setp.ne.u32 p0, t, 0;\n"
+        SPDP_Q4_ROW " @p7 fma.rn.f32 %7, w, %10, %7;\n @p7 mul.lo.u32 %8, %8, 16;\n"
+        SPDP_Q4_ROW " @p6 fma.rn.f32 %6, w, %10, %6;\n @p6 mul.lo.u32 %8, %8, 16;\n"
+        SPDP_Q4_ROW " @p5 fma.rn.f32 %5, w, %10, %5;\n @p5 mul.lo.u32 %8, %8, 16;\n"
+        SPDP_Q4_ROW " @p4 fma.rn.f32 %4, w, %10, %4;\n @p4 mul.lo.u32 %8, %8, 16;\n"
+        SPDP_Q4_ROW " @p3 fma.rn.f32 %3, w, %10, %3;\n @p3 mul.lo.u32 %8, %8, 16;\n"
+        SPDP_Q4_ROW " @p2 fma.rn.f32 %2, w, %10, %2;\n @p2 mul.lo.u32 %8, %8, 16;\n"
+        SPDP_Q4_ROW " @p1 fma.rn.f32 %1, w, %10, %1;\n @p1 mul.lo.u32 %8, %8, 16;\n"
+        SPDP_Q4_ROW " @p0 fma.rn.f32 %0, w, %10, %0;\n"
         "}"
         : "+f"(acc[0]), "+f"(acc[1]), "+f"(acc[2]), "+f"(acc[3]), "+f"(acc[4]), "+f"(acc[5]), "+f"(acc[6]), "+f"(acc[7]),
           "+r"(span)
