@@ -116,22 +116,23 @@ __device__ __forceinline__ uint64_t operand_desc(uint32_t smem_addr, uint32_t lb
     d |= static_cast<uint64_t>(layout) << 61;
     return d;
 }
-// Instruction descriptor: fp16 x fp16 -> fp32, A M-major (bit 15), B K-major, kM rows, kN tokens.
-template <int kM, int kN>
-constexpr uint32_t kInstrDesc = (1u << 4) | (1u << 15) | (static_cast<uint32_t>(kN >> 3) << 17) | (static_cast<uint32_t>(kM >> 4) << 24);
+// Instruction descriptor: fp16 x fp16 -> fp32, A M-major (bit 15), B K-major, m rows, n tokens.  n is what a tile's tokens need, in
+// units of 16 (pairs: 32), and not the tile's width: products, their reads and their power for tokens that exist.
+__host__ __device__ constexpr uint32_t instr_desc(int m, int n) {
+    return (1u << 4) | (1u << 15) | (static_cast<uint32_t>(n >> 3) << 17) | (static_cast<uint32_t>(m >> 4) << 24);
+}
 // D[tmem] (+)= A * B, one CTA (M = 128) or a CTA pair (M = 256).  The one-CTA form takes the operand descriptors as halves: the upper
 // ones are constants, and the lower ones move by constants, without a carry.
-template <int kN, uint32_t kAHigh, uint32_t kBHigh>
-__device__ __forceinline__ void mma_f16_one(uint32_t d_tmem, uint32_t a_low, uint32_t b_low, uint32_t accumulate) {
+template <uint32_t kAHigh, uint32_t kBHigh>
+__device__ __forceinline__ void mma_f16_one(uint32_t d_tmem, uint32_t a_low, uint32_t b_low, uint32_t instr_desc, uint32_t accumulate) {
     asm volatile("{\n .reg .pred p;\n .reg .b64 a, b;\n setp.ne.b32 p, %4, 0;\n mov.b64 a, {%1, %5};\n mov.b64 b, {%2, %6};\n"
                  " tcgen05.mma.cta_group::1.kind::f16 [%0], a, b, %3, p;\n}"
-                 ::"r"(d_tmem), "r"(a_low), "r"(b_low), "r"(kInstrDesc<128, kN>), "r"(accumulate), "n"(kAHigh), "n"(kBHigh) : "memory");
+                 ::"r"(d_tmem), "r"(a_low), "r"(b_low), "r"(instr_desc), "r"(accumulate), "n"(kAHigh), "n"(kBHigh) : "memory");
 }
-template <int kN>
-__device__ __forceinline__ void mma_f16_pair(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc, bool accumulate) {
+__device__ __forceinline__ void mma_f16_pair(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc, uint32_t instr_desc, bool accumulate) {
     asm volatile("{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
                  " tcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %3, p;\n}"
-                 ::"r"(d_tmem), "l"(a_desc), "l"(b_desc), "r"(kInstrDesc<256, kN>), "r"(accumulate ? 1u : 0u) : "memory");
+                 ::"r"(d_tmem), "l"(a_desc), "l"(b_desc), "r"(instr_desc), "r"(accumulate ? 1u : 0u) : "memory");
 }
 // Lets `bar` complete when the products this thread has issued so far are done.
 __device__ __forceinline__ void commit_one(unsigned long long* bar) {
@@ -579,6 +580,9 @@ spmm_kernel(const __grid_constant__ Params p, const __grid_constant__ CUtensorMa
                     ok = wait_parity(&sm.acc_free, (k - 1) & 1);
                     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
                 }
+                // the tile's tokens, in the units of the instruction
+                const int64_t left = p.N - static_cast<int64_t>(s.tile % p.nblocks) * F::kNI;
+                const uint32_t id = instr_desc(128, left < F::kNI ? static_cast<int>(left + 15) / 16 * 16 : F::kNI);
                 for (int kb = 0; ok && kb < s.n; ++kb) {
                     ok = wait_parity(&sm.x_full[sb], pb);                                       // the X tile is in place
                     for (int h = 0; ok && h < kSubs; ++h) {
@@ -591,9 +595,9 @@ spmm_kernel(const __grid_constant__ Params p, const __grid_constant__ CUtensorMa
                         for (int a = 0; a < 2; ++a) {                   // the two row halves
 #pragma unroll
                             for (int kk = 0; kk < kSub / 16; ++kk)      // the start address is the low field, in 16-byte units
-                                mma_f16_one<F::kNI, kDescHigh<kAChunkStride, 0u>, kDescHigh<kBAtomBytes, 2u>>(
+                                mma_f16_one<kDescHigh<kAChunkStride, 0u>, kDescHigh<kBAtomBytes, 2u>>(
                                     tmem + a * F::kNI, al + ((a * F::kATileBytes + kk * 2 * kAKGroupStride) >> 4), bl + ((kk * 32) >> 4),
-                                    kk > 0 ? 1u : add);
+                                    id, kk > 0 ? 1u : add);
                         }
                         commit_one(&sm.a_free[sa]);
                         issued = true;
@@ -744,19 +748,26 @@ constexpr int kNT = kNTiles * kNI;            // tokens per CTA pair
 constexpr int kStages = 3;                    // decoded W in flight
 constexpr int kMeta = 6;                      // stored K-blocks in flight, at most
 constexpr int kBTileBytes = (kNI / 2) * kBRowBytes;    // this CTA's 128 tokens of one X tile
-constexpr int kBBytes = kNTiles * kBTileBytes;
 static_assert(kNTiles * kNI == kTmemCols, "the accumulators fill tensor memory");
 
-// kXStages = X tiles in flight
-template <int kXStages>
+// X tiles in flight; a K-block has one for each accumulator.  With four of them each has barriers of its own, so that it is free again
+// half a K-block's products earlier than with its K-block, for which the products waited: a tile takes as long to come as the
+// products of a K-block.  us per call, by K-block -> by tile: 28672x8192 x 300 tokens at 50 % 236 -> 213, x 512 251 -> 226, x 1024
+// 406 -> 386, 11008x4096 x 1024 92.9 -> 88.5, 18944x4096 x 512 71.6 -> 67.5; called without a pause, 28672x8192 x 1024 at the power
+// limit 471 -> 455.  Six, for sparse layers, are handed on with their K-block: more barriers cost 3 % there (18944x4096 x 512
+// at 90 % 60.5 / 64.4), five instead of four gain nothing.
+template <int kXTiles>
+constexpr bool kByTile = kXTiles < 2 * kStages;
+template <int kXTiles>
 struct __align__(1024) Smem {
-    unsigned char B[kXStages][kBBytes];             // my halves of the X tiles (each on a 1024-byte boundary: swizzle atoms)
+    unsigned char B[kXTiles][kBTileBytes];          // my halves of the X tiles (each on a 1024-byte boundary: swizzle atoms)
     unsigned char A[kStages][kATileBytes];          // decoded W: my 128 rows
     Meta meta[kMeta];
-    alignas(8) unsigned long long mma_done[kStages];    // the tensor cores are done with A stage s and B stage s (both CTAs)
+    alignas(8) unsigned long long mma_done[kStages];    // the tensor cores are done with A stage s (both CTAs)
+    alignas(8) unsigned long long x_done[kXTiles];      // they are done with the X tile
+    alignas(8) unsigned long long x_full[kXTiles];      // my half of the X tile has arrived (first CTA: and the second CTA's)
     alignas(8) unsigned long long comp_free[kMeta];     // my decode warps are done with the stored K-block
-    alignas(8) unsigned long long ready[kStages];       // A stage s is written and my X tiles of B stage s have arrived
-                                                        // (first CTA: and the second CTA says the same of its own)
+    alignas(8) unsigned long long ready[kStages];       // A stage s is written (first CTA: and the second CTA's)
     alignas(8) unsigned long long comp_full[kMeta];     // the stored K-block has arrived
     alignas(16) uint2 tab[kWarps][32];              // per warp: bitmap word and the address of its first value
     uint32_t tmem_base;
@@ -766,20 +777,28 @@ struct __align__(1024) Smem {
                                                         // 28672x8192 x 1024 at 50 % 410 us, this 397
 };
 constexpr size_t kSmemBytes = 227 * 1024;               // the dynamic shared memory is aligned by hand
-template <int kXStages>
-constexpr uint32_t kRingBytes = (static_cast<uint32_t>(kSmemBytes) - 1024u - static_cast<uint32_t>(offsetof(Smem<kXStages>, ring)) - 64u) / 128u * 128u;
-// A third X tile in flight pays where the ring still holds four K-blocks beside it; where it does not, the decode waits for
+template <int kXTiles>
+constexpr uint32_t kRingBytes = (static_cast<uint32_t>(kSmemBytes) - 1024u - static_cast<uint32_t>(offsetof(Smem<kXTiles>, ring)) - 64u) / 128u * 128u;
+// A third X tile for each accumulator pays where the ring still holds four K-blocks beside it; where it does not, the decode waits for
 // copies instead.  us with 2 / 3 X tiles, 18944x3872 x 416 tokens at 67 %: 66 / 60; 18944x4096 x 512 at 90, 50, 30 %: 70 / 62,
 // 71 / 70, 74 / 85; 4096x4096 x 1024 at 50 %: 50 / 57.
 constexpr int64_t kThirdXBytes = 13 * 1024;             // bytes of values per K-block up to which there are three
 static_assert(kBTileBytes % 1024 == 0, "every X tile on a swizzle-atom boundary");
 
-template <int kXStages>
+struct XTile {                                          // place of an X tile in the ring of tiles, and its barriers' parity
+    unsigned at = 0, parity = 0;
+    template <int kXTiles>
+    __device__ __forceinline__ void next() {
+        if (++at == kXTiles) { at = 0; parity ^= 1u; }
+    }
+};
+
+template <int kXTiles>
 __global__ void __launch_bounds__(kThreads, 1)
 spmm_kernel(const __grid_constant__ Params p, const __grid_constant__ CUtensorMap xmap) {
-    static_assert(kRingBytes<kXStages> >= 2 * kKB * kTileM, "the ring holds at least one full K-block");
+    static_assert(kRingBytes<kXTiles> >= 2 * kKB * kTileM, "the ring holds at least one full K-block");
     extern __shared__ unsigned char smem_raw[];
-    Smem<kXStages>& sm = *reinterpret_cast<Smem<kXStages>*>(smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u));
+    Smem<kXTiles>& sm = *reinterpret_cast<Smem<kXTiles>*>(smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u));
     const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
     const int c = static_cast<int>(blockIdx.x & 1u);                  // my rank in the pair = my half of the row tile
     const unsigned pr = blockIdx.x >> 1;
@@ -789,14 +808,21 @@ spmm_kernel(const __grid_constant__ Params p, const __grid_constant__ CUtensorMa
     const int nb = static_cast<int>(tile - static_cast<unsigned>(r) * static_cast<unsigned>(p.nblocks));
     const int64_t n0 = static_cast<int64_t>(nb) * kNT;
     const int ntiles = (p.N - n0 > kNI) ? 2 : 1;                      // accumulators in use
+    // the last one's tokens, in the units of the instruction: half of them in each CTA's X tile
+    const int last_tokens = min(kNI, static_cast<int>((min(p.N - n0, static_cast<int64_t>(kNT)) - (ntiles - 1) * kNI + 31) / 32) * 32);
 
     // ---- set-up: the barriers, and tensor memory (both CTAs of the pair allocate together) ----
     if (t == 0) {
 #pragma unroll
         for (int s = 0; s < kStages; ++s) {
             barrier_init(&sm.mma_done[s], 1);
-            // arrivals on ready[]: my decode warps, my copy thread (with the X tiles' bytes), in the first CTA the second CTA
-            barrier_init(&sm.ready[s], kBlockWarps + 1 + (c == 0 ? 1 : 0));
+            // my decode warps, without barriers for X tiles my copy thread (with their bytes), in the first CTA the second CTA
+            barrier_init(&sm.ready[s], kBlockWarps + (kByTile<kXTiles> ? 0 : 1) + (c == 0 ? 1 : 0));
+        }
+#pragma unroll
+        for (int s = 0; s < kXTiles; ++s) {
+            barrier_init(&sm.x_done[s], 1);
+            barrier_init(&sm.x_full[s], 1 + (c == 0 ? 1 : 0));               // my copy thread (with the tile's bytes), in the first CTA the second CTA
         }
 #pragma unroll
         for (int s = 0; s < kMeta; ++s) {
@@ -832,33 +858,41 @@ spmm_kernel(const __grid_constant__ Params p, const __grid_constant__ CUtensorMa
         asm volatile("griddepcontrol.wait;" ::: "memory");
         if (one && c == 0) {
             // ================= tensor-core thread (first CTA): issues the K-blocks' products for the pair =================
+            XTile x;
             for (int kb = 0; kb < nkb; ++kb) {
                 const int s = kb % kStages;
-                if (ok) ok = wait_parity(&sm.ready[s], (kb / kStages) & 1);      // both CTAs' decoded W tiles and X tiles are in place
-                asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+                if (ok) ok = wait_parity(&sm.ready[s], (kb / kStages) & 1);          // both CTAs' decoded W is in place
                 const uint64_t ad0 = operand_desc(smem_u32(&sm.A[s][0]), kAKGroupStride, kAChunkStride, 0u);
-                const uint64_t bd0 = operand_desc(smem_u32(&sm.B[kb % kXStages][0]), 16, kBAtomBytes, 2u);
-                for (int i = 0; i < ntiles; ++i) {
+                for (int i = 0; i < ntiles; ++i, x.next<kXTiles>()) {
+                    if (kByTile<kXTiles> && ok) ok = wait_parity(&sm.x_full[x.at], x.parity);        // and both halves of the X tile
+                    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+                    const uint64_t bd0 = operand_desc(smem_u32(&sm.B[x.at][0]), 16, kBAtomBytes, 2u);
+                    const uint32_t id = instr_desc(256, i == ntiles - 1 ? last_tokens : kNI);
 #pragma unroll
                     for (int kk = 0; kk < kKB / 16; ++kk)    // the start address is the descriptor's low field, in 16-byte units
-                        mma_f16_pair<kNI>(tmem + i * kNI, ad0 + ((kk * 2 * kAKGroupStride) >> 4), bd0 + ((i * kBTileBytes + kk * 32) >> 4),
-                                     kb > 0 || kk > 0);
+                        mma_f16_pair(tmem + i * kNI, ad0 + ((kk * 2 * kAKGroupStride) >> 4), bd0 + ((kk * 32) >> 4), id, kb > 0 || kk > 0);
+                    if (kByTile<kXTiles>) commit_pair(&sm.x_done[x.at]);
                 }
                 commit_pair(&sm.mma_done[s]);
             }
         } else if (one) {
-            // ================= second CTA: tell the first when my tiles of a block are ready =================
+            // ================= second CTA: tell the first when my part of a block is ready =================
+            XTile x;
             for (int kb = 0; kb < nkb; ++kb) {
                 const int s = kb % kStages;
                 if (ok) ok = wait_parity(&sm.ready[s], (kb / kStages) & 1);
                 arrive_at(&sm.ready[s], 0u);
+                for (int i = 0; kByTile<kXTiles> && i < ntiles; ++i, x.next<kXTiles>()) {
+                    if (ok) ok = wait_parity(&sm.x_full[x.at], x.parity);
+                    arrive_at(&sm.x_full[x.at], 0u);
+                }
             }
         }
         __syncwarp();           // the other lanes wait here, not on a barrier in shared memory
     } else if (warp == kWarps + 1) {
         // ================= copy warp: moves the stored K-blocks =================
         CopyState cs;
-        ok = copy_blocks<kMeta>(p, cs, smem_u32(&sm.ring[0]), kRingBytes<kXStages>, sm.meta, sm.comp_full, sm.comp_free, &sm.abort,
+        ok = copy_blocks<kMeta>(p, cs, smem_u32(&sm.ring[0]), kRingBytes<kXTiles>, sm.meta, sm.comp_full, sm.comp_free, &sm.abort,
                                 static_cast<int64_t>(r) * p.C, kb0, nkb, lane, ok);
         ok = await_copies<kMeta>(cs, sm.comp_full) && ok;
         __syncwarp();
@@ -866,14 +900,21 @@ spmm_kernel(const __grid_constant__ Params p, const __grid_constant__ CUtensorMa
         // ================= X warp: one thread moves my halves of the X tiles =================
         if (elect_one()) {
             asm volatile("griddepcontrol.wait;" ::: "memory");          // X may come from the kernel before this one
-            for (int kb = 0; kb < nkb; ++kb) {
-                // my X tiles of block kb go where block kb - kXStages multiplied from, once that work is complete
-                const int s = kb % kStages, before = kb - kXStages;
-                if (before >= 0 && ok) ok = wait_parity(&sm.mma_done[before % kStages], (before / kStages) & 1);
-                expect_bytes(&sm.ready[s], static_cast<uint32_t>(ntiles) * kBTileBytes);
-                for (int i = 0; i < ntiles; ++i)            // my 128 tokens of each tile: one tiled bulk-tensor copy
-                    tensor_copy(&sm.B[kb % kXStages][i * kBTileBytes], &xmap, (kb0 + kb) * kKB, static_cast<int>(n0) + i * kNI + c * (kNI / 2), &sm.ready[s]);
-            }
+            XTile x;
+            for (int kb = 0; kb < nkb; ++kb)
+                for (int i = 0; i < ntiles; ++i, x.next<kXTiles>()) {       // my 128 tokens of each tile: one tiled bulk-tensor copy
+                    // it goes where the tile kXTiles before was multiplied from, once that work is complete
+                    unsigned long long* const full = kByTile<kXTiles> ? &sm.x_full[x.at] : &sm.ready[kb % kStages];
+                    if (kByTile<kXTiles>) {
+                        if (kb * ntiles + i >= kXTiles && ok) ok = wait_parity(&sm.x_done[x.at], x.parity ^ 1u);
+                        expect_bytes(full, kBTileBytes);
+                    } else if (i == 0) {
+                        if (kb >= kStages && ok) ok = wait_parity(&sm.mma_done[kb % kStages], ((kb / kStages) & 1u) ^ 1u);
+                        expect_bytes(full, static_cast<uint32_t>(ntiles) * kBTileBytes);
+                    }
+                    tensor_copy(&sm.B[x.at][0], &xmap, (kb0 + kb) * kKB, static_cast<int>(n0) + i * kNI + c * ((i == ntiles - 1 ? last_tokens : kNI) / 2),
+                                full);
+                }
         }
         __syncwarp();
     } else if (warp == kWarps + 2) {
@@ -881,8 +922,13 @@ spmm_kernel(const __grid_constant__ Params p, const __grid_constant__ CUtensorMa
         // one thread passes it on to the second CTA's =================
         if (lane == 0 && c == 0) {
             asm volatile("griddepcontrol.wait;" ::: "memory");
+            XTile x;
             for (int kb = 0; kb < nkb; ++kb) {
                 const int s = kb % kStages;
+                for (int i = 0; kByTile<kXTiles> && i < ntiles; ++i, x.next<kXTiles>()) {
+                    if (ok) ok = wait_parity(&sm.x_done[x.at], x.parity);
+                    arrive_at(&sm.x_done[x.at], 1u);
+                }
                 if (ok) ok = wait_parity(&sm.mma_done[s], (kb / kStages) & 1);
                 arrive_at(&sm.mma_done[s], 1u);
             }
@@ -977,8 +1023,8 @@ spdp_status configure_spmm_kernel() {
         SPDP_CUDA_TRY(cudaFuncSetAttribute(one::spmm_kernel<One32>, cudaFuncAttributeMaxDynamicSharedMemorySize, one::kSmemBytes));
         SPDP_CUDA_TRY(cudaFuncSetAttribute(one::spmm_kernel<One128>, cudaFuncAttributeMaxDynamicSharedMemorySize, one::kSmemBytes));
         SPDP_CUDA_TRY(cudaFuncSetAttribute(one::spmm_kernel<One256>, cudaFuncAttributeMaxDynamicSharedMemorySize, one::kSmemBytes));
-        SPDP_CUDA_TRY(cudaFuncSetAttribute(pair::spmm_kernel<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(pair::kSmemBytes)));
-        SPDP_CUDA_TRY(cudaFuncSetAttribute(pair::spmm_kernel<3>, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(pair::kSmemBytes)));
+        SPDP_CUDA_TRY(cudaFuncSetAttribute(pair::spmm_kernel<4>, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(pair::kSmemBytes)));
+        SPDP_CUDA_TRY(cudaFuncSetAttribute(pair::spmm_kernel<6>, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(pair::kSmemBytes)));
         configured[dev] = true;
     }
     return SPDP_OK;
@@ -1112,7 +1158,7 @@ spdp_status launch_pairs(const Params& p, const CUtensorMap& xmap, int64_t pairs
     attr[1].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 2;
-    SPDP_CUDA_TRY(cudaLaunchKernelEx(&cfg, block_bytes <= pair::kThirdXBytes ? pair::spmm_kernel<3> : pair::spmm_kernel<2>, p, xmap));
+    SPDP_CUDA_TRY(cudaLaunchKernelEx(&cfg, block_bytes <= pair::kThirdXBytes ? pair::spmm_kernel<6> : pair::spmm_kernel<4>, p, xmap));
     return SPDP_OK;
 }
 
