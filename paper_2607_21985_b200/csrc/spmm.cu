@@ -22,7 +22,8 @@
 // time, so that a warp's loads for 128 rows fall into at most 256 contiguous bytes: rank = set bits before the
 // nibble, three aligned 32-bit loads cover its at most 4 values wherever they start, two funnel shifts align
 // them, and two byte permutes with selectors computed from the nibble put them into their rows, one 8-byte store
-// per lane.  (A walk over the 8 rows of a bitmap byte with predicated 16-bit loads, as before, took twice the
+// per lane; the permute of rows 2 and 3 starts from the values shifted by what rows 0 and 1 have, so that either permute has a zero
+// word for clear rows.  (A walk over the 8 rows of a bitmap byte with predicated 16-bit loads, as before, took twice the
 // instructions, and 43-49 % of the shared-memory wavefronts were bank conflicts.)
 //
 //   one::   one CTA = one row tile (256 rows = two M = 128 accumulators) x up to 32, 128 or 256 tokens.  The CTAs stay for
@@ -241,7 +242,8 @@ __device__ __forceinline__ void scan4(const Params& p, const uint32_t (*bm)[8], 
 // half's tile, 16 bytes further the next column (at most 8: one k-group).  The loads of 4 steps are issued together; they
 // may reach 12 bytes past the stored values.  What bounds it is shared memory: 2 wavefronts for the table, one or two for
 // each value load, 2 for the store.  (Selectors from a 16-entry table in shared memory instead of the two multiplications
-// cost 2 more wavefronts per step and 3 % on the whole kernel.)
+// cost 2 more wavefronts per step and 3 % on the whole kernel.  Rows 2 and 3 selected from all four values and masked took two
+// instructions more: 8192x8192 x 64 tokens at 80 % 36.3 -> 35.3 us, 11008x4096 x 128 34.2 -> 33.5, 28672x8192 x 16 95.8 -> 93.0.)
 template <int kSteps, int kHalves>
 __device__ __forceinline__ void expand4(uint32_t tab_l, uint32_t a_dst, uint32_t half_bytes, unsigned below, unsigned top) {
     static_assert(kSteps % 4 == 0 && kSteps / kHalves <= 8, "4 steps at a time, one k-group");
@@ -265,11 +267,9 @@ __device__ __forceinline__ void expand4(uint32_t tab_l, uint32_t a_dst, uint32_t
         for (int q = 0; q < 4; ++q) {
             const unsigned mis = a[q] << 3;                     // 16 if the first value is an upper half (mod 32)
             const unsigned t0 = __funnelshift_r(s0[q], s1[q], mis), t1 = __funnelshift_r(s1[q], s2[q], mis);
-            // byte i: 0x22 * (set bits before row i) + 0x10 = the two byte selectors of row i's value
-            const unsigned sel = bits[q] * 0x22222200u + 0x10101010u;
-            const unsigned m = bits[q] * 0xFFu;
-            sts_v2(a_dst + ((q0 + q) % kHalves) * half_bytes + ((q0 + q) / kHalves) * 16u, permute(t0, 0u, bits[q] * 0x21CCu + 0x4444u),
-                   permute(t0, t1, sel >> 16) & permute(m, m, 0x3322u));
+            const unsigned t23 = __funnelshift_rc(t0, t1, __dp4a(bits[q], kShift23, 0u));       // the values from row 2 on
+            sts_v2(a_dst + ((q0 + q) % kHalves) * half_bytes + ((q0 + q) / kHalves) * 16u, permute(t0, 0u, bits[q] * kSelect01 + kSelectNone),
+                   permute(t23, 0u, __dp2a_hi(kSelect23, bits[q], kSelectNone)));
         }
     }
 }

@@ -142,15 +142,14 @@ template <bool kSparse>
 __device__ __forceinline__ void place_nibble(const Nibble<kSparse>& n, unsigned& r01, unsigned& r23) {
     const unsigned mis = n.a << 3;                                      // 16 if the first value is an upper half (mod 32)
     const unsigned t0 = __funnelshift_r(n.s0, n.s1, mis), t1 = __funnelshift_r(n.s1, n.s2, mis);
-    const unsigned sel = n.bits * 0x22222200u + 0x10101010u;            // byte i: the two byte selectors of row i's value
-    const unsigned m = n.bits * 0xFFu;
-    r01 = permute(t0, 0u, n.bits * 0x21CCu + 0x4444u);                  // rows 0, 1 need t0 alone: a clear row selects zero bytes
-    r23 = permute(t0, t1, sel >> 16) & permute(m, m, 0x3322u);
+    const unsigned t23 = __funnelshift_rc(t0, t1, __dp4a(n.bits, kShift23, 0u));        // the values from row 2 on
+    r01 = permute(t0, 0u, n.bits * kSelect01 + kSelectNone);            // two rows need one word: a clear row selects zero bytes
+    r23 = permute(t23, 0u, __dp2a_hi(kSelect23, n.bits, kSelectNone));
 }
 // The form for sparse layers: the two values that rows 0 and 1 may have and the two that rows 2 and 3 may have are loaded one by one,
 // whether they are there or not.  A 16-bit load leaves the upper half of its register zero, which is what a clear row selects, so that
-// nothing has to be aligned or masked: 18 instructions in place of 24 for 4 rows, 5 of them on the integer pipe in place of
-// 11, but one shared-memory access more, and those cost more the denser the layer is.
+// nothing has to be aligned: 18 instructions in place of 22 for 4 rows, 5 of them on the integer pipe in place of
+// 9, but one shared-memory access more, and those cost more the denser the layer is.
 template <>
 struct Nibble<true> { unsigned v0, v1, v2, v3, bits; };
 template <>

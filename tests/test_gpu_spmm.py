@@ -346,3 +346,23 @@ def test_spmm_cut_tiles_into_any_y(S, R, K, N, dt):
             assert bool((Y[:, M:] == 7.0).all()) and bool((buf[:at] == 7.0).all()) and bool((buf[at + N * (M + pad):] == 7.0).all())
     finally:
         S.spdp_free(h)
+
+
+@pytest.mark.parametrize("R,K", [(75, 1000), (3, 712)])
+def test_spmm_token_counts_around_the_instructions_units(S, R, K):
+    """The tensor-core instructions take a tile's tokens in units of 16 (one CTA) or 32 (CTA pairs, half of them in each CTA's shared
+    memory): token counts around those units, around the tiles and around the pairs' second accumulator.  Integers: exact."""
+    M = 256 * R - 100
+    g = torch.Generator(device="cuda").manual_seed(R)
+    W = torch.randint(-4, 5, (M, K), generator=g, device="cuda").half() * (torch.rand(M, K, generator=g, device="cuda") < 0.5)
+    h = S.spdp_pack_tiled_cbc(W)
+    try:
+        for N in (1, 15, 16, 17, 31, 32, 33, 127, 129, 145, 255, 256, 257, 272, 288, 289, 479, 481, 511, 513, 545, 768, 770):
+            X = torch.randint(-3, 4, (N, K), generator=g, device="cuda").half()
+            Y = torch.full((N, M), float("nan"), dtype=torch.float32, device="cuda")
+            S.spdp_spmm(h, X, Y)
+            torch.cuda.synchronize()
+            assert S.spdp_last_device_status(h) == 0
+            assert torch.equal(Y.double(), X.double() @ W.double().T), N            # |sums| <= 1000 * 12 < 2^24
+    finally:
+        S.spdp_free(h)
