@@ -93,7 +93,7 @@ spdp_status alloc_arrays(spdp_matrix* h, cudaStream_t s) {
     const size_t bitmap = place(cols * kWordsPerCol * sizeof(uint64_t)), colinfo = place(cols * sizeof(uint32_t)),
                  tileoffset = place((h->NGT + 1) * sizeof(uint32_t)), scales = place(h->q4 ? cols * sizeof(__half) : 0),
                  x = place(h->K * sizeof(__half)), mask = place((h->K + 31) / 32 * sizeof(uint32_t)), y = place(h->M * sizeof(float)),
-                 status = place(2 * sizeof(int));
+                 status = place(2 * sizeof(int) + 2 * sizeof(unsigned long long));
     spdp_status st = handle_alloc(h->device, at, &h->arrays);
     if (st != SPDP_OK) return st;
     char* base = static_cast<char*>(h->arrays.p);
@@ -105,7 +105,8 @@ spdp_status alloc_arrays(spdp_matrix* h, cudaStream_t s) {
     h->mask_stage = reinterpret_cast<uint32_t*>(base + mask);
     h->y_stage = base + y;
     h->status_word = reinterpret_cast<int*>(base + status);
-    SPDP_CUDA_TRY(cudaMemsetAsync(h->status_word, 0, 2 * sizeof(int), s));
+    h->pack_totals = reinterpret_cast<unsigned long long*>(h->status_word + 2);
+    SPDP_CUDA_TRY(cudaMemsetAsync(h->status_word, 0, 2 * sizeof(int) + 2 * sizeof(unsigned long long), s));
     return SPDP_OK;
 }
 
@@ -143,9 +144,7 @@ spdp_status build_partition(spdp_matrix* h, int num_ctas, cudaStream_t s) {
 
 // The rest of a handle's set-up; synchronises `s`.
 spdp_status finish_handle(spdp_matrix* h, cudaStream_t s) {
-    spdp_status st = build_partition(h, 0, s);
-    if (st != SPDP_OK) return st;
-    st = configure_spmspv_kernel();
+    spdp_status st = configure_spmspv_kernel();
     if (st != SPDP_OK) return st;
     st = configure_spmspv_batch_kernel();
     if (st != SPDP_OK) return st;
@@ -285,6 +284,7 @@ spdp_status spdp_pack_tiled_cbc_ex(const void* W_dev, int64_t M, int64_t K, int6
     spdp_status st = new_handle(M, K, pad_elems, &h);
     if (st != SPDP_OK) return st;
     st = alloc_arrays(h, static_cast<cudaStream_t>(stream));
+    if (st == SPDP_OK) st = build_partition(h, 0, static_cast<cudaStream_t>(stream));    // emptied before the kernels, not behind them
     if (st == SPDP_OK) st = pack_device(h, static_cast<const __half*>(W_dev), ldw, static_cast<cudaStream_t>(stream));
     if (st == SPDP_OK) st = finish_handle(h, static_cast<cudaStream_t>(stream));
     if (st != SPDP_OK) { release(h); return st; }
@@ -308,6 +308,7 @@ spdp_status spdp_pack_tiled_cbc_q4(const void* W_dev, int64_t M, int64_t K, int6
     if (st != SPDP_OK) return st;
     h->q4 = 1;
     st = alloc_arrays(h, static_cast<cudaStream_t>(stream));
+    if (st == SPDP_OK) st = build_partition(h, 0, static_cast<cudaStream_t>(stream));    // emptied before the kernels, not behind them
     if (st == SPDP_OK) st = pack_device(h, static_cast<const __half*>(W_dev), ldw, static_cast<cudaStream_t>(stream));
     if (st == SPDP_OK) st = finish_handle(h, static_cast<cudaStream_t>(stream));
     if (st != SPDP_OK) { release(h); return st; }
@@ -369,6 +370,7 @@ spdp_status spdp_import_tiled_cbc(int64_t M, int64_t K, int pad_elems, const voi
     auto body = [&]() -> spdp_status {
         cudaStream_t s = nullptr;
         spdp_status a = alloc_arrays(h, s);
+        if (a == SPDP_OK) a = build_partition(h, 0, s);
         if (a == SPDP_OK) a = handle_alloc(h->device, vbytes < 16 ? 16 : vbytes, &h->values_block);
         if (a != SPDP_OK) return a;
         h->values = static_cast<__half*>(h->values_block.p);
@@ -535,6 +537,7 @@ spdp_status spdp_row_shard(int64_t M, int world, int rank, int64_t* first_row_ou
 spdp_status spdp_free(spdp_handle h) {
     if (h == nullptr) {                     // no handle: give back the memory that freed handles left
         give_back_all();
+        give_back_pack_totals();
         return SPDP_OK;
     }
     if (!valid(h)) return SPDP_ERR_INVALID_ARG;

@@ -8,6 +8,8 @@
 // 11008x4096 at 60 % sparsity, each kernel alone with cold caches: count 28.9 -> 21.6 us, scan 9.3 -> 6.4, emit 45.4 -> 32.4, unpack
 // 46.2 -> 27.6; the bytes alone would take 14, 0, 20 and 20.  Pack, unpack and free together 173 -> 133 us (memory of freed
 // handles is kept, see memory.cu), the rest of it synchronisations.
+#include <mutex>
+
 #include "spdp_internal.h"
 #include "spmspv_device.cuh"
 
@@ -114,10 +116,11 @@ pack_count_kernel(const unsigned short* __restrict__ W, int64_t ldw, int64_t M, 
 }
 
 // Pass 2: exclusive scan of the padded GTile lengths into TileOffset (one CTA; a warp takes one contiguous part, its lanes
-// 4 neighbouring entries at a time).  total_out receives the 64-bit total.
+// 4 neighbouring entries at a time).  totals[0] receives the 64-bit total; it and the nonzeros in totals[1] also go to host_totals,
+// if there is such.
 __global__ void __launch_bounds__(1024)
 pack_scan_kernel(const uint32_t* __restrict__ tile_len, int64_t NGT, uint32_t* __restrict__ tileoffset,
-                 unsigned long long* __restrict__ total_out) {
+                 unsigned long long* __restrict__ totals, unsigned long long* host_totals) {
     __shared__ unsigned long long part[32];
     const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
     const int64_t per = (NGT + 4095) / 4096 * 128, lo = min(NGT, warp * per), hi = min(NGT, lo + per);
@@ -165,7 +168,11 @@ pack_scan_kernel(const uint32_t* __restrict__ tile_len, int64_t NGT, uint32_t* _
     }
     if (t == 0) {
         tileoffset[NGT] = static_cast<uint32_t>(total);
-        *total_out = total;
+        totals[0] = total;
+        if (host_totals != nullptr) {
+            host_totals[0] = total;
+            host_totals[1] = totals[1];
+        }
     }
 }
 
@@ -364,6 +371,63 @@ pack_q4_emit_kernel(const unsigned short* __restrict__ W, int64_t ldw, int64_t M
 
 }  // namespace
 
+namespace {
+
+// Page-locked words that the scan writes the totals of a pack call to, a pair for each call on its way, so that nothing has to be
+// copied (a copy to ordinary memory and its staging cost a call 6 us).  One allocation, made by the first call and freed by
+// spdp_free(NULL) when no call uses it; a call that finds no pair copies.
+struct HostTotals {
+    static constexpr int kPairs = 64;
+    std::mutex mu;
+    unsigned long long* words = nullptr;
+    int in_use = 0;
+    bool used[kPairs] = {};
+};
+HostTotals g_host_totals;
+
+class TotalsPair {
+    int pair_ = -1;
+    unsigned long long* words_ = nullptr;
+
+public:
+    TotalsPair() {
+        HostTotals& t = g_host_totals;
+        std::lock_guard<std::mutex> lock(t.mu);
+        void* p = nullptr;
+        if (t.words == nullptr) {
+            if (cudaHostAlloc(&p, HostTotals::kPairs * 2 * sizeof(unsigned long long), cudaHostAllocPortable | cudaHostAllocMapped) != cudaSuccess) {
+                cudaGetLastError();
+                return;
+            }
+            t.words = static_cast<unsigned long long*>(p);
+        }
+        for (int i = 0; i < HostTotals::kPairs && pair_ < 0; ++i)
+            if (!t.used[i]) pair_ = i;
+        if (pair_ < 0) return;
+        t.used[pair_] = true;
+        ++t.in_use;
+        words_ = t.words + 2 * pair_;
+    }
+    ~TotalsPair() {
+        if (pair_ < 0) return;
+        std::lock_guard<std::mutex> lock(g_host_totals.mu);
+        g_host_totals.used[pair_] = false;
+        --g_host_totals.in_use;
+    }
+    TotalsPair(const TotalsPair&) = delete;
+    TotalsPair& operator=(const TotalsPair&) = delete;
+    unsigned long long* words() const { return words_; }       // null: none to be had.  The same address on the device
+};
+
+}  // namespace
+
+void give_back_pack_totals() {
+    std::lock_guard<std::mutex> lock(g_host_totals.mu);
+    if (g_host_totals.in_use > 0 || g_host_totals.words == nullptr) return;
+    if (cudaFreeHost(g_host_totals.words) != cudaSuccess) cudaGetLastError();
+    g_host_totals.words = nullptr;
+}
+
 // Count and scan, then the emit pass of the handle's variant (fp16 values, or 4-bit codes with scales).  The arrays whose
 // sizes follow from the shape are allocated already; the length of Values is known after the scan, which is what the one
 // synchronisation in the middle is for.  The caller synchronises after the emit pass.
@@ -372,19 +436,22 @@ spdp_status pack_device(spdp_matrix* h, const __half* W, int64_t ldw, cudaStream
     const unsigned short* Wb = reinterpret_cast<const unsigned short*>(W);
     const int blocks = static_cast<int>((h->C + kGT - 1) / kGT);
     const unsigned grid = static_cast<unsigned>(h->R * blocks);
-    uint32_t* tile_len = nullptr;
-    unsigned long long* total_dev = nullptr;               // [0] Values length, [1] nnz
-    spdp_status st = handle_alloc(h->device, 2 * sizeof(unsigned long long) + NGT * sizeof(uint32_t), &h->packing);
+    spdp_status st = handle_alloc(h->device, NGT * sizeof(uint32_t), &h->packing);
     if (st != SPDP_OK) return st;
-    total_dev = static_cast<unsigned long long*>(h->packing.p);
-    tile_len = reinterpret_cast<uint32_t*>(total_dev + 2);
+    uint32_t* tile_len = static_cast<uint32_t*>(h->packing.p);
+    unsigned long long* total_dev = h->pack_totals;        // [0] Values length, [1] nnz; both zero so far
     unsigned long long totals[2] = {0, 0};
-    SPDP_CUDA_TRY(cudaMemsetAsync(total_dev, 0, 2 * sizeof(unsigned long long), s));
+    const TotalsPair host;
     pack_count_kernel<<<grid, kTileM, 0, s>>>(Wb, ldw, h->M, h->K, h->C, blocks, h->pad_elems, h->bitmap, h->colinfo, tile_len,
                                               total_dev + 1);
-    pack_scan_kernel<<<1, 1024, 0, s>>>(tile_len, NGT, h->tileoffset, total_dev);
-    SPDP_CUDA_TRY(cudaMemcpyAsync(totals, total_dev, sizeof(totals), cudaMemcpyDeviceToHost, s));
-    SPDP_CUDA_TRY(cudaStreamSynchronize(s));
+    pack_scan_kernel<<<1, 1024, 0, s>>>(tile_len, NGT, h->tileoffset, total_dev, host.words());
+    const cudaError_t launched = cudaGetLastError();
+    if (host.words() == nullptr && launched == cudaSuccess)
+        SPDP_CUDA_TRY(cudaMemcpyAsync(totals, total_dev, sizeof(totals), cudaMemcpyDeviceToHost, s));
+    SPDP_CUDA_TRY(cudaStreamSynchronize(s));               // behind it nothing writes the words any more
+    SPDP_CUDA_TRY(launched);
+    if (host.words() != nullptr)
+        for (int i = 0; i < 2; ++i) totals[i] = static_cast<volatile unsigned long long*>(host.words())[i];
     if (totals[0] >= (1ull << 32)) return SPDP_ERR_OVERFLOW;
     h->values_len = static_cast<int64_t>(totals[0]);
     h->nnz = static_cast<int64_t>(totals[1]);

@@ -50,8 +50,9 @@ struct spdp_matrix {
     float* workspace;       // device [P*256] split-K tree nodes, one row per CTA (all zero between calls)
     float* workspace_batch; // device [P*8*256] tree nodes of the small-batch call (all zero between calls)
     spdp::DeviceBlock workspace_block;  // both
-    spdp::DeviceBlock packing;          // lengths and totals while packing
+    spdp::DeviceBlock packing;          // lengths of the GTiles while packing
     int* status_word;       // device [2]: the status word, and a sink word the benchmark probes may write
+    unsigned long long* pack_totals;    // device [2]: length of Values and nonzeros, counted while packing
     int64_t workspace_bytes;
 
     // Staging for the host-vector entry point
@@ -117,6 +118,7 @@ spdp_status scratch_alloc(int device, size_t bytes, cudaStream_t s, void** out);
 // pack.cu
 spdp_status pack_device(spdp_matrix* h, const __half* W, int64_t ldw, cudaStream_t s);     // either variant
 spdp_status unpack_device(const spdp_matrix* h, __half* W, int64_t ldw, cudaStream_t s);
+void give_back_pack_totals();                  // page-locked words of the pack calls, if none is on its way
 
 // spmspv.cu
 int default_ctas_per_sm();   // CTAs of the spMspV kernel that share one SM
