@@ -106,6 +106,25 @@ def _check(st: int, where: str):
 
 
 _raw_stream = _device = None
+_f16 = _f32 = None          # torch.float16, torch.float32: an import statement in every call costs more than its checks
+
+
+def _load_dtypes():
+    global _f16, _f32
+    import torch
+    _f16, _f32 = torch.float16, torch.float32
+
+
+def _ydt(y):
+    """The output type that y's dtype selects."""
+    if _f16 is None:
+        _load_dtypes()
+    t = y.dtype
+    if t is _f16:
+        return SPDP_Y_F16
+    if t is _f32:
+        return SPDP_Y_F32
+    return None
 
 
 def _stream(stream):
@@ -208,13 +227,13 @@ def spdp_import_tiled_cbc(M: int, K: int, tileoffset, colinfo, bitmap, values, p
 
 def spdp_spmspv(h: int, x, rule: int, thr: float, y, mask=None, stream=None) -> None:
     """x: fp16 CUDA [K]; y: fp16 or fp32 CUDA [M] (its dtype selects the output type)."""
-    import torch
-    ydt = SPDP_Y_F32 if y.dtype == torch.float32 else SPDP_Y_F16
-    if y.dtype not in (torch.float16, torch.float32) or x.dtype != torch.float16:
+    ydt = _ydt(y)
+    if ydt is None or x.dtype is not _f16:
         raise ValueError("x must be fp16 and y fp16 or fp32")
-    st = lib().call_spmspv(h, _dev_ptr(x, "x"), rule, float(thr), _dev_ptr(mask, "mask", True), _dev_ptr(y, "y"),
-                           ydt, _stream(stream))
-    _check(st, "spdp_spmspv")
+    st = (_lib or lib()).call_spmspv(h, _dev_ptr(x, "x"), rule, float(thr), None if mask is None else _dev_ptr(mask, "mask"),
+                                     _dev_ptr(y, "y"), ydt, _stream(stream))
+    if st:
+        _check(st, "spdp_spmspv")
 
 
 def spdp_spmspv_host(h: int, x_host, rule: int, thr: float, y_host, mask_host=None, stream=None) -> None:
@@ -245,33 +264,33 @@ def spdp_spmspv_noalloc(tileoffset, colinfo, bitmap, values, M: int, K: int, x, 
 def spdp_spmspv_batch(h: int, X, rule: int, thr: float, Y, mask=None, stream=None) -> None:
     """Small-batch call: X fp16 CUDA [B][K] (rows may be strided), Y fp16 or fp32 CUDA [B][M], 1 <= B <= 8;
     mask (SPDP_DP_MASK only) int32/uint32 CUDA [B][>= ceil(K/32)] words."""
-    import torch
-    if X.dim() != 2 or Y.dim() != 2 or X.shape[0] != Y.shape[0]:
+    xs, ys = X.shape, Y.shape
+    if len(xs) != 2 or len(ys) != 2 or xs[0] != ys[0]:
         raise ValueError("X must be [B][K] and Y [B][M]")
-    if Y.dtype not in (torch.float16, torch.float32) or X.dtype != torch.float16:
+    ydt = _ydt(Y)
+    if ydt is None or X.dtype is not _f16:
         raise ValueError("X must be fp16 and Y fp16 or fp32")
-    if X.stride(1) != 1 or Y.stride(1) != 1 or (mask is not None and (mask.dim() != 2 or mask.stride(1) != 1)):
+    (ldx, cx), (ldy, cy) = X.stride(), Y.stride()
+    if cx != 1 or cy != 1 or (mask is not None and (mask.dim() != 2 or mask.stride(1) != 1)):
         raise ValueError("the last dimension of X, Y and mask must be contiguous")
-    ydt = SPDP_Y_F32 if Y.dtype == torch.float32 else SPDP_Y_F16
-    B = int(X.shape[0])
-    ldx = int(X.stride(0)) if B > 1 else int(X.shape[1])
-    ldy = int(Y.stride(0)) if B > 1 else int(Y.shape[1])
+    B = xs[0]
+    if B <= 1:
+        ldx, ldy = xs[1], ys[1]
     mstride = 0 if mask is None else (int(mask.stride(0)) if B > 1 else int(mask.shape[1]))
     if not X.is_cuda or not Y.is_cuda or (mask is not None and not mask.is_cuda):
         raise ValueError("X, Y and mask must be CUDA tensors")
-    st = lib().call_spmspv_batch(h, X.data_ptr(), ldx, B, rule, float(thr),
-                                 None if mask is None else mask.data_ptr(), mstride, Y.data_ptr(), ldy, ydt,
-                                 _stream(stream))
-    _check(st, "spdp_spmspv_batch")
+    st = (_lib or lib()).call_spmspv_batch(h, X.data_ptr(), ldx, B, rule, float(thr), None if mask is None else mask.data_ptr(), mstride,
+                                           Y.data_ptr(), ldy, ydt, _stream(stream))
+    if st:
+        _check(st, "spdp_spmspv_batch")
 
 
 def spdp_spmm(h: int, X, Y, stream=None) -> None:
     """Prefill call: X fp16 CUDA [N][K] (rows may be strided), Y fp16 or fp32 CUDA [N][M]."""
-    import torch
-    xs, ys, ytype = X.shape, Y.shape, Y.dtype            # each attribute once: 512x512 x 32 tokens, bound by the host, 8.3 -> 7.4 us
+    xs, ys, ydt = X.shape, Y.shape, _ydt(Y)              # each attribute once: 512x512 x 32 tokens, bound by the host, 8.3 -> 7.4 us
     if len(xs) != 2 or len(ys) != 2 or xs[0] != ys[0] or not X.is_cuda or not Y.is_cuda:
         raise ValueError("X must be CUDA [N][K] and Y CUDA [N][M]")
-    if ytype not in (torch.float16, torch.float32) or X.dtype != torch.float16:
+    if ydt is None or X.dtype is not _f16:
         raise ValueError("X must be fp16 and Y fp16 or fp32")
     (ldx, cx), (ldy, cy) = X.stride(), Y.stride()
     if cx != 1 or cy != 1:
@@ -279,16 +298,18 @@ def spdp_spmm(h: int, X, Y, stream=None) -> None:
     N = xs[0]
     if N <= 1:
         ldx, ldy = max(xs[1], ldx), max(ys[1], ldy)
-    ydt = SPDP_Y_F32 if ytype == torch.float32 else SPDP_Y_F16
-    _check(lib().call_spmm(h, X.data_ptr(), N, ldx, Y.data_ptr(), ldy, ydt, _stream(stream)), "spdp_spmm")
+    st = (_lib or lib()).call_spmm(h, X.data_ptr(), N, ldx, Y.data_ptr(), ldy, ydt, _stream(stream))
+    if st:
+        _check(st, "spdp_spmm")
 
 
 def spdp_swiglu_dp(gate, up, thr: float, x_out, mask_out, count_out=None, stream=None) -> None:
     """x_out = silu(gate) * up (fp16 CUDA [K]) and the K-bit keep-mask of its columns in one pass."""
-    K = int(gate.shape[0])
-    st = lib().call_swiglu_dp(_dev_ptr(gate, "gate"), _dev_ptr(up, "up"), K, float(thr), _dev_ptr(x_out, "x_out"),
-                              _dev_ptr(mask_out, "mask_out"), _dev_ptr(count_out, "count_out", True), _stream(stream))
-    _check(st, "spdp_swiglu_dp")
+    st = (_lib or lib()).call_swiglu_dp(_dev_ptr(gate, "gate"), _dev_ptr(up, "up"), gate.shape[0], float(thr), _dev_ptr(x_out, "x_out"),
+                                        _dev_ptr(mask_out, "mask_out"), None if count_out is None else _dev_ptr(count_out, "count_out"),
+                                        _stream(stream))
+    if st:
+        _check(st, "spdp_swiglu_dp")
 
 
 def spdp_row_shard(M: int, world: int, rank: int):
