@@ -274,14 +274,44 @@ __device__ __forceinline__ void expand4(uint32_t tab_l, uint32_t a_dst, uint32_t
     }
 }
 
+// Turns 4 values of each of 4 neighbouring lanes: lane l's v[i] becomes what lane (l & ~3) + i had in v[l & 3].
+__device__ __forceinline__ void transpose4(uint32_t& v0, uint32_t& v1, uint32_t& v2, uint32_t& v3, int lane) {
+    const bool odd = (lane & 1) != 0, upper = (lane & 2) != 0;
+    const uint32_t a = __shfl_xor_sync(0xFFFFFFFFu, odd ? v0 : v1, 1), b = __shfl_xor_sync(0xFFFFFFFFu, odd ? v2 : v3, 1);
+    if (odd) { v0 = a; v2 = b; } else { v1 = a; v3 = b; }
+    const uint32_t c = __shfl_xor_sync(0xFFFFFFFFu, upper ? v0 : v2, 2), d = __shfl_xor_sync(0xFFFFFFFFu, upper ? v1 : v3, 2);
+    if (upper) { v0 = c; v1 = d; } else { v2 = c; v3 = d; }
+}
+// May 4 consecutive rows of a token, the first a multiple of 4, be stored to Y at once?
+__device__ __forceinline__ bool y_in_fours(const Params& p) {
+    const unsigned size = p.ydt == SPDP_Y_F32 ? 4u : 2u;
+    return (p.ldy & 3) == 0 && (reinterpret_cast<uintptr_t>(p.Y) & (4u * size - 1u)) == 0;
+}
+__device__ __forceinline__ void store_four(void* Y, int ydt, int64_t at, float a, float b, float c, float d) {
+    if (ydt == SPDP_Y_F32) {
+        *reinterpret_cast<float4*>(static_cast<float*>(Y) + at) = make_float4(a, b, c, d);
+    } else {
+        const __half2 lo = __floats2half2_rn(a, b), hi = __floats2half2_rn(c, d);
+        *reinterpret_cast<uint2*>(static_cast<__half*>(Y) + at) = make_uint2(*reinterpret_cast<const unsigned*>(&lo), *reinterpret_cast<const unsigned*>(&hi));
+    }
+}
+
 // Accumulators of one tile: tensor-memory lanes [lane_base, +32) x columns [c_begin, c_end) of the tile's tokens (first
 // token n0).  A thread holds one row, 16 tokens at a time, so a warp's stores of one token are 32 consecutive rows.  With
-// slot >= 0 they go, as fp32, into that slot of the scratch memory instead of Y.  The whole warp calls this together.
+// slot >= 0 they go, as fp32, into that slot of the scratch memory instead of Y.  The whole warp calls this together; row_in is its first
+// row's.  kFours: four neighbouring threads trade values first, so that each stores 4 rows of every fourth token at once, where Y allows it (a
+// store of 32 single values costs as much as one of 32 fours): CTA pairs, which store whole tiles more often than not, 28672x8192 x 300
+// tokens 207.8 -> 203.2 us, 18944x4096 x 512 65.5 -> 64.0, 3000x700 x 1024 16.7 -> 15.9.  The one-CTA forms mostly leave partial sums, whose
+// stores gain nothing by it, and are 1 to 2 % slower with the longer code.
+template <bool kFours>
 __device__ __forceinline__ void store_accumulators(const Params& p, uint32_t tmem, int lane_base, int c_begin, int c_end,
                                                    int r, int row_in, int64_t n0, int slot) {
-    const int64_t row = static_cast<int64_t>(r) * kTileM + row_in;
+    const int lane = threadIdx.x & 31;
     const int valid = static_cast<int>(min(p.N - n0, static_cast<int64_t>(c_end)));
-    float* part = p.partial + (static_cast<size_t>(slot < 0 ? 0 : slot) * p.ptok) * kTileM + row_in;
+    const int64_t row0 = static_cast<int64_t>(r) * kTileM + row_in;
+    const bool fours = kFours && slot < 0 && y_in_fours(p) && row0 + 32 <= p.M;
+    const int64_t row = row0 + (fours ? lane & ~3 : lane);
+    float* part = p.partial + (static_cast<size_t>(slot < 0 ? 0 : slot) * p.ptok) * kTileM + row_in + lane;
     for (int c0 = c_begin; c0 < valid; c0 += 16) {
         uint32_t v[16];
         asm volatile("tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%16];"
@@ -289,7 +319,16 @@ __device__ __forceinline__ void store_accumulators(const Params& p, uint32_t tme
                        "=r"(v[8]), "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]), "=r"(v[14]), "=r"(v[15])
                      : "r"(tmem + (static_cast<uint32_t>(lane_base) << 16) + c0) : "memory");
         asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-        if (slot >= 0) {
+        if (kFours && fours) {
+#pragma unroll
+            for (int i = 0; i < 16; i += 4) {
+                transpose4(v[i], v[i + 1], v[i + 2], v[i + 3], lane);
+                const int tok = c0 + i + (lane & 3);
+                if (tok < valid)
+                    store_four(p.Y, p.ydt, (n0 + tok) * p.ldy + row, __uint_as_float(v[i]), __uint_as_float(v[i + 1]), __uint_as_float(v[i + 2]),
+                               __uint_as_float(v[i + 3]));
+            }
+        } else if (slot >= 0) {
 #pragma unroll
             for (int i = 0; i < 16; ++i)
                 if (c0 + i < valid) part[static_cast<size_t>(c0 + i) * kTileM] = __uint_as_float(v[i]);
@@ -318,20 +357,38 @@ __device__ __forceinline__ void void_rows(const Params& p, int slot, int row0, i
 // fixed grid a thread took 320 instructions, most of them 64-bit divisions behind that wait.)  us per call, before -> now:
 // 1024x1024 x 64 tokens 10.4 -> 8.8, 2048x2048 x 128 15.2 -> 13.2, 4096x11008 x 128 31.2 -> 29.4, 11008x4096 x 128 35.4 -> 33.9.
 constexpr int kReduceTokens = 4;
+// Sums that a thread has on their way at once.  A layer of few row tiles is cut into dozens of pieces a tile for a handful of blocks, which
+// wait for one load behind the other.  us per call with four / eight: 1024x11008 x 64 tokens (37 pieces a tile) 19.7 / 17.2, 1024x1024 x 64
+// (16) 8.9 / 7.8, 4096x4096 x 128 (9) 18.0 / 17.3.  Sixteen are longer code, fetched for the first time in every call: 4096x4096 x 16
+// tokens 11.6 -> 13.8.
+constexpr int kFewSums = 4, kManySums = 8, kManySumsFrom = 8;
 // Adds the partial sums of 4 rows at `first` and, count - 1 of them and `stride` floats apart, from `next` on, in this order, and
 // stores them at token n, rows row .. row + 3.
+template <int kDepth>
 __device__ __forceinline__ void add_partials(const Params& p, const float* first, const float* next, size_t stride, int count, int64_t n, int64_t row) {
     float4 sum = __ldcg(reinterpret_cast<const float4*>(first));
     bool there = __float_as_uint(sum.w) != kNoSum;                   // no CTA of the tile gave up
-#pragma unroll 4
-    for (int i = 1; i < count; ++i) {
-        const float4 v = __ldcg(reinterpret_cast<const float4*>(next));
-        next += stride;
+    const auto add = [&](const float4& v) {
         there = there && __float_as_uint(v.w) != kNoSum;
         sum.x += v.x;
         sum.y += v.y;
         sum.z += v.z;
         sum.w += v.w;
+    };
+    if constexpr (kDepth == kFewSums) {
+#pragma unroll kFewSums
+        for (int i = 1; i < count; ++i, next += stride) add(__ldcg(reinterpret_cast<const float4*>(next)));
+    } else {
+#pragma unroll 1
+        for (int left = count - 1; left > 0; left -= kDepth, next += kDepth * stride) {
+            float4 v[kDepth];
+#pragma unroll
+            for (int i = 0; i < kDepth; ++i)
+                if (i < left) v[i] = __ldcg(reinterpret_cast<const float4*>(next + i * stride));
+#pragma unroll
+            for (int i = 0; i < kDepth; ++i)
+                if (i < left) add(v[i]);
+        }
     }
     if (!there) return;
     const int64_t at = n * p.ldy + row;
@@ -691,8 +748,8 @@ spmm_kernel(const __grid_constant__ Params p, const __grid_constant__ CUtensorMa
             if (ok && !__any_sync(0xFFFFFFFFu, *static_cast<volatile int*>(&sm.abort) != 0)) {
                 // warp w: row half (w / 4) % 2, tensor-memory lanes 32 * (w % 4).., token columns [(w / 8) * kNI / 2, + kNI / 2)
                 const int half = (warp >> 2) & 1, cbase = (warp >> 3) * (F::kNI / 2), lane_base = 32 * (warp & 3);
-                store_accumulators(p, tmem + half * F::kNI, lane_base, cbase, cbase + F::kNI / 2, s.tile / p.nblocks,
-                                   half * 128 + lane_base + lane, static_cast<int64_t>(s.tile % p.nblocks) * F::kNI, s.slot);
+                store_accumulators<false>(p, tmem + half * F::kNI, lane_base, cbase, cbase + F::kNI / 2, s.tile / p.nblocks,
+                                   half * 128 + lane_base, static_cast<int64_t>(s.tile % p.nblocks) * F::kNI, s.slot);
             }
             asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
             __syncwarp();
@@ -717,6 +774,7 @@ spmm_kernel(const __grid_constant__ Params p, const __grid_constant__ CUtensorMa
 }
 
 // Adds, in CTA order, the partial sums of the tiles that several CTAs fed, and writes their part of Y.
+template <int kDepth>
 __global__ void __launch_bounds__(256)
 reduce_pieces_kernel(const Params p, int tile0, int chunks, int tile_tokens) {
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
@@ -731,7 +789,7 @@ reduce_pieces_kernel(const Params p, int tile0, int chunks, int tile_tokens) {
     const float* sums = p.partial + static_cast<size_t>(tok) * kTileM + row_in;
     asm volatile("griddepcontrol.wait;" ::: "memory");          // (every thread: the kernel after this one relies on it)
     if (first == last || tok >= p.ptok || n >= p.N || row >= p.M) return;        // a tile that one CTA had is stored already
-    add_partials(p, sums + first_slot * slot, sums + 2u * (first + 1u) * slot, 2u * slot, static_cast<int>(last - first) + 1, n, row);
+    add_partials<kDepth>(p, sums + first_slot * slot, sums + 2u * (first + 1u) * slot, 2u * slot, static_cast<int>(last - first) + 1, n, row);
 }
 
 }  // namespace one
@@ -976,7 +1034,7 @@ spmm_kernel(const __grid_constant__ Params p, const __grid_constant__ CUtensorMa
     // ---- epilogue.  Warp w reads lanes 32*(w%4).. (my rows 32*(w%4)..), token columns [(w/4)*128, +128) of the 512 ----
     if (!*static_cast<volatile int*>(&sm.abort) && warp < kStoreWarps) {
         const int lane_base = 32 * (warp & 3), cbase = (warp >> 2) * (kNT / 4);
-        store_accumulators(p, tmem, lane_base, cbase, cbase + kNT / 4, r, c * 128 + lane_base + lane, n0,
+        store_accumulators<true>(p, tmem, lane_base, cbase, cbase + kNT / 4, r, c * 128 + lane_base, n0,
                            p.partial == nullptr ? -1 : static_cast<int>(pr));
     } else if (*static_cast<volatile int*>(&sm.abort) && p.partial != nullptr) {
         void_rows(p, static_cast<int>(pr), c * 128, 128, t, kThreads);
@@ -989,6 +1047,7 @@ spmm_kernel(const __grid_constant__ Params p, const __grid_constant__ CUtensorMa
 }
 
 // Adds the K-slices of the tiles that were cut along K, in slice order, and writes their part of Y.
+template <int kDepth>
 __global__ void __launch_bounds__(256)
 reduce_slices_kernel(const Params p, int chunks) {
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
@@ -1001,7 +1060,7 @@ reduce_slices_kernel(const Params p, int chunks) {
     const float* sums = p.partial + static_cast<size_t>(t) * p.kslices * slot + static_cast<size_t>(tok) * kTileM + row_in;
     asm volatile("griddepcontrol.wait;" ::: "memory");
     if (tok >= p.ptok || n >= p.N || row >= p.M) return;
-    add_partials(p, sums, sums + slot, slot, p.kslices, n, row);
+    add_partials<kDepth>(p, sums, sums + slot, slot, p.kslices, n, row);
 }
 
 }  // namespace pair
@@ -1194,6 +1253,7 @@ spdp_status run_plan(const spdp_matrix* h, Params p, const Plan& plan, const __h
         if (st != SPDP_OK) return st;
     }
     const int chunks = (p.ptok + kReduceTokens - 1) / kReduceTokens;
+    const bool many = plan.sharers >= kManySumsFrom * plan.rest;             // sums a tile
     if (plan.kernel == 3) {
         const int64_t block_bytes = 2 * h->values_len / (h->R * p.nkb);      // values of an average K-block
         Params whole = p;                                                    // whole tiles first, then the last tiles cut along K
@@ -1203,7 +1263,7 @@ spdp_status run_plan(const spdp_matrix* h, Params p, const Plan& plan, const __h
             p.tile0 = static_cast<int>(plan.tiles - plan.rest);
             p.kslices = plan.slices;
             st = launch_pairs(p, xmap, plan.rest * plan.slices, block_bytes, s);
-            if (st == SPDP_OK) st = launch_reduce(pair::reduce_slices_kernel, plan.rest, chunks, s, p, chunks);
+            if (st == SPDP_OK) st = launch_reduce(many ? pair::reduce_slices_kernel<kManySums> : pair::reduce_slices_kernel<kFewSums>, plan.rest, chunks, s, p, chunks);
         }
     } else {
         p.workers = plan.workers;
@@ -1212,7 +1272,7 @@ spdp_status run_plan(const spdp_matrix* h, Params p, const Plan& plan, const __h
         p.rest_units = static_cast<unsigned>(plan.rest * p.nkb);
         st = plan.kernel == 0 ? launch_one<One32>(p, xmap, s) : plan.kernel == 1 ? launch_one<One128>(p, xmap, s) : launch_one<One256>(p, xmap, s);
         if (st == SPDP_OK && cut)
-            st = launch_reduce(one::reduce_pieces_kernel, plan.rest, chunks, s, p, plan.rounds * plan.workers, chunks, nt);
+            st = launch_reduce(many ? one::reduce_pieces_kernel<kManySums> : one::reduce_pieces_kernel<kFewSums>, plan.rest, chunks, s, p, plan.rounds * plan.workers, chunks, nt);
     }
     if (cut) cudaFreeAsync(p.partial, s);
     return st;
