@@ -40,6 +40,7 @@
 #include <cstddef>
 #include <mutex>
 
+#include "nibble_place.cuh"
 #include "spdp_internal.h"
 #include "spmspv_device.cuh"
 

@@ -132,12 +132,6 @@ __device__ __forceinline__ unsigned threshold_pair(float thr) {
 __device__ __forceinline__ unsigned nibble_top(unsigned i) { return 1u << (28u - 4u * i); }
 __device__ __forceinline__ unsigned nibble_below(unsigned i) { return i ? 1u << (32u - 4u * i) : 0u; }
 
-// Placing a nibble's values in its four rows, with bit i of the nibble in byte i of `bits`.  Two rows are one byte permute of a
-// word of two values with a zero word; its selectors, the first row's in the low byte: 0x44 (zero bytes) for a clear row, 0x10 for the
-// first set one, 0x32 for the second.  bits * kSelect01 + kSelectNone has them for rows 0 and 1, dp2a_hi(kSelect23, bits, kSelectNone)
-// for rows 2 and 3, whose word starts dp4a(bits, kShift23, 0) bits (16 for each value of rows 0 and 1) behind the others'.
-constexpr unsigned kSelectNone = 0x4444u, kSelect01 = 0x21CCu, kSelect23 = 0xCC0021CCu, kShift23 = 0x00001010u;
-
 // Active-column list of a batch (Sec. 4.2 steps (1)-(3)).  List positions [0, nlist) hold the columns of piece A
 // ([0, nA)), then, if `two`, from vB0 (a multiple of 64) those of piece B.  keep(v) tests the two columns at positions v
 // and v + 1 (v even, also beyond the list's end) and answers in bits 0 and 31; write(item, v, k0, k1, inB) stores the records
