@@ -60,6 +60,10 @@ constexpr int kKB = 64;                // columns per K-block: one 128-byte swiz
 constexpr int kSub = 32;               // columns per sub-block
 constexpr int kSubs = kKB / kSub;
 constexpr int kGTB = kKB / kTileK;     // GTiles per K-block
+// Shared memory of a CTA, of the 227 KB that it could have: a block of the second kernel needs 1 KB beside it.  With all of it taken the second
+// kernel of a cut call can start only where a CTA has left: 8192x8192 x 16 tokens 32.0 -> 29.5 us, 11008x4096 x 16 25.4 -> 24.6,
+// 3000x700 x 64 9.23 -> 8.86; most other calls the same.
+constexpr int kSmemKB = 225;
 constexpr int kBlockWarps = kSubs * kGroupWarps;      // warps that decode a K-block
 static_assert(kSub == 4 * kGroupWarps, "a scan takes 4 columns");
 static_assert(kWarps >= kStoreWarps, "16 warps store");
@@ -511,7 +515,7 @@ struct Form {
         // X tiles are small: 4096x4096 x 16 tokens 13.0 -> 11.7 us, 28672x8192 x 16 99.9 -> 95.6 (with 128 tokens five stages and two
         // X tiles gained nothing).
     static constexpr int kBStages = kNI <= 128 ? 3 : 2;
-    static constexpr int kMeta = 8;                                   // stored K-blocks in flight, at most
+    static constexpr int kMeta = kNI <= 128 ? 8 : 6;                  // stored K-blocks in flight, at most
     static_assert(kBBytes % 1024 == 0, "every X tile on a swizzle-atom boundary");
     static_assert(kAStages >= 2 * kSubs && kAStages >= kGroups, "the first two K-blocks fit in the first A stages, and every decode warp has a sub-block among the next kAStages");
 };
@@ -573,7 +577,7 @@ struct __align__(1024) Smem {
     alignas(128) unsigned char ring[1];             // values of the K-blocks in flight (fills the rest): the sparser the
                                                     // matrix, the more K-blocks are on their way
 };
-constexpr uint32_t kSmemBytes = 227u * 1024u;       // the dynamic shared memory is aligned by hand
+constexpr uint32_t kSmemBytes = kSmemKB * 1024u;    // the dynamic shared memory is aligned by hand
 template <class F>
 constexpr uint32_t kRingBytes = (kSmemBytes - 1024u - static_cast<uint32_t>(offsetof(Smem<F>, ring)) - 64u) / 128u * 128u;
 
@@ -835,7 +839,7 @@ struct __align__(1024) Smem {
                                                         // stages of a full K-block's size the decode waited for copies:
                                                         // 28672x8192 x 1024 at 50 % 410 us, this 397
 };
-constexpr size_t kSmemBytes = 227 * 1024;               // the dynamic shared memory is aligned by hand
+constexpr size_t kSmemBytes = kSmemKB * 1024;           // the dynamic shared memory is aligned by hand
 template <int kXTiles>
 constexpr uint32_t kRingBytes = (static_cast<uint32_t>(kSmemBytes) - 1024u - static_cast<uint32_t>(offsetof(Smem<kXTiles>, ring)) - 64u) / 128u * 128u;
 // A third X tile for each accumulator pays where the ring still holds four K-blocks beside it; where it does not, the decode waits for
