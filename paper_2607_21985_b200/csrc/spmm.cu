@@ -42,6 +42,7 @@
 
 #include "nibble_place.cuh"
 #include "spdp_internal.h"
+#include "spmm_plan.h"
 #include "spmspv_device.cuh"
 
 namespace spdp {
@@ -842,10 +843,6 @@ struct __align__(1024) Smem {
 constexpr size_t kSmemBytes = kSmemKB * 1024;           // the dynamic shared memory is aligned by hand
 template <int kXTiles>
 constexpr uint32_t kRingBytes = (static_cast<uint32_t>(kSmemBytes) - 1024u - static_cast<uint32_t>(offsetof(Smem<kXTiles>, ring)) - 64u) / 128u * 128u;
-// A third X tile for each accumulator pays where the ring still holds four K-blocks beside it; where it does not, the decode waits for
-// copies instead.  us with 2 / 3 X tiles, 18944x3872 x 416 tokens at 67 %: 66 / 60; 18944x4096 x 512 at 90, 50, 30 %: 70 / 62,
-// 71 / 70, 74 / 85; 4096x4096 x 1024 at 50 %: 50 / 57.
-constexpr int64_t kThirdXBytes = 13 * 1024;             // bytes of values per K-block up to which there are three
 static_assert(kBTileBytes % 1024 == 0, "every X tile on a swizzle-atom boundary");
 
 struct XTile {                                          // place of an X tile in the ring of tiles, and its barriers' parity
@@ -1125,68 +1122,12 @@ spdp_status encode_x(CUtensorMap* map, const __half* X, int64_t N, int64_t K, in
     return SPDP_OK;
 }
 
-// How a call is cut.  kernel 0, 1, 2: 32, 128 or 256 tokens per CTA, `workers` CTAs, `rounds` whole rounds of tiles, the
-// K-blocks of the `rest` tiles after them cut into `sharers` ranges.  kernel 3: CTA pairs, 512 tokens, all tiles but the last
-// `rest` whole, those cut into `slices` slices each (sharers = rest * slices).
-struct Plan {
-    double us;
-    int kernel;
-    int workers, rounds, sharers, slices;
-    int64_t tiles, rest;
-};
-// The estimate of a call's time: (K-blocks of the busiest CTA) x (time of a K-block) + a tile's start and end + what the
-// partial sums cost.  Fitted to the four kernels' times, calls in a row on a stream, on 10 layers from 512x512 to 28672x8192
-// (30 to 80 % sparse) with 16 to 1024 tokens each.  Measured again over those 80 calls, the form that is chosen is 0.6 % behind the best form on
-// average, 8 % at worst (512x512 x 16 tokens, 8.3 against 7.6 us).  (Fitted to graph replays, where the CTA pairs' plain launch costs nothing, it took pairs for small layers, and cuts that
-// cross tiles as readily as those that do not: 1024x1024 x 32 tokens 14.4 -> 8.3 us, 2048x2048 x 64 16.5 -> 12.8, 4096x4096 x
-// 128 22.9 -> 19.6, x 16 17.7 -> 14.8, 4096x11008 x 128 34.0 -> 31.4, 4001x4098 x 200 30.8 -> 26.3.)
-constexpr double kCallUs[4] = {3.0, 3.7, 3.2, 6.5};                     // a call's fixed part
-constexpr double kBlockUs[4] = {0.88, 0.97, 1.22, 0.69};                // a K-block (64 columns x 256 rows), us
-constexpr double kBlockTokenUs[4] = {8.3e-4, 1.8e-4, 0.0, 4.8e-4};      // and per token of the tile
-constexpr double kTileUs = 2.1, kTileTokenUs = 2.3e-3;                  // a tile's start and end, and per token
-constexpr double kReduceUs = 1.9, kReducePerMB = 0.223;                 // the second kernel; writing and reading a MB of partial sums
-constexpr int kTokens[4] = {One32::kNI, One128::kNI, One256::kNI, pair::kNT};
-
-Plan make_plan(int64_t R, int64_t nkb, int64_t N, int sms, bool may_cut) {
-    Plan best = {};
-    best.us = -1.0;
-    for (int f = 0; f < 4; ++f) {
-        Plan q = {};
-        q.kernel = f;
-        q.tiles = R * ((N + kTokens[f] - 1) / kTokens[f]);
-        const int64_t slots = f == 3 ? sms / 2 : sms;                            // CTAs or pairs resident at once
-        const int64_t rounds = q.tiles / slots, left = q.tiles - rounds * slots;
-        const double tok = static_cast<double>(std::min<int64_t>(N, kTokens[f])), mb = tok * kTileM * 4.0e-6;   // MB of a tile's sums
-        const double block = kBlockUs[f] + kBlockTokenUs[f] * tok, tile = kTileUs + kTileTokenUs * tok;
-        const double whole = kCallUs[f] + (block * static_cast<double>(nkb) + tile) * static_cast<double>(rounds);
-        q.rounds = static_cast<int>(rounds);
-        q.slices = 1;
-        q.sharers = left > 0 ? static_cast<int>(left) : 1;
-        q.workers = static_cast<int>(rounds > 0 ? slots : left);
-        q.rest = f == 3 ? 0 : left;
-        q.us = whole + (left > 0 ? block * static_cast<double>(nkb) + tile : 0.0);
-        if (best.us < 0.0 || q.us < best.us) best = q;
-        if (left == 0 || !may_cut) continue;
-        const auto consider = [&](int64_t w) {                                   // w CTAs (pairs) share the tiles that are left
-            if (f == 3) {
-                q.slices = static_cast<int>(std::min<int64_t>(w / left, nkb));
-                w = q.slices * left;
-                q.rest = left;
-            }
-            if (w <= left || w > left * nkb) return;
-            q.sharers = static_cast<int>(w);
-            q.workers = static_cast<int>(rounds > 0 ? slots : w);
-            // a CTA whose range crosses into the next tile starts and ends two
-            q.us = whole + block * static_cast<double>((left * nkb + w - 1) / w) + tile * (w % left ? 2.0 : 1.0) + kReduceUs +
-                   kReducePerMB * mb * static_cast<double>(w + left);
-            if (q.us < best.us) best = q;
-        };
-        for (int64_t share = 2 * left; share < slots; share *= 2) consider(share);
-        consider(slots / left * left);                                           // the most that do not cross tiles
-        if (f != 3) consider(slots);
-    }
-    return best;
-}
+using plan::kTokens;
+using plan::make_plan;
+using plan::pair_x_tiles;
+using plan::Plan;
+static_assert(plan::kTileRows == kTileM && kTokens[0] == One32::kNI && kTokens[1] == One128::kNI && kTokens[2] == One256::kNI && kTokens[3] == pair::kNT,
+              "the plan counts in the kernels' tiles");
 
 template <class F>
 spdp_status launch_one(const Params& p, const CUtensorMap& xmap, cudaStream_t s) {
@@ -1207,7 +1148,7 @@ spdp_status launch_one(const Params& p, const CUtensorMap& xmap, cudaStream_t s)
 // Programmatic launch for the pairs too: a call's set-up, first copies and first three decoded K-blocks overlap the kernel before.
 // us per call, calls in a row: 4001x4098 x 300 tokens 32.8 -> 28.7, 4096x4096 x 300 28.7 -> 25.3, x 1024 48.1 -> 44.6, 11008x4096 x 300
 // 60.3 -> 56.6.
-spdp_status launch_pairs(const Params& p, const CUtensorMap& xmap, int64_t pairs, int64_t block_bytes, cudaStream_t s) {
+spdp_status launch_pairs(const Params& p, const CUtensorMap& xmap, int64_t pairs, int x_tiles, cudaStream_t s) {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(static_cast<unsigned>(2 * pairs));
     cfg.blockDim = dim3(pair::kThreads);
@@ -1222,7 +1163,7 @@ spdp_status launch_pairs(const Params& p, const CUtensorMap& xmap, int64_t pairs
     attr[1].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 2;
-    SPDP_CUDA_TRY(cudaLaunchKernelEx(&cfg, block_bytes <= pair::kThirdXBytes ? pair::spmm_kernel<6> : pair::spmm_kernel<4>, p, xmap));
+    SPDP_CUDA_TRY(cudaLaunchKernelEx(&cfg, x_tiles == 6 ? pair::spmm_kernel<6> : pair::spmm_kernel<4>, p, xmap));
     return SPDP_OK;
 }
 
@@ -1260,14 +1201,14 @@ spdp_status run_plan(const spdp_matrix* h, Params p, const Plan& plan, const __h
     const int chunks = (p.ptok + kReduceTokens - 1) / kReduceTokens;
     const bool many = plan.sharers >= kManySumsFrom * plan.rest;             // sums a tile
     if (plan.kernel == 3) {
-        const int64_t block_bytes = 2 * h->values_len / (h->R * p.nkb);      // values of an average K-block
+        const int x_tiles = pair_x_tiles(h->values_len, h->R, p.nkb);
         Params whole = p;                                                    // whole tiles first, then the last tiles cut along K
         whole.partial = nullptr;
-        if (plan.tiles > plan.rest) st = launch_pairs(whole, xmap, plan.tiles - plan.rest, block_bytes, s);
+        if (plan.tiles > plan.rest) st = launch_pairs(whole, xmap, plan.tiles - plan.rest, x_tiles, s);
         if (st == SPDP_OK && cut) {
             p.tile0 = static_cast<int>(plan.tiles - plan.rest);
             p.kslices = plan.slices;
-            st = launch_pairs(p, xmap, plan.rest * plan.slices, block_bytes, s);
+            st = launch_pairs(p, xmap, plan.rest * plan.slices, x_tiles, s);
             if (st == SPDP_OK) st = launch_reduce(many ? pair::reduce_slices_kernel<kManySums> : pair::reduce_slices_kernel<kFewSums>, plan.rest, chunks, s, p, chunks);
         }
     } else {
