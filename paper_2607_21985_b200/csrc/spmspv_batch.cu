@@ -18,6 +18,7 @@
 
 #include "nibble_place.cuh"
 #include "spdp_internal.h"
+#include "spmspv_batch_form.h"
 #include "spmspv_device.cuh"
 
 namespace spdp {
@@ -503,10 +504,6 @@ spdp_status configure_spmspv_batch_kernel() {
     return SPDP_OK;
 }
 
-// Layers whose average column tile holds at most this many values take the form with 16-bit loads.  us, aligned words / 16-bit loads,
-// at 60, 70, 80 and 90 % sparsity (102, 77, 51, 26 values): 28672x8192 x 8 tokens 96.0 / 102.6, 93.3 / 93.4, 92.1 / 85.7, 91.8 / 83.7;
-// 4096x4096 x 8 13.9 / 14.1, 13.5 / 13.3, 13.1 / 12.4, 13.0 / 12.2; 11008x4096 x 3 25.3 / 26.0, 24.7 / 24.3, 23.9 / 22.5, 23.6 / 22.0.
-constexpr int64_t kSparseValues = 80;
 spdp_status launch_spmspv_batch(const spdp_matrix* h, const __half* x, int64_t ldx, int batch, int rule, float thr,
                                 const uint32_t* mask, int64_t mask_stride, void* y, int64_t ldy, int ydt,
                                 cudaStream_t s) {
@@ -544,7 +541,7 @@ spdp_status launch_spmspv_batch(const spdp_matrix* h, const __half* x, int64_t l
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    const bool sparse = h->nnz <= kSparseValues * h->R * h->K;
+    const bool sparse = plan::batch_loads_one_by_one(h->nnz, h->M, h->K);
     SPDP_CUDA_TRY(cudaLaunchKernelEx(&cfg, sparse ? spmspv_batch_kernel<true> : spmspv_batch_kernel<false>, p));
     return SPDP_OK;
 }

@@ -1,5 +1,5 @@
-"""The batch kernel has two forms of its expansion, chosen by the values of an average column tile (80 of 256, rows beyond the
-matrix counted as clear): the 16-bit loads up to it, aligned words above.  Both sides of that line, and columns from empty to full in
+"""The batch kernel has two forms of its expansion, chosen by the values that a full column tile of average density has (of
+256): 16-bit loads up to 80, aligned words above.  Both sides of that line, and columns from empty to full in
 either form, give exact sums on integers; values that are not finite read the same in both."""
 import numpy as np
 import pytest
@@ -33,7 +33,9 @@ def test_both_forms_exact_on_integers(values, M, K, B):
         S.spdp_free(h)
 
 
-LINE = 80               # values of an average column tile up to which the 16-bit loads are taken
+def line(M, K):
+    """The most values of a layer that takes the 16-bit loads."""
+    return 80 * M * K // 256
 
 
 @pytest.mark.parametrize("beyond", [0, 1])
@@ -51,7 +53,7 @@ def test_exactly_at_the_line(beyond, M, K, B):
     fixed = np.zeros(K, bool)
     fixed[rng.permutation(K)[:K // 5]] = True
     counts[:, fixed] = np.where(rng.random((R, fixed.sum())) < 0.5, 0, np.array(rows)[:, None])
-    want_nnz = LINE * R * K + beyond
+    want_nnz = line(M, K) + beyond
     while (d := want_nnz - int(counts.sum())) != 0:                     # the other columns make up the rest
         r, k = rng.integers(R), rng.integers(K)
         if not fixed[k]:
@@ -65,7 +67,7 @@ def test_exactly_at_the_line(beyond, M, K, B):
     want = X.astype(np.float64) @ W.astype(np.float64).T                # |sums| <= 1001 * 32 < 2^24: exact in fp32
     h = S.spdp_pack_tiled_cbc(torch.from_numpy(W).cuda())
     try:
-        assert (S.spdp_get_info(h).nnz > LINE * R * K) == bool(beyond) and S.spdp_get_info(h).nnz == want_nnz
+        assert S.spdp_get_info(h).nnz == want_nnz
         for ctas in (0, 2):
             S.spdp_set_num_ctas(h, ctas)
             Y = torch.full((B, M), float("nan"), dtype=torch.float32, device="cuda")
@@ -97,7 +99,7 @@ def test_non_finite_values_in_both_forms(density):
     want = np.where(np.isfinite(X), X, 0).astype(np.float64) @ finite.T
     h = S.spdp_pack_tiled_cbc(torch.from_numpy(W).cuda())
     try:
-        assert (S.spdp_get_info(h).nnz <= LINE * 2 * K) == (density < 0.3)
+        assert (S.spdp_get_info(h).nnz <= line(M, K)) == (density < 0.3)
         Y = torch.zeros((B, M), dtype=torch.float32, device="cuda")
         S.spdp_spmspv_batch(h, torch.from_numpy(X).cuda(), rule, thr, Y)
         torch.cuda.synchronize()

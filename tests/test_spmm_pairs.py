@@ -32,9 +32,9 @@ INTO_ANY_Y = (148, 712, 300)
 
 @pytest.fixture(scope="module")
 def plan(tmp_path_factory):
-    out = tmp_path_factory.mktemp("plan") / "libspmm_plan_shim.so"
+    out = tmp_path_factory.mktemp("plan") / "libplan_shim.so"
     subprocess.run(["g++", "-O1", "-shared", "-fPIC", "-I", os.path.join(ROOT, "paper_2607_21985_b200", "csrc"),
-                    "-o", str(out), os.path.join(ROOT, "tests", "spmm_plan_shim.cpp")], check=True)
+                    "-o", str(out), os.path.join(ROOT, "tests", "plan_shim.cpp")], check=True)
     L = ctypes.CDLL(str(out))
     L.shim_make_plan.argtypes = [ctypes.c_longlong] * 3 + [ctypes.c_int] * 2 + [ctypes.c_void_p]
     L.shim_pair_x_tiles.argtypes = [ctypes.c_longlong] * 3
