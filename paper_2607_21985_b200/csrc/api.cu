@@ -93,7 +93,7 @@ spdp_status alloc_arrays(spdp_matrix* h, cudaStream_t s) {
     const size_t bitmap = place(cols * kWordsPerCol * sizeof(uint64_t)), colinfo = place(cols * sizeof(uint32_t)),
                  tileoffset = place((h->NGT + 1) * sizeof(uint32_t)), scales = place(h->q4 ? cols * sizeof(__half) : 0),
                  x = place(h->K * sizeof(__half)), mask = place((h->K + 31) / 32 * sizeof(uint32_t)), y = place(h->M * sizeof(float)),
-                 status = place(2 * sizeof(int) + 2 * sizeof(unsigned long long));
+                 status = place(2 * sizeof(int) + kPackTotals * sizeof(unsigned long long));
     spdp_status st = handle_alloc(h->device, at, &h->arrays);
     if (st != SPDP_OK) return st;
     char* base = static_cast<char*>(h->arrays.p);
@@ -106,7 +106,7 @@ spdp_status alloc_arrays(spdp_matrix* h, cudaStream_t s) {
     h->y_stage = base + y;
     h->status_word = reinterpret_cast<int*>(base + status);
     h->pack_totals = reinterpret_cast<unsigned long long*>(h->status_word + 2);
-    SPDP_CUDA_TRY(cudaMemsetAsync(h->status_word, 0, 2 * sizeof(int) + 2 * sizeof(unsigned long long), s));
+    SPDP_CUDA_TRY(cudaMemsetAsync(h->status_word, 0, 2 * sizeof(int) + kPackTotals * sizeof(unsigned long long), s));
     return SPDP_OK;
 }
 
@@ -348,7 +348,7 @@ spdp_status spdp_import_tiled_cbc(int64_t M, int64_t K, int pad_elems, const voi
     const uint32_t* ci = static_cast<const uint32_t*>(colinfo_host);
     const uint64_t* bm = static_cast<const uint64_t*>(bitmap_host);
     // Structural validation of the arrays (Sec. 4.1): offsets are prefix sums of the padded counts.
-    int64_t nnz = 0;
+    int64_t nnz = 0, uneven = 0;
     bool ok = (to[0] == 0) && (static_cast<int64_t>(to[h->NGT]) == values_len);
     for (int64_t g = 0; ok && g < h->NGT; ++g) {
         int64_t off = 0;
@@ -360,11 +360,14 @@ spdp_status spdp_import_tiled_cbc(int64_t M, int64_t K, int pad_elems, const voi
             if (static_cast<int64_t>(ci[slot] >> 16) != off || pc != n) { ok = false; break; }
             off += (n + pad_elems - 1) / pad_elems * pad_elems;
             nnz += n;
+            const int64_t column = g % h->C * kTileK + cc, diff = n - static_cast<int64_t>(ci[slot ^ 1] & 0xFFFFu);
+            if ((column | 1) < K) uneven += diff * diff;
         }
         if (ok && static_cast<int64_t>(to[g + 1]) - static_cast<int64_t>(to[g]) != off) ok = false;
     }
     if (!ok) { release(h); return SPDP_ERR_INVALID_ARG; }
     h->nnz = nnz;
+    h->uneven = uneven;
     h->values_len = values_len;
     const size_t vbytes = static_cast<size_t>(values_len) * sizeof(__half);
     auto body = [&]() -> spdp_status {

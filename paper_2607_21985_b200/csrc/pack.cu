@@ -71,13 +71,14 @@ __device__ __forceinline__ uint32_t stored_halves(uint32_t v) {
     return r;
 }
 
-// Pass 1: bitmap words, per-column nonzero counts, ColInfo, padded length of each GTile.  A lane collects the bits of its two
+// Pass 1: bitmap words, per-column nonzero counts, ColInfo, padded length of each GTile; sums[0] gets the nonzeros, sums[1] what
+// plan::batch_loads_one_by_one wants to know of the columns' differences.  A lane collects the bits of its two
 // columns over the 32 rows of its warp, one comparison and one logic operation for two elements; nothing is staged and
 // nothing is exchanged until the words are there.
 __global__ void __launch_bounds__(kTileM)
 pack_count_kernel(const unsigned short* __restrict__ W, int64_t ldw, int64_t M, int64_t K, int64_t C, int blocks,
                   int pad_elems, uint64_t* __restrict__ bitmap, uint32_t* __restrict__ colinfo,
-                  uint32_t* __restrict__ tile_len, unsigned long long* __restrict__ nnz_total) {
+                  uint32_t* __restrict__ tile_len, unsigned long long* __restrict__ sums) {
     __shared__ uint32_t words[kCols][kWords + 1];
     const int64_t r = blockIdx.x / static_cast<unsigned>(blocks), cb = blockIdx.x % static_cast<unsigned>(blocks);
     const int64_t g0 = r * C + cb * kGT;
@@ -110,14 +111,19 @@ pack_count_kernel(const unsigned short* __restrict__ W, int64_t ldw, int64_t M, 
             colinfo[g0 * kTileK + t] = ((end - padded) << 16) | n;
             if ((t & (kTileK - 1)) == kTileK - 1) tile_len[g0 + t / kTileK] = end;
         }
+        const int diff = static_cast<int>(n) - static_cast<int>(__shfl_xor_sync(0xFFFFFFFFu, n, 1));
         const unsigned sum = __reduce_add_sync(0xFFFFFFFFu, n);
-        if (lane == 0 && sum) atomicAdd(nnz_total, static_cast<unsigned long long>(sum));
+        const unsigned uneven = __reduce_add_sync(0xFFFFFFFFu, cb * kCols + (t | 1) < K ? static_cast<unsigned>(diff * diff) : 0u);
+        if (lane == 0 && sum) {
+            atomicAdd(sums, static_cast<unsigned long long>(sum));
+            if (uneven) atomicAdd(sums + 1, static_cast<unsigned long long>(uneven));
+        }
     }
 }
 
 // Pass 2: exclusive scan of the padded GTile lengths into TileOffset (one CTA; a warp takes one contiguous part, its lanes
-// 4 neighbouring entries at a time).  totals[0] receives the 64-bit total; it and the nonzeros in totals[1] also go to host_totals,
-// if there is such.
+// 4 neighbouring entries at a time).  totals[0] receives the 64-bit total; it and the sums of the first pass in totals[1] and [2] also
+// go to host_totals, if there is such.
 __global__ void __launch_bounds__(1024)
 pack_scan_kernel(const uint32_t* __restrict__ tile_len, int64_t NGT, uint32_t* __restrict__ tileoffset,
                  unsigned long long* __restrict__ totals, unsigned long long* host_totals) {
@@ -172,6 +178,7 @@ pack_scan_kernel(const uint32_t* __restrict__ tile_len, int64_t NGT, uint32_t* _
         if (host_totals != nullptr) {
             host_totals[0] = total;
             host_totals[1] = totals[1];
+            host_totals[2] = totals[2];
         }
     }
 }
@@ -373,49 +380,49 @@ pack_q4_emit_kernel(const unsigned short* __restrict__ W, int64_t ldw, int64_t M
 
 namespace {
 
-// Page-locked words that the scan writes the totals of a pack call to, a pair for each call on its way, so that nothing has to be
+// Page-locked words that the scan writes the totals of a pack call to, three for each call on its way, so that nothing has to be
 // copied (a copy to ordinary memory and its staging cost a call 6 us).  One allocation, made by the first call and freed by
-// spdp_free(NULL) when no call uses it; a call that finds no pair copies.
+// spdp_free(NULL) when no call uses it; a call that finds none free copies.
 struct HostTotals {
-    static constexpr int kPairs = 64;
+    static constexpr int kSlots = 64;
     std::mutex mu;
     unsigned long long* words = nullptr;
     int in_use = 0;
-    bool used[kPairs] = {};
+    bool used[kSlots] = {};
 };
 HostTotals g_host_totals;
 
-class TotalsPair {
-    int pair_ = -1;
+class TotalsSlot {
+    int slot_ = -1;
     unsigned long long* words_ = nullptr;
 
 public:
-    TotalsPair() {
+    TotalsSlot() {
         HostTotals& t = g_host_totals;
         std::lock_guard<std::mutex> lock(t.mu);
         void* p = nullptr;
         if (t.words == nullptr) {
-            if (cudaHostAlloc(&p, HostTotals::kPairs * 2 * sizeof(unsigned long long), cudaHostAllocPortable | cudaHostAllocMapped) != cudaSuccess) {
+            if (cudaHostAlloc(&p, HostTotals::kSlots * kPackTotals * sizeof(unsigned long long), cudaHostAllocPortable | cudaHostAllocMapped) != cudaSuccess) {
                 cudaGetLastError();
                 return;
             }
             t.words = static_cast<unsigned long long*>(p);
         }
-        for (int i = 0; i < HostTotals::kPairs && pair_ < 0; ++i)
-            if (!t.used[i]) pair_ = i;
-        if (pair_ < 0) return;
-        t.used[pair_] = true;
+        for (int i = 0; i < HostTotals::kSlots && slot_ < 0; ++i)
+            if (!t.used[i]) slot_ = i;
+        if (slot_ < 0) return;
+        t.used[slot_] = true;
         ++t.in_use;
-        words_ = t.words + 2 * pair_;
+        words_ = t.words + kPackTotals * slot_;
     }
-    ~TotalsPair() {
-        if (pair_ < 0) return;
+    ~TotalsSlot() {
+        if (slot_ < 0) return;
         std::lock_guard<std::mutex> lock(g_host_totals.mu);
-        g_host_totals.used[pair_] = false;
+        g_host_totals.used[slot_] = false;
         --g_host_totals.in_use;
     }
-    TotalsPair(const TotalsPair&) = delete;
-    TotalsPair& operator=(const TotalsPair&) = delete;
+    TotalsSlot(const TotalsSlot&) = delete;
+    TotalsSlot& operator=(const TotalsSlot&) = delete;
     unsigned long long* words() const { return words_; }       // null: none to be had.  The same address on the device
 };
 
@@ -439,9 +446,9 @@ spdp_status pack_device(spdp_matrix* h, const __half* W, int64_t ldw, cudaStream
     spdp_status st = handle_alloc(h->device, NGT * sizeof(uint32_t), &h->packing);
     if (st != SPDP_OK) return st;
     uint32_t* tile_len = static_cast<uint32_t*>(h->packing.p);
-    unsigned long long* total_dev = h->pack_totals;        // [0] Values length, [1] nnz; both zero so far
-    unsigned long long totals[2] = {0, 0};
-    const TotalsPair host;
+    unsigned long long* total_dev = h->pack_totals;        // [0] Values length, [1] nnz, [2] unevenness; all zero so far
+    unsigned long long totals[kPackTotals] = {};
+    const TotalsSlot host;
     pack_count_kernel<<<grid, kTileM, 0, s>>>(Wb, ldw, h->M, h->K, h->C, blocks, h->pad_elems, h->bitmap, h->colinfo, tile_len,
                                               total_dev + 1);
     pack_scan_kernel<<<1, 1024, 0, s>>>(tile_len, NGT, h->tileoffset, total_dev, host.words());
@@ -451,10 +458,11 @@ spdp_status pack_device(spdp_matrix* h, const __half* W, int64_t ldw, cudaStream
     SPDP_CUDA_TRY(cudaStreamSynchronize(s));               // behind it nothing writes the words any more
     SPDP_CUDA_TRY(launched);
     if (host.words() != nullptr)
-        for (int i = 0; i < 2; ++i) totals[i] = static_cast<volatile unsigned long long*>(host.words())[i];
+        for (int i = 0; i < kPackTotals; ++i) totals[i] = static_cast<volatile unsigned long long*>(host.words())[i];
     if (totals[0] >= (1ull << 32)) return SPDP_ERR_OVERFLOW;
     h->values_len = static_cast<int64_t>(totals[0]);
     h->nnz = static_cast<int64_t>(totals[1]);
+    h->uneven = static_cast<int64_t>(totals[2]);
     if (h->q4) {
         const size_t cbytes = static_cast<size_t>(totals[0]) / 2 + 16;     // + 16: the decode reads one word past a span
         spdp_status a = handle_alloc(h->device, cbytes, &h->values_block);

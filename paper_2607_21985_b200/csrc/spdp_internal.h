@@ -12,6 +12,7 @@ namespace spdp {
 constexpr int kTileM = 256;        // rows per column tile (Sec. 4.1)
 constexpr int kTileK = 16;         // column tiles per GTile (Sec. 4.2.3)
 constexpr int kWordsPerCol = 4;    // 64-bit bitmap words per column tile (Sec. 4.1)
+constexpr int kPackTotals = 3;     // sums over a layer that packing hands to the host
 constexpr uint64_t kMagic = 0x5350445042323030ull;   // "SPDPB200"
 
 // A piece of device memory that a handle owns (memory.cu).
@@ -32,6 +33,7 @@ struct spdp_matrix {
     int64_t M, K, R, C, NGT;
     int pad_elems;
     int64_t nnz;
+    int64_t uneven;         // see plan::batch_loads_one_by_one
     int64_t values_len;
 
     // Tiled-CBC arrays (device).  `arrays` is the allocation that holds every array whose size follows from the shape:
@@ -52,7 +54,7 @@ struct spdp_matrix {
     spdp::DeviceBlock workspace_block;  // both
     spdp::DeviceBlock packing;          // lengths of the GTiles while packing
     int* status_word;       // device [2]: the status word, and a sink word the benchmark probes may write
-    unsigned long long* pack_totals;    // device [2]: length of Values and nonzeros, counted while packing
+    unsigned long long* pack_totals;    // device [kPackTotals]: length of Values, nonzeros and unevenness, counted while packing
     int64_t workspace_bytes;
 
     // Staging for the host-vector entry point

@@ -541,7 +541,7 @@ spdp_status launch_spmspv_batch(const spdp_matrix* h, const __half* x, int64_t l
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    const bool sparse = plan::batch_loads_one_by_one(h->nnz, h->M, h->K);
+    const bool sparse = plan::batch_loads_one_by_one(h->nnz, h->uneven, h->M, h->K);
     SPDP_CUDA_TRY(cudaLaunchKernelEx(&cfg, sparse ? spmspv_batch_kernel<true> : spmspv_batch_kernel<false>, p));
     return SPDP_OK;
 }

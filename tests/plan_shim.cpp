@@ -9,4 +9,6 @@ extern "C" void shim_make_plan(long long R, long long nkb, long long N, int sms,
     for (int i = 0; i < 7; ++i) out[i] = v[i];
 }
 extern "C" int shim_pair_x_tiles(long long values_len, long long R, long long nkb) { return spdp::plan::pair_x_tiles(values_len, R, nkb); }
-extern "C" int shim_batch_loads_one_by_one(long long nnz, long long M, long long K) { return spdp::plan::batch_loads_one_by_one(nnz, M, K); }
+extern "C" int shim_batch_loads_one_by_one(long long nnz, long long uneven, long long M, long long K) {
+    return spdp::plan::batch_loads_one_by_one(nnz, uneven, M, K);
+}

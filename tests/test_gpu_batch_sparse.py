@@ -1,10 +1,12 @@
-"""The batch kernel has two forms of its expansion, chosen by the values that a full column tile of average density has (of
-256): 16-bit loads up to 80, aligned words above.  Both sides of that line, and columns from empty to full in
+"""The batch kernel has two forms of its expansion, chosen by the values of an average column tile and by how much the
+columns differ: 16-bit loads below a line, aligned words above.  Both sides of that line, and columns from empty to full in
 either form, give exact sums on integers; values that are not finite read the same in both."""
 import numpy as np
 import pytest
 
 torch = pytest.importorskip("torch")
+
+from test_batch_form import compile_rule, rows_of
 
 pytestmark = pytest.mark.gpu
 
@@ -33,41 +35,42 @@ def test_both_forms_exact_on_integers(values, M, K, B):
         S.spdp_free(h)
 
 
-def line(M, K):
-    """The most values of a layer that takes the 16-bit loads."""
-    return 80 * M * K // 256
+@pytest.fixture(scope="module")
+def one_by_one(tmp_path_factory):
+    return compile_rule(tmp_path_factory.mktemp("form"))
 
 
-@pytest.mark.parametrize("beyond", [0, 1])
-@pytest.mark.parametrize("M,K,B", [(512, 300, 3), (700, 1001, 8), (256, 64, 5)])
-def test_exactly_at_the_line(beyond, M, K, B):
-    """A layer with exactly as many values as the 16-bit loads take, and one with one more: full and empty columns (the loads of a
-    full one run past its last value) and every count between in both."""
+# values of a column tile of so many rows, in column k, and whether the layer takes the 16-bit loads
+LAYERS = {
+    "last before the line": (lambda rows, k, rng: rows * 96 // 256, True),
+    "first behind the line": (lambda rows, k, rng: -(-rows * 97 // 256), False),
+    "a few full columns among sparse ones": (lambda rows, k, rng: rows if k % 150 == 7 else rng.integers(0, 10), True),
+    "from empty to full": (lambda rows, k, rng: (0, rows, rng.integers(0, rows + 1))[k % 3], False),
+    "sparse and uneven": (lambda rows, k, rng: rows * (10 if k % 2 else 70) // 256, False),
+}
+
+
+@pytest.mark.parametrize("layer", list(LAYERS))
+@pytest.mark.parametrize("M,K,B", [(512, 300, 3), (700, 1001, 8), (256, 200, 5)])
+def test_both_sides_of_the_line(one_by_one, layer, M, K, B):
+    """Layers on either side of the line, down to one value a tile from it, and full columns in both forms (their loads run past the last
+    value)."""
     if not torch.cuda.is_available():
         pytest.skip("needs a CUDA device")
     from paper_2607_21985_b200 import spdp as S
     rng = np.random.Generator(np.random.PCG64(M + K))
-    R = (M + 255) // 256
-    rows = [min(256, M - 256 * r) for r in range(R)]
-    counts = np.stack([rng.integers(0, rows[r] + 1, K) for r in range(R)])
-    fixed = np.zeros(K, bool)
-    fixed[rng.permutation(K)[:K // 5]] = True
-    counts[:, fixed] = np.where(rng.random((R, fixed.sum())) < 0.5, 0, np.array(rows)[:, None])
-    want_nnz = line(M, K) + beyond
-    while (d := want_nnz - int(counts.sum())) != 0:                     # the other columns make up the rest
-        r, k = rng.integers(R), rng.integers(K)
-        if not fixed[k]:
-            counts[r, k] = min(rows[r], max(0, counts[r, k] + max(-40, min(40, d))))
+    count, loads = LAYERS[layer]
+    counts = np.array([[count(rows, k, rng) for k in range(K)] for rows in rows_of(M)])
+    assert one_by_one(counts, M) == loads
     W = np.zeros((M, K), np.float16)
-    for r in range(R):
+    for r, rows in enumerate(rows_of(M)):
         for k in range(K):
-            at = 256 * r + rng.permutation(rows[r])[:counts[r, k]]
+            at = 256 * r + rng.permutation(rows)[:counts[r, k]]
             W[at, k] = rng.integers(1, 9, len(at)) * rng.choice([-1, 1], len(at))
     X = rng.integers(-4, 5, (B, K)).astype(np.float16)
     want = X.astype(np.float64) @ W.astype(np.float64).T                # |sums| <= 1001 * 32 < 2^24: exact in fp32
     h = S.spdp_pack_tiled_cbc(torch.from_numpy(W).cuda())
     try:
-        assert S.spdp_get_info(h).nnz == want_nnz
         for ctas in (0, 2):
             S.spdp_set_num_ctas(h, ctas)
             Y = torch.full((B, M), float("nan"), dtype=torch.float32, device="cuda")
@@ -80,7 +83,7 @@ def test_exactly_at_the_line(beyond, M, K, B):
 
 
 @pytest.mark.parametrize("density", [0.25, 0.9])
-def test_non_finite_values_in_both_forms(density):
+def test_non_finite_values_in_both_forms(one_by_one, density):
     """An infinite weight or a NaN among the weights stays in its row, in the tokens that keep its column; a token that skips
     the column gets NaN there (0 * Inf) where another token makes it fetched; a NaN activation reaches every row of its token."""
     if not torch.cuda.is_available():
@@ -97,9 +100,9 @@ def test_non_finite_values_in_both_forms(density):
     rule, thr = S.SPDP_DP_ABS_GT, 0.0                                   # skips exact zeros
     finite = np.where(np.isfinite(W), W, 0).astype(np.float64)
     want = np.where(np.isfinite(X), X, 0).astype(np.float64) @ finite.T
+    assert one_by_one((W.reshape(2, 256, K) != 0).sum(1), M) == (density < 0.3)
     h = S.spdp_pack_tiled_cbc(torch.from_numpy(W).cuda())
     try:
-        assert (S.spdp_get_info(h).nnz <= line(M, K)) == (density < 0.3)
         Y = torch.zeros((B, M), dtype=torch.float32, device="cuda")
         S.spdp_spmspv_batch(h, torch.from_numpy(X).cuda(), rule, thr, Y)
         torch.cuda.synchronize()
