@@ -6,8 +6,9 @@
 // and moves in 16-byte pieces.  (With the block in shared memory and a lane per row, a ballot or a popcount per row and column,
 // the three took 5300, 8000 and 8500 warp instructions per block, twice to three times what they take now.)
 // 11008x4096 at 60 % sparsity, each kernel alone with cold caches: count 28.9 -> 21.6 us, scan 9.3 -> 6.4, emit 45.4 -> 32.4, unpack
-// 46.2 -> 27.6; the bytes alone would take 14, 0, 20 and 20.  Pack, unpack and free together 173 -> 133 us (memory of freed
-// handles is kept, see memory.cu), the rest of it synchronisations.
+// 46.2 -> 27.6; the bytes alone would take 14, 0, 20 and 20.  Pack, unpack and free together 173 -> 133 us, 125 with the totals in
+// page-locked words and the workspace emptied ahead of the kernels (memory of freed handles is kept, see memory.cu), the rest of it
+// synchronisations.
 #include <mutex>
 
 #include "spdp_internal.h"

@@ -28,10 +28,11 @@ struct Plan {
 };
 // The estimate of a call's time: (K-blocks of the busiest CTA) x (time of a K-block) + a tile's start and end + what the
 // partial sums cost.  Fitted to the four kernels' times, calls in a row on a stream, on 10 layers from 512x512 to 28672x8192
-// (30 to 80 % sparse) with 16 to 1024 tokens each.  Measured again over those 80 calls, the form that is chosen is 0.6 % behind the best form on
-// average, 8 % at worst (512x512 x 16 tokens, 8.3 against 7.6 us).  (Fitted to graph replays, where the CTA pairs' plain launch costs nothing, it took pairs for small layers, and cuts that
-// cross tiles as readily as those that do not: 1024x1024 x 32 tokens 14.4 -> 8.3 us, 2048x2048 x 64 16.5 -> 12.8, 4096x4096 x
-// 128 22.9 -> 19.6, x 16 17.7 -> 14.8, 4096x11008 x 128 34.0 -> 31.4, 4001x4098 x 200 30.8 -> 26.3.)
+// (30 to 80 % sparse) with 16 to 1024 tokens each, when pairs waited for the kernel before (most of their fixed part below) and the second kernel took 1.5
+// to 2 us more.  With the kernels as they are now, over 221 calls of 13 such layers, the form taken is 3.7 % behind the best form on average (49 % at
+// worst), and form and cut 5.6 % behind the best of both.  Most of it are layers of few row tiles, which all SMs share where half to seven eighths of
+// them are faster: below 4000 rows 7.2 and 10.4 % (700x5000 x 32 tokens 13.4 us, with 72 CTAs 9.0; 1024x11008 x 32 15.9, with 128 CTAs 11.2, as pairs
+// 13.4; 3000x700 x 64 9.3, as CTAs of 128 tokens 7.8), from 4000 rows on 0.8 and 1.4 % (8192x8192 x 700 113, as pairs 98).
 constexpr double kCallUs[4] = {3.0, 3.7, 3.2, 6.5};                     // a call's fixed part
 constexpr double kBlockUs[4] = {0.88, 0.97, 1.22, 0.69};                // a K-block (64 columns x 256 rows), us
 constexpr double kBlockTokenUs[4] = {8.3e-4, 1.8e-4, 0.0, 4.8e-4};      // and per token of the tile

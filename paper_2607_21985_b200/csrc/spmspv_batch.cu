@@ -125,7 +125,7 @@ __device__ __forceinline__ unsigned nibble_bits(unsigned W, unsigned top) {     
 // permutes put them into their rows, zero where the bit is clear.  In two parts, so that the loads of several nibbles
 // are under way together.  (One value at a time -- a popcount, a predicated 16-bit load and a select per row -- takes as
 // many instructions and four times the popcounts: 116 us against 113 on the largest layer.  What bounds both is shared
-// memory (its wavefronts take 75 % of the clocks on the largest layer) with the integer pipe behind it (55 %): two warps per K-block with 32 accumulators each, 24 warps
+// memory (its wavefronts take 75 % of the clocks on the largest layer) with the integer pipe behind it (48 %): two warps per K-block with 32 accumulators each, 24 warps
 // per SM, gained nothing.)
 template <bool kSparse>
 struct Nibble { unsigned a, s0, s1, s2, bits; };
