@@ -63,7 +63,8 @@ constexpr int kSubs = kKB / kSub;
 constexpr int kGTB = kKB / kTileK;     // GTiles per K-block
 // Shared memory of a CTA, of the 227 KB that it could have: a block of the second kernel needs 1 KB beside it.  With all of it taken the second
 // kernel of a cut call can start only where a CTA has left: 8192x8192 x 16 tokens 32.0 -> 29.5 us, 11008x4096 x 16 25.4 -> 24.6,
-// 3000x700 x 64 9.23 -> 8.86; most other calls the same.
+// 3000x700 x 64 9.23 -> 8.86, 28672x8192 x 250 149.0 -> 144.7; most other calls the same, whole tiles of pairs among them (both in turn, rested before each:
+// 28672x8192 x 1024 389.1 / 389.1, x 512 218.2 / 218.3, 18944x4096 x 512 66.9 / 66.8), 28672x8192 x 128 114.4 -> 115.1.
 constexpr int kSmemKB = 225;
 constexpr int kBlockWarps = kSubs * kGroupWarps;      // warps that decode a K-block
 static_assert(kSub == 4 * kGroupWarps, "a scan takes 4 columns");

@@ -16,8 +16,8 @@ namespace plan {
 // and 90 % sparsity; "12 %": the columns' sparsities lie up to 12 % to either side of the mean, s = 19:
 //   4096x4096 x 8 tokens   equal 13.4 / 13.7, 13.0 / 12.8, 12.8 / 12.3, 12.7 / 12.2;  12 % 13.5 / 14.1, 13.1 / 13.5, 12.8 / 12.8
 //   28672x8192 x 8         equal 90.8 / 97.6, 88.4 / 90.2, 87.4 / 85.4, 87.1 / 83.9;  12 % 92.6 / 103.1, 89.6 / 97.9, 88.3 / 93.0
-// Large layers change over 14 values earlier: theirs come from HBM whatever was called before.  The form that this line takes is 0.8 % behind the
-// other one at worst, over seven layers, 66 to 90 %, columns 0 to 20 % apart.  (By the average alone, a line at 80 values took loads at up to
+// Large layers change over 14 values earlier: theirs come from HBM whatever was called before.  The form that this line takes is 1.3 % behind the
+// other one at worst, over 315 calls of seven layers, 66 to 90 %, columns 0 to 20 % apart.  (By the average alone, a line at 80 values took loads at up to
 // 12 % more than words where columns differ, and with rows that are not there counted as clear 2 % more on 300x4096.)
 constexpr double kFullTile = 256.0, kPerDeviation = 3.5, kLine = 96.5, kLargeLine = 82.5;
 constexpr int64_t kLargeLayer = 200000;                 // column tiles of 256 rows
