@@ -148,10 +148,10 @@ __device__ __forceinline__ void place_nibble(const Nibble<kSparse>& n, unsigned 
     r01 = permute(t0, 0u, n.bits * kSelect01 + kSelectNone);            // two rows need one word: a clear row selects zero bytes
     r23 = permute(t23, 0u, __dp2a_hi(kSelect23, n.bits, kSelectNone));
 }
-// The form for sparse layers: the two values that rows 0 and 1 may have and the two that rows 2 and 3 may have are loaded one by one,
+// The form for sparse layers with like columns: the two values that rows 0 and 1 may have and the two that rows 2 and 3 may have are loaded one by one,
 // whether they are there or not.  A 16-bit load leaves the upper half of its register zero, which is what a clear row selects, so that
 // nothing has to be aligned: 18 instructions in place of 22 for 4 rows, 5 of them on the integer pipe in place of
-// 9, but one shared-memory access more, and those cost more the denser the layer is.
+// 9, but one shared-memory access more, and those cost more the denser the layer is and the more its columns differ (spmspv_batch_form.h).
 template <>
 struct Nibble<true> { unsigned v0, v1, v2, v3, bits; };
 template <>
