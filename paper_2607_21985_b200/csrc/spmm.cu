@@ -26,6 +26,13 @@
 // word for clear rows.  (A walk over the 8 rows of a bitmap byte with predicated 16-bit loads, as before, took twice the
 // instructions, and 43-49 % of the shared-memory wavefronts were bank conflicts.)
 //
+// That is how W reaches shared memory, where the forms for more than 128 tokens have it.  Up to 128 tokens the accumulators leave
+// room in tensor memory, and decoded W goes there instead (expand_rows): a lane expands the two rows of a column that are its own in
+// the two accumulators, 16 columns at a time, and stores them with tcgen05.st.  Shared memory, which bounded the other way, then neither takes decoded
+// W nor gives it to the tensor cores (per column tile 8 of 20 wavefronts of the decode, and 4 of the products), its loads are
+// single wavefronts at any density, and a warp scans only its own 64 rows.  28672x8192 at 50 % x 16 / 128 tokens 93.2 -> 72.4 / 115.7 -> 91.9 us,
+// 18944x4096 36.0 -> 28.5 / 45.2 -> 38.1, 11008x4096 at 60 % 24.8 -> 23.2 / 33.4 -> 31.8.
+//
 //   one::   one CTA = one row tile (256 rows = two M = 128 accumulators) x up to 32, 128 or 256 tokens.  The CTAs stay for
 //           the whole call: whole rounds of tiles first, one tile per CTA; the K-blocks of the tiles that are left are cut
 //           into equal contiguous ranges, one per CTA.  A tile fed by several CTAs leaves fp32 partial sums in scratch
@@ -106,6 +113,7 @@ struct Params {
     float* partial;         // partial sums [slot][token in tile < ptok][256 rows]; slot = pair i, or 2 * CTA + (0: its first
                             // piece, 1: its last); pair:: null = whole tiles
     int ptok;
+    int xbox;               // one:: tokens that an X tile's copy brings
     int* status;
     int64_t values_len;
 };
@@ -129,6 +137,8 @@ __device__ __forceinline__ uint64_t operand_desc(uint32_t smem_addr, uint32_t lb
 __host__ __device__ constexpr uint32_t instr_desc(int m, int n) {
     return (1u << 4) | (1u << 15) | (static_cast<uint32_t>(n >> 3) << 17) | (static_cast<uint32_t>(m >> 4) << 24);
 }
+// The same with A in tensor memory, where it is K-major: lane = row, a 32-bit column = two neighbouring columns of W.
+__host__ __device__ constexpr uint32_t instr_desc_tmem(int m, int n) { return instr_desc(m, n) & ~(1u << 15); }
 // D[tmem] (+)= A * B, one CTA (M = 128) or a CTA pair (M = 256).  The one-CTA form takes the operand descriptors as halves: the upper
 // ones are constants, and the lower ones move by constants, without a carry.
 template <uint32_t kAHigh, uint32_t kBHigh>
@@ -136,6 +146,12 @@ __device__ __forceinline__ void mma_f16_one(uint32_t d_tmem, uint32_t a_low, uin
     asm volatile("{\n .reg .pred p;\n .reg .b64 a, b;\n setp.ne.b32 p, %4, 0;\n mov.b64 a, {%1, %5};\n mov.b64 b, {%2, %6};\n"
                  " tcgen05.mma.cta_group::1.kind::f16 [%0], a, b, %3, p;\n}"
                  ::"r"(d_tmem), "r"(a_low), "r"(b_low), "r"(instr_desc), "r"(accumulate), "n"(kAHigh), "n"(kBHigh) : "memory");
+}
+template <uint32_t kBHigh>
+__device__ __forceinline__ void mma_f16_tmem(uint32_t d_tmem, uint32_t a_tmem, uint32_t b_low, uint32_t instr_desc, uint32_t accumulate) {
+    asm volatile("{\n .reg .pred p;\n .reg .b64 b;\n setp.ne.b32 p, %4, 0;\n mov.b64 b, {%2, %5};\n"
+                 " tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], b, %3, p;\n}"
+                 ::"r"(d_tmem), "r"(a_tmem), "r"(b_low), "r"(instr_desc), "r"(accumulate), "n"(kBHigh) : "memory");
 }
 __device__ __forceinline__ void mma_f16_pair(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc, uint32_t instr_desc, bool accumulate) {
     asm volatile("{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
@@ -281,6 +297,93 @@ __device__ __forceinline__ void expand4(uint32_t tab_l, uint32_t a_dst, uint32_t
     }
 }
 
+struct alignas(16) Meta {                       // a K-block as stored, without its values
+    alignas(16) uint32_t bm[kKB][8];            // bitmaps
+    alignas(16) uint32_t ci[kKB];               // ColInfo words
+    alignas(16) uint32_t start[kGTB];           // shared-memory address of each GTile's first value
+    alignas(16) uint32_t vstart;                // copy warp: virtual ring offset of its values
+    uint32_t limit;                             // (checked build) values of the K-block
+    int ngt;                                    // GTiles it really has
+    uint32_t unused;
+};
+
+template <int kOff>
+__device__ __forceinline__ unsigned lds_u16_at(uint32_t addr) {
+    unsigned v;
+    asm volatile("ld.shared.u16 %0, [%1+%2];" : "=r"(v) : "r"(addr), "n"(kOff));
+    return v;
+}
+__device__ __forceinline__ void tmem_store8(uint32_t at, const uint32_t (&v)[8]) {
+    asm volatile("tcgen05.st.sync.aligned.32x32b.x8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};"
+                 ::"r"(at), "r"(v[0]), "r"(v[1]), "r"(v[2]), "r"(v[3]), "r"(v[4]), "r"(v[5]), "r"(v[6]), "r"(v[7]) : "memory");
+}
+__device__ __forceinline__ void tmem_load8(uint32_t at, uint32_t (&v)[8]) {
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+                 : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7]) : "r"(at) : "memory");
+}
+
+// Scan for the expansion into tensor memory: lane = column j of the K-block, for the 64 rows of quarter q of the row tile.  The two
+// bitmap words of those rows and the address of each one's first value go to tab[lane] (rows 0 .. 31 of the quarter) and
+// tab[kTabRow + lane] (rows 32 .. 63).  Four words are read, the half of the column tile that the quarter is in; the values before the
+// quarter are counted from the end of the column tile that this half touches, by factors that only the quarter decides (Quarter).
+constexpr int kTabRow = 34;             // the two rows of the table start 16 bytes apart in the banks, and are read together
+struct Quarter {
+    int from_end, first_pair, second_pair;      // values before it = from_end * nnz + first_pair * (words 0, 1) + second_pair * (words 2, 3)
+    bool odd;
+    __device__ __forceinline__ explicit Quarter(int q)
+        : from_end(pinned(q >> 1)), first_pair(pinned(q == 1 ? 1 : q == 2 ? -1 : 0)), second_pair(pinned(q >= 2 ? -1 : 0)), odd((q & 1) != 0) {}
+};
+__device__ __forceinline__ void scan_quarter(const Params& p, const Meta& mt, int j, const Quarter& q, uint32_t tab) {
+    const uint32_t ciw = mt.ci[j];
+    uint4 w = *reinterpret_cast<const uint4*>(&mt.bm[j][4 * q.from_end]);
+    uint32_t first = mt.start[j >> 4] + 2u * (ciw >> 16);
+    const bool there = (j >> 4) < mt.ngt && SPDP_CHECK(p.status, (first - mt.start[0]) / 2u, ciw & 0xFFFFu, mt.limit, kSiteValuesSpan);
+    if (!there) {                       // behind the last GTile of the matrix (or, in the checked build, not what the format says)
+        w = make_uint4(0u, 0u, 0u, 0u);
+        first = mt.start[0];
+    }
+    const int px = __popc(w.x) + __popc(w.y), pz = __popc(w.z) + __popc(w.w);
+    const int before = static_cast<int>(there ? ciw & 0xFFFFu : 0u) * q.from_end + px * q.first_pair + pz * q.second_pair;
+    const unsigned lo = q.odd ? w.z : w.x, hi = q.odd ? w.w : w.y;
+    first += 2u * static_cast<unsigned>(before);
+    sts_v2(tab, lo, first);
+    sts_v2(tab + 8u * kTabRow, hi, first + 2u * __popc(lo));
+}
+
+// Expands 16 columns x 64 rows into registers for tensor memory: even[i] holds columns 2i and 2i + 1 of the lane's even row, odd[i] of
+// its odd row.  A lane has rows 2l and 2l + 1 (l = lane % 16) of word lane / 16; top = 1 << (30 - 2l) puts their bits on top of the
+// word and leaves the bits below, so that one popcount leads past the last value of either; the two values before that place are
+// loaded one by one, whether they are there or not, the bits become masks (bytes filled with their sign), and the masks say which value
+// a row takes, if any.  Two columns at a time share masks and selections.  Per column and 64 rows 5 instructions go to the integer pipe, 4 to the
+// multipliers (`two` is a 2 that the compiler does not know, or the addresses went to the integer pipe too) and 2.5 to shared memory, one
+// wavefront each.  What bounds it is issue: 24 warps that all expand keep the schedulers 95 % busy.  (Selectors from a table of four
+// instead of masks take one instruction more for two columns and measured 1 to 2 % more; 16 columns unrolled twice spill.)
+__device__ __forceinline__ void expand_rows(uint32_t tab_l, unsigned top, unsigned two, uint32_t (&even)[8], uint32_t (&odd)[8]) {
+    constexpr int kAtOnce = 8;              // columns whose loads are under way together (four: 0 to 2 % slower)
+#pragma unroll
+    for (int c0 = 0; c0 < 16; c0 += kAtOnce) {
+        unsigned bits[kAtOnce / 2], last[kAtOnce], before[kAtOnce];
+#pragma unroll
+        for (int c = 0; c < kAtOnce; c += 2) {
+            const uint4 v = lds_v4<0>(tab_l + 8u * (c0 + c));
+            const unsigned s0 = v.x * top, s1 = v.z * top;
+            const uint32_t a0 = v.y + two * __popc(s0), a1 = v.w + two * __popc(s1);
+            bits[c / 2] = permute(s0, s1, 0x7632u);         // the upper halves: odd row's bit on top, even row's under it
+            last[c] = lds_u16_at<-2>(a0);
+            before[c] = lds_u16_at<-4>(a0);
+            last[c + 1] = lds_u16_at<-2>(a1);
+            before[c + 1] = lds_u16_at<-4>(a1);
+        }
+#pragma unroll
+        for (int c = 0; c < kAtOnce; c += 2) {
+            const unsigned has_odd = permute(bits[c / 2], 0u, 0xBB99u), has_even = permute(bits[c / 2] * two, 0u, 0xBB99u);
+            const unsigned l = last[c + 1] * 65536u + last[c], b = before[c + 1] * 65536u + before[c];
+            odd[(c0 + c) / 2] = l & has_odd;
+            even[(c0 + c) / 2] = ((l & ~has_odd) | (b & has_odd)) & has_even;
+        }
+    }
+}
+
 // Turns 4 values of each of 4 neighbouring lanes: lane l's v[i] becomes what lane (l & ~3) + i had in v[l & 3].
 __device__ __forceinline__ void transpose4(uint32_t& v0, uint32_t& v1, uint32_t& v2, uint32_t& v3, int lane) {
     const bool odd = (lane & 1) != 0, upper = (lane & 2) != 0;
@@ -348,6 +451,40 @@ __device__ __forceinline__ void store_accumulators(const Params& p, uint32_t tme
     }
 }
 
+// The same for the forms with W in tensor memory, where lane l of quarter q holds row 64q + 2l in the first accumulator and the row
+// after it in the second, kNI columns further: tokens [c0, c0 + 8), two neighbouring rows at once.
+template <int kNI>
+__device__ __forceinline__ void store_row_pairs(const Params& p, uint32_t tmem, int q, int c0, int valid, int r, int64_t n0, int slot) {
+    const int lane = threadIdx.x & 31, row_in = 64 * q + 2 * lane;
+    uint32_t v[8], w[8];
+    tmem_load8(tmem + (static_cast<uint32_t>(32 * q) << 16) + c0, v);
+    tmem_load8(tmem + (static_cast<uint32_t>(32 * q) << 16) + kNI + c0, w);
+    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+    if (slot >= 0) {
+        float* part = p.partial + (static_cast<size_t>(slot) * p.ptok + c0) * kTileM + row_in;
+#pragma unroll
+        for (int i = 0; i < 8; ++i)
+            if (c0 + i < valid) *reinterpret_cast<float2*>(part + i * kTileM) = make_float2(__uint_as_float(v[i]), __uint_as_float(w[i]));
+        return;
+    }
+    const int64_t row = static_cast<int64_t>(r) * kTileM + row_in;
+    const unsigned size = p.ydt == SPDP_Y_F32 ? 4u : 2u;
+    const bool twos = (p.ldy & 1) == 0 && (reinterpret_cast<uintptr_t>(p.Y) & (2u * size - 1u)) == 0 && row + 2 <= p.M;
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+        if (c0 + i >= valid) break;
+        const int64_t at = (n0 + c0 + i) * p.ldy + row;
+        const float a = __uint_as_float(v[i]), b = __uint_as_float(w[i]);
+        if (twos) {
+            if (p.ydt == SPDP_Y_F32) *reinterpret_cast<float2*>(static_cast<float*>(p.Y) + at) = make_float2(a, b);
+            else *reinterpret_cast<__half2*>(static_cast<__half*>(p.Y) + at) = __floats2half2_rn(a, b);
+        } else {
+            if (row < p.M) store_y(p.Y, p.ydt, at, a);
+            if (row + 1 < p.M) store_y(p.Y, p.ydt, at + 1, b);
+        }
+    }
+}
+
 // A CTA that gave up fills its slots of the scratch memory with this word, so that the second kernel leaves the rows it feeds
 // unwritten instead of adding what an earlier call left there.  No sum can be this word: a NaN that arithmetic makes is 0x7FFFFFFF.
 // (Only the fourth rows are tested, one comparison per 16 bytes.  A word per CTA beside the slots, written by every CTA and
@@ -411,15 +548,6 @@ __device__ __forceinline__ void add_partials(const Params& p, const float* first
         if (row + e < p.M) store_y(p.Y, p.ydt, at + e, v[e]);
 }
 
-struct alignas(16) Meta {                       // a K-block as stored, without its values
-    alignas(16) uint32_t bm[kKB][8];            // bitmaps
-    alignas(16) uint32_t ci[kKB];               // ColInfo words
-    uint32_t start[kGTB];                       // shared-memory address of each GTile's first value
-    uint32_t limit;                             // (checked build) values of the K-block
-    uint32_t vstart;                            // copy warp: virtual ring offset of its values
-    int ngt;                                    // GTiles it really has
-};
-
 // ---- the copy warp's work: stored K-blocks into a ring ----
 struct CopyState {
     unsigned i = 0, done = 0;                               // K-blocks started / known to be decoded
@@ -427,40 +555,41 @@ struct CopyState {
 };
 // Starts the copies of K-blocks kb0 .. kb0 + n - 1 of the row tile whose first GTile is g_row.  The values of the blocks in
 // flight lie in a ring of bytes, so that the sparser the matrix, the more blocks are on their way; bitmaps and ColInfo in
-// kMeta slots.  The lanes hold the TileOffset words of 32 K-blocks (and of the next 32) and walk them together; one lane
-// issues.  After a failure nothing is copied any more, but every block's barrier still completes.
+// kMeta slots.  A lane holds the TileOffset words of one K-block in 32, looks them over and says where its values start; what is left per
+// block is short, because this one warp shares its scheduler with six that decode, and each of its instructions waits for its turn.  After a
+// failure nothing is copied any more, but every block's barrier still completes.
 template <int kMeta>
 __device__ __forceinline__ bool copy_blocks(const Params& p, CopyState& c, uint32_t ring, uint32_t ring_bytes, Meta* meta, unsigned long long* full,
                                             unsigned long long* freed, int* abort, int64_t g_row, int kb0, int n, int lane, bool ok) {
-    uint32_t cur[kGTB + 1], nxt[kGTB + 1];
+    uint32_t to[kGTB + 1], nxt[kGTB + 1];
     auto fetch = [&](int b, uint32_t (&o)[kGTB + 1]) {      // words of K-block kb0 + b + lane: its GTiles and the one after
         const int g0 = (kb0 + b + lane) * kGTB;
 #pragma unroll
         for (int q = 0; q <= kGTB; ++q) o[q] = (b + lane < n) ? __ldg(p.tileoffset + g_row + min(g0 + q, p.C)) : 0u;
     };
-    fetch(0, cur);
+    fetch(0, to);
+    const uint64_t* bm = p.bitmap + (g_row + static_cast<int64_t>(kb0) * kGTB) * kTileK * 4;
+    const uint32_t* ci = p.colinfo + (g_row + static_cast<int64_t>(kb0) * kGTB) * kTileK;
     for (int b = 0; b < n; b += 32) {
         fetch(b + 32, nxt);
+        const uint32_t nvals = to[kGTB] - to[0];
+        const bool bad = to[kGTB] < to[0] || nvals > static_cast<uint32_t>(kKB * kTileM) || static_cast<int64_t>(to[kGTB]) > p.values_len;
+        if (__any_sync(0xFFFFFFFFu, bad)) {                 // not what the format says
+            if (lane == 0) {
+                atomicCAS(p.status, 0, SPDP_ERR_OVERFLOW);
+                *static_cast<volatile int*>(abort) = 1;     // the outputs stay unwritten
+            }
+            ok = false;
+        }
         const int lim = min(32, n - b);
         for (int q = 0; q < lim; ++q, ++c.i) {
-            uint32_t to[kGTB + 1];
-#pragma unroll
-            for (int e = 0; e <= kGTB; ++e) to[e] = __shfl_sync(0xFFFFFFFFu, cur[e], q);
-            const int g0 = (kb0 + b + q) * kGTB;
-            const int ngt = min(kGTB, p.C - g0);
-            const uint32_t nvals = to[kGTB] - to[0];
-            if (to[kGTB] < to[0] || nvals > static_cast<uint32_t>(kKB * kTileM) ||
-                static_cast<int64_t>(to[kGTB]) > p.values_len) {                        // not what the format says
-                atomicCAS(p.status, 0, SPDP_ERR_OVERFLOW);
-                *static_cast<volatile int*>(abort) = 1;                                 // the outputs stay unwritten
-                ok = false;
-            }
-            const uint32_t bytes = ok ? 2u * nvals : 0u;
+            const uint32_t from = __shfl_sync(0xFFFFFFFFu, to[0], q), bytes = __shfl_sync(0xFFFFFFFFu, ok ? 2u * nvals : 0u, q);
             if (c.pos + bytes > ring_bytes) {               // the values of a K-block stay in one piece
                 c.vhead += ring_bytes - c.pos;
                 c.pos = 0;
             }
-            while (c.i - c.done >= kMeta || c.vhead + bytes - c.vtail > ring_bytes) {
+            const uint32_t vend = c.vhead + bytes;
+            while (c.i - c.done >= kMeta || vend - c.vtail > ring_bytes) {
                 if (c.done == c.i) { c.vtail = c.vhead; continue; }
                 if (c.done == 0u) asm volatile("griddepcontrol.wait;" ::: "memory");    // the decode waits for products, these for X
                 if (ok) ok = wait_parity(&freed[c.done % kMeta], (c.done / kMeta) & 1);
@@ -470,27 +599,32 @@ __device__ __forceinline__ bool copy_blocks(const Params& p, CopyState& c, uint3
             ok = __all_sync(0xFFFFFFFFu, ok);
             const unsigned m = c.i % kMeta;
             Meta& mt = meta[m];
+            const int ngt = min(kGTB, p.C - (kb0 + b + q) * kGTB);
+            if (lane == q) {                                // my K-block
+                const uint32_t at = ring + c.pos - 2u * to[0];
+                static_assert(kGTB == 4, "one store");
+                *reinterpret_cast<uint4*>(&mt.start[0]) = make_uint4(at + 2u * to[0], at + 2u * to[1], at + 2u * to[2], at + 2u * to[3]);
+                *reinterpret_cast<uint4*>(&mt.vstart) = make_uint4(c.vhead, nvals, ok ? static_cast<unsigned>(ngt) : 0u, 0u);
+            }
+            __syncwarp();
             if (elect_one()) {
-                mt.vstart = c.vhead;
-                mt.ngt = ok ? ngt : 0;
-                mt.limit = nvals;
-#pragma unroll
-                for (int e = 0; e < kGTB; ++e) mt.start[e] = ring + c.pos + (ok ? 2u * (to[e] - to[0]) : 0u);
                 if (ok) {
                     expect_bytes(&full[m], bytes + static_cast<uint32_t>(ngt) * (kTileK * 32u + kTileK * 4u));
-                    bulk_copy(smem_u32(&mt.bm[0][0]), p.bitmap + (g_row + g0) * kTileK * 4, static_cast<uint32_t>(ngt) * kTileK * 32u, &full[m]);
-                    bulk_copy(smem_u32(&mt.ci[0]), p.colinfo + (g_row + g0) * kTileK, static_cast<uint32_t>(ngt) * kTileK * 4u, &full[m]);
-                    if (bytes) bulk_copy(ring + c.pos, p.values + to[0], bytes, &full[m]);
+                    if (bytes) bulk_copy(ring + c.pos, p.values + from, bytes, &full[m]);
+                    bulk_copy(smem_u32(&mt.bm[0][0]), bm, static_cast<uint32_t>(ngt) * kTileK * 32u, &full[m]);
+                    bulk_copy(smem_u32(&mt.ci[0]), ci, static_cast<uint32_t>(ngt) * kTileK * 4u, &full[m]);
                 } else {
                     arrive(&full[m]);
                 }
             }
             __syncwarp();
+            bm += kKB * 4;
+            ci += kKB;
             c.vhead += ok ? bytes : 0u;
             c.pos += ok ? bytes : 0u;
         }
 #pragma unroll
-        for (int q = 0; q <= kGTB; ++q) cur[q] = nxt[q];
+        for (int q = 0; q <= kGTB; ++q) to[q] = nxt[q];
     }
     return ok;
 }
@@ -508,18 +642,22 @@ namespace one {     // one CTA = one row tile x kNI tokens
 template <int kNIT>
 struct Form {
     static constexpr int kNI = kNIT;                                  // the N of the tensor-core instruction = tokens per tile
-    static constexpr int kTmemCols = 2 * kNI;                         // two accumulators: the row halves
+    static constexpr bool kTmemW = kNI <= 128;                        // decoded W in tensor memory, where there is room for it
+    static constexpr int kGroupWarps = kTmemW ? 4 : spdp::kGroupWarps;
+    static constexpr int kGroups = kWarps / kGroupWarps;
+    static constexpr int kTmemCols = kTmemW ? 512 : 2 * kNI;          // two accumulators (of 128 rows each), and W
     static constexpr int kBBytes = kNI * kBRowBytes;
     static constexpr int kATileBytes = (kSub / 8) * kAKGroupStride;   // 128 rows x kSub columns
-    static constexpr int kABytes = 2 * kATileBytes;
-    static constexpr int kAStages = kNI == 32 ? 6 : 4;                // decoded sub-blocks.  Three groups decode at once, so four
-        // leave one to spare and the groups wait a fifth of their time for the tensor cores to be done with a stage.  Six, where
-        // X tiles are small: 4096x4096 x 16 tokens 13.0 -> 11.7 us, 28672x8192 x 16 99.9 -> 95.6 (with 128 tokens five stages and two
-        // X tiles gained nothing).
-    static constexpr int kBStages = kNI <= 128 ? 3 : 2;
-    static constexpr int kMeta = kNI <= 128 ? 8 : 6;                  // stored K-blocks in flight, at most
+    static constexpr int kABytes = kTmemW ? 0 : 2 * kATileBytes;      // a stage of decoded W in shared memory
+    static constexpr int kACols = kSub;                               // and in tensor memory: 32-bit columns, half of them for either accumulator
+    static constexpr int kAStages = kTmemW ? 8 : 4;                   // decoded sub-blocks
+    static constexpr int kBStages = kNI <= 128 ? 4 : 2;
+    static constexpr int kMeta = kNI <= 128 ? 8 : 6;                 // stored K-blocks in flight, at most
+    static constexpr int kTab = kTmemW ? 2 * kTabRow : 32;            // table entries per warp
+    static constexpr int kStorers = kTmemW ? kWarps : kStoreWarps;
     static_assert(kBBytes % 1024 == 0, "every X tile on a swizzle-atom boundary");
     static_assert(kAStages >= 2 * kSubs && kAStages >= kGroups, "the first two K-blocks fit in the first A stages, and every decode warp has a sub-block among the next kAStages");
+    static_assert(!kTmemW || 2 * kNI + kAStages * kACols <= kTmemCols, "accumulators and W fit tensor memory");
 };
 
 // CTA w's share of the tiles that are cut along K: K-blocks [rest_begin(w), rest_begin(w + 1)).
@@ -562,9 +700,9 @@ __device__ __forceinline__ bool piece(const Params& p, int w, int k, Piece& s) {
 template <class F>
 struct __align__(1024) Smem {
     unsigned char B[F::kBStages][F::kBBytes];       // X tiles (each on a 1024-byte boundary: swizzle atoms)
-    unsigned char A[F::kAStages][F::kABytes];       // decoded W
+    alignas(16) unsigned char A[F::kTmemW ? 16 : F::kAStages * F::kABytes];     // decoded W
     Meta meta[F::kMeta];
-    alignas(16) uint2 tab[kWarps][32];              // per warp: bitmap word and the address of its first value
+    alignas(16) uint2 tab[kWarps][F::kTab];         // per warp: bitmap word and the address of its first value
     alignas(8) unsigned long long comp_full[F::kMeta];  // the stored K-block has arrived
     alignas(8) unsigned long long comp_free[F::kMeta];  // the decode warps are done with it
     alignas(8) unsigned long long a_ready[F::kAStages]; // A stage is written
@@ -583,13 +721,16 @@ constexpr uint32_t kSmemBytes = kSmemKB * 1024u;    // the dynamic shared memory
 template <class F>
 constexpr uint32_t kRingBytes = (kSmemBytes - 1024u - static_cast<uint32_t>(offsetof(Smem<F>, ring)) - 64u) / 128u * 128u;
 
+// 64 registers a thread, which leaves room for a block of the second kernel beside a CTA (with 72, as for kThreads alone, 0.5 % more time
+// over 7 layers x 4 token counts).
+constexpr int kLaunchBound = 1024;
 template <class F>
-__global__ void __launch_bounds__(kThreads, 1)
+__global__ void __launch_bounds__(kLaunchBound, 1)
 spmm_kernel(const __grid_constant__ Params p, const __grid_constant__ CUtensorMap xmap) {
     static_assert(kRingBytes<F> >= 2 * kKB * kTileM * 2, "the ring holds at least two full K-blocks");
     extern __shared__ unsigned char smem_raw[];
     Smem<F>& sm = *reinterpret_cast<Smem<F>*>(smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u));
-    const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
+    const int t = threadIdx.x, lane = t & 31, warp = __shfl_sync(0xFFFFFFFFu, t >> 5, 0);      // the same in all lanes, and known to be
     const int me = static_cast<int>(blockIdx.x);
 
     // ---- set-up: the barriers and tensor memory ----
@@ -597,11 +738,11 @@ spmm_kernel(const __grid_constant__ Params p, const __grid_constant__ CUtensorMa
 #pragma unroll
         for (int s = 0; s < F::kMeta; ++s) {
             barrier_init(&sm.comp_full[s], 1);
-            barrier_init(&sm.comp_free[s], kBlockWarps);
+            barrier_init(&sm.comp_free[s], kSubs * F::kGroupWarps);
         }
 #pragma unroll
         for (int s = 0; s < F::kAStages; ++s) {
-            barrier_init(&sm.a_ready[s], kGroupWarps);
+            barrier_init(&sm.a_ready[s], F::kGroupWarps);
             barrier_init(&sm.a_free[s], 1);
         }
 #pragma unroll
@@ -610,7 +751,7 @@ spmm_kernel(const __grid_constant__ Params p, const __grid_constant__ CUtensorMa
             barrier_init(&sm.x_free[s], 1);
         }
         barrier_init(&sm.acc_full, 1);
-        barrier_init(&sm.acc_free, kStoreWarps);
+        barrier_init(&sm.acc_free, F::kStorers);
         barrier_init(&sm.drained, 1);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         sm.abort = 0;
@@ -637,7 +778,7 @@ spmm_kernel(const __grid_constant__ Params p, const __grid_constant__ CUtensorMa
         if (elect_one()) {
             unsigned sa = 0, pa = 0, sb = 0, pb = 0;                    // stage and parity of the next sub-block and X tile
             bool issued = false;
-            const uint32_t a_base = desc_low(smem_u32(&sm.A[0][0]), kAKGroupStride), b_base = desc_low(smem_u32(&sm.B[0][0]), 16);
+            const uint32_t a_base = desc_low(smem_u32(&sm.A[0]), kAKGroupStride), b_base = desc_low(smem_u32(&sm.B[0][0]), 16);
             asm volatile("griddepcontrol.wait;" ::: "memory");
             for (int k = 0; ok && piece(p, me, k, s); ++k) {
                 if (k > 0) {
@@ -646,7 +787,8 @@ spmm_kernel(const __grid_constant__ Params p, const __grid_constant__ CUtensorMa
                 }
                 // the tile's tokens, in the units of the instruction
                 const int64_t left = p.N - static_cast<int64_t>(s.tile % p.nblocks) * F::kNI;
-                const uint32_t id = instr_desc(128, left < F::kNI ? static_cast<int>(left + 15) / 16 * 16 : F::kNI);
+                const int n = left < F::kNI ? static_cast<int>(left + 15) / 16 * 16 : F::kNI;
+                const uint32_t id = F::kTmemW ? instr_desc_tmem(128, n) : instr_desc(128, n);
                 for (int kb = 0; ok && kb < s.n; ++kb) {
                     ok = wait_parity(&sm.x_full[sb], pb);                                       // the X tile is in place
                     for (int h = 0; ok && h < kSubs; ++h) {
@@ -659,7 +801,9 @@ spmm_kernel(const __grid_constant__ Params p, const __grid_constant__ CUtensorMa
                         for (int a = 0; a < 2; ++a) {                   // the two row halves
 #pragma unroll
                             for (int kk = 0; kk < kSub / 16; ++kk)      // the start address is the low field, in 16-byte units
-                                mma_f16_one<kDescHigh<kAChunkStride, 0u>, kDescHigh<kBAtomBytes, 2u>>(
+                                if constexpr (F::kTmemW) mma_f16_tmem<kDescHigh<kBAtomBytes, 2u>>(
+                                    tmem + a * F::kNI, tmem + 2 * F::kNI + sa * F::kACols + a * (F::kACols / 2) + kk * 8, bl + ((kk * 32) >> 4), id, kk > 0 ? 1u : add);
+                                else mma_f16_one<kDescHigh<kAChunkStride, 0u>, kDescHigh<kBAtomBytes, 2u>>(
                                     tmem + a * F::kNI, al + ((a * F::kATileBytes + kk * 2 * kAKGroupStride) >> 4), bl + ((kk * 32) >> 4),
                                     id, kk > 0 ? 1u : add);
                         }
@@ -697,7 +841,7 @@ spmm_kernel(const __grid_constant__ Params p, const __grid_constant__ CUtensorMa
                     const unsigned sb = u % F::kBStages;
                     if (u >= F::kBStages && ok) ok = wait_parity(&sm.x_free[sb], (u / F::kBStages - 1u) & 1);
                     if (!ok) { arrive(&sm.x_full[sb]); continue; }
-                    expect_bytes(&sm.x_full[sb], F::kBBytes);
+                    expect_bytes(&sm.x_full[sb], static_cast<uint32_t>(p.xbox) * kBRowBytes);
                     tensor_copy(&sm.B[sb][0], &xmap, (s.kb0 + kb) * kKB, n0, &sm.x_full[sb]);
                 }
             }
@@ -706,11 +850,17 @@ spmm_kernel(const __grid_constant__ Params p, const __grid_constant__ CUtensorMa
         __syncwarp();
     } else {
         // ================= decode warps =================
-        const unsigned group = static_cast<unsigned>(warp) / kGroupWarps, wm = static_cast<unsigned>(warp) % kGroupWarps;
-        const unsigned top = pinned(nibble_top(lane & 7)), below = pinned(nibble_below(lane & 7));
-        const uint32_t tab_l = pinned(smem_u32(&sm.tab[warp][0]) + 8u * (lane >> 3));
-        const uint32_t a_lane = pinned(smem_u32(&sm.A[0][0]) + (lane >> 1) * kAChunkStride + (lane & 1) * 8 +
-                                       (wm >> 1) * kAKGroupStride + (wm & 1u) * 64u);
+        // W in shared memory: warp wm of the group has 4 columns of a sub-block, all 256 rows.  In tensor memory: 64 rows, which are the 32
+        // lanes that the hardware lets this warp write, of all 32 columns.
+        constexpr unsigned kGroups = F::kGroups;
+        const unsigned group = static_cast<unsigned>(warp) / F::kGroupWarps, wm = static_cast<unsigned>(warp) % F::kGroupWarps;
+        const unsigned top = pinned(F::kTmemW ? 1u << (30u - 2u * (lane & 15u)) : nibble_top(lane & 7)), below = pinned(nibble_below(lane & 7));
+        const uint32_t tab_l = pinned(smem_u32(&sm.tab[warp][0]) + 8u * (F::kTmemW ? kTabRow * (lane >> 4) : lane >> 3));
+        const uint32_t a_lane = pinned(F::kTmemW ? tmem + (32u * wm << 16) + 2u * F::kNI
+                                                 : smem_u32(&sm.A[0]) + (lane >> 1) * kAChunkStride + (lane & 1) * 8 + (wm >> 1) * kAKGroupStride + (wm & 1u) * 64u);
+        const uint32_t tab_me = pinned(smem_u32(&sm.tab[warp][0]) + 8u * lane);
+        const Quarter quarter(static_cast<int>(wm));
+        const unsigned two = pinned(2u);
         unsigned i0 = 0;                                                // sub-blocks before this piece
         for (int k = 0; ok && piece(p, me, k, s); ++k) {
             const unsigned i1 = i0 + static_cast<unsigned>(s.n) * kSubs;
@@ -721,7 +871,8 @@ spmm_kernel(const __grid_constant__ Params p, const __grid_constant__ CUtensorMa
                     ok = wait_parity(&sm.comp_full[m], (u / F::kMeta) & 1);                          // the stored K-block has arrived
                     __syncwarp();
                     const Meta& mt = sm.meta[m];
-                    scan4(p, mt.bm, mt.ci, mt.start, mt.ngt, mt.limit, static_cast<int>((i % kSubs) * kSub + 4u * wm), lane, &sm.tab[warp][0]);
+                    if constexpr (F::kTmemW) scan_quarter(p, mt, static_cast<int>((i % kSubs) * kSub) + lane, quarter, tab_me);
+                    else scan4(p, mt.bm, mt.ci, mt.start, mt.ngt, mt.limit, static_cast<int>((i % kSubs) * kSub + 4u * wm), lane, &sm.tab[warp][0]);
                     __syncwarp();
                     if (i >= F::kAStages) {
                         if (i < 2 * F::kAStages) asm volatile("griddepcontrol.wait;" ::: "memory");  // the products wait for X
@@ -729,9 +880,22 @@ spmm_kernel(const __grid_constant__ Params p, const __grid_constant__ CUtensorMa
                     }
                     ok = __all_sync(0xFFFFFFFFu, ok);
                     if (!ok) break;
-                    expand4<8, 2>(tab_l, a_lane + sa * F::kABytes, F::kATileBytes, below, top);
-                    // the operand tile was written through the generic proxy; the tensor cores read through the async proxy
-                    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+                    if constexpr (F::kTmemW) {
+                        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+#pragma unroll 1
+                        for (int c0 = 0; c0 < kSub; c0 += 16) {
+                            uint32_t even[8], odd[8];
+                            expand_rows(tab_l + 8u * c0, top, two, even, odd);
+                            tmem_store8(a_lane + sa * F::kACols + c0 / 2, even);
+                            tmem_store8(a_lane + sa * F::kACols + F::kACols / 2 + c0 / 2, odd);
+                        }
+                        asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
+                        asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+                    } else {
+                        expand4<8, 2>(tab_l, a_lane + sa * F::kABytes, F::kATileBytes, below, top);
+                        // the operand tile was written through the generic proxy; the tensor cores read through the async proxy
+                        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+                    }
                     __syncwarp();
                     if (lane == 0) {
                         arrive(&sm.a_ready[sa]);
@@ -746,17 +910,23 @@ spmm_kernel(const __grid_constant__ Params p, const __grid_constant__ CUtensorMa
                     asm volatile("griddepcontrol.wait;" ::: "memory");
             }
             i0 = i1;
-            if (warp >= kStoreWarps) continue;
+            if (warp >= F::kStorers) continue;
             // ---- the piece's products are complete: store the accumulators ----
             asm volatile("griddepcontrol.wait;" ::: "memory");          // Y and the scratch may belong to the kernel before this one
             if (ok) ok = wait_parity(&sm.acc_full, k & 1);
             asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
             ok = __all_sync(0xFFFFFFFFu, ok);
             if (ok && !__any_sync(0xFFFFFFFFu, *static_cast<volatile int*>(&sm.abort) != 0)) {
-                // warp w: row half (w / 4) % 2, tensor-memory lanes 32 * (w % 4).., token columns [(w / 8) * kNI / 2, + kNI / 2)
-                const int half = (warp >> 2) & 1, cbase = (warp >> 3) * (F::kNI / 2), lane_base = 32 * (warp & 3);
-                store_accumulators<false>(p, tmem + half * F::kNI, lane_base, cbase, cbase + F::kNI / 2, s.tile / p.nblocks,
-                                   half * 128 + lane_base, static_cast<int64_t>(s.tile % p.nblocks) * F::kNI, s.slot);
+                const int64_t n0 = static_cast<int64_t>(s.tile % p.nblocks) * F::kNI;
+                if constexpr (F::kTmemW) {
+                    const int valid = static_cast<int>(min(p.N - n0, static_cast<int64_t>(F::kNI)));
+                    for (int c0 = 8 * static_cast<int>(group); c0 < valid; c0 += 8 * F::kGroups)
+                        store_row_pairs<F::kNI>(p, tmem, static_cast<int>(wm), c0, valid, s.tile / p.nblocks, n0, s.slot);
+                } else {
+                    // warp w: row half (w / 4) % 2, tensor-memory lanes 32 * (w % 4).., token columns [(w / 8) * kNI / 2, + kNI / 2)
+                    const int half = (warp >> 2) & 1, cbase = (warp >> 3) * (F::kNI / 2), lane_base = 32 * (warp & 3);
+                    store_accumulators<false>(p, tmem + half * F::kNI, lane_base, cbase, cbase + F::kNI / 2, s.tile / p.nblocks, half * 128 + lane_base, n0, s.slot);
+                }
             }
             asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
             __syncwarp();
@@ -1191,7 +1361,8 @@ spdp_status run_plan(const spdp_matrix* h, Params p, const Plan& plan, const __h
     p.ptok = static_cast<int>(std::min<int64_t>(p.N, nt));
     p.kslices = 1;
     CUtensorMap xmap;
-    spdp_status st = encode_x(&xmap, X, p.N, h->K, ldx, plan.kernel == 3 ? pair::kNI / 2 : nt);
+    p.xbox = plan.kernel == 3 ? pair::kNI / 2 : (p.ptok + 15) / 16 * 16;
+    spdp_status st = encode_x(&xmap, X, p.N, h->K, ldx, p.xbox);
     if (st != SPDP_OK) return st;
     const bool cut = plan.rest > 0 && plan.sharers > plan.rest;              // partial sums and a second kernel
     if (cut) {
