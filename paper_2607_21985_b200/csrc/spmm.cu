@@ -552,12 +552,14 @@ __device__ __forceinline__ void add_partials(const Params& p, const float* first
 struct CopyState {
     unsigned i = 0, done = 0;                               // K-blocks started / known to be decoded
     uint32_t vhead = 0, vtail = 0, pos = 0;                 // virtual ring offsets, and vhead's position in the ring
+    bool refused = false;                                   // the matrix is not what the format says: nothing more is copied
 };
 // Starts the copies of K-blocks kb0 .. kb0 + n - 1 of the row tile whose first GTile is g_row.  The values of the blocks in
 // flight lie in a ring of bytes, so that the sparser the matrix, the more blocks are on their way; bitmaps and ColInfo in
 // kMeta slots.  A lane holds the TileOffset words of one K-block in 32, looks them over and says where its values start; what is left per
 // block is short, because this one warp shares its scheduler with six that decode, and each of its instructions waits for its turn.  After a
-// failure nothing is copied any more, but every block's barrier still completes.
+// failure nothing is copied any more, but every block's barrier still completes, and no sooner than its place is free: a barrier that ran two
+// phases ahead of who waits for it would look like one that has not completed.
 template <int kMeta>
 __device__ __forceinline__ bool copy_blocks(const Params& p, CopyState& c, uint32_t ring, uint32_t ring_bytes, Meta* meta, unsigned long long* full,
                                             unsigned long long* freed, int* abort, int64_t g_row, int kb0, int n, int lane, bool ok) {
@@ -579,11 +581,11 @@ __device__ __forceinline__ bool copy_blocks(const Params& p, CopyState& c, uint3
                 atomicCAS(p.status, 0, SPDP_ERR_OVERFLOW);
                 *static_cast<volatile int*>(abort) = 1;     // the outputs stay unwritten
             }
-            ok = false;
+            c.refused = true;
         }
         const int lim = min(32, n - b);
         for (int q = 0; q < lim; ++q, ++c.i) {
-            const uint32_t from = __shfl_sync(0xFFFFFFFFu, to[0], q), bytes = __shfl_sync(0xFFFFFFFFu, ok ? 2u * nvals : 0u, q);
+            const uint32_t from = __shfl_sync(0xFFFFFFFFu, to[0], q), bytes = __shfl_sync(0xFFFFFFFFu, ok && !c.refused ? 2u * nvals : 0u, q);
             if (c.pos + bytes > ring_bytes) {               // the values of a K-block stay in one piece
                 c.vhead += ring_bytes - c.pos;
                 c.pos = 0;
@@ -604,24 +606,25 @@ __device__ __forceinline__ bool copy_blocks(const Params& p, CopyState& c, uint3
                 const uint32_t at = ring + c.pos - 2u * to[0];
                 static_assert(kGTB == 4, "one store");
                 *reinterpret_cast<uint4*>(&mt.start[0]) = make_uint4(at + 2u * to[0], at + 2u * to[1], at + 2u * to[2], at + 2u * to[3]);
-                *reinterpret_cast<uint4*>(&mt.vstart) = make_uint4(c.vhead, nvals, ok ? static_cast<unsigned>(ngt) : 0u, 0u);
+                *reinterpret_cast<uint4*>(&mt.vstart) = make_uint4(c.vhead, nvals, ok && !c.refused ? static_cast<unsigned>(ngt) : 0u, 0u);
             }
             __syncwarp();
             if (elect_one()) {
-                if (ok) {
+                if (ok && !c.refused) {
                     expect_bytes(&full[m], bytes + static_cast<uint32_t>(ngt) * (kTileK * 32u + kTileK * 4u));
                     if (bytes) bulk_copy(ring + c.pos, p.values + from, bytes, &full[m]);
                     bulk_copy(smem_u32(&mt.bm[0][0]), bm, static_cast<uint32_t>(ngt) * kTileK * 32u, &full[m]);
                     bulk_copy(smem_u32(&mt.ci[0]), ci, static_cast<uint32_t>(ngt) * kTileK * 4u, &full[m]);
                 } else {
+                    *static_cast<volatile int*>(abort) = 1;
                     arrive(&full[m]);
                 }
             }
             __syncwarp();
             bm += kKB * 4;
             ci += kKB;
-            c.vhead += ok ? bytes : 0u;
-            c.pos += ok ? bytes : 0u;
+            c.vhead += bytes;
+            c.pos += bytes;
         }
 #pragma unroll
         for (int q = 0; q <= kGTB; ++q) to[q] = nxt[q];
@@ -840,7 +843,11 @@ spmm_kernel(const __grid_constant__ Params p, const __grid_constant__ CUtensorMa
                 for (int kb = 0; kb < s.n; ++kb, ++u) {
                     const unsigned sb = u % F::kBStages;
                     if (u >= F::kBStages && ok) ok = wait_parity(&sm.x_free[sb], (u / F::kBStages - 1u) & 1);
-                    if (!ok) { arrive(&sm.x_full[sb]); continue; }
+                    if (!ok) {
+                        *static_cast<volatile int*>(&sm.abort) = 1;     // before anything is multiplied with what is not there
+                        arrive(&sm.x_full[sb]);
+                        continue;
+                    }
                     expect_bytes(&sm.x_full[sb], static_cast<uint32_t>(p.xbox) * kBRowBytes);
                     tensor_copy(&sm.B[sb][0], &xmap, (s.kb0 + kb) * kKB, n0, &sm.x_full[sb]);
                 }
@@ -1004,6 +1011,7 @@ struct __align__(1024) Smem {
     alignas(8) unsigned long long comp_free[kMeta];     // my decode warps are done with the stored K-block
     alignas(8) unsigned long long ready[kStages];       // A stage s is written (first CTA: and the second CTA's)
     alignas(8) unsigned long long comp_full[kMeta];     // the stored K-block has arrived
+    alignas(8) unsigned long long drained;              // every product that was issued is complete (first CTA)
     alignas(16) uint2 tab[kWarps][32];              // per warp: bitmap word and the address of its first value
     uint32_t tmem_base;
     int abort;
@@ -1060,6 +1068,7 @@ spmm_kernel(const __grid_constant__ Params p, const __grid_constant__ CUtensorMa
             barrier_init(&sm.comp_full[s], 1);
             barrier_init(&sm.comp_free[s], kBlockWarps);
         }
+        barrier_init(&sm.drained, 1);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         sm.abort = 0;
     }
@@ -1100,12 +1109,14 @@ spmm_kernel(const __grid_constant__ Params p, const __grid_constant__ CUtensorMa
                     const uint64_t bd0 = operand_desc(smem_u32(&sm.B[x.at][0]), 16, kBAtomBytes, 2u);
                     const uint32_t id = instr_desc(256, i == ntiles - 1 ? last_tokens : kNI);
 #pragma unroll
-                    for (int kk = 0; kk < kKB / 16; ++kk)    // the start address is the descriptor's low field, in 16-byte units
+                    for (int kk = 0; ok && kk < kKB / 16; ++kk)    // the start address is the descriptor's low field, in 16-byte units
                         mma_f16_pair(tmem + i * kNI, ad0 + ((kk * 2 * kAKGroupStride) >> 4), bd0 + ((kk * 32) >> 4), id, kb > 0 || kk > 0);
                     if (kByTile<kXTiles>) commit_pair(&sm.x_done[x.at]);
                 }
                 commit_pair(&sm.mma_done[s]);
             }
+            commit_pair(&sm.drained);                                   // neither CTA frees tensor memory under running products, whatever ran out
+            ok = wait_parity(&sm.drained, 0u) && ok;
         } else if (one) {
             // ================= second CTA: tell the first when my part of a block is ready =================
             XTile x;
@@ -1132,20 +1143,33 @@ spmm_kernel(const __grid_constant__ Params p, const __grid_constant__ CUtensorMa
         if (elect_one()) {
             asm volatile("griddepcontrol.wait;" ::: "memory");          // X may come from the kernel before this one
             XTile x;
+            int copied = 0;
             for (int kb = 0; kb < nkb; ++kb)
                 for (int i = 0; i < ntiles; ++i, x.next<kXTiles>()) {       // my 128 tokens of each tile: one tiled bulk-tensor copy
                     // it goes where the tile kXTiles before was multiplied from, once that work is complete
                     unsigned long long* const full = kByTile<kXTiles> ? &sm.x_full[x.at] : &sm.ready[kb % kStages];
                     if (kByTile<kXTiles>) {
                         if (kb * ntiles + i >= kXTiles && ok) ok = wait_parity(&sm.x_done[x.at], x.parity ^ 1u);
-                        expect_bytes(full, kBTileBytes);
+                        if (ok) expect_bytes(full, kBTileBytes);
                     } else if (i == 0) {
                         if (kb >= kStages && ok) ok = wait_parity(&sm.mma_done[kb % kStages], ((kb / kStages) & 1u) ^ 1u);
-                        expect_bytes(full, static_cast<uint32_t>(ntiles) * kBTileBytes);
+                        if (ok) expect_bytes(full, static_cast<uint32_t>(ntiles) * kBTileBytes);
                     }
+                    if (!ok) {                                          // nothing is copied to a place that may be in use
+                        *static_cast<volatile int*>(&sm.abort) = 1;
+                        if (kByTile<kXTiles> || i == 0) arrive(full);
+                        continue;
+                    }
+                    ++copied;
                     tensor_copy(&sm.B[x.at][0], &xmap, (kb0 + kb) * kKB, static_cast<int>(n0) + i * kNI + c * ((i == ntiles - 1 ? last_tokens : kNI) / 2),
                                 full);
                 }
+            // the last ones have arrived, whatever ran out
+            if (kByTile<kXTiles>) {
+                for (int q = max(0, copied - kXTiles); q < copied; ++q) ok = wait_parity(&sm.x_full[q % kXTiles], (q / kXTiles) & 1) && ok;
+            } else {
+                for (int kb = max(0, copied / ntiles - kStages); kb < copied / ntiles; ++kb) ok = wait_parity(&sm.ready[kb % kStages], (kb / kStages) & 1) && ok;
+            }
         }
         __syncwarp();
     } else if (warp == kWarps + 2) {
