@@ -114,6 +114,7 @@ struct Params {
                             // piece, 1: its last); pair:: null = whole tiles
     int ptok;
     int xbox;               // one:: tokens that an X tile's copy brings
+    int cluster;            // one::, builds for clusters: CTAs of a cluster, which share a tile and add its sums themselves
     int* status;
     int64_t values_len;
 };
@@ -205,8 +206,18 @@ __device__ __forceinline__ void arrive_at(unsigned long long* bar, uint32_t rank
     asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(remote) : "r"(smem_u32(bar)), "r"(rank));
     asm volatile("mbarrier.arrive.shared::cluster.b64 _, [%0];" ::"r"(remote) : "memory");
 }
+// The cluster's barrier, for whole warps.
+__device__ __forceinline__ void cluster_arrive() {
+    __syncwarp();
+    asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+}
+__device__ __forceinline__ void cluster_wait() {
+    __syncwarp();
+    asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
 __device__ __forceinline__ void pair_sync() {
-    asm volatile("barrier.cluster.arrive.release.aligned;\n barrier.cluster.wait.acquire.aligned;" ::: "memory");
+    cluster_arrive();
+    cluster_wait();
 }
 // Bulk copy global -> shared (16-byte aligned, a multiple of 16 bytes), completing on a shared-memory barrier.
 __device__ __forceinline__ void bulk_copy(uint32_t dst, const void* src, uint32_t bytes, unsigned long long* bar) {
@@ -451,10 +462,23 @@ __device__ __forceinline__ void store_accumulators(const Params& p, uint32_t tme
     }
 }
 
+// Two neighbouring rows of a token to Y.
+__device__ __forceinline__ void store_two(const Params& p, int64_t n, int64_t row, float a, float b) {
+    const unsigned size = p.ydt == SPDP_Y_F32 ? 4u : 2u;
+    const int64_t at = n * p.ldy + row;
+    if ((p.ldy & 1) == 0 && (reinterpret_cast<uintptr_t>(p.Y) & (2u * size - 1u)) == 0 && row + 2 <= p.M) {
+        if (p.ydt == SPDP_Y_F32) *reinterpret_cast<float2*>(static_cast<float*>(p.Y) + at) = make_float2(a, b);
+        else *reinterpret_cast<__half2*>(static_cast<__half*>(p.Y) + at) = __floats2half2_rn(a, b);
+        return;
+    }
+    if (row < p.M) store_y(p.Y, p.ydt, at, a);
+    if (row + 1 < p.M) store_y(p.Y, p.ydt, at + 1, b);
+}
 // The same for the forms with W in tensor memory, where lane l of quarter q holds row 64q + 2l in the first accumulator and the row
-// after it in the second, kNI columns further: tokens [c0, c0 + 8), two neighbouring rows at once.
-template <int kNI>
-__device__ __forceinline__ void store_row_pairs(const Params& p, uint32_t tmem, int q, int c0, int valid, int r, int64_t n0, int slot) {
+// after it in the second, kNI columns further: tokens [c0, c0 + 8), two neighbouring rows at once.  Tokens [own0, own1) of partial sums go to
+// shared memory (at `own`) instead.
+template <int kNI, bool kOwn>
+__device__ __forceinline__ void store_row_pairs(const Params& p, uint32_t tmem, int q, int c0, int valid, int r, int64_t n0, int slot, int own0, int own1, uint32_t own) {
     const int lane = threadIdx.x & 31, row_in = 64 * q + 2 * lane;
     uint32_t v[8], w[8];
     tmem_load8(tmem + (static_cast<uint32_t>(32 * q) << 16) + c0, v);
@@ -462,27 +486,18 @@ __device__ __forceinline__ void store_row_pairs(const Params& p, uint32_t tmem, 
     asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
     if (slot >= 0) {
         float* part = p.partial + (static_cast<size_t>(slot) * p.ptok + c0) * kTileM + row_in;
+        const uint32_t at = own + 4u * static_cast<uint32_t>((c0 - own0) * kTileM + row_in);
 #pragma unroll
-        for (int i = 0; i < 8; ++i)
-            if (c0 + i < valid) *reinterpret_cast<float2*>(part + i * kTileM) = make_float2(__uint_as_float(v[i]), __uint_as_float(w[i]));
+        for (int i = 0; i < 8; ++i) {
+            if (kOwn && c0 + i >= own0 && c0 + i < own1) sts_v2(at + 4u * kTileM * i, v[i], w[i]);
+            else if (c0 + i < valid) *reinterpret_cast<float2*>(part + i * kTileM) = make_float2(__uint_as_float(v[i]), __uint_as_float(w[i]));
+        }
         return;
     }
     const int64_t row = static_cast<int64_t>(r) * kTileM + row_in;
-    const unsigned size = p.ydt == SPDP_Y_F32 ? 4u : 2u;
-    const bool twos = (p.ldy & 1) == 0 && (reinterpret_cast<uintptr_t>(p.Y) & (2u * size - 1u)) == 0 && row + 2 <= p.M;
 #pragma unroll
-    for (int i = 0; i < 8; ++i) {
-        if (c0 + i >= valid) break;
-        const int64_t at = (n0 + c0 + i) * p.ldy + row;
-        const float a = __uint_as_float(v[i]), b = __uint_as_float(w[i]);
-        if (twos) {
-            if (p.ydt == SPDP_Y_F32) *reinterpret_cast<float2*>(static_cast<float*>(p.Y) + at) = make_float2(a, b);
-            else *reinterpret_cast<__half2*>(static_cast<__half*>(p.Y) + at) = __floats2half2_rn(a, b);
-        } else {
-            if (row < p.M) store_y(p.Y, p.ydt, at, a);
-            if (row + 1 < p.M) store_y(p.Y, p.ydt, at + 1, b);
-        }
-    }
+    for (int i = 0; i < 8; ++i)
+        if (c0 + i < valid) store_two(p, n0 + c0 + i, row, __uint_as_float(v[i]), __uint_as_float(w[i]));
 }
 
 // A CTA that gave up fills its slots of the scratch memory with this word, so that the second kernel leaves the rows it feeds
@@ -495,6 +510,16 @@ __device__ __forceinline__ void void_rows(const Params& p, int slot, int row0, i
     for (int i = t; i < p.ptok * rows; i += nthreads) part[static_cast<size_t>(i / rows) * kTileM + row0 + i % rows] = kNoSum;
 }
 
+// A tile that a cluster shares: CTA `rank` adds up tokens [own_begin(rank), own_begin(rank + 1)), which the others have left in scratch memory.
+// What it saves is the second kernel, which waits for every CTA of the call and holds up the next call's start: 3.5 us of 4096x4096 x 128
+// tokens, 5 of 700x5000, 7 of 11008x4096 x 128.  11008x4096 at 60 % x 128, three CTAs a tile, in cluster / 129 CTAs and second kernel / 148 and second kernel
+// 26.3 / 28.8 / 31.5 us, 18944x4096 x 100 in twos 33.3 / - / 36.3, 8192x4096 x 64 in fours 19.6 / 20.7 / 22.7, 1024x1024 x 16 in eights 6.4 / 7.0 / 7.5,
+// 700x5000 x 16 in sixteens 7.9 / 8.5 / 12.9.  What bounds it is one latency behind the other: stores to L2 (3900 clocks of 11008x4096 x 128), the
+// barrier that releases them (2500), copies back (1300), additions.  Tried and slower: sums read by each thread for itself (28.0), own sums
+// left in tensor memory (27.7), stores to the other CTAs' shared memory (27.4: 12 bytes per clock and SM), sums staged in shared memory and written by bulk
+// copies with an arrival at each CTA in place of the barrier (28.4: a released remote arrival takes 400 to 800 clocks).
+__device__ __forceinline__ int own_begin(const Params& p, int rank) { return p.ptok * rank / p.cluster; }
+
 // The second kernel of a cut call: a block of 256 threads takes 4 tokens x 256 rows of a tile, a thread 4 consecutive rows of
 // one token.  What bounds it is the partial sums' way through L2, behind a launch and one chain of latencies: what a block has to know of
 // its tile is worked out once, with 32-bit divisions, and before the wait for the first kernel.  (With elements dealt out over a
@@ -506,6 +531,20 @@ constexpr int kReduceTokens = 4;
 // (16) 8.9 / 7.8, 4096x4096 x 128 (9) 18.0 / 17.3.  Sixteen are longer code, fetched for the first time in every call: 4096x4096 x 16
 // tokens 11.6 -> 13.8.
 constexpr int kFewSums = 4, kManySums = 8, kManySumsFrom = 8;
+// Four consecutive rows of token n, the first a multiple of 4.
+__device__ __forceinline__ void store_rows(const Params& p, int64_t n, int64_t row, const float4& sum) {
+    const int64_t at = n * p.ldy + row;
+    if (p.ydt != SPDP_Y_F32 && row + 4 <= p.M && ((reinterpret_cast<uintptr_t>(p.Y) + 2u * static_cast<uintptr_t>(at)) & 7u) == 0) {
+        const __half2 lo = __floats2half2_rn(sum.x, sum.y), hi = __floats2half2_rn(sum.z, sum.w);
+        *reinterpret_cast<uint2*>(static_cast<__half*>(p.Y) + at) =
+            make_uint2(*reinterpret_cast<const unsigned*>(&lo), *reinterpret_cast<const unsigned*>(&hi));
+        return;
+    }
+    const float v[4] = {sum.x, sum.y, sum.z, sum.w};
+#pragma unroll
+    for (int e = 0; e < 4; ++e)
+        if (row + e < p.M) store_y(p.Y, p.ydt, at + e, v[e]);
+}
 // Adds the partial sums of 4 rows at `first` and, count - 1 of them and `stride` floats apart, from `next` on, in this order, and
 // stores them at token n, rows row .. row + 3.
 template <int kDepth>
@@ -534,18 +573,7 @@ __device__ __forceinline__ void add_partials(const Params& p, const float* first
                 if (i < left) add(v[i]);
         }
     }
-    if (!there) return;
-    const int64_t at = n * p.ldy + row;
-    if (p.ydt != SPDP_Y_F32 && row + 4 <= p.M && ((reinterpret_cast<uintptr_t>(p.Y) + 2u * static_cast<uintptr_t>(at)) & 7u) == 0) {
-        const __half2 lo = __floats2half2_rn(sum.x, sum.y), hi = __floats2half2_rn(sum.z, sum.w);
-        *reinterpret_cast<uint2*>(static_cast<__half*>(p.Y) + at) =
-            make_uint2(*reinterpret_cast<const unsigned*>(&lo), *reinterpret_cast<const unsigned*>(&hi));
-        return;
-    }
-    const float v[4] = {sum.x, sum.y, sum.z, sum.w};
-#pragma unroll
-    for (int e = 0; e < 4; ++e)
-        if (row + e < p.M) store_y(p.Y, p.ydt, at + e, v[e]);
+    if (there) store_rows(p, n, row, sum);
 }
 
 // ---- the copy warp's work: stored K-blocks into a ring ----
@@ -642,10 +670,12 @@ __device__ __forceinline__ bool await_copies(const CopyState& c, unsigned long l
 // ===================================================================================================
 namespace one {     // one CTA = one row tile x kNI tokens
 
-template <int kNIT>
+template <int kNIT, bool kClusterT = false>
 struct Form {
     static constexpr int kNI = kNIT;                                  // the N of the tensor-core instruction = tokens per tile
     static constexpr bool kTmemW = kNI <= 128;                        // decoded W in tensor memory, where there is room for it
+    static constexpr bool kCluster = kClusterT;                       // clusters share tiles; a build of its own, whose code costs the others up to 2 %
+    static_assert(!kCluster || kTmemW, "only with W in tensor memory");
     static constexpr int kGroupWarps = kTmemW ? 4 : spdp::kGroupWarps;
     static constexpr int kGroups = kWarps / kGroupWarps;
     static constexpr int kTmemCols = kTmemW ? 512 : 2 * kNI;          // two accumulators (of 128 rows each), and W
@@ -715,6 +745,7 @@ struct __align__(1024) Smem {
     alignas(8) unsigned long long acc_full;         // the piece's products are complete
     alignas(8) unsigned long long acc_free;         // its accumulators have been stored
     alignas(8) unsigned long long drained;          // every product that was issued is complete
+    alignas(8) unsigned long long gathered;         // the cluster's other sums of my tokens have arrived
     uint32_t tmem_base;
     int abort;
     alignas(128) unsigned char ring[1];             // values of the K-blocks in flight (fills the rest): the sparser the
@@ -731,10 +762,14 @@ template <class F>
 __global__ void __launch_bounds__(kLaunchBound, 1)
 spmm_kernel(const __grid_constant__ Params p, const __grid_constant__ CUtensorMap xmap) {
     static_assert(kRingBytes<F> >= 2 * kKB * kTileM * 2, "the ring holds at least two full K-blocks");
+    static_assert(!F::kTmemW || (kRingBytes<F> >= plan::kGatherTokens * kTileM * sizeof(float) && sizeof(Smem<F>::B) >= F::kNI / 2 * kTileM * sizeof(float)),
+                  "and a cluster's sums, those of the CTA's own tokens where the X tiles were");
     extern __shared__ unsigned char smem_raw[];
     Smem<F>& sm = *reinterpret_cast<Smem<F>*>(smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u));
     const int t = threadIdx.x, lane = t & 31, warp = __shfl_sync(0xFFFFFFFFu, t >> 5, 0);      // the same in all lanes, and known to be
     const int me = static_cast<int>(blockIdx.x);
+    constexpr bool shared_tile = F::kCluster;                         // this CTA's work is one slice of one tile
+    const int rank = shared_tile ? me % p.cluster : 0;
 
     // ---- set-up: the barriers and tensor memory ----
     if (t == 0) {
@@ -756,6 +791,7 @@ spmm_kernel(const __grid_constant__ Params p, const __grid_constant__ CUtensorMa
         barrier_init(&sm.acc_full, 1);
         barrier_init(&sm.acc_free, F::kStorers);
         barrier_init(&sm.drained, 1);
+        barrier_init(&sm.gathered, 1);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         sm.abort = 0;
     }
@@ -923,17 +959,28 @@ spmm_kernel(const __grid_constant__ Params p, const __grid_constant__ CUtensorMa
             if (ok) ok = wait_parity(&sm.acc_full, k & 1);
             asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
             ok = __all_sync(0xFFFFFFFFu, ok);
-            if (ok && !__any_sync(0xFFFFFFFFu, *static_cast<volatile int*>(&sm.abort) != 0)) {
+            const bool complete = ok && !__any_sync(0xFFFFFFFFu, *static_cast<volatile int*>(&sm.abort) != 0);
+            if (complete) {
                 const int64_t n0 = static_cast<int64_t>(s.tile % p.nblocks) * F::kNI;
                 if constexpr (F::kTmemW) {
                     const int valid = static_cast<int>(min(p.N - n0, static_cast<int64_t>(F::kNI)));
+                    const int own0 = shared_tile ? own_begin(p, rank) : 0, own1 = shared_tile ? own_begin(p, rank + 1) : 0;
                     for (int c0 = 8 * static_cast<int>(group); c0 < valid; c0 += 8 * F::kGroups)
-                        store_row_pairs<F::kNI>(p, tmem, static_cast<int>(wm), c0, valid, s.tile / p.nblocks, n0, s.slot);
+                        store_row_pairs<F::kNI, shared_tile>(p, tmem, static_cast<int>(wm), c0, valid, s.tile / p.nblocks, n0, s.slot, own0, own1, smem_u32(&sm.B[0][0]));
                 } else {
                     // warp w: row half (w / 4) % 2, tensor-memory lanes 32 * (w % 4).., token columns [(w / 8) * kNI / 2, + kNI / 2)
                     const int half = (warp >> 2) & 1, cbase = (warp >> 3) * (F::kNI / 2), lane_base = 32 * (warp & 3);
                     store_accumulators<false>(p, tmem + half * F::kNI, lane_base, cbase, cbase + F::kNI / 2, s.tile / p.nblocks, half * 128 + lane_base, n0, s.slot);
                 }
+            }
+            if constexpr (shared_tile) {
+                if (!complete) {                                       // nobody may add what I have not stored
+                    *static_cast<volatile int*>(&sm.abort) = 1;
+                    for (int c = static_cast<int>(group); c < p.ptok; c += F::kGroups)
+                        for (int e = lane; e < 64; e += 32)
+                            reinterpret_cast<unsigned*>(p.partial)[(static_cast<size_t>(s.slot) * p.ptok + c) * kTileM + 64 * wm + e] = kNoSum;
+                }
+                break;
             }
             asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
             __syncwarp();
@@ -946,9 +993,55 @@ spmm_kernel(const __grid_constant__ Params p, const __grid_constant__ CUtensorMa
         atomicCAS(p.status, 0, SPDP_ERR_TIMEOUT);
     }
     __syncwarp();
+    if constexpr (shared_tile) {
+        // ---- my tokens of the tile: my own sums are where the X tiles were, the other CTAs' come, by one bulk copy for each, to where
+        // the values were; they are added in CTA order ----
+        asm volatile("fence.proxy.async.global;" ::: "memory");       // sums were written through the generic proxy, the copies read through the async one
+        cluster_arrive();                                             // (every warp of the cluster gets here, whatever it gave up)
+        piece(p, me, 0, s);
+        const int64_t n0 = static_cast<int64_t>(s.tile % p.nblocks) * F::kNI;
+        const int own0 = own_begin(p, rank), own1 = static_cast<int>(min(static_cast<int64_t>(own_begin(p, rank + 1)), p.N - n0));
+        const uint32_t part_bytes = static_cast<uint32_t>(max(own1 - own0, 0)) * kTileM * 4u;
+        cluster_wait();
+        if (*static_cast<volatile int*>(&sm.abort) == 0 && own0 < own1) {
+            if (warp == kWarps + 1) {
+                if (elect_one()) {
+                    asm volatile("fence.proxy.async.global;" ::: "memory");
+                    expect_bytes(&sm.gathered, static_cast<uint32_t>(p.cluster - 1) * part_bytes);
+                    uint32_t to = smem_u32(&sm.ring[0]);
+                    for (int r = 0; r < p.cluster; ++r) {
+                        if (r == rank) continue;
+                        bulk_copy(to, p.partial + (static_cast<size_t>(2 * (me - rank + r)) * p.ptok + own0) * kTileM, part_bytes, &sm.gathered);
+                        to += part_bytes;
+                    }
+                }
+                __syncwarp();
+            }
+            ok = wait_parity(&sm.gathered, 0u);
+            const int64_t row0 = static_cast<int64_t>(s.tile / p.nblocks) * kTileM;
+            const uint32_t own = smem_u32(&sm.B[0][0]) - static_cast<uint32_t>(rank) * part_bytes, before = smem_u32(&sm.ring[0]), behind = before - part_bytes;
+            // 4 rows of a token at a time, by all threads
+#pragma unroll 1
+            for (uint32_t i = 16u * t; i < part_bytes; i += 16u * kThreads) {
+                float4 sum = make_float4(-0.f, -0.f, -0.f, -0.f);     // x + -0 is x, whatever x is
+                bool there = ok;
+#pragma unroll 4
+                for (int r = 0; r < p.cluster; ++r) {
+                    const uint4 v = lds_v4<0>((r == rank ? own : r < rank ? before : behind) + static_cast<uint32_t>(r) * part_bytes + i);
+                    there = there && v.w != kNoSum;
+                    sum.x += __uint_as_float(v.x);
+                    sum.y += __uint_as_float(v.y);
+                    sum.z += __uint_as_float(v.z);
+                    sum.w += __uint_as_float(v.w);
+                }
+                if (there) store_rows(p, n0 + own0 + static_cast<int>(i / (4u * kTileM)), row0 + (i / 4u) % kTileM, sum);
+            }
+        }
+        if (!ok) atomicCAS(p.status, 0, SPDP_ERR_TIMEOUT);
+    }
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
-    if (*static_cast<volatile int*>(&sm.abort) != 0 && p.partial != nullptr && me < p.sharers) {
+    if (*static_cast<volatile int*>(&sm.abort) != 0 && p.partial != nullptr && me < p.sharers && !shared_tile) {
         void_rows(p, 2 * me, 0, kTileM, t, kThreads);
         void_rows(p, 2 * me + 1, 0, kTileM, t, kThreads);
         __syncwarp();
@@ -1264,8 +1357,41 @@ reduce_slices_kernel(const Params p, int chunks) {
 
 using One32 = one::Form<32>;
 using One128 = one::Form<128>;
+using Cluster32 = one::Form<32, true>;
+using Cluster128 = one::Form<128, true>;
 using One256 = one::Form<256>;
 
+}  // namespace
+
+namespace {
+// Clusters of c CTAs of the forms with W in tensor memory that the device holds at once, per device and c.  They differ from part to part: a cluster lies
+// within a group of SMs, and these are not equally large.  Written once, before the device's first handle exists.
+int g_resident[64][plan::kMaxCluster + 1];
+
+spdp_status resident_clusters(int dev) {
+    for (const auto kernel : {one::spmm_kernel<Cluster32>, one::spmm_kernel<Cluster128>}) {
+        SPDP_CUDA_TRY(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, one::kSmemBytes));
+        SPDP_CUDA_TRY(cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
+    }
+    for (int c = 2; c <= plan::kMaxCluster; ++c) {
+        cudaLaunchConfig_t cfg = {};
+        cfg.gridDim = dim3(static_cast<unsigned>(c));
+        cfg.blockDim = dim3(kThreads);
+        cfg.dynamicSmemBytes = one::kSmemBytes;
+        cudaLaunchAttribute attr[1];
+        attr[0].id = cudaLaunchAttributeClusterDimension;
+        attr[0].val.clusterDim.x = static_cast<unsigned>(c);
+        attr[0].val.clusterDim.y = 1;
+        attr[0].val.clusterDim.z = 1;
+        cfg.attrs = attr;
+        cfg.numAttrs = 1;
+        if (cudaOccupancyMaxActiveClusters(&g_resident[dev][c], one::spmm_kernel<Cluster128>, &cfg) != cudaSuccess) {
+            (void)cudaGetLastError();                       // none of this size
+            g_resident[dev][c] = 0;
+        }
+    }
+    return SPDP_OK;
+}
 }  // namespace
 
 spdp_status configure_spmm_kernel() {
@@ -1281,6 +1407,8 @@ spdp_status configure_spmm_kernel() {
         SPDP_CUDA_TRY(cudaFuncSetAttribute(one::spmm_kernel<One256>, cudaFuncAttributeMaxDynamicSharedMemorySize, one::kSmemBytes));
         SPDP_CUDA_TRY(cudaFuncSetAttribute(pair::spmm_kernel<4>, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(pair::kSmemBytes)));
         SPDP_CUDA_TRY(cudaFuncSetAttribute(pair::spmm_kernel<6>, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(pair::kSmemBytes)));
+        const spdp_status st = resident_clusters(dev);
+        if (st != SPDP_OK) return st;
         configured[dev] = true;
     }
     return SPDP_OK;
@@ -1331,11 +1459,15 @@ spdp_status launch_one(const Params& p, const CUtensorMap& xmap, cudaStream_t s)
     cfg.blockDim = dim3(kThreads);
     cfg.dynamicSmemBytes = one::kSmemBytes;
     cfg.stream = s;
-    cudaLaunchAttribute attr[1];
+    cudaLaunchAttribute attr[2];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
+    attr[1].id = cudaLaunchAttributeClusterDimension;
+    attr[1].val.clusterDim.x = static_cast<unsigned>(p.cluster);
+    attr[1].val.clusterDim.y = 1;
+    attr[1].val.clusterDim.z = 1;
     cfg.attrs = attr;
-    cfg.numAttrs = 1;
+    cfg.numAttrs = F::kCluster ? 2 : 1;
     SPDP_CUDA_TRY(cudaLaunchKernelEx(&cfg, one::spmm_kernel<F>, p, xmap));
     return SPDP_OK;
 }
@@ -1384,6 +1516,7 @@ spdp_status run_plan(const spdp_matrix* h, Params p, const Plan& plan, const __h
     p.nblocks = static_cast<int>((p.N + nt - 1) / nt);
     p.ptok = static_cast<int>(std::min<int64_t>(p.N, nt));
     p.kslices = 1;
+    p.cluster = plan.cluster;
     CUtensorMap xmap;
     p.xbox = plan.kernel == 3 ? pair::kNI / 2 : (p.ptok + 15) / 16 * 16;
     spdp_status st = encode_x(&xmap, X, p.N, h->K, ldx, p.xbox);
@@ -1412,8 +1545,9 @@ spdp_status run_plan(const spdp_matrix* h, Params p, const Plan& plan, const __h
         p.rounds = plan.rounds;
         p.sharers = plan.sharers;
         p.rest_units = static_cast<unsigned>(plan.rest * p.nkb);
-        st = plan.kernel == 0 ? launch_one<One32>(p, xmap, s) : plan.kernel == 1 ? launch_one<One128>(p, xmap, s) : launch_one<One256>(p, xmap, s);
-        if (st == SPDP_OK && cut)
+        if (plan.cluster > 1) st = plan.kernel == 0 ? launch_one<Cluster32>(p, xmap, s) : launch_one<Cluster128>(p, xmap, s);
+        else st = plan.kernel == 0 ? launch_one<One32>(p, xmap, s) : plan.kernel == 1 ? launch_one<One128>(p, xmap, s) : launch_one<One256>(p, xmap, s);
+        if (st == SPDP_OK && cut && plan.cluster == 1)
             st = launch_reduce(many ? one::reduce_pieces_kernel<kManySums> : one::reduce_pieces_kernel<kFewSums>, plan.rest, chunks, s, p, plan.rounds * plan.workers, chunks, nt);
     }
     if (cut) cudaFreeAsync(p.partial, s);
@@ -1440,7 +1574,7 @@ spdp_status launch_spmm(const spdp_matrix* h, const __half* X, int64_t N, int64_
     p.values_len = h->values_len;
     p.nkb = static_cast<int>((h->K + kKB - 1) / kKB);
     const int sms = h->sm_count > 1 ? h->sm_count : 2;
-    spdp_status st = run_plan(h, p, make_plan(h->R, p.nkb, N, sms, true), X, ldx, s);
+    spdp_status st = run_plan(h, p, make_plan(h->R, p.nkb, N, sms, true, g_resident[h->device]), X, ldx, s);
     // No memory for partial sums: whole tiles only, which need none.  Slower, and another order of the sums.
     if (st == SPDP_ERR_ALLOC) st = run_plan(h, p, make_plan(h->R, p.nkb, N, sms, false), X, ldx, s);
     return st;

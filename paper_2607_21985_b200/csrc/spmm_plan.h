@@ -25,7 +25,10 @@ struct Plan {
     int kernel;
     int workers, rounds, sharers, slices;
     int64_t tiles, rest;
+    int cluster;            // CTAs to a tile that add its sums themselves, 1: a second kernel does
 };
+constexpr int kMaxCluster = 16;                                         // CTAs
+constexpr int kGatherTokens = 126;      // tokens' sums (of 256 rows) that a CTA of a cluster has room for
 // The estimate of a call's time: (K-blocks of the busiest CTA) x (time of a K-block) + a tile's start and end + what the
 // partial sums cost.  Fitted to the four kernels' times, calls in a row on a stream, on 10 layers from 512x512 to 28672x8192
 // (30 to 80 % sparse) with 16 to 1024 tokens each, when pairs waited for the kernel before (most of their fixed part below) and the second kernel took 1.5
@@ -39,7 +42,10 @@ constexpr double kBlockTokenUs[4] = {8.3e-4, 1.8e-4, 0.0, 4.8e-4};      // and p
 constexpr double kTileUs = 2.1, kTileTokenUs = 2.3e-3;                  // a tile's start and end, and per token
 constexpr double kReduceUs = 1.9, kReducePerMB = 0.223;                 // the second kernel; writing and reading a MB of partial sums
 
-inline Plan make_plan(int64_t R, int64_t nkb, int64_t N, int sms, bool may_cut) {
+constexpr double kClusterUs = 1.0, kClusterPerMB = 0.15;                // the same within clusters
+
+// resident[c]: clusters of c CTAs that the device holds at once, or null: no clusters.
+inline Plan make_plan(int64_t R, int64_t nkb, int64_t N, int sms, bool may_cut, const int* resident = nullptr) {
     Plan best = {};
     best.us = -1.0;
     for (int f = 0; f < 4; ++f) {
@@ -53,6 +59,7 @@ inline Plan make_plan(int64_t R, int64_t nkb, int64_t N, int sms, bool may_cut) 
         const double whole = kCallUs[f] + (block * static_cast<double>(nkb) + tile) * static_cast<double>(rounds);
         q.rounds = static_cast<int>(rounds);
         q.slices = 1;
+        q.cluster = 1;
         q.sharers = left > 0 ? static_cast<int>(left) : 1;
         q.workers = static_cast<int>(rounds > 0 ? slots : left);
         q.rest = f == 3 ? 0 : left;
@@ -76,6 +83,16 @@ inline Plan make_plan(int64_t R, int64_t nkb, int64_t N, int sms, bool may_cut) 
         for (int64_t share = 2 * left; share < slots; share *= 2) consider(share);
         consider(slots / left * left);                                           // the most that do not cross tiles
         if (f != 3) consider(slots);
+        if (resident == nullptr || rounds > 0 || f > 1) continue;                // (the forms with W in tensor memory)
+        for (int c = 2; c <= kMaxCluster && c <= nkb; ++c) {
+            const int64_t tokens = std::min<int64_t>(N, kTokens[f]);             // a CTA adds up to a c-th of them, which come from all others
+            if (left > resident[c] || (c - 1) * ((tokens + c - 1) / c) > kGatherTokens) continue;
+            q.sharers = q.workers = static_cast<int>(c * left);
+            q.rest = left;
+            q.cluster = c;
+            q.us = kCallUs[f] + block * static_cast<double>((nkb + c - 1) / c) + tile + kClusterUs + kClusterPerMB * mb * static_cast<double>(q.sharers - left);
+            if (q.us < best.us) best = q;
+        }
     }
     return best;
 }
