@@ -37,10 +37,15 @@
 //           the whole call: whole rounds of tiles first, one tile per CTA; the K-blocks of the tiles that are left are cut
 //           into equal contiguous ranges, one per CTA.  A tile fed by several CTAs leaves fp32 partial sums in scratch
 //           memory, which a second kernel adds in CTA order (the result does not depend on timing).
+//           Where the CTAs of all tiles fit the device as clusters, those of a tile add its sums themselves.
 //   pair::  two CTAs on neighbouring SMs (a cluster of 2) = one row tile x 512 tokens: tcgen05.mma.cta_group::2
 //           multiplies M = 256 (128 rows from each CTA's shared memory) by N = 256 (128 tokens from each CTA's shared
 //           memory) and leaves 128 rows x 256 fp32 columns in each CTA's tensor memory; two such accumulators fill the
-//           512 columns.  Each CTA decodes only ITS 128 rows of every column tile: half the decode per token.
+//           512 columns.  Each CTA decodes only ITS 128 rows of every column tile: half the decode per token.  With decoded W in
+//           tensor memory a tile has up to 384 tokens (two accumulators of 192, or one of 256) and the decode takes half the
+//           instructions: 4001x4098 x 300 tokens 28.2 -> 25.2 us, 18944x4096 x 150 / 384 47.3 -> 41.6 / 58.2 -> 55.1, 16128x8192 x 316
+//           101 -> 91.  For 385 to 512 and 769 to 1024 tokens that is one tile more, and W in shared memory is faster
+//           (28672x8192 x 512 / 1024 259 -> 215 / 460 -> 407).
 #include <cuda.h>
 
 #include <algorithm>
@@ -92,6 +97,10 @@ constexpr int kBAtomBytes = 8 * kBRowBytes;
 constexpr int kWaitTries = SPDP_SPMM_WAIT_TRIES;
 static_assert(kBRowBytes == 128, "one X row of a K-block is one 128-byte swizzle row");
 
+// 64 registers a thread, which leaves room for a block of the second kernel beside a CTA (with 72, as for kThreads alone, 0.5 % more time
+// over 7 layers x 4 token counts).
+constexpr int kLaunchBound = 1024;
+
 struct Params {
     const uint32_t* tileoffset;
     const uint32_t* colinfo;
@@ -110,6 +119,7 @@ struct Params {
     unsigned rest_units;
     // pair:: pair i works on tile tile0 + i / kslices, on slice i % kslices of the tile's K-blocks
     int tile0, kslices;
+    int acc_tokens, tile_tokens;    // tokens of an accumulator, and of a tile
     float* partial;         // partial sums [slot][token in tile < ptok][256 rows]; slot = pair i, or 2 * CTA + (0: its first
                             // piece, 1: its last); pair:: null = whole tiles
     int ptok;
@@ -158,6 +168,11 @@ __device__ __forceinline__ void mma_f16_pair(uint32_t d_tmem, uint64_t a_desc, u
     asm volatile("{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
                  " tcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %3, p;\n}"
                  ::"r"(d_tmem), "l"(a_desc), "l"(b_desc), "r"(instr_desc), "r"(accumulate ? 1u : 0u) : "memory");
+}
+__device__ __forceinline__ void mma_f16_pair_tmem(uint32_t d_tmem, uint32_t a_tmem, uint64_t b_desc, uint32_t instr_desc, bool accumulate) {
+    asm volatile("{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
+                 " tcgen05.mma.cta_group::2.kind::f16 [%0], [%1], %2, %3, p;\n}"
+                 ::"r"(d_tmem), "r"(a_tmem), "l"(b_desc), "r"(instr_desc), "r"(accumulate ? 1u : 0u) : "memory");
 }
 // Lets `bar` complete when the products this thread has issued so far are done.
 __device__ __forceinline__ void commit_one(unsigned long long* bar) {
@@ -395,6 +410,49 @@ __device__ __forceinline__ void expand_rows(uint32_t tab_l, unsigned top, unsign
     }
 }
 
+// The same for a CTA pair, where a CTA has 128 rows of the tile and a lane one of them: lane = column j of the K-block, bitmap word `w` of
+// the column's half `half`.
+struct Eighth {
+    int half, w, k0, k1, k2, k3;                // values before word w of the half: from its end (half 1) or its begin
+    __device__ __forceinline__ Eighth(int half_, int w_) : half(pinned(half_)), w(pinned(w_)) {
+        k0 = half ? (w <= 0 ? -1 : 0) : (w > 0 ? 1 : 0);
+        k1 = half ? (w <= 1 ? -1 : 0) : (w > 1 ? 1 : 0);
+        k2 = half ? (w <= 2 ? -1 : 0) : (w > 2 ? 1 : 0);
+        k3 = half ? -1 : 0;
+    }
+};
+__device__ __forceinline__ void scan_eighth(const Params& p, const Meta& mt, int j, const Eighth& q, uint32_t tab) {
+    const uint32_t ciw = mt.ci[j];
+    uint4 w = *reinterpret_cast<const uint4*>(&mt.bm[j][4 * q.half]);
+    uint32_t first = mt.start[j >> 4] + 2u * (ciw >> 16);
+    const bool there = (j >> 4) < mt.ngt && SPDP_CHECK(p.status, (first - mt.start[0]) / 2u, ciw & 0xFFFFu, mt.limit, kSiteValuesSpan);
+    if (!there) {
+        w = make_uint4(0u, 0u, 0u, 0u);
+        first = mt.start[0];
+    }
+    const int before = static_cast<int>(there ? ciw & 0xFFFFu : 0u) * q.half + __popc(w.x) * q.k0 + __popc(w.y) * q.k1 + __popc(w.z) * q.k2 + __popc(w.w) * q.k3;
+    sts_v2(tab, q.w < 2 ? (q.w == 0 ? w.x : w.y) : (q.w == 2 ? w.z : w.w), first + 2u * static_cast<unsigned>(before));
+}
+// Expands 16 columns x 32 rows: out[i] holds columns 2i and 2i + 1 of the lane's row; top = 1 << (31 - lane) puts the row's bit on top of the
+// word and leaves the bits below, so that a popcount leads past its value.  6 instructions per column and 32 rows where the expansion into
+// shared memory takes 11 for as many, one wavefront of values and half a one of the table.
+__device__ __forceinline__ void expand_row(uint32_t tab, unsigned top, unsigned two, uint32_t (&out)[8]) {
+#pragma unroll
+    for (int c0 = 0; c0 < 16; c0 += 8) {
+        unsigned has[4], v[8];
+#pragma unroll
+        for (int c = 0; c < 8; c += 2) {
+            const uint4 e = lds_v4<0>(tab + 8u * (c0 + c));
+            const unsigned s0 = e.x * top, s1 = e.z * top;
+            v[c] = lds_u16_at<-2>(e.y + two * __popc(s0));
+            v[c + 1] = lds_u16_at<-2>(e.w + two * __popc(s1));
+            has[c / 2] = permute(s0, s1, 0xFFBBu);
+        }
+#pragma unroll
+        for (int c = 0; c < 8; c += 2) out[(c0 + c) / 2] = (v[c + 1] * 65536u + v[c]) & has[c / 2];
+    }
+}
+
 // Turns 4 values of each of 4 neighbouring lanes: lane l's v[i] becomes what lane (l & ~3) + i had in v[l & 3].
 __device__ __forceinline__ void transpose4(uint32_t& v0, uint32_t& v1, uint32_t& v2, uint32_t& v3, int lane) {
     const bool odd = (lane & 1) != 0, upper = (lane & 2) != 0;
@@ -426,13 +484,13 @@ __device__ __forceinline__ void store_four(void* Y, int ydt, int64_t at, float a
 // stores gain nothing by it, and are 1 to 2 % slower with the longer code.
 template <bool kFours>
 __device__ __forceinline__ void store_accumulators(const Params& p, uint32_t tmem, int lane_base, int c_begin, int c_end,
-                                                   int r, int row_in, int64_t n0, int slot) {
+                                                   int r, int row_in, int64_t n0, int slot, int tok0 = 0) {
     const int lane = threadIdx.x & 31;
     const int valid = static_cast<int>(min(p.N - n0, static_cast<int64_t>(c_end)));
     const int64_t row0 = static_cast<int64_t>(r) * kTileM + row_in;
     const bool fours = kFours && slot < 0 && y_in_fours(p) && row0 + 32 <= p.M;
     const int64_t row = row0 + (fours ? lane & ~3 : lane);
-    float* part = p.partial + (static_cast<size_t>(slot < 0 ? 0 : slot) * p.ptok) * kTileM + row_in + lane;
+    float* part = p.partial + (static_cast<size_t>(slot < 0 ? 0 : slot) * p.ptok + tok0) * kTileM + row_in + lane;
     for (int c0 = c_begin; c0 < valid; c0 += 16) {
         uint32_t v[16];
         asm volatile("tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%16];"
@@ -755,9 +813,6 @@ constexpr uint32_t kSmemBytes = kSmemKB * 1024u;    // the dynamic shared memory
 template <class F>
 constexpr uint32_t kRingBytes = (kSmemBytes - 1024u - static_cast<uint32_t>(offsetof(Smem<F>, ring)) - 64u) / 128u * 128u;
 
-// 64 registers a thread, which leaves room for a block of the second kernel beside a CTA (with 72, as for kThreads alone, 0.5 % more time
-// over 7 layers x 4 token counts).
-constexpr int kLaunchBound = 1024;
 template <class F>
 __global__ void __launch_bounds__(kLaunchBound, 1)
 spmm_kernel(const __grid_constant__ Params p, const __grid_constant__ CUtensorMap xmap) {
@@ -1074,14 +1129,18 @@ reduce_pieces_kernel(const Params p, int tile0, int chunks, int tile_tokens) {
 // ===================================================================================================
 namespace pair {    // two CTAs (a cluster of 2) = one row tile x 512 tokens
 
-constexpr int kNI = 256;                      // the N of the tensor-core instruction
+constexpr int kNI = 256;                      // the N of the tensor-core instruction, at most
 constexpr int kTmemCols = 512;
+constexpr int kWCols = 128;                   // of them for decoded W, where it is in tensor memory: then two accumulators have 192 tokens each, or one 256
+static_assert(plan::kPairAccTokens == kNI && 2 * plan::kPairHalfTokens + kWCols == kTmemCols, "the plan counts in the kernel's accumulators");
 constexpr int kATileBytes = (kKB / 8) * kAKGroupStride;    // 128 rows x kKB columns
 constexpr int kThreads = (kWarps + 4) * 32;   // decode, tensor-core, copy, relay and X warps
 constexpr int kNTiles = 2;                    // accumulators per CTA
 constexpr int kNT = kNTiles * kNI;            // tokens per CTA pair
-constexpr int kStages = 3;                    // decoded W in flight
-constexpr int kMeta = 6;                      // stored K-blocks in flight, at most
+template <bool kTmemW>
+constexpr int kStages = kTmemW ? 4 : 3;       // decoded K-blocks in flight
+template <bool kTmemW>
+constexpr int kMeta = kTmemW ? 8 : 6;         // stored K-blocks in flight, at most
 constexpr int kBTileBytes = (kNI / 2) * kBRowBytes;    // this CTA's 128 tokens of one X tile
 static_assert(kNTiles * kNI == kTmemCols, "the accumulators fill tensor memory");
 
@@ -1091,19 +1150,19 @@ static_assert(kNTiles * kNI == kTmemCols, "the accumulators fill tensor memory")
 // 406 -> 386, 11008x4096 x 1024 92.9 -> 88.5, 18944x4096 x 512 71.6 -> 67.5; called without a pause, 28672x8192 x 1024 at the power
 // limit 471 -> 455.  Six, for sparse layers, are handed on with their K-block: more barriers cost 3 % there (18944x4096 x 512
 // at 90 % 60.5 / 64.4), five instead of four gain nothing.
-template <int kXTiles>
-constexpr bool kByTile = kXTiles < 2 * kStages;
-template <int kXTiles>
+template <int kXTiles, bool kTmemW>
+constexpr bool kByTile = kTmemW || kXTiles < 2 * kStages<false>;
+template <int kXTiles, bool kTmemW>
 struct __align__(1024) Smem {
     unsigned char B[kXTiles][kBTileBytes];          // my halves of the X tiles (each on a 1024-byte boundary: swizzle atoms)
-    unsigned char A[kStages][kATileBytes];          // decoded W: my 128 rows
-    Meta meta[kMeta];
-    alignas(8) unsigned long long mma_done[kStages];    // the tensor cores are done with A stage s (both CTAs)
+    alignas(16) unsigned char A[kTmemW ? 1 : kStages<false>][kTmemW ? 16 : kATileBytes];      // decoded W: my 128 rows
+    Meta meta[kMeta<kTmemW>];
+    alignas(8) unsigned long long mma_done[kStages<kTmemW>];    // the tensor cores are done with A stage s (both CTAs)
     alignas(8) unsigned long long x_done[kXTiles];      // they are done with the X tile
     alignas(8) unsigned long long x_full[kXTiles];      // my half of the X tile has arrived (first CTA: and the second CTA's)
-    alignas(8) unsigned long long comp_free[kMeta];     // my decode warps are done with the stored K-block
-    alignas(8) unsigned long long ready[kStages];       // A stage s is written (first CTA: and the second CTA's)
-    alignas(8) unsigned long long comp_full[kMeta];     // the stored K-block has arrived
+    alignas(8) unsigned long long comp_free[kMeta<kTmemW>];     // my decode warps are done with the stored K-block
+    alignas(8) unsigned long long ready[kStages<kTmemW>];       // A stage s is written (first CTA: and the second CTA's)
+    alignas(8) unsigned long long comp_full[kMeta<kTmemW>];     // the stored K-block has arrived
     alignas(8) unsigned long long drained;              // every product that was issued is complete (first CTA)
     alignas(16) uint2 tab[kWarps][32];              // per warp: bitmap word and the address of its first value
     uint32_t tmem_base;
@@ -1113,8 +1172,8 @@ struct __align__(1024) Smem {
                                                         // 28672x8192 x 1024 at 50 % 410 us, this 397
 };
 constexpr size_t kSmemBytes = kSmemKB * 1024;           // the dynamic shared memory is aligned by hand
-template <int kXTiles>
-constexpr uint32_t kRingBytes = (static_cast<uint32_t>(kSmemBytes) - 1024u - static_cast<uint32_t>(offsetof(Smem<kXTiles>, ring)) - 64u) / 128u * 128u;
+template <int kXTiles, bool kTmemW, class SmemOf = Smem<kXTiles, kTmemW>>
+constexpr uint32_t kRingBytes = (static_cast<uint32_t>(kSmemBytes) - 1024u - static_cast<uint32_t>(offsetof(SmemOf, ring)) - 64u) / 128u * 128u;
 static_assert(kBTileBytes % 1024 == 0, "every X tile on a swizzle-atom boundary");
 
 struct XTile {                                          // place of an X tile in the ring of tiles, and its barriers' parity
@@ -1125,23 +1184,26 @@ struct XTile {                                          // place of an X tile in
     }
 };
 
-template <int kXTiles>
-__global__ void __launch_bounds__(kThreads, 1)
+template <int kXTiles, bool kTmemW>
+__global__ void __launch_bounds__(kTmemW ? kLaunchBound : kThreads, 1)
 spmm_kernel(const __grid_constant__ Params p, const __grid_constant__ CUtensorMap xmap) {
-    static_assert(kRingBytes<kXTiles> >= 2 * kKB * kTileM, "the ring holds at least one full K-block");
+    static_assert(kRingBytes<kXTiles, kTmemW> >= 2 * kKB * kTileM, "the ring holds at least one full K-block");
     extern __shared__ unsigned char smem_raw[];
-    Smem<kXTiles>& sm = *reinterpret_cast<Smem<kXTiles>*>(smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u));
-    const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
+    Smem<kXTiles, kTmemW>& sm = *reinterpret_cast<Smem<kXTiles, kTmemW>*>(smem_raw + ((1024u - (smem_u32(smem_raw) & 1023u)) & 1023u));
+    const int t = threadIdx.x, lane = t & 31, warp = __shfl_sync(0xFFFFFFFFu, t >> 5, 0);
+    constexpr int kMeta = pair::kMeta<kTmemW>, kStages = pair::kStages<kTmemW>, kColumnWarps = kTmemW ? kBlockWarps / 2 : kBlockWarps;    // decode warps that have a part of a K-block
     const int c = static_cast<int>(blockIdx.x & 1u);                  // my rank in the pair = my half of the row tile
     const unsigned pr = blockIdx.x >> 1;
     const unsigned tile = static_cast<unsigned>(p.tile0) + pr / static_cast<unsigned>(p.kslices);
     const int slice = static_cast<int>(pr % static_cast<unsigned>(p.kslices));
     const int r = static_cast<int>(tile / static_cast<unsigned>(p.nblocks));
     const int nb = static_cast<int>(tile - static_cast<unsigned>(r) * static_cast<unsigned>(p.nblocks));
-    const int64_t n0 = static_cast<int64_t>(nb) * kNT;
-    const int ntiles = (p.N - n0 > kNI) ? 2 : 1;                      // accumulators in use
+    const int64_t n0 = static_cast<int64_t>(nb) * p.tile_tokens;
+    const int acc = p.acc_tokens;                                     // tokens of an accumulator
+    const int ntiles = (p.tile_tokens > acc && p.N - n0 > acc) ? 2 : 1;      // accumulators in use
+    constexpr uint32_t kNextAcc = kTmemW ? plan::kPairHalfTokens : kNI;      // tensor-memory columns from one to the other
     // the last one's tokens, in the units of the instruction: half of them in each CTA's X tile
-    const int last_tokens = min(kNI, static_cast<int>((min(p.N - n0, static_cast<int64_t>(kNT)) - (ntiles - 1) * kNI + 31) / 32) * 32);
+    const int last_tokens = min(acc, static_cast<int>((min(p.N - n0, static_cast<int64_t>(p.tile_tokens)) - (ntiles - 1) * acc + 31) / 32) * 32);
 
     // ---- set-up: the barriers, and tensor memory (both CTAs of the pair allocate together) ----
     if (t == 0) {
@@ -1149,7 +1211,7 @@ spmm_kernel(const __grid_constant__ Params p, const __grid_constant__ CUtensorMa
         for (int s = 0; s < kStages; ++s) {
             barrier_init(&sm.mma_done[s], 1);
             // my decode warps, without barriers for X tiles my copy thread (with their bytes), in the first CTA the second CTA
-            barrier_init(&sm.ready[s], kBlockWarps + (kByTile<kXTiles> ? 0 : 1) + (c == 0 ? 1 : 0));
+            barrier_init(&sm.ready[s], kColumnWarps + (kByTile<kXTiles, kTmemW> ? 0 : 1) + (c == 0 ? 1 : 0));
         }
 #pragma unroll
         for (int s = 0; s < kXTiles; ++s) {
@@ -1159,7 +1221,7 @@ spmm_kernel(const __grid_constant__ Params p, const __grid_constant__ CUtensorMa
 #pragma unroll
         for (int s = 0; s < kMeta; ++s) {
             barrier_init(&sm.comp_full[s], 1);
-            barrier_init(&sm.comp_free[s], kBlockWarps);
+            barrier_init(&sm.comp_free[s], kColumnWarps);
         }
         barrier_init(&sm.drained, 1);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -1195,16 +1257,18 @@ spmm_kernel(const __grid_constant__ Params p, const __grid_constant__ CUtensorMa
             for (int kb = 0; kb < nkb; ++kb) {
                 const int s = kb % kStages;
                 if (ok) ok = wait_parity(&sm.ready[s], (kb / kStages) & 1);          // both CTAs' decoded W is in place
-                const uint64_t ad0 = operand_desc(smem_u32(&sm.A[s][0]), kAKGroupStride, kAChunkStride, 0u);
+                const uint64_t ad0 = kTmemW ? 0u : operand_desc(smem_u32(&sm.A[kTmemW ? 0 : s][0]), kAKGroupStride, kAChunkStride, 0u);
                 for (int i = 0; i < ntiles; ++i, x.next<kXTiles>()) {
-                    if (kByTile<kXTiles> && ok) ok = wait_parity(&sm.x_full[x.at], x.parity);        // and both halves of the X tile
+                    if (kByTile<kXTiles, kTmemW> && ok) ok = wait_parity(&sm.x_full[x.at], x.parity);        // and both halves of the X tile
                     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
                     const uint64_t bd0 = operand_desc(smem_u32(&sm.B[x.at][0]), 16, kBAtomBytes, 2u);
-                    const uint32_t id = instr_desc(256, i == ntiles - 1 ? last_tokens : kNI);
+                    const int tokens = i == ntiles - 1 ? last_tokens : acc;
+                    const uint32_t id = kTmemW ? instr_desc_tmem(256, tokens) : instr_desc(256, tokens);
 #pragma unroll
                     for (int kk = 0; ok && kk < kKB / 16; ++kk)    // the start address is the descriptor's low field, in 16-byte units
-                        mma_f16_pair(tmem + i * kNI, ad0 + ((kk * 2 * kAKGroupStride) >> 4), bd0 + ((kk * 32) >> 4), id, kb > 0 || kk > 0);
-                    if (kByTile<kXTiles>) commit_pair(&sm.x_done[x.at]);
+                        if constexpr (kTmemW) mma_f16_pair_tmem(tmem + i * kNextAcc, tmem + (kTmemCols - kWCols) + s * (kWCols / kStages) + kk * 8, bd0 + ((kk * 32) >> 4), id, kb > 0 || kk > 0);
+                        else mma_f16_pair(tmem + i * kNextAcc, ad0 + ((kk * 2 * kAKGroupStride) >> 4), bd0 + ((kk * 32) >> 4), id, kb > 0 || kk > 0);
+                    if (kByTile<kXTiles, kTmemW>) commit_pair(&sm.x_done[x.at]);
                 }
                 commit_pair(&sm.mma_done[s]);
             }
@@ -1217,7 +1281,7 @@ spmm_kernel(const __grid_constant__ Params p, const __grid_constant__ CUtensorMa
                 const int s = kb % kStages;
                 if (ok) ok = wait_parity(&sm.ready[s], (kb / kStages) & 1);
                 arrive_at(&sm.ready[s], 0u);
-                for (int i = 0; kByTile<kXTiles> && i < ntiles; ++i, x.next<kXTiles>()) {
+                for (int i = 0; kByTile<kXTiles, kTmemW> && i < ntiles; ++i, x.next<kXTiles>()) {
                     if (ok) ok = wait_parity(&sm.x_full[x.at], x.parity);
                     arrive_at(&sm.x_full[x.at], 0u);
                 }
@@ -1227,7 +1291,7 @@ spmm_kernel(const __grid_constant__ Params p, const __grid_constant__ CUtensorMa
     } else if (warp == kWarps + 1) {
         // ================= copy warp: moves the stored K-blocks =================
         CopyState cs;
-        ok = copy_blocks<kMeta>(p, cs, smem_u32(&sm.ring[0]), kRingBytes<kXTiles>, sm.meta, sm.comp_full, sm.comp_free, &sm.abort,
+        ok = copy_blocks<kMeta>(p, cs, smem_u32(&sm.ring[0]), kRingBytes<kXTiles, kTmemW>, sm.meta, sm.comp_full, sm.comp_free, &sm.abort,
                                 static_cast<int64_t>(r) * p.C, kb0, nkb, lane, ok);
         ok = await_copies<kMeta>(cs, sm.comp_full) && ok;
         __syncwarp();
@@ -1240,25 +1304,25 @@ spmm_kernel(const __grid_constant__ Params p, const __grid_constant__ CUtensorMa
             for (int kb = 0; kb < nkb; ++kb)
                 for (int i = 0; i < ntiles; ++i, x.next<kXTiles>()) {       // my 128 tokens of each tile: one tiled bulk-tensor copy
                     // it goes where the tile kXTiles before was multiplied from, once that work is complete
-                    unsigned long long* const full = kByTile<kXTiles> ? &sm.x_full[x.at] : &sm.ready[kb % kStages];
-                    if (kByTile<kXTiles>) {
+                    unsigned long long* const full = kByTile<kXTiles, kTmemW> ? &sm.x_full[x.at] : &sm.ready[kb % kStages];
+                    if (kByTile<kXTiles, kTmemW>) {
                         if (kb * ntiles + i >= kXTiles && ok) ok = wait_parity(&sm.x_done[x.at], x.parity ^ 1u);
-                        if (ok) expect_bytes(full, kBTileBytes);
+                        if (ok) expect_bytes(full, static_cast<uint32_t>(p.xbox) * kBRowBytes);
                     } else if (i == 0) {
                         if (kb >= kStages && ok) ok = wait_parity(&sm.mma_done[kb % kStages], ((kb / kStages) & 1u) ^ 1u);
-                        if (ok) expect_bytes(full, static_cast<uint32_t>(ntiles) * kBTileBytes);
+                        if (ok) expect_bytes(full, static_cast<uint32_t>(ntiles * p.xbox) * kBRowBytes);
                     }
                     if (!ok) {                                          // nothing is copied to a place that may be in use
                         *static_cast<volatile int*>(&sm.abort) = 1;
-                        if (kByTile<kXTiles> || i == 0) arrive(full);
+                        if (kByTile<kXTiles, kTmemW> || i == 0) arrive(full);
                         continue;
                     }
                     ++copied;
-                    tensor_copy(&sm.B[x.at][0], &xmap, (kb0 + kb) * kKB, static_cast<int>(n0) + i * kNI + c * ((i == ntiles - 1 ? last_tokens : kNI) / 2),
+                    tensor_copy(&sm.B[x.at][0], &xmap, (kb0 + kb) * kKB, static_cast<int>(n0) + i * acc + c * ((i == ntiles - 1 ? last_tokens : acc) / 2),
                                 full);
                 }
             // the last ones have arrived, whatever ran out
-            if (kByTile<kXTiles>) {
+            if (kByTile<kXTiles, kTmemW>) {
                 for (int q = max(0, copied - kXTiles); q < copied; ++q) ok = wait_parity(&sm.x_full[q % kXTiles], (q / kXTiles) & 1) && ok;
             } else {
                 for (int kb = max(0, copied / ntiles - kStages); kb < copied / ntiles; ++kb) ok = wait_parity(&sm.ready[kb % kStages], (kb / kStages) & 1) && ok;
@@ -1273,7 +1337,7 @@ spmm_kernel(const __grid_constant__ Params p, const __grid_constant__ CUtensorMa
             XTile x;
             for (int kb = 0; kb < nkb; ++kb) {
                 const int s = kb % kStages;
-                for (int i = 0; kByTile<kXTiles> && i < ntiles; ++i, x.next<kXTiles>()) {
+                for (int i = 0; kByTile<kXTiles, kTmemW> && i < ntiles; ++i, x.next<kXTiles>()) {
                     if (ok) ok = wait_parity(&sm.x_done[x.at], x.parity);
                     arrive_at(&sm.x_done[x.at], 1u);
                 }
@@ -1284,12 +1348,15 @@ spmm_kernel(const __grid_constant__ Params p, const __grid_constant__ CUtensorMa
         __syncwarp();
     } else {
         // ================= decode warps: my 128 rows of 4 columns of every sub-block of the group =================
-        const unsigned group = static_cast<unsigned>(warp) / kGroupWarps, wm = static_cast<unsigned>(warp) % kGroupWarps;
-        const unsigned top = pinned(nibble_top(lane & 7)), below = pinned(nibble_below(lane & 7));
-        const uint32_t tab_l = pinned(smem_u32(&sm.tab[warp][0]) + 32u * c + 8u * (lane >> 3));
-        const uint32_t a_lane = pinned(smem_u32(&sm.A[0][0]) + (lane >> 1) * kAChunkStride + (lane & 1) * 8);
+        // W in shared memory: a warp has 4 columns of a sub-block, all 128 rows; in tensor memory 32 rows, those lanes that it may write, of all 32.
+        constexpr unsigned kInGroup = kTmemW ? 4 : kGroupWarps, kGroups = kWarps / kInGroup;
+        const unsigned group = static_cast<unsigned>(warp) / kInGroup, wm = static_cast<unsigned>(warp) % kInGroup;
+        const unsigned top = pinned(kTmemW ? 1u << (31 - lane) : nibble_top(lane & 7)), below = pinned(nibble_below(lane & 7)), two = pinned(2u);
+        const uint32_t tab_l = pinned(smem_u32(&sm.tab[warp][0]) + (kTmemW ? 0u : 32u * c + 8u * (lane >> 3))), tab_me = pinned(smem_u32(&sm.tab[warp][lane]));
+        const uint32_t a_lane = pinned(kTmemW ? tmem + (32u * wm << 16) + (kTmemCols - kWCols) : smem_u32(&sm.A[0][0]) + (lane >> 1) * kAChunkStride + (lane & 1) * 8);
+        const Eighth eighth(c, static_cast<int>(wm & 3u));
         for (unsigned i = group; i < static_cast<unsigned>(nkb) * kSubs; i += kGroups) {
-            const unsigned kb = i / kSubs, s = kb % kStages, j0 = (i % kSubs) * kSub + 4u * wm;      // my first column of the K-block
+            const unsigned kb = i / kSubs, s = kb % kStages, j0 = (i % kSubs) * kSub + (kTmemW ? 0u : 4u * wm);      // my first column of the K-block
             const unsigned m = kb % kMeta;
             // The first K-block finds room in the ring in any case and kStages of them are decoded before any product; one that
             // is still outside then waits for room, and so, like everything behind the first products, for X.
@@ -1297,12 +1364,26 @@ spmm_kernel(const __grid_constant__ Params p, const __grid_constant__ CUtensorMa
             if (ok) ok = wait_parity(&sm.comp_full[m], (kb / kMeta) & 1);                   // the stored block has arrived
             const Meta& mt = sm.meta[m];
             __syncwarp();
-            scan4(p, mt.bm, mt.ci, mt.start, mt.ngt, mt.limit, static_cast<int>(j0), lane, &sm.tab[warp][0]);
+            if constexpr (kTmemW) scan_eighth(p, mt, static_cast<int>(j0) + lane, eighth, tab_me);
+            else scan4(p, mt.bm, mt.ci, mt.start, mt.ngt, mt.limit, static_cast<int>(j0), lane, &sm.tab[warp][0]);
             __syncwarp();
             if (kb >= kStages && ok) ok = wait_parity(&sm.mma_done[s], ((kb / kStages) & 1u) ^ 1u);  // the tensor cores are done with this A stage
-            expand4<4, 1>(tab_l, a_lane + s * kATileBytes + (j0 >> 3) * kAKGroupStride + (j0 & 7u) * 16u, 0u, below, top);
-            // the operand tile was written through the generic proxy; the tensor cores read through the async proxy
-            asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+            if constexpr (kTmemW) {
+                __syncwarp();
+                asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+#pragma unroll 1
+                for (int c0 = 0; c0 < kSub; c0 += 16) {
+                    uint32_t v[8];
+                    expand_row(tab_l + 8u * c0, top, two, v);
+                    tmem_store8(a_lane + s * (kWCols / kStages) + (j0 + c0) / 2, v);
+                }
+                asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
+                asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+            } else {
+                expand4<4, 1>(tab_l, a_lane + s * kATileBytes + (j0 >> 3) * kAKGroupStride + (j0 & 7u) * 16u, 0u, below, top);
+                // the operand tile was written through the generic proxy; the tensor cores read through the async proxy
+                asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+            }
             __syncwarp();
             if (lane == 0) {
                 arrive(&sm.comp_free[m]);
@@ -1321,11 +1402,12 @@ spmm_kernel(const __grid_constant__ Params p, const __grid_constant__ CUtensorMa
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     __syncthreads();
 
-    // ---- epilogue.  Warp w reads lanes 32*(w%4).. (my rows 32*(w%4)..), token columns [(w/4)*128, +128) of the 512 ----
+    // ---- epilogue.  Warp w reads lanes 32*(w%4).. (my rows 32*(w%4)..), a quarter of the tile's token columns ----
     if (!*static_cast<volatile int*>(&sm.abort) && warp < kStoreWarps) {
-        const int lane_base = 32 * (warp & 3), cbase = (warp >> 2) * (kNT / 4);
-        store_accumulators<true>(p, tmem, lane_base, cbase, cbase + kNT / 4, r, c * 128 + lane_base, n0,
-                           p.partial == nullptr ? -1 : static_cast<int>(pr));
+        const int lane_base = 32 * (warp & 3), i = ntiles == 2 ? warp >> 3 : 0;               // my accumulator
+        const int part = ntiles == 2 ? acc / 2 : (acc / 4 + 15) / 16 * 16, cbase = (ntiles == 2 ? (warp >> 2) & 1 : warp >> 2) * part;
+        store_accumulators<true>(p, tmem + i * kNextAcc, lane_base, cbase, min(cbase + part, acc), r, c * 128 + lane_base, n0 + i * acc,
+                           p.partial == nullptr ? -1 : static_cast<int>(pr), i * acc);
     } else if (*static_cast<volatile int*>(&sm.abort) && p.partial != nullptr) {
         void_rows(p, static_cast<int>(pr), c * 128, 128, t, kThreads);
     }
@@ -1345,7 +1427,7 @@ reduce_slices_kernel(const Params p, int chunks) {
     const int tok = static_cast<int>(blockIdx.x - t * static_cast<unsigned>(chunks)) * kReduceTokens + static_cast<int>(threadIdx.x >> 6);
     const unsigned tile = static_cast<unsigned>(p.tile0) + t, r = tile / static_cast<unsigned>(p.nblocks), nb = tile - r * static_cast<unsigned>(p.nblocks);
     const int row_in = 4 * static_cast<int>(threadIdx.x & 63u);
-    const int64_t n = static_cast<int64_t>(nb) * kNT + tok, row = static_cast<int64_t>(r) * kTileM + row_in;
+    const int64_t n = static_cast<int64_t>(nb) * p.tile_tokens + tok, row = static_cast<int64_t>(r) * kTileM + row_in;
     const size_t slot = static_cast<size_t>(p.ptok) * kTileM;
     const float* sums = p.partial + static_cast<size_t>(t) * p.kslices * slot + static_cast<size_t>(tok) * kTileM + row_in;
     asm volatile("griddepcontrol.wait;" ::: "memory");
@@ -1405,8 +1487,10 @@ spdp_status configure_spmm_kernel() {
         SPDP_CUDA_TRY(cudaFuncSetAttribute(one::spmm_kernel<One32>, cudaFuncAttributeMaxDynamicSharedMemorySize, one::kSmemBytes));
         SPDP_CUDA_TRY(cudaFuncSetAttribute(one::spmm_kernel<One128>, cudaFuncAttributeMaxDynamicSharedMemorySize, one::kSmemBytes));
         SPDP_CUDA_TRY(cudaFuncSetAttribute(one::spmm_kernel<One256>, cudaFuncAttributeMaxDynamicSharedMemorySize, one::kSmemBytes));
-        SPDP_CUDA_TRY(cudaFuncSetAttribute(pair::spmm_kernel<4>, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(pair::kSmemBytes)));
-        SPDP_CUDA_TRY(cudaFuncSetAttribute(pair::spmm_kernel<6>, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(pair::kSmemBytes)));
+        SPDP_CUDA_TRY(cudaFuncSetAttribute(pair::spmm_kernel<4, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(pair::kSmemBytes)));
+        SPDP_CUDA_TRY(cudaFuncSetAttribute(pair::spmm_kernel<6, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(pair::kSmemBytes)));
+        SPDP_CUDA_TRY(cudaFuncSetAttribute(pair::spmm_kernel<4, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(pair::kSmemBytes)));
+        SPDP_CUDA_TRY(cudaFuncSetAttribute(pair::spmm_kernel<6, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(pair::kSmemBytes)));
         const spdp_status st = resident_clusters(dev);
         if (st != SPDP_OK) return st;
         configured[dev] = true;
@@ -1475,7 +1559,7 @@ spdp_status launch_one(const Params& p, const CUtensorMap& xmap, cudaStream_t s)
 // Programmatic launch for the pairs too: a call's set-up, first copies and first three decoded K-blocks overlap the kernel before.
 // us per call, calls in a row: 4001x4098 x 300 tokens 32.8 -> 28.7, 4096x4096 x 300 28.7 -> 25.3, x 1024 48.1 -> 44.6, 11008x4096 x 300
 // 60.3 -> 56.6.
-spdp_status launch_pairs(const Params& p, const CUtensorMap& xmap, int64_t pairs, int x_tiles, cudaStream_t s) {
+spdp_status launch_pairs(const Params& p, const CUtensorMap& xmap, int64_t pairs, int x_tiles, bool tmem_w, cudaStream_t s) {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(static_cast<unsigned>(2 * pairs));
     cfg.blockDim = dim3(pair::kThreads);
@@ -1490,7 +1574,8 @@ spdp_status launch_pairs(const Params& p, const CUtensorMap& xmap, int64_t pairs
     attr[1].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 2;
-    SPDP_CUDA_TRY(cudaLaunchKernelEx(&cfg, x_tiles == 6 ? pair::spmm_kernel<6> : pair::spmm_kernel<4>, p, xmap));
+    const auto kernel = tmem_w ? (x_tiles == 6 ? pair::spmm_kernel<6, true> : pair::spmm_kernel<4, true>) : x_tiles == 6 ? pair::spmm_kernel<6, false> : pair::spmm_kernel<4, false>;
+    SPDP_CUDA_TRY(cudaLaunchKernelEx(&cfg, kernel, p, xmap));
     return SPDP_OK;
 }
 
@@ -1512,32 +1597,35 @@ spdp_status launch_reduce(Kernel kernel, int64_t tiles, int chunks, cudaStream_t
 
 spdp_status run_plan(const spdp_matrix* h, Params p, const Plan& plan, const __half* X, int64_t ldx, cudaStream_t s) {
     if (plan.tiles * p.nkb >= (int64_t(1) << 31)) return SPDP_ERR_UNSUPPORTED_SHAPE;
-    const int nt = kTokens[plan.kernel];
+    const bool pairs = plan.kernel >= 3;
+    p.acc_tokens = plan.kernel == 4 ? plan::pair_acc_tokens(p.N) : pair::kNI;
+    p.tile_tokens = plan.kernel == 4 ? plan::pair_tile_tokens(p.N) : kTokens[plan.kernel];
+    const int nt = p.tile_tokens;
     p.nblocks = static_cast<int>((p.N + nt - 1) / nt);
     p.ptok = static_cast<int>(std::min<int64_t>(p.N, nt));
     p.kslices = 1;
     p.cluster = plan.cluster;
     CUtensorMap xmap;
-    p.xbox = plan.kernel == 3 ? pair::kNI / 2 : (p.ptok + 15) / 16 * 16;
+    p.xbox = pairs ? p.acc_tokens / 2 : (p.ptok + 15) / 16 * 16;
     spdp_status st = encode_x(&xmap, X, p.N, h->K, ldx, p.xbox);
     if (st != SPDP_OK) return st;
     const bool cut = plan.rest > 0 && plan.sharers > plan.rest;              // partial sums and a second kernel
     if (cut) {
-        const size_t slots = static_cast<size_t>(plan.kernel == 3 ? plan.sharers : 2 * plan.sharers);
+        const size_t slots = static_cast<size_t>(pairs ? plan.sharers : 2 * plan.sharers);
         st = scratch_alloc(h->device, slots * p.ptok * kTileM * sizeof(float), s, reinterpret_cast<void**>(&p.partial));
         if (st != SPDP_OK) return st;
     }
     const int chunks = (p.ptok + kReduceTokens - 1) / kReduceTokens;
     const bool many = plan.sharers >= kManySumsFrom * plan.rest;             // sums a tile
-    if (plan.kernel == 3) {
+    if (pairs) {
         const int x_tiles = pair_x_tiles(h->values_len, h->R, p.nkb);
         Params whole = p;                                                    // whole tiles first, then the last tiles cut along K
         whole.partial = nullptr;
-        if (plan.tiles > plan.rest) st = launch_pairs(whole, xmap, plan.tiles - plan.rest, x_tiles, s);
+        if (plan.tiles > plan.rest) st = launch_pairs(whole, xmap, plan.tiles - plan.rest, x_tiles, plan.kernel == 4, s);
         if (st == SPDP_OK && cut) {
             p.tile0 = static_cast<int>(plan.tiles - plan.rest);
             p.kslices = plan.slices;
-            st = launch_pairs(p, xmap, plan.rest * plan.slices, x_tiles, s);
+            st = launch_pairs(p, xmap, plan.rest * plan.slices, x_tiles, plan.kernel == 4, s);
             if (st == SPDP_OK) st = launch_reduce(many ? pair::reduce_slices_kernel<kManySums> : pair::reduce_slices_kernel<kFewSums>, plan.rest, chunks, s, p, chunks);
         }
     } else {
