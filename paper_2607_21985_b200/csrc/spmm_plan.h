@@ -41,6 +41,7 @@ struct Plan {
     int cluster;            // CTAs to a tile that add its sums themselves, 1: a second kernel does
 };
 constexpr int kMostSlices = 9;          // of a tile of pairs, where all slices do not fit the device at once
+constexpr int64_t kScratchTokens = 2 * 148 * 256;     // and then no more sums (of 256 rows each) in scratch memory than kernel 2 leaves on 148 SMs
 constexpr int kMaxCluster = 16;                                         // CTAs
 constexpr int kGatherTokens = 126;      // tokens' sums (of 256 rows) that a CTA of a cluster has room for
 
@@ -135,7 +136,7 @@ inline Plan make_plan(int64_t R, int64_t nkb, int64_t N, int sms, bool may_cut, 
             consider(2 * most / 3 * left);
         }
         if (f == 4)                                                              // three pairs to two tiles, say, as five slices each in three rounds
-            for (int slices = most + 1; slices <= kMostSlices; ++slices) consider(slices * left);
+            for (int slices = most + 1; slices <= kMostSlices && slices * left * tokens <= kScratchTokens; ++slices) consider(slices * left);
         if (resident == nullptr || rounds > 0 || f > 1) continue;                // clusters: the one-CTA forms with W in tensor memory
         const int c0 = blocks_at_best(kClusterEach + kClusterPerMB * mb * static_cast<double>(left));
         int largest = kMaxCluster;

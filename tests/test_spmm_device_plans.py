@@ -64,6 +64,7 @@ def test_plans_hold_together(plan, resident):
                     seen.add((q["kernel"], q["cluster"] > 1))
                     assert q["tiles"] == R * -(-N // tokens)
                     assert not cut or q["sharers"] <= q["rest"] * nkb
+                    assert not cut or (1 if pairs else 2) * q["sharers"] * min(N, tokens) <= 2 * 148 * 256       # 77 MB of scratch memory
                     assert q["kernel"] == 4 or q["sharers"] <= max(slots, q["rest"])
                     if pairs:
                         assert q["cluster"] == 1 and q["slices"] >= 1 and (not cut or q["sharers"] == q["slices"] * q["rest"]) and q["slices"] <= max(nkb, 1)
