@@ -95,6 +95,13 @@ constexpr int kBAtomBytes = 8 * kBRowBytes;
 #define SPDP_SPMM_WAIT_TRIES (1 << 22)
 #endif
 constexpr int kWaitTries = SPDP_SPMM_WAIT_TRIES;
+constexpr int kDrainTries = 1 << 18;   // of a wait for what the CTA itself has under way, after which it leaves: these land in microseconds
+#ifdef SPDP_CHECKED
+__device__ int g_wait_tries = kWaitTries;      // checked build: a test makes waits run out (spdp_checked_wait_tries)
+__device__ __forceinline__ int wait_tries() { return *static_cast<volatile int*>(&g_wait_tries); }
+#else
+__device__ __forceinline__ constexpr int wait_tries() { return kWaitTries; }
+#endif
 static_assert(kBRowBytes == 128, "one X row of a K-block is one 128-byte swizzle row");
 
 // 64 registers a thread, which leaves room for a block of the second kernel beside a CTA (with 72, as for kThreads alone, 0.5 % more time
@@ -201,10 +208,10 @@ __device__ __forceinline__ bool phase_done(unsigned long long* bar, unsigned par
                  : "=r"(done) : "r"(smem_u32(bar)), "r"(parity) : "memory");
     return done != 0u;
 }
-__device__ __forceinline__ bool wait_parity(unsigned long long* bar, unsigned parity) {
+__device__ __forceinline__ bool wait_parity(unsigned long long* bar, unsigned parity, int limit = wait_tries()) {
     const uint32_t a = smem_u32(bar);
     if (phase_done(bar, parity)) return true;       // usually: a test costs less than a wait that may suspend
-    for (int tries = 0; tries < kWaitTries; ++tries) {
+    for (int tries = 0; tries < limit; ++tries) {
         unsigned done;
         asm volatile("{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n selp.u32 %0, 1, 0, p;\n}"
                      : "=r"(done) : "r"(a), "r"(parity) : "memory");
@@ -643,12 +650,14 @@ struct CopyState {
 // Starts the copies of K-blocks kb0 .. kb0 + n - 1 of the row tile whose first GTile is g_row.  The values of the blocks in
 // flight lie in a ring of bytes, so that the sparser the matrix, the more blocks are on their way; bitmaps and ColInfo in
 // kMeta slots.  A lane holds the TileOffset words of one K-block in 32, looks them over and says where its values start; what is left per
-// block is short, because this one warp shares its scheduler with six that decode, and each of its instructions waits for its turn.  After a
-// failure nothing is copied any more, but every block's barrier still completes, and no sooner than its place is free: a barrier that ran two
-// phases ahead of who waits for it would look like one that has not completed.
+// block is short, because this one warp shares its scheduler with six that decode, and each of its instructions waits for its turn.  From a block
+// that is refused on nothing is copied any more, but every block's barrier still completes, and no sooner than its place is free: a barrier that ran two
+// phases ahead of who waits for it would look like one that has not completed.  A wait that runs out ends the work: a place that was
+// not given back is not written to, for a decode warp may still read there.
 template <int kMeta>
 __device__ __forceinline__ bool copy_blocks(const Params& p, CopyState& c, uint32_t ring, uint32_t ring_bytes, Meta* meta, unsigned long long* full,
-                                            unsigned long long* freed, int* abort, int64_t g_row, int kb0, int n, int lane, bool ok) {
+                                            unsigned long long* freed, int* abort, int64_t g_row, int kb0, int n, int lane) {
+    bool ok = true;
     uint32_t to[kGTB + 1], nxt[kGTB + 1];
     auto fetch = [&](int b, uint32_t (&o)[kGTB + 1]) {      // words of K-block kb0 + b + lane: its GTiles and the one after
         const int g0 = (kb0 + b + lane) * kGTB;
@@ -671,7 +680,7 @@ __device__ __forceinline__ bool copy_blocks(const Params& p, CopyState& c, uint3
         }
         const int lim = min(32, n - b);
         for (int q = 0; q < lim; ++q, ++c.i) {
-            const uint32_t from = __shfl_sync(0xFFFFFFFFu, to[0], q), bytes = __shfl_sync(0xFFFFFFFFu, ok && !c.refused ? 2u * nvals : 0u, q);
+            const uint32_t from = __shfl_sync(0xFFFFFFFFu, to[0], q), bytes = __shfl_sync(0xFFFFFFFFu, c.refused ? 0u : 2u * nvals, q);
             if (c.pos + bytes > ring_bytes) {               // the values of a K-block stay in one piece
                 c.vhead += ring_bytes - c.pos;
                 c.pos = 0;
@@ -684,7 +693,7 @@ __device__ __forceinline__ bool copy_blocks(const Params& p, CopyState& c, uint3
                 ++c.done;
                 c.vtail = c.done < c.i ? meta[c.done % kMeta].vstart : c.vhead;
             }
-            ok = __all_sync(0xFFFFFFFFu, ok);
+            if (!__all_sync(0xFFFFFFFFu, ok)) return false;
             const unsigned m = c.i % kMeta;
             Meta& mt = meta[m];
             const int ngt = min(kGTB, p.C - (kb0 + b + q) * kGTB);
@@ -692,17 +701,16 @@ __device__ __forceinline__ bool copy_blocks(const Params& p, CopyState& c, uint3
                 const uint32_t at = ring + c.pos - 2u * to[0];
                 static_assert(kGTB == 4, "one store");
                 *reinterpret_cast<uint4*>(&mt.start[0]) = make_uint4(at + 2u * to[0], at + 2u * to[1], at + 2u * to[2], at + 2u * to[3]);
-                *reinterpret_cast<uint4*>(&mt.vstart) = make_uint4(c.vhead, nvals, ok && !c.refused ? static_cast<unsigned>(ngt) : 0u, 0u);
+                *reinterpret_cast<uint4*>(&mt.vstart) = make_uint4(c.vhead, nvals, c.refused ? 0u : static_cast<unsigned>(ngt), 0u);
             }
             __syncwarp();
             if (elect_one()) {
-                if (ok && !c.refused) {
+                if (!c.refused) {
                     expect_bytes(&full[m], bytes + static_cast<uint32_t>(ngt) * (kTileK * 32u + kTileK * 4u));
                     if (bytes) bulk_copy(ring + c.pos, p.values + from, bytes, &full[m]);
                     bulk_copy(smem_u32(&mt.bm[0][0]), bm, static_cast<uint32_t>(ngt) * kTileK * 32u, &full[m]);
                     bulk_copy(smem_u32(&mt.ci[0]), ci, static_cast<uint32_t>(ngt) * kTileK * 4u, &full[m]);
                 } else {
-                    *static_cast<volatile int*>(abort) = 1;
                     arrive(&full[m]);
                 }
             }
@@ -715,13 +723,13 @@ __device__ __forceinline__ bool copy_blocks(const Params& p, CopyState& c, uint3
 #pragma unroll
         for (int q = 0; q <= kGTB; ++q) to[q] = nxt[q];
     }
-    return ok;
+    return true;
 }
 // Before the CTA may leave, every copy that was started has arrived.
 template <int kMeta>
 __device__ __forceinline__ bool await_copies(const CopyState& c, unsigned long long* full) {
     bool ok = true;
-    for (unsigned q = (c.i > kMeta ? c.i - kMeta : 0u); q < c.i; ++q) ok = wait_parity(&full[q % kMeta], (q / kMeta) & 1) && ok;
+    for (unsigned q = (c.i > kMeta ? c.i - kMeta : 0u); q < c.i; ++q) ok = wait_parity(&full[q % kMeta], (q / kMeta) & 1, kDrainTries) && ok;
     return ok;
 }
 
@@ -912,16 +920,16 @@ spmm_kernel(const __grid_constant__ Params p, const __grid_constant__ CUtensorMa
             }
             if (issued) {                                               // tensor memory is not freed under running products
                 commit_one(&sm.drained);
-                ok = wait_parity(&sm.drained, 0u) && ok;
+                ok = wait_parity(&sm.drained, 0u, kDrainTries) && ok;
             }
         }
         __syncwarp();           // the other lanes wait here, not on a barrier in shared memory
     } else if (warp == kWarps + 1) {
         // ================= copy warp: moves the stored K-blocks =================
         CopyState cs;
-        for (int k = 0; piece(p, me, k, s); ++k)
+        for (int k = 0; ok && piece(p, me, k, s); ++k)
             ok = copy_blocks<F::kMeta>(p, cs, smem_u32(&sm.ring[0]), kRingBytes<F>, sm.meta, sm.comp_full, sm.comp_free, &sm.abort,
-                                       static_cast<int64_t>(s.tile / p.nblocks) * p.C, s.kb0, s.n, lane, ok);
+                                       static_cast<int64_t>(s.tile / p.nblocks) * p.C, s.kb0, s.n, lane);
         ok = await_copies<F::kMeta>(cs, sm.comp_full) && ok;
         __syncwarp();
     } else if (warp == kWarps + 2) {
@@ -929,21 +937,17 @@ spmm_kernel(const __grid_constant__ Params p, const __grid_constant__ CUtensorMa
         if (elect_one()) {
             asm volatile("griddepcontrol.wait;" ::: "memory");          // X may come from the kernel before this one
             unsigned u = 0;
-            for (int k = 0; piece(p, me, k, s); ++k) {
+            for (int k = 0; ok && piece(p, me, k, s); ++k) {
                 const int n0 = (s.tile % p.nblocks) * F::kNI;
                 for (int kb = 0; kb < s.n; ++kb, ++u) {
                     const unsigned sb = u % F::kBStages;
-                    if (u >= F::kBStages && ok) ok = wait_parity(&sm.x_free[sb], (u / F::kBStages - 1u) & 1);
-                    if (!ok) {
-                        *static_cast<volatile int*>(&sm.abort) = 1;     // before anything is multiplied with what is not there
-                        arrive(&sm.x_full[sb]);
-                        continue;
-                    }
+                    if (u >= F::kBStages) ok = wait_parity(&sm.x_free[sb], (u / F::kBStages - 1u) & 1);
+                    if (!ok) break;
                     expect_bytes(&sm.x_full[sb], static_cast<uint32_t>(p.xbox) * kBRowBytes);
                     tensor_copy(&sm.B[sb][0], &xmap, (s.kb0 + kb) * kKB, n0, &sm.x_full[sb]);
                 }
             }
-            for (unsigned q = (u > F::kBStages ? u - F::kBStages : 0u); q < u; ++q) ok = wait_parity(&sm.x_full[q % F::kBStages], (q / F::kBStages) & 1) && ok;
+            for (unsigned q = (u > F::kBStages ? u - F::kBStages : 0u); q < u; ++q) ok = wait_parity(&sm.x_full[q % F::kBStages], (q / F::kBStages) & 1, kDrainTries) && ok;
         }
         __syncwarp();
     } else {
@@ -966,15 +970,15 @@ spmm_kernel(const __grid_constant__ Params p, const __grid_constant__ CUtensorMa
             for (unsigned upto = min(i1, 2u * kSubs);; upto = upto < F::kAStages ? min(i1, static_cast<unsigned>(F::kAStages)) : i1) {
                 for (; i < upto; i += kGroups) {
                     const unsigned u = i / kSubs, m = u % F::kMeta, sa = i % F::kAStages;
-                    ok = wait_parity(&sm.comp_full[m], (u / F::kMeta) & 1);                          // the stored K-block has arrived
-                    __syncwarp();
+                    ok = __all_sync(0xFFFFFFFFu, wait_parity(&sm.comp_full[m], (u / F::kMeta) & 1));    // the stored K-block has arrived
+                    if (!ok) break;
                     const Meta& mt = sm.meta[m];
                     if constexpr (F::kTmemW) scan_quarter(p, mt, static_cast<int>((i % kSubs) * kSub) + lane, quarter, tab_me);
                     else scan4(p, mt.bm, mt.ci, mt.start, mt.ngt, mt.limit, static_cast<int>((i % kSubs) * kSub + 4u * wm), lane, &sm.tab[warp][0]);
                     __syncwarp();
                     if (i >= F::kAStages) {
                         if (i < 2 * F::kAStages) asm volatile("griddepcontrol.wait;" ::: "memory");  // the products wait for X
-                        ok = wait_parity(&sm.a_free[sa], (i / F::kAStages - 1u) & 1) && ok;          // the tensor cores are done with this A stage
+                        ok = wait_parity(&sm.a_free[sa], (i / F::kAStages - 1u) & 1);                // the tensor cores are done with this A stage
                     }
                     ok = __all_sync(0xFFFFFFFFu, ok);
                     if (!ok) break;
@@ -1073,6 +1077,7 @@ spmm_kernel(const __grid_constant__ Params p, const __grid_constant__ CUtensorMa
                 __syncwarp();
             }
             ok = wait_parity(&sm.gathered, 0u);
+            if (!ok) wait_parity(&sm.gathered, 0u, kDrainTries);      // nobody leaves while they are under way
             const int64_t row0 = static_cast<int64_t>(s.tile / p.nblocks) * kTileM;
             const uint32_t own = smem_u32(&sm.B[0][0]) - static_cast<uint32_t>(rank) * part_bytes, before = smem_u32(&sm.ring[0]), behind = before - part_bytes;
             // 4 rows of a token at a time, by all threads
@@ -1243,8 +1248,9 @@ spmm_kernel(const __grid_constant__ Params p, const __grid_constant__ CUtensorMa
     const int nkb_all = p.nkb;
     const int kb0 = static_cast<int>(static_cast<int64_t>(nkb_all) * slice / p.kslices);
     const int nkb = static_cast<int>(static_cast<int64_t>(nkb_all) * (slice + 1) / p.kslices) - kb0;
-    // A wait that runs out (it never should) clears `ok`: the thread then stops waiting but keeps walking the
-    // same barriers as the others, the status word gets SPDP_ERR_TIMEOUT and the outputs stay unwritten.  As in the one-CTA forms,
+    // A wait that runs out (it never should) clears `ok`: the thread's role ends, as in the one-CTA forms, and the others' waits run out in turn,
+    // in both CTAs: what is not complete is never stored.  A role that walked on without waiting would hand on what others still read or
+    // have not written, and arrive on barriers more often than they count.  As in the one-CTA forms,
     // whatever depends on X first waits for the kernel before this one (griddepcontrol.wait), which no bounded wait covers.
     bool ok = true;
 
@@ -1254,36 +1260,37 @@ spmm_kernel(const __grid_constant__ Params p, const __grid_constant__ CUtensorMa
         if (one && c == 0) {
             // ================= tensor-core thread (first CTA): issues the K-blocks' products for the pair =================
             XTile x;
-            for (int kb = 0; kb < nkb; ++kb) {
+            for (int kb = 0; ok && kb < nkb; ++kb) {
                 const int s = kb % kStages;
-                if (ok) ok = wait_parity(&sm.ready[s], (kb / kStages) & 1);          // both CTAs' decoded W is in place
+                ok = wait_parity(&sm.ready[s], (kb / kStages) & 1);                  // both CTAs' decoded W is in place
                 const uint64_t ad0 = kTmemW ? 0u : operand_desc(smem_u32(&sm.A[kTmemW ? 0 : s][0]), kAKGroupStride, kAChunkStride, 0u);
-                for (int i = 0; i < ntiles; ++i, x.next<kXTiles>()) {
-                    if (kByTile<kXTiles, kTmemW> && ok) ok = wait_parity(&sm.x_full[x.at], x.parity);        // and both halves of the X tile
+                for (int i = 0; ok && i < ntiles; ++i, x.next<kXTiles>()) {
+                    if (kByTile<kXTiles, kTmemW>) ok = wait_parity(&sm.x_full[x.at], x.parity);              // and both halves of the X tile
+                    if (!ok) break;
                     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
                     const uint64_t bd0 = operand_desc(smem_u32(&sm.B[x.at][0]), 16, kBAtomBytes, 2u);
                     const int tokens = i == ntiles - 1 ? last_tokens : acc;
                     const uint32_t id = kTmemW ? instr_desc_tmem(256, tokens) : instr_desc(256, tokens);
 #pragma unroll
-                    for (int kk = 0; ok && kk < kKB / 16; ++kk)    // the start address is the descriptor's low field, in 16-byte units
+                    for (int kk = 0; kk < kKB / 16; ++kk)    // the start address is the descriptor's low field, in 16-byte units
                         if constexpr (kTmemW) mma_f16_pair_tmem(tmem + i * kNextAcc, tmem + (kTmemCols - kWCols) + s * (kWCols / kStages) + kk * 8, bd0 + ((kk * 32) >> 4), id, kb > 0 || kk > 0);
                         else mma_f16_pair(tmem + i * kNextAcc, ad0 + ((kk * 2 * kAKGroupStride) >> 4), bd0 + ((kk * 32) >> 4), id, kb > 0 || kk > 0);
                     if (kByTile<kXTiles, kTmemW>) commit_pair(&sm.x_done[x.at]);
                 }
-                commit_pair(&sm.mma_done[s]);
+                if (ok) commit_pair(&sm.mma_done[s]);
             }
             commit_pair(&sm.drained);                                   // neither CTA frees tensor memory under running products, whatever ran out
-            ok = wait_parity(&sm.drained, 0u) && ok;
+            ok = wait_parity(&sm.drained, 0u, kDrainTries) && ok;
         } else if (one) {
             // ================= second CTA: tell the first when my part of a block is ready =================
             XTile x;
-            for (int kb = 0; kb < nkb; ++kb) {
+            for (int kb = 0; ok && kb < nkb; ++kb) {
                 const int s = kb % kStages;
-                if (ok) ok = wait_parity(&sm.ready[s], (kb / kStages) & 1);
-                arrive_at(&sm.ready[s], 0u);
-                for (int i = 0; kByTile<kXTiles, kTmemW> && i < ntiles; ++i, x.next<kXTiles>()) {
-                    if (ok) ok = wait_parity(&sm.x_full[x.at], x.parity);
-                    arrive_at(&sm.x_full[x.at], 0u);
+                ok = wait_parity(&sm.ready[s], (kb / kStages) & 1);
+                if (ok) arrive_at(&sm.ready[s], 0u);
+                for (int i = 0; ok && kByTile<kXTiles, kTmemW> && i < ntiles; ++i, x.next<kXTiles>()) {
+                    ok = wait_parity(&sm.x_full[x.at], x.parity);
+                    if (ok) arrive_at(&sm.x_full[x.at], 0u);
                 }
             }
         }
@@ -1292,7 +1299,7 @@ spmm_kernel(const __grid_constant__ Params p, const __grid_constant__ CUtensorMa
         // ================= copy warp: moves the stored K-blocks =================
         CopyState cs;
         ok = copy_blocks<kMeta>(p, cs, smem_u32(&sm.ring[0]), kRingBytes<kXTiles, kTmemW>, sm.meta, sm.comp_full, sm.comp_free, &sm.abort,
-                                static_cast<int64_t>(r) * p.C, kb0, nkb, lane, ok);
+                                static_cast<int64_t>(r) * p.C, kb0, nkb, lane);
         ok = await_copies<kMeta>(cs, sm.comp_full) && ok;
         __syncwarp();
     } else if (warp == kWarps + 3) {
@@ -1301,31 +1308,27 @@ spmm_kernel(const __grid_constant__ Params p, const __grid_constant__ CUtensorMa
             asm volatile("griddepcontrol.wait;" ::: "memory");          // X may come from the kernel before this one
             XTile x;
             int copied = 0;
-            for (int kb = 0; kb < nkb; ++kb)
+            for (int kb = 0; ok && kb < nkb; ++kb)
                 for (int i = 0; i < ntiles; ++i, x.next<kXTiles>()) {       // my 128 tokens of each tile: one tiled bulk-tensor copy
                     // it goes where the tile kXTiles before was multiplied from, once that work is complete
                     unsigned long long* const full = kByTile<kXTiles, kTmemW> ? &sm.x_full[x.at] : &sm.ready[kb % kStages];
                     if (kByTile<kXTiles, kTmemW>) {
-                        if (kb * ntiles + i >= kXTiles && ok) ok = wait_parity(&sm.x_done[x.at], x.parity ^ 1u);
+                        if (kb * ntiles + i >= kXTiles) ok = wait_parity(&sm.x_done[x.at], x.parity ^ 1u);
                         if (ok) expect_bytes(full, static_cast<uint32_t>(p.xbox) * kBRowBytes);
                     } else if (i == 0) {
-                        if (kb >= kStages && ok) ok = wait_parity(&sm.mma_done[kb % kStages], ((kb / kStages) & 1u) ^ 1u);
+                        if (kb >= kStages) ok = wait_parity(&sm.mma_done[kb % kStages], ((kb / kStages) & 1u) ^ 1u);
                         if (ok) expect_bytes(full, static_cast<uint32_t>(ntiles * p.xbox) * kBRowBytes);
                     }
-                    if (!ok) {                                          // nothing is copied to a place that may be in use
-                        *static_cast<volatile int*>(&sm.abort) = 1;
-                        if (kByTile<kXTiles, kTmemW> || i == 0) arrive(full);
-                        continue;
-                    }
+                    if (!ok) break;                                     // nothing is copied to a place that may be in use
                     ++copied;
                     tensor_copy(&sm.B[x.at][0], &xmap, (kb0 + kb) * kKB, static_cast<int>(n0) + i * acc + c * ((i == ntiles - 1 ? last_tokens : acc) / 2),
                                 full);
                 }
             // the last ones have arrived, whatever ran out
             if (kByTile<kXTiles, kTmemW>) {
-                for (int q = max(0, copied - kXTiles); q < copied; ++q) ok = wait_parity(&sm.x_full[q % kXTiles], (q / kXTiles) & 1) && ok;
+                for (int q = max(0, copied - kXTiles); q < copied; ++q) ok = wait_parity(&sm.x_full[q % kXTiles], (q / kXTiles) & 1, kDrainTries) && ok;
             } else {
-                for (int kb = max(0, copied / ntiles - kStages); kb < copied / ntiles; ++kb) ok = wait_parity(&sm.ready[kb % kStages], (kb / kStages) & 1) && ok;
+                for (int kb = max(0, copied / ntiles - kStages); kb < copied / ntiles; ++kb) ok = wait_parity(&sm.ready[kb % kStages], (kb / kStages) & 1, kDrainTries) && ok;
             }
         }
         __syncwarp();
@@ -1335,14 +1338,14 @@ spmm_kernel(const __grid_constant__ Params p, const __grid_constant__ CUtensorMa
         if (lane == 0 && c == 0) {
             asm volatile("griddepcontrol.wait;" ::: "memory");
             XTile x;
-            for (int kb = 0; kb < nkb; ++kb) {
+            for (int kb = 0; ok && kb < nkb; ++kb) {
                 const int s = kb % kStages;
-                for (int i = 0; kByTile<kXTiles, kTmemW> && i < ntiles; ++i, x.next<kXTiles>()) {
-                    if (ok) ok = wait_parity(&sm.x_done[x.at], x.parity);
-                    arrive_at(&sm.x_done[x.at], 1u);
+                for (int i = 0; ok && kByTile<kXTiles, kTmemW> && i < ntiles; ++i, x.next<kXTiles>()) {
+                    ok = wait_parity(&sm.x_done[x.at], x.parity);
+                    if (ok) arrive_at(&sm.x_done[x.at], 1u);
                 }
                 if (ok) ok = wait_parity(&sm.mma_done[s], (kb / kStages) & 1);
-                arrive_at(&sm.mma_done[s], 1u);
+                if (ok) arrive_at(&sm.mma_done[s], 1u);
             }
         }
         __syncwarp();
@@ -1361,15 +1364,16 @@ spmm_kernel(const __grid_constant__ Params p, const __grid_constant__ CUtensorMa
             // The first K-block finds room in the ring in any case and kStages of them are decoded before any product; one that
             // is still outside then waits for room, and so, like everything behind the first products, for X.
             if (kb > 0 && kb < 2 * kStages && (kb >= kStages || !phase_done(&sm.comp_full[m], 0u))) asm volatile("griddepcontrol.wait;" ::: "memory");
-            if (ok) ok = wait_parity(&sm.comp_full[m], (kb / kMeta) & 1);                   // the stored block has arrived
+            ok = __all_sync(0xFFFFFFFFu, wait_parity(&sm.comp_full[m], (kb / kMeta) & 1));  // the stored block has arrived
+            if (!ok) break;
             const Meta& mt = sm.meta[m];
-            __syncwarp();
             if constexpr (kTmemW) scan_eighth(p, mt, static_cast<int>(j0) + lane, eighth, tab_me);
             else scan4(p, mt.bm, mt.ci, mt.start, mt.ngt, mt.limit, static_cast<int>(j0), lane, &sm.tab[warp][0]);
             __syncwarp();
-            if (kb >= kStages && ok) ok = wait_parity(&sm.mma_done[s], ((kb / kStages) & 1u) ^ 1u);  // the tensor cores are done with this A stage
+            if (kb >= kStages) ok = wait_parity(&sm.mma_done[s], ((kb / kStages) & 1u) ^ 1u);        // the tensor cores are done with this A stage
+            ok = __all_sync(0xFFFFFFFFu, ok);
+            if (!ok) break;
             if constexpr (kTmemW) {
-                __syncwarp();
                 asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
 #pragma unroll 1
                 for (int c0 = 0; c0 < kSub; c0 += 16) {
@@ -1475,6 +1479,14 @@ spdp_status resident_clusters(int dev) {
     return SPDP_OK;
 }
 }  // namespace
+
+#ifdef SPDP_CHECKED
+// Checked build: waits of the prefill kernels of the current device run out after `tries` attempts, so that a test sees what is left then.
+extern "C" SPDP_API spdp_status spdp_checked_wait_tries(int tries) {
+    SPDP_CUDA_TRY(cudaMemcpyToSymbol(g_wait_tries, &tries, sizeof(int)));
+    return SPDP_OK;
+}
+#endif
 
 spdp_status configure_spmm_kernel() {
     static std::mutex mu;

@@ -1,0 +1,98 @@
+"""Waits of the prefill kernels that run out.  The checked build lets a test set after how many attempts they do; with a few, roles give up all over the
+call, each at another place.  What is left then: the kernels end, the status says so, no output is wrong (it is right or unwritten) although the
+scratch memory still holds an earlier call's sums, and the next call is whole.  Small whole numbers, so that sums are exact in any order.
+Nothing here reads or writes out of range or waits without a limit: a role that gives up touches nothing any more, hands nothing on, and a CTA leaves when
+its copies and products have landed."""
+import ctypes
+
+import pytest
+
+torch = pytest.importorskip("torch")
+
+from device_plan import device_plan
+
+# row tiles, K, tokens, sparsity -> kernel, cut, CTA ranges that cross tiles
+ONE = {
+    (1, 2600, 1, 0.5): (0, True, False),
+    (149, 64, 20, 0.0): (0, False, False),
+    (50, 2600, 20, 0.5): (1, True, True),
+    (150, 1000, 30, 0.9): (1, True, False),
+    (75, 2000, 129, 0.5): (2, True, True),
+    (60, 64, 100, 0.5): (2, False, False),
+}
+# -> kernel, whole tiles, cut tiles (sparse layers have three X tiles in flight for each accumulator)
+PAIRS = {
+    (75, 640, 400, 0.5): (3, True, True),
+    (75, 640, 400, 0.9): (3, True, True),
+    (3, 12000, 1024, 0.9): (3, False, True),
+    (8, 3000, 150, 0.5): (4, False, True),
+    (8, 3000, 150, 0.9): (4, False, True),
+    (22, 700, 1024, 0.5): (4, True, False),
+    (38, 5000, 257, 0.5): (4, False, True),
+}
+
+
+@pytest.mark.parametrize("shape", list(ONE))
+def test_shapes_of_one_cta(shape):
+    q = device_plan(*shape[:3])
+    assert (q["kernel"], q["cut"], q["crosses"]) == ONE[shape] and q["cluster"] == 1
+
+
+@pytest.mark.parametrize("shape", list(PAIRS))
+def test_shapes_of_pairs(shape):
+    q = device_plan(*shape[:3])
+    assert (q["kernel"], q["tiles"] > q["rest"], q["cut"]) == PAIRS[shape]
+
+
+@pytest.fixture(scope="module")
+def S():
+    if not torch.cuda.is_available():
+        pytest.skip("needs a CUDA device")
+    from paper_2607_21985_b200 import build, spdp
+    saved = (spdp.LIB_PATH, spdp._lib)
+    spdp.LIB_PATH, spdp._lib = build.build_checked(), None
+    spdp.lib().spdp_checked_wait_tries.argtypes = [ctypes.c_int]
+    yield spdp
+    spdp.LIB_PATH, spdp._lib = saved
+
+
+def give_up(S, R, K, N, sparsity):
+    M = 256 * R - 5
+    g = torch.Generator(device="cuda").manual_seed(R * K + N)
+    W = torch.randint(1, 5, (M, K), generator=g, device="cuda").half() * (2 * torch.randint(0, 2, (M, K), generator=g, device="cuda") - 1).half()
+    W[torch.rand(M, K, generator=g, device="cuda") < sparsity] = 0
+    X = torch.zeros(N, (K + 7) // 8 * 8, dtype=torch.float16, device="cuda")
+    X[:, :K] = torch.randint(1, 3, (N, K), generator=g, device="cuda").half()
+    want = X[:, :K].double() @ W.double().T
+    other = -X                                                  # whose sums are in the scratch memory
+    h = S.spdp_pack_tiled_cbc(W)
+    L = S.lib()
+    limit = 1 << 22
+    incomplete = 0
+    try:
+        def call(x):
+            Y = torch.full((N, M), float("nan"), device="cuda")
+            S.spdp_spmm(h, x[:, :K], Y)
+            return Y.double(), S.spdp_last_device_status(h)
+        for tries in (0, 1, 2, 4, 8, 16, 32, 64, 128):
+            Y, status = call(other)
+            assert status == 0 and torch.equal(Y, -want)
+            assert L.spdp_checked_wait_tries(tries) == 0
+            Y, status = call(X)
+            assert L.spdp_checked_wait_tries(limit) == 0
+            unwritten = torch.isnan(Y)
+            assert bool((unwritten | (Y == want)).all()), tries
+            assert status == S.SPDP_ERR_TIMEOUT or (status == 0 and not bool(unwritten.any())), tries
+            incomplete += bool(unwritten.any())
+        assert incomplete > 0                                   # without any attempt nobody gets far
+        Y, status = call(X)
+        assert status == 0 and torch.equal(Y, want)
+    finally:
+        L.spdp_checked_wait_tries(limit)
+        S.spdp_free(h)
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("shape", list(ONE) + list(PAIRS))
+def test_nothing_wrong_is_left(S, shape):
+    give_up(S, *shape)
