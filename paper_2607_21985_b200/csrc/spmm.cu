@@ -97,10 +97,16 @@ constexpr int kBAtomBytes = 8 * kBRowBytes;
 constexpr int kWaitTries = SPDP_SPMM_WAIT_TRIES;
 constexpr int kDrainTries = 1 << 18;   // of a wait for what the CTA itself has under way, after which it leaves: these land in microseconds
 #ifdef SPDP_CHECKED
-__device__ int g_wait_tries = kWaitTries;      // checked build: a test makes waits run out (spdp_checked_wait_tries)
-__device__ __forceinline__ int wait_tries() { return *static_cast<volatile int*>(&g_wait_tries); }
+// Checked build: a test makes waits run out (spdp_checked_wait_tries), those of some warps of some CTAs (by their number modulo 16) sooner than
+// the others': all waits, or only those for a piece's products to be complete.
+struct WaitTries { int chosen, others; unsigned warps, ctas; int products_only; };
+__device__ WaitTries g_wait_tries = {kWaitTries, kWaitTries, 0u, 0u, 0};
+__device__ __forceinline__ int wait_tries(bool products = false) {
+    const volatile WaitTries& g = g_wait_tries;
+    return (g.warps >> (threadIdx.x >> 5) & 1u) != 0u && (g.ctas >> (blockIdx.x & 15u) & 1u) != 0u && (products || g.products_only == 0) ? g.chosen : g.others;
+}
 #else
-__device__ __forceinline__ constexpr int wait_tries() { return kWaitTries; }
+__device__ __forceinline__ constexpr int wait_tries(bool = false) { return kWaitTries; }
 #endif
 static_assert(kBRowBytes == 128, "one X row of a K-block is one 128-byte swizzle row");
 
@@ -1015,7 +1021,7 @@ spmm_kernel(const __grid_constant__ Params p, const __grid_constant__ CUtensorMa
             if (warp >= F::kStorers) continue;
             // ---- the piece's products are complete: store the accumulators ----
             asm volatile("griddepcontrol.wait;" ::: "memory");          // Y and the scratch may belong to the kernel before this one
-            if (ok) ok = wait_parity(&sm.acc_full, k & 1);
+            if (ok) ok = wait_parity(&sm.acc_full, k & 1, wait_tries(true));
             asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
             ok = __all_sync(0xFFFFFFFFu, ok);
             const bool complete = ok && !__any_sync(0xFFFFFFFFu, *static_cast<volatile int*>(&sm.abort) != 0);
@@ -1033,11 +1039,12 @@ spmm_kernel(const __grid_constant__ Params p, const __grid_constant__ CUtensorMa
                 }
             }
             if constexpr (shared_tile) {
-                if (!complete) {                                       // nobody may add what I have not stored
+                if (!complete) {                                       // nobody may add what I have not stored: my rows of my tokens, as above
                     *static_cast<volatile int*>(&sm.abort) = 1;
-                    for (int c = static_cast<int>(group); c < p.ptok; c += F::kGroups)
-                        for (int e = lane; e < 64; e += 32)
-                            reinterpret_cast<unsigned*>(p.partial)[(static_cast<size_t>(s.slot) * p.ptok + c) * kTileM + 64 * wm + e] = kNoSum;
+                    for (int c0 = 8 * static_cast<int>(group); c0 < p.ptok; c0 += 8 * F::kGroups)
+                        for (int e = lane; e < 8 * 64; e += 32)
+                            if (c0 + e / 64 < p.ptok)
+                                reinterpret_cast<unsigned*>(p.partial)[(static_cast<size_t>(s.slot) * p.ptok + c0 + e / 64) * kTileM + 64 * wm + e % 64] = kNoSum;
                 }
                 break;
             }
@@ -1398,7 +1405,7 @@ spmm_kernel(const __grid_constant__ Params p, const __grid_constant__ CUtensorMa
     // the last blocks' tensor-core work, for which X has to be there; Y and the scratch may belong to the kernel before this one, too
     asm volatile("griddepcontrol.wait;" ::: "memory");
     for (int kb = (nkb > kStages ? nkb - kStages : 0); ok && kb < nkb; ++kb)
-        ok = wait_parity(&sm.mma_done[kb % kStages], (kb / kStages) & 1);
+        ok = wait_parity(&sm.mma_done[kb % kStages], (kb / kStages) & 1, wait_tries(true));
     if (!ok) {
         sm.abort = 1;
         if (lane == 0) atomicCAS(p.status, 0, SPDP_ERR_TIMEOUT);
@@ -1481,9 +1488,11 @@ spdp_status resident_clusters(int dev) {
 }  // namespace
 
 #ifdef SPDP_CHECKED
-// Checked build: waits of the prefill kernels of the current device run out after `tries` attempts, so that a test sees what is left then.
-extern "C" SPDP_API spdp_status spdp_checked_wait_tries(int tries) {
-    SPDP_CUDA_TRY(cudaMemcpyToSymbol(g_wait_tries, &tries, sizeof(int)));
+// Checked build: how many attempts the waits of the current device's prefill kernels make, so that a test sees what is left when they run out.
+// A negative number is the ordinary limit.
+extern "C" SPDP_API spdp_status spdp_checked_wait_tries(int chosen, int others, unsigned warps, unsigned ctas, int products_only) {
+    const WaitTries g = {chosen < 0 ? kWaitTries : chosen, others < 0 ? kWaitTries : others, warps, ctas, products_only};
+    SPDP_CUDA_TRY(cudaMemcpyToSymbol(g_wait_tries, &g, sizeof(g)));
     return SPDP_OK;
 }
 #endif

@@ -30,6 +30,21 @@ PAIRS = {
     (22, 700, 1024, 0.5): (4, True, False),
     (38, 5000, 257, 0.5): (4, False, True),
 }
+# -> kernel, CTAs of a cluster: each adds up a share of the tokens, where another's sums are missing if that one gave up
+CLUSTERS = {
+    (35, 200, 20, 0.5): (0, 2),
+    (27, 1000, 2, 0.5): (0, 4),
+    (6, 1600, 2, 0.9): (0, 9),
+    (26, 640, 250, 0.5): (1, 2),
+    (43, 4096, 128, 0.6): (1, 3),
+    (15, 9000, 128, 0.5): (1, 9),
+}
+
+
+@pytest.mark.parametrize("shape", list(CLUSTERS))
+def test_shapes_of_clusters(shape):
+    q = device_plan(*shape[:3])
+    assert (q["kernel"], q["cluster"]) == CLUSTERS[shape]
 
 
 @pytest.mark.parametrize("shape", list(ONE))
@@ -51,35 +66,46 @@ def S():
     from paper_2607_21985_b200 import build, spdp
     saved = (spdp.LIB_PATH, spdp._lib)
     spdp.LIB_PATH, spdp._lib = build.build_checked(), None
-    spdp.lib().spdp_checked_wait_tries.argtypes = [ctypes.c_int]
+    spdp.lib().spdp_checked_wait_tries.argtypes = [ctypes.c_int, ctypes.c_int, ctypes.c_uint, ctypes.c_uint, ctypes.c_int]
     yield spdp
     spdp.LIB_PATH, spdp._lib = saved
 
 
-def give_up(S, R, K, N, sparsity):
+# attempts of the chosen warps and of the others, chosen warps, chosen CTAs (modulo 16): all at once, then one role at a time, in all CTAs, in every
+# second, in one of 16; then only where a warp waits for the products before it stores them (all warps do in a pair).  Warps 0 to 23 decode, the first of them store; behind them
+# the tensor-core, copy and X or relay warps.
+ALL, LATE = 0xFFFFFFFF, 1 << 12
+LIMITS = [(tries, tries, ALL, 0xFFFF, 0) for tries in (0, 1, 2, 4, 8, 16, 32, 64, 128)]
+LIMITS += [(tries, LATE, 1 << warp, ctas, 0) for warp in (0, 5, 10, 15, 23, 24, 25, 26, 27) for ctas in (0xFFFF, 0x5555, 0xAAAA, 0x0200) for tries in (0, 2, 16)]
+LIMITS += [(0, LATE, warps, ctas, 1) for warps in (1, 1 << 5, 1 << 10, 1 << 23, 1 << 24, ALL) for ctas in (0xFFFF, 0x5555, 0xAAAA, 0x0200)]
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("shape", list(ONE) + list(PAIRS) + list(CLUSTERS))
+def test_nothing_wrong_is_left(S, shape):
+    R, K, N, sparsity = shape
     M = 256 * R - 5
     g = torch.Generator(device="cuda").manual_seed(R * K + N)
     W = torch.randint(1, 5, (M, K), generator=g, device="cuda").half() * (2 * torch.randint(0, 2, (M, K), generator=g, device="cuda") - 1).half()
     W[torch.rand(M, K, generator=g, device="cuda") < sparsity] = 0
     X = torch.zeros(N, (K + 7) // 8 * 8, dtype=torch.float16, device="cuda")
     X[:, :K] = torch.randint(1, 3, (N, K), generator=g, device="cuda").half()
-    want = X[:, :K].double() @ W.double().T
+    want = (X[:, :K].double() @ W.double().T).float()
     other = -X                                                  # whose sums are in the scratch memory
     h = S.spdp_pack_tiled_cbc(W)
-    L = S.lib()
-    limit = 1 << 22
+    limit = S.lib().spdp_checked_wait_tries
     incomplete = 0
     try:
         def call(x):
             Y = torch.full((N, M), float("nan"), device="cuda")
             S.spdp_spmm(h, x[:, :K], Y)
-            return Y.double(), S.spdp_last_device_status(h)
-        for tries in (0, 1, 2, 4, 8, 16, 32, 64, 128):
+            return Y, S.spdp_last_device_status(h)
+        for tries in LIMITS:
             Y, status = call(other)
             assert status == 0 and torch.equal(Y, -want)
-            assert L.spdp_checked_wait_tries(tries) == 0
+            assert limit(*tries) == 0
             Y, status = call(X)
-            assert L.spdp_checked_wait_tries(limit) == 0
+            assert limit(-1, -1, 0, 0, 0) == 0
             unwritten = torch.isnan(Y)
             assert bool((unwritten | (Y == want)).all()), tries
             assert status == S.SPDP_ERR_TIMEOUT or (status == 0 and not bool(unwritten.any())), tries
@@ -88,11 +114,5 @@ def give_up(S, R, K, N, sparsity):
         Y, status = call(X)
         assert status == 0 and torch.equal(Y, want)
     finally:
-        L.spdp_checked_wait_tries(limit)
+        limit(-1, -1, 0, 0, 0)
         S.spdp_free(h)
-
-
-@pytest.mark.gpu
-@pytest.mark.parametrize("shape", list(ONE) + list(PAIRS))
-def test_nothing_wrong_is_left(S, shape):
-    give_up(S, *shape)
