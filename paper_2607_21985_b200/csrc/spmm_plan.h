@@ -139,7 +139,7 @@ inline Plan make_plan(int64_t R, int64_t nkb, int64_t N, int sms, bool may_cut, 
             for (int slices = most + 1; slices <= kMostSlices && slices * left * tokens <= kScratchTokens; ++slices) consider(slices * left);
         if (resident == nullptr || rounds > 0 || f > 1) continue;                // clusters: the one-CTA forms with W in tensor memory
         const int c0 = blocks_at_best(kClusterEach + kClusterPerMB * mb * static_cast<double>(left));
-        int largest = kMaxCluster;
+        int largest = std::min(kMaxCluster, blocks);        // every CTA has a K-block
         while (largest > 1 && (left > resident[largest] || (largest - 1) * ((tokens + largest - 1) / largest) > kGatherTokens)) --largest;
         for (int n = std::max(1, c0 - 1), last = 1; n <= c0 + 4; ++n) {
             const int c = n == c0 + 4 ? largest : std::min((blocks + n - 1) / n, largest);

@@ -78,6 +78,16 @@ def test_plans_hold_together(plan, resident):
     assert resident is RESIDENT or not any(c for _, c in seen)
 
 
+def test_every_cta_of_a_cluster_has_a_k_block(plan):
+    """Whatever sizes of clusters a device holds, sizes in between not among them."""
+    for only in range(2, 17):
+        resident = [148, 148] + [7 if c == only else 0 for c in range(2, 17)]
+        for R in (1, 2, 3, 5, 7):
+            for nkb in range(1, 20):
+                for N in (1, 7, 16, 33, 128):
+                    assert plan(R, 64 * nkb, N, resident=resident)["cluster"] <= nkb
+
+
 def test_shapes_take_the_pairs(plan):
     whole, more, cut = 0, 0, 0
     for M, K, N, _ in PAIRS:
