@@ -86,7 +86,6 @@ inline Plan make_plan(int64_t R, int64_t nkb, int64_t N, int sms, bool may_cut, 
         Plan q = {};
         q.kernel = f;
         q.tiles = R * ((N + tile_tokens - 1) / tile_tokens);
-        if (f == 4 && q.tiles * nkb > INT32_MAX) continue;                       // K-blocks are counted in 31 bits: fewer, larger tiles then
         const int64_t slots = pairs ? sms / 2 : sms;                             // CTAs or pairs resident at once
         const int64_t rounds = q.tiles / slots, left = q.tiles - rounds * slots;
         const int64_t tokens = std::min<int64_t>(N, tile_tokens);
