@@ -20,6 +20,7 @@ def lib():
             _lib = ctypes.CDLL(out)
         _lib.shim_device_plan.argtypes = [ctypes.c_longlong] * 3 + [ctypes.c_int] + [ctypes.c_void_p] * 2
         _lib.shim_pair_acc_tokens.argtypes = _lib.shim_pair_tile_tokens.argtypes = [ctypes.c_longlong]
+        _lib.shim_pair_tiles_in_flight.argtypes = [ctypes.c_longlong] * 3
     return _lib
 
 
@@ -30,3 +31,8 @@ def device_plan(R, K, N, sms=148, resident=RESIDENT):
     q["cut"] = q["rest"] > 0 and q["sharers"] > q["rest"]
     q["crosses"] = q["cut"] and q["kernel"] < 3 and q["sharers"] % q["rest"] > 0        # a CTA's range may end in the next tile
     return q
+
+
+def pair_x_tiles(R, K, sparsity):
+    """X tiles that a CTA pair has in flight."""
+    return lib().shim_pair_tiles_in_flight(int(256 * R * K * (1.0 - sparsity)), R, (K + 63) // 64)

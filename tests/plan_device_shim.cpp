@@ -9,3 +9,4 @@ extern "C" void shim_device_plan(long long R, long long nkb, long long N, int sm
 }
 extern "C" int shim_pair_acc_tokens(long long N) { return spdp::plan::pair_acc_tokens(N); }
 extern "C" int shim_pair_tile_tokens(long long N) { return spdp::plan::pair_tile_tokens(N); }
+extern "C" int shim_pair_tiles_in_flight(long long values_len, long long R, long long nkb) { return spdp::plan::pair_x_tiles(values_len, R, nkb); }
