@@ -184,7 +184,8 @@ SPDP_API spdp_status spdp_spmspv_batch(spdp_handle h, const void* x_dev, int64_t
  * work, or a pair's.  Where whole tiles would leave SMs idle, which is the rule for short prompts and small
  * layers, the tiles that do not fill a round (often all of them) are cut along K: several CTAs leave fp32 partial
  * sums of a tile in scratch memory, and they (as a thread-block cluster) or a further kernel add them in a fixed order.  Which tiles are
- * cut follows from M, K, N and the device alone (its SMs and the clusters that it holds at once), so repeated calls give identical bits.
+ * cut follows from M, K, N, ydt and the device alone (its SMs and the clusters that it holds at once), so repeated calls give identical bits.
+ * 32-bit results are added up in shorter pieces where the fastest cut would make them less exact.
  *   The scratch memory, up to 77 MB on 148 SMs, comes from a stream-ordered pool of the library's (cudaMallocFromPoolAsync /
  * cudaFreeAsync on `stream`; in a stream capture it becomes memory of the graph).  The pool keeps up to 96 MB until the
  * device's last handle is freed; spdp_free(NULL) gives back what is unused.  Where there is no memory for it the call

@@ -133,6 +133,7 @@ struct Params {
     // pair:: pair i works on tile tile0 + i / kslices, on slice i % kslices of the tile's K-blocks
     int tile0, kslices;
     int acc_tokens, tile_tokens;    // tokens of an accumulator, and of a tile
+    int sets, set_columns;  // accumulators that a tile's (sub-)blocks are added to in turn; one:: tensor-memory columns from one to the next
     float* partial;         // partial sums [slot][token in tile < ptok][256 rows]; slot = pair i, or 2 * CTA + (0: its first
                             // piece, 1: its last); pair:: null = whole tiles
     int ptok;
@@ -361,6 +362,19 @@ __device__ __forceinline__ void tmem_load8(uint32_t at, uint32_t (&v)[8]) {
                  : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7]) : "r"(at) : "memory");
 }
 
+// Adds eight columns each of two places to v and w.
+__device__ __forceinline__ void add_tmem8(uint32_t at_v, uint32_t at_w, uint32_t (&v)[8], uint32_t (&w)[8]) {
+    uint32_t a[8], b[8];
+    tmem_load8(at_v, a);
+    tmem_load8(at_w, b);
+    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+        v[i] = __float_as_uint(__uint_as_float(v[i]) + __uint_as_float(a[i]));
+        w[i] = __float_as_uint(__uint_as_float(w[i]) + __uint_as_float(b[i]));
+    }
+}
+
 // Scan for the expansion into tensor memory: lane = column j of the K-block, for the 64 rows of quarter q of the row tile.  The two
 // bitmap words of those rows and the address of each one's first value go to tab[lane] (rows 0 .. 31 of the quarter) and
 // tab[kTabRow + lane] (rows 32 .. 63).  Four words are read, the half of the column tile that the quarter is in; the values before the
@@ -494,10 +508,11 @@ __device__ __forceinline__ void store_four(void* Y, int ydt, int64_t at, float a
 // row's.  kFours: four neighbouring threads trade values first, so that each stores 4 rows of every fourth token at once, where Y allows it (a
 // store of 32 single values costs as much as one of 32 fours): CTA pairs, which store whole tiles more often than not, 28672x8192 x 300
 // tokens 207.8 -> 203.2 us, 18944x4096 x 512 65.5 -> 64.0, 3000x700 x 1024 16.7 -> 15.9.  The one-CTA forms mostly leave partial sums, whose
-// stores gain nothing by it, and are 1 to 2 % slower with the longer code.
+// stores gain nothing by it, and are 1 to 2 % slower with the longer code.  second: columns to the other accumulator that belongs to the sums, 0: there
+// is none.
 template <bool kFours>
 __device__ __forceinline__ void store_accumulators(const Params& p, uint32_t tmem, int lane_base, int c_begin, int c_end,
-                                                   int r, int row_in, int64_t n0, int slot, int tok0 = 0) {
+                                                   int r, int row_in, int64_t n0, int slot, int tok0 = 0, uint32_t second = 0) {
     const int lane = threadIdx.x & 31;
     const int valid = static_cast<int>(min(p.N - n0, static_cast<int64_t>(c_end)));
     const int64_t row0 = static_cast<int64_t>(r) * kTileM + row_in;
@@ -511,6 +526,10 @@ __device__ __forceinline__ void store_accumulators(const Params& p, uint32_t tme
                        "=r"(v[8]), "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]), "=r"(v[14]), "=r"(v[15])
                      : "r"(tmem + (static_cast<uint32_t>(lane_base) << 16) + c0) : "memory");
         asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+        if (kFours && second != 0u) {
+            const uint32_t at = tmem + second + (static_cast<uint32_t>(lane_base) << 16) + c0;
+            add_tmem8(at, at + 8u, reinterpret_cast<uint32_t(&)[8]>(v[0]), reinterpret_cast<uint32_t(&)[8]>(v[8]));
+        }
         if (kFours && fours) {
 #pragma unroll
             for (int i = 0; i < 16; i += 4) {
@@ -546,15 +565,18 @@ __device__ __forceinline__ void store_two(const Params& p, int64_t n, int64_t ro
     if (row + 1 < p.M) store_y(p.Y, p.ydt, at + 1, b);
 }
 // The same for the forms with W in tensor memory, where lane l of quarter q holds row 64q + 2l in the first accumulator and the row
-// after it in the second, kNI columns further: tokens [c0, c0 + 8), two neighbouring rows at once.  Tokens [own0, own1) of partial sums go to
-// shared memory (at `own`) instead.
-template <int kNI, bool kOwn>
-__device__ __forceinline__ void store_row_pairs(const Params& p, uint32_t tmem, int q, int c0, int valid, int r, int64_t n0, int slot, int own0, int own1, uint32_t own) {
+// after it in the second, kAccCols columns further: tokens [c0, c0 + 8), two neighbouring rows at once.  Tokens [own0, own1) of partial sums go to
+// shared memory (at `own`) instead.  `sets` accumulators, p.set_columns apart, make up the sums.
+template <int kAccCols, bool kOwn>
+__device__ __forceinline__ void store_row_pairs(const Params& p, uint32_t tmem, int q, int c0, int valid, int r, int64_t n0, int slot, int own0, int own1, uint32_t own, int sets) {
     const int lane = threadIdx.x & 31, row_in = 64 * q + 2 * lane;
+    const uint32_t at_tmem = tmem + (static_cast<uint32_t>(32 * q) << 16) + c0;
     uint32_t v[8], w[8];
-    tmem_load8(tmem + (static_cast<uint32_t>(32 * q) << 16) + c0, v);
-    tmem_load8(tmem + (static_cast<uint32_t>(32 * q) << 16) + kNI + c0, w);
+    tmem_load8(at_tmem, v);
+    tmem_load8(at_tmem + kAccCols, w);
     asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+#pragma unroll 1
+    for (int e = 1; e < sets; ++e) add_tmem8(at_tmem + e * p.set_columns, at_tmem + kAccCols + e * p.set_columns, v, w);
     if (slot >= 0) {
         float* part = p.partial + (static_cast<size_t>(slot) * p.ptok + c0) * kTileM + row_in;
         const uint32_t at = own + 4u * static_cast<uint32_t>((c0 - own0) * kTileM + row_in);
@@ -742,14 +764,16 @@ __device__ __forceinline__ bool await_copies(const CopyState& c, unsigned long l
 // ===================================================================================================
 namespace one {     // one CTA = one row tile x kNI tokens
 
-template <int kNIT, bool kClusterT = false>
+template <int kNIT, bool kClusterT = false, bool kSetsT = false>
 struct Form {
     static constexpr int kNI = kNIT;                                  // the N of the tensor-core instruction = tokens per tile
     static constexpr bool kTmemW = kNI <= 128;                        // decoded W in tensor memory, where there is room for it
     static constexpr bool kCluster = kClusterT;                       // clusters share tiles; a build of its own, whose code costs the others up to 2 %
-    static_assert(!kCluster || kTmemW, "only with W in tensor memory");
+    static constexpr bool kSets = kSetsT;                             // several accumulators (Params::sets); a build of its own, or the others are 1 to 1.5 % slower
+    static_assert((!kCluster && !kSets) || kTmemW, "only with W in tensor memory");
     static constexpr int kGroupWarps = kTmemW ? 4 : spdp::kGroupWarps;
     static constexpr int kGroups = kWarps / kGroupWarps;
+    static constexpr int kAccCols = kSets ? plan::kSetColumns : kNI;  // columns for either row half's accumulator, or accumulators
     static constexpr int kTmemCols = kTmemW ? 512 : 2 * kNI;          // two accumulators (of 128 rows each), and W
     static constexpr int kBBytes = kNI * kBRowBytes;
     static constexpr int kATileBytes = (kSub / 8) * kAKGroupStride;   // 128 rows x kSub columns
@@ -762,7 +786,7 @@ struct Form {
     static constexpr int kStorers = kTmemW ? kWarps : kStoreWarps;
     static_assert(kBBytes % 1024 == 0, "every X tile on a swizzle-atom boundary");
     static_assert(kAStages >= 2 * kSubs && kAStages >= kGroups, "the first two K-blocks fit in the first A stages, and every decode warp has a sub-block among the next kAStages");
-    static_assert(!kTmemW || 2 * kNI + kAStages * kACols <= kTmemCols, "accumulators and W fit tensor memory");
+    static_assert(kNI <= kAccCols && (!kTmemW || 2 * kAccCols + kAStages * kACols <= kTmemCols), "accumulators and W fit tensor memory");
 };
 
 // CTA w's share of the tiles that are cut along K: K-blocks [rest_begin(w), rest_begin(w + 1)).
@@ -904,15 +928,17 @@ spmm_kernel(const __grid_constant__ Params p, const __grid_constant__ CUtensorMa
                         if (!ok) break;
                         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
                         const uint32_t al = a_base + sa * (F::kABytes >> 4), bl = b_base + sb * (F::kBBytes >> 4) + h * ((2 * kSub) >> 4);
-                        const uint32_t add = static_cast<uint32_t>(kb + h);      // the first product of a piece starts the sums
+                        const uint32_t step = static_cast<uint32_t>(kb * kSubs + h);
+                        const uint32_t add = F::kSets ? (step >= static_cast<uint32_t>(p.sets) ? 1u : 0u) : static_cast<uint32_t>(kb + h);      // the first products of a piece start the sums
+                        const uint32_t sums = F::kSets ? tmem + (step & static_cast<uint32_t>(p.sets - 1)) * static_cast<uint32_t>(p.set_columns) : tmem;
 #pragma unroll
                         for (int a = 0; a < 2; ++a) {                   // the two row halves
 #pragma unroll
                             for (int kk = 0; kk < kSub / 16; ++kk)      // the start address is the low field, in 16-byte units
                                 if constexpr (F::kTmemW) mma_f16_tmem<kDescHigh<kBAtomBytes, 2u>>(
-                                    tmem + a * F::kNI, tmem + 2 * F::kNI + sa * F::kACols + a * (F::kACols / 2) + kk * 8, bl + ((kk * 32) >> 4), id, kk > 0 ? 1u : add);
+                                    sums + a * F::kAccCols, tmem + 2 * F::kAccCols + sa * F::kACols + a * (F::kACols / 2) + kk * 8, bl + ((kk * 32) >> 4), id, kk > 0 ? 1u : add);
                                 else mma_f16_one<kDescHigh<kAChunkStride, 0u>, kDescHigh<kBAtomBytes, 2u>>(
-                                    tmem + a * F::kNI, al + ((a * F::kATileBytes + kk * 2 * kAKGroupStride) >> 4), bl + ((kk * 32) >> 4),
+                                    sums + a * F::kAccCols, al + ((a * F::kATileBytes + kk * 2 * kAKGroupStride) >> 4), bl + ((kk * 32) >> 4),
                                     id, kk > 0 ? 1u : add);
                         }
                         commit_one(&sm.a_free[sa]);
@@ -964,7 +990,7 @@ spmm_kernel(const __grid_constant__ Params p, const __grid_constant__ CUtensorMa
         const unsigned group = static_cast<unsigned>(warp) / F::kGroupWarps, wm = static_cast<unsigned>(warp) % F::kGroupWarps;
         const unsigned top = pinned(F::kTmemW ? 1u << (30u - 2u * (lane & 15u)) : nibble_top(lane & 7)), below = pinned(nibble_below(lane & 7));
         const uint32_t tab_l = pinned(smem_u32(&sm.tab[warp][0]) + 8u * (F::kTmemW ? kTabRow * (lane >> 4) : lane >> 3));
-        const uint32_t a_lane = pinned(F::kTmemW ? tmem + (32u * wm << 16) + 2u * F::kNI
+        const uint32_t a_lane = pinned(F::kTmemW ? tmem + (32u * wm << 16) + 2u * F::kAccCols
                                                  : smem_u32(&sm.A[0]) + (lane >> 1) * kAChunkStride + (lane & 1) * 8 + (wm >> 1) * kAKGroupStride + (wm & 1u) * 64u);
         const uint32_t tab_me = pinned(smem_u32(&sm.tab[warp][0]) + 8u * lane);
         const Quarter quarter(static_cast<int>(wm));
@@ -1031,7 +1057,8 @@ spmm_kernel(const __grid_constant__ Params p, const __grid_constant__ CUtensorMa
                     const int valid = static_cast<int>(min(p.N - n0, static_cast<int64_t>(F::kNI)));
                     const int own0 = shared_tile ? own_begin(p, rank) : 0, own1 = shared_tile ? own_begin(p, rank + 1) : 0;
                     for (int c0 = 8 * static_cast<int>(group); c0 < valid; c0 += 8 * F::kGroups)
-                        store_row_pairs<F::kNI, shared_tile>(p, tmem, static_cast<int>(wm), c0, valid, s.tile / p.nblocks, n0, s.slot, own0, own1, smem_u32(&sm.B[0][0]));
+                        store_row_pairs<F::kAccCols, shared_tile>(p, tmem, static_cast<int>(wm), c0, valid, s.tile / p.nblocks, n0, s.slot, own0, own1, smem_u32(&sm.B[0][0]),
+                                                                  F::kSets ? min(p.sets, s.n * kSubs) : 1);
                 } else {
                     // warp w: row half (w / 4) % 2, tensor-memory lanes 32 * (w % 4).., token columns [(w / 8) * kNI / 2, + kNI / 2)
                     const int half = (warp >> 2) & 1, cbase = (warp >> 3) * (F::kNI / 2), lane_base = 32 * (warp & 3);
@@ -1277,11 +1304,12 @@ spmm_kernel(const __grid_constant__ Params p, const __grid_constant__ CUtensorMa
                     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
                     const uint64_t bd0 = operand_desc(smem_u32(&sm.B[x.at][0]), 16, kBAtomBytes, 2u);
                     const int tokens = i == ntiles - 1 ? last_tokens : acc;
+                    const uint32_t sums = tmem + static_cast<uint32_t>(i + (kb & (p.sets - 1))) * kNextAcc;      // (two sets: one accumulator each)
                     const uint32_t id = kTmemW ? instr_desc_tmem(256, tokens) : instr_desc(256, tokens);
 #pragma unroll
                     for (int kk = 0; kk < kKB / 16; ++kk)    // the start address is the descriptor's low field, in 16-byte units
-                        if constexpr (kTmemW) mma_f16_pair_tmem(tmem + i * kNextAcc, tmem + (kTmemCols - kWCols) + s * (kWCols / kStages) + kk * 8, bd0 + ((kk * 32) >> 4), id, kb > 0 || kk > 0);
-                        else mma_f16_pair(tmem + i * kNextAcc, ad0 + ((kk * 2 * kAKGroupStride) >> 4), bd0 + ((kk * 32) >> 4), id, kb > 0 || kk > 0);
+                        if constexpr (kTmemW) mma_f16_pair_tmem(sums, tmem + (kTmemCols - kWCols) + s * (kWCols / kStages) + kk * 8, bd0 + ((kk * 32) >> 4), id, kb >= p.sets || kk > 0);
+                        else mma_f16_pair(sums, ad0 + ((kk * 2 * kAKGroupStride) >> 4), bd0 + ((kk * 32) >> 4), id, kb >= p.sets || kk > 0);
                     if (kByTile<kXTiles, kTmemW>) commit_pair(&sm.x_done[x.at]);
                 }
                 if (ok) commit_pair(&sm.mma_done[s]);
@@ -1418,7 +1446,7 @@ spmm_kernel(const __grid_constant__ Params p, const __grid_constant__ CUtensorMa
         const int lane_base = 32 * (warp & 3), i = ntiles == 2 ? warp >> 3 : 0;               // my accumulator
         const int part = ntiles == 2 ? acc / 2 : (acc / 4 + 15) / 16 * 16, cbase = (ntiles == 2 ? (warp >> 2) & 1 : warp >> 2) * part;
         store_accumulators<true>(p, tmem + i * kNextAcc, lane_base, cbase, min(cbase + part, acc), r, c * 128 + lane_base, n0 + i * acc,
-                           p.partial == nullptr ? -1 : static_cast<int>(pr), i * acc);
+                           p.partial == nullptr ? -1 : static_cast<int>(pr), i * acc, p.sets > 1 && nkb > 1 ? kNextAcc : 0u);
     } else if (*static_cast<volatile int*>(&sm.abort) && p.partial != nullptr) {
         void_rows(p, static_cast<int>(pr), c * 128, 128, t, kThreads);
     }
@@ -1452,6 +1480,10 @@ using One32 = one::Form<32>;
 using One128 = one::Form<128>;
 using Cluster32 = one::Form<32, true>;
 using Cluster128 = one::Form<128, true>;
+using OneSets32 = one::Form<32, false, true>;
+using OneSets128 = one::Form<128, false, true>;
+using ClusterSets32 = one::Form<32, true, true>;
+using ClusterSets128 = one::Form<128, true, true>;
 using One256 = one::Form<256>;
 
 }  // namespace
@@ -1462,7 +1494,7 @@ namespace {
 int g_resident[64][plan::kMaxCluster + 1];
 
 spdp_status resident_clusters(int dev) {
-    for (const auto kernel : {one::spmm_kernel<Cluster32>, one::spmm_kernel<Cluster128>}) {
+    for (const auto kernel : {one::spmm_kernel<Cluster32>, one::spmm_kernel<Cluster128>, one::spmm_kernel<ClusterSets32>, one::spmm_kernel<ClusterSets128>}) {
         SPDP_CUDA_TRY(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, one::kSmemBytes));
         SPDP_CUDA_TRY(cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1));
     }
@@ -1507,6 +1539,8 @@ spdp_status configure_spmm_kernel() {
     if (!configured[dev]) {
         SPDP_CUDA_TRY(cudaFuncSetAttribute(one::spmm_kernel<One32>, cudaFuncAttributeMaxDynamicSharedMemorySize, one::kSmemBytes));
         SPDP_CUDA_TRY(cudaFuncSetAttribute(one::spmm_kernel<One128>, cudaFuncAttributeMaxDynamicSharedMemorySize, one::kSmemBytes));
+        SPDP_CUDA_TRY(cudaFuncSetAttribute(one::spmm_kernel<OneSets32>, cudaFuncAttributeMaxDynamicSharedMemorySize, one::kSmemBytes));
+        SPDP_CUDA_TRY(cudaFuncSetAttribute(one::spmm_kernel<OneSets128>, cudaFuncAttributeMaxDynamicSharedMemorySize, one::kSmemBytes));
         SPDP_CUDA_TRY(cudaFuncSetAttribute(one::spmm_kernel<One256>, cudaFuncAttributeMaxDynamicSharedMemorySize, one::kSmemBytes));
         SPDP_CUDA_TRY(cudaFuncSetAttribute(pair::spmm_kernel<4, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(pair::kSmemBytes)));
         SPDP_CUDA_TRY(cudaFuncSetAttribute(pair::spmm_kernel<6, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(pair::kSmemBytes)));
@@ -1626,6 +1660,8 @@ spdp_status run_plan(const spdp_matrix* h, Params p, const Plan& plan, const __h
     p.ptok = static_cast<int>(std::min<int64_t>(p.N, nt));
     p.kslices = 1;
     p.cluster = plan.cluster;
+    p.sets = plan.sets;
+    p.set_columns = plan::kSetColumns / plan.sets;
     CUtensorMap xmap;
     p.xbox = pairs ? p.acc_tokens / 2 : (p.ptok + 15) / 16 * 16;
     spdp_status st = encode_x(&xmap, X, p.N, h->K, ldx, p.xbox);
@@ -1654,7 +1690,9 @@ spdp_status run_plan(const spdp_matrix* h, Params p, const Plan& plan, const __h
         p.rounds = plan.rounds;
         p.sharers = plan.sharers;
         p.rest_units = static_cast<unsigned>(plan.rest * p.nkb);
-        if (plan.cluster > 1) st = plan.kernel == 0 ? launch_one<Cluster32>(p, xmap, s) : launch_one<Cluster128>(p, xmap, s);
+        if (plan.cluster > 1 && plan.sets > 1) st = plan.kernel == 0 ? launch_one<ClusterSets32>(p, xmap, s) : launch_one<ClusterSets128>(p, xmap, s);
+        else if (plan.cluster > 1) st = plan.kernel == 0 ? launch_one<Cluster32>(p, xmap, s) : launch_one<Cluster128>(p, xmap, s);
+        else if (plan.sets > 1) st = plan.kernel == 0 ? launch_one<OneSets32>(p, xmap, s) : launch_one<OneSets128>(p, xmap, s);
         else st = plan.kernel == 0 ? launch_one<One32>(p, xmap, s) : plan.kernel == 1 ? launch_one<One128>(p, xmap, s) : launch_one<One256>(p, xmap, s);
         if (st == SPDP_OK && cut && plan.cluster == 1)
             st = launch_reduce(many ? one::reduce_pieces_kernel<kManySums> : one::reduce_pieces_kernel<kFewSums>, plan.rest, chunks, s, p, plan.rounds * plan.workers, chunks, nt);
@@ -1683,7 +1721,7 @@ spdp_status launch_spmm(const spdp_matrix* h, const __half* X, int64_t N, int64_
     p.values_len = h->values_len;
     p.nkb = static_cast<int>((h->K + kKB - 1) / kKB);
     const int sms = h->sm_count > 1 ? h->sm_count : 2;
-    spdp_status st = run_plan(h, p, make_plan(h->R, p.nkb, N, sms, true, g_resident[h->device]), X, ldx, s);
+    spdp_status st = run_plan(h, p, make_plan(h->R, p.nkb, N, sms, true, g_resident[h->device], ydt == SPDP_Y_F32), X, ldx, s);
     // No memory for partial sums: whole tiles only, which need none.  Slower, and another order of the sums.
     if (st == SPDP_ERR_ALLOC) st = run_plan(h, p, make_plan(h->R, p.nkb, N, sms, false), X, ldx, s);
     return st;

@@ -4,6 +4,7 @@
 #include <algorithm>
 #include <cmath>
 #include <cstdint>
+#include <numeric>
 
 namespace spdp {
 namespace plan {
@@ -23,6 +24,14 @@ inline int pair_tile_tokens(int64_t N) {
     return pair_acc_tokens(N) * (tokens > kPairAccTokens ? 2 : 1);
 }
 
+// Accumulators that a tile's (sub-)blocks can be added to in turn, so that each adds fewer: as many as tensor memory has room for.  Adding them up costs 0.1 to
+// 0.5 us of a call, another cut 1 to 4: 1536x6144 x 33 tokens 9.3 us with one, 9.7 with two, 11.9 cut anew.
+constexpr int kSetColumns = 128;        // kernels 0 and 1: tensor-memory columns for the accumulators of 128 rows
+inline int most_sets(int kernel, int64_t N) {
+    if (kernel <= 1) return std::min<int64_t>(N, kTokens[kernel]) <= kSetColumns / 4 ? 4 : N <= kSetColumns / 2 ? 2 : 1;
+    return kernel == 3 ? (N <= kPairAccTokens ? 2 : 1) : kernel == 4 && N <= kPairHalfTokens ? 2 : 1;      // pairs: the second accumulator, where no tile needs it
+}
+
 // A third X tile for each accumulator pays where the ring still holds four K-blocks beside it; where it does not, the decode waits for
 // copies instead.  us with 2 / 3 X tiles, 18944x3872 x 416 tokens at 67 %: 66 / 60; 18944x4096 x 512 at 90, 50, 30 %: 70 / 62,
 // 71 / 70, 74 / 85; 4096x4096 x 1024 at 50 %: 50 / 57.
@@ -39,6 +48,7 @@ struct Plan {
     int workers, rounds, sharers, slices;
     int64_t tiles, rest;
     int cluster;            // CTAs to a tile that add its sums themselves, 1: a second kernel does
+    int sets;               // accumulators that a tile's (sub-)blocks are added to in turn
 };
 constexpr int kMostSlices = 9;          // of a tile of pairs, where all slices do not fit the device at once
 constexpr int64_t kScratchTokens = 2 * 148 * 256;     // and then no more sums (of 256 rows each) in scratch memory than kernel 2 leaves on 148 SMs
@@ -68,13 +78,82 @@ constexpr double kTwoLaunchesUs = 7.6;    // what the host needs for a call of t
 constexpr double kFullUs = 1.17, kFullShare = 0.9;
 constexpr double kLateUs = 1.82;          // of a call whose successor finds no SM free to start on before it ends
 
-// resident[c]: clusters of c CTAs that the device holds at once; null: no clusters, and kernels 0 to 3 only.  Every call works its plan out anew, so few
-// cuts are looked at: a tile's time is (K-blocks of a CTA) * block + (CTAs of the tile) * each, so those around the minimum of n * block + nkb / n * each
-// are, and as many as fit (all of them took 1.5 to 2.6 us of a call of few row tiles, these 0.4 to 0.8).
-inline Plan make_plan(int64_t R, int64_t nkb, int64_t N, int sms, bool may_cut, const int* resident = nullptr) {
+// Mean square over a call's results of the K-blocks that one accumulator adds, which the error of 32-bit results goes with: the sum of their cubes over a tile's
+// accumulators, over its K-blocks.  Of ranges that cross tiles, those with a border inside have half the sum of cubes on average.
+inline double sums_squared(const Plan& q, int64_t nkb) {
+    const int64_t sets = q.sets, steps = q.kernel >= 3 ? 1 : 2;            // of a K-block, which go to the accumulators in turn
+    const auto cubes = [&](int64_t blocks) {
+        const int64_t n = steps * blocks / sets, longer = steps * blocks % sets;
+        const double a = static_cast<double>(n), b = static_cast<double>(n + 1);
+        return (static_cast<double>(longer) * b * b * b + static_cast<double>(sets - longer) * a * a * a) / static_cast<double>(steps * steps * steps);
+    };
+    const double whole = cubes(nkb) / static_cast<double>(nkb);
+    if (q.rest == 0 || q.sharers <= q.rest) return whole;
+    const int64_t units = q.rest * nkb, n = units / q.sharers, longer = units - n * q.sharers;
+    const double crossing = q.sharers % q.rest == 0 ? 0.0 : static_cast<double>(q.rest - std::gcd(q.rest, static_cast<int64_t>(q.sharers)));
+    const double cut = (static_cast<double>(longer) * cubes(n + 1) + static_cast<double>(q.sharers - longer) * cubes(n)) / static_cast<double>(units) *
+                       (1.0 - 0.5 * crossing / static_cast<double>(q.sharers));
+    return whole + (cut - whole) * static_cast<double>(q.rest) / static_cast<double>(q.tiles);
+}
+
+// The cut that 32-bit results are held against.  The tensor cores do not round what they add to an accumulator to nearest, so the error of a result grows
+// with the K-blocks that one accumulator adds, 5e-8 to 1e-7 of the results' root mean square for each (28672x8192 at 50 %, 128 of them, 9.6e-6; 2560x6144 in
+// sums of 7 and 14 5.5e-7 and 10.6e-7); the partial sums are added with rounding.  (16-bit results have 2.4e-4 by their own rounding.)  The fastest cut has long sums
+// often, because few CTAs make few of them: over 80 calls the estimate below, left to itself, was 1.13 times as far off as this cut, 2.0 times in some.  What is taken
+// here spreads the tiles over all SMs: it is the choice, for kernels 0 to 3, by the times that they had with decoded W in shared memory and the second kernel alone.
+// With it as the limit the error is 0.92 times this cut's on average and no more in any call, and the 32-bit calls take 2.4 % longer (half of them nothing, one in ten 10 to
+// 43 %: 7168x5120 x 761 tokens 63 -> 90 us, whole tiles of 80 K-blocks against sums of 38).
+inline Plan even_cut(int64_t R, int64_t nkb, int64_t N, int sms) {
+    constexpr double kCall[4] = {3.0, 3.7, 3.2, 6.5}, kBlock[4] = {0.88, 0.97, 1.22, 0.69}, kBlockToken[4] = {8.3e-4, 1.8e-4, 0.0, 4.8e-4};     // us
+    constexpr double kTile = 2.1, kTileToken = 2.3e-3, kReduce = 1.9, kReduceMB = 0.223;
     Plan best = {};
     best.us = -1.0;
-    const auto take = [&best](Plan q, double host) {        // (behind the host's time the device's still decides)
+    for (int f = 0; f < 4; ++f) {
+        Plan q = {};
+        q.kernel = f;
+        q.cluster = q.sets = 1;
+        q.tiles = R * ((N + kTokens[f] - 1) / kTokens[f]);
+        const int64_t slots = f == 3 ? sms / 2 : sms, rounds = q.tiles / slots, left = q.tiles - rounds * slots;
+        const double tok = static_cast<double>(std::min<int64_t>(N, kTokens[f])), mb = tok * kTileRows * 4.0e-6;
+        const double block = kBlock[f] + kBlockToken[f] * tok, tile = kTile + kTileToken * tok;
+        const double whole = kCall[f] + (block * static_cast<double>(nkb) + tile) * static_cast<double>(rounds);
+        q.rounds = static_cast<int>(rounds);
+        const auto consider = [&](int64_t w) {              // w CTAs (pairs) for the tiles that are left; as many as these: whole tiles
+            q.slices = f == 3 && w > left ? static_cast<int>(std::min(w / left, nkb)) : 1;
+            if (f == 3) w = q.slices * left;
+            const bool cut = w > left;
+            if (cut && w > left * nkb) return;
+            q.rest = f == 3 && !cut ? 0 : left;
+            q.sharers = static_cast<int>(std::max<int64_t>(w, 1));
+            q.workers = static_cast<int>(rounds > 0 ? slots : w);
+            q.us = whole;
+            if (left > 0) q.us += block * static_cast<double>((left * nkb + w - 1) / w) + tile * (w % left ? 2.0 : 1.0);
+            if (cut) q.us += kReduce + kReduceMB * mb * static_cast<double>(w + left);
+            if (best.us < 0.0 || q.us < best.us) best = q;
+        };
+        consider(left);
+        if (left == 0) continue;
+        for (int64_t share = 2 * left; share < slots; share *= 2) consider(share);
+        if (slots / left > 1) consider(slots / left * left);                    // the most that do not cross tiles
+        if (f != 3) consider(slots);
+    }
+    return best;
+}
+
+// resident[c]: clusters of c CTAs that the device holds at once; null: no clusters, and kernels 0 to 3 only.  Every call works its plan out anew, so few
+// cuts are looked at: a tile's time is (K-blocks of a CTA) * block + (CTAs of the tile) * each, so those around the minimum of n * block + nkb / n * each
+// are, and as many as fit (all of them took 1.5 to 2.6 us of a call of few row tiles, these 0.4 to 0.8).  wide: 32-bit results, whose sums are no
+// longer than those of the even cut, in the mean of their squares.
+inline Plan make_plan(int64_t R, int64_t nkb, int64_t N, int sms, bool may_cut, const int* resident = nullptr, bool wide = false) {
+    Plan best = {};
+    best.us = -1.0;
+    const Plan even = wide && may_cut ? even_cut(R, nkb, N, sms) : Plan{};
+    const double longest = wide && may_cut ? sums_squared(even, nkb) : HUGE_VAL;
+    const auto take = [&](Plan q, double host) {            // (behind the host's time the device's still decides)
+        while (wide && sums_squared(q, nkb) > longest) {
+            if (q.sets == most_sets(q.kernel, N)) return;
+            q.sets *= 2;
+        }
         q.us = std::max(q.us, host) + 0.02 * q.us;
         if (best.us < 0.0 || q.us < best.us) best = q;
     };
@@ -93,7 +172,7 @@ inline Plan make_plan(int64_t R, int64_t nkb, int64_t N, int sms, bool may_cut, 
         const double block = k.block + k.block_token * tok, tile = k.tile + k.tile_token * tok;
         const double whole = k.call + (block * static_cast<double>(nkb) + tile) * static_cast<double>(rounds);
         q.rounds = static_cast<int>(rounds);
-        q.slices = q.cluster = 1;
+        q.slices = q.cluster = q.sets = 1;
         q.sharers = left > 0 ? static_cast<int>(left) : 1;
         q.workers = static_cast<int>(rounds > 0 ? slots : left);
         q.rest = pairs ? 0 : left;
@@ -152,7 +231,7 @@ inline Plan make_plan(int64_t R, int64_t nkb, int64_t N, int sms, bool may_cut, 
             take(q, 0.0);
         }
     }
-    return best;
+    return best.us < 0.0 ? even : best;
 }
 
 }  // namespace plan

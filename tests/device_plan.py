@@ -18,16 +18,17 @@ def lib():
             subprocess.run(["g++", "-O1", "-shared", "-fPIC", "-I", os.path.join(ROOT, "paper_2607_21985_b200", "csrc"),
                             "-o", out, os.path.join(ROOT, "tests", "plan_device_shim.cpp")], check=True)
             _lib = ctypes.CDLL(out)
-        _lib.shim_device_plan.argtypes = [ctypes.c_longlong] * 3 + [ctypes.c_int] + [ctypes.c_void_p] * 2
+        _lib.shim_device_plan.argtypes = _lib.shim_device_plan_wide.argtypes = [ctypes.c_longlong] * 3 + [ctypes.c_int] + [ctypes.c_void_p] * 2
         _lib.shim_pair_acc_tokens.argtypes = _lib.shim_pair_tile_tokens.argtypes = [ctypes.c_longlong]
         _lib.shim_pair_tiles_in_flight.argtypes = [ctypes.c_longlong] * 3
     return _lib
 
 
-def device_plan(R, K, N, sms=148, resident=RESIDENT):
-    v = (ctypes.c_longlong * 8)()
-    lib().shim_device_plan(R, (K + 63) // 64, N, sms, (ctypes.c_int * 17)(*resident), v)
-    q = dict(zip(("kernel", "workers", "rounds", "sharers", "slices", "tiles", "rest", "cluster"), v))
+def device_plan(R, K, N, sms=148, resident=RESIDENT, wide=False):
+    """wide: for 32-bit results."""
+    v = (ctypes.c_longlong * 9)()
+    (lib().shim_device_plan_wide if wide else lib().shim_device_plan)(R, (K + 63) // 64, N, sms, (ctypes.c_int * 17)(*resident), v)
+    q = dict(zip(("kernel", "workers", "rounds", "sharers", "slices", "tiles", "rest", "cluster", "sets"), v))
     q["cut"] = q["rest"] > 0 and q["sharers"] > q["rest"]
     q["crosses"] = q["cut"] and q["kernel"] < 3 and q["sharers"] % q["rest"] > 0        # a CTA's range may end in the next tile
     return q

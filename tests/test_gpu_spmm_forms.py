@@ -1,7 +1,8 @@
 """Prefill products by every form and cut that the library takes on a device of 148 SMs: one CTA per tile of 32, 128 or 256 tokens, whole, cut with a second
 kernel, with ranges that cross tiles; clusters of every size that the rule chooses; CTA pairs of 512 tokens with both numbers of X tiles in flight and
 one or two accumulators in the last token block; pairs with W in tensor memory.  What a shape is there for is held, without a GPU, against the rule with
-the cluster counts that the library hands it.  Whole numbers, so that sums are exact in any order and the results have to be equal."""
+the cluster counts that the library hands it; that is the rule for 16-bit results (32-bit ones are cut more finely, or added to several accumulators in
+turn, and run beside them).  Whole numbers, so that sums are exact in any order and the results have to be equal."""
 import pytest
 
 torch = pytest.importorskip("torch")
@@ -49,6 +50,7 @@ CLUSTERS = {
 PAIRS = {
     (51, 100, 200, 0.0): (3, 4, 51, 0, 1, 1),
     (51, 100, 200, 0.9): (3, 6, 51, 0, 1, 1),
+    (38, 64, 100, 0.5): (3, 4, 38, 0, 1, 1),            # one K-block
     (148, 712, 300, 0.9): (3, 6, 148, 0, 1, 2),
     (37, 5000, 700, 0.0): (3, 4, 74, 0, 1, 1),          # full columns: the ring of values holds two K-blocks
     (37, 5000, 700, 0.8): (3, 6, 74, 0, 1, 1),          # the ring of X tiles moves by one per K-block
@@ -65,6 +67,15 @@ PAIRS = {
     (75, 1000, 300, 0.8): (4, 6, 74, 1, 8, 2),
     (75, 2048, 700, 0.5): (4, 4, 148, 2, 16, 2),
     (5, 4096, 512, 0.5): (4, 4, 0, 10, 7, 1),
+}
+# 32-bit results -> kernel, CTAs of a cluster, accumulators that the K-blocks go to in turn (some of the shapes above have two)
+SETS = {
+    (6, 1000, 40, 0.5): (0, 6, 4),
+    (29, 300, 17, 0.0): (0, 2, 4),
+    (7, 2500, 31, 0.5): (1, 1, 4),
+    (12, 1000, 40, 0.9): (1, 4, 2),
+    (14, 1250, 150, 0.9): (3, 1, 2),
+    (14, 4096, 127, 0.5): (4, 1, 2),
 }
 
 
@@ -92,6 +103,12 @@ def test_shapes_of_pairs(shape):
     assert (q["kernel"], pair_x_tiles(R, K, sparsity), q["tiles"] - q["rest"], q["rest"], q["slices"], 2 if last > acc else 1) == PAIRS[shape]
 
 
+@pytest.mark.parametrize("shape", list(SETS))
+def test_shapes_of_several_accumulators(shape):
+    q = device_plan(*shape[:3], wide=True)
+    assert (q["kernel"], q["cluster"], q["sets"]) == SETS[shape]
+
+
 # ---- the products, on the GPU ----
 
 @pytest.fixture(scope="module")
@@ -115,7 +132,7 @@ def integers(R, K, N, sparsity, short=0):
 
 
 @pytest.mark.gpu
-@pytest.mark.parametrize("shape", list(ONE) + list(CLUSTERS) + list(PAIRS))
+@pytest.mark.parametrize("shape", sorted(set(ONE) | set(CLUSTERS) | set(PAIRS) | set(SETS)))
 def test_products_are_exact(S, shape):
     """Calls in a row, which start beside one another and find an earlier call's sums in the scratch memory; in the last ones a copy just before the
     call makes its input."""
@@ -152,15 +169,17 @@ REFUSED = [(8, 1250, 128, 0.9), (65, 3000, 5, 0.9), (8, 1000, 129, 0.5), (75, 17
 
 
 @pytest.mark.gpu
+@pytest.mark.parametrize("dt", ["float16", "float32"])
 @pytest.mark.parametrize("shape", REFUSED)
-def test_a_refused_tile_stays_unwritten(S, shape):
+def test_a_refused_tile_stays_unwritten(S, shape, dt):
     """A TileOffset word that cannot be (the kernels' own check refuses the K-blocks at it and copies nothing): the status says so, and the tile's outputs stay
     unwritten although other CTAs have left their partial sums of it and the scratch memory holds an earlier call's."""
     R, K, N, sparsity = shape
     h, X, want = integers(R, K, N, sparsity)
+    want = want.to(getattr(torch, dt))
     try:
         def call():
-            Y = torch.full((N, 256 * R), float("nan"), device="cuda")
+            Y = torch.full((N, 256 * R), float("nan"), dtype=want.dtype, device="cuda")
             S.spdp_spmm(h, X, Y)
             torch.cuda.synchronize()
             return Y, S.spdp_last_device_status(h)

@@ -39,12 +39,25 @@ CLUSTERS = {
     (43, 4096, 128, 0.6): (1, 3),
     (15, 9000, 128, 0.5): (1, 9),
 }
+# 32-bit results, whose K-blocks go to several accumulators in turn -> kernel, CTAs of a cluster, accumulators
+SETS = {
+    (60, 2176, 30, 0.5): (1, 2, 2),
+    (43, 4096, 64, 0.6): (1, 3, 2),
+    (10, 6144, 146, 0.5): (4, 1, 2),
+    (10, 9216, 219, 0.9): (3, 1, 2),
+}
 
 
 @pytest.mark.parametrize("shape", list(CLUSTERS))
 def test_shapes_of_clusters(shape):
     q = device_plan(*shape[:3])
     assert (q["kernel"], q["cluster"]) == CLUSTERS[shape]
+
+
+@pytest.mark.parametrize("shape", list(SETS))
+def test_shapes_of_several_accumulators(shape):
+    q = device_plan(*shape[:3], wide=True)
+    assert (q["kernel"], q["cluster"], q["sets"]) == SETS[shape]
 
 
 @pytest.mark.parametrize("shape", list(ONE))
@@ -81,8 +94,8 @@ LIMITS += [(0, LATE, warps, ctas, 1) for warps in (1, 1 << 5, 1 << 10, 1 << 23, 
 
 
 @pytest.mark.gpu
-@pytest.mark.parametrize("shape", list(ONE) + list(PAIRS) + list(CLUSTERS))
-def test_nothing_wrong_is_left(S, shape):
+@pytest.mark.parametrize("shape,dt", [(shape, "float16") for shape in list(ONE) + list(PAIRS) + list(CLUSTERS)] + [(shape, "float32") for shape in SETS])
+def test_nothing_wrong_is_left(S, shape, dt):
     R, K, N, sparsity = shape
     M = 256 * R - 5
     g = torch.Generator(device="cuda").manual_seed(R * K + N)
@@ -90,14 +103,14 @@ def test_nothing_wrong_is_left(S, shape):
     W[torch.rand(M, K, generator=g, device="cuda") < sparsity] = 0
     X = torch.zeros(N, (K + 7) // 8 * 8, dtype=torch.float16, device="cuda")
     X[:, :K] = torch.randint(1, 3, (N, K), generator=g, device="cuda").half()
-    want = (X[:, :K].double() @ W.double().T).float()
+    want = (X[:, :K].double() @ W.double().T).to(getattr(torch, dt))
     other = -X                                                  # whose sums are in the scratch memory
     h = S.spdp_pack_tiled_cbc(W)
     limit = S.lib().spdp_checked_wait_tries
     incomplete = 0
     try:
         def call(x):
-            Y = torch.full((N, M), float("nan"), device="cuda")
+            Y = torch.full((N, M), float("nan"), dtype=want.dtype, device="cuda")
             S.spdp_spmm(h, x[:, :K], Y)
             return Y, S.spdp_last_device_status(h)
         for tries in LIMITS:
