@@ -201,3 +201,64 @@ def test_a_refused_tile_stays_unwritten(S, shape, dt):
         assert status == 0 and torch.equal(Y, want)
     finally:
         S.spdp_free(h)
+
+
+# clusters, ranges that cross tiles, cut pairs of both kinds
+OTHERWISE = [(35, 300, 5, 0.5), (17, 600, 31, 0.0), (43, 4096, 128, 0.6), (75, 1700, 129, 0.9), (14, 1250, 150, 0.5), (5, 4096, 512, 0.5)]
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("dt", [torch.float16, torch.float32])
+@pytest.mark.parametrize("shape", OTHERWISE)
+def test_in_a_graph_and_on_two_streams(S, shape, dt):
+    """A captured pair of calls, whose partial sums are memory of the graph, replayed on new inputs with calls on two streams in between."""
+    R, K, N, sparsity = shape
+    h, X, want = integers(R, K, N, sparsity)
+    want = want.to(dt)
+    other = torch.cuda.Stream()
+    try:
+        buf, minus = (torch.zeros(N, X.stride(0), dtype=torch.float16, device="cuda")[:, :K] for _ in range(2))
+        minus.copy_(-X)
+        Y, beside = torch.empty_like(want), [torch.empty_like(want) for _ in range(2)]
+        S.spdp_spmm(h, buf, Y)
+        torch.cuda.synchronize()
+        graph = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(graph):
+            S.spdp_spmm(h, buf, Y)
+            S.spdp_spmm(h, buf, Y)
+        for x, sign in ((X, 1), (minus, -1), (X, 1)):
+            buf.copy_(x)
+            for y in [Y] + beside:
+                y.fill_(float("nan"))
+            torch.cuda.synchronize()
+            graph.replay()
+            S.spdp_spmm(h, minus, beside[0])
+            S.spdp_spmm(h, X, beside[1], stream=other)
+            graph.replay()
+            torch.cuda.synchronize()
+            assert torch.equal(Y, sign * want) and torch.equal(beside[0], -want) and torch.equal(beside[1], want)
+        assert S.spdp_last_device_status(h) == 0
+        del graph
+    finally:
+        S.spdp_free(h)
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("dt", [torch.float16, torch.float32])
+@pytest.mark.parametrize("shape", OTHERWISE)
+def test_into_any_y(S, shape, dt):
+    """Rows that end inside a group that is stored at once, a Y whose base and row stride are off that group's boundary: nothing outside Y is written."""
+    R, K, N, sparsity = shape
+    M = 256 * R - 6
+    h, X, want = integers(R, K, N, sparsity, short=6)
+    try:
+        for pad, at in ((0, 0), (1, 1), (2, 2), (3, 4), (5, 3)):
+            buf = torch.full((N * (M + pad) + at + 8,), 7.0, dtype=dt, device="cuda")
+            Y = buf[at:at + N * (M + pad)].view(N, M + pad)
+            S.spdp_spmm(h, X, Y[:, :M])
+            torch.cuda.synchronize()
+            assert torch.equal(Y[:, :M], want.to(dt))
+            assert bool((Y[:, M:] == 7.0).all()) and bool((buf[:at] == 7.0).all()) and bool((buf[at + N * (M + pad):] == 7.0).all())
+        assert S.spdp_last_device_status(h) == 0
+    finally:
+        S.spdp_free(h)
