@@ -81,18 +81,18 @@ constexpr double kLateUs = 1.82;          // of a call whose successor finds no 
 // Mean square over a call's results of the K-blocks that one accumulator adds, which the error of 32-bit results goes with: the sum of their cubes over a tile's
 // accumulators, over its K-blocks.  Of ranges that cross tiles, those with a border inside have half the sum of cubes on average.
 inline double sums_squared(const Plan& q, int64_t nkb) {
-    const int64_t sets = q.sets, steps = q.kernel >= 3 ? 1 : 2;            // of a K-block, which go to the accumulators in turn
-    const auto cubes = [&](int64_t blocks) {
-        const int64_t n = steps * blocks / sets, longer = steps * blocks % sets;
-        const double a = static_cast<double>(n), b = static_cast<double>(n + 1);
-        return (static_cast<double>(longer) * b * b * b + static_cast<double>(sets - longer) * a * a * a) / static_cast<double>(steps * steps * steps);
+    const unsigned sets = static_cast<unsigned>(q.sets), steps = q.kernel >= 3 ? 1u : 2u;       // of a K-block, which go to the accumulators in turn
+    const auto cubes = [&](unsigned blocks) {               // (a power of two of accumulators)
+        const unsigned longer = steps * blocks & (sets - 1u), n = (steps * blocks - longer) / sets;
+        const double a = n, b = n + 1u;
+        return (longer * b * b * b + (sets - longer) * a * a * a) * (steps == 1u ? 1.0 : 0.125);
     };
-    const double whole = cubes(nkb) / static_cast<double>(nkb);
+    const double whole = cubes(static_cast<unsigned>(nkb)) / static_cast<double>(nkb);
     if (q.rest == 0 || q.sharers <= q.rest) return whole;
-    const int64_t units = q.rest * nkb, n = units / q.sharers, longer = units - n * q.sharers;
-    const double crossing = q.sharers % q.rest == 0 ? 0.0 : static_cast<double>(q.rest - std::gcd(q.rest, static_cast<int64_t>(q.sharers)));
-    const double cut = (static_cast<double>(longer) * cubes(n + 1) + static_cast<double>(q.sharers - longer) * cubes(n)) / static_cast<double>(units) *
-                       (1.0 - 0.5 * crossing / static_cast<double>(q.sharers));
+    // (fewer than 2^31 K-blocks in all, or the call is refused)
+    const unsigned w = static_cast<unsigned>(q.sharers), rest = static_cast<unsigned>(q.rest), units = rest * static_cast<unsigned>(nkb), n = units / w, longer = units - n * w;
+    const double crossing = w % rest == 0u ? 0.0 : static_cast<double>(rest - std::gcd(rest, w));
+    const double cut = (longer * cubes(n + 1u) + (w - longer) * cubes(n)) / units * (1.0 - 0.5 * crossing / w);
     return whole + (cut - whole) * static_cast<double>(q.rest) / static_cast<double>(q.tiles);
 }
 
@@ -150,12 +150,13 @@ inline Plan make_plan(int64_t R, int64_t nkb, int64_t N, int sms, bool may_cut, 
     const Plan even = wide && may_cut ? even_cut(R, nkb, N, sms) : Plan{};
     const double longest = wide && may_cut ? sums_squared(even, nkb) : HUGE_VAL;
     const auto take = [&](Plan q, double host) {            // (behind the host's time the device's still decides)
+        q.us = std::max(q.us, host) + 0.02 * q.us;
+        if (best.us >= 0.0 && q.us >= best.us) return;
         while (wide && sums_squared(q, nkb) > longest) {
             if (q.sets == most_sets(q.kernel, N)) return;
             q.sets *= 2;
         }
-        q.us = std::max(q.us, host) + 0.02 * q.us;
-        if (best.us < 0.0 || q.us < best.us) best = q;
+        best = q;
     };
     for (int f = 0; f < (resident != nullptr ? 5 : 4); ++f) {
         if (f == 0 ? N > 256 : f >= 2 && N <= 64) continue;                      // never the best where measured
