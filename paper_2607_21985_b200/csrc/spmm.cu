@@ -607,7 +607,7 @@ __device__ __forceinline__ void void_rows(const Params& p, int slot, int row0, i
 // What it saves is the second kernel, which waits for every CTA of the call and holds up the next call's start: 3.5 us of 4096x4096 x 128
 // tokens, 5 of 700x5000, 7 of 11008x4096 x 128.  11008x4096 at 60 % x 128, three CTAs a tile, in cluster / 129 CTAs and second kernel / 148 and second kernel
 // 26.3 / 28.8 / 31.5 us, 18944x4096 x 100 in twos 33.3 / - / 36.3, 8192x4096 x 64 in fours 19.6 / 20.7 / 22.7, 1024x1024 x 16 in eights 6.4 / 7.0 / 7.5,
-// 700x5000 x 16 in sixteens 7.9 / 8.5 / 12.9.  What bounds it is one latency behind the other: stores to L2 (3900 clocks of 11008x4096 x 128), the
+// 700x5000 x 16 in sixteens 7.9 / 8.5 / 12.9 (there the rule takes the second).  What bounds it is one latency behind the other: stores to L2 (3900 clocks of 11008x4096 x 128), the
 // barrier that releases them (2500), copies back (1300), additions.  Tried and slower: sums read by each thread for itself (28.0), own sums
 // left in tensor memory (27.7), stores to the other CTAs' shared memory (27.4: 12 bytes per clock and SM), sums staged in shared memory and written by bulk
 // copies with an arrival at each CTA in place of the barrier (28.4: a released remote arrival takes 400 to 800 clocks).

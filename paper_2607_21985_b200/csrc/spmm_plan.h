@@ -57,7 +57,7 @@ constexpr int kGatherTokens = 126;      // tokens' sums (of 256 rows) that a CTA
 
 // The estimate of a call's time: (K-blocks of the busiest CTA) x (time of a K-block) + a tile's start and end + what the
 // partial sums cost.  Fitted to 399 calls of layers from 512x512 to 28672x8192 (30 to 90 % sparse) with 16 to 1024 tokens, calls in a row on a stream, 5 to 25
-// forms and cuts of each measured: the one taken is 1.5 % behind the best on average, 6 % in one call of ten, 13 % at worst.
+// forms and cuts of each measured: the one taken is 1.5 % behind the best on average, 6 % in one call of ten, 13 % at worst; over 168 other calls 3.5, 12 and 26 %.
 struct Cost {
     double call;                        // a call's fixed part, us
     double block, block_token;          // a K-block (64 columns x 256 rows), and per token of the tile
@@ -101,8 +101,8 @@ inline double sums_squared(const Plan& q, int64_t nkb) {
 // sums of 7 and 14 5.5e-7 and 10.6e-7); the partial sums are added with rounding.  (16-bit results have 2.4e-4 by their own rounding.)  The fastest cut has long sums
 // often, because few CTAs make few of them: over 80 calls the estimate below, left to itself, was 1.13 times as far off as this cut, 2.0 times in some.  What is taken
 // here spreads the tiles over all SMs: it is the choice, for kernels 0 to 3, by the times that they had with decoded W in shared memory and the second kernel alone.
-// With it as the limit the error is 0.92 times this cut's on average and no more in any call, and the 32-bit calls take 2.4 % longer (half of them nothing, one in ten 10 to
-// 43 %: 7168x5120 x 761 tokens 63 -> 90 us, whole tiles of 80 K-blocks against sums of 38).
+// With it as the limit the error is 0.92 times this cut's on average and no more in any call, and the 32-bit calls take 2.3 % longer (most of them nothing, one in ten 10 to
+// 44 %: 7168x5120 x 761 tokens 63 -> 90 us, whole tiles of 80 K-blocks against sums of 38).
 inline Plan even_cut(int64_t R, int64_t nkb, int64_t N, int sms) {
     constexpr double kCall[4] = {3.0, 3.7, 3.2, 6.5}, kBlock[4] = {0.88, 0.97, 1.22, 0.69}, kBlockToken[4] = {8.3e-4, 1.8e-4, 0.0, 4.8e-4};     // us
     constexpr double kTile = 2.1, kTileToken = 2.3e-3, kReduce = 1.9, kReduceMB = 0.223;
